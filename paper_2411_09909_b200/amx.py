@@ -2,18 +2,25 @@
 
 Argument marshalling only: every function checks tensor types, allocates outputs with
 torch (device memory and streams are all torch is used for) and forwards pointers to the
-entry point of the same name.  There is no fallback of any kind: if ``libamx_b200.so``
-has not been built (``python -m paper_2411_09909_b200.build``) the first call raises.
+entry point of the same name.  The functions a program calls per layer do this in an
+extension module (``csrc/binding.cpp``: a small layer takes the GPU less time than ctypes
+takes to convert its arguments), the others through ctypes.  There is no fallback of any
+kind: if the library has not been built (``python -m paper_2411_09909_b200.build``) the
+first call raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libamx_b200.so")
+_NATIVE_PATH = os.path.join(os.path.dirname(_LIB_PATH), "_amx_native.so")
 _lib = None
+_native_module = None
 
 OUT_BF16, OUT_F32 = 0x0, 0x1
 GEMM_AUTO, GEMM_SIMT, GEMM_TC, GEMM_FP4 = 0x0, 0x10, 0x20, 0x40
@@ -125,6 +132,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _native():
+    """The extension module behind the per-layer functions (it links against libamx_b200.so)."""
+    global _native_module
+    if _native_module is None:
+        if not os.path.exists(_NATIVE_PATH):
+            raise AmxError(f"{_NATIVE_PATH} is missing: build it with `python -m paper_2411_09909_b200.build`")
+        lib()
+        loader = importlib.machinery.ExtensionFileLoader("_amx_native", _NATIVE_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_amx_native", _NATIVE_PATH, loader=loader))
+        loader.exec_module(module)
+        module.set_error(AmxError)
+        _native_module = module
+    return _native_module
+
+
 def status_string(rc: int) -> str:
     return lib().amx_status_string(int(rc)).decode()
 
@@ -150,33 +172,12 @@ def _ws(nbytes: int, device) -> torch.Tensor:
 
 def quantize(x: torch.Tensor, group_size: int = 32, fmt: int = FMT_AMXFP4):
     """bf16 [rows, K] (row stride allowed) -> (codes u8 [rows, K/2], scales u8 [rows, K/gs, 2])."""
-    _dev(x, torch.bfloat16, "x")
-    assert x.dim() == 2 and x.stride(1) == 1
-    rows, K = x.shape
-    codes = torch.empty((rows, K // 2), dtype=torch.uint8, device=x.device)
-    scales = torch.empty((rows, max(K // group_size, 0), 2), dtype=torch.uint8, device=x.device)
-    ld = x.stride(0) if rows > 1 else max(K, x.stride(0))
-    if fmt == FMT_AMXFP4:
-        _check(lib().amx_quantize(x.data_ptr(), rows, K, ld, group_size, codes.data_ptr(), scales.data_ptr(), _stream()),
-               "amx_quantize")
-    else:
-        _check(lib().amx_quantize_fmt(x.data_ptr(), rows, K, ld, group_size, fmt, codes.data_ptr(), scales.data_ptr(),
-                                      _stream()), "amx_quantize_fmt")
-    return codes, scales
+    return (_native_module or _native()).quantize(x, group_size, fmt)
 
 
 def fake_quantize(x: torch.Tensor, group_size: int = 32, fmt: int = FMT_AMXFP4, out: torch.Tensor | None = None):
     """bf16 [rows, K] (row stride allowed) -> the dequantized cast of x as bf16 (same strides rules); out may be x."""
-    _dev(x, torch.bfloat16, "x")
-    assert x.dim() == 2 and x.stride(1) == 1
-    rows, K = x.shape
-    if out is None:
-        out = torch.empty((rows, K), dtype=torch.bfloat16, device=x.device)
-    assert out.shape == x.shape and out.stride(1) == 1
-    ld = lambda t: t.stride(0) if rows > 1 else max(K, t.stride(0))
-    _check(lib().amx_fake_quantize(x.data_ptr(), rows, K, ld(x), group_size, fmt, out.data_ptr(), ld(out), _stream()),
-           "amx_fake_quantize")
-    return out
+    return (_native_module or _native()).fake_quantize(x, group_size, fmt, out)
 
 
 def quantize_t(x: torch.Tensor, group_size: int = 32):
@@ -192,45 +193,18 @@ def quantize_t(x: torch.Tensor, group_size: int = 32):
 
 
 def dequantize(codes: torch.Tensor, scales: torch.Tensor, group_size: int = 32, dtype=torch.bfloat16):
-    _dev(codes, torch.uint8, "codes"), _dev(scales, torch.uint8, "scales")
-    rows, K = codes.shape[0], codes.shape[1] * 2
-    out = torch.empty((rows, K), dtype=dtype, device=codes.device)
-    flag = {torch.bfloat16: OUT_BF16, torch.float32: OUT_F32}[dtype]
-    _check(lib().amx_dequantize(codes.data_ptr(), scales.data_ptr(), rows, K, group_size, flag,
-                                out.data_ptr(), K, _stream()), "amx_dequantize")
-    return out
+    return (_native_module or _native()).dequantize(codes, scales, group_size, {torch.bfloat16: True, torch.float32: False}[dtype])
 
 
 def quant_error(x: torch.Tensor, codes: torch.Tensor, scales: torch.Tensor, group_size: int = 32) -> torch.Tensor:
     """Device tensor of 4 doubles: sum x^2, sum (x - xhat)^2, its part from clamped elements, their count."""
-    _dev(x, torch.bfloat16, "x"), _dev(codes, torch.uint8, "codes"), _dev(scales, torch.uint8, "scales")
-    assert x.dim() == 2 and x.stride(1) == 1 and codes.is_contiguous() and scales.is_contiguous()
-    rows, K = x.shape
-    out = torch.empty(4, dtype=torch.float64, device=x.device)
-    ws = torch.empty(lib().amx_quant_error_workspace_bytes(), dtype=torch.uint8, device=x.device)
-    _check(lib().amx_quant_error(x.data_ptr(), rows, K, x.stride(0), codes.data_ptr(), scales.data_ptr(), group_size,
-                                 out.data_ptr(), ws.data_ptr(), ws.numel(), _stream()), "amx_quant_error")
-    return out
+    return (_native_module or _native()).quant_error(x, codes, scales, group_size)
 
 
 def gemm(a_codes, a_scales, w_codes, w_scales, group_size: int = 32, flags: int = GEMM_AUTO,
          out: torch.Tensor | None = None, workspace: torch.Tensor | None = None):
     """fp32 [M, N] = decoded A [M, K] times decoded W [N, K] transposed."""
-    for t, n in ((a_codes, "a_codes"), (a_scales, "a_scales"), (w_codes, "w_codes"), (w_scales, "w_scales")):
-        _dev(t, torch.uint8, n)
-        assert t.is_contiguous()
-    M, K = a_codes.shape[0], a_codes.shape[1] * 2
-    N = w_codes.shape[0]
-    assert w_codes.shape[1] * 2 == K
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.float32, device=a_codes.device)
-    need = lib().amx_workspace_bytes(M, N, K, group_size, flags)
-    if workspace is None:
-        workspace = _ws(need, a_codes.device)
-    _check(lib().amx_gemm(a_codes.data_ptr(), a_scales.data_ptr(), w_codes.data_ptr(), w_scales.data_ptr(),
-                          M, N, K, group_size, flags, out.data_ptr(), out.stride(0), workspace.data_ptr(),
-                          workspace.numel(), _stream()), "amx_gemm")
-    return out
+    return (_native_module or _native()).gemm(a_codes, a_scales, w_codes, w_scales, group_size, flags, out, workspace)
 
 
 def prepare(codes: torch.Tensor, scales: torch.Tensor, is_weight: bool, group_size: int = 32) -> torch.Tensor:
@@ -246,22 +220,7 @@ def prepare(codes: torch.Tensor, scales: torch.Tensor, is_weight: bool, group_si
 def quantize_prepared(x: torch.Tensor, is_weight: bool, group_size: int = 32, prepared: torch.Tensor | None = None,
                       fmt: int = FMT_AMXFP4, want_codes: bool = True):
     """Cast and prepare in one go: returns (codes, scales, prepared); codes is None when want_codes is False."""
-    _dev(x, torch.bfloat16, "x")
-    assert x.is_contiguous()
-    rows, K = x.shape
-    codes = torch.empty((rows, K // 2), dtype=torch.uint8, device=x.device) if want_codes else None
-    scales = torch.empty((rows, K // group_size, 2), dtype=torch.uint8, device=x.device)
-    buf = prepared if prepared is not None else _ws(lib().amx_prepared_bytes(rows, K, group_size, int(is_weight)), x.device)
-    if fmt == FMT_AMXFP4:
-        _check(lib().amx_quantize_prepared(x.data_ptr(), rows, K, group_size, int(is_weight),
-                                           codes.data_ptr() if want_codes else None,
-                                           scales.data_ptr(), buf.data_ptr(), buf.numel(), _stream()), "amx_quantize_prepared")
-    else:
-        _check(lib().amx_quantize_prepared_fmt(x.data_ptr(), rows, K, group_size, int(is_weight), fmt,
-                                               codes.data_ptr() if want_codes else None,
-                                               scales.data_ptr(), buf.data_ptr(), buf.numel(), _stream()),
-               "amx_quantize_prepared_fmt")
-    return codes, scales, buf
+    return (_native_module or _native()).quantize_prepared(x, is_weight, group_size, prepared, fmt, want_codes)
 
 
 def gemm_prepared(a_prepared: torch.Tensor, w_prepared: torch.Tensor, M: int, N: int, K: int, group_size: int = 32,
@@ -269,20 +228,8 @@ def gemm_prepared(a_prepared: torch.Tensor, w_prepared: torch.Tensor, M: int, N:
                   out_dtype=torch.float32):
     """sym: both operands are in a symmetric format (amx_gemm_prepared_sym; a violated promise shows in gemm_status);
     out_dtype torch.bfloat16: the result rounded to bf16 in the epilogue (amx_gemm_prepared_ex)."""
-    if out is None:
-        out = torch.empty((M, N), dtype=out_dtype, device=a_prepared.device)
-    if workspace is None:
-        workspace = _ws(lib().amx_gemm_prepared_workspace_bytes(M, N, K, group_size), a_prepared.device)
-    if out.dtype == torch.bfloat16:
-        _check(lib().amx_gemm_prepared_ex(a_prepared.data_ptr(), w_prepared.data_ptr(), M, N, K, group_size,
-                                          PREP_OUT_BF16 | (PREP_ONE_PLANE if sym else 0), out.data_ptr(), out.stride(0),
-                                          workspace.data_ptr(), workspace.numel(), _stream()), "amx_gemm_prepared_ex")
-        return out
-    _dev(out, torch.float32, "out")
-    fn = lib().amx_gemm_prepared_sym if sym else lib().amx_gemm_prepared
-    _check(fn(a_prepared.data_ptr(), w_prepared.data_ptr(), M, N, K, group_size, out.data_ptr(),
-              out.stride(0), workspace.data_ptr(), workspace.numel(), _stream()), "amx_gemm_prepared")
-    return out
+    return (_native_module or _native()).gemm_prepared(a_prepared, w_prepared, M, N, K, group_size, out, workspace, sym,
+                                                       out_dtype == torch.bfloat16)
 
 
 def gemm_status(workspace: torch.Tensor) -> int:
@@ -293,26 +240,7 @@ def quant_gemm(a: torch.Tensor, w_codes=None, w_scales=None, group_size: int = 3
                out: torch.Tensor | None = None, workspace: torch.Tensor | None = None, w_bf16: torch.Tensor | None = None):
     """fp32 [M, N] = AMXFP4(a) x W; a is bf16 [M, K]; W is either quantized (w_codes, w_scales) or bf16 [N, K]
     (w_bf16), which the call casts too."""
-    _dev(a, torch.bfloat16, "a")
-    M, K = a.shape
-    if w_bf16 is not None:
-        _dev(w_bf16, torch.bfloat16, "w_bf16")
-        assert w_codes is None and w_scales is None and w_bf16.stride(1) == 1
-    N = w_bf16.shape[0] if w_bf16 is not None else w_codes.shape[0]
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.float32, device=a.device)
-    need = lib().amx_quant_gemm_workspace_bytes(M, N, K, group_size, (flags & ~GEMM_CAST_IN_KERNEL) |
-                                                (WEIGHT_BF16 if w_bf16 is not None else 0))
-    if workspace is None:
-        workspace = _ws(need, a.device)
-    _check(lib().amx_quant_gemm(a.data_ptr(), a.stride(0),
-                                w_codes.data_ptr() if w_codes is not None else None,
-                                w_scales.data_ptr() if w_scales is not None else None,
-                                w_bf16.data_ptr() if w_bf16 is not None else None,
-                                w_bf16.stride(0) if w_bf16 is not None else 0, M, N, K,
-                                group_size, flags, out.data_ptr(), out.stride(0), workspace.data_ptr(),
-                                workspace.numel(), _stream()), "amx_quant_gemm")
-    return out
+    return (_native_module or _native()).quant_gemm(a, w_codes, w_scales, group_size, flags, out, workspace, w_bf16)
 
 
 def gemm_flushed_scales(workspace: torch.Tensor) -> int:
@@ -374,20 +302,7 @@ NV_ASYMMETRIC = 0x1
 
 def quantize_nvfp4(x: torch.Tensor, asym: bool, prepared_as: str | None = None):
     """bf16 [rows, K] -> (codes, E4M3 scales [rows, K/16, 2], tensor_scale (2 floats: t, max|x|)[, prepared])."""
-    _dev(x, torch.bfloat16, "x")
-    assert x.dim() == 2 and x.stride(1) == 1
-    rows, K = x.shape
-    codes = torch.empty((rows, K // 2), dtype=torch.uint8, device=x.device)
-    scales = torch.empty((rows, K // 16, 2), dtype=torch.uint8, device=x.device)
-    ts = torch.empty(2, dtype=torch.float32, device=x.device)
-    is_w = int(prepared_as == "w")
-    prep = None
-    if prepared_as is not None:
-        prep = torch.full((lib().amx_nvfp4_prepared_bytes(rows, K, is_w),), 0xFF, dtype=torch.uint8, device=x.device)
-    _check(lib().amx_quantize_nvfp4(x.data_ptr(), rows, K, x.stride(0), NV_ASYMMETRIC if asym else 0, codes.data_ptr(),
-                                    scales.data_ptr(), ts.data_ptr(), is_w, prep.data_ptr() if prep is not None else None,
-                                    prep.numel() if prep is not None else 0, _stream()), "amx_quantize_nvfp4")
-    return (codes, scales, ts) if prep is None else (codes, scales, ts, prep)
+    return (_native_module or _native()).quantize_nvfp4(x, asym, {None: 0, "a": 1, "w": 2}[prepared_as])
 
 
 def dequantize_nvfp4(codes: torch.Tensor, scales: torch.Tensor, ts: torch.Tensor, dtype=torch.float32):
@@ -401,13 +316,7 @@ def dequantize_nvfp4(codes: torch.Tensor, scales: torch.Tensor, ts: torch.Tensor
 
 def gemm_nvfp4(a_prepared: torch.Tensor, w_prepared: torch.Tensor, M: int, N: int, K: int, workspace: torch.Tensor | None = None,
                sym: bool = False):
-    out = torch.empty((M, N), dtype=torch.float32, device=a_prepared.device)
-    if workspace is None:
-        workspace = _ws(256, a_prepared.device)
-    fn = lib().amx_gemm_nvfp4_sym if sym else lib().amx_gemm_nvfp4
-    _check(fn(a_prepared.data_ptr(), w_prepared.data_ptr(), M, N, K, out.data_ptr(), N, workspace.data_ptr(),
-              workspace.numel(), _stream()), "amx_gemm_nvfp4")
-    return out
+    return (_native_module or _native()).gemm_nvfp4(a_prepared, w_prepared, M, N, K, workspace, sym)
 
 
 F16S_ASYMMETRIC = 0x1
@@ -497,22 +406,7 @@ def attention_heads(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, flags: in
                     workspace: torch.Tensor | None = None):
     """Fully quantized attention for all heads through the single C entry point.  q: bf16 [H, L, d]; k, v: bf16
     [H_kv, L, d] with H % H_kv == 0 (grouped queries when H_kv < H); all contiguous.  Returns O fp32 [H, L, d]."""
-    for t in (q, k, v):
-        _dev(t, torch.bfloat16, "q/k/v")
-        assert t.is_contiguous() and t.shape[1:] == q.shape[1:]
-    assert k.shape == v.shape
-    H, Lq, d = q.shape
-    need = lib().amx_attention_workspace_bytes_for(Lq, d, flags)
-    if workspace is None:
-        workspace = _ws(need, q.device)
-    out = torch.empty((H, Lq, d), dtype=torch.float32, device=q.device)
-    if k.shape[0] == H:
-        _check(lib().amx_attention(q.data_ptr(), k.data_ptr(), v.data_ptr(), H, Lq, d, flags, out.data_ptr(),
-                                   workspace.data_ptr(), workspace.numel(), _stream()), "amx_attention")
-    else:
-        _check(lib().amx_attention_gqa(q.data_ptr(), k.data_ptr(), v.data_ptr(), H, k.shape[0], Lq, d, flags, out.data_ptr(),
-                                       workspace.data_ptr(), workspace.numel(), _stream()), "amx_attention_gqa")
-    return out
+    return (_native_module or _native()).attention_heads(q, k, v, flags, workspace)
 
 
 def attention(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, group_size: int = 32, flags: int = GEMM_AUTO):

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> paper_2411_09909_b200/libamx_b200.so (sm_100a).
+"""Builds in-tree: csrc/*.cu -> paper_2411_09909_b200/libamx_b200.so (sm_100a), and the extension module
+csrc/binding.cpp -> paper_2411_09909_b200/_amx_native.so on top of it.
 
     python -m paper_2411_09909_b200.build [--force] [--verbose]
 
@@ -10,6 +11,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +19,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libamx_b200.so")
+NATIVE = os.path.join(PKG, "_amx_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -57,7 +60,32 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         subprocess.check_call([_nvcc(), "-shared", "-Wno-deprecated-gpu-targets", "-o", tmp, *objs])
         os.replace(tmp, LIB)
+    _build_native(force, verbose)
     return LIB
+
+
+def _build_native(force: bool, verbose: bool) -> None:
+    """The CPython extension over the library (host C++ only; links libamx_b200.so beside it and torch's libraries)."""
+    src, header = os.path.join(CSRC, "binding.cpp"), os.path.join(ROOT, "include", "amx.h")
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= max(os.path.getmtime(src), os.path.getmtime(header)):
+        return
+    import torch
+    torch_dir = os.path.dirname(torch.__file__)
+    cuda_home = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
+    includes = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+                sysconfig.get_paths()["include"], os.path.join(cuda_home, "include"), os.path.join(ROOT, "include")]
+    tmp = NATIVE + f".{os.getpid()}.tmp"
+    lib_dir = os.path.join(torch_dir, "lib")
+    cmd = ["g++", "-O2", "-std=c++20", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *[f"-I{i}" for i in includes], src, "-o", tmp,
+           f"-L{PKG}", "-l:libamx_b200.so", "-Wl,-rpath,$ORIGIN", f"-L{lib_dir}", f"-Wl,-rpath,{lib_dir}", "-ltorch_python", "-ltorch",
+           "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode:
+        sys.stderr.write(res.stdout + res.stderr)
+    if res.returncode:
+        raise RuntimeError("building the extension module failed")
+    os.replace(tmp, NATIVE)
 
 
 if __name__ == "__main__":
