@@ -72,11 +72,11 @@ typedef enum amx_status {
 /* flags for amx_dequantize: output element type (default bf16) */
 #define AMX_OUT_BF16 0x0u
 #define AMX_OUT_F32 0x1u
-/* flags for amx_gemm / amx_quant_gemm: kernel choice.  Default (AMX_GEMM_AUTO): group size 32 runs on
- * the tensor cores - the FP4 kernel when M*N*K >= 2^28, the exact bf16-decode kernel below that and for
- * at most 64 rows of A against a large weight (decode-like shapes: that kernel then cuts K into slices over
- * CTAs and adds the partial products in slice order) - except that at most 64 rows of A with K >= 512 and
- * K % 128 == 0 go to the weight-streaming kernel (AMX_GEMM_ROWS); other group sizes run on the SIMT kernel.
+/* flags for amx_gemm / amx_quant_gemm: kernel choice.  Default (AMX_GEMM_AUTO): at most 64 rows of A with K >= 512 and
+ * K % 128 == 0 go to the weight-streaming kernel (AMX_GEMM_ROWS), as do up to 256 rows of a small product or against a
+ * large weight (in blocks of rows); otherwise group size 32 runs on the tcgen05 tensor cores - the FP4 kernel when
+ * M*N*K >= 2^28, the exact bf16-decode kernel below that (which cuts K into slices over CTAs when a product has few
+ * output tiles and adds the partial products in slice order); what remains runs on the SIMT kernel.
  * AUTO never loses a scale: where it picks the FP4 kernel and preparing the operands had to flush one (see
  * AMX_GEMM_FP4), the FP4 kernel returns at once and the exact bf16-decode kernel computes the product instead.
  * The decision is taken on the device, from the count amx_gemm_flushed_scales() reports; it costs one empty
@@ -97,9 +97,9 @@ typedef enum amx_status {
                               * amx_gemm_flushed_scales / amx_prepared_flushed_scales.  Needs the larger
                               * workspace amx_workspace_bytes() reports. */
 #define AMX_GEMM_ROWS 0x100u /* weight-streaming kernel for M <= 64 rows of A (decode phase): reads the canonical
-                              * weight once, exact bf16 decode, K ranges added in a fixed order; gs = 32,
+                              * weight once, exact decode to f16, K ranges added in a fixed order; gs 16, 32, 64 or 128,
                               * K % 128 == 0, else AMX_ERR_SHAPE; w_scales 4-byte aligned, else AMX_ERR_ALIGN
-                              * (also when AMX_GEMM_AUTO picked this kernel) */
+                              * (also in amx_quant_gemm when AMX_GEMM_AUTO picked this kernel for at most 64 rows) */
 /* extra flag for amx_quant_gemm, only together with AMX_GEMM_TC: one launch, the GEMM's operand-staging
  * warps cast each activation tile to AMXFP4 in registers instead of reading codes a separate cast launch
  * wrote.  Bit-identical result.  The tile is cast once per column of output tiles, and the staging warps

@@ -26,18 +26,22 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     if (want == AMX_GEMM_TC) return tc ? AMX_GEMM_TC : 0;
     if (want == AMX_GEMM_SIMT) return AMX_GEMM_SIMT;
     const bool rows = gemm_rows_supported(M, N, K, gs);
-    if (want == AMX_GEMM_ROWS) return rows ? AMX_GEMM_ROWS : 0;
+    if (want == AMX_GEMM_ROWS) return rows && M <= 64 ? AMX_GEMM_ROWS : 0;
     // AMX_GEMM_AUTO: the FP4-pipe kernel for anything that fills the machine (it is about twice as fast as
     // the bf16-decode kernel); the exact bf16-decode kernel for small products (below 2^28 multiply-adds), where
     // launch count matters more than throughput - the FP4 route costs two launches more: one preparation per
     // operand, and under AUTO the gated exact kernel behind it; the SIMT kernel for group sizes the tensor-core kernels do not take.
     // A few token rows against a big weight (decode-like): too few 128 x 256 tiles to fill the machine, and the
     // FP4 kernel would have to prepare the whole weight for them; the bf16-decode kernel slices K over CTAs.
-    // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.
-    if (rows && K >= 512) return AMX_GEMM_ROWS;
+    // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows it still wins,
+    // in blocks of 64 rows, where the product is small (one launch against three to five) or the weight is what has to
+    // be moved (from 2^23 elements; the FP4 kernel would first prepare all of it for one or two row blocks of output).
+    const double mnk = (double)M * (double)N * (double)K;
+    if (rows && K >= 512 && (M <= 64 || mnk < 268435456.0 || (mnk < 536870912.0 && N >= 512) || N * K >= (1ll << 23)))
+        return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
-    if (gemm_fp4_supported(M, N, K, gs) && (double)M * (double)N * (double)K >= 256.0 * 1024.0 * 1024.0) return AMX_GEMM_FP4;
+    if (gemm_fp4_supported(M, N, K, gs) && mnk >= 268435456.0) return AMX_GEMM_FP4;
     return tc ? AMX_GEMM_TC : AMX_GEMM_SIMT;
 }
 
@@ -50,7 +54,7 @@ size_t kernel_workspace(uint32_t kernel, int64_t M, int64_t N, int64_t K, bool f
     if (kernel == AMX_GEMM_TC) return round_up(gemm_tc_workspace_bytes(M, N, K));
     if (kernel == AMX_GEMM_FP4)
         return round_up(gemm_fp4_workspace_bytes(M, N, K)) + (fallback ? round_up(gemm_tc_workspace_bytes(M, N, K)) : 0);
-    if (kernel == AMX_GEMM_ROWS) return round_up(gemm_rows_workspace_bytes(M, K));
+    if (kernel == AMX_GEMM_ROWS) return round_up(gemm_rows_workspace_bytes(M, N, K));
     return 0;
 }
 
@@ -110,13 +114,12 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (kernel == AMX_GEMM_SIMT)
         return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st);
-    if (!aligned(a_codes, 16) || !aligned(w_codes, 16)) return AMX_ERR_ALIGN;
-    // AUTO picked the weight-streaming kernel but the weight's scales miss its alignment (4-byte asynchronous
-    // copies): the plain kernel takes any 2-byte aligned scales and needs no scratch
-    if (kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) {
-        if ((flags & kKernelMask) == AMX_GEMM_ROWS) return AMX_ERR_ALIGN;
+    // AUTO picked a kernel whose alignment the operands miss (the weight-streaming kernel copies scales 4 bytes at a time;
+    // 16-byte codes for group sizes that used to run on the plain kernel): the plain kernel takes them and needs no scratch
+    const bool codes16 = aligned(a_codes, 16) && aligned(w_codes, 16), is_auto = (flags & kKernelMask) == AMX_GEMM_AUTO;
+    if (is_auto && ((kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) || (group_size != 32 && !codes16)))
         return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st);
-    }
+    if (!codes16 || (kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4))) return AMX_ERR_ALIGN;
     const bool fallback = auto_fallback(flags, kernel);
     const size_t need = kernel_workspace(kernel, M, N, K, fallback);
     if (need && (!workspace || workspace_bytes < need)) return AMX_ERR_WORKSPACE;
@@ -129,7 +132,7 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
                        static_cast<uint8_t*>(workspace) + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
     }
     if (kernel == AMX_GEMM_ROWS)
-        return gemm_rows(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c, workspace, st);
+        return gemm_rows(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, workspace, st);
     return gemm_tc(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c, workspace, st);
 }
 
@@ -219,13 +222,18 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
     flags &= kKernelMask;
     if (cast_in_kernel && flags != AMX_GEMM_TC) return AMX_ERR_FLAGS;
     if (!gemm_shape_ok(M, N, K, group_size) || ld_a < K || ld_c < N || (w_is_bf16 && ld_w < K)) return AMX_ERR_SHAPE;
-    const uint32_t kernel = pick_kernel(M, N, K, group_size, flags);
+    uint32_t kernel = pick_kernel(M, N, K, group_size, flags);
     if (!kernel) return (flags & (flags - 1)) ? AMX_ERR_FLAGS : AMX_ERR_SHAPE;
     if (M == 0 || N == 0) return AMX_OK;
     // exactly one form of the weight
     if (!A || !C || (w_is_bf16 ? (w_codes || w_scales) : (!w_codes || !w_scales))) return AMX_ERR_NULL;
     const size_t need = amx_quant_gemm_workspace_bytes(M, N, K, group_size, flags | (w_is_bf16 ? AMX_WEIGHT_BF16 : 0));
     if (!workspace || workspace_bytes < need) return AMX_ERR_WORKSPACE;
+    // as in amx_gemm: operands that miss the alignment of the kernel AUTO picked run on the plain kernel (with groups of
+    // 32 and at most 64 rows they are refused, as documented at AMX_GEMM_ROWS)
+    if (flags == AMX_GEMM_AUTO && !w_is_bf16 && !(group_size == 32 && M <= 64) &&
+        ((kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) || (group_size != 32 && !aligned(w_codes, 16))))
+        kernel = AMX_GEMM_SIMT;
     const int code_align = kernel == AMX_GEMM_SIMT ? 4 : 16;
     if (!aligned(workspace, kAlign) || !aligned(A, 16) || ld_a % 8 || !aligned(C, 4) ||
         (w_is_bf16 ? (!aligned(W_bf16, 16) || ld_w % 8) : (!aligned(w_codes, code_align) || !aligned(w_scales, 2))))
@@ -282,7 +290,7 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
         return gemm_tc_cast(A, ld_a, w_codes, w_scales, M, N, K, C, ld_c, base, st);
     if (kernel == AMX_GEMM_ROWS)
         // the cast of the few rows writes the decoded operand of the weight-streaming kernel directly: two launches
-        return gemm_rows_cast(A, ld_a, w_codes, w_scales, M, N, K, C, ld_c, base, st);
+        return gemm_rows_cast(A, ld_a, w_codes, w_scales, M, N, K, group_size, C, ld_c, base, st);
     rc = amx_quantize(A, M, K, ld_a, group_size, a_codes, a_scales, stream);
     if (rc != AMX_OK) return rc;
     return amx_gemm(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, kernel, C, ld_c, base, gemm_ws, stream);

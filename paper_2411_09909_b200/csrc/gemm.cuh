@@ -27,14 +27,16 @@ int gemm_tc_cast(const void* x, int64_t ld_a, const uint8_t* w_codes, const uint
                  int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
 int gemm_tc_status(const void* workspace, cudaStream_t st);
 
-// Weight-streaming kernel for at most 64 rows of A (mma.sync on exactly decoded bf16, K ranges over a cluster):
-// the workspace holds the decoded rows; gemm_rows_cast casts the bf16 rows X [M, ld_x] itself.
+// Weight-streaming kernel for few rows of A (mma.sync on exactly decoded f16, K ranges over a cluster; any fixed group
+// size, K % 128 == 0).  Up to kRowsMaxM rows: blocks of at most 64 rows re-read the weight.  The workspace holds the
+// status words and room for the decoded rows; gemm_rows_cast casts the bf16 rows X [M, ld_x] itself.
+constexpr int64_t kRowsMaxM = 256;
 bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs);
-size_t gemm_rows_workspace_bytes(int64_t M, int64_t K);
+size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K);
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
-              int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
+              int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
 int gemm_rows_cast(const void* x, int64_t ld_x, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N,
-                   int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
+                   int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
 
 // FP4-pipe kernel (four block-scaled MMAs per tile pair): same contract; the workspace also holds
 // the prepared operands (sign planes, UE4M3 scale-factor blocks, row offsets).

@@ -1,40 +1,47 @@
-// AMXFP4 x AMXFP4 -> fp32 for at most 64 rows of A against a large weight (the decode phase of inference):
+// AMXFP4 x AMXFP4 -> fp32 for few rows of A against a large weight (the decode phase of inference, small layers):
 // C[m,n] = sum_k Ahat[m,k] * What[n,k] (arXiv 2411.09909, Section 4.3), bound by streaming the 4.5-bit weight
-// from HBM once, not by arithmetic.
+// from HBM once.
 //
-// The weight is read in its canonical layout (codes [N, K/2], scales [N, K/32, 2]); nothing is prepared ahead.
-// The few activation rows are cast and decoded to bf16 once by a small kernel (decoded values are exact in bf16,
-// Eq. 1), already in the order the multiply instruction's fragments want.
+// The weight is read in its canonical layout (codes [N, K/2], scales [N, K/gs, 2]); nothing is prepared ahead.
+// Warp-level mma.sync m16n8k16 (f16 in, fp32 accumulate) with 16 weight rows as the M side and 8 token rows as the
+// N side, so that a single token wastes 7 of 8 columns and not 15 of 16 rows.  The contraction index may be permuted
+// freely as long as both operands use the same permutation: lane (g, t) (g = lane / 4, t = lane % 4) owns, per step
+// of 128 elements of K, the 32-element piece t of weight rows g and g + 8 of each of its warp's two 16-row blocks.
 //
-// Streaming kernel: warp-level mma.sync m16n8k16 (bf16 in, fp32 accumulate) with 16 token rows as the M side and
-// 8 weight rows as the N side; up to four tiles of 16 token rows reuse the decoded weight registers of a step.
-// The contraction index may be permuted freely as long as both operands use the same permutation; here lane
-// (g, t) (g = lane / 4, t = lane % 4) owns, for one step of 128 elements of K, the whole 32-element group
-// 4 * step + t of weight row g of each of its two 8-row tiles: 16 bytes of codes and the group's two scales per
-// tile, brought in by asynchronous copies into a per-warp ring in shared memory four steps ahead (no registers
-// are held by loads in flight) and decoded in registers with packed bf16 multiplies (decode_pairs below).
-// The matching activation values (rows g and g + 8, same group) are read from global memory in 16-byte pieces,
-// 512 contiguous bytes per warp and load; every warp of every CTA on an SM reads the same few hundred KB, so they
-// come from the L1 (staging them in shared memory needed a block barrier every few steps and measured slower).
-// Eight MMAs per tile and step consume four elements per lane each.  What bounds the kernel is instruction
-// issue (decode on the integer/logic pipe), not the tensor cores: the MMAs are a few percent of the instructions.
+// Exactness.  Operands are decoded to f16: E2M1 x E5M2 has at most 5 significant bits and magnitudes between 2^-17 and
+// 6 * 57344; times 2^-4 every value is a (possibly subnormal) f16 number, on both sides, and the result is multiplied
+// by 2^8.  Products are exact in fp32; only the fp32 additions round.
 //
-// A CTA of eight warps covers 128 weight rows and one range of K; the ranges of K of the same 128 rows are the
-// CTAs of one thread-block cluster (up to 8), which add their partial products over distributed shared memory
-// in rank order - deterministic, no scratch in global memory and no second launch.
+// Decode.  cvt.rn.f16x2.e2m1x2 turns a code byte into two signed values; the positive ones take the positive side's
+// scale, the negative ones the other: v = relu(w * s_p) + min(w, 0) * s_n (one of the two terms is zero).  This is what
+// bounds the kernel where the memory does not: 6.6 cycles of a warp per pair of elements, the MMAs included, with four
+// warps on a scheduler.  Measured in the same loop: max/min, multiply, multiply-add 7.8; two clamped multiply-adds
+// and a subtraction 7.4; the scale chosen by a sign mask 7.7; code bits shifted into bf16 fields and the scale chosen
+// by a mask (the earlier form) 8.7; the signs kept apart through two MMAs 7.1.
 //
-// The two launches of a call are chained by programmatic dependent launch: the streaming kernel is allowed onto the
-// SMs while the fragments kernel still runs, sets up and fills its weight rings (the weight does not depend on the
-// fragments), and only then waits for the fragments kernel to complete; the fragments kernel in turn waits for
-// whatever ran before it in the stream before it writes anything.  Measured on a 16-row step over four weights:
-// 87 -> 71 us with plain launches; replayed from a CUDA graph the same step takes 71 us without these edges and
-// 81 us with them, so a stream that is being captured gets ordinary launches.
+// A CTA of eight warps covers 128 weight rows and one range of K: warp = (row group of 32) + 4 * (parity of its
+// steps).  The codes come through a ring in shared memory by asynchronous copies, a slot per warp and step (a lane reads
+// back only its own copies; no registers are held by loads in flight): the copies alone stream at 5.4-5.8 TB/s.  The
+// scales of the whole range are copied once at the start, along the rows.  (Copied per step beside the codes, 8 bytes
+// per row at 32 different rows per instruction, they took more of the load path than the codes themselves: streaming
+// alone 7.5-9 instead of 4.7 us for 12288 x 4096.)  The K ranges of the same rows are the CTAs of one thread-block
+// cluster (up to 8), which add their partial products over distributed shared memory in rank order - deterministic,
+// no scratch in global memory and no second launch.
+//
+// The token rows, two ways:
+//   CAST      every CTA casts its K range of the rows itself (one launch per call): one tile of 8 rows, or a small
+//             product, where launches are what costs.  The redundant casts grow with the rows: at 16 rows they would
+//             be half of the decode work.
+//   otherwise a small kernel casts (or decodes) the rows once into the fragment order, and the main kernel copies the
+//             fragments of a step into its ring beside the weight.
+// Launches are chained by programmatic dependent launch outside stream capture: a kernel fills its weight rings while
+// its predecessor still runs, and waits for it before it reads the rows or writes anything.  (Replayed from a CUDA
+// graph the same chain was slower than plain edges, so a capturing stream gets ordinary launches.)
 #include <cooperative_groups.h>
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "cast_math.cuh"
 #include "cp_async.cuh"
-#include "decode_math.cuh"
 #include "gemm.cuh"
 
 namespace cg = cooperative_groups;
@@ -42,233 +49,641 @@ namespace cg = cooperative_groups;
 namespace amx {
 namespace {
 
-using namespace decode;
-
-constexpr int kMaxRows = 16;                 // token rows of one tile (the M side of one MMA)
-constexpr int kMaxRowTiles = 4;              // up to 64 token rows
 constexpr int kWarps = 8, kThreads = kWarps * 32;
-constexpr int kTiles = 2;                    // 8-row weight tiles per warp
-constexpr int kCtaRows = kWarps * kTiles * 8;   // 128 weight rows per CTA
-constexpr int kStepK = 128;                  // elements of K per step: one group per lane of a quad
-constexpr int kStepBytes = kMaxRows * kStepK * 2;   // activation fragments of one step: 4 KB
-constexpr int kMaxSlices = 8;                // portable cluster size
-constexpr int kPartPitch = 136;              // floats per token row of the partial-product tile (bank spread)
+constexpr int kRowGroups = 4, kStepGroups = 2;     // warps: 4 groups of 32 weight rows x 2 step parities
+constexpr int kCtaRows = kRowGroups * 32;
+constexpr int kStepK = 128;
+constexpr int kTok = 8;                            // token rows of one tile (the N side of one MMA)
+constexpr int kFragBytes = kTok * kStepK * 2;      // fragments of one tile and step
+constexpr int kCodeBytes = 4 * 512;                // codes of 32 rows and one step: 4 pieces of 16 bytes per lane
+constexpr int kMaxSlices = 8;                      // portable cluster size
+constexpr int kPartPitch = kCtaRows + 4;           // floats per token row of the partial-product tile (bank spread)
+constexpr int kMaxTiles = 8;                       // token tiles per CTA
+constexpr int kScaleSteps = 32;                    // steps whose scales are held at a time
 
-// Fragment order of the decoded activation, per step of 128 elements: [row tile mt][unit j = 0..3][half 0..1]
-// [lane 0..31] pieces of 16 bytes; the piece of lane (g, t) holds elements 8j .. 8j+7 of group 4 * step + t of row
-// 16 * mt + 8 * half + g (in the pair order and scaling of pair_order_scaled).  mts = row tiles (1, 2 or 4).
-__device__ __forceinline__ int64_t fragment_piece(int64_t step, int mts, int mt, int j, int half, int g, int t) {
-    return ((((step * mts + mt) * 4 + j) * 2 + half) * 32) + g * 4 + t;
-}
-
-// The streaming kernel decodes a word of eight weight codes into the bf16 pairs (e0, e4), (e1, e5), (e2, e6),
-// (e3, e7), each value 2^-63 times the true one (decode_pairs in decode_math.cuh); the activation pieces are stored in the same
-// pair order and multiplied by 2^63, so that every product is the true one.  Both scalings are exact: a decoded
-// value times 2^+-63 stays far inside the bf16 range.
-__device__ __forceinline__ uint4 pair_order_scaled(uint4 o) {      // o: pairs (e0,e1), (e2,e3), (e4,e5), (e6,e7)
-    const uint32_t two63 = 0x5F005F00u;
-    uint4 r;
-    r.x = mul_bf16x2(prmt(o.x, o.z, 0x5410), two63);
-    r.y = mul_bf16x2(prmt(o.x, o.z, 0x7632), two63);
-    r.z = mul_bf16x2(prmt(o.y, o.w, 0x5410), two63);
-    r.w = mul_bf16x2(prmt(o.y, o.w, 0x7632), two63);
-    return r;
-}
-
-// One thread per 8 elements of the slab of 16 * mts rows (four adjacent lanes share a 32-element group and
-// exchange their side maxima with two shuffles): decode, or cast then decode (CAST), and write one 16-byte piece.
-// Rows past M are written as zeros.  The kernel is a few thousand threads of pure latency, so the work of a group
-// is spread over lanes instead of being one long dependent chain.
 // griddepcontrol.wait: returns once every grid this one programmatically depends on has completed and its writes
 // are visible (at once when the launch carried no such dependency).  griddepcontrol.launch_dependents: the grid
 // launched behind this one with programmatic serialization may start once every CTA here has said so or exited.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-template <bool CAST>
+__device__ __forceinline__ __half2 h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
+__device__ __forceinline__ uint32_t u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
+
+// The two side scales of a group as f16 pairs times 2^-4.  An E5M2 byte is the upper byte of the same half.
+struct Scales {
+    __half2 pos, neg;
+};
+__device__ __forceinline__ Scales make_scales(uint32_t sc) {
+    const __half2 down = h2(0x2C002C00u);                            // 2^-4
+    return {__hmul2(h2(__byte_perm(sc, 0, 0x0404)), down), __hmul2(h2(__byte_perm(sc, 0, 0x1414)), down)};
+}
+// Two elements from byte I of a code word.
+template <int I>
+__device__ __forceinline__ uint32_t decode_pair(uint32_t w, const Scales& s) {
+    uint32_t v;
+    if (I == 0) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, a;}" : "=r"(v) : "r"(w));
+    if (I == 1) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, b;}" : "=r"(v) : "r"(w));
+    if (I == 2) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, c;}" : "=r"(v) : "r"(w));
+    if (I == 3) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, d;}" : "=r"(v) : "r"(w));
+    uint32_t pos;
+    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(pos) : "r"(v), "r"(u32(s.pos)), "r"(0u));
+    return u32(__hfma2(__hmin2(h2(v), h2(0u)), s.neg, h2(pos)));
+}
+__device__ __forceinline__ uint4 decode_word(uint32_t w, const Scales& s) {
+    return make_uint4(decode_pair<0>(w, s), decode_pair<1>(w, s), decode_pair<2>(w, s), decode_pair<3>(w, s));
+}
+
+// Fragment order of the token rows, per step and tile of 8 rows: pieces of 16 bytes [j = 0..3][lane 0..31]; the piece
+// of (j, lane (g, t)) holds elements 32 t + 8 j .. + 7 of the step, row g of the tile.  Piece (j, l) sits at position
+// l ^ (2 j): the casting lanes (same row, consecutive pieces of 8 elements) then hit eight bank groups.
+__device__ __forceinline__ int frag_pos(int j, int l) { return j * 32 + (l ^ (2 * j)); }
+
+// 8 consecutive elements of a row cast and decoded; TPG lanes hold one group.
+template <int TPG>
+__device__ __forceinline__ uint4 cast_piece(const uint4 q) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    uint32_t c = cast::side_maxima<4>(w);
+#pragma unroll
+    for (int d = 1; d < TPG; d <<= 1) c = __vmaxs2(c, __shfl_xor_sync(0xFFFFFFFFu, c, d));
+    float inv_p, inv_n;
+    const uint32_t sc = cast::group_scales(c, inv_p, inv_n);
+    return decode_word(cast::encode8(w, inv_p, inv_n), make_scales(sc));
+}
+
+// One thread per piece of 8 elements (grid y: the row).  Rows past M are zeros.  The kernel is a few thousand threads of
+// pure latency, so a group's work is spread over lanes.
+template <bool CAST, int GS>
 __global__ void __launch_bounds__(128) rows_fragments_kernel(const uint8_t* __restrict__ codes,
                                                              const uint8_t* __restrict__ scales,
                                                              const uint16_t* __restrict__ x, int64_t ld_x, int M,
-                                                             int mts, int64_t K, uint4* __restrict__ frag,
+                                                             int tiles, int64_t K, uint4* __restrict__ frag,
                                                              int* __restrict__ status) {
-    const int64_t groups = K / 32;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t per_row = K / 8;
+    const int64_t k8 = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int row = blockIdx.y;
     grid_dependency_wait();                    // the previous call on this stream may still read the workspace
-    grid_launch_dependents();                  // the streaming kernel may start filling its rings
-    if (idx == 0) status[0] = status[1] = 0;   // no device-side wait that can expire, no scale is flushed: both words read 0
-    const bool live = idx < groups * 4 * kMaxRows * mts;           // whole groups: the four lanes agree
-    const int j = (int)(idx & 3);
-    const int64_t gidx = idx >> 2;
-    const int row = live ? (int)(gidx / groups) : M;
-    const int64_t grp = gidx % groups;
-    uint32_t word = 0, sc = 0;
+    grid_launch_dependents();                  // the main kernel may start filling its rings
+    if (k8 == 0 && row == 0) status[0] = status[1] = 0;   // no device-side wait that can expire, no scale is flushed
+    const bool live = k8 < per_row, seen = live && row < M;
+    uint4 out = make_uint4(0, 0, 0, 0);
     if (CAST) {
-        uint32_t w[4] = {0, 0, 0, 0};
-        if (row < M) {
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(x + row * ld_x + grp * 32) + j);
-            w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
-        }
-        uint32_t c = cast::side_maxima<4>(w);
-        c = __vmaxs2(c, __shfl_xor_sync(0xFFFFFFFFu, c, 1));
-        c = __vmaxs2(c, __shfl_xor_sync(0xFFFFFFFFu, c, 2));
-        float inv_p, inv_n;
-        sc = cast::group_scales(c, inv_p, inv_n);
-        word = cast::encode8(w, inv_p, inv_n);
-    } else if (row < M) {
-        word = __ldg(reinterpret_cast<const uint32_t*>(codes + (row * groups + grp) * 16) + j);
-        sc = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * groups + grp) * 2));
+        uint4 q = make_uint4(0, 0, 0, 0);
+        if (seen) q = __ldg(reinterpret_cast<const uint4*>(x + row * ld_x + k8 * 8));
+        out = cast_piece<GS / 8>(q);           // zeros cast to zeros
+    } else if (seen) {
+        const uint32_t word = __ldg(reinterpret_cast<const uint32_t*>(codes + row * (K / 2) + k8 * 4));
+        const uint32_t sc = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * (K / GS) + k8 * 8 / GS) * 2));
+        out = decode_word(word, make_scales(sc));
     }
     if (!live) return;
-    const GroupTables tb = make_tables(sc);
-    const int64_t step = grp >> 2;
-    const int t = (int)(grp & 3), g = row & 7, half = (row >> 3) & 1, mt = row >> 4;
-    frag[fragment_piece(step, mts, mt, j, half, g, t)] = pair_order_scaled(decode_word(word, tb));
+    const int64_t step = k8 >> 4;
+    const int j = (int)k8 & 3, t = (int)(k8 >> 2) & 3;
+    frag[(step * tiles + (row >> 3)) * 128 + frag_pos(j, (row & 7) * 4 + t)] = out;
 }
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Shared memory of a CTA: one ring of kDepth steps per warp for the weight stream.  A ring slot holds, per 8-row
-// tile, the 32 lanes' 16 bytes of codes and 4 bytes of scales (the two groups 4 * step + 2 * (t / 2) + {0, 1}; the
-// lane uses the half t % 2).  Every lane reads back only what its own copies wrote, so the ring needs no barrier,
-// only the lane's own wait.
-constexpr int kDepth = 4;
-constexpr int kSlotCodes = kTiles * 32 * 16, kSlotBytes = kSlotCodes + kTiles * 32 * 4;
-constexpr int kRingBytes = kDepth * kSlotBytes;   // per warp
-constexpr int kSmemBytes = kWarps * kRingBytes;
-static_assert(4 * kMaxRows * kPartPitch * 4 <= kWarps * kRingBytes, "the partial-product tile reuses the rings");
+struct RowsParams {
+    const uint16_t* x;           // CAST: bf16 rows [M, ld_x]
+    int64_t ld_x;
+    const uint4* frag;           // otherwise: fragments [step][tiles of all rows]
+    const uint8_t *w_codes, *w_scales;
+    int M;
+    int64_t N, K;
+    float* C;
+    int64_t ld_c;
+    int steps_max;               // steps of the longest range
+    int* status;                 // CAST: the two status words of the workspace (or nullptr), cleared here
+};
 
-// MT: tiles of 16 token rows (1, 2 or 4).  The decoded weight registers of a step are used by every row tile.
-template <int MT>
-__global__ void __launch_bounds__(kThreads, MT == 1 ? 4 : 2) gemm_rows_kernel(const uint4* __restrict__ frag,
-                                                                const uint8_t* __restrict__ w_codes,
-                                                                const uint8_t* __restrict__ w_scales, int M, int64_t N,
-                                                                int64_t K, float* __restrict__ C, int64_t ld_c) {
+// Shared-memory geometry.  kDepth ring slots per warp (kDepth - 1 steps in flight); with up to four token tiles two
+// CTAs share an SM, which is what keeps enough of the weight in flight.
+template <int NT, int GS>
+struct Ring {
+    static constexpr int kDepth = NT == 3 || NT == 4 ? 3 : 4;
+    static constexpr int kFragSlot = NT * kFragBytes;
+    static constexpr int kBytes = kWarps * kDepth * kCodeBytes;
+    static constexpr int kFragRing = kStepGroups * kDepth * kFragSlot;
+    static constexpr int kPart = NT * kTok * kPartPitch * 4;
+    static_assert(kPart <= kBytes, "the partial-product tile reuses the rings");
+};
+// Scales of one weight row over `n` steps: 4-byte words copied (groups of 128: two bytes per step, copied as the aligned
+// words around them), and the pitch of the rows in shared memory - twice an odd number of words, so that the words of
+// eight rows that a warp reads together lie in different banks (groups of 16: four words per step, four times an odd number).
+__host__ __device__ constexpr int scale_words(int n, int gs) { return gs == 128 ? n / 2 + 1 : n * (64 / gs); }
+__host__ __device__ constexpr int scale_pitch(int n, int gs) {
+    return gs == 16 ? (n | 1) * 4 : gs == 32 ? (n | 1) * 2 : gs == 64 ? (n | 1) : (n / 2 + 1) | 1;
+}
+__host__ __device__ constexpr int scale_bytes(int n, int gs) { return (kCtaRows * scale_pitch(n, gs) * 4 + 15) / 16 * 16; }
+
+// NT: tiles of 8 token rows per CTA.
+template <int NT, bool CAST, int GS>
+__global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(const RowsParams p) {
+    using R = Ring<NT, GS>;
+    constexpr int kDepth = R::kDepth, kFragSlot = R::kFragSlot;
     extern __shared__ __align__(16) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int slices = (int)gridDim.y, slice = (int)blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int64_t groups = K / 32, steps = K / kStepK;
+    const int wr = warp & 3, wk = warp >> 2;
+    const int64_t steps = p.K / kStepK;
     const int64_t s_begin = steps * slice / slices;
     const int n_total = (int)(steps * (slice + 1) / slices - s_begin);
-    const int64_t row0 = (int64_t)blockIdx.x * kCtaRows + warp * (kTiles * 8);
+    const int64_t row0 = (int64_t)blockIdx.x * kCtaRows;
+    const int m0 = (int)blockIdx.z * (NT * kTok);
 
-    // this lane's stream positions at step s_begin: codes of group 4 * step + t, scales of the group pair
-    const uint8_t* pc[kTiles];
-    const uint8_t* ps[kTiles];
+    uint8_t* ring = smem + warp * (kDepth * kCodeBytes);
+    const int held = min(p.steps_max, kScaleSteps), pitch = scale_pitch(held, GS);
+    uint32_t* scale_s = reinterpret_cast<uint32_t*>(smem + R::kBytes);
+    uint8_t* frag_s = smem + R::kBytes + scale_bytes(held, GS);      // CAST: the range's fragments; else a ring per step parity
+
+    // this lane's streams: piece t of rows g, g + 8 (block 0), g + 16, g + 24 (block 1) of the warp's 32 rows
+    const uint8_t* pc[4];
+    int odd[4];                                // groups of 128: which half of its word a row's first scale is
 #pragma unroll
-    for (int i = 0; i < kTiles; ++i) {
-        int64_t r = row0 + i * 8 + g;
-        r = r < N ? r : N - 1;               // rows past the weight read its last row; their sums are not stored
-        pc[i] = w_codes + (r * groups + s_begin * 4 + t) * 16;
-        ps[i] = w_scales + (r * groups + s_begin * 4 + (t & 2)) * 2;
+    for (int q = 0; q < 4; ++q) {
+        int64_t r = row0 + wr * 32 + q * 8 + g;
+        r = r < p.N ? r : p.N - 1;             // rows past the weight read its last row; their sums are not stored
+        pc[q] = p.w_codes + r * (p.K / 2) + s_begin * 64 + t * 16;
+        odd[q] = GS == 128 ? (int)((r * steps + s_begin) & 1) : 0;
     }
-    uint8_t* ring = smem + warp * kRingBytes;
-    auto issue = [&](int step) {             // step relative to s_begin; one commit group per call
-        if (step < n_total) {
-            uint8_t* slot = ring + (step % kDepth) * kSlotBytes;
+    const int n_mine = (n_total - wk + 1) / kStepGroups;             // this warp's steps: wk, wk + 2, ...
+    auto issue_codes = [&](int i) {
+        if (i < n_mine) {
+            uint8_t* slot = ring + (i % kDepth) * kCodeBytes + lane * 16;
+            const int64_t off = (int64_t)(wk + i * kStepGroups) * 64;
 #pragma unroll
-            for (int i = 0; i < kTiles; ++i) {
-                cp_async16(slot + i * 512 + lane * 16, pc[i] + (int64_t)step * 64);
-                cp_async4(slot + kSlotCodes + i * 128 + lane * 4, ps[i] + (int64_t)step * 8);
-            }
+            for (int q = 0; q < 4; ++q) cp_async16(slot + q * 512, pc[q] + off);
         }
-        cp_async_commit();
     };
-#pragma unroll
-    for (int d = 0; d < kDepth; ++d) issue(d);
-    grid_launch_dependents();                // whatever follows waits for this grid's completion by itself
-    grid_dependency_wait();                  // the fragments (and the previous user of C) are complete from here on
-
-    float acc[MT][kTiles][4];
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int i = 0; i < kTiles; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[mt][i][j] = 0.f;
-
-    for (int step = 0; step < n_total; ++step) {
-        const uint4* a = frag + (s_begin + step) * (MT * kStepBytes / 16) + lane;
-        uint4 a_lo[4], a_hi[4];                                  // rows g and g + 8 of a tile, elements 8j .. 8j + 7
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            a_lo[j] = __ldg(a + (j * 2) * 32);
-            a_hi[j] = __ldg(a + (j * 2 + 1) * 32);
+    // scales of steps [first, first + n) of the range, all 128 rows: consecutive threads copy consecutive words of a row
+    auto issue_scales = [&](int first, int n) {
+        const int words = scale_words(n, GS);
+        for (int i = threadIdx.x; i < kCtaRows * words; i += kThreads) {
+            const int r_in = i / words, w = i - r_in * words;
+            int64_t r = row0 + r_in;
+            r = r < p.N ? r : p.N - 1;
+            const uint8_t* src = p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2;
+            if (GS == 128) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
+            cp_async4(scale_s + r_in * pitch + w, src + w * 4);
         }
-        cp_async_wait<kDepth - 1>();                             // this step's group has landed
-        const uint8_t* slot = ring + (step % kDepth) * kSlotBytes;
-        uint4 b[kTiles][4];
+    };
+    auto issue_frags = [&](int i) {            // the four warps of a step parity share the copies
+        if (i < n_mine) {
+            uint8_t* slot = frag_s + (wk * kDepth + i % kDepth) * kFragSlot;
+            const int tiles_all = (int)gridDim.z * NT;
+            const uint4* src = p.frag + ((s_begin + wk + i * kStepGroups) * tiles_all + (int)blockIdx.z * NT) * 128;
 #pragma unroll
-        for (int i = 0; i < kTiles; ++i) {
-            const uint4 cw = *reinterpret_cast<const uint4*>(slot + i * 512 + lane * 16);
-            const uint32_t sw = *reinterpret_cast<const uint32_t*>(slot + kSlotCodes + i * 128 + lane * 4);
-            const GroupScales gs = make_scales((t & 1) ? sw >> 16 : sw & 0xFFFFu);
-            const uint32_t w[4] = {cw.x, cw.y, cw.z, cw.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[i][j] = decode_pairs(w[j], gs);
+            for (int q = 0; q < NT; ++q) cp_async16(slot + (q * 128 + wr * 32 + lane) * 16, src + q * 128 + wr * 32 + lane);
         }
+    };
+    issue_scales(0, min(n_total, kScaleSteps));    // part of the first copy group
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            if (mt > 0) {
+    for (int d = 0; d < kDepth - 1; ++d) {
+        issue_codes(d);
+        cp_async_commit();
+    }
+    grid_launch_dependents();                  // whatever follows waits for this grid's completion by itself
+    grid_dependency_wait();                    // the rows (and the previous user of C) are complete from here on
+    if (CAST) {
+        if (p.status && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 2) p.status[threadIdx.x] = 0;
+        // Tokens over warps; with fewer than eight tokens, `parts` warps share a token's K range.
+        const int n_tok = NT * kTok, live_tok = min(n_tok, p.M - m0);
+        auto put_piece = [&](int tok, int k8, const uint4& v) {
+            *reinterpret_cast<uint4*>(frag_s + (k8 >> 4) * kFragSlot + (tok >> 3) * kFragBytes +
+                                      frag_pos(k8 & 3, (tok & 7) * 4 + ((k8 >> 2) & 3)) * 16) = v;
+        };
+        int parts = 1;
+        if (NT == 1)
+            while (parts < 8 && live_tok * parts * 2 <= 8) parts *= 2;
+        for (int tok = warp / parts; tok < live_tok; tok += kWarps / parts) {
+            const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)(m0 + tok) * p.ld_x + s_begin * kStepK);
+            for (int k0 = (warp % parts) * 32; k0 < n_total * 16; k0 += parts * 32) {
+                const int k8 = k0 + lane;
+                uint4 q = make_uint4(0, 0, 0, 0);
+                if (k8 < n_total * 16) q = __ldg(src + k8);
+                const uint4 v = cast_piece<GS / 8>(q);
+                if (k8 < n_total * 16) put_piece(tok, k8, v);
+            }
+        }
+        for (int tok = live_tok + warp; tok < n_tok; tok += kWarps)          // rows past M
+            for (int k8 = lane; k8 < n_total * 16; k8 += 32) put_piece(tok, k8, make_uint4(0, 0, 0, 0));
+        cp_async_wait<kDepth - 2>();           // the first group: the scales
+    } else {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    a_lo[j] = __ldg(a + ((mt * 4 + j) * 2) * 32);
-                    a_hi[j] = __ldg(a + ((mt * 4 + j) * 2 + 1) * 32);
+        for (int d = 0; d < kDepth - 1; ++d) {
+            issue_frags(d);
+            cp_async_commit();
+        }
+        cp_async_wait<2 * kDepth - 3>();       // the first group
+    }
+    __syncthreads();
+
+    float acc[2][NT][4];
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[b][n][j] = 0.f;
+
+    int scale_first = 0;                       // first step whose scales are held
+    for (int i = 0; i < (n_total + 1) / kStepGroups; ++i) {
+        const int ls = wk + i * kStepGroups;
+        if (i * kStepGroups - scale_first == kScaleSteps) {      // a long range: the next steps' scales (all warps together)
+            scale_first += kScaleSteps;
+            __syncthreads();
+            issue_scales(scale_first, min(n_total - scale_first, kScaleSteps));
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncthreads();
+        }
+        if (i >= n_mine) break;                // an odd range: one step less for the second parity
+        cp_async_wait<kDepth - 2>();           // this step's copies have landed
+        if (!CAST) {                           // the fragments are visible to the parity's four warps, last step's slots free
+            if (wk == 0) asm volatile("bar.sync 1, %0;" ::"n"(kRowGroups * 32) : "memory");
+            else asm volatile("bar.sync 2, %0;" ::"n"(kRowGroups * 32) : "memory");
+        }
+        issue_codes(i + kDepth - 1);
+        if (!CAST) issue_frags(i + kDepth - 1);
+        cp_async_commit();
+        const uint8_t* slot = ring + (i % kDepth) * kCodeBytes;
+        const uint8_t* fs = CAST ? frag_s + ls * kFragSlot : frag_s + (wk * kDepth + i % kDepth) * kFragSlot;
+        uint4 cw[4];
+        uint32_t sc[4];                        // the scale bytes of the lane's group (groups of 16: of both)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            cw[q] = *reinterpret_cast<const uint4*>(slot + q * 512 + lane * 16);
+            const uint32_t* w = scale_s + (wr * 32 + q * 8 + g) * pitch;
+            const int s_in = ls - scale_first;
+            if (GS == 16) sc[q] = w[s_in * 4 + t];
+            else if (GS == 32) sc[q] = w[s_in * 2 + (t >> 1)] >> (16 * (t & 1));
+            else if (GS == 64) sc[q] = w[s_in] >> (16 * (t >> 1));
+            else {                             // the first held step may start in the upper half of its word
+                const int h = odd[q] + s_in;
+                sc[q] = w[h >> 1] >> (16 * (h & 1));
+            }
+        }
+        Scales s[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {          // pieces of 8 elements of the lane's 32
+            if (j == 0 || (GS == 16 && j == 2)) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = make_scales(j ? sc[q] >> 16 : sc[q]);
+            }
+            uint4 b[NT];
+#pragma unroll
+            for (int n = 0; n < NT; ++n) b[n] = *reinterpret_cast<const uint4*>(fs + n * kFragBytes + frag_pos(j, lane) * 16);
+#pragma unroll
+            for (int blk = 0; blk < 2; ++blk) {
+                const uint32_t w0 = j == 0 ? cw[2 * blk].x : j == 1 ? cw[2 * blk].y : j == 2 ? cw[2 * blk].z : cw[2 * blk].w;
+                const uint32_t w1 = j == 0 ? cw[2 * blk + 1].x : j == 1 ? cw[2 * blk + 1].y : j == 2 ? cw[2 * blk + 1].z : cw[2 * blk + 1].w;
+                const uint4 a0 = decode_word(w0, s[2 * blk]), a1 = decode_word(w1, s[2 * blk + 1]);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    mma_f16(acc[blk][n], a0.x, a1.x, a0.y, a1.y, b[n].x, b[n].y);
+                    mma_f16(acc[blk][n], a0.z, a1.z, a0.w, a1.w, b[n].z, b[n].w);
                 }
             }
-#pragma unroll
-            for (int i = 0; i < kTiles; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    mma_bf16(acc[mt][i], a_lo[j].x, a_hi[j].x, a_lo[j].y, a_hi[j].y, b[i][j].x, b[i][j].y);
-                    mma_bf16(acc[mt][i], a_lo[j].z, a_hi[j].z, a_lo[j].w, a_hi[j].w, b[i][j].z, b[i][j].w);
-                }
         }
-        issue(step + kDepth);                                    // refill the slot just consumed
     }
     cp_async_wait<0>();
 
-    // Partial products of this range of K: [16 token rows][128 weight rows] in shared memory (over the rings, which
-    // are drained), then every CTA of
-    // the cluster adds its share of the outputs over all ranks, in rank order.
+    // Partial products [token][128 weight rows] in shared memory (over the rings, which are drained): odd steps first,
+    // even steps added on top, then every CTA of the cluster adds its share of the outputs over all ranks, in rank order.
     __syncthreads();
     float* part = reinterpret_cast<float*>(smem);
+    auto at = [&](int blk, int n, int j) -> float& {
+        return part[(n * kTok + 2 * t + (j & 1)) * kPartPitch + wr * 32 + blk * 16 + (j >> 1) * 8 + g];
+    };
+    if (wk == 1)
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
-        for (int i = 0; i < kTiles; ++i) {
-            const int col = warp * (kTiles * 8) + i * 8 + 2 * t;
-            *reinterpret_cast<float2*>(part + (mt * 16 + g) * kPartPitch + col) = make_float2(acc[mt][i][0], acc[mt][i][1]);
-            *reinterpret_cast<float2*>(part + (mt * 16 + g + 8) * kPartPitch + col) = make_float2(acc[mt][i][2], acc[mt][i][3]);
-        }
-    cluster.sync();
-    const int per = MT * kMaxRows * kCtaRows / slices;           // outputs this CTA adds up (a multiple of 256)
-    for (int o = slice * per + threadIdx.x; o < (slice + 1) * per; o += kThreads) {
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) at(b, n, j) = acc[b][n][j];
+    __syncthreads();
+    if (wk == 0)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int n = 0; n < NT; ++n)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) at(b, n, j) += acc[b][n][j];
+    if (slices > 1) cluster.sync();
+    else __syncthreads();
+    const int outputs = min(NT * kTok, p.M - m0) * kCtaRows;
+    for (int o = slice * kThreads + threadIdx.x; o < outputs; o += slices * kThreads) {
         const int m = o / kCtaRows, col = o % kCtaRows;
-        float v[kMaxSlices];
-#pragma unroll
-        for (int r = 0; r < kMaxSlices; ++r)                     // all remote reads in flight together
-            v[r] = r < slices ? cluster.map_shared_rank(part, r)[m * kPartPitch + col] : 0.f;
         float sum = 0.f;
+        if (slices > 1) {
+            float v[kMaxSlices];
 #pragma unroll
-        for (int r = 0; r < kMaxSlices; ++r) sum += v[r];
-        const int64_t n = (int64_t)blockIdx.x * kCtaRows + col;
-        if (m < M && n < N) C[m * ld_c + n] = sum;
+            for (int r = 0; r < kMaxSlices; ++r)                     // all remote reads in flight together
+                v[r] = r < slices ? cluster.map_shared_rank(part, r)[m * kPartPitch + col] : 0.f;
+#pragma unroll
+            for (int r = 0; r < kMaxSlices; ++r) sum += v[r];
+        } else sum = part[m * kPartPitch + col];
+        const int64_t n = row0 + col;
+        if (n < p.N) p.C[(int64_t)(m0 + m) * p.ld_c + n] = sum * 256.0f;
     }
-    cluster.sync();                                              // no CTA leaves while its tile is still read
+    if (slices > 1) cluster.sync();                                  // no CTA leaves while its tile is still read
 }
 
-using RowsKernel = void (*)(const uint4*, const uint8_t*, const uint8_t*, int, int64_t, int64_t, float*, int64_t);
+// ---- few rows (up to four token tiles): a CTA of eight warps covers 32 weight rows, its warps split the K range.
+// No cluster for the usual layers (enough rows to fill the SMs), three CTAs on an SM, so a chain of calls keeps the weight
+// stream going: the CTAs of the next call move in one by one as this call's leave.  (With 128 rows per CTA and a cluster
+// over K, 288 CTAs did not all fit - clusters of three leave slots empty in every GPC - and a second wave of a few
+// clusters doubled the time; clusters of four were packed on two thirds of the SMs.)  A warp's steps are consecutive, so
+// its scales come along the rows, four steps (32 bytes per row with groups of 32) at a time.
+constexpr int kStreamRows = 32, kScaleSlotSteps = 4;
 
-// Row tiles for M token rows (1, 2 or 4) and the kernel instantiation for them.
-int row_tiles(int64_t M) { return M <= kMaxRows ? 1 : M <= 2 * kMaxRows ? 2 : 4; }
-RowsKernel kernel_for_tiles(int mts) {
-    return mts == 1 ? gemm_rows_kernel<1> : mts == 2 ? gemm_rows_kernel<2> : gemm_rows_kernel<4>;
+template <int GS>
+struct StreamRing {
+    static constexpr int kDepth = 3;
+    static constexpr int kWords = GS == 128 ? 3 : kScaleSlotSteps * 64 / GS;      // scale words per row and slot (128: aligned around)
+    // Words of eight rows in different banks: an odd pitch (in units of the words a quad reads together), or rows of 8
+    // words whose halves are exchanged on every other four rows.
+    static constexpr int kPitch = GS == 16 ? 20 : GS == 32 ? 8 : GS == 64 ? 5 : 3;
+    __device__ static int at(int r, int w) { return r * kPitch + (GS == 32 ? w ^ (r & 4) : w); }
+    static constexpr int kScaleBytes = kStreamRows * kPitch * 4;                  // one slot; two per warp
+    static constexpr int kWarpBytes = kDepth * kCodeBytes + 2 * kScaleBytes;
+    static constexpr int kBytes = kWarps * kWarpBytes;
+};
+
+template <int NT, bool CAST, int GS>
+__global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_kernel(const RowsParams p) {
+    using R = StreamRing<GS>;
+    constexpr int kDepth = R::kDepth;
+    static_assert(!CAST || NT == 1, "rows are cast inside for one tile only");
+    extern __shared__ __align__(16) uint8_t smem[];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int slices = (int)gridDim.y, slice = (int)blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int64_t steps = p.K / kStepK;
+    const int64_t cta_begin = steps * slice / slices, cta_steps = steps * (slice + 1) / slices - cta_begin;
+    const int64_t w_first = cta_steps * warp / kWarps;               // this warp's steps inside the CTA's range
+    const int n = (int)(cta_steps * (warp + 1) / kWarps - w_first);
+    const int64_t s_begin = cta_begin + w_first;
+    const int64_t row0 = (int64_t)blockIdx.x * kStreamRows;
+
+    uint8_t* ring = smem + warp * R::kWarpBytes;
+    uint8_t* scale_ring = ring + kDepth * kCodeBytes;
+    uint8_t* frag_s = smem + R::kBytes;        // CAST: the live rows' fragments of the CTA's range
+
+    // piece t of rows g, g + 8 (block 0), g + 16, g + 24 (block 1).  Rows past the weight are not copied: what their
+    // slots hold only reaches sums that are not stored.
+    const uint8_t* pc = p.w_codes + (row0 + g) * (p.K / 2) + s_begin * 64 + t * 16;
+    const int64_t rows8 = p.K * 4;             // bytes between rows 8 apart
+    const int rows_left = (int)min((int64_t)kStreamRows, p.N - row0);
+    auto issue = [&](int i) {
+        if (i < n) {
+            uint8_t* slot = ring + (i % kDepth) * kCodeBytes + lane * 16;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q * 8 + g < rows_left) cp_async16(slot + q * 512, pc + q * rows8 + (int64_t)i * 64);
+        }
+    };
+    auto issue_scales = [&](int slot) {
+        const int first = slot * kScaleSlotSteps;
+        if (first >= n) return;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(scale_ring + (slot & 1) * R::kScaleBytes);
+        // words past the warp's last step may lie past the end of the tensor
+        const int words = min(R::kWords, GS == 128 ? (min(n - first, kScaleSlotSteps)) / 2 + 1 : (n - first) * (64 / GS));
+#pragma unroll
+        for (int i = 0; i < (kStreamRows * R::kWords + 31) / 32; ++i) {
+            const int item = i * 32 + lane, r_in = item / R::kWords, w = item - r_in * R::kWords;
+            int64_t r = row0 + r_in;
+            r = r < p.N ? r : p.N - 1;
+            const uint8_t* src = p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2;
+            if (GS == 128) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
+            if (w < words) cp_async4(dst + R::at(r_in, w), src + w * 4);
+        }
+    };
+    issue_scales(0);
+#pragma unroll
+    for (int d = 0; d < kDepth - 1; ++d) {
+        issue(d);
+        cp_async_commit();
+    }
+    grid_launch_dependents();                  // whatever follows waits for this grid's completion by itself
+    grid_dependency_wait();                    // the rows (and the previous user of C) are complete from here on
+    const int m0 = (int)blockIdx.z * (NT * kTok), live_tok = min(NT * kTok, p.M - m0);
+    if (CAST) {                                // (one block of tokens: m0 = 0)
+        if (p.status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) p.status[threadIdx.x] = 0;
+        // pieces of 8 elements, all loads of a thread's next four in flight together
+        const int pieces = (int)cta_steps * 16;
+        for (int tok = 0; tok < live_tok; ++tok) {
+            const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)tok * p.ld_x + cta_begin * kStepK);
+            for (int k0 = warp * 32; k0 < pieces; k0 += 4 * kThreads) {
+                uint4 q[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k8 = k0 + i * kThreads + lane;
+                    q[i] = k8 < pieces ? __ldg(src + k8) : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k8 = k0 + i * kThreads + lane;
+                    if (k8 - lane >= pieces) break;                  // uniform over the warp
+                    const uint4 v = cast_piece<GS / 8>(q[i]);
+                    // [step][j][token][t] pieces of 16 bytes
+                    if (k8 < pieces)
+                        *reinterpret_cast<uint4*>(frag_s + ((((k8 >> 4) * 4 + (k8 & 3)) * live_tok + tok) * 4 + ((k8 >> 2) & 3)) * 16) = v;
+                }
+            }
+        }
+        __syncthreads();
+    }
+
+    float acc[2][NT][4];
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int m = 0; m < NT; ++m)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[b][m][j] = 0.f;
+
+    for (int i = 0; i < n; ++i) {
+        cp_async_wait<kDepth - 2>();           // this step's copies have landed
+        __syncwarp();                          // the scales are read across lanes
+        if ((i & (kScaleSlotSteps - 1)) == 0) issue_scales(i / kScaleSlotSteps + 1);
+        issue(i + kDepth - 1);
+        cp_async_commit();
+        const uint8_t* slot = ring + (i % kDepth) * kCodeBytes;
+        const uint32_t* sw = reinterpret_cast<const uint32_t*>(scale_ring + ((i / kScaleSlotSteps) & 1) * R::kScaleBytes);
+        const int s_in = i & (kScaleSlotSteps - 1);
+        uint4 cw[4];
+        uint32_t sc[4];                        // the scale bytes of the lane's group (groups of 16: of both)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            cw[q] = *reinterpret_cast<const uint4*>(slot + q * 512 + lane * 16);
+            const int r_in = q * 8 + g;
+            if (GS == 16) sc[q] = sw[R::at(r_in, s_in * 4 + t)];
+            else if (GS == 32) sc[q] = sw[R::at(r_in, s_in * 2 + (t >> 1))] >> (16 * (t & 1));
+            else if (GS == 64) sc[q] = sw[R::at(r_in, s_in)] >> (16 * (t >> 1));
+            else {                             // the slot's first step may start in the upper half of its word
+                const int h = (int)((min(row0 + r_in, p.N - 1) * steps + s_begin + (i - s_in)) & 1) + s_in;
+                sc[q] = sw[R::at(r_in, h >> 1)] >> (16 * (h & 1));
+            }
+        }
+        Scales s[4];
+        const uint4* fg = p.frag + ((s_begin + i) * gridDim.z + blockIdx.z) * (NT * 128);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {          // pieces of 8 elements of the lane's 32
+            if (j == 0 || (GS == 16 && j == 2)) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = make_scales(j ? sc[q] >> 16 : sc[q]);
+            }
+            uint4 b[NT];
+            if (CAST) {
+                b[0] = make_uint4(0, 0, 0, 0);
+                if (g < live_tok)
+                    b[0] = *reinterpret_cast<const uint4*>(frag_s + ((((w_first + i) * 4 + j) * live_tok + g) * 4 + t) * 16);
+            } else {
+#pragma unroll
+                for (int m = 0; m < NT; ++m) b[m] = __ldg(fg + m * 128 + frag_pos(j, lane));
+            }
+#pragma unroll
+            for (int blk = 0; blk < 2; ++blk) {
+                const uint32_t w0 = j == 0 ? cw[2 * blk].x : j == 1 ? cw[2 * blk].y : j == 2 ? cw[2 * blk].z : cw[2 * blk].w;
+                const uint32_t w1 = j == 0 ? cw[2 * blk + 1].x : j == 1 ? cw[2 * blk + 1].y : j == 2 ? cw[2 * blk + 1].z : cw[2 * blk + 1].w;
+                const uint4 a0 = decode_word(w0, s[2 * blk]), a1 = decode_word(w1, s[2 * blk + 1]);
+#pragma unroll
+                for (int m = 0; m < NT; ++m) {
+                    mma_f16(acc[blk][m], a0.x, a1.x, a0.y, a1.y, b[m].x, b[m].y);
+                    mma_f16(acc[blk][m], a0.z, a1.z, a0.w, a1.w, b[m].z, b[m].w);
+                }
+            }
+        }
+    }
+    cp_async_wait<0>();
+    __syncthreads();                           // the rings become the partial products [warp][token][row]
+    constexpr int kPitch = kStreamRows + 4, kTokens = NT * kTok;
+    static_assert(kWarps * kTokens * kPitch * 4 <= R::kBytes, "the partial products reuse the rings");
+    float* part = reinterpret_cast<float*>(smem);
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int m = 0; m < NT; ++m)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                part[(warp * kTokens + m * kTok + 2 * t + (j & 1)) * kPitch + b * 16 + (j >> 1) * 8 + g] = acc[b][m][j];
+    __syncthreads();
+    const int outputs = live_tok * kStreamRows;
+    if (slices == 1) {
+        for (int o = threadIdx.x; o < outputs; o += kThreads) {
+            const int m = o / kStreamRows, col = o % kStreamRows;
+            float sum = 0.f;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) sum += part[(w * kTokens + m) * kPitch + col];
+            if (row0 + col < p.N) p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = sum * 256.0f;
+        }
+        return;
+    }
+    for (int o = threadIdx.x; o < outputs; o += kThreads) {          // the CTA's sum over its warps, on top of warp 0's part
+        const int m = o / kStreamRows, col = o % kStreamRows;
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) sum += part[(w * kTokens + m) * kPitch + col];
+        part[m * kPitch + col] = sum;
+    }
+    cluster.sync();
+    for (int o = slice * kThreads + threadIdx.x; o < outputs; o += slices * kThreads) {
+        const int m = o / kStreamRows, col = o % kStreamRows;
+        float sum = 0.f;
+        for (int r = 0; r < slices; ++r) sum += cluster.map_shared_rank(part, r)[m * kPitch + col];
+        if (row0 + col < p.N) p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = sum * 256.0f;
+    }
+    cluster.sync();                            // no CTA leaves while its sums are still read
+}
+
+// How a call is laid out: which kernel, token tiles per CTA, blocks of tokens, K ranges (= cluster size).
+struct RowsPlan {
+    bool stream;
+    int nt, m_blocks, slices, steps_max;
+    int tiles() const { return nt * m_blocks; }
+};
+
+constexpr int kSmCount = 148;
+
+RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
+    const int64_t steps = K / kStepK;
+    const int tiles = (int)((M + kTok - 1) / kTok);
+    const int whole = tiles <= 4 ? tiles : tiles <= 6 ? 6 : 8;
+    RowsPlan best{};
+    // Up to 32 tokens, or blocks of 32 tokens while all of them together are resident at once (a small layer).
+    const int64_t stream_blocks = (N + kStreamRows - 1) / kStreamRows;
+    const int m_blocks32 = (tiles + 3) / 4;
+    if (tiles > 4 && stream_blocks * m_blocks32 <= 2 * kSmCount && N * K <= (1ll << 21)) return {true, 4, m_blocks32, 1, (int)steps};
+    if (tiles <= 4) {
+        // one and a half CTAs per SM, and at least one step per warp
+        int s = 1;
+        const int64_t blocks = stream_blocks;
+        while (s < kMaxSlices && blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
+        return {true, tiles, 1, s, (int)((steps + s - 1) / s)};
+    }
+    // Time model, in cycles of one SM: a warp's step costs 256 cycles of the logic pipe for the decode of 32 rows x 128
+    // elements or 128 per token tile on the tensor pipe, whichever is larger; two warps of a CTA share a scheduler and
+    // take alternate steps, so a CTA needs that per step; start, casts and the reduction cost about 2500 cycles.
+    // Up to 64 rows one block of tokens (the weight is read and decoded once); above, blocks of 64 or of 32 rows.
+    const int64_t row_blocks = (N + kCtaRows - 1) / kCtaRows;
+    double best_cost = 1e300;
+    for (int nt = whole; nt >= 4; nt -= 4) {
+        if (nt != whole && tiles <= kMaxTiles) break;
+        const int m_blocks = (tiles + nt - 1) / nt;
+        const double per_step = 128.0 * nt;
+        for (int s = 1; s <= kMaxSlices && s <= steps; ++s) {
+            const int64_t ctas = row_blocks * s * m_blocks, waves = (ctas + kSmCount - 1) / kSmCount;
+            const double cost = (double)waves * ((double)((steps + s - 1) / s) * per_step + 2500.0);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = {false, nt, m_blocks, s, (int)((steps + s - 1) / s)};
+            }
+        }
+    }
+    return best;
+}
+
+constexpr size_t kMaxSmem = 227 * 1024;
+
+// The CTAs cast their rows themselves: one or two rows (the redundant casts are a small share of the decode), or a
+// product so small that the second launch would cost more than the casts (below 2^28 multiply-adds); in either case
+// only while the fragments leave room for a second CTA on the SM.
+bool cast_inside(const RowsPlan& pl, int64_t M, int64_t N, int64_t K) {
+    if (pl.stream) return M <= 2 && (size_t)pl.steps_max * M * kStepK * 2 <= 40 * 1024;
+    return (double)M * (double)N * (double)K < 268435456.0 && (size_t)pl.steps_max * pl.nt * kFragBytes <= 32 * 1024;
+}
+
+struct RowsKernel {
+    void (*fn)(const RowsParams);
+    size_t ring_bytes, frag_ring_bytes;
+};
+
+template <int GS>
+RowsKernel kernel_for(const RowsPlan& pl, bool cast) {
+    constexpr size_t kStream = StreamRing<GS>::kBytes;
+    if (pl.stream) {
+        if (cast) return {gemm_rows_stream_kernel<1, true, GS>, kStream, 0};
+        switch (pl.nt) {
+            case 1: return {gemm_rows_stream_kernel<1, false, GS>, kStream, 0};
+            case 2: return {gemm_rows_stream_kernel<2, false, GS>, kStream, 0};
+            case 3: return {gemm_rows_stream_kernel<3, false, GS>, kStream, 0};
+            default: return {gemm_rows_stream_kernel<4, false, GS>, kStream, 0};
+        }
+    }
+    switch (pl.nt) {
+        case 4: return {cast ? gemm_rows_kernel<4, true, GS> : gemm_rows_kernel<4, false, GS>, Ring<4, GS>::kBytes, Ring<4, GS>::kFragRing};
+        case 6: return {cast ? gemm_rows_kernel<6, true, GS> : gemm_rows_kernel<6, false, GS>, Ring<6, GS>::kBytes, Ring<6, GS>::kFragRing};
+        default: return {cast ? gemm_rows_kernel<8, true, GS> : gemm_rows_kernel<8, false, GS>, Ring<8, GS>::kBytes, Ring<8, GS>::kFragRing};
+    }
 }
 
 // Programmatic dependent launch is used outside stream capture only (see the file header).
@@ -281,123 +696,124 @@ bool programmatic_launch_ok(cudaStream_t st) {
     return cs == cudaStreamCaptureStatusNone;
 }
 
-void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, unsigned row_blocks, int slices, cudaStream_t st,
-                    bool programmatic = false) {
-    cfg = {};
-    cfg.gridDim = dim3(row_blocks, (unsigned)slices, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = (unsigned)slices;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic ? 2 : 1;
-}
-
-// How many clusters of `slices` CTAs the device holds at once (asked once per kernel and cluster size; 0 if the
-// query fails).
-int resident_clusters(int mts, int slices) {
-    static int cached[kMaxRowTiles + 1][kMaxSlices + 1] = {};
-    int& c = cached[mts][slices];
-    if (c) return c > 0 ? c : 0;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[2];
-    cluster_config(cfg, attr, 1, slices, nullptr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel_for_tiles(mts), &cfg) != cudaSuccess || n <= 0) {
-        cudaGetLastError();
-        n = -1;
-    }
-    c = n;
-    return n > 0 ? n : 0;
-}
-
-// Ranges of K per 128 weight rows: as many as give every range at least two steps and still let all clusters
-// be resident at once (a second wave of CTAs would start its stream from an empty pipeline).
-int slices_for(int mts, int64_t N, int64_t K) {
-    const int64_t steps = K / kStepK, row_blocks = (N + kCtaRows - 1) / kCtaRows;
-    int s = kMaxSlices;
-    while (s > 1 && (steps < 2 * s || row_blocks > resident_clusters(mts, s))) s >>= 1;
-    return s;
-}
-
-int launch_rows(const uint4* frag, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N, int64_t K,
-                float* C, int64_t ld_c, cudaStream_t st) {
-    static bool configured[64] = {};         // the opt-in to > 48 KB of dynamic shared memory is per device
+int launch_rows(RowsParams p, const RowsPlan& pl, bool cast, int gs, bool programmatic, cudaStream_t st) {
+    const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl, cast) : gs == 32 ? kernel_for<32>(pl, cast)
+                            : gs == 64 ? kernel_for<64>(pl, cast) : kernel_for<128>(pl, cast);
+    static bool configured[64][2][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
-    if (!configured[dev]) {
-        for (int mts = 1; mts <= kMaxRowTiles; mts *= 2)
-            if (cudaFuncSetAttribute(kernel_for_tiles(mts), cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
-                cudaSuccess) {
-                cudaGetLastError();
-                return AMX_ERR_CUDA;
-            }
-        configured[dev] = true;
+    bool& done = configured[dev][pl.stream][cast][gs == 16 ? 0 : gs == 32 ? 1 : gs == 64 ? 2 : 3][pl.nt];
+    if (!done) {
+        if (cudaFuncSetAttribute(kernel.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
+            cudaGetLastError();
+            return AMX_ERR_CUDA;
+        }
+        done = true;
     }
-    const int mts = row_tiles(M);
-    cudaLaunchConfig_t cfg;
+    const int held = pl.steps_max < kScaleSteps ? pl.steps_max : kScaleSteps;
+    p.steps_max = pl.steps_max;
+    cudaLaunchConfig_t cfg = {};
+    const int cta_rows = pl.stream ? kStreamRows : kCtaRows;
+    cfg.gridDim = dim3((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = pl.stream ? kernel.ring_bytes + (cast ? (size_t)pl.steps_max * p.M * kStepK * 2 : 0)
+                                     : kernel.ring_bytes + (size_t)scale_bytes(held, gs) +
+                                           (cast ? (size_t)pl.steps_max * pl.nt * kFragBytes : kernel.frag_ring_bytes);
+    cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    cluster_config(cfg, attr, (unsigned)((N + kCtaRows - 1) / kCtaRows), slices_for(mts, N, K), st, programmatic_launch_ok(st));
-    if (cudaLaunchKernelEx(&cfg, kernel_for_tiles(mts), frag, w_codes, w_scales, (int)M, N, K, C, ld_c) != cudaSuccess) {
+    int n = 0;
+    if (pl.slices > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = 1;
+        attr[n].val.clusterDim.y = (unsigned)pl.slices;
+        attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (programmatic) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    if (cudaLaunchKernelEx(&cfg, kernel.fn, p) != cudaSuccess) {
         cudaGetLastError();
         return AMX_ERR_CUDA;
     }
     return AMX_OK;
 }
 
-// Workspace: 256 bytes whose first word is the status word amx_gemm_status reads, then the decoded rows.
+// Workspace: 256 bytes whose first word is the status word amx_gemm_status reads, then the fragments of the rows.
 constexpr size_t kHeaderBytes = 256;
-uint4* fragments_of(void* workspace) { return reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes); }
 
-template <bool CAST>
-int launch_fragments(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K,
-                     void* workspace, cudaStream_t st) {
-    const int mts = row_tiles(M);
-    const int64_t threads = (int64_t)kMaxRows * mts * (K / 32) * 4;
+template <bool CAST, int GS>
+int launch_fragments_gs(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int tiles,
+                        void* workspace, bool programmatic, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((threads + 127) / 128), 1, 1);
+    cfg.gridDim = dim3((unsigned)((K / 8 + 127) / 128), (unsigned)(tiles * kTok), 1);
     cfg.blockDim = dim3(128, 1, 1);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = programmatic_launch_ok(st) ? 1 : 0;
-    if (cudaLaunchKernelEx(&cfg, rows_fragments_kernel<CAST>, codes, scales, x, ld_x, (int)M, mts, K,
-                           fragments_of(workspace), static_cast<int*>(workspace)) != cudaSuccess) {
+    cfg.numAttrs = programmatic ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, rows_fragments_kernel<CAST, GS>, codes, scales, x, ld_x, (int)M, tiles, K,
+                           reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes),
+                           static_cast<int*>(workspace)) != cudaSuccess) {
         cudaGetLastError();
         return AMX_ERR_CUDA;
     }
     return AMX_OK;
 }
+template <bool CAST>
+int launch_fragments(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int gs,
+                     int tiles, void* workspace, bool programmatic, cudaStream_t st) {
+    auto* fn = gs == 16 ? launch_fragments_gs<CAST, 16> : gs == 32 ? launch_fragments_gs<CAST, 32>
+             : gs == 64 ? launch_fragments_gs<CAST, 64> : launch_fragments_gs<CAST, 128>;
+    return fn(codes, scales, x, ld_x, M, K, tiles, workspace, programmatic, st);
+}
+
+// x != nullptr: bf16 rows, cast here; otherwise quantized rows.
+int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int64_t ld_x, const uint8_t* w_codes,
+             const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace,
+             cudaStream_t st) {
+    const RowsPlan pl = plan_rows(M, N, K);
+    const bool cast = x && cast_inside(pl, M, N, K), programmatic = programmatic_launch_ok(st);
+    RowsParams p{};
+    p.x = static_cast<const uint16_t*>(x);
+    p.ld_x = ld_x;
+    p.frag = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(workspace) + kHeaderBytes);
+    p.w_codes = w_codes; p.w_scales = w_scales;
+    p.M = (int)M; p.N = N; p.K = K; p.C = C; p.ld_c = ld_c;
+    p.status = static_cast<int*>(workspace);
+    if (!cast) {
+        const int rc = x ? launch_fragments<true>(nullptr, nullptr, p.x, ld_x, M, K, gs, pl.tiles(), workspace, programmatic, st)
+                         : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, programmatic, st);
+        if (rc != AMX_OK) return rc;
+    }
+    return launch_rows(p, pl, cast, gs, programmatic, st);
+}
 
 }  // namespace
 
 bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs) {
-    return gs == 32 && M >= 1 && M <= kMaxRows * kMaxRowTiles && N >= 1 && K >= kStepK && K % kStepK == 0 &&
-           (N + kCtaRows - 1) / kCtaRows <= 0x7FFFFFFF;
+    return fixed_group_size(gs) && M >= 1 && M <= kRowsMaxM && N >= 1 && K >= kStepK && K % kStepK == 0 &&
+           (N + kStreamRows - 1) / kStreamRows <= 0x7FFFFFFF;
 }
 
-size_t gemm_rows_workspace_bytes(int64_t M, int64_t K) {
-    return kHeaderBytes + (size_t)kMaxRows * row_tiles(M) * (size_t)K * 2;
+size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K) {
+    return kHeaderBytes + (size_t)plan_rows(M, N, K).tiles() * kTok * (size_t)K * 2;
 }
 
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
-              int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
-    if (launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, workspace, st) != AMX_OK) return AMX_ERR_CUDA;
-    return launch_rows(fragments_of(workspace), w_codes, w_scales, M, N, K, C, ld_c, st);
+              int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
+    return run_rows(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, gs, C, ld_c, workspace, st);
 }
 
 int gemm_rows_cast(const void* x, int64_t ld_x, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N,
-                   int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
-    if (launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, workspace, st) != AMX_OK)
-        return AMX_ERR_CUDA;
-    return launch_rows(fragments_of(workspace), w_codes, w_scales, M, N, K, C, ld_c, st);
+                   int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
+    return run_rows(nullptr, nullptr, x, ld_x, w_codes, w_scales, M, N, K, gs, C, ld_c, workspace, st);
 }
 
 }  // namespace amx

@@ -1,0 +1,57 @@
+"""The weight-streaming kernel at the edges of its tiles: token tiles of 8 (1 to 8 of them, and blocks of 64 rows above),
+weight rows around a CTA's 128, K ranges of unequal length and longer than the scales held at a time, every fixed group
+size; rows cast inside the kernel and ahead of it; weights whose scales start at an odd half word (groups of 128)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2411_09909_b200 import amx, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def dev_bf16(bits):
+    return torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
+
+
+@pytest.mark.parametrize("gs", [16, 32, 64, 128])
+@pytest.mark.parametrize("M,N,K", [(1, 129, 512), (3, 8, 640), (8, 1030, 1152), (9, 128, 2176), (24, 300, 896), (32, 127, 1024),
+                                   (40, 257, 640), (64, 130, 1408), (65, 140, 512), (130, 1024, 1024), (256, 260, 768),
+                                   (2, 20, 33920)])
+def test_few_rows_against_oracle(M, N, K, gs):
+    a_bits = inputs.random_groups(3000 + M, M, K, "mixed" if gs % 32 == 0 else "normal")
+    w_bits = inputs.random_groups(3100 + N, N, K, "normal")
+    qa, qw = oracle.quantize(a_bits, gs), oracle.quantize(w_bits, gs)
+    ref = oracle.gemm(*qa, *qw, gs)
+    dev = [torch.from_numpy(t).cuda() for t in (*qa, *qw)]
+    assert amx.lib().amx_gemm_kernel_for(M, N, K, gs, amx.GEMM_AUTO) == amx.GEMM_ROWS
+    wide = torch.full((M, N + 3), 5.0, dtype=torch.float32, device="cuda")
+    got = amx.gemm(*dev, gs, out=wide[:, :N])
+    assert torch.all(wide[:, N:] == 5.0)
+    g = got.cpu().numpy().astype(np.float64)
+    for m in range(M):                                # "mixed" rows differ by many orders of magnitude
+        if np.all(np.isfinite(ref[m])) and np.linalg.norm(ref[m]) > 0:
+            assert np.linalg.norm(g[m] - ref[m]) <= 1e-5 * np.linalg.norm(ref[m]), m
+    strided = torch.zeros((M, K + 24), dtype=torch.bfloat16, device="cuda")
+    strided[:, 8:8 + K] = dev_bf16(a_bits)
+    assert torch.equal(amx.quant_gemm(strided[:, 8:8 + K], dev[2], dev[3], gs), got.contiguous())
+    assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), group_size=gs, w_bf16=dev_bf16(w_bits)), got.contiguous())
+
+
+def test_back_to_back_calls_share_a_workspace():
+    """Calls chained on one stream, every one of them on the same workspace and output: each sees its own rows."""
+    N, K = 512, 4096
+    w_bits = inputs.random_groups(3200, N, K, "normal")
+    wc, ws = amx.quantize(dev_bf16(w_bits))
+    for M in (1, 20):
+        xs = [dev_bf16(inputs.random_groups(3201 + i, M, K, "normal")) for i in range(6)]
+        want = [amx.quant_gemm(x, wc, ws).clone() for x in xs]
+        torch.cuda.synchronize()
+        work = torch.empty(amx.lib().amx_quant_gemm_workspace_bytes(M, N, K, 32, 0), dtype=torch.uint8, device="cuda")
+        out = torch.empty((M, N), dtype=torch.float32, device="cuda")
+        got = []
+        for x in xs:
+            got.append(amx.quant_gemm(x, wc, ws, out=out, workspace=work).clone())
+        assert all(torch.equal(g, w) for g, w in zip(got, want))
+        assert amx.gemm_status(work) == 0
