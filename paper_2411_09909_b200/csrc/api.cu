@@ -41,19 +41,21 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
         return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
-    if (gemm_fp4_supported(M, N, K, gs) && mnk >= 268435456.0) return AMX_GEMM_FP4;
+    // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)
+    if (fixed_group_size(gs) && gemm_fp4_supported(M, N, K, 32) && mnk >= 268435456.0) return AMX_GEMM_FP4;
     return tc ? AMX_GEMM_TC : AMX_GEMM_SIMT;
 }
 
 // AMX_GEMM_AUTO on the FP4 kernel: when preparing the operands flushed a scale (see to_ue4m3), the FP4 kernel
-// returns at once and the exact bf16-decode kernel runs instead - decided on the device, from the count in the
-// workspace's second word.  That kernel's scratch follows the FP4 kernel's.
+// returns at once and the exact bf16-decode kernel (groups other than 32: the plain kernel, which has no scratch)
+// runs instead - decided on the device, from the count in the workspace's second word.  That kernel's scratch follows
+// the FP4 kernel's.
 bool auto_fallback(uint32_t flags, uint32_t kernel) { return (flags & kKernelMask) == AMX_GEMM_AUTO && kernel == AMX_GEMM_FP4; }
 
-size_t kernel_workspace(uint32_t kernel, int64_t M, int64_t N, int64_t K, bool fallback = false) {
+size_t kernel_workspace(uint32_t kernel, int64_t M, int64_t N, int64_t K, bool fallback = false, int gs = 32) {
     if (kernel == AMX_GEMM_TC) return round_up(gemm_tc_workspace_bytes(M, N, K));
     if (kernel == AMX_GEMM_FP4)
-        return round_up(gemm_fp4_workspace_bytes(M, N, K)) + (fallback ? round_up(gemm_tc_workspace_bytes(M, N, K)) : 0);
+        return round_up(gemm_fp4_workspace_bytes(M, N, K)) + (fallback && gs == 32 ? round_up(gemm_tc_workspace_bytes(M, N, K)) : 0);
     if (kernel == AMX_GEMM_ROWS) return round_up(gemm_rows_workspace_bytes(M, N, K));
     return 0;
 }
@@ -80,7 +82,7 @@ extern "C" uint32_t amx_gemm_kernel_for(int64_t M, int64_t N, int64_t K, int gro
 extern "C" size_t amx_workspace_bytes(int64_t M, int64_t N, int64_t K, int group_size, uint32_t flags) {
     if (!gemm_shape_ok(M, N, K, group_size)) return 0;
     const uint32_t kernel = pick_kernel(M, N, K, group_size, flags);
-    return kernel_workspace(kernel, M, N, K, auto_fallback(flags, kernel));
+    return kernel_workspace(kernel, M, N, K, auto_fallback(flags, kernel), group_size);
 }
 
 extern "C" size_t amx_quant_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int group_size, uint32_t flags) {
@@ -121,13 +123,15 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
         return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st);
     if (!codes16 || (kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4))) return AMX_ERR_ALIGN;
     const bool fallback = auto_fallback(flags, kernel);
-    const size_t need = kernel_workspace(kernel, M, N, K, fallback);
+    const size_t need = kernel_workspace(kernel, M, N, K, fallback, group_size);
     if (need && (!workspace || workspace_bytes < need)) return AMX_ERR_WORKSPACE;
     if (need && !aligned(workspace, kAlign)) return AMX_ERR_ALIGN;
     if (kernel == AMX_GEMM_FP4) {
-        int rc = gemm_fp4(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c, workspace, st, fallback);
+        int rc = gemm_fp4(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c, workspace, st, fallback, group_size);
         if (rc != AMX_OK || !fallback) return rc;
         int* words = static_cast<int*>(workspace);       // [0] status, [1] flushed scales
+        if (group_size != 32)
+            return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st, words + 1);
         return gemm_tc(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c,
                        static_cast<uint8_t*>(workspace) + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
     }
@@ -241,7 +245,7 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
     if (kernel == AMX_GEMM_ROWS && !w_is_bf16 && !aligned(w_scales, 4)) return AMX_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const bool fallback = auto_fallback(flags, kernel);
-    size_t gemm_ws = kernel_workspace(kernel, M, N, K, fallback);
+    size_t gemm_ws = kernel_workspace(kernel, M, N, K, fallback, group_size);
     if (gemm_ws < 256) gemm_ws = 256;                       // the plain kernel has no scratch of its own: header only
     const QuantSizes a = quant_sizes(M, K, group_size), w = quant_sizes(N, K, group_size);
     uint8_t* base = static_cast<uint8_t*>(workspace);
@@ -258,23 +262,26 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
         uint8_t* pw = pa + gemm_fp4_prepared_bytes(M, K, false);
         int* words = reinterpret_cast<int*>(base);
         if (cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
-        if (ld_a == K) rc = gemm_fp4_quantize_prepared(A, M, K, false, a_codes, a_scales, pa, st, 0, AMX_FMT_AMXFP4, words + 1);
+        if (ld_a == K && group_size == 32) rc = gemm_fp4_quantize_prepared(A, M, K, false, a_codes, a_scales, pa, st, 0, AMX_FMT_AMXFP4, words + 1);
         else {
             rc = amx_quantize(A, M, K, ld_a, group_size, a_codes, a_scales, stream);
-            if (rc == AMX_OK) rc = gemm_fp4_prepare(a_codes, a_scales, M, K, false, pa, st, 0, words + 1);
+            if (rc == AMX_OK) rc = gemm_fp4_prepare(a_codes, a_scales, M, K, false, pa, st, 0, words + 1, group_size);
         }
         if (rc != AMX_OK) return rc;
-        if (w_is_bf16 && ld_w == K)
+        if (w_is_bf16 && ld_w == K && group_size == 32)
             rc = gemm_fp4_quantize_prepared(W_bf16, N, K, true, wq_codes, wq_scales, pw, st, 0, AMX_FMT_AMXFP4, words + 1);
         else {
             if (w_is_bf16) rc = amx_quantize(W_bf16, N, K, ld_w, group_size, wq_codes, wq_scales, stream);
             if (rc == AMX_OK)
                 rc = gemm_fp4_prepare(w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, N, K, true, pw, st, 0,
-                                      words + 1);
+                                      words + 1, group_size);
         }
         if (rc != AMX_OK) return rc;
         rc = gemm_fp4_prepared(pa, pw, M, N, K, C, ld_c, base, st, 256, fallback ? words + 1 : nullptr);
         if (rc != AMX_OK || !fallback) return rc;
+        if (group_size != 32)
+            return gemm_simt(a_codes, a_scales, w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, M, N, K, group_size,
+                             C, ld_c, st, words + 1);
         return gemm_tc(a_codes, a_scales, w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, M, N, K, C, ld_c,
                        base + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
     }

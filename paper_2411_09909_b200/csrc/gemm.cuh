@@ -7,7 +7,7 @@ namespace amx {
 
 int gemm_simt(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes,
               const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C,
-              int64_t ld_c, cudaStream_t st);
+              int64_t ld_c, cudaStream_t st, const int* run_if_nonzero = nullptr /* device word: nothing is done when zero */);
 
 // The same kernel on operands with binary16 shared scales ([rows, K/gs, 2] uint16).
 int gemm_simt_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8_t* w_codes,
@@ -44,13 +44,13 @@ bool gemm_fp4_supported(int64_t M, int64_t N, int64_t K, int gs);
 size_t gemm_fp4_workspace_bytes(int64_t M, int64_t N, int64_t K);
 int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes,
              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c,
-             void* workspace, cudaStream_t st, bool gate_on_flushed = false);
+             void* workspace, cudaStream_t st, bool gate_on_flushed = false, int gs = 32);
 // The same in two phases, so that an operand (typically the weight) is prepared once and reused.
 size_t gemm_fp4_prepared_bytes(int64_t rows, int64_t K, bool is_weight);
 // flushed_total (optional, device): incremented by the number of nonzero scales that fell below the UE4M3 range
 // of their row and were flushed; the per-row counts are in the row words either way.
 int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
-                     void* prepared, cudaStream_t st, int64_t layout_rows = 0 /* 0: rows */, int* flushed_total = nullptr);
+                     void* prepared, cudaStream_t st, int64_t layout_rows = 0 /* 0: rows */, int* flushed_total = nullptr, int gs = 32);
 int gemm_fp4_quantize_prepared(const void* x, int64_t rows, int64_t K, bool is_weight, uint8_t* codes,
                                uint8_t* scales, void* prepared, cudaStream_t st, int64_t layout_rows = 0,
                                int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr);

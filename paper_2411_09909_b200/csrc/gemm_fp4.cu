@@ -108,22 +108,23 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
 __host__ __device__ constexpr uint32_t instr_desc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24); }
 
 // ------------------------------------------------------------------------- preparation --
-// One launch per operand; one block per 32 operand rows (rows beyond R, up to the padded row count,
+// One launch per operand; one block per kPrepRows operand rows (rows beyond R, up to the padded row count,
 // get zero scale factors so that padded tile rows multiply zero codes by a finite scale).
 //   1. row words: a warp per row finds the largest exponent key kmax among the row's scales (kmax - 25 is the
 //      power of two by which the row's UE4M3 scales understate the true ones) and which sides occur at all
 //   2. sign planes: every nibble goes to the plane of its sign bit, zero in the other plane
 //   3. scale factors of both planes in the layout the MMA reads:
 //      [plane][row block of 128][K/64 block][512 B], byte (r%32)*16 + (r/32)*4 + (k16 % 4);
-//      one scale per 16 elements, so each 32-group's scale is written twice
+//      one scale per 16 elements, so a group's scale is written gs / 16 times (GS = 16: the MMA's own block)
 constexpr int kPrepRows = 8;
+template <int GS>
 __global__ void __launch_bounds__(256)
 prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int64_t R, int64_t K,
                        int nk64, uint4* __restrict__ pos, uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos,
                        uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total) {
     __shared__ int kmax_s[kPrepRows];
     __shared__ int unsplit_s[kPrepRows];
-    const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / 32;
+    const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / GS;         // G: scale pairs per row
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int r = warp; r < kPrepRows; r += 8) {
         const int64_t row = row0 + r;
@@ -165,13 +166,14 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
     // sign planes of this block's rows (contiguous in memory: rows are K/2 bytes apart)
     __syncthreads();                                             // unsplit_s is complete
     const int64_t rows_here = min((int64_t)kPrepRows, R - row0);
+    const int vec_per_row = (int)(K / 32);
     if (rows_here > 0) {
-        const int64_t v0 = row0 * (K / 32), n_vec = rows_here * (K / 32);
+        const int64_t v0 = row0 * vec_per_row, n_vec = rows_here * vec_per_row;
         const uint4* src = reinterpret_cast<const uint4*>(codes) + v0;
         for (int64_t i = threadIdx.x; i < n_vec; i += 256) {
             const uint4 w = __ldg(src + i);
             const uint32_t v[4] = {w.x, w.y, w.z, w.w};
-            const uint32_t keep = unsplit_s[(int)i / (int)G] ? 0u : 0xFFFFFFFFu;   // i < 8 rows x G: 32-bit division
+            const uint32_t keep = unsplit_s[(int)i / vec_per_row] ? 0u : 0xFFFFFFFFu;   // i < 8 rows: 32-bit division
             uint32_t p[4], n[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -187,6 +189,7 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
     // scale factors: item = (K/64 block c, row r); consecutive threads take consecutive rows
     const int64_t rb = row0 / 128;
     const int r_in_blk0 = (int)(row0 % 128);
+    constexpr int kPer = GS >= 64 ? 1 : 64 / GS;                 // scale pairs of a 64-element block
     for (int item = threadIdx.x; item < nk64 * kPrepRows; item += 256) {
         const int c = item / kPrepRows, r = item % kPrepRows;
         const int64_t row = row0 + r;
@@ -194,13 +197,13 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
         if (row < R) {
             const int kmax = kmax_s[r];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {                        // the two 32-groups of this 64-element block
-                const int64_t g = (int64_t)c * 2 + h;
+            for (int h = 0; h < kPer; ++h) {
+                const int64_t g = GS >= 64 ? (int64_t)c * 64 / GS : (int64_t)c * kPer + h;
                 if (g < G) {
                     const uint32_t v = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * G + g) * 2));
-                    const uint32_t up = to_ue4m3(v & 0xFF, kmax), un = unsplit_s[r] ? 0u : to_ue4m3(v >> 8, kmax);
-                    wp |= (up | (up << 8)) << (16 * h);
-                    wn |= (un | (un << 8)) << (16 * h);
+                    const uint32_t rep = GS == 16 ? 1u : GS == 32 ? 0x0101u : 0x01010101u;      // copies of the byte
+                    wp |= to_ue4m3(v & 0xFF, kmax) * rep << (32 / kPer * h);
+                    wn |= (unsplit_s[r] ? 0u : to_ue4m3(v >> 8, kmax)) * rep << (32 / kPer * h);
                 }
             }
         }
@@ -669,9 +672,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
 // ---------------------------------------------------------------------------------- host --
 int prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, const OperandLayout& o,
-            uint8_t* base, cudaStream_t st, int* flushed_total = nullptr) {
+            uint8_t* base, cudaStream_t st, int* flushed_total = nullptr, int gs = 32) {
     const int64_t padded_rows = o.row_blocks * 128;
-    prepare_operand_kernel<<<(unsigned)(padded_rows / kPrepRows), 256, 0, st>>>(
+    auto* kernel = gs == 16 ? prepare_operand_kernel<16> : gs == 32 ? prepare_operand_kernel<32>
+                 : gs == 64 ? prepare_operand_kernel<64> : prepare_operand_kernel<128>;
+    kernel<<<(unsigned)(padded_rows / kPrepRows), 256, 0, st>>>(
         codes, scales, rows, K, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
         base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf),
         flushed_total);
@@ -847,9 +852,9 @@ int gemm_fp4_softmax_prepared(const float* S, int64_t rows, int64_t cols, int64_
 }
 
 int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
-                     void* prepared, cudaStream_t st, int64_t layout_rows, int* flushed_total) {
+                     void* prepared, cudaStream_t st, int64_t layout_rows, int* flushed_total, int gs) {
     return prepare(codes, scales, rows, K, operand_layout(layout_rows ? layout_rows : rows, K, is_weight ? BN : BM),
-                   static_cast<uint8_t*>(prepared), st, flushed_total);
+                   static_cast<uint8_t*>(prepared), st, flushed_total, gs);
 }
 
 // Workspace: word 0 the status, word 1 the number of scales flushed while preparing the two operands (see
@@ -857,15 +862,15 @@ int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, 
 // not zero (the caller follows with the exact kernel, gated the other way).
 int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
              int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st,
-             bool gate_on_flushed) {
+             bool gate_on_flushed, int gs) {
     const OperandLayout oa = operand_layout(M, K, BM), ow = operand_layout(N, K, BN);
     uint8_t* base = static_cast<uint8_t*>(workspace);
     uint8_t* pa = base + 256;
     uint8_t* pw = pa + oa.total;
     int* flushed = reinterpret_cast<int*>(base) + 1;
     if (cudaMemsetAsync(base, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
-    int rc = prepare(a_codes, a_scales, M, K, oa, pa, st, flushed);
-    if (rc == AMX_OK) rc = prepare(w_codes, w_scales, N, K, ow, pw, st, flushed);
+    int rc = prepare(a_codes, a_scales, M, K, oa, pa, st, flushed, gs);
+    if (rc == AMX_OK) rc = prepare(w_codes, w_scales, N, K, ow, pw, st, flushed, gs);
     if (rc != AMX_OK) return rc;
     return gemm_fp4_prepared(pa, pw, M, N, K, C, ld_c, base, st, 256, gate_on_flushed ? flushed : nullptr);
 }

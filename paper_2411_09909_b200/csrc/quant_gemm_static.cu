@@ -65,7 +65,13 @@ extern "C" int amx_quant_gemm_static(const void* A, int64_t ld_a, const uint8_t*
     if (M == 0 || N == 0) return AMX_OK;
     // Nothing below needs to start at zero except the GEMM's status word, which the GEMM launcher
     // clears itself on `stream`; the quantized activation is fully overwritten before it is read.
-    if (amx_quant_gemm_workspace_bytes(M, N, K, group_size, flags) > kStaticScratchBytes) return AMX_ERR_TOO_LARGE;
+    if (amx_quant_gemm_workspace_bytes(M, N, K, group_size, flags) > kStaticScratchBytes) {
+        // group sizes other than 32 still fit on the plain kernel, which keeps no prepared operands
+        if (flags != AMX_GEMM_AUTO || group_size == 32 ||
+            amx_quant_gemm_workspace_bytes(M, N, K, group_size, AMX_GEMM_SIMT) > kStaticScratchBytes)
+            return AMX_ERR_TOO_LARGE;
+        flags = AMX_GEMM_SIMT;
+    }
     void* scratch = nullptr;
     const int rc = static_scratch(&scratch);
     if (rc != AMX_OK) return rc;

@@ -55,3 +55,34 @@ def test_back_to_back_calls_share_a_workspace():
             got.append(amx.quant_gemm(x, wc, ws, out=out, workspace=work).clone())
         assert all(torch.equal(g, w) for g, w in zip(got, want))
         assert amx.gemm_status(work) == 0
+
+
+@pytest.mark.parametrize("gs", [16, 64, 128])
+@pytest.mark.parametrize("M,N,K", [(300, 1000, 1152), (513, 776, 1024), (257, 2048, 640), (300, 3000, 320)])
+def test_other_group_sizes_on_the_fp4_kernel(M, N, K, gs):
+    """Groups of 16, 64 and 128 through the FP4 kernel (AUTO, from 2^28 multiply-adds): ragged rows, K tails inside a
+    64-element block of scale factors; a flushed scale sends the product to the exact kernel."""
+    if K % gs:
+        pytest.skip("K not a multiple of the group size")
+    a_bits, w_bits = inputs.random_groups(3300 + M, M, K, "normal"), inputs.random_groups(3400 + N, N, K, "normal")
+    L = amx.lib()
+    want = amx.GEMM_FP4 if M * N * K >= 1 << 28 else L.amx_gemm_kernel_for(M, N, K, gs, 0)
+    assert L.amx_gemm_kernel_for(M, N, K, gs, amx.GEMM_AUTO) == want
+    for spread in (0, 20):                            # 20 binades between the groups of row 3: scales are flushed
+        if spread:
+            a_bits = a_bits.copy()
+            f = inputs.bf16_bits_to_f32(a_bits)
+            f[3, :gs] *= 2.0 ** 12
+            f[3, gs:] *= 2.0 ** (12 - spread)
+            a_bits = inputs.f32_to_bf16_bits(f)
+        qa, qw = oracle.quantize(a_bits, gs), oracle.quantize(w_bits, gs)
+        dev = [torch.from_numpy(t).cuda() for t in (*qa, *qw)]
+        rows = np.unique(np.concatenate([[0, 3, M - 1], np.arange(0, M, 37)]))
+        ref = oracle.gemm(*qa, *qw, gs, rows=rows)
+        work = torch.empty(L.amx_workspace_bytes(M, N, K, gs, 0) + 256, dtype=torch.uint8, device="cuda")
+        got = amx.gemm(*dev, gs, workspace=work)
+        if want == amx.GEMM_FP4:
+            assert amx.gemm_status(work) == 0 and (amx.gemm_flushed_scales(work) > 0) == bool(spread)
+        assert np.linalg.norm(got.cpu().numpy()[rows] - ref) <= 1e-5 * np.linalg.norm(ref)
+        assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), dev[2], dev[3], gs), got)
+        assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), group_size=gs, w_bf16=dev_bf16(w_bits)), got)
