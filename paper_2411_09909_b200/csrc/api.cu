@@ -28,7 +28,7 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     const bool rows = gemm_rows_supported(M, N, K, gs);
     if (want == AMX_GEMM_ROWS) return rows && M <= 64 ? AMX_GEMM_ROWS : 0;
     // AMX_GEMM_AUTO: the FP4-pipe kernel for anything that fills the machine (it is about twice as fast as
-    // the bf16-decode kernel); the exact bf16-decode kernel for small products (below 2^28 multiply-adds), where
+    // the bf16-decode kernel); the exact bf16-decode kernel for small products (below 2^27 multiply-adds), where
     // launch count matters more than throughput - the FP4 route costs two launches more: one preparation per
     // operand, and under AUTO the gated exact kernel behind it; the SIMT kernel for group sizes the tensor-core kernels do not take.
     // A few token rows against a big weight (decode-like): too few 128 x 256 tiles to fill the machine, and the
@@ -42,7 +42,7 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
     // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)
-    if (fixed_group_size(gs) && gemm_fp4_supported(M, N, K, 32) && mnk >= 268435456.0) return AMX_GEMM_FP4;
+    if (fixed_group_size(gs) && gemm_fp4_supported(M, N, K, 32) && mnk >= 134217728.0) return AMX_GEMM_FP4;
     return tc ? AMX_GEMM_TC : AMX_GEMM_SIMT;
 }
 
@@ -476,64 +476,107 @@ extern "C" int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, 
 }
 
 namespace {
-// Workspace of amx_attention.  Heads are taken in chunks: the casts of Q, K and V (small per head) run once per
-// chunk on the stacked heads, the two products and the softmax once per head.  Holds the canonical codes and
-// scales of the chunk's Q, K and V^T and of one head's P, the logits S of one head, then either the prepared
-// operands of the FP4 kernel (Q and P as left-hand, K and V^T as right-hand operands) or the other kernels' own
-// scratch, and the status word.
-constexpr int64_t kAttnChunk = 8, kAttnChunkFused = 16;
-int64_t attn_chunk(int64_t L, int64_t d) {
-    if (attn_fused_supported(L, d)) return kAttnChunkFused;   // 16 x (L / 128) items: an even load for 148 persistent CTAs
-    return (L % 128 == 0 && d % 128 == 0) ? kAttnChunk : 1;
-}
-
+// Workspace of amx_attention.  Heads are taken in chunks: the casts of Q, K and V (small per head) run once per chunk
+// on the stacked heads.  Two ways from there:
+//   fused   (head dimension 128 or 64, products on the FP4 kernel) both products and the softmax in two launches of the
+//           fused kernel for all heads of the chunk; Q, K and V^T as prepared operands, every head padded to whole
+//           blocks of 128 rows
+//   stored  the logits and the cast map of `batch` heads at a time in the workspace: batched launches of the bf16-decode
+//           kernel (one product, one softmax and cast, one product per batch), or head by head on the other kernels
 struct AttnLayout {
+    int64_t chunk, batch;
     size_t qc, qs, kc, ks, vc, vs, pc, ps, S, pq, pk, pv, pp, stats, gemm, total;
 };
-// fused_only: the fused kernel will run (both products on the FP4 kernel, attn_fused_supported): no room for one
-// head's logits, cast map and prepared map, nor for the other kernels' scratch.
-AttnLayout attn_layout(int64_t L, int64_t d, bool fused_only = false) {
-    AttnLayout a;
-    const int64_t hc = attn_chunk(L, d);
-    const QuantSizes qd = quant_sizes(hc * L, d, 32), ql = quant_sizes(L, L, 32), qv = quant_sizes(hc * d, L, 32);
+
+AttnLayout attn_layout_fused(int64_t L, int64_t d) {
+    AttnLayout a{};
+    const int64_t Lp = attn_fused_padded(L);
+    // 16 heads x (8192 / 128) blocks of queries load 148 persistent CTAs evenly; shorter sequences take more heads
+    a.chunk = 131072 / Lp < 16 ? 16 : 131072 / Lp > 64 ? 64 : 131072 / Lp;
+    size_t off = 0;
+    auto take = [&](size_t bytes) { size_t o = off; off += round_up(bytes); return o; };
+    a.qs = take((size_t)a.chunk * Lp * (d / 32) * 2);
+    a.ks = take((size_t)a.chunk * Lp * (d / 32) * 2);
+    a.vs = take((size_t)a.chunk * 128 * (L / 32) * 2);
+    a.pq = take(gemm_fp4_prepared_bytes(a.chunk * Lp, d, false));
+    a.pk = take(gemm_fp4_prepared_bytes(a.chunk * Lp, d, true));
+    a.pv = take(gemm_fp4_prepared_bytes(a.chunk * 128, L, true));
+    a.stats = take(attn_fused_scratch_bytes(a.chunk, L));
+    a.gemm = off;
+    a.total = off + 256;
+    return a;
+}
+
+constexpr int64_t kAttnChunk = 8;
+// tc: both products on the bf16-decode kernel.
+AttnLayout attn_layout_stored(int64_t L, int64_t d, bool tc) {
+    AttnLayout a{};
+    // batches of heads whose logits stay near the L2's size
+    const int64_t fit = (64ll << 20) / (L * L * 4);
+    a.batch = !tc ? 1 : fit < 1 ? 1 : fit > 32 ? 32 : fit;
+    a.chunk = tc ? (a.batch > kAttnChunk ? a.batch : kAttnChunk) : (L % 128 == 0 && d % 128 == 0) ? kAttnChunk : 1;
+    const QuantSizes qd = quant_sizes(a.chunk * L, d, 32), ql = quant_sizes(a.batch * L, L, 32), qv = quant_sizes(a.chunk * d, L, 32);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += round_up(bytes); return o; };
     a.qc = take(qd.codes); a.qs = take(qd.scales); a.kc = take(qd.codes); a.ks = take(qd.scales);
     a.vc = take(qv.codes); a.vs = take(qv.scales);
-    a.pc = take(fused_only ? 0 : ql.codes); a.ps = take(fused_only ? 0 : ql.scales);
-    a.S = take(fused_only ? 0 : (size_t)L * L * 4);
-    // right-hand operands are laid out for 128 rows more: the last head's 256-row tiles may reach past the stack
-    a.pq = take(gemm_fp4_prepared_bytes(hc * L, d, false));
-    a.pk = take(gemm_fp4_prepared_bytes(hc * L + 128, d, true));
-    a.pv = take(gemm_fp4_prepared_bytes(hc * d + 128, L, true));
-    a.pp = take(fused_only ? 0 : gemm_fp4_prepared_bytes(L, L, false));
-    a.stats = take(attn_fused_supported(L, d) ? attn_fused_scratch_bytes(hc, L) : 0);
+    a.pc = take(ql.codes); a.ps = take(ql.scales);
+    a.S = take((size_t)a.batch * L * L * 4);
+    if (!tc) {
+        // right-hand operands are laid out for 128 rows more: the last head's 256-row tiles may reach past the stack
+        a.pq = take(gemm_fp4_prepared_bytes(a.chunk * L, d, false));
+        a.pk = take(gemm_fp4_prepared_bytes(a.chunk * L + 128, d, true));
+        a.pv = take(gemm_fp4_prepared_bytes(a.chunk * d + 128, L, true));
+        a.pp = take(gemm_fp4_prepared_bytes(L, L, false));
+    }
     a.gemm = off;
-    const size_t g1 = fused_only ? 0 : amx_workspace_bytes(L, L, d, 32, AMX_GEMM_TC);
-    const size_t g2 = fused_only ? 0 : amx_workspace_bytes(L, d, L, 32, AMX_GEMM_TC);
-    a.total = off + (g1 > g2 ? g1 : g2) + 256;
+    const size_t g1 = tc ? gemm_tc_batched_workspace_bytes(a.batch, L, L, d) : amx_workspace_bytes(L, L, d, 32, AMX_GEMM_TC);
+    const size_t g2 = tc ? gemm_tc_batched_workspace_bytes(a.batch, L, d, L) : amx_workspace_bytes(L, d, L, 32, AMX_GEMM_TC);
+    a.total = off + round_up(g1 > g2 ? g1 : g2) + 256;
     return a;
+}
+
+// The kernels of the two products under these flags (0: flags that cannot be honoured).  AUTO: where the logits or the
+// attention product would be small, the bf16-decode kernel, never the weight-streaming one (there is no weight).
+uint32_t attn_kernel(int64_t M, int64_t N, int64_t K, uint32_t flags) {
+    const uint32_t k = pick_kernel(M, N, K, 32, flags);
+    return (k == AMX_GEMM_ROWS && (flags & kKernelMask) == AMX_GEMM_AUTO) ? AMX_GEMM_TC : k;
+}
+// Whether a call runs the fused kernel: asked for the FP4 kernel, or AUTO from 2^25 multiply-adds per product and head on
+// (512 tokens at head dimension 128; below, a batched launch of each step is as fast and the kernel's two passes do
+// not fill their pipeline).
+bool attn_runs_fused(int64_t L, int64_t d, uint32_t flags) {
+    flags &= ~AMX_ATTN_CAUSAL;
+    if (!attn_fused_supported(L, d)) return false;
+    return flags == AMX_GEMM_FP4 || (flags == AMX_GEMM_AUTO && (double)L * (double)L * (double)d >= 33554432.0);
+}
+// Short sequences used to run on the exact kernel under AUTO: there a scale the FP4 kernel cannot represent must not be
+// lost, and the casts' count decides on the device.  (From 2^28 on the FP4 kernel was AUTO's choice without this check.)
+bool attn_gated(int64_t L, int64_t d, uint32_t flags) {
+    return (flags & kKernelMask) == AMX_GEMM_AUTO && (double)L * (double)L * (double)d < 268435456.0 && attn_exact_supported(L, d);
 }
 }  // namespace
 
 extern "C" size_t amx_attention_workspace_bytes(int64_t L, int64_t d) {
     if (L <= 0 || d <= 0 || L % 32 || d % 32) return 0;
-    return attn_layout(L, d).total;
+    size_t n = attn_layout_stored(L, d, true).total;
+    const size_t m = attn_layout_stored(L, d, false).total;
+    if (m > n) n = m;
+    if (attn_fused_supported(L, d) && attn_layout_fused(L, d).total > n) n = attn_layout_fused(L, d).total;
+    return n;
 }
 
 namespace {
-// Whether a call with these flags runs the fused kernel.
-bool attn_runs_fused(int64_t L, int64_t d, uint32_t flags) {
+AttnLayout attn_layout_for(int64_t L, int64_t d, uint32_t flags) {
     flags &= ~AMX_ATTN_CAUSAL;
-    if (flags & ~kKernelMask) return false;
-    return attn_fused_supported(L, d) && pick_kernel(L, L, d, 32, flags) == AMX_GEMM_FP4 &&
-           pick_kernel(L, d, L, 32, flags) == AMX_GEMM_FP4;
+    if (attn_runs_fused(L, d, flags)) return attn_layout_fused(L, d);
+    return attn_layout_stored(L, d, attn_kernel(L, L, d, flags) == AMX_GEMM_TC && attn_kernel(L, d, L, flags) == AMX_GEMM_TC);
 }
 }  // namespace
 
 extern "C" size_t amx_attention_workspace_bytes_for(int64_t L, int64_t d, uint32_t flags) {
     if (L <= 0 || d <= 0 || L % 32 || d % 32) return 0;
-    return attn_layout(L, d, attn_runs_fused(L, d, flags)).total;
+    return attn_layout_for(L, d, flags).total;
 }
 
 extern "C" int amx_attention(const void* q, const void* k, const void* v, int64_t heads, int64_t L, int64_t d,
@@ -550,25 +593,26 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
     if (heads < 0 || L <= 0 || d <= 0 || L % 32 || d % 32) return AMX_ERR_SHAPE;
     if (heads > 0 && (kv_heads <= 0 || heads % kv_heads)) return AMX_ERR_SHAPE;
     const int64_t group = heads > 0 ? heads / kv_heads : 1;        // query heads per head of keys and values
-    const uint32_t k_qk = pick_kernel(L, L, d, 32, flags), k_pv = pick_kernel(L, d, L, 32, flags);
+    const uint32_t k_qk = attn_kernel(L, L, d, flags), k_pv = attn_kernel(L, d, L, flags);
     if (!k_qk || !k_pv) return ((flags & kKernelMask) & ((flags & kKernelMask) - 1)) ? AMX_ERR_FLAGS : AMX_ERR_SHAPE;
     if (heads == 0) return AMX_OK;
     if (!q || !k || !v || !o) return AMX_ERR_NULL;
-    const AttnLayout a = attn_layout(L, d, attn_runs_fused(L, d, flags));
+    const AttnLayout a = attn_layout_for(L, d, flags);
     if (!workspace || workspace_bytes < a.total) return AMX_ERR_WORKSPACE;
     if (!aligned(workspace, kAlign) || !aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(o, 4))
         return AMX_ERR_ALIGN;
     uint8_t* w = static_cast<uint8_t*>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t gemm_bytes = a.total - a.gemm;
     const float alpha = 1.0f / sqrtf((float)d);
-    float* S = reinterpret_cast<float*>(w + a.S);
-    const int64_t chunk_max = attn_chunk(L, d);
+    const bool fused = attn_runs_fused(L, d, flags), gated = attn_gated(L, d, flags);
+    const bool tc = !fused && k_qk == AMX_GEMM_TC && k_pv == AMX_GEMM_TC;
     // a chunk holds whole groups of query heads (or, when a group is larger than a chunk, part of one group)
-    const int64_t chunk = group >= chunk_max ? chunk_max : (chunk_max / group) * group;
-    // both products on the FP4 kernel at head dimension 128: one fused kernel, logits and attention map stay on chip
-    const bool fused = k_qk == AMX_GEMM_FP4 && k_pv == AMX_GEMM_FP4 && attn_fused_supported(L, d);
+    const int64_t chunk_max = a.chunk, chunk = group >= chunk_max ? chunk_max : (chunk_max / group) * group;
     const size_t head_in = (size_t)L * d * 2;                       // bytes of one head of q, k or v
+    const size_t gemm_bytes = a.total - a.gemm;
+    int* words = reinterpret_cast<int*>(w + a.gemm);                // fused: [0] status, [1] flushed scales of the call
+    if (fused && cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+    float* S = reinterpret_cast<float*>(w + a.S);
     const size_t qk_codes = (size_t)L * d / 2, qk_scales = (size_t)L * (d / 32) * 2;   // one head of Q or K, canonical
     const size_t v_codes = (size_t)d * L / 2, v_scales = (size_t)d * (L / 32) * 2;     // one head of V^T
     for (int64_t h0 = 0; h0 < heads;) {
@@ -581,8 +625,34 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
         const uint8_t* qh = static_cast<const uint8_t*>(q) + h0 * head_in;
         const uint8_t* kh = static_cast<const uint8_t*>(k) + kv0 * head_in;
         const uint8_t* vh = static_cast<const uint8_t*>(v) + kv0 * head_in;
-        // casts of the chunk's heads, stacked row-wise: Q and K along head_dim, V along the sequence (V^T)
         int rc;
+        if (fused) {
+            // casts of the chunk's heads straight into prepared operands: Q and K along head_dim, V along the sequence
+            // (V^T).  The chunk starts at a group boundary unless the group is larger than a chunk, in which case it
+            // lies inside one group (every head maps to the chunk's one head of keys and values either way).
+            const int64_t Lp = attn_fused_padded(L);
+            rc = gemm_fp4_quantize_prepared(qh, hc * Lp, d, false, nullptr, w + a.qs, w + a.pq, st, chunk_max * Lp, AMX_FMT_AMXFP4,
+                                            words + 1, L, Lp);
+            if (rc == AMX_OK)
+                rc = gemm_fp4_quantize_prepared(kh, kvc * Lp, d, true, nullptr, w + a.ks, w + a.pk, st, chunk_max * Lp,
+                                                AMX_FMT_AMXFP4, words + 1, L, Lp);
+            if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(vh, kvc, L, d, 128, chunk_max * 128, w + a.vs, w + a.pv, st, words + 1);
+            const int kv_group = (int)(group >= chunk_max ? chunk_max : group);
+            float* oh = o + (size_t)h0 * L * d;
+            if (rc == AMX_OK)
+                rc = attn_fused({w + a.pq, hc * Lp, chunk_max * Lp, 0}, {w + a.pk, kvc * Lp, chunk_max * Lp, 0},
+                                {w + a.pv, kvc * 128, chunk_max * 128, 0}, (int)hc, L, d, alpha, causal, w + a.stats, oh, words, st,
+                                nullptr, nullptr, nullptr, nullptr, kv_group, gated ? words + 1 : nullptr);
+            if (rc == AMX_OK && gated) {
+                const size_t plane_q = gemm_fp4_plane_bytes(chunk_max * Lp, d), plane_v = gemm_fp4_plane_bytes(chunk_max * 128, L);
+                rc = attn_exact({w + a.pq, w + a.pq + plane_q, w + a.qs}, {w + a.pk, w + a.pk + plane_q, w + a.ks},
+                                {w + a.pv, w + a.pv + plane_v, w + a.vs}, (int)hc, L, d, kv_group, alpha, causal, oh, words + 1, st);
+            }
+            if (rc != AMX_OK) return rc;
+            h0 += hc;
+            continue;
+        }
+        // casts of the chunk's heads, stacked row-wise: Q and K along head_dim, V along the sequence (V^T)
         if (k_qk == AMX_GEMM_FP4) {
             rc = gemm_fp4_quantize_prepared(qh, hc * L, d, false, nullptr, w + a.qs, w + a.pq, st, chunk_max * L);
             if (rc == AMX_OK)
@@ -595,21 +665,24 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
         if (rc == AMX_OK && k_pv == AMX_GEMM_FP4)
             rc = gemm_fp4_prepare(w + a.vc, w + a.vs, kvc * d, L, true, w + a.pv, st, chunk_max * d + 128);
         if (rc != AMX_OK) return rc;
-        if (fused) {
-            // head dimension 128: both products and the softmax of all the chunk's heads in two launches.  The chunk
-            // starts at a group boundary unless the group is larger than a chunk, in which case it lies inside one
-            // group (every head maps to the chunk's one head of keys and values either way).
-            rc = attn_fused({w + a.pq, hc * L, chunk_max * L, 0}, {w + a.pk, kvc * L, chunk_max * L + 128, 0},
-                            {w + a.pv, kvc * d, chunk_max * d + 128, 0}, (int)hc, L, alpha, causal, w + a.stats,
-                            o + (size_t)h0 * L * d, w + a.gemm, st, nullptr, nullptr, nullptr, nullptr,
-                            (int)(group >= chunk_max ? chunk_max : group));
-            if (rc != AMX_OK) return rc;
-            h0 += hc;
-            continue;
-        }
-        for (int64_t i = 0; i < hc; ++i) {
-            const int64_t kv = (h_off + i) / group;                 // this head's keys and values inside the chunk
+        for (int64_t i = 0; i < hc;) {
             float* oh = o + (size_t)(h0 + i) * L * d;
+            if (tc) {
+                // a batch of heads per launch of each step
+                const int64_t nb = hc - i < a.batch ? hc - i : a.batch;
+                rc = gemm_tc_batched(w + a.qc + i * qk_codes, w + a.qs + i * qk_scales, w + a.kc, w + a.ks, nb, h_off + i, group, L, L, d,
+                                     S, causal, w + a.gemm, st);
+                if (rc == AMX_OK)
+                    rc = softmax_cast_rows(S, nb * L, L, L, alpha, w + a.pc, w + a.ps, nullptr, nullptr, nullptr, nullptr, nullptr, 0,
+                                           nb * L, st, causal ? L : 0);
+                if (rc == AMX_OK)
+                    rc = gemm_tc_batched(w + a.pc, w + a.ps, w + a.vc, w + a.vs, nb, h_off + i, group, L, d, L, oh, false, w + a.gemm,
+                                         st);
+                if (rc != AMX_OK) return rc;
+                i += nb;
+                continue;
+            }
+            const int64_t kv = (h_off + i) / group;                 // this head's keys and values inside the chunk
             // S = AMX(Q) AMX(K)^T
             if (k_qk == AMX_GEMM_FP4)
                 rc = gemm_fp4_prepared_at({w + a.pq, hc * L, chunk_max * L, i * L},
@@ -620,18 +693,19 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
             if (rc != AMX_OK) return rc;
             // softmax, rounding to bf16 and the cast of P in one kernel; O = AMX(P) AMX(V)
             if (k_pv == AMX_GEMM_FP4) {
-                rc = gemm_fp4_softmax_prepared(S, L, L, L, alpha, false, w + a.pc, w + a.ps, w + a.pp, st, causal);
+                rc = gemm_fp4_softmax_prepared(S, L, L, L, alpha, false, w + a.pc, w + a.ps, w + a.pp, st, causal ? L : 0);
                 if (rc == AMX_OK)
                     rc = gemm_fp4_prepared_at({w + a.pp, L, L, 0}, {w + a.pv, kvc * d, chunk_max * d + 128, kv * d}, L, d, L, oh,
                                               d, w + a.gemm, st);
             } else {
                 rc = softmax_cast_rows(S, L, L, L, alpha, w + a.pc, w + a.ps, nullptr, nullptr, nullptr, nullptr, nullptr, 0, L,
-                                       st, causal);
+                                       st, causal ? L : 0);
                 if (rc == AMX_OK)
                     rc = amx_gemm(w + a.pc, w + a.ps, w + a.vc + kv * v_codes, w + a.vs + kv * v_scales, L, d, L, 32, k_pv, oh,
                                   d, w + a.gemm, gemm_bytes, stream);
             }
             if (rc != AMX_OK) return rc;
+            ++i;
         }
         h0 += hc;
     }
@@ -643,10 +717,11 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
                                  size_t prepared_bytes, void* workspace, size_t workspace_bytes, void* stream) {
     const int causal = (flags & AMX_ATTN_CAUSAL) ? 1 : 0;
     if (flags & ~AMX_ATTN_CAUSAL) return AMX_ERR_FLAGS;
-    if (L <= 0 || d <= 0 || !attn_fused_supported(L, d)) return AMX_ERR_SHAPE;
+    if (L <= 0 || d != 128 || L % 128 || !attn_fused_supported(L, d)) return AMX_ERR_SHAPE;
     if (!q || !k || !v || !o || !p_prepared) return AMX_ERR_NULL;
-    const AttnLayout a = attn_layout(L, d);
-    if (!workspace || workspace_bytes < a.total || prepared_bytes < amx_prepared_bytes(L, L, 32, 0)) return AMX_ERR_WORKSPACE;
+    const AttnLayout a = attn_layout_fused(L, d);
+    if (!workspace || workspace_bytes < amx_attention_workspace_bytes(L, d) || prepared_bytes < amx_prepared_bytes(L, L, 32, 0))
+        return AMX_ERR_WORKSPACE;
     if (!aligned(workspace, kAlign) || !aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(o, 16) ||
         !aligned(p_prepared, kAlign) || !aligned(p_bf16, 16) || !aligned(p_codes, 16) || !aligned(p_scales, 2))
         return AMX_ERR_ALIGN;
@@ -661,13 +736,14 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     }
     // one head through the launch sequence of amx_attention: casts of Q, K (along head_dim) and V (along the
     // sequence), then the two passes
+    int* words = reinterpret_cast<int*>(w + a.gemm);
+    if (cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
     int rc = gemm_fp4_quantize_prepared(q, L, d, false, nullptr, w + a.qs, w + a.pq, st);
     if (rc == AMX_OK) rc = gemm_fp4_quantize_prepared(k, L, d, true, nullptr, w + a.ks, w + a.pk, st);
-    if (rc == AMX_OK) rc = quantize_cols_batched(v, 1, L, d, w + a.vc, w + a.vs, st);
-    if (rc == AMX_OK) rc = gemm_fp4_prepare(w + a.vc, w + a.vs, d, L, true, w + a.pv, st);
+    if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(v, 1, L, d, 128, 128, w + a.vs, w + a.pv, st, nullptr);
     if (rc != AMX_OK) return rc;
-    return attn_fused({w + a.pq, L, L, 0}, {w + a.pk, L, L, 0}, {w + a.pv, d, d, 0}, 1, L, 1.0f / sqrtf((float)d), causal,
-                      w + a.stats, o, w + a.gemm, st, p_bf16, p_codes, p_scales, p_prepared);
+    return attn_fused({w + a.pq, L, L, 0}, {w + a.pk, L, L, 0}, {w + a.pv, 128, 128, 0}, 1, L, d, 1.0f / sqrtf((float)d), causal,
+                      w + a.stats, o, words, st, p_bf16, p_codes, p_scales, p_prepared);
 }
 
 extern "C" int amx_gemm_status(const void* workspace, void* stream) {

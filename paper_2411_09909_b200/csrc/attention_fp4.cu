@@ -1,4 +1,4 @@
-// Fully quantized attention on the FP4 tensor-core pipe for head dimension 128 (arXiv 2411.09909, Appendix C:
+// Fully quantized attention on the FP4 tensor-core pipe for head dimensions 128 and 64 (arXiv 2411.09909, Appendix C:
 // Query, Key, the self-attention map and Value are all cast to AMXFP4; Section 1: at long context these products
 // are a large share of the prefill work).  Neither the logits nor the attention map ever reach global memory.
 //
@@ -9,7 +9,11 @@
 //           negative element: one sign plane), written to shared memory in the layout the MMA reads, its scale
 //           factors copied to tensor memory, and O += P V on the tensor cores in the same kernel.
 // Both products use the sign split of the GEMM (gemm_fp4.cu): S = Q+K+ + Q+K- + Q-K+ + Q-K- (8 block-scaled MMAs
-// per 128 x 128 tile at K = 128), O += P V+ + P V- (4 MMAs per tile of 128 keys).
+// per 128 x 128 tile at K = 128, 4 at K = 64), O += P V+ + P V- (4 MMAs per tile of 128 keys).
+// Any sequence length: every head's Q and K rows are padded to whole 128-row blocks (zero scale factors, zero row
+// words), V^T to 128 rows; keys past the sequence are masked in the last key tile, queries past it are not stored.
+// At head dimension 64 the K tile's rows are half as long (the TMA box fills the rest with zeros and one K step is
+// issued) and O is 64 columns wide.
 //
 // One persistent CTA per SM walks over (head, block of 128 queries) items; per item it loops over the key tiles:
 //   warp 0      TMA: the item's Q tile; per key tile the K tile and (pass 2) the V^T tile, {+, -} planes each, into a
@@ -40,7 +44,8 @@ namespace {
 using namespace tc;
 using namespace fp4;
 
-constexpr int BM = 128, BNK = 128, HD = 128;         // queries per item, keys per tile, head dimension
+constexpr int BM = 128, BNK = 128;                   // queries per item, keys per tile
+constexpr int kVRows = 128;                           // rows of one head of V^T (padded at head dimension 64)
 constexpr int kStages = 3;
 // Ring of the per-tile column factors: its writers (scale-factor warps) run at most kStages tiles ahead of the MMAs
 // and those at most 2 tiles ahead of the readers (epilogue), so 8 slots never collide and need no barrier of their own.
@@ -77,22 +82,24 @@ static_assert(sizeof(Control) <= 512, "Control must fit its reserved space");
 __device__ __forceinline__ uint64_t desc_sw64(uint32_t addr) {
     return (uint64_t)((addr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
 }
-// kind::mxf4nvf4 block-scaled, A and B E2M1, K-major, UE4M3 scale factors, M = N = 128, K = 64 per instruction
-constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// kind::mxf4nvf4 block-scaled, A and B E2M1, K-major, UE4M3 scale factors, M = 128, K = 64 per instruction
+__host__ __device__ constexpr uint32_t idesc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24); }
 
 struct Params {
     // prepared operands (fp4_operand.cuh); row ranges of stacked heads: head h of the launch has its queries at
-    // rows q_row0 + h * L of Q, its keys at k_row0 + (h / kv_group) * L of K, its 128 V^T rows at
+    // rows q_row0 + h * Lp of Q, its keys at k_row0 + (h / kv_group) * Lp of K, its V^T rows at
     // v_row0 + (h / kv_group) * 128 (kv_group query heads share one head of keys and values: grouped-query attention)
     const uint8_t *sfq[2], *sfk[2], *sfv[2];         // scale-factor chunks of the planes, from the operand's first chunk
     const int *q_words, *k_words, *v_words;          // row words, from the operand's first row
     int64_t q_row0, k_row0, v_row0;
     int nk64_q, nk64_k, nk64_v;
-    int heads, m_tiles, causal, kv_group;
-    int64_t L;
+    int vec_o;               // O is 16-byte aligned
+    int heads, m_tiles, kv_group;
+    int64_t L, Lp;           // sequence length, and padded to whole blocks of 128
     float alpha;
-    float2* part;            // [heads * L][4]: per row and key-group column {max, sum of 2^(t - max)}, base-2 units
-    float* O;                // pass 2 out: [heads][L][128]
+    const int* gate;         // not NULL: nothing is done when this word is nonzero (the caller runs the exact kernel then)
+    float2* part;            // [heads * Lp][4]: per row and key-group column {max, sum of 2^(t - max)}, base-2 units
+    float* O;                // pass 2 out: [heads][L][head dimension]
     int* status;
     // optional outputs of pass 2 for head 0 of the launch (verification): the bf16 map the cast started from
     // [L][L/2 words], canonical codes [L][L/32] x 16 bytes, scale bytes, and the prepared form of P (plane, scale
@@ -104,21 +111,30 @@ struct Params {
     int p_nk64;
 };
 
-template <int PASS, bool CAUSAL>
+// Which keys a tile masks: none (whole tiles, no causal mask), the causal diagonal, or those past a ragged sequence.
+enum Mask { kMaskNone, kMaskCausal, kMaskTail };
+
+template <int PASS, int MASK, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const Params p) {
     using S_ = Smem<PASS>;
+    constexpr bool CAUSAL = MASK == kMaskCausal;
+    constexpr int kQkSteps = HD / 64;                     // MMAs along the head dimension per sign pair
+    if (p.gate && *p.gate != 0) return;                   // uniform over the grid: nothing was set up yet
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Control* ctl = reinterpret_cast<Control*>(sm + S_::kOffCtl);
     float* kc_all = reinterpret_cast<float*>(sm + S_::kOffKc);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_items = p.heads * p.m_tiles;
-    // item -> (head, query block); under a causal mask the long items (late query blocks) come first
+    // The CTA's item number ii: a boustrophedon over the CTAs, so that under a causal mask - long items (late query blocks)
+    // first - a CTA that starts with a long item goes on with a short one.
+    auto item_id = [&](int ii) { return ii * (int)gridDim.x + ((ii & 1) ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x); };
+    // item -> (head, query block)
     auto item_head = [&](int id) { return id % p.heads; };
-    auto item_m = [&](int id) { const int mi = id / p.heads; return (CAUSAL && p.causal) ? p.m_tiles - 1 - mi : mi; };
-    auto tiles_of = [&](int m_blk) { return (CAUSAL && p.causal) ? m_blk + 1 : (int)(p.L / BNK); };
+    auto item_m = [&](int id) { const int mi = id / p.heads; return CAUSAL ? p.m_tiles - 1 - mi : mi; };
+    auto tiles_of = [&](int m_blk) { return CAUSAL ? m_blk + 1 : p.m_tiles; };
 
     if (threadIdx.x == 0) {
         mbar_init(&ctl->q_full, 1 + kSfWarps);
@@ -149,12 +165,12 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         if (lane == 0) {
             int it = 0, ii = 0;
             bool ok = true;
-            for (int id = blockIdx.x; id < n_items && ok; id += gridDim.x, ++ii) {
+            for (int id = item_id(ii); id < n_items && ok; id = item_id(++ii)) {
                 const int h = item_head(id), m_blk = item_m(id);
                 // the previous item's logits MMAs have read the Q tile
                 if (ii > 0 && !mbar_wait(&ctl->q_empty, (ii - 1) & 1, &ctl->abort, p.status)) break;
                 mbar_expect_tx(&ctl->q_full, kTileBytes);
-                tma_load_3d(sm + S_::kOffQ, &tm_q, 0, (int)(p.q_row0 + (int64_t)h * p.L + m_blk * BM), 0, &ctl->q_full);
+                tma_load_3d(sm + S_::kOffQ, &tm_q, 0, (int)(p.q_row0 + (int64_t)h * p.Lp + m_blk * BM), 0, &ctl->q_full);
                 const int T = tiles_of(m_blk);
                 for (int j = 0; j < T; ++j, ++it) {
                     const int s = it % kStages;
@@ -164,8 +180,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     }
                     uint8_t* st = sm + S_::kOffKV + s * S_::kStageBytes;
                     mbar_expect_tx(&ctl->kv_full[s], S_::kStageBytes);
-                    tma_load_3d(st, &tm_k, 0, (int)(p.k_row0 + (int64_t)(h / p.kv_group) * p.L + j * BNK), 0, &ctl->kv_full[s]);
-                    if (PASS == 2) tma_load_3d(st + kTileBytes, &tm_v, j * 64, (int)(p.v_row0 + (int64_t)(h / p.kv_group) * HD), 0, &ctl->kv_full[s]);
+                    tma_load_3d(st, &tm_k, 0, (int)(p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK), 0, &ctl->kv_full[s]);
+                    if (PASS == 2) tma_load_3d(st + kTileBytes, &tm_v, j * 64, (int)(p.v_row0 + (int64_t)(h / p.kv_group) * kVRows), 0, &ctl->kv_full[s]);
                 }
             }
             // after a timeout: let the copies already in flight land before shared memory is released
@@ -198,9 +214,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 #pragma unroll
                     for (int pw = 0; pw < 2; ++pw)
 #pragma unroll
-                        for (int kk = 0; kk < 2; ++kk) {
+                        for (int kk = 0; kk < kQkSteps; ++kk) {
                             mma_fp4_block16(tmem + kColS + b * 128, desc_sw64(q_addr + pa * kPlane + kk * 32),
-                                            desc_sw64(k_addr + pw * kPlane + kk * 32), kIdesc, sfq + (pa * 2 + kk) * 4,
+                                            desc_sw64(k_addr + pw * kPlane + kk * 32), idesc(128), sfq + (pa * 2 + kk) * 4,
                                             sfk + (pw * 2 + kk) * 4, acc);
                             acc = 1;
                         }
@@ -229,7 +245,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk) {
                         mma_fp4_block16(tmem + kColO, desc_sw64(p_addr + kk * 32), desc_sw64(v_addr + pv * kPlane + kk * 32),
-                                        kIdesc, sfp + kk * 4, sfv + (pv * 2 + kk) * 4, acc);
+                                        idesc(HD), sfp + kk * 4, sfv + (pv * 2 + kk) * 4, acc);
                         acc = 1;
                     }
                 mma_commit(&ctl->kv_empty[s]);
@@ -237,7 +253,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             __syncwarp();
         };
-        for (int id = blockIdx.x; id < n_items; id += gridDim.x, ++ii) {
+        for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
             const int T = tiles_of(item_m(id));
             if (ok) ok = mbar_wait(&ctl->q_full, ii & 1, &ctl->abort, p.status);
             // the logits run two key tiles ahead of P V (both accumulators in use); after the item's last S the Q
@@ -268,9 +284,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         auto chunk = [&](const uint8_t* sf, int64_t row0, int nk64, int k64) {
             return __ldg(reinterpret_cast<const uint4*>(sf + ((row0 >> 7) * nk64 + k64) * (int64_t)kSfChunk + lane * 16));
         };
-        for (int id = blockIdx.x; id < n_items; id += gridDim.x, ++ii) {
+        for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
             const int h = item_head(id), m_blk = item_m(id);
-            const int64_t q_row = p.q_row0 + (int64_t)h * p.L + m_blk * BM;
+            const int64_t q_row = p.q_row0 + (int64_t)h * p.Lp + m_blk * BM;
             uint4 v[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[i] = chunk(p.sfq[i >> 1], q_row, p.nk64_q, i & 1);
@@ -287,13 +303,13 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const int T = tiles_of(m_blk);
             for (int j = 0; j < T; ++j, ++it) {
                 const int s = it % kStages;
-                const int64_t k_row = p.k_row0 + (int64_t)(h / p.kv_group) * p.L + j * BNK;
+                const int64_t k_row = p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK;
                 uint4 vk[4], vv[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) vk[i] = chunk(p.sfk[i >> 1], k_row, p.nk64_k, i & 1);
                 if (PASS == 2) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) vv[i] = chunk(p.sfv[i >> 1], p.v_row0 + (int64_t)(h / p.kv_group) * HD, p.nk64_v, j * 2 + (i & 1));
+                    for (int i = 0; i < 4; ++i) vv[i] = chunk(p.sfv[i >> 1], p.v_row0 + (int64_t)(h / p.kv_group) * kVRows, p.nk64_v, j * 2 + (i & 1));
                 }
                 const int kw = row_word_exp(__ldg(p.k_words + k_row + t));
                 if (ok && it >= kStages) ok = mbar_wait(&ctl->kv_empty[s], ((it / kStages) - 1) & 1, &ctl->abort, p.status);
@@ -327,10 +343,10 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(y));
             return v;
         };
-        for (int id = blockIdx.x; id < n_items; id += gridDim.x, ++ii) {
+        for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
             const int h = item_head(id), m_blk = item_m(id);
             const int64_t m = (int64_t)m_blk * BM + r;                // query index inside the head
-            const int64_t grow = (int64_t)h * p.L + m;               // row of the launch's stacked heads
+            const int64_t grow = (int64_t)h * p.Lp + m;              // row of the launch's stacked heads
             const int a_exp = row_word_exp(__ldg(p.q_words + p.q_row0 + grow));
             const float ra = __uint_as_float((uint32_t)(a_exp + 127) << 23);
             // pass 2: the row's statistics, merged from the four partial results of pass 1 in a fixed order
@@ -379,8 +395,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         u2[2 * c] = cast::mul_f32x2(cast::pack_f32x2(acc[4 * c], acc[4 * c + 1]), k2.x);
                         u2[2 * c + 1] = cast::mul_f32x2(cast::pack_f32x2(acc[4 * c + 2], acc[4 * c + 3]), k2.y);
                     }
-                    if (CAUSAL && p.causal && j == m_blk) {            // the diagonal tile: keys after the query are masked
-                        const int n_local = (int)(m - (int64_t)j * BNK) - cg * 32;   // last visible column of this group
+                    // the diagonal tile: keys after the query are masked; the last tile of a ragged sequence: keys past it
+                    if (MASK != kMaskNone && j == (CAUSAL ? m_blk : T - 1)) {
+                        const int n_local = (int)((CAUSAL ? m : p.L - 1) - (int64_t)j * BNK) - cg * 32;   // last visible column of this group
 #pragma unroll
                         for (int c = 0; c < 16; ++c) {
                             float lo, hi;
@@ -480,26 +497,34 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 if (ok) ok = mbar_wait(&ctl->o_full, ii & 1, &ctl->abort, p.status);
                 if (!ok) continue;
                 tc_fence_after();
-                uint32_t acc[32];
-                tmem_ld32(tq + kColO + cg_o * 32, acc);
+                constexpr int kCols = HD / 4;                          // columns of O per warp
+                uint32_t acc[kCols];
+                if constexpr (HD == 128) tmem_ld32(tq + kColO + cg_o * kCols, acc);
+                else tmem_ld16(tq + kColO + cg_o * kCols, acc);
                 tmem_ld_wait();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl->o_empty);
-                const int4* vw = reinterpret_cast<const int4*>(p.v_words + p.v_row0 + (int64_t)(h / p.kv_group) * HD + cg_o * 32);
-                float* out = p.O + ((int64_t)h * p.L + m) * HD + cg_o * 32;
+                const int4* vw = reinterpret_cast<const int4*>(p.v_words + p.v_row0 + (int64_t)(h / p.kv_group) * kVRows + cg_o * kCols);
+                float* out = p.O + ((int64_t)h * p.L + m) * HD + cg_o * kCols;
                 const int p_exp = kmax ? kmax - 25 : 0;
+                if (MASK == kMaskNone || m < p.L) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int4 w4 = __ldg(vw + c);
-                    const int ex[4] = {row_word_exp(w4.x), row_word_exp(w4.y), row_word_exp(w4.z), row_word_exp(w4.w)};
-                    float f[4];
+                    for (int c = 0; c < kCols / 4; ++c) {
+                        const int4 w4 = __ldg(vw + c);
+                        const int ex[4] = {row_word_exp(w4.x), row_word_exp(w4.y), row_word_exp(w4.z), row_word_exp(w4.w)};
+                        float f[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int sh = min(127, max(-126, p_exp + ex[i]));
-                        f[i] = __uint_as_float(acc[4 * c + i]) * __uint_as_float((uint32_t)(sh + 127) << 23);
+                        for (int i = 0; i < 4; ++i) {
+                            const int sh = min(127, max(-126, p_exp + ex[i]));
+                            f[i] = __uint_as_float(acc[4 * c + i]) * __uint_as_float((uint32_t)(sh + 127) << 23);
+                        }
+                        if (p.vec_o) *reinterpret_cast<float4*>(out + 4 * c) = make_float4(f[0], f[1], f[2], f[3]);
+                        else {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) out[4 * c + i] = f[i];
+                        }
                     }
-                    *reinterpret_cast<float4*>(out + 4 * c) = make_float4(f[0], f[1], f[2], f[3]);
                 }
             }
         }
@@ -512,12 +537,12 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
 }
 
-template <int PASS, bool CAUSAL>
+template <int PASS, int MASK, int HD>
 int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev, int sms,
                 cudaStream_t st) {
     static bool configured[64] = {};
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(attention_fp4_kernel<PASS, CAUSAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<PASS>::kBytes) !=
+        if (cudaFuncSetAttribute(attention_fp4_kernel<PASS, MASK, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<PASS>::kBytes) !=
             cudaSuccess) {
             cudaGetLastError();
             return AMX_ERR_CUDA;
@@ -525,40 +550,59 @@ int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensor
         configured[dev] = true;
     }
     const int items = p.heads * p.m_tiles;
-    attention_fp4_kernel<PASS, CAUSAL><<<(unsigned)(items < sms ? items : sms), kThreads, Smem<PASS>::kBytes, st>>>(tm_q, tm_k, tm_v, p);
+    attention_fp4_kernel<PASS, MASK, HD><<<(unsigned)(items < sms ? items : sms), kThreads, Smem<PASS>::kBytes, st>>>(tm_q, tm_k, tm_v, p);
     return launch_status();
 }
 
 }  // namespace
 
-bool attn_fused_supported(int64_t L, int64_t d) { return d == HD && L > 0 && L % BNK == 0 && L / BNK <= 32767; }
+bool attn_fused_supported(int64_t L, int64_t d) {
+    return (d == 128 || d == 64) && L > 0 && L % 32 == 0 && L / BNK <= 32766;
+}
+
+int64_t attn_fused_padded(int64_t L) { return (L + BM - 1) / BM * BM; }
 
 // per-row partial softmax statistics of the heads of one launch
-size_t attn_fused_scratch_bytes(int64_t heads, int64_t L) { return up256((size_t)heads * L * 4 * sizeof(float2)); }
+size_t attn_fused_scratch_bytes(int64_t heads, int64_t L) { return up256((size_t)heads * attn_fused_padded(L) * 4 * sizeof(float2)); }
 
-// Attention for `heads` stacked heads whose operands were prepared ahead: q (left-hand layout, heads * L rows, K = 128),
-// k (right-hand layout, same rows), vt (right-hand layout, heads * 128 rows of V^T, K = L).  O: fp32 [heads][L][128].
-// workspace: 256 bytes (status word).  dbg_*: optional verification outputs for head 0 (see Params).
-int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, float alpha, int causal,
-               void* scratch, float* O, void* workspace, cudaStream_t st, void* dbg_bits, uint8_t* dbg_codes, uint8_t* dbg_scales,
-               void* dbg_prepared, int kv_group) {
-    if (!attn_fused_supported(L, HD) || heads <= 0 || q.row0 % 128 || k.row0 % 128 || vt.row0 % 128) return AMX_ERR_SHAPE;
+namespace {
+template <int MASK, int HD>
+int launch_both(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev, int sms,
+                cudaStream_t st) {
+    const int rc = launch_pass<1, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+    return rc != AMX_OK ? rc : launch_pass<2, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+}
+template <int HD>
+int launch_mask(int mask, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev,
+                int sms, cudaStream_t st) {
+    return mask == kMaskCausal ? launch_both<kMaskCausal, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
+         : mask == kMaskTail   ? launch_both<kMaskTail, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
+                               : launch_both<kMaskNone, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+}
+}  // namespace
+
+// Attention for `heads` stacked heads whose operands were prepared ahead, Lp = attn_fused_padded(L) rows per head: q
+// (left-hand layout, K = d), k (right-hand layout), vt (right-hand layout, 128 rows of V^T per head, K = L).  O: fp32
+// [heads][L][d].  workspace: 256 bytes (status word).  dbg_*: optional verification outputs for head 0 (see Params).
+int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, int64_t d, float alpha,
+               int causal, void* scratch, float* O, void* workspace, cudaStream_t st, void* dbg_bits, uint8_t* dbg_codes,
+               uint8_t* dbg_scales, void* dbg_prepared, int kv_group, const int* gate) {
+    if (!attn_fused_supported(L, d) || heads <= 0 || q.row0 % 128 || k.row0 % 128 || vt.row0 % 128) return AMX_ERR_SHAPE;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
     static int sm_count[64] = {};
     if (!sm_count[dev] && cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return AMX_ERR_CUDA;
-    const OperandLayout oq = operand_layout(q.layout_rows, HD, 128), ok_ = operand_layout(k.layout_rows, HD, 256),
+    const OperandLayout oq = operand_layout(q.layout_rows, d, 128), ok_ = operand_layout(k.layout_rows, d, 256),
                         ov = operand_layout(vt.layout_rows, L, 256);
     const uint8_t* pq = static_cast<const uint8_t*>(q.prepared);
     const uint8_t* pk = static_cast<const uint8_t*>(k.prepared);
     const uint8_t* pv = static_cast<const uint8_t*>(vt.prepared);
     CUtensorMap tm_q, tm_k, tm_v;
-    if (!make_map(&tm_q, pq, q.rows_total, HD, oq.plane, 128, 64) || !make_map(&tm_k, pk, k.rows_total, HD, ok_.plane, 128, 64) ||
+    if (!make_map(&tm_q, pq, q.rows_total, d, oq.plane, 128, 64) || !make_map(&tm_k, pk, k.rows_total, d, ok_.plane, 128, 64) ||
         !make_map(&tm_v, pv, vt.rows_total, L, ov.plane, 128, 64))
         return AMX_ERR_CUDA;
-    int* status = static_cast<int*>(workspace);
-    if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;
+    int* status = static_cast<int*>(workspace);              // cleared by the caller
     Params p{};
     p.sfq[0] = pq + 2 * oq.plane;   p.sfq[1] = p.sfq[0] + oq.sf;
     p.sfk[0] = pk + 2 * ok_.plane;  p.sfk[1] = p.sfk[0] + ok_.sf;
@@ -568,11 +612,12 @@ int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, i
     p.v_words = reinterpret_cast<const int*>(pv + 2 * ov.plane + 2 * ov.sf);
     p.q_row0 = q.row0; p.k_row0 = k.row0; p.v_row0 = vt.row0;
     p.nk64_q = oq.nk64; p.nk64_k = ok_.nk64; p.nk64_v = ov.nk64;
-    p.heads = heads; p.m_tiles = (int)(L / BM); p.causal = causal ? 1 : 0;
+    p.heads = heads; p.Lp = attn_fused_padded(L); p.m_tiles = (int)(p.Lp / BM); p.gate = gate;
     p.kv_group = kv_group > 0 ? kv_group : 1;
     p.L = L; p.alpha = alpha;
     p.part = static_cast<float2*>(scratch);
     p.O = O;
+    p.vec_o = aligned(O, 16);
     p.status = status;
     if (dbg_prepared) {
         const OperandLayout op = operand_layout(L, L, 128);
@@ -585,11 +630,9 @@ int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, i
         p.p_codes = reinterpret_cast<uint4*>(dbg_codes);
         p.p_scales = reinterpret_cast<uint16_t*>(dbg_scales);
     }
-    int rc = causal ? launch_pass<1, true>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st)
-                    : launch_pass<1, false>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st);
-    if (rc != AMX_OK) return rc;
-    return causal ? launch_pass<2, true>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st)
-                  : launch_pass<2, false>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st);
+    const int mask = causal ? kMaskCausal : L % BNK ? kMaskTail : kMaskNone;
+    return d == 128 ? launch_mask<128>(mask, tm_q, tm_k, tm_v, p, dev, sm_count[dev], st)
+                    : launch_mask<64>(mask, tm_q, tm_k, tm_v, p, dev, sm_count[dev], st);
 }
 
 }  // namespace amx

@@ -47,24 +47,33 @@ int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_c
              void* workspace, cudaStream_t st, bool gate_on_flushed = false, int gs = 32);
 // The same in two phases, so that an operand (typically the weight) is prepared once and reused.
 size_t gemm_fp4_prepared_bytes(int64_t rows, int64_t K, bool is_weight);
+size_t gemm_fp4_plane_bytes(int64_t rows, int64_t K);
 // flushed_total (optional, device): incremented by the number of nonzero scales that fell below the UE4M3 range
 // of their row and were flushed; the per-row counts are in the row words either way.
 int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
                      void* prepared, cudaStream_t st, int64_t layout_rows = 0 /* 0: rows */, int* flushed_total = nullptr, int gs = 32);
 int gemm_fp4_quantize_prepared(const void* x, int64_t rows, int64_t K, bool is_weight, uint8_t* codes,
                                uint8_t* scales, void* prepared, cudaStream_t st, int64_t layout_rows = 0,
-                               int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr);
+                               int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr,
+                               int64_t seg_rows = 0, int64_t seg_pad = 0 /* not 0: x holds segments of seg_rows rows, each padded
+                               to seg_pad operand rows (`rows` counts operand rows) with zero scale factors and row words */);
+int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64_t d, int64_t seg_pad, int64_t layout_rows,
+                                  uint8_t* scales, void* prepared, cudaStream_t st, int* flushed_total);
+int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int64_t seg_pad, void* pos, void* neg, uint8_t* scales,
+                         cudaStream_t st);
 int quantize_rows_prepared(const void* x, int64_t rows, int64_t K, uint8_t* codes, uint8_t* scales, void* pos,
                            void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows,
-                           cudaStream_t st, int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr);
+                           cudaStream_t st, int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr, int64_t seg_rows = 0,
+                           int64_t seg_pad = 0);
 const int* gemm_fp4_row_words(const void* prepared, int64_t rows, int64_t K, bool is_weight);
 // Softmax of the rows of S, rounded to bf16 and cast in one launch (cols % 32 == 0); pos == nullptr: canonical
 // output only.  gemm_fp4_softmax_prepared lays the prepared operand out like gemm_fp4_quantize_prepared.
 int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, float alpha, uint8_t* codes,
                       uint8_t* scales, void* pos, void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64,
-                      int64_t padded_rows, cudaStream_t st, int causal = 0);
+                      int64_t padded_rows, cudaStream_t st,
+                      int64_t causal = 0 /* rows per matrix: row i of a matrix sees columns 0 .. i */);
 int gemm_fp4_softmax_prepared(const float* S, int64_t rows, int64_t cols, int64_t ld_s, float alpha, bool is_weight,
-                              uint8_t* codes, uint8_t* scales, void* prepared, cudaStream_t st, int causal = 0);
+                              uint8_t* codes, uint8_t* scales, void* prepared, cudaStream_t st, int64_t causal = 0);
 // A prepared operand that stacks several matrices row-wise (rows_total rows, laid out for layout_rows >=
 // rows_total rows) and the first row of the one to multiply; row0 % 128 == 0.  A right-hand operand whose 256-row
 // tiles can reach past rows_total needs layout_rows >= rows_total + 128.
@@ -86,14 +95,30 @@ size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // C[m][n] = sum over `slices` partial products [slices][M][N], in slice order (defined with the bf16-decode kernel)
 int reduce_slices(const float* part, int slices, int64_t M, int64_t N, float* C, int64_t ld_c, cudaStream_t st,
                   const int* run_if_nonzero = nullptr);
-// Fused attention for head dimension 128 (attention_fp4.cu): both products and the softmax in two launches, logits
-// and attention map never in global memory.  Operands prepared ahead, heads stacked row-wise.
+// Fused attention for head dimensions 128 and 64 (attention_fp4.cu): both products and the softmax in two launches, logits
+// and attention map never in global memory.  Operands prepared ahead, heads stacked row-wise, padded to whole blocks of 128.
 bool attn_fused_supported(int64_t L, int64_t d);
+int64_t attn_fused_padded(int64_t L);
 size_t attn_fused_scratch_bytes(int64_t heads, int64_t L);
-int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, float alpha, int causal,
-               void* scratch, float* O, void* workspace /* 256 B: status word */, cudaStream_t st, void* dbg_bits = nullptr,
-               uint8_t* dbg_codes = nullptr, uint8_t* dbg_scales = nullptr, void* dbg_prepared = nullptr,
-               int kv_group = 1 /* query heads per head of keys and values; k and vt then stack heads / kv_group heads */);
+int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, int64_t d, float alpha,
+               int causal, void* scratch, float* O, void* workspace /* 256 B: status word, cleared by the caller */,
+               cudaStream_t st, void* dbg_bits = nullptr, uint8_t* dbg_codes = nullptr, uint8_t* dbg_scales = nullptr,
+               void* dbg_prepared = nullptr, int kv_group = 1 /* query heads per head of keys and values */,
+               const int* gate = nullptr /* device word: the kernels do nothing when it is nonzero */);
+// The same attention on CUDA cores from the planes (or-ed: the codes) and canonical scales of those operands, any scale
+// range; nothing is done when *run_if_nonzero is zero.  attention_exact.cu
+struct ExactOperand {
+    const uint8_t *pos, *neg, *scales;
+};
+bool attn_exact_supported(int64_t L, int64_t d);
+int attn_exact(const ExactOperand& q, const ExactOperand& k, const ExactOperand& vt, int heads, int64_t L, int64_t d, int kv_group,
+               float alpha, int causal, float* O, const int* run_if_nonzero, cudaStream_t st);
+// Batched bf16-decode products (gemm_tc.cu): `batch` left operands one after another, right operand (first + b) / group for
+// product b.  causal: tiles that lie entirely above the diagonal are left out (C there is not written).
+size_t gemm_tc_batched_workspace_bytes(int64_t batch, int64_t M, int64_t N, int64_t K);
+int gemm_tc_batched(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales, int64_t batch,
+                    int64_t first, int64_t group, int64_t M, int64_t N, int64_t K, float* C, bool causal, void* workspace,
+                    cudaStream_t st);
 int quantize_cols_batched(const void* x, int64_t batch, int64_t R, int64_t C, uint8_t* codes, uint8_t* scales,
                           cudaStream_t st);
 int gemm_fp4_prepared(const void* a_prepared, const void* w_prepared, int64_t M, int64_t N, int64_t K,

@@ -116,21 +116,25 @@ __host__ __device__ constexpr uint32_t instr_desc(int n) { return (1u << 7) | (1
 //   3. scale factors of both planes in the layout the MMA reads:
 //      [plane][row block of 128][K/64 block][512 B], byte (r%32)*16 + (r/32)*4 + (k16 % 4);
 //      one scale per 16 elements, so a group's scale is written gs / 16 times (GS = 16: the MMA's own block)
+// PLANES = false: the sign planes are there already, steps 1 and 3 only.
 constexpr int kPrepRows = 8;
-template <int GS>
+template <int GS, bool PLANES = true>
 __global__ void __launch_bounds__(256)
 prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int64_t R, int64_t K,
                        int nk64, uint4* __restrict__ pos, uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos,
-                       uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total) {
+                       uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total,
+                       int seg_rows = 0, int seg_pad = 0) {
     __shared__ int kmax_s[kPrepRows];
     __shared__ int unsplit_s[kPrepRows];
     const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / GS;         // G: scale pairs per row
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // seg_pad: operand rows come in segments of seg_pad rows of which the first seg_rows are in use
+    auto in_use = [&](int64_t row) { return row < R && (!seg_pad || (int)(row % seg_pad) < seg_rows); };
     for (int r = warp; r < kPrepRows; r += 8) {
         const int64_t row = row0 + r;
         int kmax = 0, sides = 0;
         uint32_t differ = 0;
-        if (row < R) {
+        if (in_use(row)) {
             const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
             for (int64_t g = lane; g < G; g += 32) {
                 const uint32_t v = __ldg(s2 + g);
@@ -144,11 +148,12 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
         differ = __reduce_or_sync(0xFFFFFFFFu, differ);
         // A row whose two scales agree in every group (a symmetric format) needs no split: sum over both signs of
         // code x scale_side = code x scale.  Its signed codes go to the positive plane as they are.
-        const bool unsplit = !differ;
+        // (Planes that are there already were split, whatever the scales.)
+        const bool unsplit = PLANES && !differ;
         if (unsplit) sides &= kRowHasPos;
         // nonzero scales that the row's offset pushes below the UE4M3 range (they are flushed in step 3)
         int flushed = 0;
-        if (row < R) {
+        if (in_use(row)) {
             const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
             for (int64_t g = lane; g < G; g += 32) {
                 const uint32_t v = __ldg(s2 + g);
@@ -159,7 +164,7 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
         if (lane == 0) {
             kmax_s[r] = kmax;
             unsplit_s[r] = unsplit;
-            if (row < R) row_exp[row] = row_word(kmax, sides, flushed);
+            if (in_use(row)) row_exp[row] = row_word(kmax, sides, flushed);
             if (flushed && flushed_total) atomicAdd(flushed_total, flushed);
         }
     }
@@ -167,7 +172,7 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
     __syncthreads();                                             // unsplit_s is complete
     const int64_t rows_here = min((int64_t)kPrepRows, R - row0);
     const int vec_per_row = (int)(K / 32);
-    if (rows_here > 0) {
+    if (PLANES && rows_here > 0) {
         const int64_t v0 = row0 * vec_per_row, n_vec = rows_here * vec_per_row;
         const uint4* src = reinterpret_cast<const uint4*>(codes) + v0;
         for (int64_t i = threadIdx.x; i < n_vec; i += 256) {
@@ -194,7 +199,7 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
         const int c = item / kPrepRows, r = item % kPrepRows;
         const int64_t row = row0 + r;
         uint32_t wp = 0, wn = 0;
-        if (row < R) {
+        if (in_use(row)) {
             const int kmax = kmax_s[r];
 #pragma unroll
             for (int h = 0; h < kPer; ++h) {
@@ -679,7 +684,7 @@ int prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K
     kernel<<<(unsigned)(padded_rows / kPrepRows), 256, 0, st>>>(
         codes, scales, rows, K, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
         base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf),
-        flushed_total);
+        flushed_total, 0, 0);
     return launch_status();
 }
 
@@ -828,13 +833,31 @@ size_t gemm_fp4_prepared_bytes(int64_t rows, int64_t K, bool is_weight) {
 
 // Fused form: one launch of the cast kernel writes the canonical operand and the prepared one.
 int gemm_fp4_quantize_prepared(const void* x, int64_t rows, int64_t K, bool is_weight, uint8_t* codes, uint8_t* scales,
-                               void* prepared, cudaStream_t st, int64_t layout_rows, int format, int* flushed_total) {
+                               void* prepared, cudaStream_t st, int64_t layout_rows, int format, int* flushed_total,
+                               int64_t seg_rows, int64_t seg_pad) {
     const OperandLayout o = operand_layout(layout_rows ? layout_rows : rows, K, is_weight ? BN : BM);
     uint8_t* base = static_cast<uint8_t*>(prepared);
     return quantize_rows_prepared(x, rows, K, codes, scales, base, base + o.plane, base + 2 * o.plane,
                                   base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), o.nk64,
-                                  o.row_blocks * 128, st, format, flushed_total);
+                                  seg_pad ? (rows + 127) / 128 * 128 : o.row_blocks * 128, st, format, flushed_total, seg_rows, seg_pad);
 }
+
+// V^T of `heads` heads [L, d], seg_pad operand rows each: cast down the rows into the planes and scales, then row words and
+// scale factors from the scales.  (The rows past d of a head, and their words, are whatever they were: not read.)
+int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64_t d, int64_t seg_pad, int64_t layout_rows,
+                                  uint8_t* scales, void* prepared, cudaStream_t st, int* flushed_total) {
+    const OperandLayout o = operand_layout(layout_rows, L, BN);
+    uint8_t* base = static_cast<uint8_t*>(prepared);
+    const int rc = quantize_cols_planes(v, heads, L, d, seg_pad, base, base + o.plane, scales, st);
+    if (rc != AMX_OK) return rc;
+    prepare_operand_kernel<32, false><<<(unsigned)(heads * seg_pad / kPrepRows), 256, 0, st>>>(
+        nullptr, scales, heads * seg_pad, L, o.nk64, nullptr, nullptr, base + 2 * o.plane, base + 2 * o.plane + o.sf,
+        reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), flushed_total, (int)d, (int)seg_pad);
+    return launch_status();
+}
+
+// Bytes from the first to the second sign plane of a prepared operand.
+size_t gemm_fp4_plane_bytes(int64_t rows, int64_t K) { return operand_layout(rows, K, BM).plane; }
 
 // Row words of a prepared operand (rows of them, device memory).
 const int* gemm_fp4_row_words(const void* prepared, int64_t rows, int64_t K, bool is_weight) {
@@ -843,7 +866,7 @@ const int* gemm_fp4_row_words(const void* prepared, int64_t rows, int64_t K, boo
 }
 
 int gemm_fp4_softmax_prepared(const float* S, int64_t rows, int64_t cols, int64_t ld_s, float alpha, bool is_weight,
-                              uint8_t* codes, uint8_t* scales, void* prepared, cudaStream_t st, int causal) {
+                              uint8_t* codes, uint8_t* scales, void* prepared, cudaStream_t st, int64_t causal) {
     const OperandLayout o = operand_layout(rows, cols, is_weight ? BN : BM);
     uint8_t* base = static_cast<uint8_t*>(prepared);
     return softmax_cast_rows(S, rows, cols, ld_s, alpha, codes, scales, base, base + o.plane, base + 2 * o.plane,

@@ -116,18 +116,27 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
                const uint16_t* __restrict__ a_x, int64_t ld_a,
                const uint8_t* __restrict__ w_codes, const uint8_t* __restrict__ w_scales,
                int64_t M, int64_t N, int64_t K, float* __restrict__ C, int64_t ld_c, int vec_store,
-               int* __restrict__ status, int kb_per_slice, int64_t slice_stride, const int* __restrict__ run_if_nonzero) {
+               int* __restrict__ status, int kb_per_slice, int64_t slice_stride, const int* __restrict__ run_if_nonzero,
+               int slices, int first, int group, int causal) {
     if (run_if_nonzero && *run_if_nonzero == 0) return;          // uniform over the grid: nothing was set up yet
-    // blockIdx.z: slice of the K range (kb_per_slice K blocks each); slice z writes its partial product to
-    // C + z * slice_stride (one slice: the result itself)
+    if (causal && (int64_t)blockIdx.x * BN > (int64_t)blockIdx.y * BM + BM - 1) return;   // a tile above the diagonal
+    // blockIdx.z: product of a batch (left operands and results one after another, `group` products share a right
+    // operand), then slice of the K range (kb_per_slice K blocks each); slice z of a product writes its partial product
+    // to C + z * slice_stride (one slice: the result itself)
+    const int batch = (int)blockIdx.z / slices, slice = (int)blockIdx.z - batch * slices;
+    a_codes += batch * (M * (K / 2));
+    a_scales += batch * (M * (K / 32) * 2);
+    w_codes += (first + batch) / group * (N * (K / 2));
+    w_scales += (first + batch) / group * (N * (K / 32) * 2);
+    C += batch * (int64_t)slices * M * N;                        // (a batch: ld_c == N)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Control* ctl = reinterpret_cast<Control*>(tiles + kStages * kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-    const int kb_begin = (int)blockIdx.z * kb_per_slice;
+    const int kb_begin = slice * kb_per_slice;
     const int num_kb = min((int)((K + BK - 1) / BK) - kb_begin, kb_per_slice);   // K blocks of this slice
-    C += (int64_t)blockIdx.z * slice_stride;
+    C += (int64_t)slice * slice_stride;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -281,6 +290,8 @@ reduce_slices_kernel(const float* __restrict__ part, int slices, int64_t M, int6
     if (run_if_nonzero && *run_if_nonzero == 0) return;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= M * N) return;
+    part += (int64_t)blockIdx.y * slices * M * N;                // grid y: product of a batch (ld_c == N)
+    C += (int64_t)blockIdx.y * M * N;
     float acc = part[i];
     for (int z = 1; z < slices; ++z) acc += part[(int64_t)z * M * N + i];
     C[(i / N) * ld_c + i % N] = acc;
@@ -296,9 +307,7 @@ size_t gemm_tc_workspace_bytes(int64_t M, int64_t N, int64_t K) {   // the statu
 
 namespace {
 
-int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a_x, int64_t ld_a,
-              const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C,
-              int64_t ld_c, void* workspace, cudaStream_t st, const int* gate = nullptr, int* status_word = nullptr) {
+int configure_tc() {
     static bool configured[64] = {};   // the opt-in to > 48 KB of dynamic shared memory is per device
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
@@ -308,6 +317,13 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
             return AMX_ERR_CUDA;
         configured[dev] = true;
     }
+    return AMX_OK;
+}
+
+int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a_x, int64_t ld_a,
+              const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C,
+              int64_t ld_c, void* workspace, cudaStream_t st, const int* gate = nullptr, int* status_word = nullptr) {
+    if (const int rc = configure_tc(); rc != AMX_OK) return rc;
     // status word: the first word of the workspace, cleared here, unless the caller shares one it cleared itself
     int* status = status_word ? status_word : static_cast<int*>(workspace);
     if (!status_word && cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;   // + flushed count: none
@@ -320,10 +336,10 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
     const int vec_store = aligned(out, 16) && ld_out % 4 == 0;   // else the epilogue stores scalars
     if (a_x)
         gemm_tc_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(nullptr, nullptr, a_x, ld_a, w_codes, w_scales, M, N, K, out,
-                                                                 ld_out, vec_store, status, kb_per, slice_stride, gate);
+                                                                 ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
     else
         gemm_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K,
-                                                                  out, ld_out, vec_store, status, kb_per, slice_stride, gate);
+                                                                  out, ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
     int rc = launch_status();
     if (rc != AMX_OK || slices == 1) return rc;
     return reduce_slices(part, slices, M, N, C, ld_c, st, gate);
@@ -352,6 +368,35 @@ int gemm_tc_cast(const void* x, int64_t ld_a, const uint8_t* w_codes, const uint
                  int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
     return launch_tc(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_a, w_codes, w_scales, M, N, K, C, ld_c,
                      workspace, st);
+}
+
+size_t gemm_tc_batched_workspace_bytes(int64_t batch, int64_t M, int64_t N, int64_t K) {
+    int kb_per;
+    const int slices = k_slices(M, N, K, kb_per);
+    return 256 + (slices > 1 ? (size_t)batch * slices * M * N * 4 : 0);
+}
+
+// The slices are those of one product, so that every result has the bits gemm_tc gives it.
+int gemm_tc_batched(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales, int64_t batch,
+                    int64_t first, int64_t group, int64_t M, int64_t N, int64_t K, float* C, bool causal, void* workspace,
+                    cudaStream_t st) {
+    int rc = configure_tc();
+    if (rc != AMX_OK) return rc;
+    int* status = static_cast<int*>(workspace);
+    if (cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;
+    int kb_per;
+    const int slices = k_slices(M, N, K, kb_per);
+    if (batch * slices > 65535) return AMX_ERR_SHAPE;
+    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM), (unsigned)(batch * slices));
+    float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
+    float* out = slices > 1 ? part : C;
+    gemm_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, out, N,
+                                                              aligned(out, 16) && N % 4 == 0 && (M * N) % 4 == 0, status, kb_per, M * N,
+                                                              nullptr, slices, (int)first, (int)group, causal);
+    rc = launch_status();
+    if (rc != AMX_OK || slices == 1) return rc;
+    reduce_slices_kernel<<<dim3((unsigned)((M * N + 255) / 256), (unsigned)batch), 256, 0, st>>>(part, slices, M, N, C, N, nullptr);
+    return launch_status();
 }
 
 int gemm_tc_status(const void* workspace, cudaStream_t st) {

@@ -218,7 +218,7 @@ constexpr int kCastMaxExchangeBytes = 96 * 1024;           // above this (K > 49
 
 template <int FMT, int GPL>
 __global__ void __launch_bounds__(kCastWarps * 32)
-cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int G, int lpr_log2, int exchange,
+cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_rows, int64_t seg_pad, int G, int lpr_log2, int exchange,
                      uint4* __restrict__ codes, uint16_t* __restrict__ scales, uint4* __restrict__ pos,
                      uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg,
                      int* __restrict__ row_exp, int nk64, int* __restrict__ flushed_total) {
@@ -230,7 +230,10 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int G, int lpr_log2
     const int k0 = ((int)blockIdx.x & ((16 >> (5 - lpr_log2)) - 1)) << (5 - lpr_log2);
     const int r_in = 32 * (wi >> 1) + 2 * (k0 + sg) + (wi & 1);  // row inside the 128-row block
     const int64_t row = rb * 128 + r_in;
-    const bool live = row < R;
+    // Segments (the heads of an attention call): seg_rows source rows each, padded to seg_pad operand rows.
+    const int64_t seg = seg_pad ? row / seg_pad : 0;
+    const bool live = row < R && (!seg_pad || row - seg * seg_pad < seg_rows);
+    const int64_t src_row = seg_pad ? seg * seg_rows + (row - seg * seg_pad) : row;
     const unsigned seg_mask = LPR == 32 ? 0xFFFFFFFFu : ((1u << LPR) - 1u) << (lane & ~(LPR - 1));
     const int64_t v_row = row * G;
     // this lane's ring: kCastDepth slots of 64 bytes (one group).  Piece j of a group sits at 16-byte position
@@ -241,7 +244,7 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int G, int lpr_log2
     const int n_own = (live && lr < G) ? ((G - lr + LPR - 1) >> lpr_log2) : 0;   // groups this lane owns
     auto issue = [&](int i) {                        // copies of the lane's i-th group, one commit group per call
         if (i < n_own) {
-            const uint4* src = x + (v_row + lr + ((int64_t)i << lpr_log2)) * 4;
+            const uint4* src = x + (src_row * G + lr + ((int64_t)i << lpr_log2)) * 4;
             uint8_t* slot = ring + (i % kCastDepth) * (32 * 64);
 #pragma unroll
             for (int j = 0; j < 4; ++j) cp_async16(slot + ((j ^ swz) << 4), src + j);
@@ -314,6 +317,7 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int G, int lpr_log2
         row_exp[row] = row_word(kmax, side_bits_of(top_p | (top_n << 8)), flushed);
         if (flushed && flushed_total) atomicAdd(flushed_total, flushed);
     }
+    if (lr == 0 && !live && row < R) row_exp[row] = 0;       // padding rows of a segment
     if (!exchange) return;                          // uniform over the block
     __syncthreads();
     // 16 bytes per thread: the words of rows q = 0..3 (32 rows apart) for one (plane, chunk, sector set, h);
@@ -336,7 +340,7 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int G, int lpr_log2
 // CACHED: the row has at most kT groups, so each thread keeps its one group in registers between the passes.
 template <bool CACHED>
 __global__ void __launch_bounds__(softmax::kT)
-softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s, float alpha, int vec, int causal,
+softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s, float alpha, int vec, int64_t causal,
                     uint4* __restrict__ codes, uint16_t* __restrict__ scales, uint4* __restrict__ pos,
                     uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg,
                     int* __restrict__ row_exp, int nk64) {
@@ -350,7 +354,7 @@ softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s,
     if (row_live) {
         const float* s = S + row * ld_s;
         const int64_t cols = (int64_t)G * 32, v_row = row * G;
-        const int64_t seen = causal ? min(cols, row + 1) : cols;     // causal: query `row` sees keys 0 .. row
+        const int64_t seen = causal ? min(cols, row % causal + 1) : cols;    // causal: query i of its matrix sees keys 0 .. i
         if (CACHED) {
             float e[32];
             const float sum = softmax::cached_row_exp(s, G, vec != 0, alpha, sh, e, seen);
@@ -378,6 +382,41 @@ softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s,
     finish_prepared_row(row, row_live, G, gx, softmax::kT, top, sc_first, scales, slot_s, sf_pos, sf_neg, row_exp, nk64);
 }
 
+// The same for rows of at most 32 groups, canonical output only: a warp per row, a lane per group.  The block kernel's
+// reductions over one warp's lanes and then over seven idle warps come to the same maximum and the same sum, so the
+// bits are the same; a row of 320 columns leaves that kernel's block with ten busy threads.
+__global__ void __launch_bounds__(256)
+softmax_cast_warp_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s, float alpha, int vec, int64_t causal,
+                         uint4* __restrict__ codes, uint16_t* __restrict__ scales) {
+    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (row >= R) return;
+    const int64_t cols = (int64_t)G * 32, seen = causal ? min(cols, row % causal + 1) : cols;
+    float e[32];
+    if (lane < G) softmax::load_group(S + row * ld_s, lane, cols, vec != 0, alpha, e, seen);
+    else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) e[i] = -INFINITY;
+    }
+    float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) mx = fmaxf(mx, e[i]);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, d));
+    const float nm = softmax::neg_max_log2e(mx);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        e[i] = softmax::exp_rel(e[i], nm);
+        sum += e[i];
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) sum = sum + __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+    if (lane >= G) return;
+    uint32_t w[16];
+    softmax::normalised_group_e(e, sum, w);
+    emit_group(w, row * G + lane, codes, scales, nullptr, nullptr);
+}
+
 template <int EPT, int TPG, int FMT = 0>
 int launch_rows(const void* x, int64_t rows, int64_t K, int64_t ld, uint8_t* codes,
                 uint8_t* scales, cudaStream_t st) {
@@ -403,7 +442,7 @@ namespace {
 template <int FMT>
 int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes, uint8_t* scales, void* pos, void* neg,
                          uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows, cudaStream_t st,
-                         int* flushed_total) {
+                         int* flushed_total, int64_t seg_rows, int64_t seg_pad) {
     int lpr_log2 = 1;
     while (lpr_log2 < 5 && (1 << lpr_log2) < G) ++lpr_log2;          // lanes per row: a power of two, 2 .. 32
     const int gpl = (int)((G + (1 << lpr_log2) - 1) >> lpr_log2);   // groups per lane
@@ -429,7 +468,7 @@ int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes,
         configured[dev][slot] = true;
     }
     kernel<<<(unsigned)blocks, kCastWarps * 32, smem, st>>>(
-        reinterpret_cast<const uint4*>(x), rows, (int)G, lpr_log2, exchange, reinterpret_cast<uint4*>(codes),
+        reinterpret_cast<const uint4*>(x), rows, seg_rows, seg_pad, (int)G, lpr_log2, exchange, reinterpret_cast<uint4*>(codes),
         reinterpret_cast<uint16_t*>(scales), reinterpret_cast<uint4*>(pos), reinterpret_cast<uint4*>(neg), sf_pos, sf_neg,
         row_exp, nk64, flushed_total);
     return launch_status();
@@ -439,23 +478,28 @@ int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes,
 // codes may be nullptr: the canonical codes are then not written (the planes hold the same nibbles).
 int quantize_rows_prepared(const void* x, int64_t rows, int64_t K, uint8_t* codes, uint8_t* scales, void* pos,
                            void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows,
-                           cudaStream_t st, int format, int* flushed_total) {
+                           cudaStream_t st, int format, int* flushed_total, int64_t seg_rows, int64_t seg_pad) {
     const int64_t G = K / 32;
     if (format == AMX_FMT_SYM_FP8)
-        return launch_cast_prepared<1>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total);
+        return launch_cast_prepared<1>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
     if (format == AMX_FMT_MXFP4)
-        return launch_cast_prepared<2>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total);
-    return launch_cast_prepared<0>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total);
+        return launch_cast_prepared<2>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
+    return launch_cast_prepared<0>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
 }
 
 // Softmax of the rows of S (fp32 [rows, ld_s], cols % 32 == 0), rounded to bf16 and cast, in one launch.  With
 // pos == nullptr only the canonical codes and scales are written.
 int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, float alpha, uint8_t* codes,
                       uint8_t* scales, void* pos, void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64,
-                      int64_t padded_rows, cudaStream_t st, int causal) {
+                      int64_t padded_rows, cudaStream_t st, int64_t causal) {
     const int64_t G = cols / 32, blocks = pos ? padded_rows : rows;
     if (blocks > 0x7FFFFFFF || G > 0x7FFFFFFF / 32) return AMX_ERR_SHAPE;
     const int vec = aligned(S, 16) && ld_s % 4 == 0;
+    if (!pos && G <= 32) {
+        softmax_cast_warp_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(S, rows, (int)G, ld_s, alpha, vec, causal,
+                                                                            reinterpret_cast<uint4*>(codes), reinterpret_cast<uint16_t*>(scales));
+        return launch_status();
+    }
     auto* kernel = G <= softmax::kT ? softmax_cast_kernel<true> : softmax_cast_kernel<false>;
     kernel<<<(unsigned)blocks, softmax::kT, 0, st>>>(S, rows, (int)G, ld_s, alpha, vec, causal, reinterpret_cast<uint4*>(codes),
                                                      reinterpret_cast<uint16_t*>(scales), reinterpret_cast<uint4*>(pos),
@@ -464,6 +508,44 @@ int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, 
 }
 
 namespace {
+
+// V of an attention call (x: [batch][R keys][C] contiguous, C = 64 or 128) cast down its rows straight into the sign planes
+// of the FP4 operand V^T (seg_pad operand rows per matrix, R / 2 bytes each) and its canonical scales [row][R / 32][2]; the
+// canonical codes are the two planes or-ed together.  A block stages 128 keys x C columns in shared memory (16-byte loads,
+// one row of a key is C * 2 contiguous bytes) and a thread owns one 32-key group of two neighbouring columns: lanes are
+// four groups x eight column pairs, so that a column's 64 bytes of codes per block leave in one piece and the XOR of the
+// column word with the group keeps the shared-memory reads free of bank conflicts.  16 heads x 8192 x 128: 54 us of the
+// 64 x 64-tile cast and 11 us of preparing its codes before.
+template <int C>
+__global__ void __launch_bounds__(256)
+cast_cols_planes_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_pad, uint4* __restrict__ pos, uint4* __restrict__ neg,
+                        uint16_t* __restrict__ scales) {
+    constexpr int kWords = C / 2, kVec = C / 8;               // 32-bit words and 16-byte pieces per key
+    __shared__ __align__(16) uint32_t tile[128 * kWords];
+    const int64_t key0 = (int64_t)blockIdx.x * 128, batch = blockIdx.y;
+    const uint4* src = x + (batch * R + key0) * kVec;
+    const int keys = (int)min((int64_t)128, R - key0);
+    for (int i = threadIdx.x; i < keys * kVec; i += 256) {
+        const int key = i / kVec, v = i % kVec;
+        *reinterpret_cast<uint4*>(&tile[key * kWords + ((v * 4) ^ ((key >> 5) * 8))]) = __ldg(src + i);
+    }
+    __syncthreads();
+    const int g = threadIdx.x & 3;                            // the tile's 32-key group
+    if (g * 32 >= keys) return;
+    const int64_t G = R / 32;
+    for (int cw = threadIdx.x >> 2; cw < kWords; cw += 64) {  // column pair
+        uint32_t lo[16], hi[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const uint32_t a = tile[(g * 32 + 2 * i) * kWords + (cw ^ (g * 8))], b = tile[(g * 32 + 2 * i + 1) * kWords + (cw ^ (g * 8))];
+            lo[i] = __byte_perm(a, b, 0x5410);
+            hi[i] = __byte_perm(a, b, 0x7632);
+        }
+        const int64_t v = (batch * seg_pad + 2 * cw) * G + key0 / 32 + g;
+        emit_group(lo, v, nullptr, scales, pos, neg);
+        emit_group(hi, v + G, nullptr, scales, pos, neg);
+    }
+}
 
 template <int TPG>
 int launch_cols(const void* x, int64_t R, int64_t C, int64_t ld, int gs, uint8_t* codes,
@@ -477,6 +559,17 @@ int launch_cols(const void* x, int64_t R, int64_t C, int64_t ld, int gs, uint8_t
 }
 
 }  // namespace
+
+// V of `batch` heads into the planes and scales of V^T (cast_cols_planes_kernel).
+int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int64_t seg_pad, void* pos, void* neg, uint8_t* scales,
+                         cudaStream_t st) {
+    if (batch > 65535 || (C != 64 && C != 128)) return AMX_ERR_SHAPE;
+    const dim3 grid((unsigned)((R + 127) / 128), (unsigned)batch);
+    auto* kernel = C == 128 ? cast_cols_planes_kernel<128> : cast_cols_planes_kernel<64>;
+    kernel<<<grid, 256, 0, st>>>(static_cast<const uint4*>(x), R, seg_pad, static_cast<uint4*>(pos), static_cast<uint4*>(neg),
+                                 reinterpret_cast<uint16_t*>(scales));
+    return launch_status();
+}
 
 // amx_quantize_t with group size 32 on `batch` matrices [R, C] stored one after another (contiguous rows); the
 // canonical outputs of their transposes follow one another too.
