@@ -18,6 +18,62 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 // Returns AMX_OK when the last launch was accepted, AMX_ERR_CUDA otherwise.
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? AMX_OK : AMX_ERR_CUDA; }
 
+// ---- launches ---------------------------------------------------------------------------------
+// Kernels of this library are chained by programmatic dependent launch: a kernel lets its successor onto the SMs as soon
+// as all of its own blocks run (grid_launch_dependents), and waits for its predecessors to complete before it touches
+// memory (grid_dependency_wait; it returns at once when the launch carried no such dependency).  The order of the stream
+// is kept, the launch latency and the gap between two kernels are not: chains of ordinary launches cost about 2 us per
+// kernel boundary.  A stream that is being captured gets ordinary launches (replayed from a graph the chains of short
+// kernels were slower with these edges).
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// First statement of a kernel.  (Every kernel waits before anything else, so "my predecessor has completed" implies the
+// same of everything before it.)
+__device__ __forceinline__ void begin_kernel() {
+    grid_launch_dependents();
+    grid_dependency_wait();
+}
+
+inline bool programmatic_launch_ok(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
+// chained = false: an ordinary launch.  For long kernels with one block per SM: started while their predecessor leaves, the
+// blocks land on the SMs in another order, which costs them 2.5-4 % (operands shared by neighbouring tiles cross the two
+// halves of the L2 more often) - more than the gap from about 200 us on.
+template <typename... P, typename... A>
+int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chained && programmatic_launch_ok(st) ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) != cudaSuccess) {
+        cudaGetLastError();
+        return AMX_ERR_CUDA;
+    }
+    return AMX_OK;
+}
+
+template <typename... P, typename... A>
+int launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_chained(true, kernel, grid, block, smem, st, static_cast<A&&>(args)...);
+}
+
+// Zeroes the first n words of a workspace (the status word, the flushed-scale count) by a kernel: a memset would break
+// the chain of launches (api.cu).
+int clear_words(void* words, cudaStream_t st, int n = 2);
+
 // ---- device-side number formats -------------------------------------------------------------
 
 // fp32 value of an E5M2 byte: E5M2 is the upper byte of an IEEE half.

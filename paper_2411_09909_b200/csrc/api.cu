@@ -69,7 +69,15 @@ QuantSizes quant_sizes(int64_t rows, int64_t K, int gs) {
 
 constexpr uint32_t kQuantGemmFlags = kKernelMask | AMX_GEMM_CAST_IN_KERNEL | AMX_WEIGHT_BF16;
 
+__global__ void clear_words_kernel(int* __restrict__ words, int n) {
+    begin_kernel();
+    if ((int)threadIdx.x < n) words[threadIdx.x] = 0;
+}
+
 }  // namespace
+
+int clear_words(void* words, cudaStream_t st, int n) { return launch(clear_words_kernel, 1, 32, 0, st, static_cast<int*>(words), n); }
+
 }  // namespace amx
 
 using namespace amx;
@@ -249,7 +257,7 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
     if (gemm_ws < 256) gemm_ws = 256;                       // the plain kernel has no scratch of its own: header only
     const QuantSizes a = quant_sizes(M, K, group_size), w = quant_sizes(N, K, group_size);
     uint8_t* base = static_cast<uint8_t*>(workspace);
-    if (kernel == AMX_GEMM_SIMT && cudaMemsetAsync(base, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (kernel == AMX_GEMM_SIMT && clear_words(base, st) != AMX_OK) return AMX_ERR_CUDA;
     uint8_t* a_codes = base + gemm_ws;
     uint8_t* a_scales = a_codes + a.codes;
     uint8_t* wq_codes = a_scales + a.scales;               // only with a bf16 weight
@@ -261,7 +269,7 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
         uint8_t* pa = base + 256;
         uint8_t* pw = pa + gemm_fp4_prepared_bytes(M, K, false);
         int* words = reinterpret_cast<int*>(base);
-        if (cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+        if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
         if (ld_a == K && group_size == 32) rc = gemm_fp4_quantize_prepared(A, M, K, false, a_codes, a_scales, pa, st, 0, AMX_FMT_AMXFP4, words + 1);
         else {
             rc = amx_quantize(A, M, K, ld_a, group_size, a_codes, a_scales, stream);
@@ -611,7 +619,7 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
     const size_t head_in = (size_t)L * d * 2;                       // bytes of one head of q, k or v
     const size_t gemm_bytes = a.total - a.gemm;
     int* words = reinterpret_cast<int*>(w + a.gemm);                // fused: [0] status, [1] flushed scales of the call
-    if (fused && cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (fused && clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
     float* S = reinterpret_cast<float*>(w + a.S);
     const size_t qk_codes = (size_t)L * d / 2, qk_scales = (size_t)L * (d / 32) * 2;   // one head of Q or K, canonical
     const size_t v_codes = (size_t)d * L / 2, v_scales = (size_t)d * (L / 32) * 2;     // one head of V^T
@@ -737,7 +745,7 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     // one head through the launch sequence of amx_attention: casts of Q, K (along head_dim) and V (along the
     // sequence), then the two passes
     int* words = reinterpret_cast<int*>(w + a.gemm);
-    if (cudaMemsetAsync(words, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
     int rc = gemm_fp4_quantize_prepared(q, L, d, false, nullptr, w + a.qs, w + a.pq, st);
     if (rc == AMX_OK) rc = gemm_fp4_quantize_prepared(k, L, d, true, nullptr, w + a.ks, w + a.pk, st);
     if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(v, 1, L, d, 128, 128, w + a.vs, w + a.pv, st, nullptr);

@@ -31,6 +31,7 @@ __device__ __forceinline__ float element(const ExactOperand& o, int64_t row, int
 __global__ void __launch_bounds__(kThreads)
 attention_exact_kernel(const ExactOperand q, const ExactOperand k, const ExactOperand v, int64_t L, int64_t Lp, int d, int kv_group,
                        float alpha, int causal, float* __restrict__ O, const int* __restrict__ run_if_nonzero) {
+    begin_kernel();
     if (*run_if_nonzero == 0) return;
     extern __shared__ float sm[];
     float* S = sm;                                   // [16][L]
@@ -114,9 +115,8 @@ int attn_exact(const ExactOperand& q, const ExactOperand& k, const ExactOperand&
         configured[dev] = true;
     }
     const dim3 grid((unsigned)((L + kRows - 1) / kRows), (unsigned)heads);
-    attention_exact_kernel<<<grid, kThreads, smem_bytes(L, d), st>>>(q, k, vt, L, attn_fused_padded(L), (int)d, kv_group, alpha, causal, O,
+    return launch(attention_exact_kernel, grid, kThreads, smem_bytes(L, d), st, q, k, vt, L, attn_fused_padded(L), (int)d, kv_group, alpha, causal, O,
                                                                      run_if_nonzero);
-    return launch_status();
 }
 
 }  // namespace amx

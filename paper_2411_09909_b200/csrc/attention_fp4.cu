@@ -118,6 +118,7 @@ template <int PASS, int MASK, int HD>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const Params p) {
+    grid_dependency_wait();
     using S_ = Smem<PASS>;
     constexpr bool CAUSAL = MASK == kMaskCausal;
     constexpr int kQkSteps = HD / 64;                     // MMAs along the head dimension per sign pair
@@ -529,6 +530,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
         }
     }
+    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -550,8 +552,8 @@ int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensor
         configured[dev] = true;
     }
     const int items = p.heads * p.m_tiles;
-    attention_fp4_kernel<PASS, MASK, HD><<<(unsigned)(items < sms ? items : sms), kThreads, Smem<PASS>::kBytes, st>>>(tm_q, tm_k, tm_v, p);
-    return launch_status();
+    return launch_chained((double)p.heads * (double)p.L * (double)p.L <= 2.7e8,   // about 140 us in the second pass
+                          attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), kThreads, Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
 }
 
 }  // namespace

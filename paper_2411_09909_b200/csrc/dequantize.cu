@@ -12,6 +12,7 @@ __global__ void __launch_bounds__(256)
 dequantize_kernel(const uint32_t* __restrict__ codes, const uint16_t* __restrict__ scales,
                   int64_t n_vec, int64_t vec_per_row, int vec_per_group, int64_t ld_out,
                   void* __restrict__ out) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // 8 elements per thread
     if (v >= n_vec) return;
     const uint32_t nib = codes[v];
@@ -59,8 +60,6 @@ extern "C" int amx_dequantize(const uint8_t* codes, const uint8_t* scales, int64
     auto* cv = reinterpret_cast<const uint32_t*>(codes);
     auto* sv = reinterpret_cast<const uint16_t*>(scales);
     if (flags & AMX_OUT_F32)
-        dequantize_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(cv, sv, n_vec, K / 8, group_size / 8, ld_out, out);
-    else
-        dequantize_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(cv, sv, n_vec, K / 8, group_size / 8, ld_out, out);
-    return launch_status();
+        return launch(dequantize_kernel<true>, (unsigned)blocks, 256, 0, st, cv, sv, n_vec, K / 8, group_size / 8, ld_out, out);
+    return launch(dequantize_kernel<false>, (unsigned)blocks, 256, 0, st, cv, sv, n_vec, K / 8, group_size / 8, ld_out, out);
 }

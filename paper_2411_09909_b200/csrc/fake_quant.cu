@@ -20,6 +20,7 @@ template <int EPT, int TPG, int FMT>
 __global__ void __launch_bounds__(kThreads)
 fake_quantize_kernel(const uint4* __restrict__ x, int64_t n_items, int64_t items_per_row, int64_t ld_vec,
                      uint4* __restrict__ out, int64_t ld_out_vec) {
+    begin_kernel();
     constexpr int NV = EPT / 8;
     const int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const bool live = v < n_items;
@@ -44,21 +45,19 @@ fake_quantize_kernel(const uint4* __restrict__ x, int64_t n_items, int64_t items
 }
 
 template <int EPT, int TPG, int FMT>
-int launch(const void* x, int64_t rows, int64_t K, int64_t ld_x, void* out, int64_t ld_out, cudaStream_t st) {
+int launch_ept(const void* x, int64_t rows, int64_t K, int64_t ld_x, void* out, int64_t ld_out, cudaStream_t st) {
     const int64_t items_per_row = K / EPT, n_items = rows * items_per_row, blocks = (n_items + kThreads - 1) / kThreads;
     if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
-    fake_quantize_kernel<EPT, TPG, FMT><<<(unsigned)blocks, kThreads, 0, st>>>(
-        static_cast<const uint4*>(x), n_items, items_per_row, ld_x / 8, static_cast<uint4*>(out), ld_out / 8);
-    return launch_status();
+    return launch(fake_quantize_kernel<EPT, TPG, FMT>, (unsigned)blocks, kThreads, 0, st, static_cast<const uint4*>(x), n_items, items_per_row, ld_x / 8, static_cast<uint4*>(out), ld_out / 8);
 }
 
 template <int FMT>
 int launch_gs(const void* x, int64_t rows, int64_t K, int64_t ld_x, int gs, void* out, int64_t ld_out, cudaStream_t st) {
     switch (gs) {
-        case 16: return launch<16, 1, FMT>(x, rows, K, ld_x, out, ld_out, st);
-        case 32: return launch<32, 1, FMT>(x, rows, K, ld_x, out, ld_out, st);
-        case 64: return launch<32, 2, FMT>(x, rows, K, ld_x, out, ld_out, st);
-        default: return launch<32, 4, FMT>(x, rows, K, ld_x, out, ld_out, st);
+        case 16: return launch_ept<16, 1, FMT>(x, rows, K, ld_x, out, ld_out, st);
+        case 32: return launch_ept<32, 1, FMT>(x, rows, K, ld_x, out, ld_out, st);
+        case 64: return launch_ept<32, 2, FMT>(x, rows, K, ld_x, out, ld_out, st);
+        default: return launch_ept<32, 4, FMT>(x, rows, K, ld_x, out, ld_out, st);
     }
 }
 

@@ -45,6 +45,7 @@ template <bool ASYM, bool E4M3>
 __global__ void __launch_bounds__(256) quantize_f16s_kernel(const uint16_t* __restrict__ x, int64_t n_groups, int64_t G,
                                                             int64_t ld_x, int gs, uint32_t* __restrict__ codes,
                                                             uint32_t* __restrict__ scales) {
+    begin_kernel();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n_groups) return;
     const int64_t row = idx / G, g = idx % G;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(256) dequantize_f16s_kernel(const uint32_t* __
                                                               const uint32_t* __restrict__ scales, int64_t n_vec,
                                                               int64_t vec_per_row, int vec_per_group, int64_t ld_out,
                                                               float* __restrict__ out) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_vec) return;
     const uint32_t nib = codes[v], sc = scales[v / vec_per_group];
@@ -124,8 +126,7 @@ extern "C" int amx_quantize_f16s(const void* x, int64_t rows, int64_t K, int64_t
     const bool asym = flags & AMX_F16S_ASYMMETRIC, e4m3 = flags & AMX_F16S_SCALE_E4M3;
     auto* kernel = asym ? (e4m3 ? quantize_f16s_kernel<true, true> : quantize_f16s_kernel<true, false>)
                         : (e4m3 ? quantize_f16s_kernel<false, true> : quantize_f16s_kernel<false, false>);
-    kernel<<<(unsigned)blocks, 256, 0, st>>>(xv, n_groups, G, ld_x, group_size, cv, sv);
-    return launch_status();
+    return launch(kernel, (unsigned)blocks, 256, 0, st, xv, n_groups, G, ld_x, group_size, cv, sv);
 }
 
 extern "C" int amx_dequantize_f16s(const uint8_t* codes, const uint16_t* scales, int64_t rows, int64_t K, int group_size,
@@ -136,10 +137,8 @@ extern "C" int amx_dequantize_f16s(const uint8_t* codes, const uint16_t* scales,
     if (!aligned(codes, 4) || !aligned(scales, 4) || !aligned(out, 16) || ld_out % 4) return AMX_ERR_ALIGN;
     const int64_t n_vec = rows * (K / 8), blocks = (n_vec + 255) / 256;
     if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
-    dequantize_f16s_kernel<<<(unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        reinterpret_cast<const uint32_t*>(codes), reinterpret_cast<const uint32_t*>(scales), n_vec, K / 8, group_size / 8,
+    return launch(dequantize_f16s_kernel, (unsigned)blocks, 256, 0, static_cast<cudaStream_t>(stream), reinterpret_cast<const uint32_t*>(codes), reinterpret_cast<const uint32_t*>(scales), n_vec, K / 8, group_size / 8,
         ld_out, out);
-    return launch_status();
 }
 
 extern "C" int amx_gemm_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8_t* w_codes,

@@ -124,6 +124,7 @@ prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restr
                        int nk64, uint4* __restrict__ pos, uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos,
                        uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total,
                        int seg_rows = 0, int seg_pad = 0) {
+    begin_kernel();
     __shared__ int kmax_s[kPrepRows];
     __shared__ int unsplit_s[kPrepRows];
     const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / GS;         // G: scale pairs per row
@@ -279,6 +280,7 @@ template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = fal
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                 const __grid_constant__ CUtensorMap tm_a1, const __grid_constant__ CUtensorMap tm_w1, const Params p) {
+    grid_dependency_wait();
     using C_ = Cfg<BK_, ONE_PLANE>;
     constexpr int kPlanes = C_::kPlanes;
     if (p.gate && *p.gate != 0) return;                          // uniform over the grid: nothing was set up yet
@@ -667,6 +669,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             tile = tile_after;
         }
     }
+    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -681,11 +684,9 @@ int prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K
     const int64_t padded_rows = o.row_blocks * 128;
     auto* kernel = gs == 16 ? prepare_operand_kernel<16> : gs == 32 ? prepare_operand_kernel<32>
                  : gs == 64 ? prepare_operand_kernel<64> : prepare_operand_kernel<128>;
-    kernel<<<(unsigned)(padded_rows / kPrepRows), 256, 0, st>>>(
-        codes, scales, rows, K, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
+    return launch(kernel, (unsigned)(padded_rows / kPrepRows), 256, 0, st, codes, scales, rows, K, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
         base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf),
         flushed_total, 0, 0);
-    return launch_status();
 }
 
 }  // namespace
@@ -722,8 +723,8 @@ int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, co
         return AMX_ERR_CUDA;
     const int64_t tiles = ((p.N + BNT - 1) / BNT) * ((p.M + BM - 1) / BM) * (SLICED ? p.slices : 1);
     const unsigned grid = (unsigned)(tiles < sm_count[dev] ? tiles : sm_count[dev]);   // one persistent CTA per SM
-    gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE><<<grid, kThreads, C_::kSmemBytes, st>>>(tm_a, tm_w, tm_a1, tm_w1, p);
-    return launch_status();
+    return launch_chained((double)p.M * (double)p.N * (double)p.K <= 1.1e11,      // about 170 us
+                          gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w, tm_a1, tm_w1, p);
 }
 
 }  // namespace
@@ -740,7 +741,6 @@ int fill_params(const Fp4Operand& a, const Fp4Operand& w, int64_t M, int64_t N, 
     const uint8_t* pa = static_cast<const uint8_t*>(a.prepared);
     const uint8_t* pw = static_cast<const uint8_t*>(w.prepared);
     int* status = static_cast<int*>(workspace);
-    if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;
     p = Params{};
     // scale factors come in chunks per 128 rows, row words per row: the range starts at a pointer offset
     const size_t a_sf0 = (size_t)(a.row0 / 128) * oa.nk64 * kSfChunk, w_sf0 = (size_t)(w.row0 / 128) * ow.nk64 * kSfChunk;
@@ -791,6 +791,8 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
     int dev;
     const int rc = fill_params(a, w, M, N, K, C, ld_c, workspace, st, p, oa, ow, dev);
     if (rc != AMX_OK) return rc;
+    // the status word; a caller that hands over a gate has cleared it (the gate is the word behind it)
+    if (!gate && clear_words(workspace, st, 1) != AMX_OK) return AMX_ERR_CUDA;
     p.gate = gate;
     p.scale_a = scale_a;
     p.scale_w = scale_w;
@@ -850,10 +852,8 @@ int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64
     uint8_t* base = static_cast<uint8_t*>(prepared);
     const int rc = quantize_cols_planes(v, heads, L, d, seg_pad, base, base + o.plane, scales, st);
     if (rc != AMX_OK) return rc;
-    prepare_operand_kernel<32, false><<<(unsigned)(heads * seg_pad / kPrepRows), 256, 0, st>>>(
-        nullptr, scales, heads * seg_pad, L, o.nk64, nullptr, nullptr, base + 2 * o.plane, base + 2 * o.plane + o.sf,
+    return launch(prepare_operand_kernel<32, false>, (unsigned)(heads * seg_pad / kPrepRows), 256, 0, st, nullptr, scales, heads * seg_pad, L, o.nk64, nullptr, nullptr, base + 2 * o.plane, base + 2 * o.plane + o.sf,
         reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), flushed_total, (int)d, (int)seg_pad);
-    return launch_status();
 }
 
 // Bytes from the first to the second sign plane of a prepared operand.
@@ -891,7 +891,7 @@ int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_c
     uint8_t* pa = base + 256;
     uint8_t* pw = pa + oa.total;
     int* flushed = reinterpret_cast<int*>(base) + 1;
-    if (cudaMemsetAsync(base, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (clear_words(base, st) != AMX_OK) return AMX_ERR_CUDA;
     int rc = prepare(a_codes, a_scales, M, K, oa, pa, st, flushed, gs);
     if (rc == AMX_OK) rc = prepare(w_codes, w_scales, N, K, ow, pw, st, flushed, gs);
     if (rc != AMX_OK) return rc;

@@ -28,15 +28,11 @@
 // cluster (up to 8), which add their partial products over distributed shared memory in rank order - deterministic,
 // no scratch in global memory and no second launch.
 //
-// The token rows, two ways:
-//   CAST      every CTA casts its K range of the rows itself (one launch per call): one tile of 8 rows, or a small
-//             product, where launches are what costs.  The redundant casts grow with the rows: at 16 rows they would
-//             be half of the decode work.
-//   otherwise a small kernel casts (or decodes) the rows once into the fragment order, and the main kernel copies the
-//             fragments of a step into its ring beside the weight.
-// Launches are chained by programmatic dependent launch outside stream capture: a kernel fills its weight rings while
-// its predecessor still runs, and waits for it before it reads the rows or writes anything.  (Replayed from a CUDA
-// graph the same chain was slower than plain edges, so a capturing stream gets ordinary launches.)
+// The token rows are cast (or decoded) once by a small kernel into the fragment order.  (Cast inside the main kernel by
+// every CTA, one launch less, measured the same for one row and slower for more.)
+// The fragments kernel waits for its predecessors before it lets the main kernel start, so the main kernel may fill its
+// rings at once - whoever wrote the weight has completed - and waits only for the fragments.  (Prefetching the weight into
+// the L2 across the boundary between two calls measured slower: the memory is not what this kernel waits for.)
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
@@ -60,12 +56,6 @@ constexpr int kMaxSlices = 8;                      // portable cluster size
 constexpr int kPartPitch = kCtaRows + 4;           // floats per token row of the partial-product tile (bank spread)
 constexpr int kMaxTiles = 8;                       // token tiles per CTA
 constexpr int kScaleSteps = 32;                    // steps whose scales are held at a time
-
-// griddepcontrol.wait: returns once every grid this one programmatically depends on has completed and its writes
-// are visible (at once when the launch carried no such dependency).  griddepcontrol.launch_dependents: the grid
-// launched behind this one with programmatic serialization may start once every CTA here has said so or exited.
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ __half2 h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 __device__ __forceinline__ uint32_t u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
@@ -150,16 +140,13 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1,
 }
 
 struct RowsParams {
-    const uint16_t* x;           // CAST: bf16 rows [M, ld_x]
-    int64_t ld_x;
-    const uint4* frag;           // otherwise: fragments [step][tiles of all rows]
+    const uint4* frag;           // [step][tiles of all rows]
     const uint8_t *w_codes, *w_scales;
     int M;
     int64_t N, K;
     float* C;
     int64_t ld_c;
     int steps_max;               // steps of the longest range
-    int* status;                 // CAST: the two status words of the workspace (or nullptr), cleared here
 };
 
 // Shared-memory geometry.  kDepth ring slots per warp (kDepth - 1 steps in flight); with up to four token tiles two
@@ -183,7 +170,7 @@ __host__ __device__ constexpr int scale_pitch(int n, int gs) {
 __host__ __device__ constexpr int scale_bytes(int n, int gs) { return (kCtaRows * scale_pitch(n, gs) * 4 + 15) / 16 * 16; }
 
 // NT: tiles of 8 token rows per CTA.
-template <int NT, bool CAST, int GS>
+template <int NT, int GS>
 __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(const RowsParams p) {
     using R = Ring<NT, GS>;
     constexpr int kDepth = R::kDepth, kFragSlot = R::kFragSlot;
@@ -201,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
     uint8_t* ring = smem + warp * (kDepth * kCodeBytes);
     const int held = min(p.steps_max, kScaleSteps), pitch = scale_pitch(held, GS);
     uint32_t* scale_s = reinterpret_cast<uint32_t*>(smem + R::kBytes);
-    uint8_t* frag_s = smem + R::kBytes + scale_bytes(held, GS);      // CAST: the range's fragments; else a ring per step parity
+    uint8_t* frag_s = smem + R::kBytes + scale_bytes(held, GS);      // a ring of fragments per step parity
 
     // this lane's streams: piece t of rows g, g + 8 (block 0), g + 16, g + 24 (block 1) of the warp's 32 rows
     const uint8_t* pc[4];
@@ -251,38 +238,12 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
     }
     grid_launch_dependents();                  // whatever follows waits for this grid's completion by itself
     grid_dependency_wait();                    // the rows (and the previous user of C) are complete from here on
-    if (CAST) {
-        if (p.status && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 2) p.status[threadIdx.x] = 0;
-        // Tokens over warps; with fewer than eight tokens, `parts` warps share a token's K range.
-        const int n_tok = NT * kTok, live_tok = min(n_tok, p.M - m0);
-        auto put_piece = [&](int tok, int k8, const uint4& v) {
-            *reinterpret_cast<uint4*>(frag_s + (k8 >> 4) * kFragSlot + (tok >> 3) * kFragBytes +
-                                      frag_pos(k8 & 3, (tok & 7) * 4 + ((k8 >> 2) & 3)) * 16) = v;
-        };
-        int parts = 1;
-        if (NT == 1)
-            while (parts < 8 && live_tok * parts * 2 <= 8) parts *= 2;
-        for (int tok = warp / parts; tok < live_tok; tok += kWarps / parts) {
-            const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)(m0 + tok) * p.ld_x + s_begin * kStepK);
-            for (int k0 = (warp % parts) * 32; k0 < n_total * 16; k0 += parts * 32) {
-                const int k8 = k0 + lane;
-                uint4 q = make_uint4(0, 0, 0, 0);
-                if (k8 < n_total * 16) q = __ldg(src + k8);
-                const uint4 v = cast_piece<GS / 8>(q);
-                if (k8 < n_total * 16) put_piece(tok, k8, v);
-            }
-        }
-        for (int tok = live_tok + warp; tok < n_tok; tok += kWarps)          // rows past M
-            for (int k8 = lane; k8 < n_total * 16; k8 += 32) put_piece(tok, k8, make_uint4(0, 0, 0, 0));
-        cp_async_wait<kDepth - 2>();           // the first group: the scales
-    } else {
 #pragma unroll
-        for (int d = 0; d < kDepth - 1; ++d) {
-            issue_frags(d);
-            cp_async_commit();
-        }
-        cp_async_wait<2 * kDepth - 3>();       // the first group
+    for (int d = 0; d < kDepth - 1; ++d) {
+        issue_frags(d);
+        cp_async_commit();
     }
+    cp_async_wait<2 * kDepth - 3>();           // the first group: the scales
     __syncthreads();
 
     float acc[2][NT][4];
@@ -306,15 +267,14 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
         }
         if (i >= n_mine) break;                // an odd range: one step less for the second parity
         cp_async_wait<kDepth - 2>();           // this step's copies have landed
-        if (!CAST) {                           // the fragments are visible to the parity's four warps, last step's slots free
-            if (wk == 0) asm volatile("bar.sync 1, %0;" ::"n"(kRowGroups * 32) : "memory");
-            else asm volatile("bar.sync 2, %0;" ::"n"(kRowGroups * 32) : "memory");
-        }
+        // the fragments are visible to the parity's four warps, last step's slots free
+        if (wk == 0) asm volatile("bar.sync 1, %0;" ::"n"(kRowGroups * 32) : "memory");
+        else asm volatile("bar.sync 2, %0;" ::"n"(kRowGroups * 32) : "memory");
         issue_codes(i + kDepth - 1);
-        if (!CAST) issue_frags(i + kDepth - 1);
+        issue_frags(i + kDepth - 1);
         cp_async_commit();
         const uint8_t* slot = ring + (i % kDepth) * kCodeBytes;
-        const uint8_t* fs = CAST ? frag_s + ls * kFragSlot : frag_s + (wk * kDepth + i % kDepth) * kFragSlot;
+        const uint8_t* fs = frag_s + (wk * kDepth + i % kDepth) * kFragSlot;
         uint4 cw[4];
         uint32_t sc[4];                        // the scale bytes of the lane's group (groups of 16: of both)
 #pragma unroll
@@ -418,11 +378,10 @@ struct StreamRing {
     static constexpr int kBytes = kWarps * kWarpBytes;
 };
 
-template <int NT, bool CAST, int GS>
+template <int NT, int GS>
 __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_kernel(const RowsParams p) {
     using R = StreamRing<GS>;
     constexpr int kDepth = R::kDepth;
-    static_assert(!CAST || NT == 1, "rows are cast inside for one tile only");
     extern __shared__ __align__(16) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int slices = (int)gridDim.y, slice = (int)blockIdx.y;
@@ -436,7 +395,6 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
 
     uint8_t* ring = smem + warp * R::kWarpBytes;
     uint8_t* scale_ring = ring + kDepth * kCodeBytes;
-    uint8_t* frag_s = smem + R::kBytes;        // CAST: the live rows' fragments of the CTA's range
 
     // piece t of rows g, g + 8 (block 0), g + 16, g + 24 (block 1).  Rows past the weight are not copied: what their
     // slots hold only reaches sums that are not stored.
@@ -474,34 +432,8 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
         cp_async_commit();
     }
     grid_launch_dependents();                  // whatever follows waits for this grid's completion by itself
-    grid_dependency_wait();                    // the rows (and the previous user of C) are complete from here on
+    grid_dependency_wait();                    // the fragments (and the previous user of C) are complete from here on
     const int m0 = (int)blockIdx.z * (NT * kTok), live_tok = min(NT * kTok, p.M - m0);
-    if (CAST) {                                // (one block of tokens: m0 = 0)
-        if (p.status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) p.status[threadIdx.x] = 0;
-        // pieces of 8 elements, all loads of a thread's next four in flight together
-        const int pieces = (int)cta_steps * 16;
-        for (int tok = 0; tok < live_tok; ++tok) {
-            const uint4* src = reinterpret_cast<const uint4*>(p.x + (int64_t)tok * p.ld_x + cta_begin * kStepK);
-            for (int k0 = warp * 32; k0 < pieces; k0 += 4 * kThreads) {
-                uint4 q[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k8 = k0 + i * kThreads + lane;
-                    q[i] = k8 < pieces ? __ldg(src + k8) : make_uint4(0, 0, 0, 0);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int k8 = k0 + i * kThreads + lane;
-                    if (k8 - lane >= pieces) break;                  // uniform over the warp
-                    const uint4 v = cast_piece<GS / 8>(q[i]);
-                    // [step][j][token][t] pieces of 16 bytes
-                    if (k8 < pieces)
-                        *reinterpret_cast<uint4*>(frag_s + ((((k8 >> 4) * 4 + (k8 & 3)) * live_tok + tok) * 4 + ((k8 >> 2) & 3)) * 16) = v;
-                }
-            }
-        }
-        __syncthreads();
-    }
 
     float acc[2][NT][4];
 #pragma unroll
@@ -543,14 +475,8 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
                 for (int q = 0; q < 4; ++q) s[q] = make_scales(j ? sc[q] >> 16 : sc[q]);
             }
             uint4 b[NT];
-            if (CAST) {
-                b[0] = make_uint4(0, 0, 0, 0);
-                if (g < live_tok)
-                    b[0] = *reinterpret_cast<const uint4*>(frag_s + ((((w_first + i) * 4 + j) * live_tok + g) * 4 + t) * 16);
-            } else {
 #pragma unroll
-                for (int m = 0; m < NT; ++m) b[m] = __ldg(fg + m * 128 + frag_pos(j, lane));
-            }
+            for (int m = 0; m < NT; ++m) b[m] = __ldg(fg + m * 128 + frag_pos(j, lane));
 #pragma unroll
             for (int blk = 0; blk < 2; ++blk) {
                 const uint32_t w0 = j == 0 ? cw[2 * blk].x : j == 1 ? cw[2 * blk].y : j == 2 ? cw[2 * blk].z : cw[2 * blk].w;
@@ -654,55 +580,35 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
 
 constexpr size_t kMaxSmem = 227 * 1024;
 
-// The CTAs cast their rows themselves: one or two rows (the redundant casts are a small share of the decode), or a
-// product so small that the second launch would cost more than the casts (below 2^28 multiply-adds); in either case
-// only while the fragments leave room for a second CTA on the SM.
-bool cast_inside(const RowsPlan& pl, int64_t M, int64_t N, int64_t K) {
-    if (pl.stream) return M <= 2 && (size_t)pl.steps_max * M * kStepK * 2 <= 40 * 1024;
-    return (double)M * (double)N * (double)K < 268435456.0 && (size_t)pl.steps_max * pl.nt * kFragBytes <= 32 * 1024;
-}
-
 struct RowsKernel {
     void (*fn)(const RowsParams);
     size_t ring_bytes, frag_ring_bytes;
 };
 
 template <int GS>
-RowsKernel kernel_for(const RowsPlan& pl, bool cast) {
+RowsKernel kernel_for(const RowsPlan& pl) {
     constexpr size_t kStream = StreamRing<GS>::kBytes;
     if (pl.stream) {
-        if (cast) return {gemm_rows_stream_kernel<1, true, GS>, kStream, 0};
         switch (pl.nt) {
-            case 1: return {gemm_rows_stream_kernel<1, false, GS>, kStream, 0};
-            case 2: return {gemm_rows_stream_kernel<2, false, GS>, kStream, 0};
-            case 3: return {gemm_rows_stream_kernel<3, false, GS>, kStream, 0};
-            default: return {gemm_rows_stream_kernel<4, false, GS>, kStream, 0};
+            case 1: return {gemm_rows_stream_kernel<1, GS>, kStream, 0};
+            case 2: return {gemm_rows_stream_kernel<2, GS>, kStream, 0};
+            case 3: return {gemm_rows_stream_kernel<3, GS>, kStream, 0};
+            default: return {gemm_rows_stream_kernel<4, GS>, kStream, 0};
         }
     }
     switch (pl.nt) {
-        case 4: return {cast ? gemm_rows_kernel<4, true, GS> : gemm_rows_kernel<4, false, GS>, Ring<4, GS>::kBytes, Ring<4, GS>::kFragRing};
-        case 6: return {cast ? gemm_rows_kernel<6, true, GS> : gemm_rows_kernel<6, false, GS>, Ring<6, GS>::kBytes, Ring<6, GS>::kFragRing};
-        default: return {cast ? gemm_rows_kernel<8, true, GS> : gemm_rows_kernel<8, false, GS>, Ring<8, GS>::kBytes, Ring<8, GS>::kFragRing};
+        case 4: return {gemm_rows_kernel<4, GS>, Ring<4, GS>::kBytes, Ring<4, GS>::kFragRing};
+        case 6: return {gemm_rows_kernel<6, GS>, Ring<6, GS>::kBytes, Ring<6, GS>::kFragRing};
+        default: return {gemm_rows_kernel<8, GS>, Ring<8, GS>::kBytes, Ring<8, GS>::kFragRing};
     }
 }
 
-// Programmatic dependent launch is used outside stream capture only (see the file header).
-bool programmatic_launch_ok(cudaStream_t st) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return cs == cudaStreamCaptureStatusNone;
-}
-
-int launch_rows(RowsParams p, const RowsPlan& pl, bool cast, int gs, bool programmatic, cudaStream_t st) {
-    const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl, cast) : gs == 32 ? kernel_for<32>(pl, cast)
-                            : gs == 64 ? kernel_for<64>(pl, cast) : kernel_for<128>(pl, cast);
-    static bool configured[64][2][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
+int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cudaStream_t st) {
+    const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl) : gs == 32 ? kernel_for<32>(pl) : gs == 64 ? kernel_for<64>(pl) : kernel_for<128>(pl);
+    static bool configured[64][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
-    bool& done = configured[dev][pl.stream][cast][gs == 16 ? 0 : gs == 32 ? 1 : gs == 64 ? 2 : 3][pl.nt];
+    bool& done = configured[dev][pl.stream][gs == 16 ? 0 : gs == 32 ? 1 : gs == 64 ? 2 : 3][pl.nt];
     if (!done) {
         if (cudaFuncSetAttribute(kernel.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
             cudaGetLastError();
@@ -716,9 +622,8 @@ int launch_rows(RowsParams p, const RowsPlan& pl, bool cast, int gs, bool progra
     const int cta_rows = pl.stream ? kStreamRows : kCtaRows;
     cfg.gridDim = dim3((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
     cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = pl.stream ? kernel.ring_bytes + (cast ? (size_t)pl.steps_max * p.M * kStepK * 2 : 0)
-                                     : kernel.ring_bytes + (size_t)scale_bytes(held, gs) +
-                                           (cast ? (size_t)pl.steps_max * pl.nt * kFragBytes : kernel.frag_ring_bytes);
+    cfg.dynamicSmemBytes = pl.stream ? kernel.ring_bytes
+                                     : kernel.ring_bytes + (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n = 0;
@@ -779,20 +684,16 @@ int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int
              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace,
              cudaStream_t st) {
     const RowsPlan pl = plan_rows(M, N, K);
-    const bool cast = x && cast_inside(pl, M, N, K), programmatic = programmatic_launch_ok(st);
+    const bool programmatic = programmatic_launch_ok(st);
     RowsParams p{};
-    p.x = static_cast<const uint16_t*>(x);
-    p.ld_x = ld_x;
     p.frag = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(workspace) + kHeaderBytes);
     p.w_codes = w_codes; p.w_scales = w_scales;
     p.M = (int)M; p.N = N; p.K = K; p.C = C; p.ld_c = ld_c;
-    p.status = static_cast<int*>(workspace);
-    if (!cast) {
-        const int rc = x ? launch_fragments<true>(nullptr, nullptr, p.x, ld_x, M, K, gs, pl.tiles(), workspace, programmatic, st)
-                         : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, programmatic, st);
-        if (rc != AMX_OK) return rc;
-    }
-    return launch_rows(p, pl, cast, gs, programmatic, st);
+    const int rc = x ? launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, gs, pl.tiles(), workspace,
+                                              programmatic, st)
+                     : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, programmatic, st);
+    if (rc != AMX_OK) return rc;
+    return launch_rows(p, pl, gs, programmatic, st);
 }
 
 }  // namespace

@@ -45,6 +45,7 @@ gemm_simt_kernel(const uint8_t* __restrict__ a_codes, const ScaleT* __restrict__
                  const uint8_t* __restrict__ w_codes, const ScaleT* __restrict__ w_scales,
                  int64_t M, int64_t N, int64_t K, int gs, float* __restrict__ C, int64_t ld_c,
                  const int* __restrict__ run_if_nonzero) {
+    begin_kernel();
     if (run_if_nonzero && *run_if_nonzero == 0) return;          // uniform over the grid
     __shared__ __align__(16) float As[BK][BM + PAD];
     __shared__ __align__(16) float Ws[BK][BN + PAD];
@@ -87,8 +88,7 @@ int gemm_simt(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_
               int64_t ld_c, cudaStream_t st, const int* run_if_nonzero) {
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
     if (grid.y > 65535) return AMX_ERR_SHAPE;
-    gemm_simt_kernel<uint8_t><<<grid, 256, 0, st>>>(a_codes, a_scales, w_codes, w_scales, M, N, K, gs, C, ld_c, run_if_nonzero);
-    return launch_status();
+    return launch(gemm_simt_kernel<uint8_t>, grid, 256, 0, st, a_codes, a_scales, w_codes, w_scales, M, N, K, gs, C, ld_c, run_if_nonzero);
 }
 
 int gemm_simt_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8_t* w_codes,
@@ -96,8 +96,7 @@ int gemm_simt_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8
                    int64_t ld_c, cudaStream_t st) {
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
     if (grid.y > 65535) return AMX_ERR_SHAPE;
-    gemm_simt_kernel<uint16_t><<<grid, 256, 0, st>>>(a_codes, a_scales, w_codes, w_scales, M, N, K, gs, C, ld_c, nullptr);
-    return launch_status();
+    return launch(gemm_simt_kernel<uint16_t>, grid, 256, 0, st, a_codes, a_scales, w_codes, w_scales, M, N, K, gs, C, ld_c, nullptr);
 }
 
 }  // namespace amx

@@ -118,6 +118,7 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
                int64_t M, int64_t N, int64_t K, float* __restrict__ C, int64_t ld_c, int vec_store,
                int* __restrict__ status, int kb_per_slice, int64_t slice_stride, const int* __restrict__ run_if_nonzero,
                int slices, int first, int group, int causal) {
+    begin_kernel();
     if (run_if_nonzero && *run_if_nonzero == 0) return;          // uniform over the grid: nothing was set up yet
     if (causal && (int64_t)blockIdx.x * BN > (int64_t)blockIdx.y * BM + BM - 1) return;   // a tile above the diagonal
     // blockIdx.z: product of a batch (left operands and results one after another, `group` products share a right
@@ -287,6 +288,7 @@ int k_slices(int64_t M, int64_t N, int64_t K, int& kb_per_slice) {
 __global__ void __launch_bounds__(256)
 reduce_slices_kernel(const float* __restrict__ part, int slices, int64_t M, int64_t N, float* __restrict__ C, int64_t ld_c,
                      const int* __restrict__ run_if_nonzero) {
+    begin_kernel();
     if (run_if_nonzero && *run_if_nonzero == 0) return;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= M * N) return;
@@ -326,7 +328,7 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
     if (const int rc = configure_tc(); rc != AMX_OK) return rc;
     // status word: the first word of the workspace, cleared here, unless the caller shares one it cleared itself
     int* status = status_word ? status_word : static_cast<int*>(workspace);
-    if (!status_word && cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;   // + flushed count: none
+    if (!status_word && clear_words(status, st) != AMX_OK) return AMX_ERR_CUDA;   // + flushed count: none
     int kb_per;
     const int slices = k_slices(M, N, K, kb_per);
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM), (unsigned)slices);
@@ -334,13 +336,13 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
     float* out = slices > 1 ? part : C;
     const int64_t ld_out = slices > 1 ? N : ld_c, slice_stride = slices > 1 ? M * N : 0;
     const int vec_store = aligned(out, 16) && ld_out % 4 == 0;   // else the epilogue stores scalars
+    int rc;
     if (a_x)
-        gemm_tc_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(nullptr, nullptr, a_x, ld_a, w_codes, w_scales, M, N, K, out,
+        rc = launch(gemm_tc_kernel<true>, grid, kThreads, kSmemBytes, st, nullptr, nullptr, a_x, ld_a, w_codes, w_scales, M, N, K, out,
                                                                  ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
     else
-        gemm_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K,
+        rc = launch(gemm_tc_kernel<false>, grid, kThreads, kSmemBytes, st, a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K,
                                                                   out, ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
-    int rc = launch_status();
     if (rc != AMX_OK || slices == 1) return rc;
     return reduce_slices(part, slices, M, N, C, ld_c, st, gate);
 }
@@ -349,8 +351,7 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
 
 int reduce_slices(const float* part, int slices, int64_t M, int64_t N, float* C, int64_t ld_c, cudaStream_t st,
                   const int* run_if_nonzero) {
-    reduce_slices_kernel<<<(unsigned)((M * N + 255) / 256), 256, 0, st>>>(part, slices, M, N, C, ld_c, run_if_nonzero);
-    return launch_status();
+    return launch(reduce_slices_kernel, (unsigned)((M * N + 255) / 256), 256, 0, st, part, slices, M, N, C, ld_c, run_if_nonzero);
 }
 
 // run_if_nonzero: the launches do nothing when that device word is zero.  status_word: where a timeout is
@@ -383,20 +384,18 @@ int gemm_tc_batched(const uint8_t* a_codes, const uint8_t* a_scales, const uint8
     int rc = configure_tc();
     if (rc != AMX_OK) return rc;
     int* status = static_cast<int*>(workspace);
-    if (cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (clear_words(status, st) != AMX_OK) return AMX_ERR_CUDA;
     int kb_per;
     const int slices = k_slices(M, N, K, kb_per);
     if (batch * slices > 65535) return AMX_ERR_SHAPE;
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM), (unsigned)(batch * slices));
     float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
     float* out = slices > 1 ? part : C;
-    gemm_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, out, N,
+    rc = launch(gemm_tc_kernel<false>, grid, kThreads, kSmemBytes, st, a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, out, N,
                                                               aligned(out, 16) && N % 4 == 0 && (M * N) % 4 == 0, status, kb_per, M * N,
                                                               nullptr, slices, (int)first, (int)group, causal);
-    rc = launch_status();
     if (rc != AMX_OK || slices == 1) return rc;
-    reduce_slices_kernel<<<dim3((unsigned)((M * N + 255) / 256), (unsigned)batch), 256, 0, st>>>(part, slices, M, N, C, N, nullptr);
-    return launch_status();
+    return launch(reduce_slices_kernel, dim3((unsigned)((M * N + 255) / 256), (unsigned)batch), 256, 0, st, part, slices, M, N, C, N, nullptr);
 }
 
 int gemm_tc_status(const void* workspace, cudaStream_t st) {

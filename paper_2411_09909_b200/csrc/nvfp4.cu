@@ -30,6 +30,7 @@ using namespace fp4;
 // bits[1], which the caller zeroed.
 __global__ void __launch_bounds__(256)
 absmax_kernel(const uint4* __restrict__ x, int64_t n_vec, int64_t vec_per_row, int64_t ld_vec, unsigned* __restrict__ bits) {
+    begin_kernel();
     uint32_t m = 0;
     for (int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x; v < n_vec; v += (int64_t)gridDim.x * 256) {
         const uint4 q = __ldg(x + (v / vec_per_row) * ld_vec + v % vec_per_row);
@@ -69,6 +70,7 @@ cast_nv_kernel(const uint4* __restrict__ x, int64_t rows, int chunks_per_row, in
                uint4* __restrict__ codes, uint2* __restrict__ scales, uint4* __restrict__ pos, uint4* __restrict__ neg,
                uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int nk64,
                float* __restrict__ prepared_scale) {
+    begin_kernel();
     const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const float amax = tensor_scale[1];
     const float t = amax > 0.0f ? __fdiv_rn(amax, 2688.0f) : 1.0f;
@@ -138,6 +140,7 @@ template <bool F32>
 __global__ void __launch_bounds__(256)
 dequantize_nv_kernel(const uint32_t* __restrict__ codes, const uint16_t* __restrict__ scales, const float* __restrict__ tensor_scale,
                      int64_t n_vec, int64_t vec_per_row, int64_t ld_out, void* __restrict__ out) {
+    begin_kernel();
     const int64_t v = (int64_t)blockIdx.x * 256 + threadIdx.x;       // 8 elements per thread, half a group
     if (v >= n_vec) return;
     const uint32_t nib = codes[v], sc = scales[v >> 1];
@@ -190,25 +193,22 @@ extern "C" int amx_quantize_nvfp4(const void* x, int64_t rows, int64_t K, int64_
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const fp4::OperandLayout o = fp4::operand_layout(rows, K, is_weight ? 256 : 128);
     uint8_t* base = static_cast<uint8_t*>(prepared);
-    if (cudaMemsetAsync(tensor_scale, 0, 8, st) != cudaSuccess) return AMX_ERR_CUDA;
     // padding rows and padding chunks of the scale factors are zero (both planes)
     if (prepared && cudaMemsetAsync(base + 2 * o.plane, 0, 2 * o.sf, st) != cudaSuccess) return AMX_ERR_CUDA;
+    if (clear_words(tensor_scale, st) != AMX_OK) return AMX_ERR_CUDA;
     const int64_t n_vec = rows * (K / 8);
     int64_t blocks = (n_vec + 255) / 256;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    absmax_kernel<<<(unsigned)blocks, 256, 0, st>>>(static_cast<const uint4*>(x), n_vec, K / 8, ld_x / 8,
+    int rc = launch(absmax_kernel, (unsigned)blocks, 256, 0, st, static_cast<const uint4*>(x), n_vec, K / 8, ld_x / 8,
                                                     reinterpret_cast<unsigned*>(tensor_scale));
-    int rc = launch_status();
     if (rc != AMX_OK) return rc;
     const int64_t items = rows * (K / 64);
     auto* kernel = (flags & AMX_NV_ASYMMETRIC) ? cast_nv_kernel<true> : cast_nv_kernel<false>;
-    kernel<<<(unsigned)((items + 255) / 256), 256, 0, st>>>(
-        static_cast<const uint4*>(x), rows, (int)(K / 64), ld_x / 8, tensor_scale, reinterpret_cast<uint4*>(codes),
+    return launch(kernel, (unsigned)((items + 255) / 256), 256, 0, st, static_cast<const uint4*>(x), rows, (int)(K / 64), ld_x / 8, tensor_scale, reinterpret_cast<uint4*>(codes),
         reinterpret_cast<uint2*>(scales), reinterpret_cast<uint4*>(base), prepared ? reinterpret_cast<uint4*>(base + o.plane) : nullptr,
         prepared ? base + 2 * o.plane : nullptr, prepared ? base + 2 * o.plane + o.sf : nullptr,
         prepared ? reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf) : nullptr, o.nk64,
         prepared ? reinterpret_cast<float*>(base + o.total) : nullptr);
-    return launch_status();
 }
 
 extern "C" int amx_dequantize_nvfp4(const uint8_t* codes, const uint8_t* scales, const float* tensor_scale, int64_t rows,
@@ -223,9 +223,8 @@ extern "C" int amx_dequantize_nvfp4(const uint8_t* codes, const uint8_t* scales,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     auto* cv = reinterpret_cast<const uint32_t*>(codes);
     auto* sv = reinterpret_cast<const uint16_t*>(scales);
-    if (flags & AMX_OUT_F32) dequantize_nv_kernel<true><<<(unsigned)blocks, 256, 0, st>>>(cv, sv, tensor_scale, n_vec, K / 8, ld_out, out);
-    else dequantize_nv_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(cv, sv, tensor_scale, n_vec, K / 8, ld_out, out);
-    return launch_status();
+    if (flags & AMX_OUT_F32) return launch(dequantize_nv_kernel<true>, (unsigned)blocks, 256, 0, st, cv, sv, tensor_scale, n_vec, K / 8, ld_out, out);
+    return launch(dequantize_nv_kernel<false>, (unsigned)blocks, 256, 0, st, cv, sv, tensor_scale, n_vec, K / 8, ld_out, out);
 }
 
 namespace {

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kThreads) quant_error_kernel(const uint16_t* _
                                                                int64_t ld_x, const uint8_t* __restrict__ codes,
                                                                const uint8_t* __restrict__ scales, int gs_log2,
                                                                double* __restrict__ partial) {
+    begin_kernel();
     __shared__ double sh[kThreads / 32][4];
     // grid x walks the 16-element chunks of a row, grid y the rows: no division per chunk
     const int64_t per_row = K / 16, groups = K >> gs_log2;
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kThreads) quant_error_kernel(const uint16_t* _
 
 __global__ void __launch_bounds__(kThreads) quant_error_final_kernel(const double* __restrict__ partial, int blocks,
                                                                      double* __restrict__ out) {
+    begin_kernel();
     __shared__ double sh[kThreads / 32][4];
     Sums s = {0, 0, 0, 0};
     for (int b = threadIdx.x; b < blocks; b += kThreads) {
@@ -141,15 +143,15 @@ int quant_error(const void* x, int64_t rows, int64_t K, int64_t ld_x, const uint
     double* partial = static_cast<double*>(workspace);
     const int gs_log2 = group_size == 16 ? 4 : group_size == 32 ? 5 : group_size == 64 ? 6 : 7;
     const dim3 grid((unsigned)bx, (unsigned)by);
+    int rc;
     if (f16s)
-        quant_error_kernel<true><<<grid, kThreads, 0, st>>>(static_cast<const uint16_t*>(x), rows, K, ld_x, codes,
+        rc = launch(quant_error_kernel<true>, grid, kThreads, 0, st, static_cast<const uint16_t*>(x), rows, K, ld_x, codes,
                                                             static_cast<const uint8_t*>(scales), gs_log2, partial);
     else
-        quant_error_kernel<false><<<grid, kThreads, 0, st>>>(static_cast<const uint16_t*>(x), rows, K, ld_x, codes,
+        rc = launch(quant_error_kernel<false>, grid, kThreads, 0, st, static_cast<const uint16_t*>(x), rows, K, ld_x, codes,
                                                              static_cast<const uint8_t*>(scales), gs_log2, partial);
-    if (launch_status() != AMX_OK) return AMX_ERR_CUDA;
-    quant_error_final_kernel<<<1, kThreads, 0, st>>>(partial, (int)blocks, out);
-    return launch_status();
+    if (rc != AMX_OK) return rc;
+    return launch(quant_error_final_kernel, 1, kThreads, 0, st, partial, (int)blocks, out);
 }
 }  // namespace
 

@@ -34,6 +34,7 @@ template <int EPT, int TPG, bool CONTIG, int FMT = 0>
 __global__ void __launch_bounds__(kThreads)
 quantize_rows_kernel(const uint4* __restrict__ x, int64_t n_items, int64_t items_per_row,
                      int64_t ld_vec, uint4* __restrict__ codes, uint16_t* __restrict__ scales) {
+    begin_kernel();
     constexpr int NV = EPT / 8;
     const int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     uint32_t w[NV * 4];
@@ -70,6 +71,7 @@ template <int FMT>
 __global__ void __launch_bounds__(kThreads)
 quantize_whole_rows_kernel(const uint4* __restrict__ x, int64_t vec_per_row, int64_t ld_vec, uint32_t* __restrict__ codes,
                            uint16_t* __restrict__ scales) {
+    begin_kernel();
     __shared__ uint32_t red[kThreads / 32];
     const int64_t row = blockIdx.x;
     const uint4* xr = x + row * ld_vec;
@@ -103,6 +105,7 @@ template <int TPG>
 __global__ void __launch_bounds__(kThreads)
 quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t R, int64_t C, int64_t ld,
                      uint32_t* __restrict__ codes, uint16_t* __restrict__ scales, int gs) {
+    begin_kernel();
     // blockIdx.z: one of several [R, C] matrices stored one after another (R * ld elements apart); their
     // transposed outputs follow one another as well
     __shared__ uint16_t tile[kTC][kTR + 2];  // [column][row], padded
@@ -222,6 +225,7 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_rows, i
                      uint4* __restrict__ codes, uint16_t* __restrict__ scales, uint4* __restrict__ pos,
                      uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg,
                      int* __restrict__ row_exp, int nk64, int* __restrict__ flushed_total) {
+    begin_kernel();
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, LPR = 1 << lpr_log2, lr = lane & (LPR - 1);
     const int RPW = 32 >> lpr_log2, sg = lane >> lpr_log2;      // rows per warp; which of them this lane works on
@@ -344,6 +348,7 @@ softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s,
                     uint4* __restrict__ codes, uint16_t* __restrict__ scales, uint4* __restrict__ pos,
                     uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg,
                     int* __restrict__ row_exp, int nk64) {
+    begin_kernel();
     __shared__ float sh[softmax::kT / 32];
     __shared__ int slot_s[4];
     const int gx = threadIdx.x;
@@ -388,6 +393,7 @@ softmax_cast_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s,
 __global__ void __launch_bounds__(256)
 softmax_cast_warp_kernel(const float* __restrict__ S, int64_t R, int G, int64_t ld_s, float alpha, int vec, int64_t causal,
                          uint4* __restrict__ codes, uint16_t* __restrict__ scales) {
+    begin_kernel();
     const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= R) return;
@@ -427,10 +433,8 @@ int launch_rows(const void* x, int64_t rows, int64_t K, int64_t ld, uint8_t* cod
     auto* cv = reinterpret_cast<uint4*>(codes);
     auto* sv = reinterpret_cast<uint16_t*>(scales);
     if (ld == K)
-        quantize_rows_kernel<EPT, TPG, true, FMT><<<(unsigned)blocks, kThreads, 0, st>>>(xv, n_items, K / EPT, ld / 8, cv, sv);
-    else
-        quantize_rows_kernel<EPT, TPG, false, FMT><<<(unsigned)blocks, kThreads, 0, st>>>(xv, n_items, K / EPT, ld / 8, cv, sv);
-    return launch_status();
+        return launch(quantize_rows_kernel<EPT, TPG, true, FMT>, (unsigned)blocks, kThreads, 0, st, xv, n_items, K / EPT, ld / 8, cv, sv);
+    return launch(quantize_rows_kernel<EPT, TPG, false, FMT>, (unsigned)blocks, kThreads, 0, st, xv, n_items, K / EPT, ld / 8, cv, sv);
 }
 
 }  // namespace
@@ -467,11 +471,9 @@ int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes,
         }
         configured[dev][slot] = true;
     }
-    kernel<<<(unsigned)blocks, kCastWarps * 32, smem, st>>>(
-        reinterpret_cast<const uint4*>(x), rows, seg_rows, seg_pad, (int)G, lpr_log2, exchange, reinterpret_cast<uint4*>(codes),
+    return launch(kernel, (unsigned)blocks, kCastWarps * 32, smem, st, reinterpret_cast<const uint4*>(x), rows, seg_rows, seg_pad, (int)G, lpr_log2, exchange, reinterpret_cast<uint4*>(codes),
         reinterpret_cast<uint16_t*>(scales), reinterpret_cast<uint4*>(pos), reinterpret_cast<uint4*>(neg), sf_pos, sf_neg,
         row_exp, nk64, flushed_total);
-    return launch_status();
 }
 }  // namespace
 
@@ -496,15 +498,13 @@ int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, 
     if (blocks > 0x7FFFFFFF || G > 0x7FFFFFFF / 32) return AMX_ERR_SHAPE;
     const int vec = aligned(S, 16) && ld_s % 4 == 0;
     if (!pos && G <= 32) {
-        softmax_cast_warp_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(S, rows, (int)G, ld_s, alpha, vec, causal,
+        return launch(softmax_cast_warp_kernel, (unsigned)((rows + 7) / 8), 256, 0, st, S, rows, (int)G, ld_s, alpha, vec, causal,
                                                                             reinterpret_cast<uint4*>(codes), reinterpret_cast<uint16_t*>(scales));
-        return launch_status();
     }
     auto* kernel = G <= softmax::kT ? softmax_cast_kernel<true> : softmax_cast_kernel<false>;
-    kernel<<<(unsigned)blocks, softmax::kT, 0, st>>>(S, rows, (int)G, ld_s, alpha, vec, causal, reinterpret_cast<uint4*>(codes),
+    return launch(kernel, (unsigned)blocks, softmax::kT, 0, st, S, rows, (int)G, ld_s, alpha, vec, causal, reinterpret_cast<uint4*>(codes),
                                                      reinterpret_cast<uint16_t*>(scales), reinterpret_cast<uint4*>(pos),
                                                      reinterpret_cast<uint4*>(neg), sf_pos, sf_neg, row_exp, nk64);
-    return launch_status();
 }
 
 namespace {
@@ -520,6 +520,7 @@ template <int C>
 __global__ void __launch_bounds__(256)
 cast_cols_planes_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_pad, uint4* __restrict__ pos, uint4* __restrict__ neg,
                         uint16_t* __restrict__ scales) {
+    begin_kernel();
     constexpr int kWords = C / 2, kVec = C / 8;               // 32-bit words and 16-byte pieces per key
     __shared__ __align__(16) uint32_t tile[128 * kWords];
     const int64_t key0 = (int64_t)blockIdx.x * 128, batch = blockIdx.y;
@@ -552,10 +553,8 @@ int launch_cols(const void* x, int64_t R, int64_t C, int64_t ld, int gs, uint8_t
                 uint8_t* scales, cudaStream_t st, int64_t batch = 1) {
     dim3 grid((unsigned)((C + kTC - 1) / kTC), (unsigned)((R + kTR - 1) / kTR), (unsigned)batch);
     if (grid.y > 65535 || batch > 65535) return AMX_ERR_SHAPE;
-    quantize_cols_kernel<TPG><<<grid, kThreads, 0, st>>>(
-        reinterpret_cast<const __nv_bfloat16*>(x), R, C, ld, reinterpret_cast<uint32_t*>(codes),
+    return launch(quantize_cols_kernel<TPG>, grid, kThreads, 0, st, reinterpret_cast<const __nv_bfloat16*>(x), R, C, ld, reinterpret_cast<uint32_t*>(codes),
         reinterpret_cast<uint16_t*>(scales), gs);
-    return launch_status();
 }
 
 }  // namespace
@@ -566,9 +565,8 @@ int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int
     if (batch > 65535 || (C != 64 && C != 128)) return AMX_ERR_SHAPE;
     const dim3 grid((unsigned)((R + 127) / 128), (unsigned)batch);
     auto* kernel = C == 128 ? cast_cols_planes_kernel<128> : cast_cols_planes_kernel<64>;
-    kernel<<<grid, 256, 0, st>>>(static_cast<const uint4*>(x), R, seg_pad, static_cast<uint4*>(pos), static_cast<uint4*>(neg),
+    return launch(kernel, grid, 256, 0, st, static_cast<const uint4*>(x), R, seg_pad, static_cast<uint4*>(pos), static_cast<uint4*>(neg),
                                  reinterpret_cast<uint16_t*>(scales));
-    return launch_status();
 }
 
 // amx_quantize_t with group size 32 on `batch` matrices [R, C] stored one after another (contiguous rows); the
@@ -587,10 +585,8 @@ int launch_rows_gs(const void* x, int64_t rows, int64_t K, int64_t ld_x, int gro
                    cudaStream_t st) {
     if (group_size == K && !fixed_group_size(group_size)) {          // whole-row grouping
         if (rows > 0x7FFFFFFF) return AMX_ERR_SHAPE;
-        quantize_whole_rows_kernel<FMT><<<(unsigned)rows, kThreads, 0, st>>>(
-            reinterpret_cast<const uint4*>(x), K / 8, ld_x / 8, reinterpret_cast<uint32_t*>(codes),
+        return launch(quantize_whole_rows_kernel<FMT>, (unsigned)rows, kThreads, 0, st, reinterpret_cast<const uint4*>(x), K / 8, ld_x / 8, reinterpret_cast<uint32_t*>(codes),
             reinterpret_cast<uint16_t*>(scales));
-        return launch_status();
     }
     switch (group_size) {
         case 16: return launch_rows<16, 1, FMT>(x, rows, K, ld_x, codes, scales, st);

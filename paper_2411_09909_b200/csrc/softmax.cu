@@ -28,6 +28,7 @@ __device__ __forceinline__ void store_group(uint16_t* __restrict__ p, int64_t g,
 __global__ void __launch_bounds__(kT)
 softmax_bf16_cached_kernel(const float* __restrict__ S, int G, int64_t ld_s, float alpha, uint16_t* __restrict__ P,
                            int64_t ld_p, int vec_in, int vec_out) {
+    begin_kernel();
     __shared__ float sh[kT / 32];
     float e[32];
     const float sum = cached_row_exp(S + (int64_t)blockIdx.x * ld_s, G, vec_in != 0, alpha, sh, e, (int64_t)G * 32);
@@ -41,6 +42,7 @@ softmax_bf16_cached_kernel(const float* __restrict__ S, int G, int64_t ld_s, flo
 __global__ void __launch_bounds__(kT)
 softmax_bf16_kernel(const float* __restrict__ S, int64_t cols, int64_t ld_s, float alpha,
                     uint16_t* __restrict__ P, int64_t ld_p, int vec_in, int vec_out) {
+    begin_kernel();
     __shared__ float sh[kT / 32];
     const float* s = S + (int64_t)blockIdx.x * ld_s;
     uint16_t* p = P + (int64_t)blockIdx.x * ld_p;
@@ -70,10 +72,6 @@ extern "C" int amx_softmax_bf16(const float* S, int64_t rows, int64_t cols, int6
     const int vec_in = whole && aligned(S, 16) && ld_s % 4 == 0;
     const int vec_out = whole && aligned(P, 16) && ld_p % 8 == 0;
     if (whole && cols / 32 <= softmax::kT)
-        softmax_bf16_cached_kernel<<<(unsigned)rows, softmax::kT, 0, static_cast<cudaStream_t>(stream)>>>(
-            S, (int)(cols / 32), ld_s, alpha, reinterpret_cast<uint16_t*>(P), ld_p, vec_in, vec_out);
-    else
-        softmax_bf16_kernel<<<(unsigned)rows, softmax::kT, 0, static_cast<cudaStream_t>(stream)>>>(
-            S, cols, ld_s, alpha, reinterpret_cast<uint16_t*>(P), ld_p, vec_in, vec_out);
-    return launch_status();
+        return launch(softmax_bf16_cached_kernel, (unsigned)rows, softmax::kT, 0, static_cast<cudaStream_t>(stream), S, (int)(cols / 32), ld_s, alpha, reinterpret_cast<uint16_t*>(P), ld_p, vec_in, vec_out);
+    return launch(softmax_bf16_kernel, (unsigned)rows, softmax::kT, 0, static_cast<cudaStream_t>(stream), S, cols, ld_s, alpha, reinterpret_cast<uint16_t*>(P), ld_p, vec_in, vec_out);
 }
