@@ -7,6 +7,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "amx_common.cuh"
 
@@ -102,4 +103,37 @@ __device__ __forceinline__ uint4 decode_pairs_up(uint32_t w, const GroupScales& 
 }
 
 }  // namespace decode
+
+// Exact decode to f16 times 2^-4: E2M1 x E5M2 has at most 5 significant bits and magnitudes between 2^-17 and 6 * 57344, so
+// that every value times 2^-4 is a (possibly subnormal) f16 number.
+namespace decode_f16 {
+
+__device__ __forceinline__ __half2 h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
+__device__ __forceinline__ uint32_t u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
+
+// The two side scales of a group as f16 pairs times 2^-4.  An E5M2 byte is the upper byte of the same half.
+struct Scales {
+    __half2 pos, neg;
+};
+__device__ __forceinline__ Scales make_scales(uint32_t sc) {
+    const __half2 down = h2(0x2C002C00u);                            // 2^-4
+    return {__hmul2(h2(__byte_perm(sc, 0, 0x0404)), down), __hmul2(h2(__byte_perm(sc, 0, 0x1414)), down)};
+}
+// Two elements from byte I of a code word.
+template <int I>
+__device__ __forceinline__ uint32_t decode_pair(uint32_t w, const Scales& s) {
+    uint32_t v;
+    if (I == 0) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, a;}" : "=r"(v) : "r"(w));
+    if (I == 1) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, b;}" : "=r"(v) : "r"(w));
+    if (I == 2) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, c;}" : "=r"(v) : "r"(w));
+    if (I == 3) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, d;}" : "=r"(v) : "r"(w));
+    uint32_t pos;
+    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(pos) : "r"(v), "r"(u32(s.pos)), "r"(0u));
+    return u32(__hfma2(__hmin2(h2(v), h2(0u)), s.neg, h2(pos)));
+}
+__device__ __forceinline__ uint4 decode_word(uint32_t w, const Scales& s) {
+    return make_uint4(decode_pair<0>(w, s), decode_pair<1>(w, s), decode_pair<2>(w, s), decode_pair<3>(w, s));
+}
+
+}  // namespace decode_f16
 }  // namespace amx

@@ -38,12 +38,15 @@
 
 #include "cast_math.cuh"
 #include "cp_async.cuh"
+#include "decode_math.cuh"
 #include "gemm.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace amx {
 namespace {
+
+using namespace decode_f16;
 
 constexpr int kWarps = 8, kThreads = kWarps * 32;
 constexpr int kRowGroups = 4, kStepGroups = 2;     // warps: 4 groups of 32 weight rows x 2 step parities
@@ -56,33 +59,6 @@ constexpr int kMaxSlices = 8;                      // portable cluster size
 constexpr int kPartPitch = kCtaRows + 4;           // floats per token row of the partial-product tile (bank spread)
 constexpr int kMaxTiles = 8;                       // token tiles per CTA
 constexpr int kScaleSteps = 32;                    // steps whose scales are held at a time
-
-__device__ __forceinline__ __half2 h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
-__device__ __forceinline__ uint32_t u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
-
-// The two side scales of a group as f16 pairs times 2^-4.  An E5M2 byte is the upper byte of the same half.
-struct Scales {
-    __half2 pos, neg;
-};
-__device__ __forceinline__ Scales make_scales(uint32_t sc) {
-    const __half2 down = h2(0x2C002C00u);                            // 2^-4
-    return {__hmul2(h2(__byte_perm(sc, 0, 0x0404)), down), __hmul2(h2(__byte_perm(sc, 0, 0x1414)), down)};
-}
-// Two elements from byte I of a code word.
-template <int I>
-__device__ __forceinline__ uint32_t decode_pair(uint32_t w, const Scales& s) {
-    uint32_t v;
-    if (I == 0) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, a;}" : "=r"(v) : "r"(w));
-    if (I == 1) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, b;}" : "=r"(v) : "r"(w));
-    if (I == 2) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, c;}" : "=r"(v) : "r"(w));
-    if (I == 3) asm("{.reg .b8 a, b, c, d; mov.b32 {a, b, c, d}, %1; cvt.rn.f16x2.e2m1x2 %0, d;}" : "=r"(v) : "r"(w));
-    uint32_t pos;
-    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(pos) : "r"(v), "r"(u32(s.pos)), "r"(0u));
-    return u32(__hfma2(__hmin2(h2(v), h2(0u)), s.neg, h2(pos)));
-}
-__device__ __forceinline__ uint4 decode_word(uint32_t w, const Scales& s) {
-    return make_uint4(decode_pair<0>(w, s), decode_pair<1>(w, s), decode_pair<2>(w, s), decode_pair<3>(w, s));
-}
 
 // Fragment order of the token rows, per step and tile of 8 rows: pieces of 16 bytes [j = 0..3][lane 0..31]; the piece
 // of (j, lane (g, t)) holds elements 32 t + 8 j .. + 7 of the step, row g of the tile.  Piece (j, l) sits at position
