@@ -123,12 +123,12 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
         return AMX_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (kernel == AMX_GEMM_SIMT)
-        return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st);
+        return gemm_simt({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, group_size, C, ld_c, st);
     // AUTO picked a kernel whose alignment the operands miss (the weight-streaming kernel copies scales 4 bytes at a time;
     // 16-byte codes for group sizes that used to run on the plain kernel): the plain kernel takes them and needs no scratch
     const bool codes16 = aligned(a_codes, 16) && aligned(w_codes, 16), is_auto = (flags & kKernelMask) == AMX_GEMM_AUTO;
     if (is_auto && ((kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) || (group_size != 32 && !codes16)))
-        return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st);
+        return gemm_simt({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, group_size, C, ld_c, st);
     if (!codes16 || (kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4))) return AMX_ERR_ALIGN;
     const bool fallback = auto_fallback(flags, kernel);
     const size_t need = kernel_workspace(kernel, M, N, K, fallback, group_size);
@@ -139,13 +139,13 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
         if (rc != AMX_OK || !fallback) return rc;
         int* words = static_cast<int*>(workspace);       // [0] status, [1] flushed scales
         if (group_size != 32)
-            return gemm_simt(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, st, words + 1);
-        return gemm_tc(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c,
+            return gemm_simt({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, group_size, C, ld_c, st, words + 1);
+        return gemm_tc({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, C, ld_c,
                        static_cast<uint8_t*>(workspace) + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
     }
     if (kernel == AMX_GEMM_ROWS)
         return gemm_rows(a_codes, a_scales, w_codes, w_scales, M, N, K, group_size, C, ld_c, workspace, st);
-    return gemm_tc(a_codes, a_scales, w_codes, w_scales, M, N, K, C, ld_c, workspace, st);
+    return gemm_tc({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, C, ld_c, workspace, st);
 }
 
 extern "C" size_t amx_prepared_bytes(int64_t rows, int64_t K, int group_size, int is_weight) {
@@ -159,7 +159,8 @@ extern "C" int amx_prepare(const uint8_t* codes, const uint8_t* scales, int64_t 
     if (!codes || !scales || !prepared) return AMX_ERR_NULL;
     if (prepared_bytes < amx_prepared_bytes(rows, K, group_size, is_weight)) return AMX_ERR_WORKSPACE;
     if (!aligned(codes, 16) || !aligned(scales, 2) || !aligned(prepared, kAlign)) return AMX_ERR_ALIGN;
-    return gemm_fp4_prepare(codes, scales, rows, K, is_weight != 0, prepared, static_cast<cudaStream_t>(stream));
+    const PrepOperand op = gemm_fp4_split_operand(codes, scales, rows, K, is_weight != 0, prepared);
+    return gemm_fp4_prepare_operands(&op, 1, K, 32, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int amx_quantize_prepared(const void* x, int64_t rows, int64_t K, int group_size, int is_weight,
@@ -177,8 +178,8 @@ extern "C" int amx_quantize_prepared_fmt(const void* x, int64_t rows, int64_t K,
     if (!x || !scales || !prepared) return AMX_ERR_NULL;       // codes may be NULL: they are then not written
     if (prepared_bytes < amx_prepared_bytes(rows, K, group_size, is_weight)) return AMX_ERR_WORKSPACE;
     if (!aligned(x, 16) || !aligned(codes, 16) || !aligned(scales, 2) || !aligned(prepared, kAlign)) return AMX_ERR_ALIGN;
-    return gemm_fp4_quantize_prepared(x, rows, K, is_weight != 0, codes, scales, prepared, static_cast<cudaStream_t>(stream),
-                                      0, format);
+    const PrepOperand op = gemm_fp4_cast_operand(x, K, rows, K, is_weight != 0, codes, scales, prepared);
+    return gemm_fp4_prepare_operands(&op, 1, K, 32, static_cast<cudaStream_t>(stream), format);
 }
 
 extern "C" size_t amx_gemm_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K, int group_size) {
@@ -264,34 +265,24 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
     uint8_t* wq_scales = wq_codes + w.codes;
     int rc = AMX_OK;
     if (kernel == AMX_GEMM_FP4) {
-        // Both casts write the kernel's operands themselves where the rows are contiguous (one launch per operand,
-        // the codes are not read again); workspace: status word and flushed-scale count, prepared A, prepared W
+        // One launch casts the activation and casts or splits the weight, straight into the kernel's operands; workspace:
+        // status word and flushed-scale count, prepared A, prepared W.  (The canonical codes of what is cast here exist
+        // only as the two planes.)
         uint8_t* pa = base + 256;
         uint8_t* pw = pa + gemm_fp4_prepared_bytes(M, K, false);
         int* words = reinterpret_cast<int*>(base);
         if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
-        if (ld_a == K && group_size == 32) rc = gemm_fp4_quantize_prepared(A, M, K, false, a_codes, a_scales, pa, st, 0, AMX_FMT_AMXFP4, words + 1);
-        else {
-            rc = amx_quantize(A, M, K, ld_a, group_size, a_codes, a_scales, stream);
-            if (rc == AMX_OK) rc = gemm_fp4_prepare(a_codes, a_scales, M, K, false, pa, st, 0, words + 1, group_size);
-        }
-        if (rc != AMX_OK) return rc;
-        if (w_is_bf16 && ld_w == K && group_size == 32)
-            rc = gemm_fp4_quantize_prepared(W_bf16, N, K, true, wq_codes, wq_scales, pw, st, 0, AMX_FMT_AMXFP4, words + 1);
-        else {
-            if (w_is_bf16) rc = amx_quantize(W_bf16, N, K, ld_w, group_size, wq_codes, wq_scales, stream);
-            if (rc == AMX_OK)
-                rc = gemm_fp4_prepare(w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, N, K, true, pw, st, 0,
-                                      words + 1, group_size);
-        }
+        const PrepOperand op[2] = {gemm_fp4_cast_operand(A, ld_a, M, K, false, nullptr, a_scales, pa),
+                                   w_is_bf16 ? gemm_fp4_cast_operand(W_bf16, ld_w, N, K, true, nullptr, wq_scales, pw)
+                                             : gemm_fp4_split_operand(w_codes, w_scales, N, K, true, pw)};
+        rc = gemm_fp4_prepare_operands(op, 2, K, group_size, st, AMX_FMT_AMXFP4, words + 1);
         if (rc != AMX_OK) return rc;
         rc = gemm_fp4_prepared(pa, pw, M, N, K, C, ld_c, base, st, 256, fallback ? words + 1 : nullptr);
         if (rc != AMX_OK || !fallback) return rc;
-        if (group_size != 32)
-            return gemm_simt(a_codes, a_scales, w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, M, N, K, group_size,
-                             C, ld_c, st, words + 1);
-        return gemm_tc(a_codes, a_scales, w_is_bf16 ? wq_codes : w_codes, w_is_bf16 ? wq_scales : w_scales, M, N, K, C, ld_c,
-                       base + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
+        const CodePlanes ac{pa, pa + gemm_fp4_plane_bytes(M, K)}, wc = w_is_bf16 ? CodePlanes{pw, pw + gemm_fp4_plane_bytes(N, K)} : CodePlanes{w_codes};
+        const uint8_t* ws = w_is_bf16 ? wq_scales : w_scales;
+        if (group_size != 32) return gemm_simt(ac, a_scales, wc, ws, M, N, K, group_size, C, ld_c, st, words + 1);
+        return gemm_tc(ac, a_scales, wc, ws, M, N, K, C, ld_c, base + round_up(gemm_fp4_workspace_bytes(M, N, K)), st, words + 1, words);
     }
     if (w_is_bf16) {
         rc = amx_quantize(W_bf16, N, K, ld_w, group_size, wq_codes, wq_scales, stream);
@@ -639,11 +630,9 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
             // (V^T).  The chunk starts at a group boundary unless the group is larger than a chunk, in which case it
             // lies inside one group (every head maps to the chunk's one head of keys and values either way).
             const int64_t Lp = attn_fused_padded(L);
-            rc = gemm_fp4_quantize_prepared(qh, hc * Lp, d, false, nullptr, w + a.qs, w + a.pq, st, chunk_max * Lp, AMX_FMT_AMXFP4,
-                                            words + 1, L, Lp);
-            if (rc == AMX_OK)
-                rc = gemm_fp4_quantize_prepared(kh, kvc * Lp, d, true, nullptr, w + a.ks, w + a.pk, st, chunk_max * Lp,
-                                                AMX_FMT_AMXFP4, words + 1, L, Lp);
+            const PrepOperand op[2] = {gemm_fp4_cast_operand(qh, d, hc * Lp, d, false, nullptr, w + a.qs, w + a.pq, chunk_max * Lp, L, Lp),
+                                       gemm_fp4_cast_operand(kh, d, kvc * Lp, d, true, nullptr, w + a.ks, w + a.pk, chunk_max * Lp, L, Lp)};
+            rc = gemm_fp4_prepare_operands(op, 2, d, 32, st, AMX_FMT_AMXFP4, words + 1);
             if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(vh, kvc, L, d, 128, chunk_max * 128, w + a.vs, w + a.pv, st, words + 1);
             const int kv_group = (int)(group >= chunk_max ? chunk_max : group);
             float* oh = o + (size_t)h0 * L * d;
@@ -662,16 +651,18 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
         }
         // casts of the chunk's heads, stacked row-wise: Q and K along head_dim, V along the sequence (V^T)
         if (k_qk == AMX_GEMM_FP4) {
-            rc = gemm_fp4_quantize_prepared(qh, hc * L, d, false, nullptr, w + a.qs, w + a.pq, st, chunk_max * L);
-            if (rc == AMX_OK)
-                rc = gemm_fp4_quantize_prepared(kh, kvc * L, d, true, nullptr, w + a.ks, w + a.pk, st, chunk_max * L + 128);
+            const PrepOperand op[2] = {gemm_fp4_cast_operand(qh, d, hc * L, d, false, nullptr, w + a.qs, w + a.pq, chunk_max * L),
+                                       gemm_fp4_cast_operand(kh, d, kvc * L, d, true, nullptr, w + a.ks, w + a.pk, chunk_max * L + 128)};
+            rc = gemm_fp4_prepare_operands(op, 2, d, 32, st);
         } else {
             rc = amx_quantize(qh, hc * L, d, d, 32, w + a.qc, w + a.qs, stream);
             if (rc == AMX_OK) rc = amx_quantize(kh, kvc * L, d, d, 32, w + a.kc, w + a.ks, stream);
         }
         if (rc == AMX_OK) rc = quantize_cols_batched(vh, kvc, L, d, w + a.vc, w + a.vs, st);
-        if (rc == AMX_OK && k_pv == AMX_GEMM_FP4)
-            rc = gemm_fp4_prepare(w + a.vc, w + a.vs, kvc * d, L, true, w + a.pv, st, chunk_max * d + 128);
+        if (rc == AMX_OK && k_pv == AMX_GEMM_FP4) {
+            const PrepOperand op = gemm_fp4_split_operand(w + a.vc, w + a.vs, kvc * d, L, true, w + a.pv, chunk_max * d + 128);
+            rc = gemm_fp4_prepare_operands(&op, 1, L, 32, st);
+        }
         if (rc != AMX_OK) return rc;
         for (int64_t i = 0; i < hc;) {
             float* oh = o + (size_t)(h0 + i) * L * d;
@@ -746,8 +737,9 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     // sequence), then the two passes
     int* words = reinterpret_cast<int*>(w + a.gemm);
     if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
-    int rc = gemm_fp4_quantize_prepared(q, L, d, false, nullptr, w + a.qs, w + a.pq, st);
-    if (rc == AMX_OK) rc = gemm_fp4_quantize_prepared(k, L, d, true, nullptr, w + a.ks, w + a.pk, st);
+    const PrepOperand op[2] = {gemm_fp4_cast_operand(q, d, L, d, false, nullptr, w + a.qs, w + a.pq),
+                               gemm_fp4_cast_operand(k, d, L, d, true, nullptr, w + a.ks, w + a.pk)};
+    int rc = gemm_fp4_prepare_operands(op, 2, d, 32, st);
     if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(v, 1, L, d, 128, 128, w + a.vs, w + a.pv, st, nullptr);
     if (rc != AMX_OK) return rc;
     return attn_fused({w + a.pq, L, L, 0}, {w + a.pk, L, L, 0}, {w + a.pv, 128, 128, 0}, 1, L, d, 1.0f / sqrtf((float)d), causal,

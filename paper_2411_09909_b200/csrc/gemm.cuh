@@ -5,9 +5,14 @@
 
 namespace amx {
 
-int gemm_simt(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes,
-              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C,
-              int64_t ld_c, cudaStream_t st, const int* run_if_nonzero = nullptr /* device word: nothing is done when zero */);
+// Codes of an operand as one plane or as two sign planes whose nibbles are or-ed (a prepared operand keeps no other copy).
+struct CodePlanes {
+    const uint8_t* a;
+    const uint8_t* b = nullptr;
+};
+int gemm_simt(CodePlanes a_codes, const uint8_t* a_scales, CodePlanes w_codes, const uint8_t* w_scales, int64_t M, int64_t N,
+              int64_t K, int gs, float* C, int64_t ld_c, cudaStream_t st,
+              const int* run_if_nonzero = nullptr /* device word: nothing is done when zero */);
 
 // The same kernel on operands with binary16 shared scales ([rows, K/gs, 2] uint16).
 int gemm_simt_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8_t* w_codes,
@@ -19,7 +24,7 @@ bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, int gs);
 size_t gemm_tc_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // run_if_nonzero (optional, device word): the launch does nothing when that word is zero.  status_word
 // (optional): a status word the caller has cleared, used instead of the workspace's first word.
-int gemm_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes,
+int gemm_tc(CodePlanes a_codes, const uint8_t* a_scales, CodePlanes w_codes,
             const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c,
             void* workspace, cudaStream_t st, const int* run_if_nonzero = nullptr, int* status_word = nullptr);
 // The same product with the cast of the bf16 activation X [M, ld_a] done inside the kernel.
@@ -48,23 +53,38 @@ int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_c
 // The same in two phases, so that an operand (typically the weight) is prepared once and reused.
 size_t gemm_fp4_prepared_bytes(int64_t rows, int64_t K, bool is_weight);
 size_t gemm_fp4_plane_bytes(int64_t rows, int64_t K);
+// One operand to prepare (quantize.cu): a bf16 matrix x to cast, or a canonical one (x == nullptr).
+struct PrepOperand {
+    const uint4* x;              // bf16 rows, ld_vec 16-byte pieces apart
+    int64_t ld_vec;
+    const uint4* in_codes;       // canonical operand
+    const uint16_t* in_scales;
+    int64_t R;                   // operand rows
+    int64_t seg_rows, seg_pad;   // seg_pad != 0: x holds segments of seg_rows rows, each padded to seg_pad operand rows with
+                                 // zero scale factors and row words
+    uint4* codes;                // out, of a cast: canonical codes (optional) and scales
+    uint16_t* scales;
+    uint4 *pos, *neg;            // out: planes, scale factors, row words
+    uint8_t *sf_pos, *sf_neg;
+    int* row_exp;
+    int64_t padded_rows;
+};
 // flushed_total (optional, device): incremented by the number of nonzero scales that fell below the UE4M3 range
 // of their row and were flushed; the per-row counts are in the row words either way.
-int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
-                     void* prepared, cudaStream_t st, int64_t layout_rows = 0 /* 0: rows */, int* flushed_total = nullptr, int gs = 32);
-int gemm_fp4_quantize_prepared(const void* x, int64_t rows, int64_t K, bool is_weight, uint8_t* codes,
-                               uint8_t* scales, void* prepared, cudaStream_t st, int64_t layout_rows = 0,
-                               int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr,
-                               int64_t seg_rows = 0, int64_t seg_pad = 0 /* not 0: x holds segments of seg_rows rows, each padded
-                               to seg_pad operand rows (`rows` counts operand rows) with zero scale factors and row words */);
+int prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, int nk64, cudaStream_t st, int format = AMX_FMT_AMXFP4,
+                     int* flushed_total = nullptr);
+// Descriptions of an operand laid out for layout_rows rows (0: rows) as the left-hand or right-hand one: a cast (ld in
+// elements), or the preparation of a canonical operand; and the launch for one or two of them.
+PrepOperand gemm_fp4_cast_operand(const void* x, int64_t ld, int64_t rows, int64_t K, bool is_weight, uint8_t* codes, uint8_t* scales,
+                                  void* prepared, int64_t layout_rows = 0, int64_t seg_rows = 0, int64_t seg_pad = 0);
+PrepOperand gemm_fp4_split_operand(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
+                                   void* prepared, int64_t layout_rows = 0);
+int gemm_fp4_prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, cudaStream_t st, int format = AMX_FMT_AMXFP4,
+                              int* flushed_total = nullptr);
 int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64_t d, int64_t seg_pad, int64_t layout_rows,
                                   uint8_t* scales, void* prepared, cudaStream_t st, int* flushed_total);
 int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int64_t seg_pad, void* pos, void* neg, uint8_t* scales,
                          cudaStream_t st);
-int quantize_rows_prepared(const void* x, int64_t rows, int64_t K, uint8_t* codes, uint8_t* scales, void* pos,
-                           void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows,
-                           cudaStream_t st, int format = AMX_FMT_AMXFP4, int* flushed_total = nullptr, int64_t seg_rows = 0,
-                           int64_t seg_pad = 0);
 const int* gemm_fp4_row_words(const void* prepared, int64_t rows, int64_t K, bool is_weight);
 // Softmax of the rows of S, rounded to bf16 and cast in one launch (cols % 32 == 0); pos == nullptr: canonical
 // output only.  gemm_fp4_softmax_prepared lays the prepared operand out like gemm_fp4_quantize_prepared.

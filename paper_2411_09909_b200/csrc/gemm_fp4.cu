@@ -108,108 +108,62 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
 __host__ __device__ constexpr uint32_t instr_desc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24); }
 
 // ------------------------------------------------------------------------- preparation --
-// One launch per operand; one block per kPrepRows operand rows (rows beyond R, up to the padded row count,
-// get zero scale factors so that padded tile rows multiply zero codes by a finite scale).
-//   1. row words: a warp per row finds the largest exponent key kmax among the row's scales (kmax - 25 is the
-//      power of two by which the row's UE4M3 scales understate the true ones) and which sides occur at all
-//   2. sign planes: every nibble goes to the plane of its sign bit, zero in the other plane
-//   3. scale factors of both planes in the layout the MMA reads:
-//      [plane][row block of 128][K/64 block][512 B], byte (r%32)*16 + (r/32)*4 + (k16 % 4);
-//      one scale per 16 elements, so a group's scale is written gs / 16 times (GS = 16: the MMA's own block)
-// PLANES = false: the sign planes are there already, steps 1 and 3 only.
+// Row words and scale factors of an operand (group size 32) whose sign planes are there already, from its canonical scales:
+// V^T of an attention call, whose cast writes the planes (quantize.cu; every other operand is prepared by the kernel
+// there).  A block has kPrepRows rows; a warp per row finds the largest exponent key kmax among the row's scales (kmax - 25 is
+// the power of two by which the row's UE4M3 scales understate the true ones) and which sides occur at all; then the
+// scale factors of both planes in the layout the MMA reads: [plane][row block of 128][K/64 block][512 B], byte
+// (r%32)*16 + (r/32)*4 + (k16 % 4), one scale per 16 elements, so a group's scale is written twice.  Operand rows come in
+// segments of seg_pad rows of which the first seg_rows are in use.
 constexpr int kPrepRows = 8;
-template <int GS, bool PLANES = true>
 __global__ void __launch_bounds__(256)
-prepare_operand_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales, int64_t R, int64_t K,
-                       int nk64, uint4* __restrict__ pos, uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos,
-                       uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total,
-                       int seg_rows = 0, int seg_pad = 0) {
+scale_factors_kernel(const uint8_t* __restrict__ scales, int64_t R, int64_t K, int nk64, uint8_t* __restrict__ sf_pos,
+                     uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total, int seg_rows, int seg_pad) {
     begin_kernel();
     __shared__ int kmax_s[kPrepRows];
-    __shared__ int unsplit_s[kPrepRows];
-    const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / GS;         // G: scale pairs per row
+    const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // seg_pad: operand rows come in segments of seg_pad rows of which the first seg_rows are in use
-    auto in_use = [&](int64_t row) { return row < R && (!seg_pad || (int)(row % seg_pad) < seg_rows); };
+    auto in_use = [&](int64_t row) { return row < R && (int)(row % seg_pad) < seg_rows; };
     for (int r = warp; r < kPrepRows; r += 8) {
         const int64_t row = row0 + r;
-        int kmax = 0, sides = 0;
-        uint32_t differ = 0;
-        if (in_use(row)) {
-            const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
+        int kmax = 0, sides = 0, flushed = 0;
+        const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
+        if (in_use(row))
             for (int64_t g = lane; g < G; g += 32) {
                 const uint32_t v = __ldg(s2 + g);
                 kmax = max(kmax, max(scale_key(v & 0xFF), scale_key(v >> 8)));
                 sides |= side_bits_of(v);
-                differ |= (v & 0xFF) ^ (v >> 8);
             }
-        }
         kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
         sides = __reduce_or_sync(0xFFFFFFFFu, sides);
-        differ = __reduce_or_sync(0xFFFFFFFFu, differ);
-        // A row whose two scales agree in every group (a symmetric format) needs no split: sum over both signs of
-        // code x scale_side = code x scale.  Its signed codes go to the positive plane as they are.
-        // (Planes that are there already were split, whatever the scales.)
-        const bool unsplit = PLANES && !differ;
-        if (unsplit) sides &= kRowHasPos;
-        // nonzero scales that the row's offset pushes below the UE4M3 range (they are flushed in step 3)
-        int flushed = 0;
-        if (in_use(row)) {
-            const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
+        if (in_use(row))                                         // scales below the row's UE4M3 range: flushed
             for (int64_t g = lane; g < G; g += 32) {
                 const uint32_t v = __ldg(s2 + g);
-                flushed += (int)ue4m3_flushes(v & 0xFF, kmax) + (int)(!unsplit && ue4m3_flushes(v >> 8, kmax));
+                flushed += (int)ue4m3_flushes(v & 0xFF, kmax) + (int)ue4m3_flushes(v >> 8, kmax);
             }
-        }
         flushed = __reduce_add_sync(0xFFFFFFFFu, flushed);
         if (lane == 0) {
             kmax_s[r] = kmax;
-            unsplit_s[r] = unsplit;
             if (in_use(row)) row_exp[row] = row_word(kmax, sides, flushed);
             if (flushed && flushed_total) atomicAdd(flushed_total, flushed);
-        }
-    }
-    // sign planes of this block's rows (contiguous in memory: rows are K/2 bytes apart)
-    __syncthreads();                                             // unsplit_s is complete
-    const int64_t rows_here = min((int64_t)kPrepRows, R - row0);
-    const int vec_per_row = (int)(K / 32);
-    if (PLANES && rows_here > 0) {
-        const int64_t v0 = row0 * vec_per_row, n_vec = rows_here * vec_per_row;
-        const uint4* src = reinterpret_cast<const uint4*>(codes) + v0;
-        for (int64_t i = threadIdx.x; i < n_vec; i += 256) {
-            const uint4 w = __ldg(src + i);
-            const uint32_t v[4] = {w.x, w.y, w.z, w.w};
-            const uint32_t keep = unsplit_s[(int)i / vec_per_row] ? 0u : 0xFFFFFFFFu;   // i < 8 rows: 32-bit division
-            uint32_t p[4], n[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t m = ((v[j] >> 3) & 0x11111111u) * 15u & keep;   // 0xF on negative nibbles
-                n[j] = v[j] & m;
-                p[j] = v[j] & ~m;
-            }
-            pos[v0 + i] = make_uint4(p[0], p[1], p[2], p[3]);
-            neg[v0 + i] = make_uint4(n[0], n[1], n[2], n[3]);
         }
     }
     __syncthreads();
     // scale factors: item = (K/64 block c, row r); consecutive threads take consecutive rows
     const int64_t rb = row0 / 128;
     const int r_in_blk0 = (int)(row0 % 128);
-    constexpr int kPer = GS >= 64 ? 1 : 64 / GS;                 // scale pairs of a 64-element block
     for (int item = threadIdx.x; item < nk64 * kPrepRows; item += 256) {
         const int c = item / kPrepRows, r = item % kPrepRows;
         const int64_t row = row0 + r;
         uint32_t wp = 0, wn = 0;
         if (in_use(row)) {
-            const int kmax = kmax_s[r];
 #pragma unroll
-            for (int h = 0; h < kPer; ++h) {
-                const int64_t g = GS >= 64 ? (int64_t)c * 64 / GS : (int64_t)c * kPer + h;
+            for (int h = 0; h < 2; ++h) {                        // the two 32-groups of this 64-element block
+                const int64_t g = (int64_t)c * 2 + h;
                 if (g < G) {
                     const uint32_t v = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * G + g) * 2));
-                    const uint32_t rep = GS == 16 ? 1u : GS == 32 ? 0x0101u : 0x01010101u;      // copies of the byte
-                    wp |= to_ue4m3(v & 0xFF, kmax) * rep << (32 / kPer * h);
-                    wn |= (unsplit_s[r] ? 0u : to_ue4m3(v >> 8, kmax)) * rep << (32 / kPer * h);
+                    wp |= to_ue4m3(v & 0xFF, kmax_s[r]) * 0x0101u << (16 * h);
+                    wn |= to_ue4m3(v >> 8, kmax_s[r]) * 0x0101u << (16 * h);
                 }
             }
         }
@@ -679,16 +633,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------------- host --
-int prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, const OperandLayout& o,
-            uint8_t* base, cudaStream_t st, int* flushed_total = nullptr, int gs = 32) {
-    const int64_t padded_rows = o.row_blocks * 128;
-    auto* kernel = gs == 16 ? prepare_operand_kernel<16> : gs == 32 ? prepare_operand_kernel<32>
-                 : gs == 64 ? prepare_operand_kernel<64> : prepare_operand_kernel<128>;
-    return launch(kernel, (unsigned)(padded_rows / kPrepRows), 256, 0, st, codes, scales, rows, K, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
-        base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf),
-        flushed_total, 0, 0);
-}
-
 }  // namespace
 
 bool gemm_fp4_supported(int64_t M, int64_t N, int64_t K, int gs) {
@@ -833,15 +777,46 @@ size_t gemm_fp4_prepared_bytes(int64_t rows, int64_t K, bool is_weight) {
     return operand_layout(rows, K, is_weight ? BN : BM).total;
 }
 
-// Fused form: one launch of the cast kernel writes the canonical operand and the prepared one.
-int gemm_fp4_quantize_prepared(const void* x, int64_t rows, int64_t K, bool is_weight, uint8_t* codes, uint8_t* scales,
-                               void* prepared, cudaStream_t st, int64_t layout_rows, int format, int* flushed_total,
-                               int64_t seg_rows, int64_t seg_pad) {
+// Parts of a prepared operand, for the launch that fills them.
+namespace {
+PrepOperand describe(int64_t rows, int64_t K, bool is_weight, void* prepared, int64_t layout_rows) {
     const OperandLayout o = operand_layout(layout_rows ? layout_rows : rows, K, is_weight ? BN : BM);
     uint8_t* base = static_cast<uint8_t*>(prepared);
-    return quantize_rows_prepared(x, rows, K, codes, scales, base, base + o.plane, base + 2 * o.plane,
-                                  base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), o.nk64,
-                                  seg_pad ? (rows + 127) / 128 * 128 : o.row_blocks * 128, st, format, flushed_total, seg_rows, seg_pad);
+    PrepOperand p{};
+    p.R = rows;
+    p.pos = reinterpret_cast<uint4*>(base);
+    p.neg = reinterpret_cast<uint4*>(base + o.plane);
+    p.sf_pos = base + 2 * o.plane;
+    p.sf_neg = p.sf_pos + o.sf;
+    p.row_exp = reinterpret_cast<int*>(p.sf_neg + o.sf);
+    p.padded_rows = o.row_blocks * 128;
+    return p;
+}
+}  // namespace
+
+PrepOperand gemm_fp4_cast_operand(const void* x, int64_t ld, int64_t rows, int64_t K, bool is_weight, uint8_t* codes, uint8_t* scales,
+                                  void* prepared, int64_t layout_rows, int64_t seg_rows, int64_t seg_pad) {
+    PrepOperand p = describe(rows, K, is_weight, prepared, layout_rows);
+    p.x = static_cast<const uint4*>(x);
+    p.ld_vec = ld / 8;
+    p.codes = reinterpret_cast<uint4*>(codes);
+    p.scales = reinterpret_cast<uint16_t*>(scales);
+    p.seg_rows = seg_rows;
+    p.seg_pad = seg_pad;
+    if (seg_pad) p.padded_rows = (rows + 127) / 128 * 128;
+    return p;
+}
+
+PrepOperand gemm_fp4_split_operand(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
+                                   void* prepared, int64_t layout_rows) {
+    PrepOperand p = describe(rows, K, is_weight, prepared, layout_rows);
+    p.in_codes = reinterpret_cast<const uint4*>(codes);
+    p.in_scales = reinterpret_cast<const uint16_t*>(scales);
+    return p;
+}
+
+int gemm_fp4_prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, cudaStream_t st, int format, int* flushed_total) {
+    return prepare_operands(op, n, K, gs, operand_layout(128, K, BM).nk64, st, format, flushed_total);
 }
 
 // V^T of `heads` heads [L, d], seg_pad operand rows each: cast down the rows into the planes and scales, then row words and
@@ -852,8 +827,9 @@ int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64
     uint8_t* base = static_cast<uint8_t*>(prepared);
     const int rc = quantize_cols_planes(v, heads, L, d, seg_pad, base, base + o.plane, scales, st);
     if (rc != AMX_OK) return rc;
-    return launch(prepare_operand_kernel<32, false>, (unsigned)(heads * seg_pad / kPrepRows), 256, 0, st, nullptr, scales, heads * seg_pad, L, o.nk64, nullptr, nullptr, base + 2 * o.plane, base + 2 * o.plane + o.sf,
-        reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), flushed_total, (int)d, (int)seg_pad);
+    return launch(scale_factors_kernel, (unsigned)(heads * seg_pad / kPrepRows), 256, 0, st, scales, heads * seg_pad, L, o.nk64,
+                  base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), flushed_total,
+                  (int)d, (int)seg_pad);
 }
 
 // Bytes from the first to the second sign plane of a prepared operand.
@@ -874,26 +850,20 @@ int gemm_fp4_softmax_prepared(const float* S, int64_t rows, int64_t cols, int64_
                              o.row_blocks * 128, st, causal);
 }
 
-int gemm_fp4_prepare(const uint8_t* codes, const uint8_t* scales, int64_t rows, int64_t K, bool is_weight,
-                     void* prepared, cudaStream_t st, int64_t layout_rows, int* flushed_total, int gs) {
-    return prepare(codes, scales, rows, K, operand_layout(layout_rows ? layout_rows : rows, K, is_weight ? BN : BM),
-                   static_cast<uint8_t*>(prepared), st, flushed_total, gs);
-}
-
 // Workspace: word 0 the status, word 1 the number of scales flushed while preparing the two operands (see
 // to_ue4m3), then the prepared operands.  gate_on_flushed: the GEMM kernel returns at once when that count is
 // not zero (the caller follows with the exact kernel, gated the other way).
 int gemm_fp4(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
              int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st,
              bool gate_on_flushed, int gs) {
-    const OperandLayout oa = operand_layout(M, K, BM), ow = operand_layout(N, K, BN);
+    const OperandLayout oa = operand_layout(M, K, BM);
     uint8_t* base = static_cast<uint8_t*>(workspace);
     uint8_t* pa = base + 256;
     uint8_t* pw = pa + oa.total;
     int* flushed = reinterpret_cast<int*>(base) + 1;
     if (clear_words(base, st) != AMX_OK) return AMX_ERR_CUDA;
-    int rc = prepare(a_codes, a_scales, M, K, oa, pa, st, flushed, gs);
-    if (rc == AMX_OK) rc = prepare(w_codes, w_scales, N, K, ow, pw, st, flushed, gs);
+    const PrepOperand op[2] = {gemm_fp4_split_operand(a_codes, a_scales, M, K, false, pa), gemm_fp4_split_operand(w_codes, w_scales, N, K, true, pw)};
+    const int rc = gemm_fp4_prepare_operands(op, 2, K, gs, st, AMX_FMT_AMXFP4, flushed);
     if (rc != AMX_OK) return rc;
     return gemm_fp4_prepared(pa, pw, M, N, K, C, ld_c, base, st, 256, gate_on_flushed ? flushed : nullptr);
 }

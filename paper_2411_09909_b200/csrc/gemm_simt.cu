@@ -19,14 +19,15 @@ __device__ __forceinline__ float scale_value(uint16_t h) { return __half2float(_
 
 // Decodes 8 codes of one row (one 32-bit word) into column `r` of a [BK][B + PAD] tile.
 template <typename ScaleT>
-__device__ __forceinline__ void decode_word(const uint8_t* __restrict__ codes,
+__device__ __forceinline__ void decode_word(const CodePlanes& codes,
                                             const ScaleT* __restrict__ scales, int64_t row,
                                             int64_t rows, int64_t K, int gs, int64_t k,
                                             float (*tile)[BM + PAD], int r, int kk) {
     uint32_t nib = 0;
     float sp = 0.f, sn = 0.f;
     if (row < rows && k < K) {
-        nib = *reinterpret_cast<const uint32_t*>(codes + row * (K / 2) + k / 2);
+        nib = *reinterpret_cast<const uint32_t*>(codes.a + row * (K / 2) + k / 2);
+        if (codes.b) nib |= *reinterpret_cast<const uint32_t*>(codes.b + row * (K / 2) + k / 2);
         const ScaleT* sc = scales + (row * (K / gs) + k / gs) * 2;
         sp = scale_value(sc[0]);
         sn = scale_value(sc[1]);
@@ -41,8 +42,8 @@ __device__ __forceinline__ void decode_word(const uint8_t* __restrict__ codes,
 
 template <typename ScaleT>
 __global__ void __launch_bounds__(256)
-gemm_simt_kernel(const uint8_t* __restrict__ a_codes, const ScaleT* __restrict__ a_scales,
-                 const uint8_t* __restrict__ w_codes, const ScaleT* __restrict__ w_scales,
+gemm_simt_kernel(const CodePlanes a_codes, const ScaleT* __restrict__ a_scales,
+                 const CodePlanes w_codes, const ScaleT* __restrict__ w_scales,
                  int64_t M, int64_t N, int64_t K, int gs, float* __restrict__ C, int64_t ld_c,
                  const int* __restrict__ run_if_nonzero) {
     begin_kernel();
@@ -83,7 +84,7 @@ gemm_simt_kernel(const uint8_t* __restrict__ a_codes, const ScaleT* __restrict__
 
 }  // namespace
 
-int gemm_simt(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes,
+int gemm_simt(CodePlanes a_codes, const uint8_t* a_scales, CodePlanes w_codes,
               const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C,
               int64_t ld_c, cudaStream_t st, const int* run_if_nonzero) {
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
@@ -96,7 +97,7 @@ int gemm_simt_f16s(const uint8_t* a_codes, const uint16_t* a_scales, const uint8
                    int64_t ld_c, cudaStream_t st) {
     dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
     if (grid.y > 65535) return AMX_ERR_SHAPE;
-    return launch(gemm_simt_kernel<uint16_t>, grid, 256, 0, st, a_codes, a_scales, w_codes, w_scales, M, N, K, gs, C, ld_c, nullptr);
+    return launch(gemm_simt_kernel<uint16_t>, grid, 256, 0, st, CodePlanes{a_codes}, a_scales, CodePlanes{w_codes}, w_scales, M, N, K, gs, C, ld_c, nullptr);
 }
 
 }  // namespace amx

@@ -62,13 +62,17 @@ struct Task {      // one 32-element group of one tile row
 };
 constexpr int kTasksPerThread = (BM + BN) * 2 / (kProducerWarps * 32);   // 3
 
-__device__ __forceinline__ Task load_task(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
+__device__ __forceinline__ Task load_task(const CodePlanes& codes, const uint8_t* __restrict__ scales,
                                           int64_t row, int64_t rows, int64_t K, int64_t k) {
     Task t;
     t.codes = make_uint4(0, 0, 0, 0);
     t.scales = 0;
     if (row < rows && k < K) {
-        t.codes = __ldg(reinterpret_cast<const uint4*>(codes + row * (K / 2) + k / 2));
+        t.codes = __ldg(reinterpret_cast<const uint4*>(codes.a + row * (K / 2) + k / 2));
+        if (codes.b) {                         // two sign planes
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(codes.b + row * (K / 2) + k / 2));
+            t.codes.x |= q.x; t.codes.y |= q.y; t.codes.z |= q.z; t.codes.w |= q.w;
+        }
         t.scales = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * (K / 32) + k / 32) * 2));
     }
     return t;
@@ -112,33 +116,23 @@ __device__ __forceinline__ Task cast_task(const RawGroup& g) {
 // from global memory and its codes never exist there (a_codes / a_scales are unused).
 template <bool CAST_A>
 __global__ void __launch_bounds__(kThreads, 2)
-gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ a_scales,
+gemm_tc_kernel(CodePlanes a_codes, const uint8_t* __restrict__ a_scales,
                const uint16_t* __restrict__ a_x, int64_t ld_a,
-               const uint8_t* __restrict__ w_codes, const uint8_t* __restrict__ w_scales,
-               int64_t M, int64_t N, int64_t K, float* __restrict__ C, int64_t ld_c, int vec_store,
+               CodePlanes w_codes, const uint8_t* __restrict__ w_scales,
+               int64_t M, int64_t N, int64_t K, float* __restrict__ C0, int64_t ld_c, int vec_store,
                int* __restrict__ status, int kb_per_slice, int64_t slice_stride, const int* __restrict__ run_if_nonzero,
-               int slices, int first, int group, int causal) {
+               int slices, int first, int group, int causal, int64_t items) {
     begin_kernel();
     if (run_if_nonzero && *run_if_nonzero == 0) return;          // uniform over the grid: nothing was set up yet
-    if (causal && (int64_t)blockIdx.x * BN > (int64_t)blockIdx.y * BM + BM - 1) return;   // a tile above the diagonal
-    // blockIdx.z: product of a batch (left operands and results one after another, `group` products share a right
-    // operand), then slice of the K range (kb_per_slice K blocks each); slice z of a product writes its partial product
-    // to C + z * slice_stride (one slice: the result itself)
-    const int batch = (int)blockIdx.z / slices, slice = (int)blockIdx.z - batch * slices;
-    a_codes += batch * (M * (K / 2));
-    a_scales += batch * (M * (K / 32) * 2);
-    w_codes += (first + batch) / group * (N * (K / 2));
-    w_scales += (first + batch) / group * (N * (K / 32) * 2);
-    C += batch * (int64_t)slices * M * N;                        // (a batch: ld_c == N)
+    // grid x: work items (tile of C, product of a batch, slice of the K range), or fewer blocks that walk over them (a gated
+    // launch, whose blocks almost always return above).  Products of a batch: left operands and results one after
+    // another, `group` products share a right operand.  Slice z of a product (kb_per_slice K blocks) writes its
+    // partial product to C + z * slice_stride (one slice: the result itself).
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     Control* ctl = reinterpret_cast<Control*>(tiles + kStages * kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-    const int kb_begin = slice * kb_per_slice;
-    const int num_kb = min((int)((K + BK - 1) / BK) - kb_begin, kb_per_slice);   // K blocks of this slice
-    C += (int64_t)slice * slice_stride;
-
+    const int n_tiles = (int)((N + BN - 1) / BN), m_tiles = (int)((M + BM - 1) / BM);
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->full[s], kProducerWarps);
@@ -148,7 +142,20 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    int kb0 = 0, n_done = 0;                                     // K blocks and items of this block so far: the barriers' phases
     if (warp == kProducerWarps) tmem_alloc(&ctl->tmem_base, kTmemCols);
+    for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int tile = (int)(item % (n_tiles * m_tiles)), z = (int)(item / (n_tiles * m_tiles));
+    const int batch = z / slices, slice = z - batch * slices;
+    const int64_t m0 = (int64_t)(tile / n_tiles) * BM, n0 = (int64_t)(tile % n_tiles) * BN;
+    if (causal && n0 > m0 + BM - 1) continue;                    // a tile above the diagonal
+    const int64_t a_off = batch * (M * (K / 2)), w_off = (first + batch) / group * (N * (K / 2));
+    const CodePlanes ac{a_codes.a + a_off, a_codes.b}, wc{w_codes.a + w_off, w_codes.b};      // (a batch has whole codes)
+    const uint8_t* as = a_scales + a_off / 8;                    // K / 32 pairs of bytes per row
+    const uint8_t* ws = w_scales + w_off / 8;
+    const int kb_begin = slice * kb_per_slice;
+    const int num_kb = min((int)((K + BK - 1) / BK) - kb_begin, kb_per_slice);   // K blocks of this slice
+    float* const C = C0 + batch * (int64_t)slices * M * N + (int64_t)slice * slice_stride;       // (a batch: ld_c == N)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -163,18 +170,18 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
         auto load_all = [&](Task (&t)[kTasksPerThread], int kb) {
             const int64_t k = (int64_t)(kb_begin + kb) * BK + half * 32;
             if (CAST_A) raw = load_raw(a_x, ld_a, m0 + r, M, K, k);
-            else t[0] = load_task(a_codes, a_scales, m0 + r, M, K, k);
+            else t[0] = load_task(ac, as, m0 + r, M, K, k);
 #pragma unroll
             for (int i = 1; i < kTasksPerThread; ++i)
-                t[i] = load_task(w_codes, w_scales, n0 + r + 128 * (i - 1), N, K, k);
+                t[i] = load_task(wc, ws, n0 + r + 128 * (i - 1), N, K, k);
         };
         load_all(cur, 0);
         if (CAST_A) cur[0] = cast_task(raw);
         bool ok = true;
         for (int kb = 0; kb < num_kb && ok; ++kb) {
-            const int s = kb % kStages;
+            const int it = kb0 + kb, s = it % kStages;
             if (kb + 1 < num_kb) load_all(nxt, kb + 1);
-            if (kb >= kStages) ok = mbar_wait(&ctl->empty[s], ((kb / kStages) - 1) & 1, &ctl->abort, status);
+            if (it >= kStages) ok = mbar_wait(&ctl->empty[s], ((it / kStages) - 1) & 1, &ctl->abort, status);
             if (!ok) break;
             uint8_t* stage = tiles + s * kStageBytes;
 #pragma unroll
@@ -207,7 +214,7 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
             if (CAST_A && kb + 1 < num_kb) cur[0] = cast_task(raw);
         }
         // ------------------------------------------------------------------ epilogue
-        if (ok) ok = mbar_wait(&ctl->accum, 0, &ctl->abort, status);
+        if (ok) ok = mbar_wait(&ctl->accum, n_done & 1, &ctl->abort, status);
         tc_fence_after();
         if (ok) {
             const int q = warp & 3, h = warp >> 2;                 // lane quarter, column half
@@ -237,8 +244,8 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
         // ------------------------------------------------------------------ MMA issuer
         bool ok = true;
         for (int kb = 0; kb < num_kb && ok; ++kb) {
-            const int s = kb % kStages;
-            ok = mbar_wait(&ctl->full[s], (kb / kStages) & 1, &ctl->abort, status);
+            const int it = kb0 + kb, s = it % kStages;
+            ok = mbar_wait(&ctl->full[s], (it / kStages) & 1, &ctl->abort, status);
             if (!ok) break;
             tc_fence_after();
             const uint32_t a_addr = smem_u32(tiles + s * kStageBytes), b_addr = a_addr + kTileA;
@@ -252,9 +259,14 @@ gemm_tc_kernel(const uint8_t* __restrict__ a_codes, const uint8_t* __restrict__ 
     }
     tc_fence_before();
     __syncthreads();
+    if (ctl->abort) break;                                       // uniform: written before the barrier
+    kb0 += num_kb;
+    ++n_done;
+    }
+    __syncthreads();
     if (warp == kProducerWarps) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        tmem_dealloc(ctl->tmem_base, kTmemCols);
     }
 }
 
@@ -322,8 +334,8 @@ int configure_tc() {
     return AMX_OK;
 }
 
-int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a_x, int64_t ld_a,
-              const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C,
+int launch_tc(CodePlanes a_codes, const uint8_t* a_scales, const uint16_t* a_x, int64_t ld_a,
+              CodePlanes w_codes, const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, float* C,
               int64_t ld_c, void* workspace, cudaStream_t st, const int* gate = nullptr, int* status_word = nullptr) {
     if (const int rc = configure_tc(); rc != AMX_OK) return rc;
     // status word: the first word of the workspace, cleared here, unless the caller shares one it cleared itself
@@ -331,18 +343,20 @@ int launch_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint16_t* a
     if (!status_word && clear_words(status, st) != AMX_OK) return AMX_ERR_CUDA;   // + flushed count: none
     int kb_per;
     const int slices = k_slices(M, N, K, kb_per);
-    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM), (unsigned)slices);
+    const int64_t items = ((N + BN - 1) / BN) * ((M + BM - 1) / BM) * slices;
+    if (items > 0x7FFFFFFF) return AMX_ERR_SHAPE;
+    const dim3 grid((unsigned)(gate && items > kSmCount ? kSmCount : items));
     float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
     float* out = slices > 1 ? part : C;
     const int64_t ld_out = slices > 1 ? N : ld_c, slice_stride = slices > 1 ? M * N : 0;
     const int vec_store = aligned(out, 16) && ld_out % 4 == 0;   // else the epilogue stores scalars
     int rc;
     if (a_x)
-        rc = launch(gemm_tc_kernel<true>, grid, kThreads, kSmemBytes, st, nullptr, nullptr, a_x, ld_a, w_codes, w_scales, M, N, K, out,
-                                                                 ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
+        rc = launch(gemm_tc_kernel<true>, grid, kThreads, kSmemBytes, st, a_codes, nullptr, a_x, ld_a, w_codes, w_scales, M, N, K, out,
+                                                                 ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0, items);
     else
         rc = launch(gemm_tc_kernel<false>, grid, kThreads, kSmemBytes, st, a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K,
-                                                                  out, ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0);
+                                                                  out, ld_out, vec_store, status, kb_per, slice_stride, gate, slices, 0, 1, 0, items);
     if (rc != AMX_OK || slices == 1) return rc;
     return reduce_slices(part, slices, M, N, C, ld_c, st, gate);
 }
@@ -356,7 +370,7 @@ int reduce_slices(const float* part, int slices, int64_t M, int64_t N, float* C,
 
 // run_if_nonzero: the launches do nothing when that device word is zero.  status_word: where a timeout is
 // recorded instead of the workspace's first word (the caller has cleared it).
-int gemm_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
+int gemm_tc(CodePlanes a_codes, const uint8_t* a_scales, CodePlanes w_codes, const uint8_t* w_scales,
             int64_t M, int64_t N, int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st,
             const int* run_if_nonzero, int* status_word) {
     return launch_tc(a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, C, ld_c, workspace, st, run_if_nonzero,
@@ -367,7 +381,7 @@ int gemm_tc(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_co
 // ld_a % 8 == 0.
 int gemm_tc_cast(const void* x, int64_t ld_a, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N,
                  int64_t K, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
-    return launch_tc(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_a, w_codes, w_scales, M, N, K, C, ld_c,
+    return launch_tc({nullptr}, nullptr, static_cast<const uint16_t*>(x), ld_a, {w_codes}, w_scales, M, N, K, C, ld_c,
                      workspace, st);
 }
 
@@ -387,13 +401,14 @@ int gemm_tc_batched(const uint8_t* a_codes, const uint8_t* a_scales, const uint8
     if (clear_words(status, st) != AMX_OK) return AMX_ERR_CUDA;
     int kb_per;
     const int slices = k_slices(M, N, K, kb_per);
-    if (batch * slices > 65535) return AMX_ERR_SHAPE;
-    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM), (unsigned)(batch * slices));
+    const int64_t items = ((N + BN - 1) / BN) * ((M + BM - 1) / BM) * batch * slices;
+    if (items > 0x7FFFFFFF) return AMX_ERR_SHAPE;
+    const dim3 grid((unsigned)items);
     float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
     float* out = slices > 1 ? part : C;
-    rc = launch(gemm_tc_kernel<false>, grid, kThreads, kSmemBytes, st, a_codes, a_scales, nullptr, 0, w_codes, w_scales, M, N, K, out, N,
+    rc = launch(gemm_tc_kernel<false>, grid, kThreads, kSmemBytes, st, CodePlanes{a_codes}, a_scales, nullptr, 0, CodePlanes{w_codes}, w_scales, M, N, K, out, N,
                                                               aligned(out, 16) && N % 4 == 0 && (M * N) % 4 == 0, status, kb_per, M * N,
-                                                              nullptr, slices, (int)first, (int)group, causal);
+                                                              nullptr, slices, (int)first, (int)group, causal, items);
     if (rc != AMX_OK || slices == 1) return rc;
     return launch(reduce_slices_kernel, dim3((unsigned)((M * N + 255) / 256), (unsigned)batch), 256, 0, st, part, slices, M, N, C, N, nullptr);
 }

@@ -5,6 +5,7 @@
 
 #include "cast_math.cuh"
 #include "cp_async.cuh"
+#include "gemm.cuh"
 #include "softmax_math.cuh"
 
 namespace amx {
@@ -177,7 +178,7 @@ quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t R, int64_t C, 
 // the 512-byte chunk of [128 rows x 64 elements]; one scale per 16 elements, so a 32-group's scale is stored
 // twice - and per row the power of two by which those scale factors understate the true scales
 // (row_exp = largest exponent key of the row - 25).  The scale factors depend on the row's largest scale, so
-// whole rows belong to one warp (cast_prepared_kernel) or, in the softmax variant, to one block
+// whole rows belong to one warp (prepare_operands_kernel) or, in the softmax variant, to one block
 // (finish_prepared_row).  Rows past the last row, and groups past the last group, get zero scale factors, so that
 // padded tile rows and columns multiply zero codes by a finite scale.
 
@@ -232,128 +233,279 @@ __device__ __forceinline__ void finish_prepared_row(int64_t row, bool row_live, 
     }
 }
 
-// The cast for an operand of the FP4 GEMM.  A row (or, when rows are short, several rows) belongs to one warp:
-// LPR = 2^lpr_log2 lanes per row, lane lr of them owns the groups lr, lr + LPR, ...  A lane streams its groups
-// through a private ring in shared memory with asynchronous copies (kCastDepth groups ahead; the loads hold no
-// registers).  First sweep: per group the cast, the stores of the planes, the scale bytes and (when asked for)
-// the canonical codes; the scale bytes stay in registers (GPL of them per lane; GPL = 0: any number, re-read from
-// the scales just stored).  Then the row's largest exponent key by a warp reduction, and the second sweep turns
-// the scale bytes into the row's scale factors, padding included, and writes the row word.
+// Operands of the FP4 GEMM, up to two of them in one launch (a small cast beside the preparation of a large weight, or
+// both casts of a layer).  Per operand either the cast of a bf16 matrix (any fixed group size) or the preparation of a
+// canonical one.  A row (or, when rows are short, several rows) belongs to one warp: LPR = 2^lpr_log2 lanes per row, lane lr
+// of them owns the 32-element pieces lr, lr + LPR, ...  A lane streams its pieces through a private ring in shared memory
+// with asynchronous copies (kCastDepth pieces ahead; the loads hold no registers).  First sweep: per piece the cast (or the
+// split of its codes), the stores of the planes, the scale bytes and (when asked for) the canonical codes; the scale bytes
+// stay in registers (GPL of them per lane; GPL = 0: any number, re-read from memory).  Then the row's largest exponent key
+// by a warp reduction, and the second sweep turns the scale bytes into the row's scale factors, padding included, and
+// writes the row word.
 // Scale factors leave the block in whole 32-byte sectors: the tensor cores' layout interleaves eight rows (r, r+1,
 // r+32, r+33, r+64, r+65, r+96, r+97, r even) in every sector, so a block of eight warps owns exactly such sets of
 // rows - warp (q, h) has the rows 32 q + 2 k + h of a 128-row block, for the block's RPW = 32 / LPR values of k -
 // collects the converted bytes in shared memory and stores them 16 bytes per thread.  (Written 2 bytes at a
 // time straight from the owning lanes, the scale factors were 4 % of the bytes and doubled the kernel's L2
 // write requests.)  Rows past the last row get zero scale factors.
-constexpr int kCastDepth = 2;                              // groups in flight per lane
+constexpr int kCastDepth = 2;                              // pieces in flight per lane
 constexpr int kCastWarps = 8;
 constexpr int kCastRingBytes = kCastWarps * kCastDepth * 32 * 64;
 constexpr int kCastMaxExchangeBytes = 96 * 1024;           // above this (K > 49152 at LPR = 32) the lanes store their bytes themselves
 
-template <int FMT, int GPL>
-__global__ void __launch_bounds__(kCastWarps * 32)
-cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_rows, int64_t seg_pad, int G, int lpr_log2, int exchange,
-                     uint4* __restrict__ codes, uint16_t* __restrict__ scales, uint4* __restrict__ pos,
-                     uint4* __restrict__ neg, uint8_t* __restrict__ sf_pos, uint8_t* __restrict__ sf_neg,
-                     int* __restrict__ row_exp, int nk64, int* __restrict__ flushed_total) {
+struct PrepParams {
+    PrepOperand op[2];
+    unsigned blocks0;                                      // blocks of the first operand; the others are the second's
+    int G, lpr_log2, exchange, nk64, gs;
+    int* flushed_total;
+};
+
+// Scale pairs {neg : pos} of one 32-element piece: of its first 16 elements in bits 15..0, of the others in bits 31..16
+// (equal unless the group size is 16), from a row's canonical scales.
+__device__ __forceinline__ uint32_t piece_scales(const uint16_t* __restrict__ row, int g, int gs) {
+    if (gs == 16) return (uint32_t)row[2 * g] | ((uint32_t)row[2 * g + 1] << 16);
+    const uint32_t v = row[gs == 32 ? g : gs == 64 ? g >> 1 : g >> 2];
+    return v | (v << 16);
+}
+
+// A piece of a group of 16, 64 or 128 elements (AMXFP4): 64- and 128-groups are two or four consecutive lanes, which agree
+// on the maxima.  Every lane of the warp takes part; `own`: the lane has a piece, number g of the row.
+__device__ __forceinline__ uint32_t cast_piece_gs(const uint32_t (&w)[16], bool own, int gs, int64_t v, int g, uint16_t* __restrict__ row_scales,
+                                                  uint4* __restrict__ codes, uint4* __restrict__ pos, uint4* __restrict__ neg) {
+    uint32_t half[2], sc[2];
+    uint64_t ip2[2], in2[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t wh[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) wh[i] = w[8 * h + i];
+        half[h] = side_maxima<8>(wh);
+    }
+    if (gs != 16) {
+        uint32_t c = __vmaxs2(half[0], half[1]);
+        if (gs >= 64) c = __vmaxs2(c, __shfl_xor_sync(0xFFFFFFFFu, c, 1));
+        if (gs == 128) c = __vmaxs2(c, __shfl_xor_sync(0xFFFFFFFFu, c, 2));
+        half[0] = half[1] = c;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float ip, in;
+        sc[h] = group_scales(half[h], ip, in);
+        ip2[h] = pack_f32x2(__float_as_uint(ip), __float_as_uint(ip));
+        in2[h] = pack_f32x2(__float_as_uint(in), __float_as_uint(in));
+    }
+    uint32_t nib[4], pp[4], nn[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t cp, cn;
+        encode8_both(w + 4 * j, ip2[j >> 1], in2[j >> 1], cp, cn);
+        const uint32_t m = negative_nibbles(cp);
+        pp[j] = cp & ~m;
+        nn[j] = cn & m;
+        nib[j] = pp[j] | nn[j];
+    }
+    if (!own) return 0;
+    if (codes) codes[v] = make_uint4(nib[0], nib[1], nib[2], nib[3]);
+    pos[v] = make_uint4(pp[0], pp[1], pp[2], pp[3]);
+    neg[v] = make_uint4(nn[0], nn[1], nn[2], nn[3]);
+    if (gs == 16) {
+        row_scales[2 * g] = (uint16_t)sc[0];
+        row_scales[2 * g + 1] = (uint16_t)sc[1];
+    } else if (gs == 64) {
+        if (!(g & 1)) row_scales[g >> 1] = (uint16_t)sc[0];
+    } else if (!(g & 3)) row_scales[g >> 2] = (uint16_t)sc[0];
+    return sc[0] | (sc[1] << 16);
+}
+
+// MODE: one cast, two casts, operands that may be canonical, or any of these with a group size other than 32.  (The plain
+// cast is kept lean - its pointers are compile-time places in constant memory: it is bound by instruction issue, and four
+// blocks have to share an SM.)
+enum PrepMode { kOneCast, kTwoCasts, kAnyKind, kAnyGroup };
+template <int FMT, int GPL, int MODE>
+__global__ void __launch_bounds__(kCastWarps * 32, 4)
+prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     begin_kernel();
     extern __shared__ __align__(16) uint8_t smem_raw[];
+    constexpr bool SPLIT = MODE >= kAnyKind, ANY_GS = MODE == kAnyGroup;
+    const bool second = MODE != kOneCast && blockIdx.x >= p.blocks0;
+    const PrepOperand& o = p.op[second];
+    const unsigned block = blockIdx.x - (second ? p.blocks0 : 0u);
+    const int G = p.G, lpr_log2 = p.lpr_log2, nk64 = p.nk64, gs = ANY_GS ? p.gs : 32;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, LPR = 1 << lpr_log2, lr = lane & (LPR - 1);
     const int RPW = 32 >> lpr_log2, sg = lane >> lpr_log2;      // rows per warp; which of them this lane works on
     // the block's rows: 128-row block rb, sector sets k0 .. k0 + RPW - 1 (16 / RPW blocks share a 128-row block)
-    const int64_t rb = (int64_t)blockIdx.x >> (lpr_log2 - 1);
-    const int k0 = ((int)blockIdx.x & ((16 >> (5 - lpr_log2)) - 1)) << (5 - lpr_log2);
+    const int64_t rb = (int64_t)block >> (lpr_log2 - 1);
+    const int k0 = ((int)block & ((16 >> (5 - lpr_log2)) - 1)) << (5 - lpr_log2);
     const int r_in = 32 * (wi >> 1) + 2 * (k0 + sg) + (wi & 1);  // row inside the 128-row block
     const int64_t row = rb * 128 + r_in;
     // Segments (the heads of an attention call): seg_rows source rows each, padded to seg_pad operand rows.
-    const int64_t seg = seg_pad ? row / seg_pad : 0;
-    const bool live = row < R && (!seg_pad || row - seg * seg_pad < seg_rows);
-    const int64_t src_row = seg_pad ? seg * seg_rows + (row - seg * seg_pad) : row;
+    const int64_t seg = o.seg_pad ? row / o.seg_pad : 0;
+    const bool live = row < o.R && (!o.seg_pad || row - seg * o.seg_pad < o.seg_rows);
+    const int64_t src_row = o.seg_pad ? seg * o.seg_rows + (row - seg * o.seg_pad) : row;
     const unsigned seg_mask = LPR == 32 ? 0xFFFFFFFFu : ((1u << LPR) - 1u) << (lane & ~(LPR - 1));
     const int64_t v_row = row * G;
-    // this lane's ring: kCastDepth slots of 64 bytes (one group).  Piece j of a group sits at 16-byte position
+    // this lane's ring: kCastDepth slots of 64 bytes (one piece).  Part j of a piece sits at 16-byte position
     // j ^ ((lane >> 1) & 3) of the slot, so that the lanes of a quarter warp read eight different bank groups.
     uint8_t* ring = smem_raw + ((wi * kCastDepth * 32) + lane) * 64;
     uint8_t* xchg = smem_raw + kCastRingBytes;        // [plane][chunk][sector set][h][q] words of 4 scale-factor bytes
     const int swz = (lane >> 1) & 3;
-    const int n_own = (live && lr < G) ? ((G - lr + LPR - 1) >> lpr_log2) : 0;   // groups this lane owns
-    auto issue = [&](int i) {                        // copies of the lane's i-th group, one commit group per call
+    const int n_own = (live && lr < G) ? ((G - lr + LPR - 1) >> lpr_log2) : 0;   // pieces this lane owns
+    const int n_max = (G + LPR - 1) >> lpr_log2;      // of any lane
+    uint16_t* const row_scales = o.scales + row * ((int64_t)G * 32 / gs);        // canonical scales: written by a cast, read otherwise
+    const uint16_t* const in_scales = !SPLIT || o.x ? row_scales : o.in_scales + row * ((int64_t)G * 32 / gs);
+    auto issue = [&](int i) {                        // copies of the lane's i-th piece, one commit group per call
         if (i < n_own) {
-            const uint4* src = x + (src_row * G + lr + ((int64_t)i << lpr_log2)) * 4;
+            const uint4* src = o.x + src_row * o.ld_vec + (lr + ((int64_t)i << lpr_log2)) * 4;
             uint8_t* slot = ring + (i % kCastDepth) * (32 * 64);
 #pragma unroll
             for (int j = 0; j < 4; ++j) cp_async16(slot + ((j ^ swz) << 4), src + j);
         }
         cp_async_commit();
     };
-    auto cast_group = [&](int i) -> uint32_t {       // the i-th group has landed: read it back, cast, store
+    auto cast_piece = [&](int i) -> uint32_t {       // the i-th piece has landed: read it back, cast, store
         const uint8_t* slot = ring + (i % kCastDepth) * (32 * 64);
+        const bool own = i < n_own;
+        if (gs == 32 && !own) return 0;
         uint32_t w[16];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint4 q = *reinterpret_cast<const uint4*>(slot + ((j ^ swz) << 4));
+            uint4 q = make_uint4(0, 0, 0, 0);
+            if (own) q = *reinterpret_cast<const uint4*>(slot + ((j ^ swz) << 4));
             w[4 * j] = q.x; w[4 * j + 1] = q.y; w[4 * j + 2] = q.z; w[4 * j + 3] = q.w;
         }
-        return emit_group<FMT>(w, v_row + lr + ((int64_t)i << lpr_log2), codes, scales, pos, neg);
+        const int g = lr + (i << lpr_log2);
+        if (ANY_GS && gs != 32) return cast_piece_gs(w, own, gs, v_row + g, g, row_scales, o.codes, o.pos, o.neg);
+        const uint32_t sc = emit_group<FMT>(w, v_row + g, o.codes, reinterpret_cast<uint16_t*>(o.scales), o.pos, o.neg);
+        return sc | (sc << 16);
     };
     uint32_t sc_reg[GPL > 0 ? GPL : 1];
-    uint32_t top = 0;                               // largest scale bytes seen by this lane, {neg : pos}
+    uint32_t top = 0;                               // largest scale bytes seen by this lane, {neg : pos} twice
+    if (!SPLIT || o.x) {
 #pragma unroll
-    for (int i = 0; i < kCastDepth - 1; ++i) issue(i);
-    if (GPL > 0) {
+        for (int i = 0; i < kCastDepth - 1; ++i) issue(i);
+        if (GPL > 0) {
 #pragma unroll
-        for (int i = 0; i < GPL; ++i) {
-            issue(i + kCastDepth - 1);
-            cp_async_wait<kCastDepth - 1>();
-            sc_reg[i] = i < n_own ? cast_group(i) : 0u;
-            top = __vmaxu4(top, sc_reg[i]);         // byte-wise maximum
+            for (int i = 0; i < GPL; ++i) {
+                issue(i + kCastDepth - 1);
+                cp_async_wait<kCastDepth - 1>();
+                sc_reg[i] = cast_piece(i);
+                top = __vmaxu4(top, sc_reg[i]);     // byte-wise maximum
+            }
+        } else {
+            for (int i = 0; i < n_max; ++i) {
+                issue(i + kCastDepth - 1);
+                cp_async_wait<kCastDepth - 1>();
+                top = __vmaxu4(top, cast_piece(i));
+            }
         }
+        cp_async_wait<0>();
     } else {
-        for (int i = 0; i < n_own; ++i) {
-            issue(i + kCastDepth - 1);
-            cp_async_wait<kCastDepth - 1>();
-            top = __vmaxu4(top, cast_group(i));
+        // canonical operand: the first codes are on their way while the scales are read - whether the row needs a split at
+        // all is known only from all of them
+        constexpr int kBatch = 4;                   // 16-byte loads in flight per lane
+        uint4 q[kBatch];
+        auto load_codes = [&](int i0) {
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i)
+                if (i0 + i < n_own) q[i] = __ldg(o.in_codes + v_row + lr + ((int64_t)(i0 + i) << lpr_log2));
+        };
+        load_codes(0);
+        uint32_t differ = 0;
+        if (GPL > 0) {
+#pragma unroll
+            for (int i = 0; i < GPL; ++i) {
+                sc_reg[i] = i < n_own ? piece_scales(in_scales, lr + (i << lpr_log2), gs) : 0u;
+                top = __vmaxu4(top, sc_reg[i]);
+                differ |= (sc_reg[i] ^ (sc_reg[i] >> 8)) & 0x00FF00FFu;
+            }
+        } else {
+            for (int i = 0; i < n_own; ++i) {
+                const uint32_t sc = piece_scales(in_scales, lr + (i << lpr_log2), gs);
+                top = __vmaxu4(top, sc);
+                differ |= (sc ^ (sc >> 8)) & 0x00FF00FFu;
+            }
         }
+        // A row whose two scales agree in every group (a symmetric format) needs no split: sum over both signs of
+        // code x scale_side = code x scale.  Its signed codes go to the positive plane as they are.
+        const bool unsplit = __reduce_or_sync(seg_mask, differ) == 0;
+        const uint32_t keep_sc = unsplit ? 0x00FF00FFu : 0xFFFFFFFFu, keep = unsplit ? 0u : 0xFFFFFFFFu;
+        top &= keep_sc;
+        if (GPL > 0) {
+#pragma unroll
+            for (int i = 0; i < GPL; ++i) sc_reg[i] &= keep_sc;
+        }
+        for (int i0 = 0; i0 < n_own; i0 += kBatch) {
+            if (i0) load_codes(i0);
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+                if (i0 + i >= n_own) break;
+                const uint32_t c[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+                uint32_t pp[4], nn[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t m = negative_nibbles(c[j]) & keep;
+                    nn[j] = c[j] & m;
+                    pp[j] = c[j] & ~m;
+                }
+                const int64_t v = v_row + lr + ((int64_t)(i0 + i) << lpr_log2);
+                o.pos[v] = make_uint4(pp[0], pp[1], pp[2], pp[3]);
+                o.neg[v] = make_uint4(nn[0], nn[1], nn[2], nn[3]);
+            }
+        }
+        if (GPL == 0) sc_reg[0] = keep_sc;          // for the second sweep
     }
-    cp_async_wait<0>();
     // The key of an E5M2 byte grows with the byte (scales carry no sign bit): the largest byte has the largest key.
+    top = __vmaxu4(top, top >> 16);
     const uint32_t top_p = __reduce_max_sync(seg_mask, top & 0xFFu), top_n = __reduce_max_sync(seg_mask, (top >> 8) & 0xFFu);
     const int kmax = scale_key(max(top_p, top_n));
     const int64_t sf_row = sf_row_offset(row, nk64);
     // word of the exchange buffer that holds this row's bytes of chunk c: ((c * RPW + sg) * 2 + h) * 4 + q
     const int x_row = (sg * 2 + (wi & 1)) * 4 + (wi >> 1), x_plane = nk64 * RPW * 8;   // in words
-    int flushed = 0;
-    auto put = [&](int g, uint32_t sc) {            // scale factors of group g (zero past the row's last group)
-        const uint32_t up = to_ue4m3(sc & 0xFFu, kmax), un = to_ue4m3(sc >> 8, kmax);
-        flushed += (int)((sc & 0xFFu) != 0 && up == 0) + (int)((sc >> 8) != 0 && un == 0);
-        if (exchange) {
+    int flushed = 0;                                // groups, not pieces, are counted
+    auto put = [&](int g, uint32_t sc) {            // scale factors of piece g (zero past the row's last one)
+        uint32_t up = to_ue4m3(sc & 0xFFu, kmax), un = to_ue4m3((sc >> 8) & 0xFFu, kmax);
+        const int lost = (int)((sc & 0xFFu) != 0 && up == 0) + (int)((sc & 0xFF00u) != 0 && un == 0);
+        if (gs <= 32 || (g & ((gs >> 5) - 1)) == 0) flushed += lost;
+        if (gs == 16) {                             // the second half has its own scales
+            const uint32_t sc1 = sc >> 16, up1 = to_ue4m3(sc1 & 0xFFu, kmax), un1 = to_ue4m3(sc1 >> 8, kmax);
+            flushed += (int)((sc1 & 0xFFu) != 0 && up1 == 0) + (int)((sc1 >> 8) != 0 && un1 == 0);
+            up |= up1 << 8;
+            un |= un1 << 8;
+        } else {
+            up |= up << 8;
+            un |= un << 8;
+        }
+        if (p.exchange) {
             uint16_t* w16 = reinterpret_cast<uint16_t*>(xchg) + (((g >> 1) * RPW * 8 + x_row) << 1) + (g & 1);
-            w16[0] = (uint16_t)(up | (up << 8));
-            w16[x_plane << 1] = (uint16_t)(un | (un << 8));
+            w16[0] = (uint16_t)up;
+            w16[x_plane << 1] = (uint16_t)un;
         } else {
             const int64_t off = sf_row + sf_group_offset(g);
-            *reinterpret_cast<uint16_t*>(sf_pos + off) = (uint16_t)(up | (up << 8));
-            *reinterpret_cast<uint16_t*>(sf_neg + off) = (uint16_t)(un | (un << 8));
+            *reinterpret_cast<uint16_t*>(o.sf_pos + off) = (uint16_t)up;
+            *reinterpret_cast<uint16_t*>(o.sf_neg + off) = (uint16_t)un;
         }
     };
-    const int g_end = nk64 * 2;                     // groups past G: padding to whole 256-element blocks
+    const int g_end = nk64 * 2;                     // pieces past G: padding to whole 256-element blocks
     if (GPL > 0) {
 #pragma unroll
         for (int i = 0; i < GPL; ++i) {
             const int g = lr + (i << lpr_log2);
-            if (g < g_end) put(g, sc_reg[i]);       // zero for a group past G and for a padding row
+            if (g < g_end) put(g, sc_reg[i]);       // zero for a piece past G and for a padding row
         }
         for (int g = lr + (GPL << lpr_log2); g < g_end; g += LPR) put(g, 0u);
     } else {
-        for (int g = lr; g < g_end; g += LPR) put(g, (live && g < G) ? (uint32_t)scales[v_row + g] : 0u);
+        // (a cast in a symmetric format wrote its one scale to both bytes; only the positive side's counts)
+        const uint32_t keep_sc = !SPLIT || o.x ? (FMT ? 0x00FF00FFu : 0xFFFFFFFFu) : sc_reg[0];
+        if (ANY_GS) __syncwarp();                   // scales of larger groups were written by neighbouring lanes
+        for (int g = lr; g < g_end; g += LPR) put(g, (live && g < G) ? piece_scales(in_scales, g, gs) & keep_sc : 0u);
     }
     flushed = __reduce_add_sync(seg_mask, flushed);
     if (lr == 0 && live) {
-        row_exp[row] = row_word(kmax, side_bits_of(top_p | (top_n << 8)), flushed);
-        if (flushed && flushed_total) atomicAdd(flushed_total, flushed);
+        o.row_exp[row] = row_word(kmax, side_bits_of(top_p | (top_n << 8)), flushed);
+        if (flushed && p.flushed_total) atomicAdd(p.flushed_total, flushed);
     }
-    if (lr == 0 && !live && row < R) row_exp[row] = 0;       // padding rows of a segment
-    if (!exchange) return;                          // uniform over the block
+    if (lr == 0 && !live && row < o.R) o.row_exp[row] = 0;       // padding rows of a segment
+    if (!p.exchange) return;                        // uniform over the block
     __syncthreads();
     // 16 bytes per thread: the words of rows q = 0..3 (32 rows apart) for one (plane, chunk, sector set, h);
     // two neighbouring threads (h = 0, 1) fill one sector
@@ -362,7 +514,7 @@ cast_prepared_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_rows, i
         const int plane = item >= per_plane, rest = item - plane * per_plane;
         const int c = rest / (RPW * 2), sh = rest - c * (RPW * 2);      // sh = sector set * 2 + h
         const uint4 v = reinterpret_cast<const uint4*>(xchg)[item];
-        uint8_t* dst = (plane ? sf_neg : sf_pos) + (rb * nk64 + c) * (int64_t)kSfChunkBytes + (2 * k0 + sh) * 16;
+        uint8_t* dst = (plane ? o.sf_neg : o.sf_pos) + (rb * nk64 + c) * (int64_t)kSfChunkBytes + (2 * k0 + sh) * 16;
         *reinterpret_cast<uint4*>(dst) = v;
     }
 }
@@ -470,26 +622,35 @@ int launch_rows(const void* x, int64_t rows, int64_t K, int64_t ld, uint8_t* cod
 
 }  // namespace
 
-// Cast with the FP4 GEMM's operand preparation in the same launch (gs = 32, contiguous rows): canonical codes
-// and scales, the two sign planes, the UE4M3 scale factors of both planes in the tensor cores' layout (nk64
-// chunks of 512 B per block of 128 rows, rows padded to padded_rows) and the rows' power-of-two offsets.
+// One launch for one or two operands of the FP4 GEMM (K and group size in common): canonical scales (and codes, when asked
+// for) of a cast, the two sign planes, the UE4M3 scale factors of both planes in the tensor cores' layout (nk64 chunks of
+// 512 B per block of 128 rows, rows padded to padded_rows) and the row words.  format: of a cast (group size 32 unless
+// AMXFP4).  flushed_total (optional): incremented by the number of scales flushed.
 namespace {
-template <int FMT>
-int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes, uint8_t* scales, void* pos, void* neg,
-                         uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows, cudaStream_t st,
-                         int* flushed_total, int64_t seg_rows, int64_t seg_pad) {
-    int lpr_log2 = 1;
-    while (lpr_log2 < 5 && (1 << lpr_log2) < G) ++lpr_log2;          // lanes per row: a power of two, 2 .. 32
-    const int gpl = (int)((G + (1 << lpr_log2) - 1) >> lpr_log2);   // groups per lane
-    const int rpw = 32 >> lpr_log2;                                  // rows per warp
-    const int64_t blocks = (padded_rows / 128) * (16 / rpw);         // a block has 8 * rpw rows of one 128-row block
+template <int FMT, int MODE>
+int launch_prepare(const PrepOperand* op, int n, int64_t K, int gs, int nk64, cudaStream_t st, int* flushed_total) {
+    PrepParams p{};
+    p.G = (int)(K / 32);
+    p.lpr_log2 = 1;
+    while (p.lpr_log2 < 5 && (1 << p.lpr_log2) < p.G) ++p.lpr_log2;  // lanes per row: a power of two, 2 .. 32
+    const int gpl = (p.G + (1 << p.lpr_log2) - 1) >> p.lpr_log2;     // pieces per lane
+    const int rpw = 32 >> p.lpr_log2;                                // rows per warp
+    int64_t blocks = 0;
+    for (int i = 0; i < n; ++i) {
+        p.op[i] = op[i];
+        blocks += (op[i].padded_rows / 128) * (16 / rpw);            // a block has 8 * rpw rows of one 128-row block
+        if (i == 0) p.blocks0 = (unsigned)blocks;
+    }
     if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
+    p.nk64 = nk64;
+    p.gs = gs;
+    p.flushed_total = flushed_total;
     const size_t exchange_bytes = (size_t)64 * rpw * nk64;           // both planes, 4 bytes per row and 64 elements
-    const int exchange = exchange_bytes <= (size_t)kCastMaxExchangeBytes;
-    const int smem = kCastRingBytes + (exchange ? (int)exchange_bytes : 0);
-    auto* kernel = gpl <= 1 ? cast_prepared_kernel<FMT, 1> : gpl <= 2 ? cast_prepared_kernel<FMT, 2>
-                 : gpl <= 4 ? cast_prepared_kernel<FMT, 4> : gpl <= 8 ? cast_prepared_kernel<FMT, 8>
-                 : cast_prepared_kernel<FMT, 0>;      // longer rows: the scale bytes are re-read, not kept in registers
+    p.exchange = exchange_bytes <= (size_t)kCastMaxExchangeBytes;
+    const int smem = kCastRingBytes + (p.exchange ? (int)exchange_bytes : 0);
+    auto* kernel = gpl <= 1 ? prepare_operands_kernel<FMT, 1, MODE> : gpl <= 2 ? prepare_operands_kernel<FMT, 2, MODE>
+                 : gpl <= 4 ? prepare_operands_kernel<FMT, 4, MODE> : gpl <= 8 ? prepare_operands_kernel<FMT, 8, MODE>
+                 : prepare_operands_kernel<FMT, 0, MODE>;   // longer rows: the scale bytes are re-read, not kept in registers
     static bool configured[64][5] = {};                 // the opt-in to > 48 KB of dynamic shared memory: per device, kernel
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
@@ -502,22 +663,17 @@ int launch_cast_prepared(const void* x, int64_t rows, int64_t G, uint8_t* codes,
         }
         configured[dev][slot] = true;
     }
-    return launch(kernel, (unsigned)blocks, kCastWarps * 32, smem, st, reinterpret_cast<const uint4*>(x), rows, seg_rows, seg_pad, (int)G, lpr_log2, exchange, reinterpret_cast<uint4*>(codes),
-        reinterpret_cast<uint16_t*>(scales), reinterpret_cast<uint4*>(pos), reinterpret_cast<uint4*>(neg), sf_pos, sf_neg,
-        row_exp, nk64, flushed_total);
+    return launch(kernel, (unsigned)blocks, kCastWarps * 32, smem, st, p);
 }
 }  // namespace
 
-// codes may be nullptr: the canonical codes are then not written (the planes hold the same nibbles).
-int quantize_rows_prepared(const void* x, int64_t rows, int64_t K, uint8_t* codes, uint8_t* scales, void* pos,
-                           void* neg, uint8_t* sf_pos, uint8_t* sf_neg, int* row_exp, int nk64, int64_t padded_rows,
-                           cudaStream_t st, int format, int* flushed_total, int64_t seg_rows, int64_t seg_pad) {
-    const int64_t G = K / 32;
-    if (format == AMX_FMT_SYM_FP8)
-        return launch_cast_prepared<1>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
-    if (format == AMX_FMT_MXFP4)
-        return launch_cast_prepared<2>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
-    return launch_cast_prepared<0>(x, rows, G, codes, scales, pos, neg, sf_pos, sf_neg, row_exp, nk64, padded_rows, st, flushed_total, seg_rows, seg_pad);
+int prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, int nk64, cudaStream_t st, int format, int* flushed_total) {
+    if (format == AMX_FMT_SYM_FP8) return launch_prepare<1, kOneCast>(op, n, K, gs, nk64, st, flushed_total);
+    if (format == AMX_FMT_MXFP4) return launch_prepare<2, kOneCast>(op, n, K, gs, nk64, st, flushed_total);
+    if (gs != 32) return launch_prepare<0, kAnyGroup>(op, n, K, gs, nk64, st, flushed_total);
+    if (!op[0].x || (n > 1 && !op[1].x)) return launch_prepare<0, kAnyKind>(op, n, K, gs, nk64, st, flushed_total);
+    return n == 1 ? launch_prepare<0, kOneCast>(op, n, K, gs, nk64, st, flushed_total)
+                  : launch_prepare<0, kTwoCasts>(op, n, K, gs, nk64, st, flushed_total);
 }
 
 // Softmax of the rows of S (fp32 [rows, ld_s], cols % 32 == 0), rounded to bf16 and cast, in one launch.  With

@@ -86,3 +86,22 @@ def test_other_group_sizes_on_the_fp4_kernel(M, N, K, gs):
         assert np.linalg.norm(got.cpu().numpy()[rows] - ref) <= 1e-5 * np.linalg.norm(ref)
         assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), dev[2], dev[3], gs), got)
         assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), group_size=gs, w_bf16=dev_bf16(w_bits)), got)
+
+
+@pytest.mark.parametrize("gs", [16, 32, 64, 128])
+@pytest.mark.parametrize("M,N,K", [(600, 520, 1152), (2100, 700, 128), (260, 300, 11008), (300, 257, 5504)])
+def test_one_launch_prepares_both_operands(M, N, K, gs):
+    """The launch that casts the activation and casts or splits the weight, at row lengths of 4 to 344 pieces (several rows
+    per warp, one row, more pieces than a lane keeps in registers), ragged rows, strided rows: against the oracle on
+    sampled rows, and the same bits from the bf16 and from the quantized weight."""
+    a_bits, w_bits = inputs.random_groups(3500 + M, M, K, "normal"), inputs.random_groups(3600 + N, N, K, "normal")
+    qw = oracle.quantize(w_bits, gs)
+    wc, ws = (torch.from_numpy(t).cuda() for t in qw)
+    rows = np.unique(np.concatenate([[0, 1, M - 1], np.arange(5, M, 61)]))
+    ref = oracle.gemm(*oracle.quantize(a_bits[rows], gs), *qw, gs)
+    got = amx.quant_gemm(dev_bf16(a_bits), wc, ws, gs)
+    assert np.linalg.norm(got.cpu().numpy()[rows] - ref) <= 1e-5 * np.linalg.norm(ref)
+    strided_a = torch.zeros((M, K + 8), dtype=torch.bfloat16, device="cuda")
+    strided_w = torch.zeros((N, K + 40), dtype=torch.bfloat16, device="cuda")
+    strided_a[:, :K], strided_w[:, 8:8 + K] = dev_bf16(a_bits), dev_bf16(w_bits)
+    assert torch.equal(amx.quant_gemm(strided_a[:, :K], group_size=gs, w_bf16=strided_w[:, 8:8 + K]), got)
