@@ -59,7 +59,7 @@ constexpr uint32_t kColS = 0, kColO = 256, kColSfQ = 384, kColSfKV = 400, kColSf
 static_assert(kColSfKV + kStages * 32 == kColSfP && kColSfP + 2 * 8 == kTmemCols, "tensor-memory budget");
 
 struct __align__(16) Control {
-    uint64_t q_full, q_empty, kv_full[kStages], kv_empty[kStages], s_full[2], s_empty[2], p_full[2], p_empty[2], o_full, o_empty;
+    uint64_t q_full, q_empty, k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages], s_full[2], s_empty[2], p_full[2], p_empty[2], o_full, o_empty;
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -67,10 +67,11 @@ struct __align__(16) Control {
 // shared-memory layout (offsets from the 1024-aligned base)
 template <int PASS>
 struct Smem {
-    static constexpr int kStageBytes = PASS == 2 ? 2 * kTileBytes : kTileBytes;   // K tile, then the V^T tile
     static constexpr int kOffQ = 0;
-    static constexpr int kOffKV = kTileBytes;
-    static constexpr int kOffP = kOffKV + kStages * kStageBytes;                  // two P planes (pass 2)
+    // K and V^T tiles in rings of their own: a K stage is free as soon as its logits are computed, two tiles before the V^T
+    // tile of the same keys is used
+    static constexpr int kOffK = kTileBytes, kOffV = kOffK + kStages * kTileBytes;
+    static constexpr int kOffP = kOffV + (PASS == 2 ? kStages * kTileBytes : 0);  // two P planes (pass 2)
     static constexpr int kOffSfP = kOffP + (PASS == 2 ? 2 * kPlane : 0);          // two buffers x two 512-byte chunks
     static constexpr int kOffKc = kOffSfP + (PASS == 2 ? 2 * 2 * 512 : 0);        // per stage: 128 column factors
     static constexpr int kOffCtl = kOffKc + kKcRing * 512;
@@ -141,8 +142,10 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         mbar_init(&ctl->q_full, 1 + kSfWarps);
         mbar_init(&ctl->q_empty, 1);
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&ctl->kv_full[s], 1 + kSfWarps);
-            mbar_init(&ctl->kv_empty[s], 1);
+            mbar_init(&ctl->k_full[s], 1 + kSfWarps);
+            mbar_init(&ctl->k_empty[s], 1);
+            mbar_init(&ctl->v_full[s], 1 + kSfWarps);
+            mbar_init(&ctl->v_empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&ctl->s_full[b], 1);
@@ -164,7 +167,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     if (warp == 0) {
         // ---------------------------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            int it = 0, ii = 0;
+            int it = 0, ii = 0, n_k = 0, n_v = 0;                   // tiles so far, copies issued
             bool ok = true;
             for (int id = item_id(ii); id < n_items && ok; id = item_id(++ii)) {
                 const int h = item_head(id), m_blk = item_m(id);
@@ -175,20 +178,31 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 const int T = tiles_of(m_blk);
                 for (int j = 0; j < T; ++j, ++it) {
                     const int s = it % kStages;
-                    if (it >= kStages && !mbar_wait(&ctl->kv_empty[s], ((it / kStages) - 1) & 1, &ctl->abort, p.status)) {
+                    const uint32_t freed = ((it / kStages) - 1) & 1;
+                    if (it >= kStages && !mbar_wait(&ctl->k_empty[s], freed, &ctl->abort, p.status)) {
                         ok = false;
                         break;
                     }
-                    uint8_t* st = sm + S_::kOffKV + s * S_::kStageBytes;
-                    mbar_expect_tx(&ctl->kv_full[s], S_::kStageBytes);
-                    tma_load_3d(st, &tm_k, 0, (int)(p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK), 0, &ctl->kv_full[s]);
-                    if (PASS == 2) tma_load_3d(st + kTileBytes, &tm_v, j * 64, (int)(p.v_row0 + (int64_t)(h / p.kv_group) * kVRows), 0, &ctl->kv_full[s]);
+                    mbar_expect_tx(&ctl->k_full[s], kTileBytes);
+                    tma_load_3d(sm + S_::kOffK + s * kTileBytes, &tm_k, 0, (int)(p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK), 0, &ctl->k_full[s]);
+                    ++n_k;
+                    if (PASS == 2) {
+                        if (it >= kStages && !mbar_wait(&ctl->v_empty[s], freed, &ctl->abort, p.status)) {
+                            ok = false;
+                            break;
+                        }
+                        mbar_expect_tx(&ctl->v_full[s], kTileBytes);
+                        tma_load_3d(sm + S_::kOffV + s * kTileBytes, &tm_v, j * 64, (int)(p.v_row0 + (int64_t)(h / p.kv_group) * kVRows), 0, &ctl->v_full[s]);
+                        ++n_v;
+                    }
                 }
             }
             // after a timeout: let the copies already in flight land before shared memory is released
             if (ctl->abort) {
-                for (int i = max(0, it - kStages); i < it; ++i)
-                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->kv_full[i % kStages], (i / kStages) & 1); ++n) {}
+                for (int i = max(0, n_k - kStages); i < n_k; ++i)
+                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->k_full[i % kStages], (i / kStages) & 1); ++n) {}
+                for (int i = max(0, n_v - kStages); i < n_v; ++i)
+                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->v_full[i % kStages], (i / kStages) & 1); ++n) {}
                 if (ii > 0)
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->q_full, (ii - 1) & 1); ++n) {}
             }
@@ -202,12 +216,12 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         // logits of key tile number `it` (global count): S[it % 2] = Q K^T, four sign pairs x two K steps of 64
         auto issue_s = [&](int it) {
             const int s = it % kStages, b = it & 1;
-            if (ok) ok = mbar_wait(&ctl->kv_full[s], (it / kStages) & 1, &ctl->abort, p.status);
+            if (ok) ok = mbar_wait(&ctl->k_full[s], (it / kStages) & 1, &ctl->abort, p.status);
             if (ok && it >= 2) ok = mbar_wait(&ctl->s_empty[b], ((it >> 1) - 1) & 1, &ctl->abort, p.status);
             if (!ok) return;
             tc_fence_after();
             if (elect_one()) {
-                const uint32_t q_addr = base + S_::kOffQ, k_addr = base + S_::kOffKV + s * S_::kStageBytes;
+                const uint32_t q_addr = base + S_::kOffQ, k_addr = base + S_::kOffK + s * kTileBytes;
                 const uint32_t sfq = tmem + kColSfQ, sfk = tmem + kColSfKV + s * 32;
                 uint32_t acc = 0;
 #pragma unroll
@@ -222,20 +236,21 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             acc = 1;
                         }
                 mma_commit(&ctl->s_full[b]);
-                if (PASS == 1) mma_commit(&ctl->kv_empty[s]);    // nothing else reads the stage
+                mma_commit(&ctl->k_empty[s]);
             }
             __syncwarp();
         };
         // O (+)= P V for key tile number `it`: P from the epilogue warps (shared memory + scale-factor chunks)
         auto issue_pv = [&](int it, bool first) {
             const int s = it % kStages, b = it & 1;
+            if (ok) ok = mbar_wait(&ctl->v_full[s], (it / kStages) & 1, &ctl->abort, p.status);
             if (ok) ok = mbar_wait(&ctl->p_full[b], (it >> 1) & 1, &ctl->abort, p.status);
             // the previous item's O has been read out before it is overwritten
             if (ok && first && ii > 0) ok = mbar_wait(&ctl->o_empty, (ii - 1) & 1, &ctl->abort, p.status);
             if (!ok) return;
             tc_fence_after();
             if (elect_one()) {
-                const uint32_t p_addr = base + S_::kOffP + b * kPlane, v_addr = base + S_::kOffKV + s * S_::kStageBytes + kTileBytes;
+                const uint32_t p_addr = base + S_::kOffP + b * kPlane, v_addr = base + S_::kOffV + s * kTileBytes;
                 const uint32_t sfp = tmem + kColSfP + b * 8, sfv = tmem + kColSfKV + s * 32 + 16;
 #pragma unroll
                 for (int kk = 0; kk < 2; ++kk)
@@ -249,7 +264,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                                         idesc(HD), sfp + kk * 4, sfv + (pv * 2 + kk) * 4, acc);
                         acc = 1;
                     }
-                mma_commit(&ctl->kv_empty[s]);
+                mma_commit(&ctl->v_empty[s]);
                 mma_commit(&ctl->p_empty[b]);
             }
             __syncwarp();
@@ -267,8 +282,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             next_s(0);
             next_s(1);
             for (int j = 0; j < T; ++j) {
+                next_s(j + 2);                       // before the wait for P(j): its accumulator is free well before P(j) is
                 if (PASS == 2) issue_pv(it_p++, j == 0);
-                next_s(j + 2);
             }
             if (PASS == 2 && ok && elect_one()) mma_commit(&ctl->o_full);
             __syncwarp();
@@ -313,20 +328,26 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     for (int i = 0; i < 4; ++i) vv[i] = chunk(p.sfv[i >> 1], p.v_row0 + (int64_t)(h / p.kv_group) * kVRows, p.nk64_v, j * 2 + (i & 1));
                 }
                 const int kw = row_word_exp(__ldg(p.k_words + k_row + t));
-                if (ok && it >= kStages) ok = mbar_wait(&ctl->kv_empty[s], ((it / kStages) - 1) & 1, &ctl->abort, p.status);
+                const uint32_t freed = ((it / kStages) - 1) & 1;
+                if (ok && it >= kStages) ok = mbar_wait(&ctl->k_empty[s], freed, &ctl->abort, p.status);
                 if (!ok) continue;
                 tc_fence_after();
                 kc_all[(it % kKcRing) * 128 + t] = p.alpha * 1.4426950408889634f * __uint_as_float((uint32_t)(kw + 127) << 23);
+                auto store = [&](uint32_t col, const uint4 (&x)[4], uint64_t* full) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) tmem_st4(tq + kColSfKV + s * 32 + i * 4, vk[i].x, vk[i].y, vk[i].z, vk[i].w);
+                    for (int i = 0; i < 4; ++i) tmem_st4(tq + col + i * 4, x[i].x, x[i].y, x[i].z, x[i].w);
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full);
+                };
+                store(kColSfKV + s * 32, vk, &ctl->k_full[s]);
                 if (PASS == 2) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) tmem_st4(tq + kColSfKV + s * 32 + 16 + i * 4, vv[i].x, vv[i].y, vv[i].z, vv[i].w);
+                    if (it >= kStages) ok = mbar_wait(&ctl->v_empty[s], freed, &ctl->abort, p.status);
+                    if (!ok) continue;
+                    tc_fence_after();
+                    store(kColSfKV + s * 32 + 16, vv, &ctl->v_full[s]);
                 }
-                tmem_st_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->kv_full[s]);
             }
         }
     } else {
@@ -379,10 +400,6 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 tc_fence_after();
                 // (the tile's column factors were stored before the scale-factor warps arrived on the stage's barrier,
                 // which the MMA warp waited for before it issued what s_full reports as complete)
-                if (PASS == 2 && it >= 2) {                           // the previous P in this buffer has been multiplied
-                    ok = mbar_wait(&ctl->p_empty[b], ((it >> 1) - 1) & 1, &ctl->abort, p.status);
-                    if (!ok) continue;
-                }
                 // u = accumulator x (alpha log2(e) 2^(K row offset)): the logit in base-2 units up to the query row's
                 // power of two ra, by which multiplying is exact: t = u ra.  (Packed fp32 pairs: same roundings as the
                 // scalar operations, half the instructions.)
@@ -452,6 +469,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         uint32_t nib[4];
                         const uint32_t sc = cast::cast_nonneg_group(w, nib);
                         const uint32_t up = to_ue4m3(sc, kmax);
+                        // the previous P in this buffer has been multiplied
+                        if (ok && it >= 2 && !(cg & 1)) ok = mbar_wait(&ctl->p_empty[b], ((it >> 1) - 1) & 1, &ctl->abort, p.status);
+                        if (!ok) return;
                         // plane: row r, 16-byte piece cg of its 64 bytes, 64-byte swizzle; scale factors: chunk of the
                         // K step cg / 2, byte (r % 32) * 16 + (r / 32) * 4 + (cg % 2) * 2, each scale twice (blocks of 16)
                         *reinterpret_cast<uint4*>(sm + S_::kOffP + b * kPlane + r * 64 + ((cg ^ ((r >> 1) & 3)) << 4)) =
