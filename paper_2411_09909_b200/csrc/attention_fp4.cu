@@ -16,18 +16,24 @@
 // issued) and O is 64 columns wide.
 //
 // One persistent CTA per SM walks over (head, block of 128 queries) items; per item it loops over the key tiles:
-//   warp 0      TMA: the item's Q tile; per key tile the K tile and (pass 2) the V^T tile, {+, -} planes each, into a
-//               ring of kStages stages
-//   warp 1      issues the MMAs two key tiles ahead: S(j+2) is issued before the wait for P(j), so the tensor cores
-//               work on the next logits while the epilogue warps turn the current ones into P
-//   warps 2-5   scale factors of Q, K, V^T: global -> registers -> tensor memory (tcgen05.st), and the per-key column
-//               factors alpha * log2(e) * 2^(K row offset) of the tile
-//   warps 6-21  epilogue, two groups of eight warps: group g takes the key tiles with (tile count) % 2 == g from the S
-//               accumulator g, so the two groups are in different phases of their tiles (tensor-memory loads and
-//               maxima in one, exponentials in the other) and keep both the issue slots and the special-function
-//               unit busy; a thread owns one query row and 64 keys of its tiles: tensor memory -> registers (the
-//               accumulator is released right after the loads), softmax arithmetic, the cast, stores to shared memory
+//   warp 0      TMA: the item's Q tile; per key tile the K tile and (pass 2) the V^T tile, {+, -} planes and scale
+//               factors each, into rings of kStages stages
+//   warp 1      issues the MMAs of the logits as far ahead as there are accumulators (three in pass 1, where the third
+//               takes O's columns, two in pass 2)
+//   warp 2      the per-key column factors alpha * log2(e) * 2^(K row offset) of the tile
+//   warp 3      (pass 2) issues the MMAs of P V.  A warp of its own: issued by warp 1 in turn with the logits, every wait
+//               for P held up the next logits (32 heads x 8192 x 128: 2198 us; now 1994)
+//   warps 4-    epilogue, groups of eight warps (three in pass 1, two in pass 2): group g takes the key tiles with
+//               (tile count) % groups == g, so the groups are in different phases of their tiles (tensor-memory loads
+//               and maxima in one, exponentials in the other) and keep both the issue slots and the special-function
+//               unit busy; a thread owns one query row and 64 keys of its tiles: tensor memory -> registers, softmax
+//               arithmetic, the cast, stores to shared memory.  (A third group in pass 2 has no accumulator of its own to
+//               work on: 2023 us.)
 //   after the last key tile of an item the epilogue warps read out O, rescale by the rows' powers of two and store.
+// Scale factors go from global to shared memory with the tiles and on to tensor memory by the issuing warps
+// (tcgen05.cp, ordered with the MMAs): four warps that carried them through registers were a sixth of all instructions.
+// What bounds it (32 heads x 8192): per key tile the tensor cores need 600 cycles in pass 1 and 900 in pass 2, the
+// special-function unit 1024 in each, the issue slots 800 and 1500; a tile takes 1500 and 2380.
 // Tensor memory: S0, S1, O (128 columns each), scale factors of Q (16), of kStages K/V^T stages (32 each), of the
 // two P tiles (8 each): 512 columns.  Every wait is bounded; on a timeout all roles run their loops out without
 // work, tensor memory is released and the status word reports AMX_ERR_TIMEOUT.
@@ -47,19 +53,25 @@ using namespace fp4;
 constexpr int BM = 128, BNK = 128;                   // queries per item, keys per tile
 constexpr int kVRows = 128;                           // rows of one head of V^T (padded at head dimension 64)
 constexpr int kStages = 3;
-// Ring of the per-tile column factors: its writers (scale-factor warps) run at most kStages tiles ahead of the MMAs
-// and those at most 2 tiles ahead of the readers (epilogue), so 8 slots never collide and need no barrier of their own.
-constexpr int kKcRing = 8;
-constexpr int kSfWarps = 4, kEpiWarps = 16;
-constexpr int kThreads = (2 + kSfWarps + kEpiWarps) * 32;
+// Ring of the per-tile column factors.  A group may still read those of tile j when it has released j's accumulator and the
+// other groups theirs, so the MMAs may be done up to tile j + 5 and the writer (warp 2), kStages ahead of those, at tile
+// j + 8: 16 slots never collide and need no barrier of their own.
+constexpr int kKcRing = 16;
+constexpr int kFirstEpi = 4;                          // warps 0-3: TMA, logits MMAs, column factors, P V MMAs
+constexpr int kOWarps = 16;                           // of the epilogue warps, those that read out O
+__host__ __device__ constexpr int epi_groups(int pass) { return pass == 1 ? 3 : 2; }
+__host__ __device__ constexpr int s_buffers(int pass) { return pass == 1 ? 3 : 2; }   // pass 1: the third in O's columns
+__host__ __device__ constexpr int threads(int pass) { return (kFirstEpi + 8 * epi_groups(pass)) * 32; }
+constexpr int kParts = 2 * epi_groups(1);             // partial row statistics of pass 1
 constexpr int kPlane = 128 * 64;                      // one sign plane of a 128 x 128 tile: 64-byte rows
 constexpr int kTileBytes = 2 * kPlane;                // {+, -}
+constexpr int kSfBytes = 4 * kSfChunk;                // a tile's scale factors: {+, -} x two K steps of 64
 // tensor-memory columns
 constexpr uint32_t kColS = 0, kColO = 256, kColSfQ = 384, kColSfKV = 400, kColSfP = 496, kTmemCols = 512;
 static_assert(kColSfKV + kStages * 32 == kColSfP && kColSfP + 2 * 8 == kTmemCols, "tensor-memory budget");
 
 struct __align__(16) Control {
-    uint64_t q_full, q_empty, k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages], s_full[2], s_empty[2], p_full[2], p_empty[2], o_full, o_empty;
+    uint64_t q_full, q_empty, k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages], s_full[3], s_empty[3], p_full[2], p_empty[3], o_full, o_empty;
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -68,21 +80,28 @@ struct __align__(16) Control {
 template <int PASS>
 struct Smem {
     static constexpr int kOffQ = 0;
-    // K and V^T tiles in rings of their own: a K stage is free as soon as its logits are computed, two tiles before the V^T
-    // tile of the same keys is used
+    // K and V^T tiles, each with its scale factors, in rings of their own: a K stage is free as soon as its logits are
+    // computed, two tiles before the V^T tile of the same keys is used
     static constexpr int kOffK = kTileBytes, kOffV = kOffK + kStages * kTileBytes;
     static constexpr int kOffP = kOffV + (PASS == 2 ? kStages * kTileBytes : 0);  // two P planes (pass 2)
     static constexpr int kOffSfP = kOffP + (PASS == 2 ? 2 * kPlane : 0);          // two buffers x two 512-byte chunks
-    static constexpr int kOffKc = kOffSfP + (PASS == 2 ? 2 * 2 * 512 : 0);        // per stage: 128 column factors
+    static constexpr int kOffSfQ = kOffSfP + (PASS == 2 ? 2 * 2 * 512 : 0);
+    static constexpr int kOffSfK = kOffSfQ + kSfBytes, kOffSfV = kOffSfK + kStages * kSfBytes;
+    static constexpr int kOffKc = kOffSfV + (PASS == 2 ? kStages * kSfBytes : 0); // 128 column factors per slot
     static constexpr int kOffCtl = kOffKc + kKcRing * 512;
     static constexpr int kBytes = kOffCtl + 512 + 1024;                           // + Control + alignment slack
 };
 static_assert(sizeof(Control) <= 512, "Control must fit its reserved space");
 
-// K-major operand rows of 64 bytes with the 64-byte swizzle: groups of 8 rows are 512 B apart.
-__device__ __forceinline__ uint64_t desc_sw64(uint32_t addr) {
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+// K-major operand rows of 64 bytes with the 64-byte swizzle: groups of 8 rows are 512 B apart.  lo: the address in units of
+// 16 bytes (the descriptor's low word); the rest is constant, so that a tile's descriptors differ by constants in one word.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr >> 4) & 0x3FFFu) | (1u << 16); }
+__device__ __forceinline__ uint64_t desc_sw64(uint32_t lo) {
+    return ((uint64_t)((512u >> 4) | (1u << 14) | (4u << 29)) << 32) | lo;
 }
+// 32 rows x 16 bytes without swizzle (the source of tcgen05.cp), likewise
+__device__ __forceinline__ uint32_t sf_lo(uint32_t addr) { return (addr >> 4) & 0x3FFFu; }
+__device__ __forceinline__ uint64_t desc_sf(uint32_t lo) { return ((uint64_t)((128u >> 4) | (1u << 14)) << 32) | lo; }
 // kind::mxf4nvf4 block-scaled, A and B E2M1, K-major, UE4M3 scale factors, M = 128, K = 64 per instruction
 __host__ __device__ constexpr uint32_t idesc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24); }
 
@@ -99,7 +118,7 @@ struct Params {
     int64_t L, Lp;           // sequence length, and padded to whole blocks of 128
     float alpha;
     const int* gate;         // not NULL: nothing is done when this word is nonzero (the caller runs the exact kernel then)
-    float2* part;            // [heads * Lp][4]: per row and key-group column {max, sum of 2^(t - max)}, base-2 units
+    float2* part;            // [heads * Lp][kParts]: per row and key-group column {max, sum of 2^(t - max)}, base-2 units
     float* O;                // pass 2 out: [heads][L][head dimension]
     int* status;
     // optional outputs of pass 2 for head 0 of the launch (verification): the bf16 map the cast started from
@@ -116,12 +135,13 @@ struct Params {
 enum Mask { kMaskNone, kMaskCausal, kMaskTail };
 
 template <int PASS, int MASK, int HD>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(threads(PASS), 1)
 attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const Params p) {
     grid_dependency_wait();
     using S_ = Smem<PASS>;
     constexpr bool CAUSAL = MASK == kMaskCausal;
+    constexpr int kGroups = epi_groups(PASS), kSBufs = s_buffers(PASS);
     constexpr int kQkSteps = HD / 64;                     // MMAs along the head dimension per sign pair
     if (p.gate && *p.gate != 0) return;                   // uniform over the grid: nothing was set up yet
     extern __shared__ uint8_t smem_raw[];
@@ -139,22 +159,24 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     auto tiles_of = [&](int m_blk) { return CAUSAL ? m_blk + 1 : p.m_tiles; };
 
     if (threadIdx.x == 0) {
-        mbar_init(&ctl->q_full, 1 + kSfWarps);
+        mbar_init(&ctl->q_full, 1);
         mbar_init(&ctl->q_empty, 1);
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&ctl->k_full[s], 1 + kSfWarps);
+            mbar_init(&ctl->k_full[s], 2);                       // the copies and the column factors
             mbar_init(&ctl->k_empty[s], 1);
-            mbar_init(&ctl->v_full[s], 1 + kSfWarps);
+            mbar_init(&ctl->v_full[s], 1);
             mbar_init(&ctl->v_empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&ctl->s_full[b], 1);
-            mbar_init(&ctl->s_empty[b], kEpiWarps / 2);          // the accumulator's own epilogue group
-            mbar_init(&ctl->p_full[b], kEpiWarps / 2);
-            mbar_init(&ctl->p_empty[b], 1);
+            mbar_init(&ctl->p_full[b], 8);
+        }
+        for (int b = 0; b < kSBufs; ++b) mbar_init(&ctl->s_empty[b], 8);   // the warps of one epilogue group
+        for (int g = 0; g < kGroups; ++g) {
+            mbar_init(&ctl->s_full[g], 1);
+            mbar_init(&ctl->p_empty[g], 1);
         }
         mbar_init(&ctl->o_full, 1);
-        mbar_init(&ctl->o_empty, kEpiWarps);
+        mbar_init(&ctl->o_empty, kOWarps);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -169,11 +191,19 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         if (lane == 0) {
             int it = 0, ii = 0, n_k = 0, n_v = 0;                   // tiles so far, copies issued
             bool ok = true;
+            // the {+, -} chunks of two K steps, from step k64 of the 128 rows from row0
+            auto load_sf = [&](int off, const uint8_t* const (&sf)[2], int64_t row0, int nk64, int k64, uint64_t* full) {
+                const int64_t c = ((row0 >> 7) * nk64 + k64) * (int64_t)kSfChunk;
+                bulk_load(sm + off, sf[0] + c, 2 * kSfChunk, full);
+                bulk_load(sm + off + 2 * kSfChunk, sf[1] + c, 2 * kSfChunk, full);
+            };
             for (int id = item_id(ii); id < n_items && ok; id = item_id(++ii)) {
                 const int h = item_head(id), m_blk = item_m(id);
                 // the previous item's logits MMAs have read the Q tile
                 if (ii > 0 && !mbar_wait(&ctl->q_empty, (ii - 1) & 1, &ctl->abort, p.status)) break;
-                mbar_expect_tx(&ctl->q_full, kTileBytes);
+                const int64_t k_row0 = p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp, v_row = p.v_row0 + (int64_t)(h / p.kv_group) * kVRows;
+                mbar_expect_tx(&ctl->q_full, kTileBytes + kSfBytes);
+                load_sf(S_::kOffSfQ, p.sfq, p.q_row0 + (int64_t)h * p.Lp + m_blk * BM, p.nk64_q, 0, &ctl->q_full);
                 tma_load_3d(sm + S_::kOffQ, &tm_q, 0, (int)(p.q_row0 + (int64_t)h * p.Lp + m_blk * BM), 0, &ctl->q_full);
                 const int T = tiles_of(m_blk);
                 for (int j = 0; j < T; ++j, ++it) {
@@ -183,16 +213,18 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         ok = false;
                         break;
                     }
-                    mbar_expect_tx(&ctl->k_full[s], kTileBytes);
-                    tma_load_3d(sm + S_::kOffK + s * kTileBytes, &tm_k, 0, (int)(p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK), 0, &ctl->k_full[s]);
+                    mbar_expect_tx(&ctl->k_full[s], kTileBytes + kSfBytes);
+                    load_sf(S_::kOffSfK + s * kSfBytes, p.sfk, k_row0 + j * BNK, p.nk64_k, 0, &ctl->k_full[s]);
+                    tma_load_3d(sm + S_::kOffK + s * kTileBytes, &tm_k, 0, (int)(k_row0 + j * BNK), 0, &ctl->k_full[s]);
                     ++n_k;
                     if (PASS == 2) {
                         if (it >= kStages && !mbar_wait(&ctl->v_empty[s], freed, &ctl->abort, p.status)) {
                             ok = false;
                             break;
                         }
-                        mbar_expect_tx(&ctl->v_full[s], kTileBytes);
-                        tma_load_3d(sm + S_::kOffV + s * kTileBytes, &tm_v, j * 64, (int)(p.v_row0 + (int64_t)(h / p.kv_group) * kVRows), 0, &ctl->v_full[s]);
+                        mbar_expect_tx(&ctl->v_full[s], kTileBytes + kSfBytes);
+                        load_sf(S_::kOffSfV + s * kSfBytes, p.sfv, v_row, p.nk64_v, j * 2, &ctl->v_full[s]);
+                        tma_load_3d(sm + S_::kOffV + s * kTileBytes, &tm_v, j * 64, (int)v_row, 0, &ctl->v_full[s]);
                         ++n_v;
                     }
                 }
@@ -207,158 +239,129 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->q_full, (ii - 1) & 1); ++n) {}
             }
         }
-    } else if (warp == 1) {
-        // ---------------------------------------------------------------------------------- MMA issuer
+    } else if (warp == 1 || (PASS == 2 && warp == 3)) {
+        // ---------------------------------------------------------------------------------- MMA issuers
         // The whole warp runs the loops (addresses stay warp-uniform); one elected lane issues.
         const uint32_t base = smem_u32(sm);
-        int it_s = 0, it_p = 0, ii = 0;
+        // scale factors of a tile, {+, -} x k_steps chunks, shared memory -> tensor memory (ordered with the MMAs of this thread)
+        auto copy_sf = [&](uint32_t col, uint32_t lo, int k_steps) {
+#pragma unroll
+            for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+                for (int kk = 0; kk < k_steps; ++kk)
+                    tmem_cp_32x128b_warpx4(col + (pl * 2 + kk) * 4, desc_sf(lo + (uint32_t)((pl * 2 + kk) * kSfChunk >> 4)));
+        };
+        int s = 0, b = 0;                                            // stage, and accumulator (logits) or P buffer of the next tile
+        uint32_t full = 0, freed = 1;                                 // their barriers' parities
         bool ok = true;
-        // logits of key tile number `it` (global count): S[it % 2] = Q K^T, four sign pairs x two K steps of 64
-        auto issue_s = [&](int it) {
-            const int s = it % kStages, b = it & 1;
-            if (ok) ok = mbar_wait(&ctl->k_full[s], (it / kStages) & 1, &ctl->abort, p.status);
-            if (ok && it >= 2) ok = mbar_wait(&ctl->s_empty[b], ((it >> 1) - 1) & 1, &ctl->abort, p.status);
-            if (!ok) return;
-            tc_fence_after();
-            if (elect_one()) {
-                const uint32_t q_addr = base + S_::kOffQ, k_addr = base + S_::kOffK + s * kTileBytes;
-                const uint32_t sfq = tmem + kColSfQ, sfk = tmem + kColSfKV + s * 32;
-                uint32_t acc = 0;
+        if (warp == 1) {
+            const uint32_t q_lo = desc_lo(base + S_::kOffQ), k_lo = desc_lo(base + S_::kOffK);
+            const uint32_t sfq_lo = sf_lo(base + S_::kOffSfQ), sfk_lo = sf_lo(base + S_::kOffSfK);
+            int g = 0, ii = 0;
+            for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
+                const int T = tiles_of(item_m(id));
+                if (ok) ok = mbar_wait(&ctl->q_full, ii & 1, &ctl->abort, p.status);
+                for (int j = 0; j < T; ++j) {
+                    // S[b] = Q K^T of key tile j, four sign pairs x K steps of 64; as far ahead of the epilogue as there are
+                    // accumulators
+                    if (ok) ok = mbar_wait(&ctl->k_full[s], full, &ctl->abort, p.status);
+                    if (ok) ok = mbar_wait(&ctl->s_empty[b], freed, &ctl->abort, p.status);   // (passes at once the first time)
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t kt = k_lo + (uint32_t)s * (kTileBytes >> 4), sfk = tmem + kColSfKV + s * 32;
+                        if (j == 0) copy_sf(tmem + kColSfQ, sfq_lo, kQkSteps);
+                        copy_sf(sfk, sfk_lo + (uint32_t)s * (kSfBytes >> 4), kQkSteps);
+                        uint32_t acc = 0;
 #pragma unroll
-                for (int pa = 0; pa < 2; ++pa)
+                        for (int pa = 0; pa < 2; ++pa)
 #pragma unroll
-                    for (int pw = 0; pw < 2; ++pw)
+                            for (int pw = 0; pw < 2; ++pw)
 #pragma unroll
-                        for (int kk = 0; kk < kQkSteps; ++kk) {
-                            mma_fp4_block16(tmem + kColS + b * 128, desc_sw64(q_addr + pa * kPlane + kk * 32),
-                                            desc_sw64(k_addr + pw * kPlane + kk * 32), idesc(128), sfq + (pa * 2 + kk) * 4,
-                                            sfk + (pw * 2 + kk) * 4, acc);
-                            acc = 1;
-                        }
-                mma_commit(&ctl->s_full[b]);
-                mma_commit(&ctl->k_empty[s]);
-            }
-            __syncwarp();
-        };
-        // O (+)= P V for key tile number `it`: P from the epilogue warps (shared memory + scale-factor chunks)
-        auto issue_pv = [&](int it, bool first) {
-            const int s = it % kStages, b = it & 1;
-            if (ok) ok = mbar_wait(&ctl->v_full[s], (it / kStages) & 1, &ctl->abort, p.status);
-            if (ok) ok = mbar_wait(&ctl->p_full[b], (it >> 1) & 1, &ctl->abort, p.status);
-            // the previous item's O has been read out before it is overwritten
-            if (ok && first && ii > 0) ok = mbar_wait(&ctl->o_empty, (ii - 1) & 1, &ctl->abort, p.status);
-            if (!ok) return;
-            tc_fence_after();
-            if (elect_one()) {
-                const uint32_t p_addr = base + S_::kOffP + b * kPlane, v_addr = base + S_::kOffV + s * kTileBytes;
-                const uint32_t sfp = tmem + kColSfP + b * 8, sfv = tmem + kColSfKV + s * 32 + 16;
-#pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
-                    tmem_cp_32x128b_warpx4(sfp + kk * 4, smem_desc_rows16(base + S_::kOffSfP + (b * 2 + kk) * 512));
-                uint32_t acc = first ? 0u : 1u;
-#pragma unroll
-                for (int pv = 0; pv < 2; ++pv)
-#pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {
-                        mma_fp4_block16(tmem + kColO, desc_sw64(p_addr + kk * 32), desc_sw64(v_addr + pv * kPlane + kk * 32),
-                                        idesc(HD), sfp + kk * 4, sfv + (pv * 2 + kk) * 4, acc);
-                        acc = 1;
+                                for (int kk = 0; kk < kQkSteps; ++kk) {
+                                    mma_fp4_block16(tmem + kColS + b * 128, desc_sw64(q_lo + ((pa * kPlane + kk * 32) >> 4)),
+                                                    desc_sw64(kt + ((pw * kPlane + kk * 32) >> 4)), idesc(128),
+                                                    tmem + kColSfQ + (pa * 2 + kk) * 4, sfk + (pw * 2 + kk) * 4, acc);
+                                    acc = 1;
+                                }
+                        mma_commit(&ctl->s_full[g]);
+                        mma_commit(&ctl->k_empty[s]);
+                        if (j == T - 1) mma_commit(&ctl->q_empty);   // the Q tile is free for the next item
                     }
-                mma_commit(&ctl->v_empty[s]);
-                mma_commit(&ctl->p_empty[b]);
+                    __syncwarp();
+                    if (++s == kStages) s = 0, full ^= 1;
+                    if (++b == kSBufs) b = 0, freed ^= 1;
+                    if (++g == kGroups) g = 0;
+                }
             }
-            __syncwarp();
-        };
+        } else if (PASS == 2) {
+            // O (+)= P V: P from the epilogue warps (shared memory + scale-factor chunks)
+            const uint32_t p_lo = desc_lo(base + S_::kOffP), v_lo = desc_lo(base + S_::kOffV);
+            const uint32_t sfp_lo = sf_lo(base + S_::kOffSfP), sfv_lo = sf_lo(base + S_::kOffSfV);
+            int g = 0, ii = 0;
+            uint32_t p_full = 0;
+            for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
+                const int T = tiles_of(item_m(id));
+                for (int j = 0; j < T; ++j) {
+                    if (ok) ok = mbar_wait(&ctl->v_full[s], full, &ctl->abort, p.status);
+                    // the previous item's O has been read out before it is overwritten
+                    if (ok && j == 0 && ii > 0) ok = mbar_wait(&ctl->o_empty, (ii - 1) & 1, &ctl->abort, p.status);
+                    if (ok) ok = mbar_wait(&ctl->p_full[b], p_full, &ctl->abort, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint32_t vt = v_lo + (uint32_t)s * (kTileBytes >> 4), pt = p_lo + (uint32_t)b * (kPlane >> 4);
+                        const uint32_t sfp = tmem + kColSfP + b * 8, sfv = tmem + kColSfKV + s * 32 + 16;
+                        copy_sf(sfv, sfv_lo + (uint32_t)s * (kSfBytes >> 4), 2);
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk) tmem_cp_32x128b_warpx4(sfp + kk * 4, desc_sf(sfp_lo + (uint32_t)((b * 2 + kk) * 512 >> 4)));
+                        uint32_t acc = j == 0 ? 0u : 1u;
+#pragma unroll
+                        for (int pv = 0; pv < 2; ++pv)
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                mma_fp4_block16(tmem + kColO, desc_sw64(pt + ((kk * 32) >> 4)), desc_sw64(vt + ((pv * kPlane + kk * 32) >> 4)),
+                                                idesc(HD), sfp + kk * 4, sfv + (pv * 2 + kk) * 4, acc);
+                                acc = 1;
+                            }
+                        mma_commit(&ctl->v_empty[s]);
+                        mma_commit(&ctl->p_empty[g]);
+                        if (j == T - 1) mma_commit(&ctl->o_full);
+                    }
+                    __syncwarp();
+                    if (++s == kStages) s = 0, full ^= 1;
+                    if (++b == 2) b = 0, p_full ^= 1;
+                    if (++g == kGroups) g = 0;
+                }
+            }
+        }
+    } else if (warp == 2) {
+        // ---------------------------------------------------------------------------------- column factors
+        int it = 0, ii = 0;
+        bool ok = true;
+        const float unit = p.alpha * 1.4426950408889634f;
         for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
             const int T = tiles_of(item_m(id));
-            if (ok) ok = mbar_wait(&ctl->q_full, ii & 1, &ctl->abort, p.status);
-            // the logits run two key tiles ahead of P V (both accumulators in use); after the item's last S the Q
-            // tile is free for the next item
-            auto next_s = [&](int j) {
-                if (j < T) issue_s(it_s++);
-                if (j == T - 1 && ok && elect_one()) mma_commit(&ctl->q_empty);
-                __syncwarp();
-            };
-            next_s(0);
-            next_s(1);
-            for (int j = 0; j < T; ++j) {
-                next_s(j + 2);                       // before the wait for P(j): its accumulator is free well before P(j) is
-                if (PASS == 2) issue_pv(it_p++, j == 0);
-            }
-            if (PASS == 2 && ok && elect_one()) mma_commit(&ctl->o_full);
-            __syncwarp();
-        }
-    } else if (warp < 2 + kSfWarps) {
-        // ---------------------------------------------------------------------------------- scale factors
-        // Warp w serves the 32-lane quarter w % 4 of tensor memory (every quarter holds a copy of the scale-factor
-        // columns): a lane reads 16 bytes of each 512-byte chunk (the words of rows lane, lane + 32, + 64, + 96)
-        // and stores them to its quarter.  Thread t of the four warps also stages the column factor of key t.
-        const int q = warp & 3, t = (warp - 2) * 32 + lane;
-        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        int it = 0, ii = 0;
-        bool ok = true;
-        auto chunk = [&](const uint8_t* sf, int64_t row0, int nk64, int k64) {
-            return __ldg(reinterpret_cast<const uint4*>(sf + ((row0 >> 7) * nk64 + k64) * (int64_t)kSfChunk + lane * 16));
-        };
-        for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
-            const int h = item_head(id), m_blk = item_m(id);
-            const int64_t q_row = p.q_row0 + (int64_t)h * p.Lp + m_blk * BM;
-            uint4 v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = chunk(p.sfq[i >> 1], q_row, p.nk64_q, i & 1);
-            if (ok && ii > 0) ok = mbar_wait(&ctl->q_empty, (ii - 1) & 1, &ctl->abort, p.status);
-            if (ok) {
-                tc_fence_after();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) tmem_st4(tq + kColSfQ + i * 4, v[i].x, v[i].y, v[i].z, v[i].w);
-                tmem_st_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->q_full);
-            }
-            const int T = tiles_of(m_blk);
-            for (int j = 0; j < T; ++j, ++it) {
-                const int s = it % kStages;
-                const int64_t k_row = p.k_row0 + (int64_t)(h / p.kv_group) * p.Lp + j * BNK;
-                uint4 vk[4], vv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) vk[i] = chunk(p.sfk[i >> 1], k_row, p.nk64_k, i & 1);
-                if (PASS == 2) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) vv[i] = chunk(p.sfv[i >> 1], p.v_row0 + (int64_t)(h / p.kv_group) * kVRows, p.nk64_v, j * 2 + (i & 1));
-                }
-                const int kw = row_word_exp(__ldg(p.k_words + k_row + t));
-                const uint32_t freed = ((it / kStages) - 1) & 1;
-                if (ok && it >= kStages) ok = mbar_wait(&ctl->k_empty[s], freed, &ctl->abort, p.status);
+            const int4* words = reinterpret_cast<const int4*>(p.k_words + p.k_row0 + (int64_t)(item_head(id) / p.kv_group) * p.Lp) + lane;
+            for (int j = 0; j < T; ++j, ++it, words += 32) {
+                const int4 w = __ldg(words);
+                auto factor = [&](int word) { return unit * __uint_as_float((uint32_t)(row_word_exp(word) + 127) << 23); };
+                if (ok && it >= kStages) ok = mbar_wait(&ctl->k_empty[it % kStages], ((it / kStages) - 1) & 1, &ctl->abort, p.status);
                 if (!ok) continue;
-                tc_fence_after();
-                kc_all[(it % kKcRing) * 128 + t] = p.alpha * 1.4426950408889634f * __uint_as_float((uint32_t)(kw + 127) << 23);
-                auto store = [&](uint32_t col, const uint4 (&x)[4], uint64_t* full) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) tmem_st4(tq + col + i * 4, x[i].x, x[i].y, x[i].z, x[i].w);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(full);
-                };
-                store(kColSfKV + s * 32, vk, &ctl->k_full[s]);
-                if (PASS == 2) {
-                    if (it >= kStages) ok = mbar_wait(&ctl->v_empty[s], freed, &ctl->abort, p.status);
-                    if (!ok) continue;
-                    tc_fence_after();
-                    store(kColSfKV + s * 32 + 16, vv, &ctl->v_full[s]);
-                }
+                reinterpret_cast<float4*>(kc_all + (it % kKcRing) * 128)[lane] = make_float4(factor(w.x), factor(w.y), factor(w.z), factor(w.w));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->k_full[it % kStages]);
             }
         }
-    } else {
+    } else if (warp >= kFirstEpi) {
         // ---------------------------------------------------------------------------------- epilogue
-        // Warp e: group g = e / 8 (the key tiles whose global count is g modulo 2, accumulator g), lane quarter
+        // Warp e: group g = e / 8 (the key tiles whose global count is g modulo the groups), lane quarter
         // q = warp % 4 (its rows), half = (e / 4) % 2 of the tile's 128 keys: a thread owns one query row and two
         // 32-key groups (64 columns) of each of its group's tiles.  For reading out O every warp takes 32 columns.
-        const int e = warp - (2 + kSfWarps), q = warp & 3, grp = e >> 3, half = (e >> 2) & 1, cg_o = e >> 2;
+        const int e = warp - kFirstEpi, q = warp & 3, grp = e >> 3, half = (e >> 2) & 1, cg_o = e >> 2;
         const int r = q * 32 + lane;                                 // row inside the item = tensor-memory lane
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        int it = 0, ii = 0;
+        int it = grp, n = 0, it0 = 0, ii = 0;                        // the group's next tile, its tiles so far, the item's first tile
         bool ok = true;
         auto exp2_approx = [](float y) {
             float v;
@@ -371,17 +374,23 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const int64_t grow = (int64_t)h * p.Lp + m;              // row of the launch's stacked heads
             const int a_exp = row_word_exp(__ldg(p.q_words + p.q_row0 + grow));
             const float ra = __uint_as_float((uint32_t)(a_exp + 127) << 23);
-            // pass 2: the row's statistics, merged from the four partial results of pass 1 in a fixed order
+            // pass 2: the row's statistics, merged from the partial results of pass 1 in a fixed order
             float neg_mx = 0.f, inv = 0.f;
             int kmax = 0;
             if (PASS == 2) {
-                const float4* pp = reinterpret_cast<const float4*>(p.part + grow * 4);
-                const float4 a = __ldg(pp), b = __ldg(pp + 1);       // {max0, sum0, max1, sum1}, {max2, sum2, max3, sum3}
-                const float mx = fmaxf(fmaxf(a.x, a.z), fmaxf(b.x, b.z));
-                float sum = a.y * exp2f(a.x - mx);
-                sum += a.w * exp2f(a.z - mx);
-                sum += b.y * exp2f(b.x - mx);
-                sum += b.w * exp2f(b.z - mx);
+                const float4* pp = reinterpret_cast<const float4*>(p.part + grow * kParts);
+                float4 a[kParts / 2];                                 // {max, sum, max, sum}
+                float mx = -INFINITY, sum = 0.f;
+#pragma unroll
+                for (int i = 0; i < kParts / 2; ++i) {
+                    a[i] = __ldg(pp + i);
+                    mx = fmaxf(mx, fmaxf(a[i].x, a[i].z));
+                }
+#pragma unroll
+                for (int i = 0; i < kParts / 2; ++i) {
+                    sum += a[i].y * exp2f(a[i].x - mx);
+                    sum += a[i].w * exp2f(a[i].z - mx);
+                }
                 inv = 1.0f / sum;
                 neg_mx = -mx;
                 // the row's largest element is 2^0 / sum: its group has the row's largest scale
@@ -392,19 +401,25 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             float run_mx = -INFINITY, run_sum = 0.f;                  // pass 1: over this thread's columns of its tiles
             const int T = tiles_of(m_blk);
-            for (int j = 0; j < T; ++j, ++it) {
-                if ((it & 1) != grp) continue;                        // the other group's tile
-                const int b = grp;
-                if (ok) ok = mbar_wait(&ctl->s_full[b], (it >> 1) & 1, &ctl->abort, p.status);
+            for (; it < it0 + T; it += kGroups, ++n) {
+                const int j = it - it0, b = it & 1;                                 // P buffer
+                const uint32_t s_col = tq + kColS + (it % kSBufs) * 128;
+                if (ok) ok = mbar_wait(&ctl->s_full[grp], n & 1, &ctl->abort, p.status);
                 if (!ok) continue;
                 tc_fence_after();
-                // (the tile's column factors were stored before the scale-factor warps arrived on the stage's barrier,
+                // (the tile's column factors were stored before warp 2 arrived on the stage's barrier,
                 // which the MMA warp waited for before it issued what s_full reports as complete)
                 // u = accumulator x (alpha log2(e) 2^(K row offset)): the logit in base-2 units up to the query row's
                 // power of two ra, by which multiplying is exact: t = u ra.  (Packed fp32 pairs: same roundings as the
                 // scalar operations, half the instructions.)
                 uint32_t acc[32];
                 uint64_t u2[16];
+                const int cg0 = half * 2;
+                auto release = [&] {                                  // both halves are in registers
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ctl->s_empty[it % kSBufs]);
+                };
                 auto scale_columns = [&](int cg) {
                     const ulonglong2* kc2 = reinterpret_cast<const ulonglong2*>(kc_all + (it % kKcRing) * 128 + cg * 32);
 #pragma unroll
@@ -466,11 +481,13 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             const __nv_bfloat162 pr = __floats2bfloat162_rn(p0, p1);
                             w[c] = *reinterpret_cast<const uint32_t*>(&pr);
                         }
+                        // the second group's accumulator is loaded while the first one is cast
+                        if (cg == cg0) tmem_ld32(s_col + (cg0 + 1) * 32, acc);
                         uint32_t nib[4];
                         const uint32_t sc = cast::cast_nonneg_group(w, nib);
                         const uint32_t up = to_ue4m3(sc, kmax);
                         // the previous P in this buffer has been multiplied
-                        if (ok && it >= 2 && !(cg & 1)) ok = mbar_wait(&ctl->p_empty[b], ((it >> 1) - 1) & 1, &ctl->abort, p.status);
+                        if (ok && it >= 2 && !(cg & 1)) ok = mbar_wait(&ctl->p_empty[(it - 2) % kGroups], ((it - 2) / kGroups) & 1, &ctl->abort, p.status);
                         if (!ok) return;
                         // plane: row r, 16-byte piece cg of its 64 bytes, 64-byte swizzle; scale factors: chunk of the
                         // K step cg / 2, byte (r % 32) * 16 + (r / 32) * 4 + (cg % 2) * 2, each scale twice (blocks of 16)
@@ -491,17 +508,13 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         }
                     }
                 };
-                // the second group's tensor-memory load is in flight while the first group is worked on
-                const int cg0 = half * 2;
-                tmem_ld32(tq + kColS + b * 128 + cg0 * 32, acc);
+                tmem_ld32(s_col + cg0 * 32, acc);
                 tmem_ld_wait();
                 scale_columns(cg0);
-                tmem_ld32(tq + kColS + b * 128 + (cg0 + 1) * 32, acc);
                 work(cg0);
+                if (PASS == 1) tmem_ld32(s_col + (cg0 + 1) * 32, acc);
                 tmem_ld_wait();
-                tc_fence_before();                                    // both halves are in registers: release the accumulator
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->s_empty[b]);
+                release();
                 scale_columns(cg0 + 1);
                 work(cg0 + 1);
                 if (PASS == 2) {
@@ -510,9 +523,10 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     if (lane == 0) mbar_arrive(&ctl->p_full[b]);
                 }
             }
+            it0 += T;
             if (PASS == 1) {
-                if (ok) p.part[grow * 4 + grp * 2 + half] = make_float2(run_mx, run_sum);
-            } else {
+                if (ok) p.part[grow * kParts + grp * 2 + half] = make_float2(run_mx, run_sum);
+            } else if (e < kOWarps) {
                 // O of the item: rows x (32 columns of the head dimension per thread), rescaled by 2^(row offset of P
                 // + row offset of V^T) - exact - and stored
                 if (ok) ok = mbar_wait(&ctl->o_full, ii & 1, &ctl->abort, p.status);
@@ -573,7 +587,7 @@ int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensor
     }
     const int items = p.heads * p.m_tiles;
     return launch_chained((double)p.heads * (double)p.L * (double)p.L <= 2.7e8,   // about 140 us in the second pass
-                          attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), kThreads, Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
+                          attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS), Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
 }
 
 }  // namespace
@@ -585,7 +599,7 @@ bool attn_fused_supported(int64_t L, int64_t d) {
 int64_t attn_fused_padded(int64_t L) { return (L + BM - 1) / BM * BM; }
 
 // per-row partial softmax statistics of the heads of one launch
-size_t attn_fused_scratch_bytes(int64_t heads, int64_t L) { return up256((size_t)heads * attn_fused_padded(L) * 4 * sizeof(float2)); }
+size_t attn_fused_scratch_bytes(int64_t heads, int64_t L) { return up256((size_t)heads * attn_fused_padded(L) * kParts * sizeof(float2)); }
 
 namespace {
 template <int MASK, int HD>
