@@ -22,18 +22,18 @@
 //               takes O's columns, two in pass 2)
 //   warp 2      the per-key column factors alpha * log2(e) * 2^(K row offset) of the tile
 //   warp 3      (pass 2) issues the MMAs of P V.  A warp of its own: issued by warp 1 in turn with the logits, every wait
-//               for P held up the next logits (32 heads x 8192 x 128: 2198 us; now 1994)
+//               for P held up the next logits (32 heads x 8192 x 128: 2198 us against 1994)
 //   warps 4-    epilogue, groups of eight warps (three in pass 1, two in pass 2): group g takes the key tiles with
 //               (tile count) % groups == g, so the groups are in different phases of their tiles (tensor-memory loads
 //               and maxima in one, exponentials in the other) and keep both the issue slots and the special-function
 //               unit busy; a thread owns one query row and 64 keys of its tiles: tensor memory -> registers, softmax
 //               arithmetic, the cast, stores to shared memory.  (A third group in pass 2 has no accumulator of its own to
-//               work on: 2023 us.)
+//               work on: 2023 us against 1994.)
 //   after the last key tile of an item the epilogue warps read out O, rescale by the rows' powers of two and store.
 // Scale factors go from global to shared memory with the tiles and on to tensor memory by the issuing warps
 // (tcgen05.cp, ordered with the MMAs): four warps that carried them through registers were a sixth of all instructions.
 // What bounds it (32 heads x 8192): per key tile the tensor cores need 600 cycles in pass 1 and 900 in pass 2, the
-// special-function unit 1024 in each, the issue slots 800 and 1500; a tile takes 1500 and 2380.
+// special-function unit 1024 in each, the issue slots 800 and 1480; a tile takes 1500 and 2250.
 // Tensor memory: S0, S1, O (128 columns each), scale factors of Q (16), of kStages K/V^T stages (32 each), of the
 // two P tiles (8 each): 512 columns.  Every wait is bounded; on a timeout all roles run their loops out without
 // work, tensor memory is released and the status word reports AMX_ERR_TIMEOUT.
@@ -61,6 +61,7 @@ constexpr int kFirstEpi = 4;                          // warps 0-3: TMA, logits 
 constexpr int kOWarps = 16;                           // of the epilogue warps, those that read out O
 __host__ __device__ constexpr int epi_groups(int pass) { return pass == 1 ? 3 : 2; }
 __host__ __device__ constexpr int s_buffers(int pass) { return pass == 1 ? 3 : 2; }   // pass 1: the third in O's columns
+static_assert(s_buffers(1) <= epi_groups(1) && s_buffers(2) <= epi_groups(2), "a group meets every phase of its s_full barrier");
 __host__ __device__ constexpr int threads(int pass) { return (kFirstEpi + 8 * epi_groups(pass)) * 32; }
 constexpr int kParts = 2 * epi_groups(1);             // partial row statistics of pass 1
 constexpr int kPlane = 128 * 64;                      // one sign plane of a 128 x 128 tile: 64-byte rows
@@ -88,7 +89,8 @@ struct Smem {
     static constexpr int kOffSfQ = kOffSfP + (PASS == 2 ? 2 * 2 * 512 : 0);
     static constexpr int kOffSfK = kOffSfQ + kSfBytes, kOffSfV = kOffSfK + kStages * kSfBytes;
     static constexpr int kOffKc = kOffSfV + (PASS == 2 ? kStages * kSfBytes : 0); // 128 column factors per slot
-    static constexpr int kOffCtl = kOffKc + kKcRing * 512;
+    static constexpr int kOffTab = kOffKc + kKcRing * 512;                        // per scale byte: see cast_group
+    static constexpr int kOffCtl = kOffTab + (PASS == 2 ? 128 * 8 : 0);
     static constexpr int kBytes = kOffCtl + 512 + 1024;                           // + Control + alignment slack
 };
 static_assert(sizeof(Control) <= 512, "Control must fit its reserved space");
@@ -104,6 +106,31 @@ __device__ __forceinline__ uint32_t sf_lo(uint32_t addr) { return (addr >> 4) & 
 __device__ __forceinline__ uint64_t desc_sf(uint32_t lo) { return ((uint64_t)((128u >> 4) | (1u << 14)) << 32) | lo; }
 // kind::mxf4nvf4 block-scaled, A and B E2M1, K-major, UE4M3 scale factors, M = 128, K = 64 per instruction
 __host__ __device__ constexpr uint32_t idesc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24); }
+
+// cast::cast_nonneg_group with what follows from the group's scale byte looked up in shared memory, {1 / scale, the UE4M3
+// byte under a row offset of zero (far below zero for a zero scale)} (32 heads x 8192: 1978 -> 1948 us).
+__device__ __forceinline__ uint2 scale_entry(uint32_t b) {
+    return make_uint2(__float_as_uint(cast::inv_scale(b)), b ? scale_norm(b) << 1 : 0x80000000u);
+}
+__device__ __forceinline__ uint32_t cast_group(const uint32_t (&w)[16], const uint2* tab, int key_ofs, uint32_t (&nib)[4], uint32_t& up) {
+    const uint32_t m0 = __vimax3_s16x2(w[0], w[1], w[2]), m1 = __vimax3_s16x2(w[3], w[4], w[5]), m2 = __vimax3_s16x2(w[6], w[7], w[8]),
+                   m3 = __vimax3_s16x2(w[9], w[10], w[11]), m4 = __vimax3_s16x2(w[12], w[13], w[14]);
+    uint32_t pm = __vimax3_s16x2(__vimax3_s16x2(m0, m1, m2), __vimax3_s16x2(m3, m4, w[15]), 0);
+    pm = __vmaxs2(pm, pm << 16) & 0xFFFF0000u;                    // the group maximum
+    const uint32_t sc = cast::cvt_e5m2x2(0.0f, cast::trunc12(__uint_as_float(pm) * cast::sixth_up())) & 0x7Fu;
+    const uint2 e = tab[sc];
+    const uint64_t inv2 = cast::pack_f32x2(e.x, e.x);
+    const int t = (int)e.y + key_ofs;
+    up = t >= 8 ? (uint32_t)t : 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint64_t q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = cast::mul_f32x2(cast::pack_f32x2(w[4 * j + i] << 16, w[4 * j + i] & 0xFFFF0000u), inv2);
+        nib[j] = cast::cvt_e2m1x8(q[0], q[1], q[2], q[3]);
+    }
+    return sc;
+}
 
 struct Params {
     // prepared operands (fp4_operand.cuh); row ranges of stacked heads: head h of the launch has its queries at
@@ -180,6 +207,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    uint2* scale_tab = reinterpret_cast<uint2*>(sm + S_::kOffTab);
+    if (PASS == 2 && threadIdx.x >= 128 && threadIdx.x < 256) scale_tab[threadIdx.x - 128] = scale_entry(threadIdx.x - 128);
     if (warp == 1) tmem_alloc(&ctl->tmem_base, kTmemCols);
     tc_fence_before();
     __syncthreads();
@@ -481,11 +510,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             const __nv_bfloat162 pr = __floats2bfloat162_rn(p0, p1);
                             w[c] = *reinterpret_cast<const uint32_t*>(&pr);
                         }
-                        // the second group's accumulator is loaded while the first one is cast
-                        if (cg == cg0) tmem_ld32(s_col + (cg0 + 1) * 32, acc);
                         uint32_t nib[4];
-                        const uint32_t sc = cast::cast_nonneg_group(w, nib);
-                        const uint32_t up = to_ue4m3(sc, kmax);
+                        uint32_t up;
+                        const uint32_t sc = cast_group(w, scale_tab, (15 - kmax) * 8, nib, up);
                         // the previous P in this buffer has been multiplied
                         if (ok && it >= 2 && !(cg & 1)) ok = mbar_wait(&ctl->p_empty[(it - 2) % kGroups], ((it - 2) / kGroups) & 1, &ctl->abort, p.status);
                         if (!ok) return;
@@ -494,11 +521,11 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         *reinterpret_cast<uint4*>(sm + S_::kOffP + b * kPlane + r * 64 + ((cg ^ ((r >> 1) & 3)) << 4)) =
                             make_uint4(nib[0], nib[1], nib[2], nib[3]);
                         *reinterpret_cast<uint16_t*>(sm + S_::kOffSfP + (b * 2 + (cg >> 1)) * 512 + (r & 31) * 16 + (r >> 5) * 4 +
-                                                     (cg & 1) * 2) = (uint16_t)(up | (up << 8));
+                                                     (cg & 1) * 2) = (uint16_t)(up * 257u);
                         if (p.p_plane && h == 0) {                    // verification outputs (head 0 of the launch)
                             const int64_t g = (int64_t)j * 4 + cg, v = m * (p.L / 32) + g;
                             p.p_plane[v] = make_uint4(nib[0], nib[1], nib[2], nib[3]);
-                            *reinterpret_cast<uint16_t*>(p.p_sf + sf_row_offset(m, p.p_nk64) + sf_group_offset((int)g)) = (uint16_t)(up | (up << 8));
+                            *reinterpret_cast<uint16_t*>(p.p_sf + sf_row_offset(m, p.p_nk64) + sf_group_offset((int)g)) = (uint16_t)(up * 257u);
                             if (p.p_codes) p.p_codes[v] = make_uint4(nib[0], nib[1], nib[2], nib[3]);
                             if (p.p_scales) p.p_scales[v] = (uint16_t)sc;
                             if (p.p_bits) {
@@ -508,13 +535,16 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         }
                     }
                 };
+                // pass 2 has the registers to take the second group before it works on the first, which frees the accumulator
+                // early (32 heads x 8192: 2001 -> 1981 us); pass 1, with 24 epilogue warps and three accumulators, has not
                 tmem_ld32(s_col + cg0 * 32, acc);
                 tmem_ld_wait();
                 scale_columns(cg0);
-                work(cg0);
-                if (PASS == 1) tmem_ld32(s_col + (cg0 + 1) * 32, acc);
+                if (PASS == 1) work(cg0);
+                tmem_ld32(s_col + (cg0 + 1) * 32, acc);
                 tmem_ld_wait();
                 release();
+                if (PASS == 2) work(cg0);
                 scale_columns(cg0 + 1);
                 work(cg0 + 1);
                 if (PASS == 2) {
