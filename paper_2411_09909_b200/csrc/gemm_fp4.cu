@@ -20,9 +20,9 @@
 //            completion on the stage's `full` mbarrier
 //   warp 1   allocates TMEM; one lane issues the stage's MMAs (4 sign pairs x K steps of 64), then
 //            commits to the stage's `empty` mbarrier
-//   warps 2-9  (two groups of four, alternating K blocks) move each stage's scale factors shared -> registers -> tensor memory (tcgen05.st; this
-//            keeps the copies off the in-order MMA queue) and arrive on the stage's `full` barrier; they follow only the
-//            `full` barriers and so run ahead into the next tile
+//   warps 2-9  (two groups of four, alternating K blocks) move each stage's scale factors, which come with its tiles, shared
+//            -> registers -> tensor memory (tcgen05.st; this keeps the copies off the in-order MMA queue) and arrive on the
+//            stage's `full` barrier; they follow only barriers and so run ahead into the next tile
 //   warps 10-17 epilogue: TMEM -> registers (double-buffered loads), power-of-two rescale, 32-byte fp32
 //            stores.  While a tile's accumulator is read out the producer already prefetches the next
 //            tile's stages, and the MMA issuer starts the next tile as soon as the columns the two tiles
@@ -74,7 +74,9 @@ struct Cfg {
     static constexpr int kOffAp = 0, kOffAn = ONE_PLANE ? 0 : kTileA, kOffWp = kPlanes * kTileA,
                          kOffWn = kOffWp + (ONE_PLANE ? 0 : kTileB);
     static constexpr int kStageBytes = kPlanes * (kTileA + kTileB);   // {A+, A-} and {W+, W-}: one TMA each
-    static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 2048 + 256;   // + alignment slack + Control
+    // scale factors of a stage: per plane one run of kSteps chunks for the A rows and for either half of the W rows
+    static constexpr int kSfRun = kSteps * kSfChunk, kSfStage = kPlanes * 3 * kSfRun;
+    static constexpr int kSmemBytes = kStages * (kStageBytes + kSfStage) + 1024 + 2048 + 512;   // + alignment slack + Control
     // TMEM columns of one stage's scale factors: A planes (4 columns per K step), then W planes (8)
     static constexpr int kSfColsA = kPlanes * kSteps * 4, kSfCols = kSfColsA + kPlanes * kSteps * 8;
     // the scale factors of kSfSlots K blocks are in tensor memory at a time (fewer than shared-memory stages: the
@@ -87,7 +89,7 @@ struct Cfg {
 constexpr int kMaxStages = 8;
 
 struct __align__(16) Control {
-    uint64_t full[kMaxStages], empty[kMaxStages], accum_full;
+    uint64_t full[kMaxStages], empty[kMaxStages], sf_full[kMaxStages], accum_full;
     uint64_t ovl_free;              // the columns a finished tile shares with the next tile's accumulator have been read
     uint64_t rest_free[2];          // its other columns have been read ([i]: tiles with number % 2 == i)
     uint64_t sides_ready[2];        // the epilogue warps have written sides[i] for the CTA's tile number 2 k + i
@@ -96,7 +98,7 @@ struct __align__(16) Control {
     volatile int sides[2][8];       // per epilogue warp: which sign planes its share of the tile's rows uses
     alignas(16) int w_exp[2][BN];   // read as int4 in the epilogue
 };
-static_assert(sizeof(Control) <= 2048 + 256, "Control must fit its reserved space");
+static_assert(sizeof(Control) <= 2048 + 512, "Control must fit its reserved space");
 
 // K-major operand rows of 64 bytes with the 64-byte swizzle: groups of 8 rows are 512 B apart.
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
@@ -245,7 +247,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     constexpr int kStageBytes = C_::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    Control* ctl = reinterpret_cast<Control*>(tiles + kStages * kStageBytes);
+    uint8_t* sf_stages = tiles + kStages * kStageBytes;
+    Control* ctl = reinterpret_cast<Control*>(sf_stages + kStages * C_::kSfStage);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Work items: tile x K range (one range unless SLICED); an item index is tile * S + range, num_kb the K blocks
     // of one item when there is one range.
@@ -291,6 +294,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->full[s], 1 + 4);               // producer (with the TMA byte count) + four scale-factor warps
             mbar_init(&ctl->empty[s], 1);
+            mbar_init(&ctl->sf_full[s], 1);
         }
         mbar_init(&ctl->accum_full, 1);
         mbar_init(&ctl->ovl_free, kEpilogueWarps);
@@ -361,7 +365,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                         ok = false;
                         break;
                     }
-                    uint8_t* st = tiles + s * kStageBytes;
+                    uint8_t *st = tiles + s * kStageBytes, *sf = sf_stages + s * C_::kSfStage;
+                    // scale factors first: they have one more step to go
+                    mbar_expect_tx(&ctl->sf_full[s], kPlanes * (NHALF ? 2 : 3) * C_::kSfRun);
+                    const int64_t ca = (m_blk * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk,
+                                  cw = (n_blk * (BNT / 128) * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk;
+#pragma unroll
+                    for (int pl = 0; pl < kPlanes; ++pl) {
+                        const uint8_t* w = (pl ? p.sfb_neg : p.sfb_pos) + cw;
+                        bulk_load(sf + (pl * 3 + 0) * C_::kSfRun, (pl ? p.sfa_neg : p.sfa_pos) + ca, C_::kSfRun, &ctl->sf_full[s]);
+                        bulk_load(sf + (pl * 3 + 1) * C_::kSfRun, w, C_::kSfRun, &ctl->sf_full[s]);
+                        if (!NHALF) bulk_load(sf + (pl * 3 + 2) * C_::kSfRun, w + (int64_t)p.nk64 * kSfChunk, C_::kSfRun, &ctl->sf_full[s]);
+                    }
                     mbar_expect_tx(&ctl->full[s], bytes);
                     const int x = (kb0 + kb) * kRowBytes;
                     // one 3-D tile per operand: {row bytes, rows, both sign planes} - or the one plane that is not zero
@@ -373,8 +388,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             }
             // after an abort: let the copies already in flight land before shared memory is released
             if (ctl->abort)
-                for (int i = max(0, it - kStages); i < it; ++i)
+                for (int i = max(0, it - kStages); i < it; ++i) {
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
+                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->sf_full[i % kStages], (i / kStages) & 1); ++n) {}
+                }
         }
     } else if (warp == 1) {
         // -------------------------------------------------------------- MMA issuer
@@ -441,64 +458,52 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
     } else if (warp < 2 + kSfWarps) {
         // -------------------------------------------------------------- scale factors
-        // Warp w serves the 32-lane quarter w % 4 of tensor memory: every quarter has to hold a copy of
-        // the scale-factor columns.  Per K block a lane reads 16 bytes of each 512-byte scale-factor block
-        // straight from global memory (the 4-byte scale words of rows lane, lane+32, lane+64, lane+96) and
-        // stores them to its quarter with tcgen05.st.  The values for the group's next K block are fetched
-        // before the wait for the TMEM buffer, so the global latency stays off the critical path, and the
-        // scale factors are normally in place before the TMA tiles of the same stage land.
-        // Two groups of four warps take alternate K blocks.
+        // Warp w serves the 32-lane quarter w % 4 of tensor memory: every quarter has to hold a copy of the scale-factor
+        // columns.  Per K block a lane reads 16 bytes of each 512-byte chunk of the stage (the 4-byte scale words of rows
+        // lane, lane+32, lane+64, lane+96) and stores them to its quarter with tcgen05.st.  Two groups of four warps take
+        // alternate K blocks.  The chunks come to shared memory with the stage's tiles, several K blocks ahead; fetched by
+        // these warps from global memory, one block ahead each, their latency bounded products of one plane per operand
+        // (MXFP4 8192 x 14336 x 4096: 375 -> 347 us).
         const int q = warp & 3, group = (warp - 2) >> 2;
-        constexpr int kBlocks = kPlanes * kSteps * 3;                  // per K block: A (1) + W (2 row blocks), x planes x steps
-        uint4 sfv[kBlocks];
-        auto fetch = [&](int64_t tile, int kb) {
-            const int64_t m_blk = blk_m(tile), n_blk = blk_n(tile);
-#pragma unroll
-            for (int pl = 0; pl < kPlanes; ++pl)
-#pragma unroll
-                for (int kk = 0; kk < kSteps; ++kk) {
-                    const int64_t c = ((int64_t)kb_begin(tile) + kb) * kSteps + kk;
-                    const uint8_t* a = (pl ? p.sfa_neg : p.sfa_pos) + (m_blk * p.nk64 + c) * kSfChunk + lane * 16;
-                    const uint8_t* w = (pl ? p.sfb_neg : p.sfb_pos) + (n_blk * (BNT / 128) * p.nk64 + c) * kSfChunk + lane * 16;
-                    sfv[(pl * kSteps + kk) * 3 + 0] = __ldg(reinterpret_cast<const uint4*>(a));
-                    sfv[(pl * kSteps + kk) * 3 + 1] = __ldg(reinterpret_cast<const uint4*>(w));
-                    sfv[(pl * kSteps + kk) * 3 + 2] =           // second block of 128 rows (none in a half-width tile)
-                        __ldg(reinterpret_cast<const uint4*>(w + (NHALF ? 0 : (int64_t)p.nk64 * kSfChunk)));
-                }
-        };
-        // this group's K blocks, in order, over all tiles: (tile, kb) with global index it = group, group + 2, ...
-        int64_t tile = blockIdx.x;
-        int kb = group;
-        while (tile < total_tiles && kb >= nkb_of(tile)) { kb -= nkb_of(tile); tile += gridDim.x; }
-        int it = group;
+        int it = 0;
         bool ok = true;
-        if (tile < total_tiles) fetch(tile, kb);
-        while (tile < total_tiles && ok) {
-            const int s = it % kStages;
-            // the slot of the scale-factor ring is free once the MMAs of K block it - kSfSlots are done (the `empty`
-            // barrier of that block's stage; it cannot complete again before this block's factors are stored)
-            if (it >= C_::kSfSlots) {
-                const int j = it - C_::kSfSlots;
-                ok = mbar_wait(&ctl->empty[j % kStages], (j / kStages) & 1, &ctl->abort, p.status);
-            }
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t sfa = tmem + ((uint32_t)(q * 32) << 16) + kTmemSf + (it % C_::kSfSlots) * C_::kSfCols, sfb = sfa + C_::kSfColsA;
+        for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+            const int end = it + nkb_of(tile);
+            // this group's K blocks (global count it % kSfGroups == group)
+            for (int i = it + ((group - it) & (kSfGroups - 1)); i < end; i += kSfGroups) {
+                const int s = i % kStages;
+                ok = mbar_wait(&ctl->sf_full[s], (i / kStages) & 1, &ctl->abort, p.status);
+                if (!ok) break;
+                const uint8_t* sf = sf_stages + s * C_::kSfStage + lane * 16;
+                uint4 v[kPlanes * kSteps * 3];
 #pragma unroll
-            for (int i = 0; i < kPlanes * kSteps; ++i) {
-                tmem_st4(sfa + i * 4, sfv[i * 3].x, sfv[i * 3].y, sfv[i * 3].z, sfv[i * 3].w);
-                tmem_st4(sfb + i * 8, sfv[i * 3 + 1].x, sfv[i * 3 + 1].y, sfv[i * 3 + 1].z, sfv[i * 3 + 1].w);
-                tmem_st4(sfb + i * 8 + 4, sfv[i * 3 + 2].x, sfv[i * 3 + 2].y, sfv[i * 3 + 2].z, sfv[i * 3 + 2].w);
+                for (int pl = 0; pl < kPlanes; ++pl)
+#pragma unroll
+                    for (int kk = 0; kk < kSteps; ++kk)
+#pragma unroll
+                        for (int x = 0; x < 3; ++x)
+                            v[(pl * kSteps + kk) * 3 + x] = *reinterpret_cast<const uint4*>(sf + (pl * 3 + (NHALF ? min(x, 1) : x)) * C_::kSfRun + kk * kSfChunk);
+                // the slot of the scale-factor ring is free once the MMAs of K block i - kSfSlots are done (the `empty`
+                // barrier of that block's stage; it cannot complete again before this block's factors are stored)
+                if (i >= C_::kSfSlots) {
+                    const int j = i - C_::kSfSlots;
+                    ok = mbar_wait(&ctl->empty[j % kStages], (j / kStages) & 1, &ctl->abort, p.status);
+                    if (!ok) break;
+                }
+                tc_fence_after();
+                const uint32_t sfa = tmem + ((uint32_t)(q * 32) << 16) + kTmemSf + (i % C_::kSfSlots) * C_::kSfCols, sfb = sfa + C_::kSfColsA;
+#pragma unroll
+                for (int c = 0; c < kPlanes * kSteps; ++c) {
+                    tmem_st4(sfa + c * 4, v[c * 3].x, v[c * 3].y, v[c * 3].z, v[c * 3].w);
+                    tmem_st4(sfb + c * 8, v[c * 3 + 1].x, v[c * 3 + 1].y, v[c * 3 + 1].z, v[c * 3 + 1].w);
+                    tmem_st4(sfb + c * 8 + 4, v[c * 3 + 2].x, v[c * 3 + 2].y, v[c * 3 + 2].z, v[c * 3 + 2].w);
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->full[s]);
             }
-            // next K block of this group
-            it += kSfGroups;
-            kb += kSfGroups;
-            while (tile < total_tiles && kb >= nkb_of(tile)) { kb -= nkb_of(tile); tile += gridDim.x; }
-            if (tile < total_tiles) fetch(tile, kb);             // in flight during the wait below
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->full[s]);
+            it = end;
         }
     } else {
         // -------------------------------------------------------------- epilogue
