@@ -47,22 +47,36 @@ inline bool programmatic_launch_ok(cudaStream_t st) {
 // blocks land on the SMs in another order, which costs them 2.5-4 % (operands shared by neighbouring tiles cross the two
 // halves of the L2 more often) - more than the gap from about 200 us on.
 template <typename... P, typename... A>
-int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+int launch_clusters(unsigned cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (chained && programmatic_launch_ok(st)) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = chained && programmatic_launch_ok(st) ? 1 : 0;
+    cfg.numAttrs = n;
     if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) != cudaSuccess) {
         cudaGetLastError();
         return AMX_ERR_CUDA;
     }
     return AMX_OK;
+}
+
+template <typename... P, typename... A>
+int launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_clusters(1, chained, kernel, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
 template <typename... P, typename... A>

@@ -14,8 +14,8 @@
 // in the epilogue (exact).  Scales more than 14 binades below their row's largest scale do not fit
 // and are flushed to zero: their groups contribute less than 2^-14 of the row's largest group.
 //
-// Persistent CTAs (one per SM) walk over 128 x 256 tiles of C; K blocks of 128 elements cycle through
-// four 48 KB shared-memory stages:
+// Persistent CTAs (one per SM) walk over 128 x 256 tiles of C - pairs of CTAs over 256 x 256 tiles (PAIR below) -; K blocks
+// cycle through four shared-memory stages:
 //   warp 0   TMA producer: per stage one 3-D tile {A+, A-} and one {W+, W-} (64-byte swizzle),
 //            completion on the stage's `full` mbarrier
 //   warp 1   allocates TMEM; one lane issues the stage's MMAs (4 sign pairs x K steps of 64), then
@@ -32,8 +32,10 @@
 // codes and scales.  Every device-side wait is bounded.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdlib>
 
+#include "cast_math.cuh"
 #include "fp4_operand.cuh"
 #include "gemm.cuh"
 #include "tcgen05.cuh"
@@ -59,18 +61,18 @@ constexpr int kAccWindow = 160;        // first column of the odd tiles' accumul
 constexpr uint32_t kTmemSf = 416;      // scale-factor columns
 constexpr int kTmemSfCols = 96;
 
-// Shared-memory stage geometry for a K block of BK = 128 elements (BK/2 = 64 bytes of codes per row and plane,
-// 64-byte swizzle): 4 stages of 48 KB.  (K blocks of 256 elements in two 96 KB stages measured slower.)
-// ONE_PLANE (BK = 128): a stage holds one plane of each operand, 8 stages of 24 KB.  For two operands in a symmetric
-// format, whose one product per K step leaves the tensor pipe waiting for loads: twice as many K blocks in flight.
-template <int BK_, bool ONE_PLANE = false>
+// Shared-memory stage geometry: four stages of a K block each.  Two planes per operand: BK = 128 elements (64-byte rows), 48 KB
+// (K blocks of 256 elements in two stages measured slower).  ONE_PLANE (both operands in a symmetric format, one product per K
+// step): BK = 256 (128-byte rows); with 128 the tensor cores waited on copies of 1 KB and on a barrier round per two MMAs
+// (MXFP4 8192 x 14336 x 4096: 347 us against 226).  PAIR: the stage of one CTA of the pair, half of the W rows.
+template <int BK_, bool ONE_PLANE = false, bool PAIR = false>
 struct Cfg {
     static constexpr int BK = BK_;
     static constexpr int kPlanes = ONE_PLANE ? 1 : 2;
     static constexpr int kRowBytes = BK / 2;
     static constexpr int kSteps = BK / 64;                            // MMAs (K = 64) per K block and sign pair
-    static constexpr int kStages = ONE_PLANE ? 8 : 4;
-    static constexpr int kTileA = BM * kRowBytes, kTileB = BN * kRowBytes;   // one plane
+    static constexpr int kStages = 4;
+    static constexpr int kTileA = BM * kRowBytes, kTileB = BN / (PAIR ? 2 : 1) * kRowBytes;   // one plane
     static constexpr int kOffAp = 0, kOffAn = ONE_PLANE ? 0 : kTileA, kOffWp = kPlanes * kTileA,
                          kOffWn = kOffWp + (ONE_PLANE ? 0 : kTileB);
     static constexpr int kStageBytes = kPlanes * (kTileA + kTileB);   // {A+, A-} and {W+, W-}: one TMA each
@@ -84,9 +86,9 @@ struct Cfg {
     static constexpr int kSfSlots = kTmemSfCols / kSfCols;
     static_assert(kSfSlots >= 2 && kSfSlots % kSfGroups == 0 && kSfSlots <= kStages, "scale-factor ring");
     static_assert(kAccWindow + BN <= (int)kTmemSf && kTmemSf + kSfSlots * kSfCols <= kTmemCols, "tensor memory map");
-    static_assert(BK == 128, "stages are laid out for 128-element K blocks (64-byte rows, 64-byte swizzle)");
+    static_assert(BK == 128 || BK == 256, "rows of 64 or 128 bytes, swizzled over their length");
 };
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 4;
 
 struct __align__(16) Control {
     uint64_t full[kMaxStages], empty[kMaxStages], sf_full[kMaxStages], accum_full;
@@ -96,7 +98,7 @@ struct __align__(16) Control {
     uint32_t tmem_base;
     volatile int abort;
     volatile int sides[2][8];       // per epilogue warp: which sign planes its share of the tile's rows uses
-    alignas(16) int w_exp[2][BN];   // read as int4 in the epilogue
+    alignas(16) float w_fac[2][BN];   // 2^(row offset of W): read four at a time in the epilogue
 };
 static_assert(sizeof(Control) <= 2048 + 512, "Control must fit its reserved space");
 
@@ -229,20 +231,27 @@ __device__ __forceinline__ void store_row16_bf16(__nv_bfloat16* out, const float
 
 // NHALF: tiles of 128 x 128 for products with at most 128 columns: the W box, the MMA and the epilogue are half as
 // wide, the stage layout keeps its size.
+// PAIR: two CTAs (a cluster) compute a tile of 256 x 256, each the accumulator of 128 of its rows and the load of its A rows and
+// of half of the W rows; their tensor cores read both halves.  The first CTA's warp 1 issues for both: all copies of a stage are
+// counted on its `full` barrier, the other CTA's scale-factor and epilogue warps arrive on its barriers too, and its commits
+// arrive on the barriers of both.
 // ONE_PLANE: the caller states that neither operand has a second sign plane (Cfg above): only the first planes and
 // their scale factors are read, one product per K step.  A tile whose row words show a second plane after all puts
 // AMX_ERR_FLAGS into the status word (the kernel runs to its end; C is then not the product).
-template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false>
+template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false, bool PAIR = false>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                 const __grid_constant__ CUtensorMap tm_a1, const __grid_constant__ CUtensorMap tm_w1, const Params p) {
     grid_dependency_wait();
-    using C_ = Cfg<BK_, ONE_PLANE>;
+    using C_ = Cfg<BK_, ONE_PLANE, PAIR>;
     constexpr int kPlanes = C_::kPlanes;
     if (p.gate && *p.gate != 0) return;                          // uniform over the grid: nothing was set up yet
     constexpr int BNT = NHALF ? BN / 2 : BN;                     // tile width
     constexpr int kOffWnT = NHALF ? C_::kOffWp + C_::kTileB / 2 : C_::kOffWn;   // the box packs its two planes
-    constexpr uint32_t kIdescT = instr_desc(BNT);
+    constexpr uint32_t kIdescT = PAIR ? instr_desc(BNT) + ((uint32_t)(BM >> 4) << 24) : instr_desc(BNT);   // PAIR: M = 256
+    constexpr int BMT = PAIR ? 2 * BM : BM;                      // tile height: of the pair
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0, worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x,
+              workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     constexpr int BK = C_::BK, kRowBytes = C_::kRowBytes, kSteps = C_::kSteps, kStages = C_::kStages;
     constexpr int kStageBytes = C_::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
@@ -257,7 +266,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     const int num_kb = kb_total / S;                             // per item; SLICED: ranges differ by at most one block
     auto kb_begin = [&](int64_t tile) -> int { return SLICED ? (int)((int)(tile % S) * kb_total / S) : 0; };
     // Persistent CTA: tiles blockIdx.x, blockIdx.x + gridDim.x, ...; neighbouring tiles share their A rows.
-    const int64_t n_tiles = (p.N + BNT - 1) / BNT, m_tiles = (p.M + BM - 1) / BM;
+    const int64_t n_tiles = (p.N + BNT - 1) / BNT, m_tiles = (p.M + BMT - 1) / BMT;
     const int64_t total_tiles = m_tiles * n_tiles * S;
     // Tile order.  The CTAs work on ~148 consecutive tiles at a time and advance through K roughly together, so what
     // they read from DRAM per wave is the operand rows the wave touches, once.  Tiles are ordered in bands of
@@ -274,10 +283,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         n = r / rows_here;
         m = b * band + (r - n * rows_here);
     };
-    auto blk_m = [&](int64_t tile) -> int64_t {
+    auto blk_m = [&](int64_t tile) -> int64_t {                  // this CTA's block of 128 rows
         uint32_t m, n;
         banded(tile, m, n);
-        return m;
+        return PAIR ? 2 * (int64_t)m + rank : (int64_t)m;
     };
     auto blk_n = [&](int64_t tile) -> int64_t {
         uint32_t m, n;
@@ -292,22 +301,28 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&ctl->full[s], 1 + 4);               // producer (with the TMA byte count) + four scale-factor warps
+            // producer (with the TMA byte count) + four scale-factor warps; a pair's stages are all reported to its first CTA
+            mbar_init(&ctl->full[s], 1 + 4 * (PAIR ? 2 : 1));
             mbar_init(&ctl->empty[s], 1);
             mbar_init(&ctl->sf_full[s], 1);
         }
         mbar_init(&ctl->accum_full, 1);
-        mbar_init(&ctl->ovl_free, kEpilogueWarps);
-        mbar_init(&ctl->rest_free[0], kEpilogueWarps);
-        mbar_init(&ctl->rest_free[1], kEpilogueWarps);
+        constexpr int kReaders = kEpilogueWarps * (PAIR ? 2 : 1);      // of an accumulator (PAIR: both CTAs' halves)
+        mbar_init(&ctl->ovl_free, kReaders);
+        mbar_init(&ctl->rest_free[0], kReaders);
+        mbar_init(&ctl->rest_free[1], kReaders);
         mbar_init(&ctl->sides_ready[0], kEpilogueWarps);
         mbar_init(&ctl->sides_ready[1], kEpilogueWarps);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) tmem_alloc(&ctl->tmem_base, kTmemCols);
+    if (warp == 1) {
+        if (PAIR) tmem_alloc_pair(&ctl->tmem_base, kTmemCols);
+        else tmem_alloc(&ctl->tmem_base, kTmemCols);
+    }
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();                                    // the other CTA's barriers are there before they are used
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
 
@@ -318,9 +333,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     auto tile_sides = [&](int64_t tile) {
         int bits = 0;
         if (tile < total_tiles) {
-            const int64_t m0 = blk_m(tile) * BM, n0 = blk_n(tile) * BNT;
+            const int64_t m0 = blk_m(tile) * BM, n0 = blk_n(tile) * BNT;  // (PAIR: only the first CTA asks)
 #pragma unroll
-            for (int i = 0; i < BM / 32; ++i)
+            for (int i = 0; i < BMT / 32; ++i)
                 if (m0 + i * 32 + lane < p.M) bits |= (__ldg(p.a_exp + m0 + i * 32 + lane) >> 16) & 3;
 #pragma unroll
             for (int i = 0; i < BNT / 32; ++i)
@@ -341,10 +356,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         // ahead anyway (sides[] in the control block): nothing on this lane's path but a barrier that has long
         // completed and eight shared-memory words.
         if (lane == 0) {
-            constexpr int kTileWT = NHALF ? C_::kTileB / 2 : C_::kTileB;   // one plane of the W tile as loaded
+            constexpr int kTileWT = NHALF ? C_::kTileB / 2 : C_::kTileB;   // one plane of the W tile as loaded (PAIR: of this CTA's half)
             int it = 0, j = 0;                                   // K blocks issued so far over all tiles; tiles so far
             bool ok = true;
-            for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++j) {
+            for (int64_t tile = worker; tile < total_tiles && ok; tile += workers, ++j) {
                 int sides = 5;                                   // ONE_PLANE: the first plane of each operand, always
                 if (!ONE_PLANE) {
                     if (!mbar_wait(&ctl->sides_ready[j & 1], (j >> 1) & 1, &ctl->abort, p.status)) break;
@@ -358,7 +373,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 const uint32_t bytes = (a_planes == 3 ? 2 : 1) * C_::kTileA + (w_planes == 3 ? 2 : 1) * kTileWT;
                 const int64_t m_blk = blk_m(tile), n_blk = blk_n(tile);
                 const int kb0 = kb_begin(tile), nkb = nkb_of(tile);
-                const int ya = (int)(p.a_row0 + m_blk * BM), yw = (int)(p.w_row0 + n_blk * BNT);
+                const int ya = (int)(p.a_row0 + m_blk * BM), yw = (int)(p.w_row0 + n_blk * BNT + (PAIR ? rank * (BNT / 2) : 0));
                 for (int kb = 0; kb < nkb; ++kb, ++it) {
                     const int s = it % kStages;
                     if (it >= kStages && !mbar_wait(&ctl->empty[s], ((it / kStages) - 1) & 1, &ctl->abort, p.status)) {
@@ -368,7 +383,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     uint8_t *st = tiles + s * kStageBytes, *sf = sf_stages + s * C_::kSfStage;
                     // scale factors first: they have one more step to go
                     mbar_expect_tx(&ctl->sf_full[s], kPlanes * (NHALF ? 2 : 3) * C_::kSfRun);
-                    const int64_t ca = (m_blk * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk,
+                    // (an odd number of row blocks leaves the second CTA of the last pair without rows: any factors will do)
+                    const int64_t ca = ((PAIR ? min(m_blk, (p.M + BM - 1) / BM - 1) : m_blk) * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk,
                                   cw = (n_blk * (BNT / 128) * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk;
 #pragma unroll
                     for (int pl = 0; pl < kPlanes; ++pl) {
@@ -377,35 +393,45 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                         bulk_load(sf + (pl * 3 + 1) * C_::kSfRun, w, C_::kSfRun, &ctl->sf_full[s]);
                         if (!NHALF) bulk_load(sf + (pl * 3 + 2) * C_::kSfRun, w + (int64_t)p.nk64 * kSfChunk, C_::kSfRun, &ctl->sf_full[s]);
                     }
-                    mbar_expect_tx(&ctl->full[s], bytes);
                     const int x = (kb0 + kb) * kRowBytes;
+                    if (!PAIR) mbar_expect_tx(&ctl->full[s], bytes);
+                    else if (rank == 0) mbar_expect_tx(&ctl->full[s], 2 * bytes);   // (the other CTA's bytes may be counted first)
+                    const uint32_t full = PAIR ? cluster_addr(&ctl->full[s], 0) : 0;
+                    auto load = [&](uint8_t* dst, const CUtensorMap* map, int y, int z) {
+                        if (PAIR) tma_load_3d_pair(dst, map, x, y, z, full);
+                        else tma_load_3d(dst, map, x, y, z, &ctl->full[s]);
+                    };
                     // one 3-D tile per operand: {row bytes, rows, both sign planes} - or the one plane that is not zero
-                    if (a_planes == 3) tma_load_3d(st + C_::kOffAp, &tm_a, x, ya, 0, &ctl->full[s]);
-                    else tma_load_3d(st + (a_planes == 2 ? C_::kOffAn : C_::kOffAp), &tm_a1, x, ya, a_planes == 2 ? 1 : 0, &ctl->full[s]);
-                    if (w_planes == 3) tma_load_3d(st + C_::kOffWp, &tm_w, x, yw, 0, &ctl->full[s]);
-                    else tma_load_3d(st + (w_planes == 2 ? kOffWnT : C_::kOffWp), &tm_w1, x, yw, w_planes == 2 ? 1 : 0, &ctl->full[s]);
+                    if (a_planes == 3) load(st + C_::kOffAp, &tm_a, ya, 0);
+                    else load(st + (a_planes == 2 ? C_::kOffAn : C_::kOffAp), &tm_a1, ya, a_planes == 2 ? 1 : 0);
+                    if (w_planes == 3) load(st + C_::kOffWp, &tm_w, yw, 0);
+                    else load(st + (w_planes == 2 ? kOffWnT : C_::kOffWp), &tm_w1, yw, w_planes == 2 ? 1 : 0);
                 }
             }
             // after an abort: let the copies already in flight land before shared memory is released
             if (ctl->abort)
                 for (int i = max(0, it - kStages); i < it; ++i) {
-                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
+                    // (PAIR: the first CTA waits for both, the other one for the first at the end of the kernel)
+                    if (rank == 0)
+                        for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->sf_full[i % kStages], (i / kStages) & 1); ++n) {}
                 }
         }
+    } else if (PAIR && warp == 1 && rank == 1) {
+        // the pair's MMAs are issued by its first CTA
     } else if (warp == 1) {
         // -------------------------------------------------------------- MMA issuer
         // The whole warp runs the loop (so that addresses and descriptors stay warp-uniform); one elected
         // lane issues.  All operand descriptors differ from the first stage's only in their 14-bit address
         // field (bytes >> 4); the per-plane and per-K-step offsets are compile-time constants.
-        const uint64_t desc0 = smem_desc_sw64(smem_u32(tiles));
+        const uint64_t desc0 = kRowBytes == 128 ? smem_desc_sw128(smem_u32(tiles)) : smem_desc_sw64(smem_u32(tiles));
         int it = 0, t = 0;
         bool ok = true, ready = false;                           // ready: the next K block's barrier was seen complete
         // (the planes of a tile: tile_sides above; the words of the next tile are fetched while the current one runs)
-        int sides_next = ONE_PLANE ? 0 : tile_sides(blockIdx.x);
-        for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+        int sides_next = ONE_PLANE ? 0 : tile_sides(worker);
+        for (int64_t tile = worker; tile < total_tiles && ok; tile += workers) {
             const int sides = ONE_PLANE ? 5 : whole_sides(sides_next);   // an all-zero operand: one product, which zeroes the tile
-            if (!ONE_PLANE) sides_next = tile_sides(tile + gridDim.x);
+            if (!ONE_PLANE) sides_next = tile_sides(tile + workers);
             const int nkb = nkb_of(tile);
             const int n_mma = ((sides & 1) + ((sides >> 1) & 1)) * (((sides >> 2) & 1) + ((sides >> 3) & 1)) * kSteps;
             // this tile's accumulator window: the columns it shares with the previous tile's must have been read, and
@@ -437,22 +463,27 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 #pragma unroll
                             for (int kk = 0; kk < kSteps; ++kk) {   // 64 elements = 32 bytes along the swizzled row
                                 if (((sides >> pa) & 1) && ((sides >> (2 + pw)) & 1)) {
-                                    mma_fp4_block16(acc, dstage + (((pa ? C_::kOffAn : C_::kOffAp) + kk * 32) >> 4),
-                                                    dstage + (((pw ? kOffWnT : C_::kOffWp) + kk * 32) >> 4), kIdescT,
-                                                    sfa + (pa * kSteps + kk) * 4, sfb + (pw * kSteps + kk) * 8,
-                                                    idx ? 1u : accumulate);
+                                    const uint64_t da = dstage + (((pa ? C_::kOffAn : C_::kOffAp) + kk * 32) >> 4),
+                                                   dw = dstage + (((pw ? kOffWnT : C_::kOffWp) + kk * 32) >> 4);
+                                    const uint32_t sa = sfa + (pa * kSteps + kk) * 4, sw = sfb + (pw * kSteps + kk) * 8;
+                                    if (PAIR) mma_fp4_block16_pair(acc, da, dw, kIdescT, sa, sw, idx ? 1u : accumulate);
+                                    else mma_fp4_block16(acc, da, dw, kIdescT, sa, sw, idx ? 1u : accumulate);
                                     // with two MMAs still to go (they keep the pipe busy meanwhile), look whether the
                                     // next K block is complete, so that its MMAs can follow without a wait
                                     if (idx == max(n_mma - 3, 0)) seen = mbar_try_wait(&ctl->full[s_next], parity_next);
                                     ++idx;
                                 }
                             }
-                    mma_commit(&ctl->empty[s]);
+                    if (PAIR) mma_commit_pair(&ctl->empty[s]);
+                    else mma_commit(&ctl->empty[s]);
                 }
                 ready = __any_sync(0xFFFFFFFFu, seen) != 0;
                 accumulate = 1;
             }
-            if (ok && elect_one()) mma_commit(&ctl->accum_full);
+            if (ok && elect_one()) {
+                if (PAIR) mma_commit_pair(&ctl->accum_full);
+                else mma_commit(&ctl->accum_full);
+            }
             __syncwarp();
             ++t;
         }
@@ -467,7 +498,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         const int q = warp & 3, group = (warp - 2) >> 2;
         int it = 0;
         bool ok = true;
-        for (int64_t tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+        for (int64_t tile = worker; tile < total_tiles && ok; tile += workers) {
             const int end = it + nkb_of(tile);
             // this group's K blocks (global count it % kSfGroups == group)
             for (int i = it + ((group - it) & (kSfGroups - 1)); i < end; i += kSfGroups) {
@@ -501,7 +532,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->full[s]);
+                if (lane == 0) {
+                    if (PAIR) mbar_arrive_remote(&ctl->full[s], 0);
+                    else mbar_arrive(&ctl->full[s]);
+                }
             }
             it = end;
         }
@@ -520,22 +554,28 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         // The per-tile constants (this thread's column offset and row offset) are fetched one tile ahead, so that
         // their latency is off the path between two tiles.
         struct TileConsts {
-            int w_ex, a_ex, planes;     // planes: bit 0/1 this thread's row of A has +/-, bit 2/3 its row of W has
+            float w_fac, a_fac;         // 2^(row offset)
+            int planes;                 // planes: bit 0/1 this thread's row of A has +/-, bit 2/3 its row of W has
         };
+        // (row offsets lie between -24 and 7, so neither a factor nor the product of two leaves the normal range: the scaled
+        // results are exact, as before the optional tensor scales' one rounding)
+        auto pow2 = [](int e) { return __uint_as_float((uint32_t)(e + 127) << 23); };
         auto load_consts = [&](int64_t tl) {
-            TileConsts c = {0, 0, 0};
+            TileConsts c = {1.f, 1.f, 0};
             if (tl < total_tiles) {
                 const int64_t n = blk_n(tl) * BNT + tid_e, mm = blk_m(tl) * BM + q * 32 + lane;
                 if (tid_e < BNT && n < p.N) {
                     const int w = __ldg(p.w_exp + n);
-                    c.w_ex = row_word_exp(w);
+                    c.w_fac = pow2(row_word_exp(w));
                     c.planes |= ((w >> 16) & 3) << 2;
                 }
                 if (mm < p.M) {
                     const int w = __ldg(p.a_exp + mm);
-                    c.a_ex = row_word_exp(w);
+                    c.a_fac = pow2(row_word_exp(w));
                     c.planes |= (w >> 16) & 3;
                 }
+                const int64_t mo = mm + (rank ? -BM : BM);       // the pair's other row block: its planes are loaded here too
+                if (PAIR && mo < p.M) c.planes |= (__ldg(p.a_exp + mo) >> 16) & 3;
             }
             return c;
         };
@@ -553,24 +593,32 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 mbar_arrive(&ctl->sides_ready[j & 1]);
             }
         };
+        auto released = [&](uint64_t* b) {                       // this warp's columns have been read: tells the issuer
+            __syncwarp();
+            if (lane == 0) {
+                if (PAIR && rank) mbar_arrive_remote(b, 0);
+                else mbar_arrive(b);
+            }
+        };
         const float out_scale = p.scale_a ? __ldg(p.scale_a) * __ldg(p.scale_w) : 1.0f;
-        int64_t tile = blockIdx.x;
+        int64_t tile = worker;
         TileConsts nxt = load_consts(tile);
         publish(nxt, tile, 0);
         while (tile < total_tiles && ok) {
             const TileConsts cur = nxt;
-            const int64_t tile_after = tile + gridDim.x;
+            const int64_t tile_after = tile + workers;
             nxt = load_consts(tile_after);                       // in flight while this tile is worked on
             publish(nxt, tile_after, t + 1);
             const int64_t m0 = blk_m(tile) * BM, n0 = blk_n(tile) * BNT;
             float* const C_item = p.C + (SLICED ? (tile % S) * p.slice_stride : 0);
-            int* w_exp = ctl->w_exp[t & 1];
-            w_exp[tid_e] = cur.w_ex;
+            float* w_fac = ctl->w_fac[t & 1];
+            w_fac[tid_e] = cur.w_fac;
             const int64_t m = m0 + q * 32 + lane;
-            const int a_exp = cur.a_ex;
+            const float a_fac = cur.a_fac * out_scale;
+            const uint64_t a_fac2 = cast::pack_f32x2(__float_as_uint(a_fac), __float_as_uint(a_fac));
             ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
             tc_fence_after();
-            // every epilogue warp has written its part of w_exp (named barrier: the other roles do not join)
+            // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join)
             asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
             if (ok) {
                 // The tile's window starts at column 0 (even t) or kAccWindow (odd t).  The kOvl columns it shares with
@@ -584,8 +632,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(odd ? kAccWindow : 0);
                 uint32_t v[2][16];
                 if (kC1 == 0) {                                  // nothing shared: the next tile may start at once
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->ovl_free);
+                    released(&ctl->ovl_free);
                 }
                 tmem_ld16(taddr + chunk_col(0), v[0]);
 #pragma unroll
@@ -594,26 +641,20 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     tmem_ld_wait();
                     if (i + 1 == kC1) {                          // the shared columns are in registers
                         tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&ctl->ovl_free);
+                        released(&ctl->ovl_free);
                     }
                     if (i + 1 == kC1 + kC2) {                    // so is the rest: tile t + 2 may overwrite the window
                         tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&ctl->rest_free[odd]);
+                        released(&ctl->rest_free[odd]);
                     }
                     if (i + 1 < kC1 + kC2) tmem_ld16(taddr + chunk_col(i + 1), v[buf ^ 1]);   // loads while this chunk is stored
                     const int col = chunk_col(i);
                     float f[16];
 #pragma unroll
                     for (int j = 0; j < 16; j += 4) {
-                        const int4 we = *reinterpret_cast<const int4*>(&w_exp[col + j]);
-                        const int ex[4] = {we.x, we.y, we.z, we.w};
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int sh = min(127, max(-126, a_exp + ex[k]));
-                            f[j + k] = __uint_as_float(v[buf][j + k]) * __uint_as_float((uint32_t)(sh + 127) << 23) * out_scale;
-                        }
+                        const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&w_fac[col + j]);
+                        cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[buf][j], v[buf][j + 1]), cast::mul_f32x2(w2.x, a_fac2)), f[j], f[j + 1]);
+                        cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[buf][j + 2], v[buf][j + 3]), cast::mul_f32x2(w2.y, a_fac2)), f[j + 2], f[j + 3]);
                     }
                     if (m < p.M) {
                         if (p.out_bf16)
@@ -631,9 +672,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
+    if (PAIR) cluster_sync();                                    // no CTA leaves while the other still uses its memory
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        if (PAIR) tmem_dealloc_pair(tmem, kTmemCols);
+        else tmem_dealloc(tmem, kTmemCols);
     }
 }
 
@@ -651,29 +694,40 @@ size_t gemm_fp4_workspace_bytes(int64_t M, int64_t N, int64_t K) {
 
 namespace {
 
-template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false>
+int sm_count(int dev) {                                              // 0: the device cannot be asked
+    static int count[64] = {};
+    if (!count[dev] && cudaDeviceGetAttribute(&count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return count[dev];
+}
+
+template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false, bool PAIR = false>
 int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, const OperandLayout& ow, int64_t a_rows,
                int64_t w_rows, Params p, int dev, cudaStream_t st) {
-    using C_ = Cfg<BK_, ONE_PLANE>;
+    using C_ = Cfg<BK_, ONE_PLANE, PAIR>;
+    constexpr int kBoxW = PAIR ? BN / 2 : NHALF ? BN / 2 : BN;
     constexpr int BNT = NHALF ? BN / 2 : BN;
     static bool configured[64] = {};
     if (!configured[dev]) {
-        if (cudaFuncSetAttribute(gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::kSmemBytes) != cudaSuccess)
+        if (cudaFuncSetAttribute(gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::kSmemBytes) != cudaSuccess)
             return AMX_ERR_CUDA;
         configured[dev] = true;
     }
     CUtensorMap tm_a, tm_w, tm_a1, tm_w1;                       // both planes of a tile in one box, and one plane alone
-    if (!make_map(&tm_a, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes) || !make_map(&tm_w, pw, w_rows, p.K, ow.plane, BNT, C_::kRowBytes) ||
+    if (!make_map(&tm_a, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes) || !make_map(&tm_w, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes) ||
         !make_map(&tm_a1, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes, 1) ||
-        !make_map(&tm_w1, pw, w_rows, p.K, ow.plane, BNT, C_::kRowBytes, 1))
+        !make_map(&tm_w1, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes, 1))
         return AMX_ERR_CUDA;
-    static int sm_count[64] = {};
-    if (!sm_count[dev] && cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return AMX_ERR_CUDA;
-    const int64_t tiles = ((p.N + BNT - 1) / BNT) * ((p.M + BM - 1) / BM) * (SLICED ? p.slices : 1);
-    const unsigned grid = (unsigned)(tiles < sm_count[dev] ? tiles : sm_count[dev]);   // one persistent CTA per SM
-    return launch_chained((double)p.M * (double)p.N * (double)p.K <= 1.1e11,      // about 170 us
-                          gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w, tm_a1, tm_w1, p);
+    if (!sm_count(dev)) return AMX_ERR_CUDA;
+    constexpr int kCtas = PAIR ? 2 : 1, BMT = BM * kCtas;
+    if (PAIR) p.band = (p.band + 1) / 2;
+    const int64_t tiles = ((p.N + BNT - 1) / BNT) * ((p.M + BMT - 1) / BMT) * (SLICED ? p.slices : 1);
+    const int64_t workers = std::min<int64_t>(tiles, sm_count(dev) / kCtas);           // one persistent CTA per SM
+    const unsigned grid = (unsigned)workers * kCtas;
+    return launch_clusters(kCtas, (double)p.M * (double)p.N * (double)p.K <= 1.1e11,      // about 170 us
+                          gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w, tm_a1, tm_w1, p);
 }
 
 }  // namespace
@@ -764,9 +818,18 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
         const int r2 = launch_fp4<128, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st);
         return r2 != AMX_OK ? r2 : reduce_slices(part, slices, M, N, C, ld_c, st);
     }
-    // both operands stated to be single planes: the deeper pipeline (full-width tiles; the other shapes are short
-    // products, where the depth does not matter, and run the general kernel, which skips absent planes by itself)
-    if (one_plane && !half) return launch_fp4<128, false, false, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st);
+    // A pair of SMs per tile (256 x 256) where there is more than a tile for every SM: either SM loads half of the W rows.
+    // 2048 x 12288 x 4096: 159 -> 154 us, 16384 x 10240 x 8192: 1720 -> 1655 (less power for the operands, higher clocks).
+    // With at most one tile per SM there is nothing to overlap the pair's longer start and end with (1024 x 4096 x 4096: 36 us
+    // alone, 39 in pairs); an odd row block leaves half a pair idle, which a sixteenth of the rows may cost.
+    const int64_t m_blocks = (M + BM - 1) / BM;
+    const bool pair = !half && m_blocks * ((N + BN - 1) / BN) > sm_count(dev) && (m_blocks % 2 == 0 || m_blocks >= 15);
+    if (pair)
+        return one_plane ? launch_fp4<256, false, false, true, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st)
+                         : launch_fp4<128, false, false, false, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st);
+    // both operands stated to be single planes (full-width tiles; the half-width ones are short products and run the general
+    // kernel, which skips absent planes by itself)
+    if (one_plane && !half) return launch_fp4<256, false, false, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st);
     return half ? launch_fp4<128, false, true>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st)
                 : launch_fp4<128>(pa, pw, oa, ow, a.rows_total, w.rows_total, p, dev, st);
 }
