@@ -845,9 +845,9 @@ def run_ours(args):
         "decode": decode,
         "clocks": clocks,
         "e2e": e2e,
-        # kernels per layer: 2 casts + the GEMM; without the fused entry points the FP4 kernel's operands need
-        # one preparation kernel each on top
-        "gpu_launches": (5 if "mxf4" in gemm_kernel and not fused_prepare else 3) * len(layers) * args.steps,
+        # kernels per layer: 2 casts, the status words' clearing and the GEMM; without the fused entry points the FP4
+        # kernel's operands need one preparation kernel each on top
+        "gpu_launches": (6 if "mxf4" in gemm_kernel and not fused_prepare else 4) * len(layers) * args.steps,
     }
     if len(layer_ids) != len(inputs.LINEAR_CONFIGS[CONFIG]["layers"]):
         line["config"]["layers"] = layer_ids

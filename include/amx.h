@@ -74,11 +74,11 @@ typedef enum amx_status {
 #define AMX_OUT_F32 0x1u
 /* flags for amx_gemm / amx_quant_gemm: kernel choice.  Default (AMX_GEMM_AUTO): at most 64 rows of A with K >= 512 and
  * K % 128 == 0 go to the weight-streaming kernel (AMX_GEMM_ROWS), as do up to 256 rows of a small product or against a
- * large weight (in blocks of rows); otherwise group size 32 runs on the tcgen05 tensor cores - the FP4 kernel when
- * M*N*K >= 2^28, the exact bf16-decode kernel below that (which cuts K into slices over CTAs when a product has few
- * output tiles and adds the partial products in slice order); what remains runs on the SIMT kernel.
+ * large weight (in blocks of rows); otherwise the FP4 kernel takes every fixed group size when M*N*K >= 2^27, the exact
+ * bf16-decode tcgen05 kernel group size 32 below that (it cuts K into slices over CTAs when a product has few output
+ * tiles and adds the partial products in slice order); what remains runs on the SIMT kernel.
  * AUTO never loses a scale: where it picks the FP4 kernel and preparing the operands had to flush one (see
- * AMX_GEMM_FP4), the FP4 kernel returns at once and the exact bf16-decode kernel computes the product instead.
+ * AMX_GEMM_FP4), the FP4 kernel returns at once and an exact kernel computes the product instead.
  * The decision is taken on the device, from the count amx_gemm_flushed_scales() reports; it costs one empty
  * launch per call and the bf16-decode kernel's scratch on top of the FP4 kernel's. */
 #define AMX_GEMM_AUTO 0x0u
@@ -289,7 +289,7 @@ int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, int64_t ld_
  * leave in 16 bits).  Per head h:
  *   S = AMX(Q_h) AMX(K_h)^T          groups along head_dim
  *   P = softmax(S / sqrt(d)) per row, fp32, rounded to bf16; no mask.  P itself is never stored.  When both
- *       products run on the FP4 kernel, d == 128 and L % 128 == 0, S is not stored either: one fused kernel does both
+ *       products run on the FP4 kernel (AMX_GEMM_AUTO: from L * L * d >= 2^25) and d is 64 or 128, S is not stored either: one fused kernel does both
  *       products and the softmax in two launches - the first pass over Q K^T keeps per-row softmax statistics, the
  *       second recomputes each tile, normalises and casts it in registers and multiplies it with V on the tensor
  *       cores (row sums are taken tile by tile, so single elements of P may round to the neighbouring bf16 value
