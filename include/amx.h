@@ -289,12 +289,13 @@ int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, int64_t ld_
  * leave in 16 bits).  Per head h:
  *   S = AMX(Q_h) AMX(K_h)^T          groups along head_dim
  *   P = softmax(S / sqrt(d)) per row, fp32, rounded to bf16; no mask.  P itself is never stored.  When both
- *       products run on the FP4 kernel (AMX_GEMM_AUTO: from L * L * d >= 2^25) and d is 64 or 128, S is not stored either: one fused kernel does both
- *       products and the softmax in two launches - the first pass over Q K^T keeps per-row softmax statistics, the
- *       second recomputes each tile, normalises and casts it in registers and multiplies it with V on the tensor
- *       cores (row sums are taken tile by tile, so single elements of P may round to the neighbouring bf16 value
- *       compared with amx_softmax_quantize on a stored S; O agrees to ~1e-5 relative).  Other shapes and kernels
- *       store one head's S in the workspace.
+ *       products run on the FP4 kernel (AMX_GEMM_AUTO: from L * L * d >= 2^25) and d is 64 or 128, S is not stored
+ *       either: one fused kernel does both products and the softmax - passes over Q K^T that keep per-row softmax
+ *       statistics, then one that recomputes each tile, normalises and casts it in registers and multiplies it with V
+ *       on the tensor cores.  P has the bits of amx_softmax_quantize on a stored S (up to 8192 keys), except with
+ *       d = 128, L % 128 == 0 and either AMX_GEMM_FP4 or L * L * d >= 2^28: there the statistics take one pass, with
+ *       another order of the row sum, and single elements of P may round to the neighbouring bf16 value, which can move
+ *       the scale of its group and with it that row of O.  Other shapes and kernels store one head's S in the workspace.
  *   O_h = AMX(P) AMX(V_h)            groups along the key axis (V is quantized down its rows)
  *   flags    AMX_GEMM_* kernel choice for both products, optionally | AMX_ATTN_CAUSAL: query i sees keys 0..i only
  *            (the mask is applied to the logits before the softmax; masked entries of P are exactly 0).  In the

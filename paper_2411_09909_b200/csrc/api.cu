@@ -477,8 +477,8 @@ extern "C" int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, 
 namespace {
 // Workspace of amx_attention.  Heads are taken in chunks: the casts of Q, K and V (small per head) run once per chunk
 // on the stacked heads.  Two ways from there:
-//   fused   (head dimension 128 or 64, products on the FP4 kernel) both products and the softmax in two launches of the
-//           fused kernel for all heads of the chunk; Q, K and V^T as prepared operands, every head padded to whole
+//   fused   (head dimension 128 or 64, products on the FP4 kernel) both products and the softmax in two or three launches of
+//           the fused kernel for all heads of the chunk; Q, K and V^T as prepared operands, every head padded to whole
 //           blocks of 128 rows
 //   stored  the logits and the cast map of `batch` heads at a time in the workspace: batched launches of the bf16-decode
 //           kernel (one product, one softmax and cast, one product per batch), or head by head on the other kernels
@@ -487,7 +487,7 @@ struct AttnLayout {
     size_t qc, qs, kc, ks, vc, vs, pc, ps, S, pq, pk, pv, pp, stats, gemm, total;
 };
 
-AttnLayout attn_layout_fused(int64_t L, int64_t d) {
+AttnLayout attn_layout_fused(int64_t L, int64_t d, bool ordered) {
     AttnLayout a{};
     const int64_t Lp = attn_fused_padded(L);
     // 16 heads x (8192 / 128) blocks of queries load 148 persistent CTAs evenly; shorter sequences take more heads
@@ -500,7 +500,7 @@ AttnLayout attn_layout_fused(int64_t L, int64_t d) {
     a.pq = take(gemm_fp4_prepared_bytes(a.chunk * Lp, d, false));
     a.pk = take(gemm_fp4_prepared_bytes(a.chunk * Lp, d, true));
     a.pv = take(gemm_fp4_prepared_bytes(a.chunk * 128, L, true));
-    a.stats = take(attn_fused_scratch_bytes(a.chunk, L));
+    a.stats = take(attn_fused_scratch_bytes(a.chunk, L, ordered));
     a.gemm = off;
     a.total = off + 256;
     return a;
@@ -542,12 +542,17 @@ uint32_t attn_kernel(int64_t M, int64_t N, int64_t K, uint32_t flags) {
     return (k == AMX_GEMM_ROWS && (flags & kKernelMask) == AMX_GEMM_AUTO) ? AMX_GEMM_TC : k;
 }
 // Whether a call runs the fused kernel: asked for the FP4 kernel, or AUTO from 2^25 multiply-adds per product and head on
-// (512 tokens at head dimension 128; below, a batched launch of each step is as fast and the kernel's two passes do
-// not fill their pipeline).
+// (512 tokens at head dimension 128; below, a batched launch of each step is as fast and the kernel's passes do not
+// fill their pipeline).
 bool attn_runs_fused(int64_t L, int64_t d, uint32_t flags) {
     flags &= ~AMX_ATTN_CAUSAL;
     if (!attn_fused_supported(L, d)) return false;
     return flags == AMX_GEMM_FP4 || (flags == AMX_GEMM_AUTO && (double)L * (double)L * (double)d >= 33554432.0);
+}
+// The form of its statistics (attention_fp4.cu).  Online only where no other kernel computes the same call: whole blocks at
+// head dimension 128, under AUTO from 2^28 multiply-adds on.  Elsewhere the map's bits are those of the stored path.
+bool attn_ordered(int64_t L, int64_t d, uint32_t flags) {
+    return d != 128 || L % 128 || ((flags & kKernelMask) == AMX_GEMM_AUTO && (double)L * (double)L * (double)d < 268435456.0);
 }
 // Short sequences used to run on the exact kernel under AUTO: there a scale the FP4 kernel cannot represent must not be
 // lost, and the casts' count decides on the device.  (From 2^28 on the FP4 kernel was AUTO's choice without this check.)
@@ -561,14 +566,15 @@ extern "C" size_t amx_attention_workspace_bytes(int64_t L, int64_t d) {
     size_t n = attn_layout_stored(L, d, true).total;
     const size_t m = attn_layout_stored(L, d, false).total;
     if (m > n) n = m;
-    if (attn_fused_supported(L, d) && attn_layout_fused(L, d).total > n) n = attn_layout_fused(L, d).total;
+    for (int ordered = 0; ordered < 2; ++ordered)
+        if (attn_fused_supported(L, d) && attn_layout_fused(L, d, ordered).total > n) n = attn_layout_fused(L, d, ordered).total;
     return n;
 }
 
 namespace {
 AttnLayout attn_layout_for(int64_t L, int64_t d, uint32_t flags) {
     flags &= ~AMX_ATTN_CAUSAL;
-    if (attn_runs_fused(L, d, flags)) return attn_layout_fused(L, d);
+    if (attn_runs_fused(L, d, flags)) return attn_layout_fused(L, d, attn_ordered(L, d, flags));
     return attn_layout_stored(L, d, attn_kernel(L, L, d, flags) == AMX_GEMM_TC && attn_kernel(L, d, L, flags) == AMX_GEMM_TC);
 }
 }  // namespace
@@ -638,8 +644,8 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
             float* oh = o + (size_t)h0 * L * d;
             if (rc == AMX_OK)
                 rc = attn_fused({w + a.pq, hc * Lp, chunk_max * Lp, 0}, {w + a.pk, kvc * Lp, chunk_max * Lp, 0},
-                                {w + a.pv, kvc * 128, chunk_max * 128, 0}, (int)hc, L, d, alpha, causal, w + a.stats, oh, words, st,
-                                nullptr, nullptr, nullptr, nullptr, kv_group, gated ? words + 1 : nullptr);
+                                {w + a.pv, kvc * 128, chunk_max * 128, 0}, (int)hc, L, d, alpha, causal, attn_ordered(L, d, flags),
+                                w + a.stats, oh, words, st, nullptr, nullptr, nullptr, nullptr, kv_group, gated ? words + 1 : nullptr);
             if (rc == AMX_OK && gated) {
                 const size_t plane_q = gemm_fp4_plane_bytes(chunk_max * Lp, d), plane_v = gemm_fp4_plane_bytes(chunk_max * 128, L);
                 rc = attn_exact({w + a.pq, w + a.pq + plane_q, w + a.qs}, {w + a.pk, w + a.pk + plane_q, w + a.ks},
@@ -718,7 +724,7 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     if (flags & ~AMX_ATTN_CAUSAL) return AMX_ERR_FLAGS;
     if (L <= 0 || d != 128 || L % 128 || !attn_fused_supported(L, d)) return AMX_ERR_SHAPE;
     if (!q || !k || !v || !o || !p_prepared) return AMX_ERR_NULL;
-    const AttnLayout a = attn_layout_fused(L, d);
+    const AttnLayout a = attn_layout_fused(L, d, false);
     if (!workspace || workspace_bytes < amx_attention_workspace_bytes(L, d) || prepared_bytes < amx_prepared_bytes(L, L, 32, 0))
         return AMX_ERR_WORKSPACE;
     if (!aligned(workspace, kAlign) || !aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(o, 16) ||
@@ -734,7 +740,7 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
             return AMX_ERR_CUDA;
     }
     // one head through the launch sequence of amx_attention: casts of Q, K (along head_dim) and V (along the
-    // sequence), then the two passes
+    // sequence), then the passes
     int* words = reinterpret_cast<int*>(w + a.gemm);
     if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
     const PrepOperand op[2] = {gemm_fp4_cast_operand(q, d, L, d, false, nullptr, w + a.qs, w + a.pq),
@@ -743,7 +749,7 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(v, 1, L, d, 128, 128, w + a.vs, w + a.pv, st, nullptr);
     if (rc != AMX_OK) return rc;
     return attn_fused({w + a.pq, L, L, 0}, {w + a.pk, L, L, 0}, {w + a.pv, 128, 128, 0}, 1, L, d, 1.0f / sqrtf((float)d), causal,
-                      w + a.stats, o, words, st, p_bf16, p_codes, p_scales, p_prepared);
+                      false, w + a.stats, o, words, st, p_bf16, p_codes, p_scales, p_prepared);
 }
 
 extern "C" int amx_gemm_status(const void* workspace, void* stream) {

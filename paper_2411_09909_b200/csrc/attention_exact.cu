@@ -2,7 +2,8 @@
 // casting Q, K or V met a scale that kernel cannot represent (see to_ue4m3: 15 or more binades below its row's largest).
 // The decision is taken on the device, from the count the casts leave in the workspace; without such a scale - every
 // input but adversarial ones - the launch returns at once.  Same arithmetic as everywhere: products of exactly decoded
-// values with fp32 accumulation, softmax in fp32, the normalised map rounded to bf16 and cast with groups of 32 keys.
+// values with fp32 accumulation, softmax in fp32 by softmax_math.cuh's expressions and order of additions, the normalised map
+// rounded to bf16 and cast with groups of 32 keys.
 //
 // A block owns 16 query rows of one head: their logits stay in shared memory as fp32, are normalised, cast and decoded
 // again in place, and multiplied with V.  Nothing is tuned: it runs where correctness needs it.
@@ -10,6 +11,7 @@
 
 #include "cast_math.cuh"
 #include "gemm.cuh"
+#include "softmax_math.cuh"
 
 namespace amx {
 namespace {
@@ -61,15 +63,20 @@ attention_exact_kernel(const ExactOperand q, const ExactOperand k, const ExactOp
         float mx = -INFINITY, sum = 0.f;
         for (int64_t i = lane; i < vis; i += 32) mx = fmaxf(mx, s[i]);
         for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, x));
-        for (int64_t i = lane; i < vis; i += 32) sum += expf(s[i] - mx);
-        for (int x = 16; x > 0; x >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, x);
+        const float nm = softmax::neg_max_log2e(mx);
+        for (int64_t g0 = 0; g0 < L / 32; g0 += 32) {            // keys in order within a group, a tree over 32 groups
+            float part = 0.f;
+            for (int64_t a = (g0 + lane) * 32; a < min(vis, (g0 + lane + 1) * 32); ++a) part += softmax::exp_rel(s[a], nm);
+            for (int x = 16; x > 0; x >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, x);
+            sum += part;
+        }
         const float inv = 1.0f / sum;
         for (int64_t g = lane; g < L / 32; g += 32) {            // a lane per group of 32 keys
             uint32_t w[16], nib[4];
             for (int i = 0; i < 16; ++i) {
                 const int64_t a = g * 32 + 2 * i;
-                const __nv_bfloat162 h = __floats2bfloat162_rn(a < vis ? expf(s[a] - mx) * inv : 0.f,
-                                                               a + 1 < vis ? expf(s[a + 1] - mx) * inv : 0.f);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(a < vis ? softmax::exp_rel(s[a], nm) * inv : 0.f,
+                                                               a + 1 < vis ? softmax::exp_rel(s[a + 1], nm) * inv : 0.f);
                 w[i] = *reinterpret_cast<const uint32_t*>(&h);
             }
             const float sc = e5m2_to_float(cast::cast_nonneg_group(w, nib));

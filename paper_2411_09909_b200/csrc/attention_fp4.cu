@@ -3,11 +3,21 @@
 // are a large share of the prefill work).  Neither the logits nor the attention map ever reach global memory.
 //
 // What is quantized is the NORMALISED map P = softmax(Q K^T / sqrt(d)), rounded to bf16, with groups of 32 along
-// the keys.  Its scales depend on the final row maximum and sum, so the product Q K^T runs twice:
-//   pass 1  S tiles -> per-row maximum and sum of exponentials (kept per thread over all key tiles of a row);
-//   pass 2  S tiles again -> P tile = 2^(s - max) / sum, rounded to bf16 and cast to AMXFP4 in registers (P has no
-//           negative element: one sign plane), written to shared memory in the layout the MMA reads, its scale
-//           factors copied to tensor memory, and O += P V on the tensor cores in the same kernel.
+// the keys.  Its scales depend on the final row maximum and sum, so the product Q K^T runs in a pass of its own for the
+// statistics before the last pass:
+//   map    S tiles -> P tile = 2^(s - max) / sum, rounded to bf16 and cast to AMXFP4 in registers (P has no negative
+//          element: one sign plane), written to shared memory in the layout the MMA reads, its scale factors copied to
+//          tensor memory, and O += P V on the tensor cores in the same kernel.
+// The statistics come in two forms.  One rounding of a row's sum or of an exponent decides now and then which bf16 value a
+// probability takes, that value which step of E5M2 its group's scale takes, and that a quarter of the group's magnitude:
+//   ordered  (ragged lengths, head dimension 64, short sequences: wherever these products also exist with the logits in
+//            global memory) a pass for the maxima, then one for the sums: same argument t log2(e) - max log2(e) with
+//            t = alpha s rounded, same order of additions as softmax_math.cuh, hence the bits of the stored path.  The
+//            logits are the same numbers too: a sum of head-dimension-many products of E2M1 codes under E5M2 scales needs
+//            fewer than 24 bits.  (Online sums moved up to 3 rows of 33792 at 32 over 8 heads x 1056, now and then an element
+//            by half of the result's rms; the second statistics pass takes 12 of 75 us there, 130 of 680 at 4000 keys.)
+//   online   (long whole blocks at head dimension 128) one pass keeps a running maximum and a rescaled sum, log2(e) folded
+//            into the column factors: a pass less.
 // Both products use the sign split of the GEMM (gemm_fp4.cu): S = Q+K+ + Q+K- + Q-K+ + Q-K- (8 block-scaled MMAs
 // per 128 x 128 tile at K = 128, 4 at K = 64), O += P V+ + P V- (4 MMAs per tile of 128 keys).
 // Any sequence length: every head's Q and K rows are padded to whole 128-row blocks (zero scale factors, zero row
@@ -16,25 +26,26 @@
 // issued) and O is 64 columns wide.
 //
 // One persistent CTA per SM walks over (head, block of 128 queries) items; per item it loops over the key tiles:
-//   warp 0      TMA: the item's Q tile; per key tile the K tile and (pass 2) the V^T tile, {+, -} planes and scale
-//               factors each, into rings of kStages stages
-//   warp 1      issues the MMAs of the logits as far ahead as there are accumulators (three in pass 1, where the third
-//               takes O's columns, two in pass 2)
-//   warp 2      the per-key column factors alpha * log2(e) * 2^(K row offset) of the tile
-//   warp 3      (pass 2) issues the MMAs of P V.  A warp of its own: issued by warp 1 in turn with the logits, every wait
+//   warp 0      TMA: the item's Q tile; per key tile the K tile and (map pass) the V^T tile, {+, -} planes and scale
+//               factors each, into rings of stages
+//   warp 1      issues the MMAs of the logits as far ahead as there are accumulators (three in the passes for online
+//               statistics and maxima, where the third takes O's columns, else two)
+//   warp 2      the per-key column factors alpha * 2^(K row offset) of the tile (online: times log2(e))
+//   warp 3      (map pass) issues the MMAs of P V.  A warp of its own: issued by warp 1 in turn with the logits, every wait
 //               for P held up the next logits (32 heads x 8192 x 128: 2198 us against 1994)
-//   warps 4-    epilogue, groups of eight warps (three in pass 1, two in pass 2): group g takes the key tiles with
+//   warps 4-    epilogue, groups of eight warps (as many as accumulators): group g takes the key tiles with
 //               (tile count) % groups == g, so the groups are in different phases of their tiles (tensor-memory loads
 //               and maxima in one, exponentials in the other) and keep both the issue slots and the special-function
 //               unit busy; a thread owns one query row and 64 keys of its tiles: tensor memory -> registers, softmax
-//               arithmetic, the cast, stores to shared memory.  (A third group in pass 2 has no accumulator of its own to
-//               work on: 2023 us against 1994.)
+//               arithmetic, the cast, stores to shared memory.  (A third group in the map pass has no accumulator of its own
+//               to work on: 2023 us against 1994.)
 //   after the last key tile of an item the epilogue warps read out O, rescale by the rows' powers of two and store.
 // Scale factors go from global to shared memory with the tiles and on to tensor memory by the issuing warps
 // (tcgen05.cp, ordered with the MMAs): four warps that carried them through registers were a sixth of all instructions.
-// What bounds it (32 heads x 8192): per key tile the tensor cores need 600 cycles in pass 1 and 900 in pass 2, the
-// special-function unit 1024 in each, the issue slots 800 and 1480; a tile takes 1500 and 2250.
-// Tensor memory: S0, S1, O (128 columns each), scale factors of Q (16), of kStages K/V^T stages (32 each), of the
+// What bounds it (32 heads x 8192): per key tile the tensor cores need 600 cycles in the statistics pass and 900 in the
+// map pass, the special-function unit 1024 in each, the issue slots 800 and 1480; a tile takes 1500 and 2250.  Neither unit
+// is within 1.45 times of its limit: the rest is waiting between the phases of a group's tiles.
+// Tensor memory: S0, S1, O (128 columns each), scale factors of Q (16), of three K and V^T stages or six of K (96), of the
 // two P tiles (8 each): 512 columns.  Every wait is bounded; on a timeout all roles run their loops out without
 // work, tensor memory is released and the status word reports AMX_ERR_TIMEOUT.
 #include <cuda_bf16.h>
@@ -42,6 +53,7 @@
 #include "cast_math.cuh"
 #include "fp4_operand.cuh"
 #include "gemm.cuh"
+#include "softmax_math.cuh"
 #include "tcgen05.cuh"
 
 namespace amx {
@@ -52,27 +64,37 @@ using namespace fp4;
 
 constexpr int BM = 128, BNK = 128;                   // queries per item, keys per tile
 constexpr int kVRows = 128;                           // rows of one head of V^T (padded at head dimension 64)
-constexpr int kStages = 3;
+enum Pass { kPassStats, kPassMapOnline, kPassMax, kPassSum, kPassMapOrdered };
+__host__ __device__ constexpr bool is_map(int pass) { return pass == kPassMapOnline || pass == kPassMapOrdered; }
+__host__ __device__ constexpr bool is_ordered(int pass) { return pass >= kPassMax; }
+// Stages of the K and V^T rings.  Without V^T its place holds three more of K: a statistics pass
+// waits for loads (32 heads x 8192: 1946 -> 1897 us).
+constexpr int kStages = 3, kStagesMax = 6;
+__host__ __device__ constexpr int k_stages(int pass) { return is_map(pass) ? kStages : kStagesMax; }
 // Ring of the per-tile column factors.  A group may still read those of tile j when it has released j's accumulator and the
-// other groups theirs, so the MMAs may be done up to tile j + 5 and the writer (warp 2), kStages ahead of those, at tile
-// j + 8: 16 slots never collide and need no barrier of their own.
+// other groups theirs, so the MMAs may be done up to tile j + 5 and the writer (warp 2), kStagesMax ahead of those, at tile
+// j + 11: 16 slots never collide and need no barrier of their own.
 constexpr int kKcRing = 16;
 constexpr int kFirstEpi = 4;                          // warps 0-3: TMA, logits MMAs, column factors, P V MMAs
 constexpr int kOWarps = 16;                           // of the epilogue warps, those that read out O
-__host__ __device__ constexpr int epi_groups(int pass) { return pass == 1 ? 3 : 2; }
-__host__ __device__ constexpr int s_buffers(int pass) { return pass == 1 ? 3 : 2; }   // pass 1: the third in O's columns
-static_assert(s_buffers(1) <= epi_groups(1) && s_buffers(2) <= epi_groups(2), "a group meets every phase of its s_full barrier");
+// Epilogue groups, each with an accumulator (the third in O's columns).  The sums take two: a thread then meets the key tiles
+// of one parity, four of every eight, in the order in which the stored path's tree adds them.
+__host__ __device__ constexpr int epi_groups(int pass) { return pass == kPassStats || pass == kPassMax ? 3 : 2; }
+__host__ __device__ constexpr int s_buffers(int pass) { return epi_groups(pass); }   // (a group meets every phase of its s_full barrier)
 __host__ __device__ constexpr int threads(int pass) { return (kFirstEpi + 8 * epi_groups(pass)) * 32; }
-constexpr int kParts = 2 * epi_groups(1);             // partial row statistics of pass 1
+constexpr int kParts = 2 * epi_groups(kPassStats);    // partial row statistics: a thread's columns of its group's tiles
+static_assert(epi_groups(kPassMax) == epi_groups(kPassStats), "kParts");
+constexpr int kSumTiles = 8, kSumParts = 8;           // ordered sums: per 8 key tiles {even, odd tiles} x 4 groups of a tile
+constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kPlane = 128 * 64;                      // one sign plane of a 128 x 128 tile: 64-byte rows
 constexpr int kTileBytes = 2 * kPlane;                // {+, -}
 constexpr int kSfBytes = 4 * kSfChunk;                // a tile's scale factors: {+, -} x two K steps of 64
 // tensor-memory columns
 constexpr uint32_t kColS = 0, kColO = 256, kColSfQ = 384, kColSfKV = 400, kColSfP = 496, kTmemCols = 512;
-static_assert(kColSfKV + kStages * 32 == kColSfP && kColSfP + 2 * 8 == kTmemCols, "tensor-memory budget");
+static_assert(kStagesMax * 16 == kStages * 32 && kColSfKV + kStages * 32 == kColSfP && kColSfP + 2 * 8 == kTmemCols, "tensor-memory budget");
 
 struct __align__(16) Control {
-    uint64_t q_full, q_empty, k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages], s_full[3], s_empty[3], p_full[2], p_empty[3], o_full, o_empty;
+    uint64_t q_full, q_empty, k_full[kStagesMax], k_empty[kStagesMax], v_full[kStages], v_empty[kStages], s_full[3], s_empty[3], p_full[2], p_empty[3], o_full, o_empty;
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -83,14 +105,14 @@ struct Smem {
     static constexpr int kOffQ = 0;
     // K and V^T tiles, each with its scale factors, in rings of their own: a K stage is free as soon as its logits are
     // computed, two tiles before the V^T tile of the same keys is used
-    static constexpr int kOffK = kTileBytes, kOffV = kOffK + kStages * kTileBytes;
-    static constexpr int kOffP = kOffV + (PASS == 2 ? kStages * kTileBytes : 0);  // two P planes (pass 2)
-    static constexpr int kOffSfP = kOffP + (PASS == 2 ? 2 * kPlane : 0);          // two buffers x two 512-byte chunks
-    static constexpr int kOffSfQ = kOffSfP + (PASS == 2 ? 2 * 2 * 512 : 0);
-    static constexpr int kOffSfK = kOffSfQ + kSfBytes, kOffSfV = kOffSfK + kStages * kSfBytes;
-    static constexpr int kOffKc = kOffSfV + (PASS == 2 ? kStages * kSfBytes : 0); // 128 column factors per slot
+    static constexpr int kOffK = kTileBytes, kOffV = kOffK + k_stages(PASS) * kTileBytes;
+    static constexpr int kOffP = kOffV + (is_map(PASS) ? kStages * kTileBytes : 0);  // two P planes (map pass)
+    static constexpr int kOffSfP = kOffP + (is_map(PASS) ? 2 * kPlane : 0);          // two buffers x two 512-byte chunks
+    static constexpr int kOffSfQ = kOffSfP + (is_map(PASS) ? 2 * 2 * 512 : 0);
+    static constexpr int kOffSfK = kOffSfQ + kSfBytes, kOffSfV = kOffSfK + k_stages(PASS) * kSfBytes;
+    static constexpr int kOffKc = kOffSfV + (is_map(PASS) ? kStages * kSfBytes : 0); // 128 column factors per slot
     static constexpr int kOffTab = kOffKc + kKcRing * 512;                        // per scale byte: see cast_group
-    static constexpr int kOffCtl = kOffTab + (PASS == 2 ? 128 * 8 : 0);
+    static constexpr int kOffCtl = kOffTab + (is_map(PASS) ? 128 * 8 : 0);
     static constexpr int kBytes = kOffCtl + 512 + 1024;                           // + Control + alignment slack
 };
 static_assert(sizeof(Control) <= 512, "Control must fit its reserved space");
@@ -145,10 +167,12 @@ struct Params {
     int64_t L, Lp;           // sequence length, and padded to whole blocks of 128
     float alpha;
     const int* gate;         // not NULL: nothing is done when this word is nonzero (the caller runs the exact kernel then)
-    float2* part;            // [heads * Lp][kParts]: per row and key-group column {max, sum of 2^(t - max)}, base-2 units
-    float* O;                // pass 2 out: [heads][L][head dimension]
+    float2* part;            // online: [heads * Lp][kParts]: per row {max, sum of 2^(t - max)}, base-2 units
+    float* row_max;          // ordered: [kParts][heads * Lp]: maxima of t = alpha s
+    float* sums;             // ordered: [heads][tiles / kSumTiles][kSumParts][Lp]: sums of exp(t - max) of a key group's tiles
+    float* O;                // map pass out: [heads][L][head dimension]
     int* status;
-    // optional outputs of pass 2 for head 0 of the launch (verification): the bf16 map the cast started from
+    // optional outputs of the online map pass for head 0 of the launch (verification): the bf16 map the cast started from
     // [L][L/2 words], canonical codes [L][L/32] x 16 bytes, scale bytes, and the prepared form of P (plane, scale
     // factors, row words)
     uint4 *p_bits, *p_codes, *p_plane;
@@ -168,7 +192,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     grid_dependency_wait();
     using S_ = Smem<PASS>;
     constexpr bool CAUSAL = MASK == kMaskCausal;
-    constexpr int kGroups = epi_groups(PASS), kSBufs = s_buffers(PASS);
+    constexpr int kGroups = epi_groups(PASS), kSBufs = s_buffers(PASS), kKStages = k_stages(PASS);
+    constexpr uint32_t kSfStage = 96 / kKStages;          // tensor-memory columns of a stage's scale factors: K, then V^T
     constexpr int kQkSteps = HD / 64;                     // MMAs along the head dimension per sign pair
     if (p.gate && *p.gate != 0) return;                   // uniform over the grid: nothing was set up yet
     extern __shared__ uint8_t smem_raw[];
@@ -188,9 +213,11 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     if (threadIdx.x == 0) {
         mbar_init(&ctl->q_full, 1);
         mbar_init(&ctl->q_empty, 1);
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < kKStages; ++s) {
             mbar_init(&ctl->k_full[s], 2);                       // the copies and the column factors
             mbar_init(&ctl->k_empty[s], 1);
+        }
+        for (int s = 0; s < kStages; ++s) {
             mbar_init(&ctl->v_full[s], 1);
             mbar_init(&ctl->v_empty[s], 1);
         }
@@ -208,7 +235,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     uint2* scale_tab = reinterpret_cast<uint2*>(sm + S_::kOffTab);
-    if (PASS == 2 && threadIdx.x >= 128 && threadIdx.x < 256) scale_tab[threadIdx.x - 128] = scale_entry(threadIdx.x - 128);
+    if (is_map(PASS) && threadIdx.x >= 128 && threadIdx.x < 256) scale_tab[threadIdx.x - 128] = scale_entry(threadIdx.x - 128);
     if (warp == 1) tmem_alloc(&ctl->tmem_base, kTmemCols);
     tc_fence_before();
     __syncthreads();
@@ -236,9 +263,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 tma_load_3d(sm + S_::kOffQ, &tm_q, 0, (int)(p.q_row0 + (int64_t)h * p.Lp + m_blk * BM), 0, &ctl->q_full);
                 const int T = tiles_of(m_blk);
                 for (int j = 0; j < T; ++j, ++it) {
-                    const int s = it % kStages;
-                    const uint32_t freed = ((it / kStages) - 1) & 1;
-                    if (it >= kStages && !mbar_wait(&ctl->k_empty[s], freed, &ctl->abort, p.status)) {
+                    const int s = it % kKStages;
+                    const uint32_t freed = ((it / kKStages) - 1) & 1;
+                    if (it >= kKStages && !mbar_wait(&ctl->k_empty[s], freed, &ctl->abort, p.status)) {
                         ok = false;
                         break;
                     }
@@ -246,7 +273,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     load_sf(S_::kOffSfK + s * kSfBytes, p.sfk, k_row0 + j * BNK, p.nk64_k, 0, &ctl->k_full[s]);
                     tma_load_3d(sm + S_::kOffK + s * kTileBytes, &tm_k, 0, (int)(k_row0 + j * BNK), 0, &ctl->k_full[s]);
                     ++n_k;
-                    if (PASS == 2) {
+                    if (is_map(PASS)) {
                         if (it >= kStages && !mbar_wait(&ctl->v_empty[s], freed, &ctl->abort, p.status)) {
                             ok = false;
                             break;
@@ -260,15 +287,15 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
             // after a timeout: let the copies already in flight land before shared memory is released
             if (ctl->abort) {
-                for (int i = max(0, n_k - kStages); i < n_k; ++i)
-                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->k_full[i % kStages], (i / kStages) & 1); ++n) {}
+                for (int i = max(0, n_k - kKStages); i < n_k; ++i)
+                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->k_full[i % kKStages], (i / kKStages) & 1); ++n) {}
                 for (int i = max(0, n_v - kStages); i < n_v; ++i)
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->v_full[i % kStages], (i / kStages) & 1); ++n) {}
                 if (ii > 0)
                     for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->q_full, (ii - 1) & 1); ++n) {}
             }
         }
-    } else if (warp == 1 || (PASS == 2 && warp == 3)) {
+    } else if (warp == 1 || (is_map(PASS) && warp == 3)) {
         // ---------------------------------------------------------------------------------- MMA issuers
         // The whole warp runs the loops (addresses stay warp-uniform); one elected lane issues.
         const uint32_t base = smem_u32(sm);
@@ -298,7 +325,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     if (!ok) break;
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint32_t kt = k_lo + (uint32_t)s * (kTileBytes >> 4), sfk = tmem + kColSfKV + s * 32;
+                        const uint32_t kt = k_lo + (uint32_t)s * (kTileBytes >> 4), sfk = tmem + kColSfKV + s * kSfStage;
                         if (j == 0) copy_sf(tmem + kColSfQ, sfq_lo, kQkSteps);
                         copy_sf(sfk, sfk_lo + (uint32_t)s * (kSfBytes >> 4), kQkSteps);
                         uint32_t acc = 0;
@@ -318,12 +345,12 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         if (j == T - 1) mma_commit(&ctl->q_empty);   // the Q tile is free for the next item
                     }
                     __syncwarp();
-                    if (++s == kStages) s = 0, full ^= 1;
+                    if (++s == kKStages) s = 0, full ^= 1;
                     if (++b == kSBufs) b = 0, freed ^= 1;
                     if (++g == kGroups) g = 0;
                 }
             }
-        } else if (PASS == 2) {
+        } else if (is_map(PASS)) {
             // O (+)= P V: P from the epilogue warps (shared memory + scale-factor chunks)
             const uint32_t p_lo = desc_lo(base + S_::kOffP), v_lo = desc_lo(base + S_::kOffV);
             const uint32_t sfp_lo = sf_lo(base + S_::kOffSfP), sfv_lo = sf_lo(base + S_::kOffSfV);
@@ -340,7 +367,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     tc_fence_after();
                     if (elect_one()) {
                         const uint32_t vt = v_lo + (uint32_t)s * (kTileBytes >> 4), pt = p_lo + (uint32_t)b * (kPlane >> 4);
-                        const uint32_t sfp = tmem + kColSfP + b * 8, sfv = tmem + kColSfKV + s * 32 + 16;
+                        const uint32_t sfp = tmem + kColSfP + b * 8, sfv = tmem + kColSfKV + s * kSfStage + 16;
                         copy_sf(sfv, sfv_lo + (uint32_t)s * (kSfBytes >> 4), 2);
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk) tmem_cp_32x128b_warpx4(sfp + kk * 4, desc_sf(sfp_lo + (uint32_t)((b * 2 + kk) * 512 >> 4)));
@@ -368,18 +395,18 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         // ---------------------------------------------------------------------------------- column factors
         int it = 0, ii = 0;
         bool ok = true;
-        const float unit = p.alpha * 1.4426950408889634f;
+        const float unit = is_ordered(PASS) ? p.alpha : p.alpha * kLog2e;
         for (int id = item_id(ii); id < n_items; id = item_id(++ii)) {
             const int T = tiles_of(item_m(id));
             const int4* words = reinterpret_cast<const int4*>(p.k_words + p.k_row0 + (int64_t)(item_head(id) / p.kv_group) * p.Lp) + lane;
             for (int j = 0; j < T; ++j, ++it, words += 32) {
                 const int4 w = __ldg(words);
                 auto factor = [&](int word) { return unit * __uint_as_float((uint32_t)(row_word_exp(word) + 127) << 23); };
-                if (ok && it >= kStages) ok = mbar_wait(&ctl->k_empty[it % kStages], ((it / kStages) - 1) & 1, &ctl->abort, p.status);
+                if (ok && it >= kKStages) ok = mbar_wait(&ctl->k_empty[it % kKStages], ((it / kKStages) - 1) & 1, &ctl->abort, p.status);
                 if (!ok) continue;
                 reinterpret_cast<float4*>(kc_all + (it % kKcRing) * 128)[lane] = make_float4(factor(w.x), factor(w.y), factor(w.z), factor(w.w));
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->k_full[it % kStages]);
+                if (lane == 0) mbar_arrive(&ctl->k_full[it % kKStages]);
             }
         }
     } else if (warp >= kFirstEpi) {
@@ -403,10 +430,41 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             const int64_t grow = (int64_t)h * p.Lp + m;              // row of the launch's stacked heads
             const int a_exp = row_word_exp(__ldg(p.q_words + p.q_row0 + grow));
             const float ra = __uint_as_float((uint32_t)(a_exp + 127) << 23);
-            // pass 2: the row's statistics, merged from the partial results of pass 1 in a fixed order
-            float neg_mx = 0.f, inv = 0.f;
+            const int T = tiles_of(m_blk);
+            // the row's statistics, merged from the partial results of the passes before in a fixed order: the exponent of
+            // an element is u x row_unit + neg_mx
+            float row_unit = ra, neg_mx = 0.f, inv = 0.f;
             int kmax = 0;
-            if (PASS == 2) {
+            if (PASS == kPassSum || PASS == kPassMapOrdered) {
+                float mx = -INFINITY;
+                const float* rm = p.row_max + grow;
+#pragma unroll
+                for (int i = 0; i < kParts; ++i) mx = fmaxf(mx, __ldg(rm + i * (int64_t)p.heads * p.Lp));
+                row_unit = ra * kLog2e;
+                neg_mx = softmax::neg_max_log2e(mx);
+                if (PASS == kPassMapOrdered) {
+                    // the stored path's order: over 32 groups a tree by strides 16, 8, 4, 2, 1 (the first two inside `sums`),
+                    // then along the row
+                    float sum = 0.f;
+                    const float* sp = p.sums + (int64_t)h * ((p.m_tiles + kSumTiles - 1) / kSumTiles) * kSumParts * p.Lp + m;
+                    for (int t0 = 0; t0 < T; t0 += kSumTiles, sp += kSumParts * p.Lp) {
+                        float c[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            c[i] = __ldg(sp + i * p.Lp);
+                            if (t0 + 1 < T) c[i] += __ldg(sp + (4 + i) * p.Lp);
+                        }
+                        sum += (c[0] + c[2]) + (c[1] + c[3]);
+                    }
+                    inv = 1.0f / sum;
+                    // the group of the row's largest element has the row's largest scale (one bf16 step above: the
+                    // approximate exponential is not promised to be monotonic)
+                    float ip, in;
+                    const uint32_t top = __bfloat16_as_ushort(__float2bfloat16_rn(softmax::exp_rel(mx, neg_mx) * inv));
+                    kmax = scale_key(cast::group_scales(top + 1, ip, in) & 0xFFu);
+                }
+            }
+            if (PASS == kPassMapOnline) {
                 const float4* pp = reinterpret_cast<const float4*>(p.part + grow * kParts);
                 float4 a[kParts / 2];                                 // {max, sum, max, sum}
                 float mx = -INFINITY, sum = 0.f;
@@ -428,8 +486,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 kmax = scale_key(sc & 0xFFu);
                 if (p.p_words && h == 0 && (e >> 2) == 0) p.p_words[m] = row_word(kmax, kRowHasPos);
             }
-            float run_mx = -INFINITY, run_sum = 0.f;                  // pass 1: over this thread's columns of its tiles
-            const int T = tiles_of(m_blk);
+            float run_mx = -INFINITY, run_sum = 0.f;                  // statistics: over this thread's columns of its tiles
+            float even[2] = {}, odd[2] = {};                          // ordered sums: every other of its tiles, per key group
             for (; it < it0 + T; it += kGroups, ++n) {
                 const int j = it - it0, b = it & 1;                                 // P buffer
                 const uint32_t s_col = tq + kColS + (it % kSBufs) * 128;
@@ -438,8 +496,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 tc_fence_after();
                 // (the tile's column factors were stored before warp 2 arrived on the stage's barrier,
                 // which the MMA warp waited for before it issued what s_full reports as complete)
-                // u = accumulator x (alpha log2(e) 2^(K row offset)): the logit in base-2 units up to the query row's
-                // power of two ra, by which multiplying is exact: t = u ra.  (Packed fp32 pairs: same roundings as the
+                // u = accumulator x column factor: the logit (online: in base-2 units) up to the query row's power of two
+                // ra, by which multiplying is exact: t = u ra.  (Packed fp32 pairs: same roundings as the
                 // scalar operations, half the instructions.)
                 uint32_t acc[32];
                 uint64_t u2[16];
@@ -470,9 +528,22 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         }
                     }
                 };
-                const uint64_t ra2 = cast::pack_f32x2(__float_as_uint(ra), __float_as_uint(ra));
+                const uint64_t ra2 = cast::pack_f32x2(__float_as_uint(row_unit), __float_as_uint(row_unit));
                 auto work = [&](int cg) {                             // one 32-key group, from u2
-                    if (PASS == 1) {
+                    if (PASS == kPassSum) {
+                        const uint64_t nm2 = cast::pack_f32x2(__float_as_uint(neg_mx), __float_as_uint(neg_mx));
+                        float sum = 0.f;                              // in the order of the keys
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            float t0, t1;
+                            cast::unpack_f32x2(cast::fma_f32x2(u2[c], ra2, nm2), t0, t1);
+                            sum += exp2_approx(t0);
+                            sum += exp2_approx(t1);
+                        }
+                        // of every eight tiles this thread's are numbers 0 .. 3: 0 + 2 and 1 + 3 first
+                        if ((j >> 1) & 1) odd[cg & 1] += sum;
+                        else even[cg & 1] += sum;
+                    } else if (!is_map(PASS)) {
                         float u[32];
 #pragma unroll
                         for (int c = 0; c < 16; ++c) cast::unpack_f32x2(u2[c], u[2 * c], u[2 * c + 1]);
@@ -481,6 +552,10 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         for (int c = 4; c < 32; ++c) c4[c & 3] = fmaxf(c4[c & 3], u[c]);
                         const float cm = fmaxf(fmaxf(c4[0], c4[1]), fmaxf(c4[2], c4[3]));
                         const float nmx = fmaxf(run_mx, cm * ra);
+                        if (PASS == kPassMax) {
+                            run_mx = nmx;
+                            return;
+                        }
                         // 2^(-inf) = 0 on the first tile; a maximum still at -inf (everything masked so far) must
                         // not meet itself in a difference
                         const float ref = nmx == -INFINITY ? 0.f : nmx;
@@ -522,7 +597,7 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                             make_uint4(nib[0], nib[1], nib[2], nib[3]);
                         *reinterpret_cast<uint16_t*>(sm + S_::kOffSfP + (b * 2 + (cg >> 1)) * 512 + (r & 31) * 16 + (r >> 5) * 4 +
                                                      (cg & 1) * 2) = (uint16_t)(up * 257u);
-                        if (p.p_plane && h == 0) {                    // verification outputs (head 0 of the launch)
+                        if (PASS == kPassMapOnline && p.p_plane && h == 0) {                    // verification outputs (head 0 of the launch)
                             const int64_t g = (int64_t)j * 4 + cg, v = m * (p.L / 32) + g;
                             p.p_plane[v] = make_uint4(nib[0], nib[1], nib[2], nib[3]);
                             *reinterpret_cast<uint16_t*>(p.p_sf + sf_row_offset(m, p.p_nk64) + sf_group_offset((int)g)) = (uint16_t)(up * 257u);
@@ -535,28 +610,39 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                         }
                     }
                 };
-                // pass 2 has the registers to take the second group before it works on the first, which frees the accumulator
-                // early (32 heads x 8192: 2001 -> 1981 us); pass 1, with 24 epilogue warps and three accumulators, has not
+                // two epilogue groups have the registers to take the second key group before they work on the first, which frees
+                // the accumulator early (32 heads x 8192: 2001 -> 1981 us); three have not
                 tmem_ld32(s_col + cg0 * 32, acc);
                 tmem_ld_wait();
                 scale_columns(cg0);
-                if (PASS == 1) work(cg0);
+                if (kGroups == 3) work(cg0);
                 tmem_ld32(s_col + (cg0 + 1) * 32, acc);
                 tmem_ld_wait();
                 release();
-                if (PASS == 2) work(cg0);
+                if (kGroups == 2) work(cg0);
                 scale_columns(cg0 + 1);
                 work(cg0 + 1);
-                if (PASS == 2) {
+                if (PASS == kPassSum && ((j >> 1) % 4 == 3 || j + 2 >= T)) {   // its last tile of these eight
+                    float* sp = p.sums + (((int64_t)h * ((p.m_tiles + kSumTiles - 1) / kSumTiles) + j / kSumTiles) * kSumParts +
+                                          (j & 1) * 4 + cg0) * p.Lp + m;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        sp[i * p.Lp] = even[i] + odd[i];
+                        even[i] = odd[i] = 0.f;
+                    }
+                }
+                if (is_map(PASS)) {
                     fence_proxy_async();                              // visible to the tensor core's reads
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->p_full[b]);
                 }
             }
             it0 += T;
-            if (PASS == 1) {
+            if (PASS == kPassStats) {
                 if (ok) p.part[grow * kParts + grp * 2 + half] = make_float2(run_mx, run_sum);
-            } else if (e < kOWarps) {
+            } else if (PASS == kPassMax) {
+                if (ok) p.row_max[(grp * 2 + half) * (int64_t)p.heads * p.Lp + grow] = run_mx;
+            } else if (is_map(PASS) && e < kOWarps) {
                 // O of the item: rows x (32 columns of the head dimension per thread), rescaled by 2^(row offset of P
                 // + row offset of V^T) - exact - and stored
                 if (ok) ok = mbar_wait(&ctl->o_full, ii & 1, &ctl->abort, p.status);
@@ -616,7 +702,7 @@ int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensor
         configured[dev] = true;
     }
     const int items = p.heads * p.m_tiles;
-    return launch_chained((double)p.heads * (double)p.L * (double)p.L <= 2.7e8,   // about 140 us in the second pass
+    return launch_chained((double)p.heads * (double)p.L * (double)p.L <= 2.7e8,   // about 140 us in the map pass
                           attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS), Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
 }
 
@@ -629,31 +715,42 @@ bool attn_fused_supported(int64_t L, int64_t d) {
 int64_t attn_fused_padded(int64_t L) { return (L + BM - 1) / BM * BM; }
 
 // per-row partial softmax statistics of the heads of one launch
-size_t attn_fused_scratch_bytes(int64_t heads, int64_t L) { return up256((size_t)heads * attn_fused_padded(L) * kParts * sizeof(float2)); }
+size_t attn_fused_scratch_bytes(int64_t heads, int64_t L, bool ordered) {
+    const int64_t rows = heads * attn_fused_padded(L), eights = (attn_fused_padded(L) / BNK + kSumTiles - 1) / kSumTiles;
+    return up256((size_t)rows * (ordered ? (kParts + eights * kSumParts) * sizeof(float) : kParts * sizeof(float2)));
+}
 
 namespace {
 template <int MASK, int HD>
-int launch_both(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev, int sms,
-                cudaStream_t st) {
-    const int rc = launch_pass<1, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
-    return rc != AMX_OK ? rc : launch_pass<2, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+int launch_ordered(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev, int sms,
+                   cudaStream_t st) {
+    int rc = launch_pass<kPassMax, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+    if (rc == AMX_OK) rc = launch_pass<kPassSum, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+    return rc != AMX_OK ? rc : launch_pass<kPassMapOrdered, MASK, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+}
+template <int MASK>
+int launch_online(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev, int sms,
+                  cudaStream_t st) {
+    const int rc = launch_pass<kPassStats, MASK, 128>(tm_q, tm_k, tm_v, p, dev, sms, st);
+    return rc != AMX_OK ? rc : launch_pass<kPassMapOnline, MASK, 128>(tm_q, tm_k, tm_v, p, dev, sms, st);
 }
 template <int HD>
 int launch_mask(int mask, const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const Params& p, int dev,
                 int sms, cudaStream_t st) {
-    return mask == kMaskCausal ? launch_both<kMaskCausal, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
-         : mask == kMaskTail   ? launch_both<kMaskTail, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
-                               : launch_both<kMaskNone, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
+    return mask == kMaskCausal ? launch_ordered<kMaskCausal, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
+         : mask == kMaskTail   ? launch_ordered<kMaskTail, HD>(tm_q, tm_k, tm_v, p, dev, sms, st)
+                               : launch_ordered<kMaskNone, HD>(tm_q, tm_k, tm_v, p, dev, sms, st);
 }
 }  // namespace
 
 // Attention for `heads` stacked heads whose operands were prepared ahead, Lp = attn_fused_padded(L) rows per head: q
 // (left-hand layout, K = d), k (right-hand layout), vt (right-hand layout, 128 rows of V^T per head, K = L).  O: fp32
-// [heads][L][d].  workspace: 256 bytes (status word).  dbg_*: optional verification outputs for head 0 (see Params).
+// [heads][L][d].  workspace: 256 bytes (status word).  ordered: the form of the statistics (see above); the online form takes
+// head dimension 128 and whole blocks only, and has the dbg_* outputs for head 0 (verification, see Params).
 int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, int64_t d, float alpha,
-               int causal, void* scratch, float* O, void* workspace, cudaStream_t st, void* dbg_bits, uint8_t* dbg_codes,
+               int causal, bool ordered, void* scratch, float* O, void* workspace, cudaStream_t st, void* dbg_bits, uint8_t* dbg_codes,
                uint8_t* dbg_scales, void* dbg_prepared, int kv_group, const int* gate) {
-    if (!attn_fused_supported(L, d) || heads <= 0 || q.row0 % 128 || k.row0 % 128 || vt.row0 % 128) return AMX_ERR_SHAPE;
+    if (!attn_fused_supported(L, d) || (!ordered && (d != 128 || L % BNK)) || heads <= 0 || q.row0 % 128 || k.row0 % 128 || vt.row0 % 128) return AMX_ERR_SHAPE;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
     static int sm_count[64] = {};
@@ -682,6 +779,8 @@ int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, i
     p.kv_group = kv_group > 0 ? kv_group : 1;
     p.L = L; p.alpha = alpha;
     p.part = static_cast<float2*>(scratch);
+    p.row_max = static_cast<float*>(scratch);
+    p.sums = p.row_max + kParts * heads * p.Lp;
     p.O = O;
     p.vec_o = aligned(O, 16);
     p.status = status;
@@ -696,6 +795,8 @@ int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, i
         p.p_codes = reinterpret_cast<uint4*>(dbg_codes);
         p.p_scales = reinterpret_cast<uint16_t*>(dbg_scales);
     }
+    if (!ordered) return causal ? launch_online<kMaskCausal>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st)
+                                : launch_online<kMaskNone>(tm_q, tm_k, tm_v, p, dev, sm_count[dev], st);
     const int mask = causal ? kMaskCausal : L % BNK ? kMaskTail : kMaskNone;
     return d == 128 ? launch_mask<128>(mask, tm_q, tm_k, tm_v, p, dev, sm_count[dev], st)
                     : launch_mask<64>(mask, tm_q, tm_k, tm_v, p, dev, sm_count[dev], st);

@@ -115,14 +115,16 @@ size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // C[m][n] = sum over `slices` partial products [slices][M][N], in slice order (defined with the bf16-decode kernel)
 int reduce_slices(const float* part, int slices, int64_t M, int64_t N, float* C, int64_t ld_c, cudaStream_t st,
                   const int* run_if_nonzero = nullptr);
-// Fused attention for head dimensions 128 and 64 (attention_fp4.cu): both products and the softmax in two launches, logits
-// and attention map never in global memory.  Operands prepared ahead, heads stacked row-wise, padded to whole blocks of 128.
+// Fused attention for head dimensions 128 and 64 (attention_fp4.cu): both products and the softmax in two or three launches,
+// logits and attention map never in global memory.  Operands prepared ahead, heads stacked row-wise, padded to whole blocks
+// of 128.
 bool attn_fused_supported(int64_t L, int64_t d);
 int64_t attn_fused_padded(int64_t L);
-size_t attn_fused_scratch_bytes(int64_t heads, int64_t L);
+size_t attn_fused_scratch_bytes(int64_t heads, int64_t L, bool ordered);
 int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, int heads, int64_t L, int64_t d, float alpha,
-               int causal, void* scratch, float* O, void* workspace /* 256 B: status word, cleared by the caller */,
-               cudaStream_t st, void* dbg_bits = nullptr, uint8_t* dbg_codes = nullptr, uint8_t* dbg_scales = nullptr,
+               int causal, bool ordered /* the softmax kernel's statistics bit for bit; otherwise online ones, d = 128 and L a
+               multiple of 128 only */,
+               void* scratch, float* O, void* workspace /* 256 B: status word, cleared by the caller */, cudaStream_t st, void* dbg_bits = nullptr, uint8_t* dbg_codes = nullptr, uint8_t* dbg_scales = nullptr,
                void* dbg_prepared = nullptr, int kv_group = 1 /* query heads per head of keys and values */,
                const int* gate = nullptr /* device word: the kernels do nothing when it is nonzero */);
 // The same attention on CUDA cores from the planes (or-ed: the codes) and canonical scales of those operands, any scale
