@@ -58,7 +58,10 @@ constexpr int kCodeBytes = 4 * 512;                // codes of 32 rows and one s
 constexpr int kMaxSlices = 8;                      // portable cluster size
 constexpr int kPartPitch = kCtaRows + 4;           // floats per token row of the partial-product tile (bank spread)
 constexpr int kMaxTiles = 8;                       // token tiles per CTA
-constexpr int kScaleSteps = 32;                    // steps whose scales are held at a time
+// Steps whose scales are held at a time: those of 32 steps in groups of 16 (67 KB) do not fit beside the rings of eight token
+// tiles (192 KB).
+__host__ __device__ constexpr int scale_steps(int gs) { return gs == 16 ? 16 : 32; }
+constexpr size_t kMaxSmem = 227 * 1024;
 
 // Fragment order of the token rows, per step and tile of 8 rows: pieces of 16 bytes [j = 0..3][lane 0..31]; the piece
 // of (j, lane (g, t)) holds elements 32 t + 8 j .. + 7 of the step, row g of the tile.  Piece (j, l) sits at position
@@ -149,7 +152,8 @@ __host__ __device__ constexpr int scale_bytes(int n, int gs) { return (kCtaRows 
 template <int NT, int GS>
 __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(const RowsParams p) {
     using R = Ring<NT, GS>;
-    constexpr int kDepth = R::kDepth, kFragSlot = R::kFragSlot;
+    constexpr int kDepth = R::kDepth, kFragSlot = R::kFragSlot, kScaleSteps = scale_steps(GS);
+    static_assert(R::kBytes + R::kFragRing + scale_bytes(kScaleSteps, GS) <= kMaxSmem, "shared memory of the longest range");
     extern __shared__ __align__(16) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int slices = (int)gridDim.y, slice = (int)blockIdx.y;
@@ -554,8 +558,6 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
     return best;
 }
 
-constexpr size_t kMaxSmem = 227 * 1024;
-
 struct RowsKernel {
     void (*fn)(const RowsParams);
     size_t ring_bytes, frag_ring_bytes;
@@ -592,7 +594,7 @@ int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cud
         }
         done = true;
     }
-    const int held = pl.steps_max < kScaleSteps ? pl.steps_max : kScaleSteps;
+    const int held = pl.steps_max < scale_steps(gs) ? pl.steps_max : scale_steps(gs);
     p.steps_max = pl.steps_max;
     cudaLaunchConfig_t cfg = {};
     const int cta_rows = pl.stream ? kStreamRows : kCtaRows;

@@ -39,6 +39,18 @@ def test_few_rows_against_oracle(M, N, K, gs):
     assert torch.equal(amx.quant_gemm(dev_bf16(a_bits), group_size=gs, w_bf16=dev_bf16(w_bits)), got.contiguous())
 
 
+@pytest.mark.parametrize("gs", [16, 32, 64, 128])
+@pytest.mark.parametrize("M,N,K", [(64, 40, 20480), (57, 130, 34048)])
+def test_long_ranges_of_eight_token_tiles(M, N, K, gs):
+    """Eight token tiles and K ranges of 20 and 34 steps: more than the scales held at a time, which for groups of 16 take
+    the most shared memory."""
+    a_bits, w_bits = inputs.random_groups(3250, M, K, "normal"), inputs.random_groups(3251, N, K, "normal")
+    qw = oracle.quantize(w_bits, gs)
+    got = amx.quant_gemm(dev_bf16(a_bits), *(torch.from_numpy(t).cuda() for t in qw), gs, flags=amx.GEMM_ROWS)
+    ref = oracle.gemm(*oracle.quantize(a_bits, gs), *qw, gs)
+    assert np.linalg.norm(got.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
 def test_back_to_back_calls_share_a_workspace():
     """Calls chained on one stream, every one of them on the same workspace and output: each sees its own rows."""
     N, K = 512, 4096
