@@ -33,11 +33,16 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // operand, and under AUTO the gated exact kernel behind it; the SIMT kernel for group sizes the tensor-core kernels do not take.
     // A few token rows against a big weight (decode-like): too few 128 x 256 tiles to fill the machine, and the
     // FP4 kernel would have to prepare the whole weight for them; the bf16-decode kernel slices K over CTAs.
-    // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows it still wins,
-    // in blocks of 64 rows, where the product is small (one launch against three to five) or the weight is what has to
-    // be moved (from 2^23 elements; the FP4 kernel would first prepare all of it for one or two row blocks of output).
+    // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows, in blocks of 64
+    // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route, which
+    // prepares the whole weight and then has few tiles: 12 us of launches, 5.7 per 1000 of K for one wave of tiles, the
+    // weight and the result moved (fitted to 16 weights of 2^17 to 2^27 elements x 65 to 256 rows, within 18 %; groups of
+    // 16, 64 and 128 are up to a fifth slower on both routes).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows
+    // 23 / 40 and at 256 36 / 43, 12288 x 4096 at 96 rows 51 / 51 and at 128 64 / 54, 4096 x 11008 at 192 rows 78 / 86,
+    // 28672 x 4096 at 72 rows 123 / 81; every product below 2^29 multiply-adds 6-26 / 15-74.
     const double mnk = (double)M * (double)N * (double)K;
-    if (rows && K >= 512 && (M <= 64 || mnk < 268435456.0 || (mnk < 536870912.0 && N >= 512) || N * K >= (1ll << 23)))
+    if (rows && K >= 512 && (M <= 64 || gemm_rows_estimated_us(M, N, K) <= 12.0 + 5.7e-3 * (double)K + 1.9e-7 * (double)N * (double)K +
+                                                                              6e-6 * (double)M * (double)N))
         return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
@@ -539,7 +544,8 @@ AttnLayout attn_layout_stored(int64_t L, int64_t d, bool tc) {
 // attention product would be small, the bf16-decode kernel, never the weight-streaming one (there is no weight).
 uint32_t attn_kernel(int64_t M, int64_t N, int64_t K, uint32_t flags) {
     const uint32_t k = pick_kernel(M, N, K, 32, flags);
-    return (k == AMX_GEMM_ROWS && (flags & kKernelMask) == AMX_GEMM_AUTO) ? AMX_GEMM_TC : k;
+    if (k != AMX_GEMM_ROWS || (flags & kKernelMask) != AMX_GEMM_AUTO) return k;
+    return gemm_fp4_supported(M, N, K, 32) && (double)M * (double)N * (double)K >= 268435456.0 ? AMX_GEMM_FP4 : AMX_GEMM_TC;
 }
 // Whether a call runs the fused kernel: asked for the FP4 kernel, or AUTO from 2^25 multiply-adds per product and head on
 // (512 tokens at head dimension 128; below, a batched launch of each step is as fast and the kernel's passes do not

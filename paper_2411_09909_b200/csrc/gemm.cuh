@@ -38,6 +38,7 @@ int gemm_tc_status(const void* workspace, cudaStream_t st);
 constexpr int64_t kRowsMaxM = 256;
 bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs);
 size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K);
+double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K);
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
               int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
 int gemm_rows_cast(const void* x, int64_t ld_x, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N,

@@ -515,6 +515,7 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
 struct RowsPlan {
     bool stream;
     int nt, m_blocks, slices, steps_max;
+    double us;                       // estimated time of both launches
     int tiles() const { return nt * m_blocks; }
 };
 
@@ -523,36 +524,36 @@ constexpr int kSmCount = 148;
 RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
     const int64_t steps = K / kStepK;
     const int tiles = (int)((M + kTok - 1) / kTok);
-    const int whole = tiles <= 4 ? tiles : tiles <= 6 ? 6 : 8;
-    RowsPlan best{};
-    // Up to 32 tokens, or blocks of 32 tokens while all of them together are resident at once (a small layer).
+    // Up to 32 tokens, or blocks of 32 tokens while all of them together are resident at once (a small layer: 6-9 us).
     const int64_t stream_blocks = (N + kStreamRows - 1) / kStreamRows;
     const int m_blocks32 = (tiles + 3) / 4;
-    if (tiles > 4 && stream_blocks * m_blocks32 <= 2 * kSmCount && N * K <= (1ll << 21)) return {true, 4, m_blocks32, 1, (int)steps};
+    if (tiles > 4 && stream_blocks * m_blocks32 <= 2 * kSmCount && N * K <= (1ll << 21)) return {true, 4, m_blocks32, 1, (int)steps, 9.0};
     if (tiles <= 4) {
         // one and a half CTAs per SM, and at least one step per warp
         int s = 1;
-        const int64_t blocks = stream_blocks;
-        while (s < kMaxSlices && blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
-        return {true, tiles, 1, s, (int)((steps + s - 1) / s)};
+        while (s < kMaxSlices && stream_blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
+        return {true, tiles, 1, s, (int)((steps + s - 1) / s), 0.0};
     }
-    // Time model, in cycles of one SM: a warp's step costs 256 cycles of the logic pipe for the decode of 32 rows x 128
-    // elements or 128 per token tile on the tensor pipe, whichever is larger; two warps of a CTA share a scheduler and
-    // take alternate steps, so a CTA needs that per step; start, casts and the reduction cost about 2500 cycles.
-    // Up to 64 rows one block of tokens (the weight is read and decoded once); above, blocks of 64 or of 32 rows.
+    // Time in us, fitted to 250 calls (N 256 to 28672, K 512 to 16384, 40 to 256 rows; weights from HBM): 4.5 for the
+    // fragments and the start, then per wave of CTAs a step's decode and MMAs and, with a cluster, its meeting at the end.
+    // Within 10 % where it matters (N K >= 2^23: 36 us estimated, 36.0 measured for 64 rows of 12288 x 4096, 50.9 / 50.0
+    // for 128 of 4096 x 11008).  Clusters of four and eight leave SMs of a GPC empty, those of three, five, six and seven
+    // more (4096 x 4096, 160 rows: three ranges 46.7 us, one 35.4).
+    // Up to 64 rows one block of tokens (the weight is read and decoded once); above, blocks of 64 or of 32 rows (of
+    // which two CTAs share an SM without being faster).
+    static constexpr struct { int slices, sms; } kFit[] = {{1, kSmCount}, {2, kSmCount}, {4, 132}, {8, 112}};
+    const int whole = tiles <= 6 ? 6 : 8;
     const int64_t row_blocks = (N + kCtaRows - 1) / kCtaRows;
-    double best_cost = 1e300;
+    RowsPlan best{};
     for (int nt = whole; nt >= 4; nt -= 4) {
         if (nt != whole && tiles <= kMaxTiles) break;
         const int m_blocks = (tiles + nt - 1) / nt;
-        const double per_step = 128.0 * nt;
-        for (int s = 1; s <= kMaxSlices && s <= steps; ++s) {
-            const int64_t ctas = row_blocks * s * m_blocks, waves = (ctas + kSmCount - 1) / kSmCount;
-            const double cost = (double)waves * ((double)((steps + s - 1) / s) * per_step + 2500.0);
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = {false, nt, m_blocks, s, (int)((steps + s - 1) / s)};
-            }
+        const double step = nt == 4 ? 0.7 : nt == 6 ? 0.8 : 0.975, meeting = nt == 4 ? 3.0 : 4.5;
+        for (const auto& f : kFit) {
+            if (f.slices > steps) break;
+            const int64_t ctas = row_blocks * f.slices * m_blocks, n = (steps + f.slices - 1) / f.slices;
+            const double us = 4.5 + (double)((ctas + f.sms - 1) / f.sms) * ((double)n * step + (f.slices > 1 ? meeting : 0.0));
+            if (!best.nt || us < best.us) best = {false, nt, m_blocks, f.slices, (int)n, us};
         }
     }
     return best;
@@ -684,6 +685,8 @@ bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs) {
 size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K) {
     return kHeaderBytes + (size_t)plan_rows(M, N, K).tiles() * kTok * (size_t)K * 2;
 }
+
+double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) { return plan_rows(M, N, K).us; }
 
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
               int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {

@@ -1,0 +1,25 @@
+"""What AMX_GEMM_AUTO picks between 65 and 256 rows, where both the weight-streaming kernel and the FP4 kernel take the call:
+the one that measured faster, at shapes where the two differ by more than a tenth (us, weights from HBM, one call)."""
+import pytest
+
+from paper_2411_09909_b200 import amx
+
+MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
+    (72, 28672, 4096, 109.6, 81.0), (128, 28672, 4096, 129.5, 89.2), (256, 28672, 4096, 224.2, 98.0),
+    (128, 12288, 4096, 64.0, 53.5), (256, 12288, 4096, 98.7, 62.2), (256, 6144, 4096, 64.0, 47.1), (160, 8192, 4096, 59.1, 48.2),
+    (72, 6144, 4096, 26.2, 40.0), (128, 8192, 4096, 35.8, 47.7), (192, 6144, 4096, 36.1, 45.3), (256, 4096, 4096, 36.2, 43.4),
+    (128, 4096, 4096, 23.5, 41.4), (128, 4096, 11008, 50.0, 85.1), (72, 4096, 14336, 62.2, 103.2), (128, 4096, 14336, 62.3, 107.8),
+    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (256, 256, 16384, 24.7, 112.8), (256, 4096, 512, 9.9, 17.5),
+    (128, 1024, 1024, 6.3, 22.7)]
+
+
+@pytest.mark.parametrize("M,N,K,rows_us,fp4_us", MEASURED)
+def test_auto_takes_the_faster_kernel(M, N, K, rows_us, fp4_us):
+    want = amx.GEMM_ROWS if rows_us < fp4_us else amx.GEMM_FP4
+    assert amx.lib().amx_gemm_kernel_for(M, N, K, 32, amx.GEMM_AUTO) == want
+
+
+@pytest.mark.parametrize("M", [1, 33, 48, 64])
+def test_up_to_64_rows_stream_the_weight(M):
+    for N, K in ((28672, 4096), (4096, 14336), (12288, 4096), (128, 512)):
+        assert amx.lib().amx_gemm_kernel_for(M, N, K, 32, amx.GEMM_AUTO) == amx.GEMM_ROWS
