@@ -44,8 +44,9 @@ inline bool programmatic_launch_ok(cudaStream_t st) {
 }
 
 // chained = false: an ordinary launch.  For long kernels with one block per SM: started while their predecessor leaves, the
-// blocks land on the SMs in another order, which costs them 2.5-4 % (operands shared by neighbouring tiles cross the two
-// halves of the L2 more often) - more than the gap from about 200 us on.
+// blocks land on the SMs in another order (operands shared by neighbouring tiles cross the two halves of the L2 more often).
+// That costs the longest of them 2-5 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
+// measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 170 and at 100 us.
 template <typename... P, typename... A>
 int launch_clusters(unsigned cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};

@@ -702,8 +702,12 @@ int launch_pass(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensor
         configured[dev] = true;
     }
     const int items = p.heads * p.m_tiles;
-    return launch_chained((double)p.heads * (double)p.L * (double)p.L <= 2.7e8,   // about 140 us in the map pass
-                          attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS), Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
+    // Chained up to about 100 us in the map pass.  32 heads of 128, the whole call: 1536 keys 128.7 us ordinary, 128.0 chained, 2048
+    // 194.6 / 195.9, 3072 369 / 380, causal 1024 76.3 / 72.9, 2560 186.7 / 186.8, 3072 237 / 241; of 64: 2048 206.8 / 205.4, 2560
+    // 297 / 300.
+    const double work = (double)p.heads * (double)p.L * (double)p.L * HD / (MASK == kMaskCausal ? 2.0 : 1.0);
+    return launch_chained(work <= 1.1e10, attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS),
+                          Smem<PASS>::kBytes, st, tm_q, tm_k, tm_v, p);
 }
 
 }  // namespace

@@ -726,8 +726,11 @@ int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, co
     const int64_t tiles = ((p.N + BNT - 1) / BNT) * ((p.M + BMT - 1) / BMT) * (SLICED ? p.slices : 1);
     const int64_t workers = std::min<int64_t>(tiles, sm_count(dev) / kCtas);           // one persistent CTA per SM
     const unsigned grid = (unsigned)workers * kCtas;
-    return launch_clusters(kCtas, (double)p.M * (double)p.N * (double)p.K <= 1.1e11,      // about 170 us
-                          gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w, tm_a1, tm_w1, p);
+    // Chained up to 4.4e11 issued products (about 170 us).  Cast and product of 2048 x 12288 x 4096: ordinary 173 us, chained 153 to
+    // 161; 4096 x 11008 x 4096 265 / 274.  One plane, 8192 x 6144 x 4096: 136 / 132, 8192 x 14336 x 4096 269 / 267.
+    const double products = (double)p.M * (double)p.N * (double)p.K * (ONE_PLANE ? 1.0 : 4.0);
+    return launch_clusters(kCtas, products <= 4.4e11, gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w,
+                           tm_a1, tm_w1, p);
 }
 
 }  // namespace
