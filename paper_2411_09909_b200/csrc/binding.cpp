@@ -40,6 +40,15 @@ const at::Tensor* device_tensor(PyObject* o, at::ScalarType dtype, const char* n
     }
     return t;
 }
+// The same for a matrix (checked first: a shape is wrong on every device).
+const at::Tensor* device_matrix(PyObject* o, at::ScalarType dtype, const char* name) {
+    const at::Tensor* t = tensor(o, name);
+    if (t && t->dim() != 2) {
+        PyErr_Format(PyExc_ValueError, "%s must be a matrix, not a tensor of %lld dimensions", name, (long long)t->dim());
+        return nullptr;
+    }
+    return t ? device_tensor(o, dtype, name) : nullptr;
+}
 at::Tensor empty(at::IntArrayRef sizes, at::ScalarType dtype, const at::Tensor& like) {
     return at::detail::empty_cuda(sizes, dtype, like.device(), std::nullopt);
 }
@@ -194,17 +203,20 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
 PyObject* quant_gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     HANDLE_TH_ERRORS
     ARGS(8)
-    const at::Tensor* x = device_tensor(a[0], at::kBFloat16, "a");
+    const at::Tensor* x = device_matrix(a[0], at::kBFloat16, "a");
     if (!x) return nullptr;
     const at::Tensor *wc = nullptr, *ws_ = nullptr, *wb = nullptr;
     if (a[7] != Py_None) {
-        wb = device_tensor(a[7], at::kBFloat16, "w_bf16");
-        if (!wb || !require(a[1] == Py_None && a[2] == Py_None && wb->stride(1) == 1, "w_bf16 is a row-major matrix and the only weight"))
+        wb = device_matrix(a[7], at::kBFloat16, "w_bf16");
+        if (!wb || !require(a[1] == Py_None && a[2] == Py_None && wb->stride(1) == 1 && wb->size(1) == x->size(1),
+                            "w_bf16 is a row-major matrix with the columns of a and the only weight"))
             return nullptr;
     } else if (!(wc = tensor(a[1], "w_codes")) || !(ws_ = tensor(a[2], "w_scales"))) return nullptr;
     const int64_t gs = as_int(a[3]), flags = as_int(a[4]);
     INTS_OK
     const int64_t M = x->size(0), K = x->size(1), N = wb ? wb->size(0) : wc->size(0);
+    if (wc && !require(wc->numel() >= N * (K / 2) && (gs <= 0 || ws_->numel() >= N * (K / gs) * 2), "the weight has fewer columns than a"))
+        return nullptr;
     at::Tensor out, ws;
     const size_t need = a[6] == Py_None
         ? amx_quant_gemm_workspace_bytes(M, N, K, (int)gs, ((uint32_t)flags & ~AMX_GEMM_CAST_IN_KERNEL) | (wb ? AMX_WEIGHT_BF16 : 0)) : 0;
