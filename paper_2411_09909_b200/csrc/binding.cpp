@@ -3,7 +3,7 @@
 // Through ctypes a call costs 15-30 us of host time (argument conversion, a Python-level allocation per output and
 // per scratch buffer, the stream lookup), more than the GPU needs for a small layer.  Here a call unpacks the tensors,
 // allocates through the caching allocator without the dispatcher, takes the current stream and enters the C ABI:
-// about 3 us plus the launches.  Nothing is kept between calls.
+// about 3 us plus the launches, which run without the interpreter lock.  Nothing is kept between calls.
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
@@ -55,6 +55,17 @@ at::Tensor empty(at::IntArrayRef sizes, at::ScalarType dtype, const at::Tensor& 
 at::Tensor scratch(size_t bytes, const at::Tensor& like) {
     return empty({(int64_t)(bytes > 256 ? bytes : 256)}, at::kByte, like);
 }
+// Enters the library with the interpreter lock given up (a launch waits when the stream's queue is full); the arguments have
+// been evaluated by then.
+struct Unlocked {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <typename... P, typename... A>
+int enter(int (*fn)(P...), A... args) {
+    const Unlocked unlocked;
+    return fn(static_cast<P>(args)...);
+}
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 uint8_t* u8(const at::Tensor& t) { return static_cast<uint8_t*>(t.data_ptr()); }
 float* f32(const at::Tensor& t) { return static_cast<float*>(t.data_ptr()); }
@@ -89,7 +100,7 @@ PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     if (gs <= 0) return fail("amx_quantize", AMX_ERR_SHAPE);
     const int64_t rows = x->size(0), K = x->size(1);
     at::Tensor codes = empty({rows, K / 2}, at::kByte, *x), scales = empty({rows, K / gs, 2}, at::kByte, *x);
-    const int rc = amx_quantize_fmt(x->data_ptr(), rows, K, lead(*x), (int)gs, (int)fmt, u8(codes), u8(scales), stream());
+    const int rc = enter(amx_quantize_fmt, x->data_ptr(), rows, K, lead(*x), (int)gs, (int)fmt, u8(codes), u8(scales), stream());
     if (rc) return fail(fmt ? "amx_quantize_fmt" : "amx_quantize", rc);
     return tuple({codes, scales});
     END_HANDLE_TH_ERRORS
@@ -112,8 +123,8 @@ PyObject* fake_quantize(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
             return nullptr;
         out = *o;
     }
-    const int rc = amx_fake_quantize(x->data_ptr(), x->size(0), x->size(1), lead(*x), (int)gs, (int)fmt, out.data_ptr(),
-                                     lead(out), stream());
+    const int rc = enter(amx_fake_quantize, x->data_ptr(), x->size(0), x->size(1), lead(*x), (int)gs, (int)fmt, out.data_ptr(),
+                         lead(out), stream());
     if (rc) return fail("amx_fake_quantize", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -130,7 +141,7 @@ PyObject* dequantize(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     INTS_OK
     const int64_t rows = c->size(0), K = c->size(1) * 2;
     at::Tensor out = empty({rows, K}, bf16 ? at::kBFloat16 : at::kFloat, *c);
-    const int rc = amx_dequantize(u8(*c), u8(*s), rows, K, (int)gs, bf16 ? AMX_OUT_BF16 : AMX_OUT_F32, out.data_ptr(), K, stream());
+    const int rc = enter(amx_dequantize, u8(*c), u8(*s), rows, K, (int)gs, bf16 ? AMX_OUT_BF16 : AMX_OUT_F32, out.data_ptr(), K, stream());
     if (rc) return fail("amx_dequantize", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -150,8 +161,8 @@ PyObject* quant_error(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     at::Tensor out = empty({4}, at::kDouble, *x);
     const size_t need = amx_quant_error_workspace_bytes();
     at::Tensor ws = scratch(need, *x);
-    const int rc = amx_quant_error(x->data_ptr(), x->size(0), x->size(1), x->stride(0), u8(*c), u8(*s), (int)gs,
-                                   static_cast<double*>(out.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(amx_quant_error, x->data_ptr(), x->size(0), x->size(1), x->stride(0), u8(*c), u8(*s), (int)gs,
+                         static_cast<double*>(out.data_ptr()), ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail("amx_quant_error", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -192,8 +203,8 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     at::Tensor out, ws;
     const size_t need = a[7] == Py_None ? amx_workspace_bytes(M, N, K, (int)gs, (uint32_t)flags) : 0;
     if (!out_and_workspace(a[6], a[7], M, N, at::kFloat, need, *t[0], out, ws)) return nullptr;
-    const int rc = amx_gemm(u8(*t[0]), u8(*t[1]), u8(*t[2]), u8(*t[3]), M, N, K, (int)gs, (uint32_t)flags, f32(out), out.stride(0),
-                            ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(amx_gemm, u8(*t[0]), u8(*t[1]), u8(*t[2]), u8(*t[3]), M, N, K, (int)gs, (uint32_t)flags, f32(out), out.stride(0),
+                         ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail("amx_gemm", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -221,9 +232,9 @@ PyObject* quant_gemm(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     const size_t need = a[6] == Py_None
         ? amx_quant_gemm_workspace_bytes(M, N, K, (int)gs, ((uint32_t)flags & ~AMX_GEMM_CAST_IN_KERNEL) | (wb ? AMX_WEIGHT_BF16 : 0)) : 0;
     if (!out_and_workspace(a[5], a[6], M, N, at::kFloat, need, *x, out, ws)) return nullptr;
-    const int rc = amx_quant_gemm(x->data_ptr(), x->stride(0), wc ? u8(*wc) : nullptr, ws_ ? u8(*ws_) : nullptr,
-                                  wb ? wb->data_ptr() : nullptr, wb ? wb->stride(0) : 0, M, N, K, (int)gs, (uint32_t)flags, f32(out),
-                                  out.stride(0), ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(amx_quant_gemm, x->data_ptr(), x->stride(0), wc ? u8(*wc) : nullptr, ws_ ? u8(*ws_) : nullptr,
+                         wb ? wb->data_ptr() : nullptr, wb ? wb->stride(0) : 0, M, N, K, (int)gs, (uint32_t)flags, f32(out),
+                         out.stride(0), ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail("amx_quant_gemm", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -248,8 +259,8 @@ PyObject* quantize_prepared(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
         if (!p) return nullptr;
         buf = *p;
     } else buf = scratch(amx_prepared_bytes(rows, K, (int)gs, is_weight), *x);
-    const int rc = amx_quantize_prepared_fmt(x->data_ptr(), rows, K, (int)gs, is_weight, (int)fmt, want_codes ? u8(codes) : nullptr,
-                                             u8(scales), buf.data_ptr(), (size_t)buf.numel(), stream());
+    const int rc = enter(amx_quantize_prepared_fmt, x->data_ptr(), rows, K, (int)gs, is_weight, (int)fmt, want_codes ? u8(codes) : nullptr,
+                         u8(scales), buf.data_ptr(), (size_t)buf.numel(), stream());
     if (rc) return fail(fmt ? "amx_quantize_prepared_fmt" : "amx_quantize_prepared", rc);
     PyObject* r = PyTuple_New(3);
     if (want_codes) PyTuple_SET_ITEM(r, 0, wrap(codes));
@@ -281,9 +292,9 @@ PyObject* gemm_prepared(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
         PyErr_SetString(g_error, "out must be a CUDA tensor of torch.float32");
         return nullptr;
     }
-    const int rc = amx_gemm_prepared_ex(pa->data_ptr(), pw->data_ptr(), M, N, K, (int)gs,
-                                        (bf16 ? AMX_PREP_OUT_BF16 : 0) | (sym ? AMX_PREP_ONE_PLANE : 0), out.data_ptr(), out.stride(0),
-                                        ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(amx_gemm_prepared_ex, pa->data_ptr(), pw->data_ptr(), M, N, K, (int)gs,
+                         (bf16 ? AMX_PREP_OUT_BF16 : 0) | (sym ? AMX_PREP_ONE_PLANE : 0), out.data_ptr(), out.stride(0),
+                         ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail(bf16 ? "amx_gemm_prepared_ex" : "amx_gemm_prepared", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -312,8 +323,8 @@ PyObject* attention_heads(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
         ws = *w;
     }
     out = empty({H, L, d}, at::kFloat, *t[0]);
-    const int rc = amx_attention_gqa(t[0]->data_ptr(), t[1]->data_ptr(), t[2]->data_ptr(), H, KV, L, d, (uint32_t)flags, f32(out),
-                                     ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(amx_attention_gqa, t[0]->data_ptr(), t[1]->data_ptr(), t[2]->data_ptr(), H, KV, L, d, (uint32_t)flags, f32(out),
+                         ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail(KV == H ? "amx_attention" : "amx_attention_gqa", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
@@ -335,8 +346,8 @@ PyObject* quantize_nvfp4(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     if (as) {
         prep = empty({(int64_t)amx_nvfp4_prepared_bytes(rows, K, as == 2)}, at::kByte, *x);
     }
-    const int rc = amx_quantize_nvfp4(x->data_ptr(), rows, K, x->stride(0), asym ? AMX_NV_ASYMMETRIC : 0, u8(codes), u8(scales), f32(ts),
-                                      as == 2, as ? prep.data_ptr() : nullptr, as ? (size_t)prep.numel() : 0, stream());
+    const int rc = enter(amx_quantize_nvfp4, x->data_ptr(), rows, K, x->stride(0), asym ? AMX_NV_ASYMMETRIC : 0, u8(codes), u8(scales), f32(ts),
+                         as == 2, as ? prep.data_ptr() : nullptr, as ? (size_t)prep.numel() : 0, stream());
     if (rc) return fail("amx_quantize_nvfp4", rc);
     return as ? tuple({codes, scales, ts, prep}) : tuple({codes, scales, ts});
     END_HANDLE_TH_ERRORS
@@ -354,7 +365,7 @@ PyObject* gemm_nvfp4(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     at::Tensor out, ws;
     if (!out_and_workspace(Py_None, a[5], M, N, at::kFloat, 256, *pa, out, ws)) return nullptr;
     auto* fn = sym ? amx_gemm_nvfp4_sym : amx_gemm_nvfp4;
-    const int rc = fn(pa->data_ptr(), pw->data_ptr(), M, N, K, f32(out), N, ws.data_ptr(), (size_t)ws.numel(), stream());
+    const int rc = enter(fn, pa->data_ptr(), pw->data_ptr(), M, N, K, f32(out), N, ws.data_ptr(), (size_t)ws.numel(), stream());
     if (rc) return fail("amx_gemm_nvfp4", rc);
     return wrap(out);
     END_HANDLE_TH_ERRORS
