@@ -228,6 +228,8 @@ def gemm_prepared(a_prepared: torch.Tensor, w_prepared: torch.Tensor, M: int, N:
                   out_dtype=torch.float32):
     """sym: both operands are in a symmetric format (amx_gemm_prepared_sym; a violated promise shows in gemm_status);
     out_dtype torch.bfloat16: the result rounded to bf16 in the epilogue (amx_gemm_prepared_ex)."""
+    if out is None and out_dtype not in (torch.float32, torch.bfloat16):
+        raise AmxError(f"out must be a CUDA tensor of {torch.float32}")
     return (_native_module or _native()).gemm_prepared(a_prepared, w_prepared, M, N, K, group_size, out, workspace, sym,
                                                        out_dtype == torch.bfloat16)
 

@@ -24,6 +24,12 @@ def test_operands_on_the_host_are_refused():
         amx.quant_gemm(bf16(4, 64), w_bf16=bf16(8, 64))
 
 
+def test_gemm_prepared_refuses_a_result_type_it_does_not_have():
+    a = torch.zeros(256, dtype=torch.uint8)
+    with pytest.raises(amx.AmxError, match="out must be a CUDA tensor"):
+        amx.gemm_prepared(a, a, 128, 128, 128, out_dtype=torch.float16)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("w", [(8, 1, 64), (8, 2, 64), (8,)])
 def test_quant_gemm_refuses_a_weight_that_is_no_matrix(w):
