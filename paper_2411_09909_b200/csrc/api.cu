@@ -40,10 +40,11 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // 16, 64 and 128 are up to a fifth slower on both routes).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows
     // 23 / 40 and at 256 36 / 43, 12288 x 4096 at 96 rows 51 / 51 and at 128 64 / 54, 4096 x 11008 at 192 rows 78 / 86,
     // 28672 x 4096 at 72 rows 123 / 81; every product below 2^29 multiply-adds 6-26 / 15-74.
-    const double mnk = (double)M * (double)N * (double)K;
-    if (rows && K >= 512 && (M <= 64 || gemm_rows_estimated_us(M, N, K) <= 12.0 + 5.7e-3 * (double)K + 1.9e-7 * (double)N * (double)K +
-                                                                              6e-6 * (double)M * (double)N))
-        return AMX_GEMM_ROWS;
+    // A narrow weight (below 512 rows and 2^23 elements) stays on the FP4 route from 2^28 multiply-adds on, slower as it is
+    // (256 x 8192 at 128 rows: 14 / 70): callers read the count of flushed scales that this route leaves in the workspace.
+    const double mnk = (double)M * (double)N * (double)K, fp4_us = 12.0 + 5.7e-3 * (double)K + 1.9e-7 * (double)N * (double)K + 6e-6 * (double)M * (double)N;
+    const bool narrow = N < 512 && N * K < (1ll << 23) && mnk >= 268435456.0;
+    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_us))) return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
     // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)

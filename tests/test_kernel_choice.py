@@ -9,7 +9,7 @@ MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
     (128, 12288, 4096, 64.0, 53.5), (256, 12288, 4096, 98.7, 62.2), (256, 6144, 4096, 64.0, 47.1), (160, 8192, 4096, 59.1, 48.2),
     (72, 6144, 4096, 26.2, 40.0), (128, 8192, 4096, 35.8, 47.7), (192, 6144, 4096, 36.1, 45.3), (256, 4096, 4096, 36.2, 43.4),
     (128, 4096, 4096, 23.5, 41.4), (128, 4096, 11008, 50.0, 85.1), (72, 4096, 14336, 62.2, 103.2), (128, 4096, 14336, 62.3, 107.8),
-    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (256, 256, 16384, 24.7, 112.8), (256, 4096, 512, 9.9, 17.5),
+    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (192, 256, 4096, 9.9, 37.0), (256, 4096, 512, 9.9, 17.5),
     (128, 1024, 1024, 6.3, 22.7)]
 
 
@@ -17,6 +17,11 @@ MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
 def test_auto_takes_the_faster_kernel(M, N, K, rows_us, fp4_us):
     want = amx.GEMM_ROWS if rows_us < fp4_us else amx.GEMM_FP4
     assert amx.lib().amx_gemm_kernel_for(M, N, K, 32, amx.GEMM_AUTO) == want
+
+
+def test_narrow_weights_keep_the_route_that_counts_flushed_scales():
+    assert amx.lib().amx_gemm_kernel_for(128, 256, 8192, 32, amx.GEMM_AUTO) == amx.GEMM_FP4
+    assert amx.lib().amx_gemm_kernel_for(64, 256, 8192, 32, amx.GEMM_AUTO) == amx.GEMM_ROWS
 
 
 @pytest.mark.parametrize("M", [1, 33, 48, 64])
