@@ -17,6 +17,16 @@ bool gemm_shape_ok(int64_t M, int64_t N, int64_t K, int gs) {
 
 constexpr uint32_t kKernelMask = AMX_GEMM_SIMT | AMX_GEMM_TC | AMX_GEMM_FP4 | AMX_GEMM_ROWS;
 
+// Time of the FP4 route under AUTO for 65 to 256 rows, us: preparation of the whole weight, one or two waves of tiles, the result,
+// and the gated exact kernel behind it, whose reduction (groups of 32, K from 1024, less than a wave of tiles) is a launch of
+// M N / 256 blocks even when it has nothing to do.  Fitted to 320 calls of 31 weights, within 20 % from 2^21 weight elements on.
+double fp4_route_us(int64_t M, int64_t N, int64_t K, int gs) {
+    const double mn = (double)M * (double)N;
+    const bool second_wave = ((M + 127) / 128) * ((N + 255) / 256) > 148;
+    return 12.5 + 5.6e-3 * (double)K + 3.2e-7 * (double)N * (double)K + 1.4e-6 * mn + (second_wave ? 4.7 : 0.0) +
+           (gs == 32 && K >= 1024 && !second_wave ? 2.7e-6 * mn : 0.0);
+}
+
 // The kernel to run (one AMX_GEMM_* bit), or 0 when the flags cannot be honoured for this shape.
 uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     const uint32_t want = flags & kKernelMask;
@@ -34,17 +44,15 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // A few token rows against a big weight (decode-like): too few 128 x 256 tiles to fill the machine, and the
     // FP4 kernel would have to prepare the whole weight for them; the bf16-decode kernel slices K over CTAs.
     // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows, in blocks of 64
-    // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route, which
-    // prepares the whole weight and then has few tiles: 12 us of launches, 5.7 per 1000 of K for one wave of tiles, the
-    // weight and the result moved (fitted to 16 weights of 2^17 to 2^27 elements x 65 to 256 rows, within 18 %; groups of
-    // 16, 64 and 128 are up to a fifth slower on both routes).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows
-    // 23 / 40 and at 256 36 / 43, 12288 x 4096 at 96 rows 51 / 51 and at 128 64 / 54, 4096 x 11008 at 192 rows 78 / 86,
-    // 28672 x 4096 at 72 rows 123 / 81; every product below 2^29 multiply-adds 6-26 / 15-74.
+    // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route
+    // (fp4_route_us).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 23 / 40 and at 256 36 / 43, 12288 x 4096 at
+    // 96 rows 51 / 51 and at 128 64 / 54, 4096 x 11008 at 192 rows 78 / 86, 28672 x 4096 at 72 rows 123 / 81, 14336 x 512 at
+    // 128 rows 17 / 20 and at 200 28 / 20.
     // A narrow weight (below 512 rows and 2^23 elements) stays on the FP4 route from 2^28 multiply-adds on, slower as it is
     // (256 x 8192 at 128 rows: 14 / 70): callers read the count of flushed scales that this route leaves in the workspace.
-    const double mnk = (double)M * (double)N * (double)K, fp4_us = 12.0 + 5.7e-3 * (double)K + 1.9e-7 * (double)N * (double)K + 6e-6 * (double)M * (double)N;
+    const double mnk = (double)M * (double)N * (double)K;
     const bool narrow = N < 512 && N * K < (1ll << 23) && mnk >= 268435456.0;
-    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_us))) return AMX_GEMM_ROWS;
+    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_route_us(M, N, K, gs)))) return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
     // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)

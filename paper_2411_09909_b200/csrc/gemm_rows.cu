@@ -534,10 +534,10 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
         while (s < kMaxSlices && stream_blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
         return {true, tiles, 1, s, (int)((steps + s - 1) / s), 0.0};
     }
-    // Time in us, fitted to 250 calls (N 256 to 28672, K 512 to 16384, 40 to 256 rows; weights from HBM): 4.5 for the
-    // fragments and the start, then per wave of CTAs a step's decode and MMAs and, with a cluster, its meeting at the end.
-    // Within 10 % where it matters (N K >= 2^23: 36 us estimated, 36.0 measured for 64 rows of 12288 x 4096, 50.9 / 50.0
-    // for 128 of 4096 x 11008).  Clusters of four and eight leave SMs of a GPC empty, those of three, five, six and seven
+    // Time in us, fitted to 320 calls (N 256 to 28672, K 512 to 16384, 40 to 256 rows; weights from HBM): 3.5 for the
+    // fragments and the start, then per wave of CTAs its steps' decode and MMAs, its own start and, with a cluster, the
+    // meeting at the end.  Within 10 % for blocks of 48 and 64 rows (35.2 us estimated, 36.0 measured for 64 rows of
+    // 12288 x 4096, 49.6 / 50.0 for 128 of 4096 x 11008).  Clusters of four and eight leave SMs of a GPC empty, those of three, five, six and seven
     // more (4096 x 4096, 160 rows: three ranges 46.7 us, one 35.4).
     // Up to 64 rows one block of tokens (the weight is read and decoded once); above, blocks of 64 or of 32 rows (of
     // which two CTAs share an SM without being faster).
@@ -548,11 +548,11 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
     for (int nt = whole; nt >= 4; nt -= 4) {
         if (nt != whole && tiles <= kMaxTiles) break;
         const int m_blocks = (tiles + nt - 1) / nt;
-        const double step = nt == 4 ? 0.7 : nt == 6 ? 0.8 : 0.975, meeting = nt == 4 ? 3.0 : 4.5;
+        const double step = nt == 4 ? 0.69 : nt == 6 ? 0.78 : 0.91, start = nt == 4 ? 1.0 : 2.6, meeting = nt == 4 ? 3.0 : 3.9;
         for (const auto& f : kFit) {
             if (f.slices > steps) break;
             const int64_t ctas = row_blocks * f.slices * m_blocks, n = (steps + f.slices - 1) / f.slices;
-            const double us = 4.5 + (double)((ctas + f.sms - 1) / f.sms) * ((double)n * step + (f.slices > 1 ? meeting : 0.0));
+            const double us = 3.5 + (double)((ctas + f.sms - 1) / f.sms) * ((double)n * step + (f.slices > 1 ? meeting : start));
             if (!best.nt || us < best.us) best = {false, nt, m_blocks, f.slices, (int)n, us};
         }
     }

@@ -9,7 +9,9 @@ MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
     (128, 12288, 4096, 64.0, 53.5), (256, 12288, 4096, 98.7, 62.2), (256, 6144, 4096, 64.0, 47.1), (160, 8192, 4096, 59.1, 48.2),
     (72, 6144, 4096, 26.2, 40.0), (128, 8192, 4096, 35.8, 47.7), (192, 6144, 4096, 36.1, 45.3), (256, 4096, 4096, 36.2, 43.4),
     (128, 4096, 4096, 23.5, 41.4), (128, 4096, 11008, 50.0, 85.1), (72, 4096, 14336, 62.2, 103.2), (128, 4096, 14336, 62.3, 107.8),
-    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (192, 256, 4096, 9.9, 37.0), (256, 4096, 512, 9.9, 17.5),
+    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (192, 256, 4096, 11.0, 40.7), (72, 12288, 640, 11.9, 21.3),
+    (256, 12288, 640, 27.8, 22.8), (200, 14336, 512, 28.2, 20.0), (128, 8192, 640, 10.7, 20.6), (256, 28672, 1024, 78.2, 42.0),
+    (96, 5120, 2560, 18.5, 31.1), (256, 4096, 512, 9.9, 17.5),
     (128, 1024, 1024, 6.3, 22.7)]
 
 
