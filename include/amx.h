@@ -394,7 +394,8 @@ int amx_linear_host_pipelined_status(const void* workspace, void* stream);
  *     library holds it until the process exits.  It holds whatever amx_quant_gemm would keep in its
  *     workspace: the status word, the quantized activation and, when AUTO picks the FP4 kernel, both
  *     operands in that kernel's form.  amx_quant_gemm_static_capacity() returns its size; a problem for which
- *     amx_quant_gemm_workspace_bytes() exceeds it is rejected with AMX_ERR_TOO_LARGE and nothing runs.
+ *     amx_quant_gemm_workspace_bytes() exceeds it runs, under AUTO, on a kernel that prepares no operands where one
+ *     fits (up to 256 rows; group sizes other than 32), and is else rejected with AMX_ERR_TOO_LARGE: nothing runs.
  *   - The entry point calls no cudaMalloc / cudaFree and no allocating library routine.
  *   - The first call on each device looks up the array's device address, which is also when the CUDA
  *     runtime loads this part of the library onto the device and the array starts to occupy memory there:

@@ -81,6 +81,13 @@ QuantSizes quant_sizes(int64_t rows, int64_t K, int gs) {
     return {round_up((size_t)rows * (size_t)(K / 2)), round_up((size_t)rows * (size_t)(K / gs) * 2)};
 }
 
+size_t quant_gemm_bytes(uint32_t kernel, bool fallback, int64_t M, int64_t N, int64_t K, int gs, bool w_is_bf16) {
+    const QuantSizes a = quant_sizes(M, K, gs), w = quant_sizes(N, K, gs);
+    // the first 256 bytes always hold the status word and the flushed-scale count, whichever kernel runs
+    const size_t gemm_ws = kernel_workspace(kernel, M, N, K, fallback, gs);
+    return (gemm_ws < 256 ? 256 : gemm_ws) + a.codes + a.scales + (w_is_bf16 ? w.codes + w.scales : 0);
+}
+
 constexpr uint32_t kQuantGemmFlags = kKernelMask | AMX_GEMM_CAST_IN_KERNEL | AMX_WEIGHT_BF16;
 
 __global__ void clear_words_kernel(int* __restrict__ words, int n) {
@@ -89,6 +96,10 @@ __global__ void clear_words_kernel(int* __restrict__ words, int n) {
 }
 
 }  // namespace
+
+size_t quant_gemm_rows_bytes(int64_t M, int64_t N, int64_t K, int gs) {
+    return K >= 512 && gemm_rows_supported(M, N, K, gs) ? quant_gemm_bytes(AMX_GEMM_ROWS, false, M, N, K, gs, false) : 0;
+}
 
 int clear_words(void* words, cudaStream_t st, int n) { return launch(clear_words_kernel, 1, 32, 0, st, static_cast<int*>(words), n); }
 
@@ -109,11 +120,8 @@ extern "C" size_t amx_workspace_bytes(int64_t M, int64_t N, int64_t K, int group
 
 extern "C" size_t amx_quant_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int group_size, uint32_t flags) {
     if (!gemm_shape_ok(M, N, K, group_size)) return 0;
-    const QuantSizes a = quant_sizes(M, K, group_size), w = quant_sizes(N, K, group_size);
-    // the first 256 bytes always hold the status word and the flushed-scale count, whichever kernel runs
-    size_t gemm_ws = amx_workspace_bytes(M, N, K, group_size, flags & kKernelMask);
-    if (gemm_ws < 256) gemm_ws = 256;
-    return gemm_ws + a.codes + a.scales + ((flags & AMX_WEIGHT_BF16) ? w.codes + w.scales : 0);
+    const uint32_t kernel = pick_kernel(M, N, K, group_size, flags & kKernelMask);
+    return quant_gemm_bytes(kernel, auto_fallback(flags, kernel), M, N, K, group_size, flags & AMX_WEIGHT_BF16);
 }
 
 extern "C" size_t amx_linear_host_workspace_bytes(int64_t M, int64_t N, int64_t K, int group_size, uint32_t flags) {
@@ -243,19 +251,25 @@ extern "C" int amx_quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_code
                               const void* W_bf16, int64_t ld_w, int64_t M, int64_t N, int64_t K, int group_size,
                               uint32_t flags, float* C, int64_t ld_c, void* workspace, size_t workspace_bytes,
                               void* stream) {
+    return quant_gemm(A, ld_a, w_codes, w_scales, W_bf16, ld_w, M, N, K, group_size, flags, 0, C, ld_c, workspace, workspace_bytes, stream);
+}
+
+int amx::quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_codes, const uint8_t* w_scales, const void* W_bf16, int64_t ld_w,
+                    int64_t M, int64_t N, int64_t K, int group_size, uint32_t flags, uint32_t auto_kernel, float* C, int64_t ld_c,
+                    void* workspace, size_t workspace_bytes, void* stream) {
     if (flags & ~kQuantGemmFlags) return AMX_ERR_FLAGS;
     const bool cast_in_kernel = flags & AMX_GEMM_CAST_IN_KERNEL;
     const bool w_is_bf16 = W_bf16 != nullptr;
     flags &= kKernelMask;
     if (cast_in_kernel && flags != AMX_GEMM_TC) return AMX_ERR_FLAGS;
     if (!gemm_shape_ok(M, N, K, group_size) || ld_a < K || ld_c < N || (w_is_bf16 && ld_w < K)) return AMX_ERR_SHAPE;
-    uint32_t kernel = pick_kernel(M, N, K, group_size, flags);
+    uint32_t kernel = auto_kernel && flags == AMX_GEMM_AUTO ? auto_kernel : pick_kernel(M, N, K, group_size, flags);
     if (!kernel) return (flags & (flags - 1)) ? AMX_ERR_FLAGS : AMX_ERR_SHAPE;
     if (M == 0 || N == 0) return AMX_OK;
     // exactly one form of the weight
     if (!A || !C || (w_is_bf16 ? (w_codes || w_scales) : (!w_codes || !w_scales))) return AMX_ERR_NULL;
-    const size_t need = amx_quant_gemm_workspace_bytes(M, N, K, group_size, flags | (w_is_bf16 ? AMX_WEIGHT_BF16 : 0));
-    if (!workspace || workspace_bytes < need) return AMX_ERR_WORKSPACE;
+    if (!workspace || workspace_bytes < quant_gemm_bytes(kernel, auto_fallback(flags, kernel), M, N, K, group_size, w_is_bf16))
+        return AMX_ERR_WORKSPACE;
     // as in amx_gemm: operands that miss the alignment of the kernel AUTO picked run on the plain kernel (with groups of
     // 32 and at most 64 rows they are refused, as documented at AMX_GEMM_ROWS)
     if (flags == AMX_GEMM_AUTO && !w_is_bf16 && !(group_size == 32 && M <= 64) &&

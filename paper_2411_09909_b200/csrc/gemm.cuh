@@ -39,6 +39,12 @@ constexpr int64_t kRowsMaxM = 256;
 bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs);
 size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K);
 double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K);
+// amx_quant_gemm with the kernel that AUTO stands for given (0: AUTO's own choice), and its workspace with a quantized weight
+// on the streaming kernel (0: that kernel does not take the shape).  api.cu
+int quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_codes, const uint8_t* w_scales, const void* W_bf16, int64_t ld_w, int64_t M,
+               int64_t N, int64_t K, int group_size, uint32_t flags, uint32_t auto_kernel, float* C, int64_t ld_c, void* workspace,
+               size_t workspace_bytes, void* stream);
+size_t quant_gemm_rows_bytes(int64_t M, int64_t N, int64_t K, int gs);
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
               int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st);
 int gemm_rows_cast(const void* x, int64_t ld_x, const uint8_t* w_codes, const uint8_t* w_scales, int64_t M, int64_t N,

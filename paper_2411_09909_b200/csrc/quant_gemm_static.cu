@@ -65,18 +65,21 @@ extern "C" int amx_quant_gemm_static(const void* A, int64_t ld_a, const uint8_t*
     if (M == 0 || N == 0) return AMX_OK;
     // Nothing below needs to start at zero except the GEMM's status word, which the GEMM launcher
     // clears itself on `stream`; the quantized activation is fully overwritten before it is read.
+    uint32_t kernel = 0;                             // AUTO's own choice
     if (amx_quant_gemm_workspace_bytes(M, N, K, group_size, flags) > kStaticScratchBytes) {
-        // group sizes other than 32 still fit on the plain kernel, which keeps no prepared operands
-        if (flags != AMX_GEMM_AUTO || group_size == 32 ||
-            amx_quant_gemm_workspace_bytes(M, N, K, group_size, AMX_GEMM_SIMT) > kStaticScratchBytes)
-            return AMX_ERR_TOO_LARGE;
-        flags = AMX_GEMM_SIMT;
+        // What keeps no prepared operands may still fit: the streaming kernel, for any other group size than 32 the plain one.
+        if (flags != AMX_GEMM_AUTO) return AMX_ERR_TOO_LARGE;
+        const size_t rows = quant_gemm_rows_bytes(M, N, K, group_size);
+        if (rows && rows <= kStaticScratchBytes) kernel = AMX_GEMM_ROWS;
+        else if (group_size != 32 && amx_quant_gemm_workspace_bytes(M, N, K, group_size, AMX_GEMM_SIMT) <= kStaticScratchBytes)
+            flags = AMX_GEMM_SIMT;
+        else return AMX_ERR_TOO_LARGE;
     }
     void* scratch = nullptr;
     const int rc = static_scratch(&scratch);
     if (rc != AMX_OK) return rc;
-    return amx_quant_gemm(A, ld_a, w_codes, w_scales, nullptr, 0, M, N, K, group_size, flags, C, ld_c, scratch,
-                          kStaticScratchBytes, stream);
+    return quant_gemm(A, ld_a, w_codes, w_scales, nullptr, 0, M, N, K, group_size, flags, kernel, C, ld_c, scratch, kStaticScratchBytes,
+                      stream);
 }
 
 // The status word of the most recent call on the current device (first word of the array).

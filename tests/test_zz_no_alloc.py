@@ -47,6 +47,15 @@ def test_static_scratch_entry_point_matches_workspace_entry_point_twice():
     assert torch.equal(_static(a, wc, ws, amx.GEMM_SIMT), amx.quant_gemm(a, wc, ws, 32, amx.GEMM_SIMT))
 
 
+def test_static_scratch_takes_few_rows_against_a_weight_larger_than_itself():
+    """AUTO would prepare the whole weight (53 MB) for the FP4 kernel here; the weight-streaming kernel needs no room for it."""
+    wc, ws = amx.quantize(_dev(inputs.weight(2, 0)), 32)
+    a = _dev(inputs.activation(2, 0, M=128))
+    assert amx.lib().amx_gemm_kernel_for(128, wc.shape[0], a.shape[1], 32, 0) == amx.GEMM_FP4
+    ref, g = (t.double().cpu().numpy() for t in (amx.quant_gemm(a, wc, ws, 32), _static(a, wc, ws)))
+    assert np.linalg.norm(g - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
 def test_static_scratch_entry_point_rejects_oversized_problems():
     L = amx.lib()
     M, N, K = 16384, 256, 4096                    # quantized activation alone is 36 MiB > 16 MiB
