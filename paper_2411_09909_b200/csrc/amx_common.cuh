@@ -48,7 +48,7 @@ inline bool programmatic_launch_ok(cudaStream_t st) {
 // That costs the longest of them 2-5 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
 // measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 170 and at 100 us.
 template <typename... P, typename... A>
-int launch_clusters(unsigned cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -60,10 +60,11 @@ int launch_clusters(unsigned cluster, bool chained, void (*kernel)(P...), dim3 g
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (cluster > 1) {
+    if (cluster.x * cluster.y * cluster.z > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = cluster;
-        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        attr[n].val.clusterDim.x = cluster.x;
+        attr[n].val.clusterDim.y = cluster.y;
+        attr[n].val.clusterDim.z = cluster.z;
         ++n;
     }
     cfg.attrs = attr;

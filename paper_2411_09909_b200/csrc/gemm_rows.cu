@@ -582,7 +582,7 @@ RowsKernel kernel_for(const RowsPlan& pl) {
     }
 }
 
-int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cudaStream_t st) {
+int launch_rows(RowsParams p, const RowsPlan& pl, int gs, cudaStream_t st) {
     const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl) : gs == 32 ? kernel_for<32>(pl) : gs == 64 ? kernel_for<64>(pl) : kernel_for<128>(pl);
     static bool configured[64][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
     int dev = 0;
@@ -597,34 +597,10 @@ int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cud
     }
     const int held = pl.steps_max < scale_steps(gs) ? pl.steps_max : scale_steps(gs);
     p.steps_max = pl.steps_max;
-    cudaLaunchConfig_t cfg = {};
     const int cta_rows = pl.stream ? kStreamRows : kCtaRows;
-    cfg.gridDim = dim3((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = pl.stream ? kernel.ring_bytes
-                                     : kernel.ring_bytes + (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    int n = 0;
-    if (pl.slices > 1) {
-        attr[n].id = cudaLaunchAttributeClusterDimension;
-        attr[n].val.clusterDim.x = 1;
-        attr[n].val.clusterDim.y = (unsigned)pl.slices;
-        attr[n].val.clusterDim.z = 1;
-        ++n;
-    }
-    if (programmatic) {
-        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n].val.programmaticStreamSerializationAllowed = 1;
-        ++n;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = n;
-    if (cudaLaunchKernelEx(&cfg, kernel.fn, p) != cudaSuccess) {
-        cudaGetLastError();
-        return AMX_ERR_CUDA;
-    }
-    return AMX_OK;
+    const dim3 grid((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
+    const size_t smem = kernel.ring_bytes + (pl.stream ? 0 : (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes);
+    return launch_clusters(dim3(1, (unsigned)pl.slices), true, kernel.fn, grid, kThreads, smem, st, p);
 }
 
 // Workspace: 256 bytes whose first word is the status word amx_gemm_status reads, then the fragments of the rows.
@@ -632,30 +608,17 @@ constexpr size_t kHeaderBytes = 256;
 
 template <bool CAST, int GS>
 int launch_fragments_gs(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int tiles,
-                        void* workspace, bool programmatic, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((K / 8 + 127) / 128), (unsigned)(tiles * kTok), 1);
-    cfg.blockDim = dim3(128, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = programmatic ? 1 : 0;
-    if (cudaLaunchKernelEx(&cfg, rows_fragments_kernel<CAST, GS>, codes, scales, x, ld_x, (int)M, tiles, K,
-                           reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes),
-                           static_cast<int*>(workspace)) != cudaSuccess) {
-        cudaGetLastError();
-        return AMX_ERR_CUDA;
-    }
-    return AMX_OK;
+                        void* workspace, cudaStream_t st) {
+    return launch(rows_fragments_kernel<CAST, GS>, dim3((unsigned)((K / 8 + 127) / 128), (unsigned)(tiles * kTok)), 128, 0, st, codes, scales,
+                  x, ld_x, (int)M, tiles, K, reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes),
+                  static_cast<int*>(workspace));
 }
 template <bool CAST>
 int launch_fragments(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int gs,
-                     int tiles, void* workspace, bool programmatic, cudaStream_t st) {
+                     int tiles, void* workspace, cudaStream_t st) {
     auto* fn = gs == 16 ? launch_fragments_gs<CAST, 16> : gs == 32 ? launch_fragments_gs<CAST, 32>
              : gs == 64 ? launch_fragments_gs<CAST, 64> : launch_fragments_gs<CAST, 128>;
-    return fn(codes, scales, x, ld_x, M, K, tiles, workspace, programmatic, st);
+    return fn(codes, scales, x, ld_x, M, K, tiles, workspace, st);
 }
 
 // x != nullptr: bf16 rows, cast here; otherwise quantized rows.
@@ -663,16 +626,14 @@ int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int
              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace,
              cudaStream_t st) {
     const RowsPlan pl = plan_rows(M, N, K);
-    const bool programmatic = programmatic_launch_ok(st);
     RowsParams p{};
     p.frag = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(workspace) + kHeaderBytes);
     p.w_codes = w_codes; p.w_scales = w_scales;
     p.M = (int)M; p.N = N; p.K = K; p.C = C; p.ld_c = ld_c;
-    const int rc = x ? launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, gs, pl.tiles(), workspace,
-                                              programmatic, st)
-                     : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, programmatic, st);
+    const int rc = x ? launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, gs, pl.tiles(), workspace, st)
+                     : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, st);
     if (rc != AMX_OK) return rc;
-    return launch_rows(p, pl, gs, programmatic, st);
+    return launch_rows(p, pl, gs, st);
 }
 
 }  // namespace
