@@ -135,22 +135,11 @@ __device__ __forceinline__ uint2 scale_entry(uint32_t b) {
     return make_uint2(__float_as_uint(cast::inv_scale(b)), b ? scale_norm(b) << 1 : 0x80000000u);
 }
 __device__ __forceinline__ uint32_t cast_group(const uint32_t (&w)[16], const uint2* tab, int key_ofs, uint32_t (&nib)[4], uint32_t& up) {
-    const uint32_t m0 = __vimax3_s16x2(w[0], w[1], w[2]), m1 = __vimax3_s16x2(w[3], w[4], w[5]), m2 = __vimax3_s16x2(w[6], w[7], w[8]),
-                   m3 = __vimax3_s16x2(w[9], w[10], w[11]), m4 = __vimax3_s16x2(w[12], w[13], w[14]);
-    uint32_t pm = __vimax3_s16x2(__vimax3_s16x2(m0, m1, m2), __vimax3_s16x2(m3, m4, w[15]), 0);
-    pm = __vmaxs2(pm, pm << 16) & 0xFFFF0000u;                    // the group maximum
-    const uint32_t sc = cast::cvt_e5m2x2(0.0f, cast::trunc12(__uint_as_float(pm) * cast::sixth_up())) & 0x7Fu;
+    const uint32_t sc = cast::nonneg_group_scale(w);
     const uint2 e = tab[sc];
-    const uint64_t inv2 = cast::pack_f32x2(e.x, e.x);
     const int t = (int)e.y + key_ofs;
     up = t >= 8 ? (uint32_t)t : 0u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        uint64_t q[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) q[i] = cast::mul_f32x2(cast::pack_f32x2(w[4 * j + i] << 16, w[4 * j + i] & 0xFFFF0000u), inv2);
-        nib[j] = cast::cvt_e2m1x8(q[0], q[1], q[2], q[3]);
-    }
+    cast::nonneg_group_codes(w, e.x, nib);
     return sc;
 }
 

@@ -237,14 +237,15 @@ __device__ __forceinline__ uint32_t emit_group(const uint32_t (&w)[16], int64_t 
 // minus everything the negative side needs.  nib: the group's 32 codes; returns the positive scale byte.
 // (The bf16 pairs are split with a shift and a mask here: this runs in the attention epilogue, where the logic pipe
 // has room and instruction issue is what counts.)
-__device__ __forceinline__ uint32_t cast_nonneg_group(const uint32_t (&w)[16], uint32_t (&nib)[4]) {
-    uint32_t pm = w[0];
-#pragma unroll
-    for (int i = 1; i + 1 < 16; i += 2) pm = __vimax3_s16x2(pm, w[i], w[i + 1]);
-    pm = __vmaxs2(pm, w[15]);
-    pm = __vmaxs2(pm, pm >> 16) & 0xFFFFu;                       // the group maximum's bf16 bits
-    const uint32_t sc = cvt_e5m2x2(0.0f, trunc12(__uint_as_float(pm << 16) * sixth_up())) & 0xFFu;
-    const uint32_t inv = __float_as_uint(inv_scale(sc));
+__device__ __forceinline__ uint32_t nonneg_group_scale(const uint32_t (&w)[16]) {
+    // (a tree: the attention kernel has the independent instructions to hide each other's latency)
+    const uint32_t m0 = __vimax3_s16x2(w[0], w[1], w[2]), m1 = __vimax3_s16x2(w[3], w[4], w[5]), m2 = __vimax3_s16x2(w[6], w[7], w[8]),
+                   m3 = __vimax3_s16x2(w[9], w[10], w[11]), m4 = __vimax3_s16x2(w[12], w[13], w[14]);
+    uint32_t pm = __vimax3_s16x2(__vimax3_s16x2(m0, m1, m2), __vimax3_s16x2(m3, m4, w[15]), 0);
+    pm = __vmaxs2(pm, pm << 16) & 0xFFFF0000u;                   // the group maximum
+    return cvt_e5m2x2(0.0f, trunc12(__uint_as_float(pm) * sixth_up())) & 0x7Fu;
+}
+__device__ __forceinline__ void nonneg_group_codes(const uint32_t (&w)[16], uint32_t inv /* fp32 bits of 1 / scale */, uint32_t (&nib)[4]) {
     const uint64_t inv2 = pack_f32x2(inv, inv);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -253,6 +254,10 @@ __device__ __forceinline__ uint32_t cast_nonneg_group(const uint32_t (&w)[16], u
         for (int i = 0; i < 4; ++i) q[i] = mul_f32x2(pack_f32x2(w[4 * j + i] << 16, w[4 * j + i] & 0xFFFF0000u), inv2);
         nib[j] = cvt_e2m1x8(q[0], q[1], q[2], q[3]);
     }
+}
+__device__ __forceinline__ uint32_t cast_nonneg_group(const uint32_t (&w)[16], uint32_t (&nib)[4]) {
+    const uint32_t sc = nonneg_group_scale(w);
+    nonneg_group_codes(w, __float_as_uint(inv_scale(sc)), nib);
     return sc;
 }
 // Stores the plane at group index v (and, when asked, the same word as the group's canonical codes: without a set
