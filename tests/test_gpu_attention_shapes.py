@@ -23,10 +23,11 @@ def dev(bits):
 
 
 def rows_agree(O, ref):
-    """Row by row: a probability that rounds to the neighbouring bf16 value can move its group's scale by a step, and with
-    it a whole row; anything wrong with the shapes moves many."""
+    """Row by row.  The oracle's exponentials are fp64 ones, so a probability may round to the neighbouring bf16 value, which
+    can move its group's scale by a step and with it the row (none of 44 000 rows of these inputs, drawn three times); the
+    other rows differ by fp32 additions alone, 1e-7.  Anything wrong at the edge of a tile moves a row of every head."""
     err = np.linalg.norm(O - ref, axis=1) / np.linalg.norm(ref, axis=1)
-    return np.mean(err > 2e-3) <= 0.1 and np.max(err) < 0.5
+    return np.sum(err > 1e-5) <= len(err) // 500 and np.max(err) < 0.5
 
 
 def reference(q, k, v, causal):
