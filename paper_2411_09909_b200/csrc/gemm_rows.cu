@@ -534,26 +534,24 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
         while (s < kMaxSlices && stream_blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
         return {true, tiles, 1, s, (int)((steps + s - 1) / s), 0.0};
     }
-    // Time in us, fitted to 320 calls (N 256 to 28672, K 512 to 16384, 40 to 256 rows; weights from HBM): 3.5 for the
-    // fragments and the start, then per wave of CTAs its steps' decode and MMAs, its own start and, with a cluster, the
-    // meeting at the end.  Within 10 % for blocks of 48 and 64 rows (35.2 us estimated, 36.0 measured for 64 rows of
-    // 12288 x 4096, 49.6 / 50.0 for 128 of 4096 x 11008).  Clusters of four and eight leave SMs of a GPC empty, those of three, five, six and seven
-    // more (4096 x 4096, 160 rows: three ranges 46.7 us, one 35.4).
-    // Up to 64 rows one block of tokens (the weight is read and decoded once); above, blocks of 64 or of 32 rows (of
-    // which two CTAs share an SM without being faster).
-    static constexpr struct { int slices, sms; } kFit[] = {{1, kSmCount}, {2, kSmCount}, {4, 132}, {8, 112}};
-    const int whole = tiles <= 6 ? 6 : 8;
+    // Time in us, fitted to 2100 calls with given layouts (39 weights of N 256 to 28672, K 512 to 16384, from HBM; 33 to 256
+    // rows): 3 for the fragments and the start, then per wave of CTAs its steps' decode and MMAs, its own start and, with a
+    // cluster, the meeting at the end.  Within 4 % on average for blocks of 48 and 64 rows, 9 % for 32; the layout it picks
+    // is within 1.2 % of the best on average.  (At most 64 rows: one block, the weight is read and decoded once.)  How many
+    // SMs a wave fills is what cudaOccupancyMaxActiveClusters answers for the cluster sizes: clusters of three and more leave
+    // SMs of a GPC empty.  64 rows of 5120 x 2560: three ranges 14.5 us, two 17.9, four (two waves) 21.6.  Blocks of 32 rows:
+    // two CTAs share an SM and take turns.
+    static constexpr int kSms[kMaxSlices] = {148, 148, 135, 132, 130, 132, 105, 120}, kSms32[kMaxSlices] = {148, 148, 139, 142, 140, 135, 129, 132};
     const int64_t row_blocks = (N + kCtaRows - 1) / kCtaRows;
     RowsPlan best{};
-    for (int nt = whole; nt >= 4; nt -= 4) {
-        if (nt != whole && tiles <= kMaxTiles) break;
+    for (int nt = 8; nt >= 4; nt -= 2) {
+        if (tiles <= kMaxTiles && nt != (tiles <= 6 ? 6 : 8)) continue;
         const int m_blocks = (tiles + nt - 1) / nt;
-        const double step = nt == 4 ? 0.69 : nt == 6 ? 0.78 : 0.91, start = nt == 4 ? 1.0 : 2.6, meeting = nt == 4 ? 3.0 : 3.9;
-        for (const auto& f : kFit) {
-            if (f.slices > steps) break;
-            const int64_t ctas = row_blocks * f.slices * m_blocks, n = (steps + f.slices - 1) / f.slices;
-            const double us = 3.5 + (double)((ctas + f.sms - 1) / f.sms) * ((double)n * step + (f.slices > 1 ? meeting : start));
-            if (!best.nt || us < best.us) best = {false, nt, m_blocks, f.slices, (int)n, us};
+        const double step = nt == 8 ? 0.93 : nt == 6 ? 0.78 : 0.72, start = nt == 4 ? 0.5 : 2.6, meeting = nt == 4 ? 3.5 : 4.3;
+        for (int s = 1; s <= kMaxSlices && s <= steps; ++s) {
+            const int64_t ctas = row_blocks * s * m_blocks, n = (steps + s - 1) / s, sms = (nt == 4 ? kSms32 : kSms)[s - 1];
+            const double us = 3.0 + (double)((ctas + sms - 1) / sms) * ((double)n * step + (s > 1 ? meeting : start));
+            if (!best.nt || us < best.us) best = {false, nt, m_blocks, s, (int)n, us};
         }
     }
     return best;
