@@ -321,8 +321,8 @@ def time_decode(steps: int, A=None, W=None):
               "frac_of_measured_copy": w_bytes / (d_us * 1e-6) / 1e9 / peaks["hbm_gbs"],
               "launches_per_step": 2 * len(layers),
               "us_per_step_more_rows": more_rows,
-              "kernel": ("weight-streaming kernel (canonical weights read once, exact bf16 decode, mma.sync; K ranges "
-                         "added over a thread-block cluster)" if decode_kernel == amx.GEMM_ROWS
+              "kernel": ("weight-streaming kernel (canonical weights read once, exact decode to f16, mma.sync; K split over a "
+                         "block's warps)" if decode_kernel == amx.GEMM_ROWS
                          else "tcgen05 kind::f16 (bf16 decode), K cut into slices over CTAs")}
     return decode
 

@@ -73,10 +73,11 @@ typedef enum amx_status {
 #define AMX_OUT_BF16 0x0u
 #define AMX_OUT_F32 0x1u
 /* flags for amx_gemm / amx_quant_gemm: kernel choice.  Default (AMX_GEMM_AUTO): at most 64 rows of A with K >= 512 and
- * K % 128 == 0 go to the weight-streaming kernel (AMX_GEMM_ROWS), as do up to 256 rows of a small product or against a
- * large weight (in blocks of rows); otherwise the FP4 kernel takes every fixed group size when M*N*K >= 2^27, the exact
- * bf16-decode tcgen05 kernel group size 32 below that (it cuts K into slices over CTAs when a product has few output
- * tiles and adds the partial products in slice order); what remains runs on the SIMT kernel.
+ * K % 128 == 0 go to the weight-streaming kernel (AMX_GEMM_ROWS), as do up to 256 rows where blocks of
+ * rows that each decode the weight again are still estimated faster than preparing it; otherwise the FP4 kernel takes
+ * every fixed group size when M*N*K >= 2^27, the exact bf16-decode tcgen05 kernel group size 32 below that (it cuts K
+ * into slices over CTAs when a product has few output tiles and adds the partial products in slice order); what remains
+ * runs on the SIMT kernel.
  * AUTO never loses a scale: where it picks the FP4 kernel and preparing the operands had to flush one (see
  * AMX_GEMM_FP4), the FP4 kernel returns at once and an exact kernel computes the product instead.
  * The decision is taken on the device, from the count amx_gemm_flushed_scales() reports; it costs one empty

@@ -45,8 +45,8 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // FP4 kernel would have to prepare the whole weight for them; the bf16-decode kernel slices K over CTAs.
     // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows, in blocks of 64
     // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route
-    // (fp4_route_us).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 23 / 40 and at 256 36 / 43, 12288 x 4096 at
-    // 96 rows 51 / 51 and at 128 64 / 54, 4096 x 11008 at 192 rows 78 / 86, 28672 x 4096 at 72 rows 123 / 81, 14336 x 512 at
+    // (fp4_route_us).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 23 / 41 and at 256 36 / 43, 12288 x 4096 at
+    // 96 rows 52 / 51 and at 128 58 / 54, 4096 x 11008 at 192 rows 72 / 86, 28672 x 4096 at 72 rows 106 / 82, 14336 x 512 at
     // 128 rows 17 / 20 and at 200 28 / 20.
     // A narrow weight (below 512 rows and 2^23 elements) stays on the FP4 route from 2^28 multiply-adds on, slower as it is
     // (256 x 8192 at 128 rows: 14 / 70): callers read the count of flushed scales that this route leaves in the workspace.

@@ -64,7 +64,7 @@ constexpr int kTmemSfCols = 96;
 // Shared-memory stage geometry: four stages of a K block each.  Two planes per operand: BK = 128 elements (64-byte rows), 48 KB
 // (K blocks of 256 elements in two stages measured slower).  ONE_PLANE (both operands in a symmetric format, one product per K
 // step): BK = 256 (128-byte rows); with 128 the tensor cores waited on copies of 1 KB and on a barrier round per two MMAs
-// (MXFP4 8192 x 14336 x 4096: 347 us against 226).  PAIR: the stage of one CTA of the pair, half of the W rows.
+// (MXFP4 8192 x 14336 x 4096: 347 us against 219).  PAIR: the stage of one CTA of the pair, half of the W rows.
 template <int BK_, bool ONE_PLANE = false, bool PAIR = false>
 struct Cfg {
     static constexpr int BK = BK_;
@@ -822,7 +822,7 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
         return r2 != AMX_OK ? r2 : reduce_slices(part, slices, M, N, C, ld_c, st);
     }
     // A pair of SMs per tile (256 x 256) where there is more than a tile for every SM: either SM loads half of the W rows.
-    // 2048 x 12288 x 4096: 159 -> 154 us, 16384 x 10240 x 8192: 1720 -> 1655 (less power for the operands, higher clocks).
+    // 2048 x 12288 x 4096: 159 -> 154 us; 16384 x 10240 x 8192: 1.4 % fewer cycles, the call 2 % shorter under the power cap.
     // With at most one tile per SM there is nothing to overlap the pair's longer start and end with (1024 x 4096 x 4096: 36 us
     // alone, 39 in pairs); an odd row block leaves half a pair idle, which a sixteenth of the rows may cost.
     const int64_t m_blocks = (M + BM - 1) / BM;

@@ -19,14 +19,21 @@
 // and a subtraction 7.4; the scale chosen by a sign mask 7.7; code bits shifted into bf16 fields and the scale chosen
 // by a mask (the earlier form) 8.7; the signs kept apart through two MMAs 7.1.
 //
-// A CTA of eight warps covers 128 weight rows and one range of K: warp = (row group of 32) + 4 * (parity of its
-// steps).  The codes come through a ring in shared memory by asynchronous copies, a slot per warp and step (a lane reads
-// back only its own copies; no registers are held by loads in flight): the copies alone stream at 5.4-5.8 TB/s.  The
-// scales of the whole range are copied once at the start, along the rows.  (Copied per step beside the codes, 8 bytes
-// per row at 32 different rows per instruction, they took more of the load path than the codes themselves: streaming
-// alone 7.5-9 instead of 4.7 us for 12288 x 4096.)  The K ranges of the same rows are the CTAs of one thread-block
-// cluster (up to 8), which add their partial products over distributed shared memory in rank order - deterministic,
-// no scratch in global memory and no second launch.
+// Two kernels share this: gemm_rows_stream_kernel for up to 32 tokens (a CTA covers 32 weight rows, its warps split K, no
+// cluster for the usual layers; described below) and gemm_rows_kernel for 33 and more, in blocks of 32, 48 or 64:
+// a CTA of eight warps covers 128 weight rows and one range of K, warp = (row group of 32) + 4 * (parity of its steps).
+// In both the codes come through a ring in shared memory by asynchronous copies, a slot per warp and step (a lane reads back
+// only its own copies; no registers are held by loads in flight): the copies alone stream at 5.4-5.8 TB/s.  Scales are
+// copied along the rows, many steps at a time.  (Copied per step beside the codes, 8 bytes per row at 32 different rows per
+// instruction, they took more of the load path than the codes themselves: streaming alone 7.5-9 instead of 4.7 us for
+// 12288 x 4096.)  The K ranges of the same rows are the CTAs of one thread-block cluster (up to 8), which add their partial
+// products over distributed shared memory in rank order - deterministic, no scratch in global memory and no second launch.
+//
+// What bounds it (counters of one call, weights from HBM): one row of 12288 x 4096 takes 16 us, 20 000 active cycles with
+// 58 % of the issue slots and 52 % of the logic pipe busy (decode), 40 MB into the SMs for 28 MB of weight; 24 rows of
+// 14336 x 4096 25 us, 33 000 cycles, issue slots 45 %, tensor pipe 28 %, 93 MB into the SMs for 33 MB of weight - the rest are
+// fragments, re-read by every CTA - and 448 CTAs on 296 places; 64 rows of 12288 x 4096 in the kernel of 128-row CTAs 38 us,
+// tensor pipe 55 % of the active cycles on 96 of 148 SMs.
 //
 // The token rows are cast (or decoded) once by a small kernel into the fragment order.  (Cast inside the main kernel by
 // every CTA, one launch less, measured the same for one row and slower for more.)

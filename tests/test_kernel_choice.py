@@ -1,12 +1,12 @@
 """What AMX_GEMM_AUTO picks between 65 and 256 rows, where both the weight-streaming kernel and the FP4 kernel take the call:
-the one that measured faster, at shapes where the two differ by more than a tenth (us, weights from HBM, one call)."""
+the one that measured faster, at shapes where the two differ by more than a twentieth (us, weights from HBM, one call)."""
 import pytest
 
 from paper_2411_09909_b200 import amx
 
 MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
-    (72, 28672, 4096, 109.6, 81.0), (128, 28672, 4096, 129.5, 89.2), (256, 28672, 4096, 224.2, 98.0),
-    (128, 12288, 4096, 64.0, 53.5), (256, 12288, 4096, 98.7, 62.2), (256, 6144, 4096, 64.0, 47.1), (160, 8192, 4096, 59.1, 48.2),
+    (72, 28672, 4096, 105.9, 81.8), (128, 28672, 4096, 129.0, 90.2), (256, 28672, 4096, 223.6, 97.4),
+    (128, 12288, 4096, 58.0, 54.3), (256, 12288, 4096, 98.2, 63.5), (256, 6144, 4096, 57.6, 46.0), (160, 8192, 4096, 59.1, 48.2),
     (72, 6144, 4096, 26.2, 40.0), (128, 8192, 4096, 35.8, 47.7), (192, 6144, 4096, 36.1, 45.3), (256, 4096, 4096, 36.2, 43.4),
     (128, 4096, 4096, 23.5, 41.4), (128, 4096, 11008, 50.0, 85.1), (72, 4096, 14336, 62.2, 103.2), (128, 4096, 14336, 62.3, 107.8),
     (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (192, 256, 4096, 11.0, 40.7), (72, 12288, 640, 11.9, 21.3),
