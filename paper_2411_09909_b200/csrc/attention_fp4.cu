@@ -84,7 +84,11 @@ __host__ __device__ constexpr int s_buffers(int pass) { return epi_groups(pass);
 __host__ __device__ constexpr int threads(int pass) { return (kFirstEpi + 8 * epi_groups(pass)) * 32; }
 constexpr int kParts = 2 * epi_groups(kPassStats);    // partial row statistics: a thread's columns of its group's tiles
 static_assert(epi_groups(kPassMax) == epi_groups(kPassStats), "kParts");
-constexpr int kSumTiles = 8, kSumParts = 8;           // ordered sums: per 8 key tiles {even, odd tiles} x 4 groups of a tile
+// Ordered sums: per 8 key tiles {even, odd tiles} x 4 groups of a tile.  Past 8192 keys (64 tiles) the stored path adds in another
+// order anyway: then once per row, so that the scratch does not grow with the square of the length.
+constexpr int kSumParts = 8;
+__host__ __device__ constexpr int sum_shift(int64_t tiles) { return tiles <= 64 ? 3 : 30; }
+__host__ __device__ constexpr int64_t sum_blocks(int64_t tiles) { return (tiles + (1 << sum_shift(tiles)) - 1) >> sum_shift(tiles); }
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kPlane = 128 * 64;                      // one sign plane of a 128 x 128 tile: 64-byte rows
 constexpr int kTileBytes = 2 * kPlane;                // {+, -}
@@ -158,7 +162,8 @@ struct Params {
     const int* gate;         // not NULL: nothing is done when this word is nonzero (the caller runs the exact kernel then)
     float2* part;            // online: [heads * Lp][kParts]: per row {max, sum of 2^(t - max)}, base-2 units
     float* row_max;          // ordered: [kParts][heads * Lp]: maxima of t = alpha s
-    float* sums;             // ordered: [heads][tiles / kSumTiles][kSumParts][Lp]: sums of exp(t - max) of a key group's tiles
+    float* sums;             // ordered: [heads][sum_blocks][kSumParts][Lp]: sums of exp(t - max) of a key group's tiles
+    int sum_shift;           // tiles of a block, log2
     float* O;                // map pass out: [heads][L][head dimension]
     int* status;
     // optional outputs of the online map pass for head 0 of the launch (verification): the bf16 map the cast started from
@@ -435,8 +440,8 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                     // the stored path's order: over 32 groups a tree by strides 16, 8, 4, 2, 1 (the first two inside `sums`),
                     // then along the row
                     float sum = 0.f;
-                    const float* sp = p.sums + (int64_t)h * ((p.m_tiles + kSumTiles - 1) / kSumTiles) * kSumParts * p.Lp + m;
-                    for (int t0 = 0; t0 < T; t0 += kSumTiles, sp += kSumParts * p.Lp) {
+                    const float* sp = p.sums + (int64_t)h * sum_blocks(p.m_tiles) * kSumParts * p.Lp + m;
+                    for (int t0 = 0; t0 < T; t0 += 1 << p.sum_shift, sp += kSumParts * p.Lp) {
                         float c[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -611,9 +616,9 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                 if (kGroups == 2) work(cg0);
                 scale_columns(cg0 + 1);
                 work(cg0 + 1);
-                if (PASS == kPassSum && ((j >> 1) % 4 == 3 || j + 2 >= T)) {   // its last tile of these eight
-                    float* sp = p.sums + (((int64_t)h * ((p.m_tiles + kSumTiles - 1) / kSumTiles) + j / kSumTiles) * kSumParts +
-                                          (j & 1) * 4 + cg0) * p.Lp + m;
+                const int last = (1 << p.sum_shift) - 2;
+                if (PASS == kPassSum && ((j & (last + 1)) >= last || j + 2 >= T)) {   // its last tile of the block
+                    float* sp = p.sums + (((int64_t)h * sum_blocks(p.m_tiles) + (j >> p.sum_shift)) * kSumParts + (j & 1) * 4 + cg0) * p.Lp + m;
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         sp[i * p.Lp] = even[i] + odd[i];
@@ -709,8 +714,8 @@ int64_t attn_fused_padded(int64_t L) { return (L + BM - 1) / BM * BM; }
 
 // per-row partial softmax statistics of the heads of one launch
 size_t attn_fused_scratch_bytes(int64_t heads, int64_t L, bool ordered) {
-    const int64_t rows = heads * attn_fused_padded(L), eights = (attn_fused_padded(L) / BNK + kSumTiles - 1) / kSumTiles;
-    return up256((size_t)rows * (ordered ? (kParts + eights * kSumParts) * sizeof(float) : kParts * sizeof(float2)));
+    const int64_t rows = heads * attn_fused_padded(L), blocks = sum_blocks(attn_fused_padded(L) / BNK);
+    return up256((size_t)rows * (ordered ? (kParts + blocks * kSumParts) * sizeof(float) : kParts * sizeof(float2)));
 }
 
 namespace {
@@ -774,6 +779,7 @@ int attn_fused(const Fp4Operand& q, const Fp4Operand& k, const Fp4Operand& vt, i
     p.part = static_cast<float2*>(scratch);
     p.row_max = static_cast<float*>(scratch);
     p.sums = p.row_max + kParts * heads * p.Lp;
+    p.sum_shift = sum_shift(p.m_tiles);
     p.O = O;
     p.vec_o = aligned(O, 16);
     p.status = status;

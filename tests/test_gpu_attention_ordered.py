@@ -38,6 +38,25 @@ def test_fused_attention_equals_the_stored_path(heads, kv, L, d, flags, causal):
 
 
 @pytest.mark.parametrize("causal", [0, amx.ATTN_CAUSAL])
+@pytest.mark.parametrize("L,d", [(8224, 128), (9216, 64)])
+def test_rows_past_the_ordered_sums(L, d, causal):
+    """Past 8192 keys both paths add in orders of their own: a row may take another bf16 value (up to 1 in 10 000 above; here
+    1 in 1000), anything wrong with the one block of sums moves all of them."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(L)
+    q, k, v = (torch.randn(1, L, d, device="cuda", generator=g).to(torch.bfloat16) for _ in range(3))
+    got = amx.attention_heads(q, k, v, causal).double()
+    want = amx.attention_heads(q, k, v, amx.GEMM_TC | causal).double()
+    err = (got - want).norm(dim=2) / want.norm(dim=2)
+    assert (err > TOL).double().mean().item() <= 1e-3 and err.max().item() < 0.5
+
+
+def test_scratch_of_long_rows_stays_linear():
+    need = [amx.lib().amx_attention_workspace_bytes_for(L, 64, 0) for L in (65536, 131072)]
+    assert need[1] <= 2.1 * need[0]
+
+
+@pytest.mark.parametrize("causal", [0, amx.ATTN_CAUSAL])
 def test_exact_attention_kernel_equals_the_stored_path(causal):
     """A scale the FP4 kernel cannot hold sends AUTO to the kernel on CUDA cores: the same softmax once more.  The wide row's
     largest element meets zeros in Q, so that the logits are sums of few binades: the same numbers in any order."""
