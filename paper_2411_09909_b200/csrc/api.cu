@@ -74,6 +74,19 @@ size_t kernel_workspace(uint32_t kernel, int64_t M, int64_t N, int64_t K, bool f
     return 0;
 }
 
+// Whether a call under AUTO whose operands miss the alignment of the kernel it picked (16 bytes for codes, 4 for the scales that
+// the streaming kernel copies) runs on the plain kernel, which needs neither alignment nor scratch; else it is refused.
+// Which shapes of groups of 32 are taken with neither alignment is fixed here, apart from the estimates above, so that what is
+// accepted does not move with them.
+bool plain_for_alignment(uint32_t kernel, bool codes16, bool scales4, int64_t M, int64_t N, int64_t K, int gs) {
+    if (gs != 32 && !codes16) return true;
+    if (scales4) return false;
+    if (codes16) return kernel == AMX_GEMM_ROWS;
+    const double mnk = (double)M * (double)N * (double)K;
+    return gemm_rows_supported(M, N, K, gs) && K >= 512 &&
+           (M <= 64 || mnk < 268435456.0 || (mnk < 536870912.0 && N >= 512) || N * K >= (1ll << 23));
+}
+
 struct QuantSizes {
     size_t codes, scales;
 };
@@ -146,10 +159,8 @@ extern "C" int amx_gemm(const uint8_t* a_codes, const uint8_t* a_scales, const u
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (kernel == AMX_GEMM_SIMT)
         return gemm_simt({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, group_size, C, ld_c, st);
-    // AUTO picked a kernel whose alignment the operands miss (the weight-streaming kernel copies scales 4 bytes at a time;
-    // 16-byte codes for group sizes that used to run on the plain kernel): the plain kernel takes them and needs no scratch
     const bool codes16 = aligned(a_codes, 16) && aligned(w_codes, 16), is_auto = (flags & kKernelMask) == AMX_GEMM_AUTO;
-    if (is_auto && ((kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) || (group_size != 32 && !codes16)))
+    if (is_auto && plain_for_alignment(kernel, codes16, aligned(w_scales, 4), M, N, K, group_size))
         return gemm_simt({a_codes}, a_scales, {w_codes}, w_scales, M, N, K, group_size, C, ld_c, st);
     if (!codes16 || (kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4))) return AMX_ERR_ALIGN;
     const bool fallback = auto_fallback(flags, kernel);
@@ -270,10 +281,9 @@ int amx::quant_gemm(const void* A, int64_t ld_a, const uint8_t* w_codes, const u
     if (!A || !C || (w_is_bf16 ? (w_codes || w_scales) : (!w_codes || !w_scales))) return AMX_ERR_NULL;
     if (!workspace || workspace_bytes < quant_gemm_bytes(kernel, auto_fallback(flags, kernel), M, N, K, group_size, w_is_bf16))
         return AMX_ERR_WORKSPACE;
-    // as in amx_gemm: operands that miss the alignment of the kernel AUTO picked run on the plain kernel (with groups of
-    // 32 and at most 64 rows they are refused, as documented at AMX_GEMM_ROWS)
+    // as in amx_gemm (with groups of 32 and at most 64 rows misaligned operands are refused, as documented at AMX_GEMM_ROWS)
     if (flags == AMX_GEMM_AUTO && !w_is_bf16 && !(group_size == 32 && M <= 64) &&
-        ((kernel == AMX_GEMM_ROWS && !aligned(w_scales, 4)) || (group_size != 32 && !aligned(w_codes, 16))))
+        plain_for_alignment(kernel, aligned(w_codes, 16), aligned(w_scales, 4), M, N, K, group_size))
         kernel = AMX_GEMM_SIMT;
     const int code_align = kernel == AMX_GEMM_SIMT ? 4 : 16;
     if (!aligned(workspace, kAlign) || !aligned(A, 16) || ld_a % 8 || !aligned(C, 4) ||
