@@ -43,12 +43,9 @@ inline bool programmatic_launch_ok(cudaStream_t st) {
     return cs == cudaStreamCaptureStatusNone;
 }
 
-// chained = false: an ordinary launch.  For long kernels with one block per SM: started while their predecessor leaves, the
-// blocks land on the SMs in another order (operands shared by neighbouring tiles cross the two halves of the L2 more often).
-// That costs the longest of them 2-5 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
-// measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 170 and at 100 us.
+// One launch; programmatic: with the edge described above (never on a stream that is being captured).
 template <typename... P, typename... A>
-int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+int launch_with(dim3 cluster, bool programmatic, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -56,7 +53,7 @@ int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid,
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     unsigned n = 0;
-    if (chained && programmatic_launch_ok(st)) {
+    if (programmatic) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }
@@ -74,6 +71,15 @@ int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid,
         return AMX_ERR_CUDA;
     }
     return AMX_OK;
+}
+
+// chained = false: an ordinary launch.  For long kernels with one block per SM: started while their predecessor leaves, the
+// blocks land on the SMs in another order (operands shared by neighbouring tiles cross the two halves of the L2 more often).
+// That costs the longest of them 2-5 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
+// measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 170 and at 100 us.
+template <typename... P, typename... A>
+int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_with(cluster, chained && programmatic_launch_ok(st), kernel, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
 template <typename... P, typename... A>

@@ -20,9 +20,10 @@ constexpr uint32_t kKernelMask = AMX_GEMM_SIMT | AMX_GEMM_TC | AMX_GEMM_FP4 | AM
 // Time of the FP4 route under AUTO for 65 to 256 rows, us: preparation of the whole weight, one or two waves of tiles, the result,
 // and the gated exact kernel behind it, whose reduction (groups of 32, K from 1024, less than a wave of tiles) is a launch of
 // M N / 256 blocks even when it has nothing to do.  Fitted to 320 calls of 31 weights, within 20 % from 2^21 weight elements on.
-double fp4_route_us(int64_t M, int64_t N, int64_t K, int gs) {
-    const double mn = (double)M * (double)N;
-    const bool second_wave = ((M + 127) / 128) * ((N + 255) / 256) > 148;
+// Taken at M = 128: with the streaming kernel's time growing with the rows, the choice then changes once as rows are added.
+double fp4_route_us(int64_t N, int64_t K, int gs) {
+    const double mn = 128.0 * (double)N;
+    const bool second_wave = (N + 255) / 256 > 148;
     return 12.5 + 5.6e-3 * (double)K + 3.2e-7 * (double)N * (double)K + 1.4e-6 * mn + (second_wave ? 4.7 : 0.0) +
            (gs == 32 && K >= 1024 && !second_wave ? 2.7e-6 * mn : 0.0);
 }
@@ -52,7 +53,7 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // (256 x 8192 at 128 rows: 14 / 70): callers read the count of flushed scales that this route leaves in the workspace.
     const double mnk = (double)M * (double)N * (double)K;
     const bool narrow = N < 512 && N * K < (1ll << 23) && mnk >= 268435456.0;
-    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_route_us(M, N, K, gs)))) return AMX_GEMM_ROWS;
+    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_route_us(N, K, gs)))) return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
     // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)

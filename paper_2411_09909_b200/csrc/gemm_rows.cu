@@ -587,7 +587,7 @@ RowsKernel kernel_for(const RowsPlan& pl) {
     }
 }
 
-int launch_rows(RowsParams p, const RowsPlan& pl, int gs, cudaStream_t st) {
+int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cudaStream_t st) {
     const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl) : gs == 32 ? kernel_for<32>(pl) : gs == 64 ? kernel_for<64>(pl) : kernel_for<128>(pl);
     static bool configured[64][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
     int dev = 0;
@@ -605,7 +605,7 @@ int launch_rows(RowsParams p, const RowsPlan& pl, int gs, cudaStream_t st) {
     const int cta_rows = pl.stream ? kStreamRows : kCtaRows;
     const dim3 grid((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
     const size_t smem = kernel.ring_bytes + (pl.stream ? 0 : (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes);
-    return launch_clusters(dim3(1, (unsigned)pl.slices), true, kernel.fn, grid, kThreads, smem, st, p);
+    return launch_with(dim3(1, (unsigned)pl.slices), programmatic, kernel.fn, grid, kThreads, smem, st, p);
 }
 
 // Workspace: 256 bytes whose first word is the status word amx_gemm_status reads, then the fragments of the rows.
@@ -613,17 +613,17 @@ constexpr size_t kHeaderBytes = 256;
 
 template <bool CAST, int GS>
 int launch_fragments_gs(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int tiles,
-                        void* workspace, cudaStream_t st) {
-    return launch(rows_fragments_kernel<CAST, GS>, dim3((unsigned)((K / 8 + 127) / 128), (unsigned)(tiles * kTok)), 128, 0, st, codes, scales,
-                  x, ld_x, (int)M, tiles, K, reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes),
-                  static_cast<int*>(workspace));
+                        void* workspace, bool programmatic, cudaStream_t st) {
+    return launch_with(1, programmatic, rows_fragments_kernel<CAST, GS>, dim3((unsigned)((K / 8 + 127) / 128), (unsigned)(tiles * kTok)), 128, 0,
+                       st, codes, scales, x, ld_x, (int)M, tiles, K, reinterpret_cast<uint4*>(static_cast<uint8_t*>(workspace) + kHeaderBytes),
+                       static_cast<int*>(workspace));
 }
 template <bool CAST>
 int launch_fragments(const uint8_t* codes, const uint8_t* scales, const uint16_t* x, int64_t ld_x, int64_t M, int64_t K, int gs,
-                     int tiles, void* workspace, cudaStream_t st) {
+                     int tiles, void* workspace, bool programmatic, cudaStream_t st) {
     auto* fn = gs == 16 ? launch_fragments_gs<CAST, 16> : gs == 32 ? launch_fragments_gs<CAST, 32>
              : gs == 64 ? launch_fragments_gs<CAST, 64> : launch_fragments_gs<CAST, 128>;
-    return fn(codes, scales, x, ld_x, M, K, tiles, workspace, st);
+    return fn(codes, scales, x, ld_x, M, K, tiles, workspace, programmatic, st);
 }
 
 // x != nullptr: bf16 rows, cast here; otherwise quantized rows.
@@ -631,14 +631,16 @@ int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int
              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace,
              cudaStream_t st) {
     const RowsPlan pl = plan_rows(M, N, K);
+    const bool programmatic = programmatic_launch_ok(st);      // asked once for both launches
     RowsParams p{};
     p.frag = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(workspace) + kHeaderBytes);
     p.w_codes = w_codes; p.w_scales = w_scales;
     p.M = (int)M; p.N = N; p.K = K; p.C = C; p.ld_c = ld_c;
-    const int rc = x ? launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, gs, pl.tiles(), workspace, st)
-                     : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, st);
+    const int rc = x ? launch_fragments<true>(nullptr, nullptr, static_cast<const uint16_t*>(x), ld_x, M, K, gs, pl.tiles(), workspace,
+                                              programmatic, st)
+                     : launch_fragments<false>(a_codes, a_scales, nullptr, 0, M, K, gs, pl.tiles(), workspace, programmatic, st);
     if (rc != AMX_OK) return rc;
-    return launch_rows(p, pl, gs, st);
+    return launch_rows(p, pl, gs, programmatic, st);
 }
 
 }  // namespace
@@ -649,7 +651,9 @@ bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs) {
 }
 
 size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K) {
-    return kHeaderBytes + (size_t)plan_rows(M, N, K).tiles() * kTok * (size_t)K * 2;
+    // (blocks of 32, 48 or 64 rows round M up differently: what suffices for M rows on this kernel also suffices for fewer)
+    const int64_t rows = (int64_t)plan_rows(M, N, K).tiles() * kTok, whole = M > 64 ? (M + 63) / 64 * 64 : 0;
+    return kHeaderBytes + (size_t)(rows > whole ? rows : whole) * (size_t)K * 2;
 }
 
 double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) { return plan_rows(M, N, K).us; }

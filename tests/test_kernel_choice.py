@@ -30,3 +30,15 @@ def test_narrow_weights_keep_the_route_that_counts_flushed_scales():
 def test_up_to_64_rows_stream_the_weight(M):
     for N, K in ((28672, 4096), (4096, 14336), (12288, 4096), (128, 512)):
         assert amx.lib().amx_gemm_kernel_for(M, N, K, 32, amx.GEMM_AUTO) == amx.GEMM_ROWS
+
+
+@pytest.mark.parametrize("gs", [16, 32, 128])
+@pytest.mark.parametrize("N,K", [(512, 512), (1024, 4096), (4096, 4096), (12288, 4096), (28672, 1024), (28672, 512), (4096, 14336), (768, 8192),
+                                 (16384, 2048), (5120, 2560)])
+def test_the_choice_changes_once_as_rows_are_added(N, K, gs):
+    """And within the streaming kernel's range no call needs more scratch than one of more rows."""
+    L = amx.lib()
+    kernels = [L.amx_gemm_kernel_for(M, N, K, gs, 0) for M in range(1, 257)]
+    assert kernels == sorted(kernels, reverse=True)                     # GEMM_ROWS (0x100), then GEMM_FP4 (0x40)
+    need = [L.amx_quant_gemm_workspace_bytes(M + 1, N, K, gs, 0) for M, k in enumerate(kernels) if k == amx.GEMM_ROWS]
+    assert need == sorted(need)
