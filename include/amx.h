@@ -293,7 +293,8 @@ int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, int64_t ld_
  *       products run on the FP4 kernel (AMX_GEMM_AUTO: from L * L * d >= 2^25) and d is 64 or 128, S is not stored
  *       either: one fused kernel does both products and the softmax - passes over Q K^T that keep per-row softmax
  *       statistics, then one that recomputes each tile, normalises and casts it in registers and multiplies it with V
- *       on the tensor cores.  P has the bits of amx_softmax_quantize on a stored S (up to 8192 keys), except with
+ *       on the tensor cores.  P has the bits of amx_softmax_quantize on a stored S (up to 8192 keys; where the logits'
+ *       sums are exact in fp32, as they are but for scales many binades apart), except with
  *       d = 128, L % 128 == 0 and either AMX_GEMM_FP4 or L * L * d >= 2^28: there the statistics take one pass, with
  *       another order of the row sum, and single elements of P may round to the neighbouring bf16 value, which can move
  *       the scale of its group and with it that row of O.  Other shapes and kernels store one head's S in the workspace.

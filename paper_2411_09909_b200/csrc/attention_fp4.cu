@@ -13,8 +13,8 @@
 //   ordered  (ragged lengths, head dimension 64, short sequences: wherever these products also exist with the logits in
 //            global memory) a pass for the maxima, then one for the sums: same argument t log2(e) - max log2(e) with
 //            t = alpha s rounded, same order of additions as softmax_math.cuh, hence the bits of the stored path.  The
-//            logits are the same numbers too: a sum of head-dimension-many products of E2M1 codes under E5M2 scales needs
-//            fewer than 24 bits.  (Online sums moved up to 3 rows of 33792 at 32 over 8 heads x 1056, now and then an element
+//            logits are the same numbers too: a sum of head-dimension-many products of E2M1 codes under E5M2 scales a few
+//            binades apart needs fewer than 24 bits.  (Online sums moved up to 3 rows of 33792 at 32 over 8 heads x 1056, now and then an element
 //            by half of the result's rms; the second statistics pass takes 12 of 75 us there, 130 of 680 at 4000 keys.)
 //   online   (long whole blocks at head dimension 128) one pass keeps a running maximum and a rescaled sum, log2(e) folded
 //            into the column factors: a pass less.
