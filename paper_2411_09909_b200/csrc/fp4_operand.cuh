@@ -72,5 +72,19 @@ inline bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The scale factors of a prepared operand as one 3-D tensor [2 planes][blocks of 128 rows][K / 64 chunks of 512 bytes], in
+// elements of 8 bytes; box = {steps chunks, blocks, planes}, zero fill outside.
+inline bool make_sf_map(CUtensorMap* map, const uint8_t* prepared, const OperandLayout& o, int steps, int blocks, int planes) {
+    EncodeTiledFn fn = encode_tiled();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)o.nk64 * (kSfChunk / 8), (cuuint64_t)o.row_blocks, 2};
+    const cuuint64_t strides[2] = {(cuuint64_t)o.nk64 * kSfChunk, (cuuint64_t)o.sf};
+    const cuuint32_t box[3] = {(cuuint32_t)(steps * (kSfChunk / 8)), (cuuint32_t)blocks, (cuuint32_t)planes};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_INT64, 3, const_cast<uint8_t*>(prepared) + 2 * o.plane, dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace fp4
 }  // namespace amx

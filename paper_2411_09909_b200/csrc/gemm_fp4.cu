@@ -14,10 +14,11 @@
 // in the epilogue (exact).  Scales more than 14 binades below their row's largest scale do not fit
 // and are flushed to zero: their groups contribute less than 2^-14 of the row's largest group.
 //
-// Persistent CTAs (one per SM) walk over 128 x 256 tiles of C - pairs of CTAs over 256 x 256 tiles (PAIR below) -; K blocks
-// cycle through four shared-memory stages:
+// Persistent CTAs (one per SM) walk over 128 x 256 tiles of C - pairs of CTAs over 256 x 256 tiles (PAIR below) -; the tiles
+// that would leave most of a last wave idle are cut into halves or quarters of their columns.  K blocks cycle through four
+// shared-memory stages (five in a pair):
 //   warp 0   TMA producer: per stage one 3-D tile {A+, A-} and one {W+, W-} (64-byte swizzle),
-//            completion on the stage's `full` mbarrier
+//            completion on the stage's `full` mbarrier, and the scale factors of either on `sf_full`
 //   warp 1   allocates TMEM; one lane issues the stage's MMAs (4 sign pairs x K steps of 64), then
 //            commits to the stage's `empty` mbarrier
 //   warps 2-9  (two groups of four, alternating K blocks) move each stage's scale factors, which come with its tiles, shared
@@ -34,6 +35,7 @@
 
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include "cast_math.cuh"
 #include "fp4_operand.cuh"
@@ -61,7 +63,8 @@ constexpr int kAccWindow = 160;        // first column of the odd tiles' accumul
 constexpr uint32_t kTmemSf = 416;      // scale-factor columns
 constexpr int kTmemSfCols = 96;
 
-// Shared-memory stage geometry: four stages of a K block each.  Two planes per operand: BK = 128 elements (64-byte rows), 48 KB
+// Shared-memory stage geometry: four stages of a K block each, five in a pair (four there: MXFP4 8192 x 14336 x 4096 240 us for
+// the call, five 223).  Two planes per operand: BK = 128 elements (64-byte rows), 48 KB
 // (K blocks of 256 elements in two stages measured slower).  ONE_PLANE (both operands in a symmetric format, one product per K
 // step): BK = 256 (128-byte rows); with 128 the tensor cores waited on copies of 1 KB and on a barrier round per two MMAs
 // (MXFP4 8192 x 14336 x 4096: 347 us against 219).  PAIR: the stage of one CTA of the pair, half of the W rows.
@@ -71,7 +74,7 @@ struct Cfg {
     static constexpr int kPlanes = ONE_PLANE ? 1 : 2;
     static constexpr int kRowBytes = BK / 2;
     static constexpr int kSteps = BK / 64;                            // MMAs (K = 64) per K block and sign pair
-    static constexpr int kStages = 4;
+    static constexpr int kStages = PAIR ? 5 : 4;
     static constexpr int kTileA = BM * kRowBytes, kTileB = BN / (PAIR ? 2 : 1) * kRowBytes;   // one plane
     static constexpr int kOffAp = 0, kOffAn = ONE_PLANE ? 0 : kTileA, kOffWp = kPlanes * kTileA,
                          kOffWn = kOffWp + (ONE_PLANE ? 0 : kTileB);
@@ -88,7 +91,7 @@ struct Cfg {
     static_assert(kAccWindow + BN <= (int)kTmemSf && kTmemSf + kSfSlots * kSfCols <= kTmemCols, "tensor memory map");
     static_assert(BK == 128 || BK == 256, "rows of 64 or 128 bytes, swizzled over their length");
 };
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 5;
 
 struct __align__(16) Control {
     uint64_t full[kMaxStages], empty[kMaxStages], sf_full[kMaxStages], accum_full;
@@ -180,7 +183,6 @@ scale_factors_kernel(const uint8_t* __restrict__ scales, int64_t R, int64_t K, i
 
 // -------------------------------------------------------------------------------- GEMM --
 struct Params {
-    const uint8_t *sfa_pos, *sfa_neg, *sfb_pos, *sfb_neg;
     const int *a_exp, *w_exp;
     int64_t M, N, K, ld_c;
     int64_t a_row0, w_row0;      // first rows of this product's operands inside the (stacked) prepared operands
@@ -189,6 +191,7 @@ struct Params {
     int nk64, vec_store;
     int out_bf16;                // C holds bf16 (each fp32 result rounded to nearest even) instead of fp32
     int band;                    // tile order: row blocks of A per band, see blk_m / blk_n
+    int whole, split_log2;       // tail: work items below `whole` are tiles, the others 1 / 2^split_log2 of a tile's columns
     int slices;                  // SLICED instantiation: K is cut into this many ranges, each (tile, range) a work item
     int64_t slice_stride;        //   whose partial product goes to C + range * slice_stride
     int* status;
@@ -241,13 +244,14 @@ __device__ __forceinline__ void store_row16_bf16(__nv_bfloat16* out, const float
 template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false, bool PAIR = false>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-                const __grid_constant__ CUtensorMap tm_a1, const __grid_constant__ CUtensorMap tm_w1, const Params p) {
-    grid_dependency_wait();
+                const __grid_constant__ CUtensorMap tm_a1, const __grid_constant__ CUtensorMap tm_w1,
+                const __grid_constant__ CUtensorMap tm_wt, const __grid_constant__ CUtensorMap tm_wt1,
+                const __grid_constant__ CUtensorMap tm_sfa, const __grid_constant__ CUtensorMap tm_sfw, const Params p) {
     using C_ = Cfg<BK_, ONE_PLANE, PAIR>;
     constexpr int kPlanes = C_::kPlanes;
-    if (p.gate && *p.gate != 0) return;                          // uniform over the grid: nothing was set up yet
     constexpr int BNT = NHALF ? BN / 2 : BN;                     // tile width
-    constexpr int kOffWnT = NHALF ? C_::kOffWp + C_::kTileB / 2 : C_::kOffWn;   // the box packs its two planes
+    constexpr uint32_t kOffWnT = NHALF ? C_::kOffWp + C_::kTileB / 2 : C_::kOffWn;   // the box packs its two planes
+    constexpr int kTileWT = NHALF ? C_::kTileB / 2 : C_::kTileB;   // one plane of the W tile as loaded (PAIR: of this CTA's half)
     constexpr uint32_t kIdescT = PAIR ? instr_desc(BNT) + ((uint32_t)(BM >> 4) << 24) : instr_desc(BNT);   // PAIR: M = 256
     constexpr int BMT = PAIR ? 2 * BM : BM;                      // tile height: of the pair
     const int rank = PAIR ? (int)(blockIdx.x & 1) : 0, worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x,
@@ -268,6 +272,15 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     // Persistent CTA: tiles blockIdx.x, blockIdx.x + gridDim.x, ...; neighbouring tiles share their A rows.
     const int64_t n_tiles = (p.N + BNT - 1) / BNT, m_tiles = (p.M + BMT - 1) / BMT;
     const int64_t total_tiles = m_tiles * n_tiles * S;
+    // Work items: the first `whole` tiles, then the parts of the tiles that are left after the last whole wave (each
+    // 1 / 2^split_log2 of a tile's columns, at most one for a CTA: its last item).
+    constexpr bool kSplits = !SLICED && !NHALF;
+    const int64_t whole = kSplits ? p.whole : total_tiles;
+    auto part_log2 = [&](int64_t item) -> int { return kSplits && item >= whole ? p.split_log2 : 0; };
+    auto tile_of = [&](int64_t item) { return kSplits && item >= whole ? whole + ((item - whole) >> p.split_log2) : item; };
+    auto part_col = [&](int64_t item) -> int {                   // first column of an item inside its tile
+        return kSplits && item >= whole ? (int)((item - whole) & ((1 << p.split_log2) - 1)) * (BNT >> p.split_log2) : 0;
+    };
     // Tile order.  The CTAs work on ~148 consecutive tiles at a time and advance through K roughly together, so what
     // they read from DRAM per wave is the operand rows the wave touches, once.  Tiles are ordered in bands of
     // p.band row blocks of A: inside a band the tile index walks down the band's row blocks first, then along N.
@@ -277,8 +290,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     // 16384 x 10240 x 8192.  A band as tall as the matrix is the plain "down M first" order (small M).
     // (two 32-bit divisions per call: the host rejects products with 2^31 tiles or more)
     const uint32_t band = (uint32_t)p.band, per_band = band * (uint32_t)n_tiles;
-    auto banded = [&](int64_t tile, uint32_t& m, uint32_t& n) {
-        const uint32_t t = (uint32_t)tile / (uint32_t)S, b = t / per_band, r = t - b * per_band;
+    auto banded = [&](int64_t item, uint32_t& m, uint32_t& n) {
+        const uint32_t t = (uint32_t)tile_of(item) / (uint32_t)S, b = t / per_band, r = t - b * per_band;
         const uint32_t rows_here = min(band, (uint32_t)m_tiles - b * band);      // the last band may be shorter
         n = r / rows_here;
         m = b * band + (r - n * rows_here);
@@ -325,6 +338,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     if (PAIR) cluster_sync();                                    // the other CTA's barriers are there before they are used
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
+    // Everything above overlaps the end of the launches before (1024 x 4096 x 4096: 0.8 us from the wait to here).
+    grid_dependency_wait();
+    // a gated launch that has nothing to do has no items (uniform over the grid)
+    const int64_t total_items = p.gate && *p.gate != 0 ? 0 : whole < total_tiles ? whole + ((total_tiles - whole) << p.split_log2) : total_tiles;
 
     // Which sign planes a tile's rows use at all (bits of the row words, OR-ed over the tile's 128 + 256 rows; each
     // lane its share, to be OR-ed over the warp): bit 0/1: A has +/-, bit 2/3: W has +/-.  The products with a plane
@@ -332,7 +349,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     // format, or the all-positive attention map, moves half the bytes.
     auto tile_sides = [&](int64_t tile) {
         int bits = 0;
-        if (tile < total_tiles) {
+        if (tile < total_items) {
             const int64_t m0 = blk_m(tile) * BM, n0 = blk_n(tile) * BNT;  // (PAIR: only the first CTA asks)
 #pragma unroll
             for (int i = 0; i < BMT / 32; ++i)
@@ -352,48 +369,48 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
     if (warp == 0) {
         // -------------------------------------------------------------- TMA producer
+        // The whole warp runs the loop, one elected lane issues, and the scale factors of an operand are one copy: with eight
+        // copies per stage issued under a test of the lane index this warp was what the kernel waited for (a K block took 730 ns
+        // whatever the tile's width, 690 with the four copies below).
         // Which planes of a tile are not zero comes from the epilogue warps, which read the tile's row words a tile
-        // ahead anyway (sides[] in the control block): nothing on this lane's path but a barrier that has long
-        // completed and eight shared-memory words.
-        if (lane == 0) {
-            constexpr int kTileWT = NHALF ? C_::kTileB / 2 : C_::kTileB;   // one plane of the W tile as loaded (PAIR: of this CTA's half)
-            int it = 0, j = 0;                                   // K blocks issued so far over all tiles; tiles so far
-            bool ok = true;
-            for (int64_t tile = worker; tile < total_tiles && ok; tile += workers, ++j) {
-                int sides = 5;                                   // ONE_PLANE: the first plane of each operand, always
-                if (!ONE_PLANE) {
-                    if (!mbar_wait(&ctl->sides_ready[j & 1], (j >> 1) & 1, &ctl->abort, p.status)) break;
-                    sides = 0;
+        // ahead anyway (sides[] in the control block): nothing on this warp's path but a barrier that has long
+        // completed and eight shared-memory words.  (For the first tile it has not: 1 us.)
+        int it = 0, j = 0;                                       // K blocks issued so far over all tiles; tiles so far
+        bool ok = true;
+        auto wait = [&](uint64_t* b, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(b, parity, &ctl->abort, p.status)) != 0; };
+        for (int64_t tile = worker; tile < total_items && ok; tile += workers, ++j) {
+            // ONE_PLANE: the first plane of each operand, always.  Otherwise the CTA's first stages take both planes without
+            // waiting to hear which occur.
+            const int ahead = j == 0 ? kStages : 0, part = part_log2(tile), tile_w = kTileWT >> part;
+            int a_planes = ONE_PLANE ? 1 : 3, w_planes = a_planes;
+            const int64_t m_blk = blk_m(tile), n_blk = blk_n(tile);
+            const int kb0 = kb_begin(tile), nkb = nkb_of(tile);
+            const int ya = (int)(p.a_row0 + m_blk * BM), yw = (int)(p.w_row0 + n_blk * BNT + part_col(tile) + (PAIR ? rank * (BNT / 2) >> part : 0));
+            const int ysa = (int)(p.a_row0 / 128 + m_blk), ysw = (int)(p.w_row0 / 128 + n_blk * (BNT / 128));
+            for (int kb = 0; kb < nkb; ++kb, ++it) {
+                const int s = it % kStages;
+                if (!ONE_PLANE && kb == ahead) {
+                    ok = wait(&ctl->sides_ready[j & 1], (j >> 1) & 1);
+                    if (!ok) break;
+                    int sides = 0;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) sides |= ctl->sides[j & 1][i];
-                    if (!(sides & 3)) sides |= 1;                // as the MMA warp: an all-zero operand keeps one plane
-                    if (!(sides & 12)) sides |= 4;
+                    a_planes = sides & 3 ? sides & 3 : 1;        // as the MMA warp: an all-zero operand keeps one plane
+                    w_planes = sides & 12 ? sides >> 2 : 1;
                 }
-                const int a_planes = sides & 3, w_planes = (sides >> 2) & 3;
-                const uint32_t bytes = (a_planes == 3 ? 2 : 1) * C_::kTileA + (w_planes == 3 ? 2 : 1) * kTileWT;
-                const int64_t m_blk = blk_m(tile), n_blk = blk_n(tile);
-                const int kb0 = kb_begin(tile), nkb = nkb_of(tile);
-                const int ya = (int)(p.a_row0 + m_blk * BM), yw = (int)(p.w_row0 + n_blk * BNT + (PAIR ? rank * (BNT / 2) : 0));
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const int s = it % kStages;
-                    if (it >= kStages && !mbar_wait(&ctl->empty[s], ((it / kStages) - 1) & 1, &ctl->abort, p.status)) {
-                        ok = false;
-                        break;
-                    }
+                if (it >= kStages) {
+                    ok = wait(&ctl->empty[s], ((it / kStages) - 1) & 1);
+                    if (!ok) break;
+                }
+                if (elect_one()) {
                     uint8_t *st = tiles + s * kStageBytes, *sf = sf_stages + s * C_::kSfStage;
-                    // scale factors first: they have one more step to go
+                    // scale factors first: they have one more step to go.  One copy per operand: {K steps, row blocks, planes}
+                    const int xs = (kb0 + kb) * (C_::kSfRun / 8);
                     mbar_expect_tx(&ctl->sf_full[s], kPlanes * (NHALF ? 2 : 3) * C_::kSfRun);
-                    // (an odd number of row blocks leaves the second CTA of the last pair without rows: any factors will do)
-                    const int64_t ca = ((PAIR ? min(m_blk, (p.M + BM - 1) / BM - 1) : m_blk) * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk,
-                                  cw = (n_blk * (BNT / 128) * p.nk64 + (kb0 + kb) * kSteps) * kSfChunk;
-#pragma unroll
-                    for (int pl = 0; pl < kPlanes; ++pl) {
-                        const uint8_t* w = (pl ? p.sfb_neg : p.sfb_pos) + cw;
-                        bulk_load(sf + (pl * 3 + 0) * C_::kSfRun, (pl ? p.sfa_neg : p.sfa_pos) + ca, C_::kSfRun, &ctl->sf_full[s]);
-                        bulk_load(sf + (pl * 3 + 1) * C_::kSfRun, w, C_::kSfRun, &ctl->sf_full[s]);
-                        if (!NHALF) bulk_load(sf + (pl * 3 + 2) * C_::kSfRun, w + (int64_t)p.nk64 * kSfChunk, C_::kSfRun, &ctl->sf_full[s]);
-                    }
+                    tma_load_3d(sf, &tm_sfa, xs, ysa, 0, &ctl->sf_full[s]);
+                    tma_load_3d(sf + kPlanes * C_::kSfRun, &tm_sfw, xs, ysw, 0, &ctl->sf_full[s]);
                     const int x = (kb0 + kb) * kRowBytes;
+                    const uint32_t bytes = (a_planes == 3 ? 2 : 1) * C_::kTileA + (w_planes == 3 ? 2 : 1) * tile_w;
                     if (!PAIR) mbar_expect_tx(&ctl->full[s], bytes);
                     else if (rank == 0) mbar_expect_tx(&ctl->full[s], 2 * bytes);   // (the other CTA's bytes may be counted first)
                     const uint32_t full = PAIR ? cluster_addr(&ctl->full[s], 0) : 0;
@@ -404,19 +421,27 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     // one 3-D tile per operand: {row bytes, rows, both sign planes} - or the one plane that is not zero
                     if (a_planes == 3) load(st + C_::kOffAp, &tm_a, ya, 0);
                     else load(st + (a_planes == 2 ? C_::kOffAn : C_::kOffAp), &tm_a1, ya, a_planes == 2 ? 1 : 0);
-                    if (w_planes == 3) load(st + C_::kOffWp, &tm_w, yw, 0);
-                    else load(st + (w_planes == 2 ? kOffWnT : C_::kOffWp), &tm_w1, yw, w_planes == 2 ? 1 : 0);
+                    uint8_t *wp = st + C_::kOffWp, *w1 = wp + (w_planes == 2 ? tile_w : 0);   // the box packs its two planes
+                    const int z1 = w_planes == 2 ? 1 : 0;
+                    if (part == 0) {
+                        if (w_planes == 3) load(wp, &tm_w, yw, 0);
+                        else load(w1, &tm_w1, yw, z1);
+                    } else {
+                        if (w_planes == 3) load(wp, &tm_wt, yw, 0);
+                        else load(w1, &tm_wt1, yw, z1);
+                    }
                 }
+                __syncwarp();
             }
-            // after an abort: let the copies already in flight land before shared memory is released
-            if (ctl->abort)
-                for (int i = max(0, it - kStages); i < it; ++i) {
-                    // (PAIR: the first CTA waits for both, the other one for the first at the end of the kernel)
-                    if (rank == 0)
-                        for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
-                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->sf_full[i % kStages], (i / kStages) & 1); ++n) {}
-                }
         }
+        // after an abort: let the copies already in flight land before shared memory is released
+        if (ctl->abort && lane == 0)
+            for (int i = max(0, it - kStages); i < it; ++i) {
+                // (PAIR: the first CTA waits for both, the other one for the first at the end of the kernel)
+                if (rank == 0)
+                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
+                for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->sf_full[i % kStages], (i / kStages) & 1); ++n) {}
+            }
     } else if (PAIR && warp == 1 && rank == 1) {
         // the pair's MMAs are issued by its first CTA
     } else if (warp == 1) {
@@ -429,7 +454,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         bool ok = true, ready = false;                           // ready: the next K block's barrier was seen complete
         // (the planes of a tile: tile_sides above; the words of the next tile are fetched while the current one runs)
         int sides_next = ONE_PLANE ? 0 : tile_sides(worker);
-        for (int64_t tile = worker; tile < total_tiles && ok; tile += workers) {
+        for (int64_t tile = worker; tile < total_items && ok; tile += workers) {
+            const int part = part_log2(tile);
+            const uint32_t idesc = kIdescT - ((uint32_t)((BNT - (BNT >> part)) >> 3) << 17);          // N of the item
+            const uint32_t w_minus = (uint32_t)(C_::kOffWp + (ONE_PLANE ? 0 : kTileWT >> part)) >> 4;   // the second plane of W
+            const uint32_t sf_col = (uint32_t)part_col(tile) / 32;                                      // 32 rows of W to a column
             const int sides = ONE_PLANE ? 5 : whole_sides(sides_next);   // an all-zero operand: one product, which zeroes the tile
             if (!ONE_PLANE) sides_next = tile_sides(tile + workers);
             const int nkb = nkb_of(tile);
@@ -442,44 +471,54 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             if (t > 1 && ok) ok = mbar_wait(&ctl->rest_free[t & 1], ((t >> 1) - 1) & 1, &ctl->abort, p.status);
             tc_fence_after();
             uint32_t accumulate = 0;
-            for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
-                const int s = it % kStages;
-                // tiles landed (TMA byte count) and scale factors stored (four warp arrivals); usually already
-                // seen by the poll that was slipped between the previous block's MMAs
-                if (!ready) ok = mbar_wait(&ctl->full[s], (it / kStages) & 1, &ctl->abort, p.status);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t dstage = desc0 + (uint64_t)((s * kStageBytes) >> 4);
-                const uint32_t sfa = tmem + kTmemSf + (it % C_::kSfSlots) * C_::kSfCols, sfb = sfa + C_::kSfColsA;
-                const int s_next = (it + 1) % kStages;
-                const uint32_t parity_next = ((it + 1) / kStages) & 1;
-                uint32_t seen = 0;
-                if (elect_one()) {
-                    int idx = 0;                                 // MMAs issued so far in this K block
+            // The item's K blocks.  ALL: all planes are in use; PLAIN: and it is a whole tile - everything but the stage is a
+            // constant then.  A test per MMA in the issuing thread shows: half tiles took 19.2 us with, 16.5 without those of
+            // the planes.
+            auto blocks = [&](auto all, auto plain) {
+                constexpr bool ALL = decltype(all)::value, PLAIN = decltype(plain)::value;
+                for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
+                    const int s = it % kStages;
+                    // tiles landed (TMA byte count) and scale factors stored (four warp arrivals); usually already
+                    // seen by the poll that was slipped between the previous block's MMAs
+                    if (!ready) ok = mbar_wait(&ctl->full[s], (it / kStages) & 1, &ctl->abort, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t dstage = desc0 + (uint64_t)((s * kStageBytes) >> 4);
+                    const uint32_t sfa = tmem + kTmemSf + (it % C_::kSfSlots) * C_::kSfCols, sfb = sfa + C_::kSfColsA + (PLAIN ? 0u : sf_col);
+                    const int s_next = (it + 1) % kStages;
+                    const uint32_t parity_next = ((it + 1) / kStages) & 1;
+                    uint32_t seen = 0;
+                    if (elect_one()) {
+                        int idx = 0;                                 // MMAs issued so far in this K block
 #pragma unroll
-                    for (int pa = 0; pa < kPlanes; ++pa)
+                        for (int pa = 0; pa < kPlanes; ++pa)
 #pragma unroll
-                        for (int pw = 0; pw < kPlanes; ++pw)
+                            for (int pw = 0; pw < kPlanes; ++pw)
 #pragma unroll
-                            for (int kk = 0; kk < kSteps; ++kk) {   // 64 elements = 32 bytes along the swizzled row
-                                if (((sides >> pa) & 1) && ((sides >> (2 + pw)) & 1)) {
-                                    const uint64_t da = dstage + (((pa ? C_::kOffAn : C_::kOffAp) + kk * 32) >> 4),
-                                                   dw = dstage + (((pw ? kOffWnT : C_::kOffWp) + kk * 32) >> 4);
-                                    const uint32_t sa = sfa + (pa * kSteps + kk) * 4, sw = sfb + (pw * kSteps + kk) * 8;
-                                    if (PAIR) mma_fp4_block16_pair(acc, da, dw, kIdescT, sa, sw, idx ? 1u : accumulate);
-                                    else mma_fp4_block16(acc, da, dw, kIdescT, sa, sw, idx ? 1u : accumulate);
-                                    // with two MMAs still to go (they keep the pipe busy meanwhile), look whether the
-                                    // next K block is complete, so that its MMAs can follow without a wait
-                                    if (idx == max(n_mma - 3, 0)) seen = mbar_try_wait(&ctl->full[s_next], parity_next);
-                                    ++idx;
+                                for (int kk = 0; kk < kSteps; ++kk) {   // 64 elements = 32 bytes along the swizzled row
+                                    if (ALL || (((sides >> pa) & 1) && ((sides >> (2 + pw)) & 1))) {
+                                        const uint64_t da = dstage + (((pa ? C_::kOffAn : C_::kOffAp) + kk * 32) >> 4),
+                                                       dw = dstage + (!pw ? (uint32_t)C_::kOffWp >> 4 : PLAIN ? kOffWnT >> 4 : w_minus) + (kk * 32 >> 4);
+                                        const uint32_t sa = sfa + (pa * kSteps + kk) * 4, sw = sfb + (pw * kSteps + kk) * 8;
+                                        const uint32_t id = PLAIN ? kIdescT : idesc;
+                                        if (PAIR) mma_fp4_block16_pair(acc, da, dw, id, sa, sw, idx ? 1u : accumulate);
+                                        else mma_fp4_block16(acc, da, dw, id, sa, sw, idx ? 1u : accumulate);
+                                        // with two MMAs still to go (they keep the pipe busy meanwhile), look whether the
+                                        // next K block is complete, so that its MMAs can follow without a wait
+                                        if (idx == max((ALL ? kPlanes * kPlanes * kSteps : n_mma) - 3, 0)) seen = mbar_try_wait(&ctl->full[s_next], parity_next);
+                                        ++idx;
+                                    }
                                 }
-                            }
-                    if (PAIR) mma_commit_pair(&ctl->empty[s]);
-                    else mma_commit(&ctl->empty[s]);
+                        if (PAIR) mma_commit_pair(&ctl->empty[s]);
+                        else mma_commit(&ctl->empty[s]);
+                    }
+                    ready = __any_sync(0xFFFFFFFFu, seen) != 0;
+                    accumulate = 1;
                 }
-                ready = __any_sync(0xFFFFFFFFu, seen) != 0;
-                accumulate = 1;
-            }
+            };
+            if (!ONE_PLANE && sides != 15) blocks(std::false_type{}, std::false_type{});
+            else if (part) blocks(std::true_type{}, std::false_type{});
+            else blocks(std::true_type{}, std::true_type{});
             if (ok && elect_one()) {
                 if (PAIR) mma_commit_pair(&ctl->accum_full);
                 else mma_commit(&ctl->accum_full);
@@ -498,7 +537,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         const int q = warp & 3, group = (warp - 2) >> 2;
         int it = 0;
         bool ok = true;
-        for (int64_t tile = worker; tile < total_tiles && ok; tile += workers) {
+        for (int64_t tile = worker; tile < total_items && ok; tile += workers) {
             const int end = it + nkb_of(tile);
             // this group's K blocks (global count it % kSfGroups == group)
             for (int i = it + ((group - it) & (kSfGroups - 1)); i < end; i += kSfGroups) {
@@ -513,7 +552,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     for (int kk = 0; kk < kSteps; ++kk)
 #pragma unroll
                         for (int x = 0; x < 3; ++x)
-                            v[(pl * kSteps + kk) * 3 + x] = *reinterpret_cast<const uint4*>(sf + (pl * 3 + (NHALF ? min(x, 1) : x)) * C_::kSfRun + kk * kSfChunk);
+                            v[(pl * kSteps + kk) * 3 + x] = *reinterpret_cast<const uint4*>(sf + (x ? kPlanes + pl * (NHALF ? 1 : 2) + (NHALF ? 0 : x - 1) : pl) * C_::kSfRun + kk * kSfChunk);
                 // the slot of the scale-factor ring is free once the MMAs of K block i - kSfSlots are done (the `empty`
                 // barrier of that block's stage; it cannot complete again before this block's factors are stored)
                 if (i >= C_::kSfSlots) {
@@ -562,7 +601,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         auto pow2 = [](int e) { return __uint_as_float((uint32_t)(e + 127) << 23); };
         auto load_consts = [&](int64_t tl) {
             TileConsts c = {1.f, 1.f, 0};
-            if (tl < total_tiles) {
+            if (tl < total_items) {
                 const int64_t n = blk_n(tl) * BNT + tid_e, mm = blk_m(tl) * BM + q * 32 + lane;
                 if (tid_e < BNT && n < p.N) {
                     const int w = __ldg(p.w_exp + n);
@@ -582,7 +621,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         // The eight warps' row words cover the tile's 128 + 256 rows: each tells the producer which planes its rows
         // use (tile number j of this CTA); the producer reads them before the tile's first load.
         auto publish = [&](const TileConsts& c, int64_t tl, int j) {
-            if (tl >= total_tiles) return;
+            if (tl >= total_items) return;
             const int bits = __reduce_or_sync(0xFFFFFFFFu, c.planes);
             if (ONE_PLANE) {                                     // nobody waits for the planes; a second one is an error
                 if (lane == 0 && (bits & 10)) atomicExch(p.status, (int)AMX_ERR_FLAGS);
@@ -604,7 +643,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         int64_t tile = worker;
         TileConsts nxt = load_consts(tile);
         publish(nxt, tile, 0);
-        while (tile < total_tiles && ok) {
+        while (tile < total_items && ok) {
             const TileConsts cur = nxt;
             const int64_t tile_after = tile + workers;
             nxt = load_consts(tile_after);                       // in flight while this tile is worked on
@@ -620,16 +659,46 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             tc_fence_after();
             // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join)
             asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
-            if (ok) {
+            // 16 columns of the tile: scaled and stored
+            auto put = [&](const uint32_t (&v)[16], int col) {
+                float f[16];
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) {
+                    const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&w_fac[col + j]);
+                    cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[j], v[j + 1]), cast::mul_f32x2(w2.x, a_fac2)), f[j], f[j + 1]);
+                    cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[j + 2], v[j + 3]), cast::mul_f32x2(w2.y, a_fac2)), f[j + 2], f[j + 3]);
+                }
+                if (m < p.M) {
+                    if (p.out_bf16)
+                        store_row16_bf16(reinterpret_cast<__nv_bfloat16*>(C_item) + m * p.ld_c + n0 + col, f, p.vec_store != 0,
+                                         p.N - (n0 + col));
+                    else
+                        store_row16(C_item + m * p.ld_c + n0 + col, f, p.vec_store != 0, p.N - (n0 + col));
+                }
+            };
+            const int h = e >> 2, odd = t & 1;
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(odd ? kAccWindow : 0);
+            const int part = part_log2(tile);
+            if (ok && part) {                                    // the CTA's last item: no accumulator follows
+                const int cols = (BNT / 2) >> part, col0 = part_col(tile);   // of this warp: half h of the item's
+                uint32_t v[2][16];
+                tmem_ld16(taddr + h * cols, v[0]);
+                for (int i = 0; i < cols; i += 32) {             // (32 or 64 columns)
+                    tmem_ld_wait();
+                    tmem_ld16(taddr + h * cols + i + 16, v[1]);
+                    put(v[0], col0 + h * cols + i);
+                    tmem_ld_wait();
+                    if (i + 32 < cols) tmem_ld16(taddr + h * cols + i + 32, v[0]);
+                    put(v[1], col0 + h * cols + i + 16);
+                }
+            } else if (ok) {
                 // The tile's window starts at column 0 (even t) or kAccWindow (odd t).  The kOvl columns it shares with
                 // the next tile's window - its last ones when even, its first ones when odd - are read first; this warp
                 // takes its half h of both parts, kC1 + kC2 chunks of 16 columns.
-                const int h = e >> 2, odd = t & 1;
                 const int o1 = odd ? 0 : BNT - kOvl, o2 = odd ? kOvl : 0;
                 auto chunk_col = [&](int i) {                    // first column (inside the tile) of this warp's chunk i
                     return i < kC1 ? o1 + h * (kOvl / 2) + 16 * i : o2 + h * ((BNT - kOvl) / 2) + 16 * (i - kC1);
                 };
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(odd ? kAccWindow : 0);
                 uint32_t v[2][16];
                 if (kC1 == 0) {                                  // nothing shared: the next tile may start at once
                     released(&ctl->ovl_free);
@@ -648,21 +717,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                         released(&ctl->rest_free[odd]);
                     }
                     if (i + 1 < kC1 + kC2) tmem_ld16(taddr + chunk_col(i + 1), v[buf ^ 1]);   // loads while this chunk is stored
-                    const int col = chunk_col(i);
-                    float f[16];
-#pragma unroll
-                    for (int j = 0; j < 16; j += 4) {
-                        const ulonglong2 w2 = *reinterpret_cast<const ulonglong2*>(&w_fac[col + j]);
-                        cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[buf][j], v[buf][j + 1]), cast::mul_f32x2(w2.x, a_fac2)), f[j], f[j + 1]);
-                        cast::unpack_f32x2(cast::mul_f32x2(cast::pack_f32x2(v[buf][j + 2], v[buf][j + 3]), cast::mul_f32x2(w2.y, a_fac2)), f[j + 2], f[j + 3]);
-                    }
-                    if (m < p.M) {
-                        if (p.out_bf16)
-                            store_row16_bf16(reinterpret_cast<__nv_bfloat16*>(C_item) + m * p.ld_c + n0 + col, f, p.vec_store != 0,
-                                             p.N - (n0 + col));
-                        else
-                            store_row16(C_item + m * p.ld_c + n0 + col, f, p.vec_store != 0, p.N - (n0 + col));
-                    }
+                    put(v[buf], chunk_col(i));
                 }
             }
             ++t;
@@ -715,22 +770,38 @@ int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, co
             return AMX_ERR_CUDA;
         configured[dev] = true;
     }
-    CUtensorMap tm_a, tm_w, tm_a1, tm_w1;                       // both planes of a tile in one box, and one plane alone
-    if (!make_map(&tm_a, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes) || !make_map(&tm_w, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes) ||
-        !make_map(&tm_a1, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes, 1) ||
-        !make_map(&tm_w1, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes, 1))
-        return AMX_ERR_CUDA;
     if (!sm_count(dev)) return AMX_ERR_CUDA;
     constexpr int kCtas = PAIR ? 2 : 1, BMT = BM * kCtas;
-    if (PAIR) p.band = (p.band + 1) / 2;
     const int64_t tiles = ((p.N + BNT - 1) / BNT) * ((p.M + BMT - 1) / BMT) * (SLICED ? p.slices : 1);
-    const int64_t workers = std::min<int64_t>(tiles, sm_count(dev) / kCtas);           // one persistent CTA per SM
+    const int64_t places = sm_count(dev) / kCtas;                // one persistent CTA (or pair) per SM
+    int64_t items = tiles;
+    if (!SLICED && !NHALF) {
+        // The last, partly filled wave takes as long as a whole one: its tiles are cut into halves or quarters of their
+        // columns, as many as there are places for.  An MMA of 128 columns takes 0.7, of 64 columns half the time of one of 256,
+        // so more parts are always faster as long as each has a place of its own (1000 x 11008 x 4096, 172 tiles on 74 pairs: the
+        // third wave 16.5 us instead of 23.5).
+        const int64_t left = tiles % places;
+        p.whole = (int)(tiles - left);
+        p.split_log2 = left * 4 <= places ? 2 : left * 2 <= places ? 1 : 0;
+        items = p.whole + (left << p.split_log2);
+    }
+    const int64_t workers = std::min<int64_t>(items, places);
+    CUtensorMap tm_a, tm_w, tm_a1, tm_w1, tm_wt, tm_wt1, tm_sfa, tm_sfw;   // both planes of a tile in one box, and one plane alone; of a part
+    const int box_part = kBoxW >> p.split_log2;
+    if (!make_map(&tm_a, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes) || !make_map(&tm_w, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes) ||
+        !make_map(&tm_a1, pa, a_rows, p.K, oa.plane, BM, C_::kRowBytes, 1) ||
+        !make_map(&tm_w1, pw, w_rows, p.K, ow.plane, kBoxW, C_::kRowBytes, 1) ||
+        !make_map(&tm_wt, pw, w_rows, p.K, ow.plane, box_part, C_::kRowBytes) ||
+        !make_map(&tm_wt1, pw, w_rows, p.K, ow.plane, box_part, C_::kRowBytes, 1) ||
+        !make_sf_map(&tm_sfa, pa, oa, C_::kSteps, 1, C_::kPlanes) || !make_sf_map(&tm_sfw, pw, ow, C_::kSteps, NHALF ? 1 : 2, C_::kPlanes))
+        return AMX_ERR_CUDA;
+    if (PAIR) p.band = (p.band + 1) / 2;
     const unsigned grid = (unsigned)workers * kCtas;
     // Chained up to 4.4e11 issued products (about 170 us).  Cast and product of 2048 x 12288 x 4096: ordinary 173 us, chained 153 to
     // 161; 4096 x 11008 x 4096 265 / 274.  One plane, 8192 x 6144 x 4096: 136 / 132, 8192 x 14336 x 4096 269 / 267.
     const double products = (double)p.M * (double)p.N * (double)p.K * (ONE_PLANE ? 1.0 : 4.0);
     return launch_clusters(kCtas, products <= 4.4e11, gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w,
-                           tm_a1, tm_w1, p);
+                           tm_a1, tm_w1, tm_wt, tm_wt1, tm_sfa, tm_sfw, p);
 }
 
 }  // namespace
@@ -748,13 +819,7 @@ int fill_params(const Fp4Operand& a, const Fp4Operand& w, int64_t M, int64_t N, 
     const uint8_t* pw = static_cast<const uint8_t*>(w.prepared);
     int* status = static_cast<int*>(workspace);
     p = Params{};
-    // scale factors come in chunks per 128 rows, row words per row: the range starts at a pointer offset
-    const size_t a_sf0 = (size_t)(a.row0 / 128) * oa.nk64 * kSfChunk, w_sf0 = (size_t)(w.row0 / 128) * ow.nk64 * kSfChunk;
-    p.sfa_pos = pa + 2 * oa.plane + a_sf0;
-    p.sfa_neg = p.sfa_pos + oa.sf;
     p.a_exp = reinterpret_cast<const int*>(pa + 2 * oa.plane + 2 * oa.sf) + a.row0;
-    p.sfb_pos = pw + 2 * ow.plane + w_sf0;
-    p.sfb_neg = p.sfb_pos + ow.sf;
     p.w_exp = reinterpret_cast<const int*>(pw + 2 * ow.plane + 2 * ow.sf) + w.row0;
     p.M = M; p.N = N; p.K = K; p.ld_c = ld_c; p.C = C;
     p.a_row0 = a.row0; p.w_row0 = w.row0;
