@@ -516,7 +516,7 @@ extern "C" int amx_softmax_quantize(const float* S, int64_t rows, int64_t cols, 
 namespace {
 // Workspace of amx_attention.  Heads are taken in chunks: the casts of Q, K and V (small per head) run once per chunk
 // on the stacked heads.  Two ways from there:
-//   fused   (head dimension 128 or 64, products on the FP4 kernel) both products and the softmax in two or three launches of
+//   fused   (head dimension 128 or 64, products on the FP4 kernel) both products and the softmax in one or two launches of
 //           the fused kernel for all heads of the chunk; Q, K and V^T as prepared operands, every head padded to whole
 //           blocks of 128 rows
 //   stored  the logits and the cast map of `batch` heads at a time in the workspace: batched launches of the bf16-decode

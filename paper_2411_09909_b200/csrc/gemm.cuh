@@ -122,7 +122,7 @@ size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K);
 // C[m][n] = sum over `slices` partial products [slices][M][N], in slice order (defined with the bf16-decode kernel)
 int reduce_slices(const float* part, int slices, int64_t M, int64_t N, float* C, int64_t ld_c, cudaStream_t st,
                   const int* run_if_nonzero = nullptr);
-// Fused attention for head dimensions 128 and 64 (attention_fp4.cu): both products and the softmax in two or three launches,
+// Fused attention for head dimensions 128 and 64 (attention_fp4.cu): both products and the softmax in one or two launches,
 // logits and attention map never in global memory.  Operands prepared ahead, heads stacked row-wise, padded to whole blocks
 // of 128.
 bool attn_fused_supported(int64_t L, int64_t d);

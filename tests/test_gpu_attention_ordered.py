@@ -22,6 +22,7 @@ TOL = 2.0 ** -23 * 8192 ** 0.5
                                                 (4, 4, 2080, 128, amx.GEMM_AUTO),       # 17 tiles: 2 x 8 + 1
                                                 (4, 4, 2560, 64, amx.GEMM_AUTO),        # 20 whole tiles
                                                 (2, 1, 8192, 64, amx.GEMM_AUTO),        # all 256 groups of the softmax kernel
+                                                (64, 16, 416, 128, amx.GEMM_FP4),       # 256 items of 4 tiles: two per CTA
                                                 (64, 64, 32, 128, amx.GEMM_FP4), (64, 64, 160, 64, amx.GEMM_FP4)])
 def test_fused_attention_equals_the_stored_path(heads, kv, L, d, flags, causal):
     for seed in range(2):
