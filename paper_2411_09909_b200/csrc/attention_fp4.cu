@@ -735,13 +735,14 @@ attention_fp4_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             }
         }
     }
-    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
+    // As the last thing: the next launch's blocks then find all SMs free, instead of crowding on those that ended first.
+    grid_launch_dependents();
 }
 
 template <int PASS, int MASK, int HD>

@@ -724,7 +724,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             tile = tile_after;
         }
     }
-    grid_launch_dependents();
     tc_fence_before();
     __syncthreads();
     if (PAIR) cluster_sync();                                    // no CTA leaves while the other still uses its memory
@@ -733,6 +732,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         if (PAIR) tmem_dealloc_pair(tmem, kTmemCols);
         else tmem_dealloc(tmem, kTmemCols);
     }
+    // As the last thing: the next launch's blocks then find all SMs free, instead of crowding on those that ended first.
+    grid_launch_dependents();
 }
 
 // ---------------------------------------------------------------------------------- host --
@@ -758,6 +759,9 @@ int sm_count(int dev) {                                              // 0: the d
     return count[dev];
 }
 
+// Into how many parts (log2) the tiles of a wave that has places for more are cut.
+int parts_log2(int64_t tiles, int64_t places) { return tiles * 4 <= places ? 2 : tiles * 2 <= places ? 1 : 0; }
+
 template <int BK_, bool SLICED = false, bool NHALF = false, bool ONE_PLANE = false, bool PAIR = false>
 int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, const OperandLayout& ow, int64_t a_rows,
                int64_t w_rows, Params p, int dev, cudaStream_t st) {
@@ -782,7 +786,7 @@ int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, co
         // third wave 16.5 us instead of 23.5).
         const int64_t left = tiles % places;
         p.whole = (int)(tiles - left);
-        p.split_log2 = left * 4 <= places ? 2 : left * 2 <= places ? 1 : 0;
+        p.split_log2 = parts_log2(left, places);
         items = p.whole + (left << p.split_log2);
     }
     const int64_t workers = std::min<int64_t>(items, places);
@@ -838,7 +842,8 @@ int fill_params(const Fp4Operand& a, const Fp4Operand& w, int64_t M, int64_t N, 
 
 // Few output tiles and a long K (a few token rows against a big weight): K ranges as separate work items, so
 // that more SMs stream the operands; their partial products go to the workspace and are added in range order.
-// Returns the number of ranges (1: none); ranges hold the same number of 128-element K blocks up to one.
+// Returns the number of ranges (1: none) a workspace is sized for; ranges hold the same number of 128-element K blocks up to
+// one.  Whether a call takes them: slices_pay.
 int gemm_fp4_slices(int64_t M, int64_t N, int64_t K) {
     const int64_t tiles = ((N + BN - 1) / BN) * ((M + BM - 1) / BM);
     const int num_kb = (int)((K + 127) / 128);
@@ -847,6 +852,20 @@ int gemm_fp4_slices(int64_t M, int64_t N, int64_t K) {
     if (s > 8) s = 8;
     return s < 2 ? 1 : s;
 }
+// K ranges or parts of tiles (launch_fp4) for a call of so few tiles, by estimates in us: a K block of a whole tile, a half or a
+// quarter takes 0.57, 0.45 or 0.39; ranges pay for the launch that adds them and for writing and reading the partial products.
+// Two planes, ranges / parts measured: 96 x 4096 x 14336 22.9 / 47.9, 250 x 4096 x 14336 35 / 48, 368 x 4096 x 11008 37 / 42,
+// 500 x 4096 x 11008 46 / 42, 368 x 4096 x 4096 26 / 19, 96 x 2560 x 2560 15 / 12.  One plane (a K block 0.16 to 0.13): parts
+// always, 500 x 4096 x 4096 26 / 9.7, 96 x 4096 x 14336 18.7 / 18.5.
+namespace {
+bool slices_pay(int64_t M, int64_t N, int64_t K, int slices, int sms, bool one_plane) {
+    if (slices < 2 || one_plane) return false;
+    const double blocks = (double)((K + 127) / 128);
+    static constexpr double kBlock[3] = {0.57, 0.45, 0.39};
+    const double parts = blocks * kBlock[parts_log2(((N + BN - 1) / BN) * ((M + BM - 1) / BM), sms)];
+    return blocks / slices * kBlock[0] + 4.0 + 0.6e-6 * 4.0 * slices * (double)M * (double)N < parts;
+}
+}  // namespace
 size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K) {
     const int s = gemm_fp4_slices(M, N, K);
     return 256 + (s > 1 ? (size_t)s * M * N * 4 : 0);
@@ -876,7 +895,8 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
     const int slices = gemm_fp4_slices(M, N, K);
     // at most 128 columns: tiles of 128 x 128, so that no half of a W tile is padding
     const bool half = N <= BN / 2 && !getenv("AMX_FP4_NO_HALF_TILE");
-    if (!gate && !scale_a && !out_bf16 && slices > 1 && workspace_bytes >= gemm_fp4_prepared_workspace_bytes(M, N, K)) {
+    if (!gate && !scale_a && !out_bf16 && slices_pay(M, N, K, slices, sm_count(dev), one_plane && !half) &&
+        workspace_bytes >= gemm_fp4_prepared_workspace_bytes(M, N, K)) {
         float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
         p.C = part;
         p.ld_c = N;
