@@ -19,9 +19,9 @@
 // and a subtraction 7.4; the scale chosen by a sign mask 7.7; code bits shifted into bf16 fields and the scale chosen
 // by a mask (the earlier form) 8.7; the signs kept apart through two MMAs 7.1.
 //
-// Two kernels share this: gemm_rows_stream_kernel for up to 32 tokens (a CTA covers 32 weight rows, its warps split K, no
-// cluster for the usual layers; described below) and gemm_rows_kernel for 33 and more, in blocks of 32, 48 or 64:
-// a CTA of eight warps covers 128 weight rows and one range of K, warp = (row group of 32) + 4 * (parity of its steps).
+// Two kernels share this: gemm_rows_stream_kernel for up to 32 tokens (a CTA covers 8 to 112 weight rows, its eight warps split K;
+// plan_stream) and gemm_rows_kernel for 33 and more, in blocks of 32, 48 or 64: a CTA of eight warps covers 128 weight rows and one
+// range of K, warp = (row group of 32) + 4 * (parity of its steps).
 // In both the codes come through a ring in shared memory by asynchronous copies, a slot per warp and step (a lane reads back
 // only its own copies; no registers are held by loads in flight): the copies alone stream at 5.4-5.8 TB/s.  Scales are
 // copied along the rows, many steps at a time.  (Copied per step beside the codes, 8 bytes per row at 32 different rows per
@@ -29,11 +29,13 @@
 // 12288 x 4096.)  The K ranges of the same rows are the CTAs of one thread-block cluster (up to 8), which add their partial
 // products over distributed shared memory in rank order - deterministic, no scratch in global memory and no second launch.
 //
-// What bounds it (counters of one call, weights from HBM): one row of 12288 x 4096 takes 16 us, 20 000 active cycles with
-// 58 % of the issue slots and 52 % of the logic pipe busy (decode), 40 MB into the SMs for 28 MB of weight; 24 rows of
-// 14336 x 4096 25 us, 33 000 cycles, issue slots 45 %, tensor pipe 28 %, 93 MB into the SMs for 33 MB of weight - the rest are
-// fragments, re-read by every CTA - and 448 CTAs on 296 places; 64 rows of 12288 x 4096 in the kernel of 128-row CTAs 38 us,
-// tensor pipe 55 % of the active cycles on 96 of 148 SMs.
+// What bounds it (times inside a chain of calls, weights from HBM).  One row of 12288 x 4096, 12.8 us: 1.9 from the end of the call
+// before to the first block (the fragments kernel and a launch), 2.4 to the first step's data, 5 for the steps - decode at 6
+// cycles of a warp per pair, six warps to a scheduler - 0.5 for the sums.  From two token tiles on mma.sync: an m16n8k16 takes a
+// scheduler about 16 cycles, for 24 rows 12 per pair of the 13 that a pair takes (14336 x 4096: 20.5 us).  Fragments are
+// re-read by every CTA, which is why few CTAs of many rows are better from 17 tokens on.  (Decoded to shared memory for
+// tcgen05.mma instead, whatever the number of tokens: 23 us - the way from the decoding warps through the MMA and back takes a
+// microsecond, and four steps of 32 KB are all that fits.)
 //
 // The token rows are cast (or decoded) once by a small kernel into the fragment order.  (Cast inside the main kernel by
 // every CTA, one launch less, measured the same for one row and slower for more.)
@@ -68,7 +70,7 @@ constexpr int kMaxTiles = 8;                       // token tiles per CTA
 // Steps whose scales are held at a time: those of 32 steps in groups of 16 (67 KB) do not fit beside the rings of eight token
 // tiles (192 KB).
 __host__ __device__ constexpr int scale_steps(int gs) { return gs == 16 ? 16 : 32; }
-constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kMaxSmem = 227 * 1024, kSmSmem = 228 * 1024, kCtaSmem = 1024;   // of a block; of an SM, which keeps some per block
 
 // Fragment order of the token rows, per step and tile of 8 rows: pieces of 16 bytes [j = 0..3][lane 0..31]; the piece
 // of (j, lane (g, t)) holds elements 32 t + 8 j .. + 7 of the step, row g of the tile.  Piece (j, l) sits at position
@@ -133,6 +135,7 @@ struct RowsParams {
     float* C;
     int64_t ld_c;
     int steps_max;               // steps of the longest range
+    int rows;                    // weight rows per CTA (streaming kernel)
 };
 
 // Shared-memory geometry.  kDepth ring slots per warp (kDepth - 1 steps in flight); with up to four token tiles two
@@ -344,13 +347,11 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
     if (slices > 1) cluster.sync();                                  // no CTA leaves while its tile is still read
 }
 
-// ---- few rows (up to four token tiles): a CTA of eight warps covers 32 weight rows, its warps split the K range.
-// No cluster for the usual layers (enough rows to fill the SMs), three CTAs on an SM, so a chain of calls keeps the weight
-// stream going: the CTAs of the next call move in one by one as this call's leave.  (With 128 rows per CTA and a cluster
-// over K, 288 CTAs did not all fit - clusters of three leave slots empty in every GPC - and a second wave of a few
-// clusters doubled the time; clusters of four were packed on two thirds of the SMs.)  A warp's steps are consecutive, so
-// its scales come along the rows, four steps (32 bytes per row with groups of 32) at a time.
-constexpr int kStreamRows = 32, kScaleSlotSteps = 4;
+// ---- few rows (up to four token tiles): a CTA of eight warps covers p.rows weight rows (a multiple of 8, at most 16 x MB), its
+// warps split the K range.  A warp's steps are consecutive, so its scales come along the rows, four steps (32 bytes per row
+// with groups of 32) at a time.  Blocks of few rows share an SM (stream_ctas), so that a chain of calls keeps the weight stream going:
+// the CTAs of the next call move in one by one as this call's leave.
+constexpr int kScaleSlotSteps = 4;
 
 template <int GS>
 struct StreamRing {
@@ -359,62 +360,73 @@ struct StreamRing {
     // Words of eight rows in different banks: an odd pitch (in units of the words a quad reads together), or rows of 8
     // words whose halves are exchanged on every other four rows.
     static constexpr int kPitch = GS == 16 ? 20 : GS == 32 ? 8 : GS == 64 ? 5 : 3;
-    __device__ static int at(int r, int w) { return r * kPitch + (GS == 32 ? w ^ (r & 4) : w); }
-    static constexpr int kScaleBytes = kStreamRows * kPitch * 4;                  // one slot; two per warp
-    static constexpr int kWarpBytes = kDepth * kCodeBytes + 2 * kScaleBytes;
-    static constexpr int kBytes = kWarps * kWarpBytes;
+    __host__ __device__ static constexpr int at(int r, int w) { return r * kPitch + (GS == 32 ? w ^ (r & 4) : w); }
+    // of one warp: code slots, then two slots of scales
+    __host__ __device__ static constexpr int warp_bytes(int rows) { return rows * (kDepth * 64 + 2 * kPitch * 4); }
 };
+__host__ __device__ constexpr int stream_part_bytes(int nt, int rows) { return kWarps * nt * kTok * (rows + 4) * 4; }
+__host__ __device__ constexpr int stream_ctas(int nt, int mb) { return mb <= 2 ? (nt == 1 ? 3 : 2) : mb <= 4 && nt <= 2 ? 2 : 1; }
 
-template <int NT, int GS>
-__global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_kernel(const RowsParams p) {
+template <int NT, int MB, int GS>
+__global__ void __launch_bounds__(kThreads, stream_ctas(NT, MB)) gemm_rows_stream_kernel(const RowsParams p) {
     using R = StreamRing<GS>;
     constexpr int kDepth = R::kDepth;
     extern __shared__ __align__(16) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int slices = (int)gridDim.y, slice = (int)blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int64_t steps = p.K / kStepK;
-    const int64_t cta_begin = steps * slice / slices, cta_steps = steps * (slice + 1) / slices - cta_begin;
-    const int64_t w_first = cta_steps * warp / kWarps;               // this warp's steps inside the CTA's range
-    const int n = (int)(cta_steps * (warp + 1) / kWarps - w_first);
-    const int64_t s_begin = cta_begin + w_first;
-    const int64_t row0 = (int64_t)blockIdx.x * kStreamRows;
+    const int rows = p.rows, steps = (int)(p.K / kStepK);
+    const int cta_begin = (int)((int64_t)steps * slice / slices), cta_steps = (int)((int64_t)steps * (slice + 1) / slices) - cta_begin;
+    const int w_first = cta_steps * warp / kWarps;                   // this warp's steps inside the CTA's range
+    const int n = cta_steps * (warp + 1) / kWarps - w_first;
+    const int s_begin = cta_begin + w_first;
+    const int64_t row0 = (int64_t)blockIdx.x * rows;
+    const int rows_left = (int)min((int64_t)rows, p.N - row0);
 
-    uint8_t* ring = smem + warp * R::kWarpBytes;
-    uint8_t* scale_ring = ring + kDepth * kCodeBytes;
+    uint8_t* ring = smem + warp * R::warp_bytes(rows);
+    const int slot_bytes = rows * 64;
+    uint32_t* scale_ring = reinterpret_cast<uint32_t*>(ring + kDepth * slot_bytes);
 
-    // piece t of rows g, g + 8 (block 0), g + 16, g + 24 (block 1).  Rows past the weight are not copied: what their
-    // slots hold only reaches sums that are not stored.
-    const uint8_t* pc = p.w_codes + (row0 + g) * (p.K / 2) + s_begin * 64 + t * 16;
+    // piece t of rows g, g + 8, ...  Rows past the weight are not copied: what their slots hold only reaches sums that are not stored.
+    const uint8_t* pc = p.w_codes + (row0 + g) * (p.K / 2) + (int64_t)s_begin * 64 + t * 16;
     const int64_t rows8 = p.K * 4;             // bytes between rows 8 apart
-    const int rows_left = (int)min((int64_t)kStreamRows, p.N - row0);
     auto issue = [&](int i) {
         if (i < n) {
-            uint8_t* slot = ring + (i % kDepth) * kCodeBytes + lane * 16;
+            uint8_t* slot = ring + (i % kDepth) * slot_bytes + lane * 16;
+            const uint8_t* src = pc + (int64_t)i * 64;
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q * 8 + g < rows_left) cp_async16(slot + q * 512, pc + q * rows8 + (int64_t)i * 64);
+            for (int q = 0; q < 2 * MB; ++q, src += rows8)
+                if (q * 8 + g < rows_left) cp_async16(slot + q * 512, src);
         }
     };
+    const int64_t scale_pitch = p.K / GS * 2;
     auto issue_scales = [&](int slot) {
         const int first = slot * kScaleSlotSteps;
         if (first >= n) return;
-        uint32_t* dst = reinterpret_cast<uint32_t*>(scale_ring + (slot & 1) * R::kScaleBytes);
+        uint32_t* dst = scale_ring + (slot & 1) * rows * R::kPitch;
+        const uint8_t* src0 = p.w_scales + row0 * scale_pitch + (int64_t)(s_begin + first) * (2 * kStepK / GS);
+        if (GS == 32 && first + kScaleSlotSteps <= n && ((reinterpret_cast<uintptr_t>(src0) | scale_pitch) & 15) == 0) {
+#pragma unroll
+            for (int i = 0; i < MB; ++i) {     // two pieces of 16 bytes per row
+                const int r = i * 16 + (lane >> 1), w = (lane & 1) * 4;
+                if (r < rows_left) cp_async16(dst + R::at(r, w), src0 + r * scale_pitch + w * 4);
+            }
+            return;
+        }
         // words past the warp's last step may lie past the end of the tensor
         const int words = min(R::kWords, GS == 128 ? (min(n - first, kScaleSlotSteps)) / 2 + 1 : (n - first) * (64 / GS));
-#pragma unroll
-        for (int i = 0; i < (kStreamRows * R::kWords + 31) / 32; ++i) {
-            const int item = i * 32 + lane, r_in = item / R::kWords, w = item - r_in * R::kWords;
-            int64_t r = row0 + r_in;
-            r = r < p.N ? r : p.N - 1;
-            const uint8_t* src = p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2;
+        for (int item = lane; item < rows_left * R::kWords; item += 32) {
+            const int r = item / R::kWords, w = item - r * R::kWords;
+            const uint8_t* src = src0 + r * scale_pitch;
             if (GS == 128) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
-            if (w < words) cp_async4(dst + R::at(r_in, w), src + w * 4);
+            if (w < words) cp_async4(dst + R::at(r, w), src + w * 4);
         }
     };
+    issue(0);
     issue_scales(0);
+    cp_async_commit();
 #pragma unroll
-    for (int d = 0; d < kDepth - 1; ++d) {
+    for (int d = 1; d < kDepth - 1; ++d) {
         issue(d);
         cp_async_commit();
     }
@@ -422,99 +434,101 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
     grid_dependency_wait();                    // the fragments (and the previous user of C) are complete from here on
     const int m0 = (int)blockIdx.z * (NT * kTok), live_tok = min(NT * kTok, p.M - m0);
 
-    float acc[2][NT][4];
+    float acc[MB][NT][4];
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < MB; ++b)
 #pragma unroll
         for (int m = 0; m < NT; ++m)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[b][m][j] = 0.f;
 
-    for (int i = 0; i < n; ++i) {
+    uint4 bf[4][NT];                           // the step's fragments
+    const uint4* fg = p.frag + ((int64_t)s_begin * gridDim.z + blockIdx.z) * (NT * 128);
+    const int64_t fg_step = (int64_t)gridDim.z * (NT * 128);
+    for (int i = 0; i < n; ++i, fg += fg_step) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int m = 0; m < NT; ++m) bf[j][m] = __ldg(fg + m * 128 + frag_pos(j, lane));
         cp_async_wait<kDepth - 2>();           // this step's copies have landed
         __syncwarp();                          // the scales are read across lanes
         if ((i & (kScaleSlotSteps - 1)) == 0) issue_scales(i / kScaleSlotSteps + 1);
         issue(i + kDepth - 1);
         cp_async_commit();
-        const uint8_t* slot = ring + (i % kDepth) * kCodeBytes;
-        const uint32_t* sw = reinterpret_cast<const uint32_t*>(scale_ring + ((i / kScaleSlotSteps) & 1) * R::kScaleBytes);
+        const uint8_t* slot = ring + (i % kDepth) * slot_bytes + lane * 16;
+        const uint32_t* sw = scale_ring + ((i / kScaleSlotSteps) & 1) * rows * R::kPitch;
         const int s_in = i & (kScaleSlotSteps - 1);
-        uint4 cw[4];
-        uint32_t sc[4];                        // the scale bytes of the lane's group (groups of 16: of both)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            cw[q] = *reinterpret_cast<const uint4*>(slot + q * 512 + lane * 16);
-            const int r_in = q * 8 + g;
-            if (GS == 16) sc[q] = sw[R::at(r_in, s_in * 4 + t)];
-            else if (GS == 32) sc[q] = sw[R::at(r_in, s_in * 2 + (t >> 1))] >> (16 * (t & 1));
-            else if (GS == 64) sc[q] = sw[R::at(r_in, s_in)] >> (16 * (t >> 1));
-            else {                             // the slot's first step may start in the upper half of its word
-                const int h = (int)((min(row0 + r_in, p.N - 1) * steps + s_begin + (i - s_in)) & 1) + s_in;
-                sc[q] = sw[R::at(r_in, h >> 1)] >> (16 * (h & 1));
+        for (int blk = 0; blk < MB; ++blk) {
+            if (blk * 16 >= rows) break;
+            uint4 cw[2];
+            uint32_t sc[2];                    // the scale bytes of the lane's group (groups of 16: of both)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int oct = min(blk * 2 + q, rows / 8 - 1);      // (an odd number of octets: the last one twice)
+                cw[q] = *reinterpret_cast<const uint4*>(slot + oct * 512);
+                const int r_in = oct * 8 + g;
+                if (GS == 16) sc[q] = sw[R::at(r_in, s_in * 4 + t)];
+                else if (GS == 32) sc[q] = sw[R::at(r_in, s_in * 2 + (t >> 1))] >> (16 * (t & 1));
+                else if (GS == 64) sc[q] = sw[R::at(r_in, s_in)] >> (16 * (t >> 1));
+                else {                         // the slot's first step may start in the upper half of its word
+                    const int h = (int)(((row0 + r_in) * steps + s_begin + (i - s_in)) & 1) + s_in;
+                    sc[q] = sw[R::at(r_in, h >> 1)] >> (16 * (h & 1));
+                }
             }
-        }
-        Scales s[4];
-        const uint4* fg = p.frag + ((s_begin + i) * gridDim.z + blockIdx.z) * (NT * 128);
+            Scales s[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {          // pieces of 8 elements of the lane's 32
-            if (j == 0 || (GS == 16 && j == 2)) {
+            for (int j = 0; j < 4; ++j) {      // pieces of 8 elements of the lane's 32
+                if (j == 0 || (GS == 16 && j == 2)) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) s[q] = make_scales(j ? sc[q] >> 16 : sc[q]);
-            }
-            uint4 b[NT];
-#pragma unroll
-            for (int m = 0; m < NT; ++m) b[m] = __ldg(fg + m * 128 + frag_pos(j, lane));
-#pragma unroll
-            for (int blk = 0; blk < 2; ++blk) {
-                const uint32_t w0 = j == 0 ? cw[2 * blk].x : j == 1 ? cw[2 * blk].y : j == 2 ? cw[2 * blk].z : cw[2 * blk].w;
-                const uint32_t w1 = j == 0 ? cw[2 * blk + 1].x : j == 1 ? cw[2 * blk + 1].y : j == 2 ? cw[2 * blk + 1].z : cw[2 * blk + 1].w;
-                const uint4 a0 = decode_word(w0, s[2 * blk]), a1 = decode_word(w1, s[2 * blk + 1]);
+                    for (int q = 0; q < 2; ++q) s[q] = make_scales(j ? sc[q] >> 16 : sc[q]);
+                }
+                const uint32_t w0 = j == 0 ? cw[0].x : j == 1 ? cw[0].y : j == 2 ? cw[0].z : cw[0].w;
+                const uint32_t w1 = j == 0 ? cw[1].x : j == 1 ? cw[1].y : j == 2 ? cw[1].z : cw[1].w;
+                const uint4 a0 = decode_word(w0, s[0]), a1 = decode_word(w1, s[1]);
 #pragma unroll
                 for (int m = 0; m < NT; ++m) {
-                    mma_f16(acc[blk][m], a0.x, a1.x, a0.y, a1.y, b[m].x, b[m].y);
-                    mma_f16(acc[blk][m], a0.z, a1.z, a0.w, a1.w, b[m].z, b[m].w);
+                    mma_f16(acc[blk][m], a0.x, a1.x, a0.y, a1.y, bf[j][m].x, bf[j][m].y);
+                    mma_f16(acc[blk][m], a0.z, a1.z, a0.w, a1.w, bf[j][m].z, bf[j][m].w);
                 }
             }
         }
     }
     cp_async_wait<0>();
     __syncthreads();                           // the rings become the partial products [warp][token][row]
-    constexpr int kPitch = kStreamRows + 4, kTokens = NT * kTok;
-    static_assert(kWarps * kTokens * kPitch * 4 <= R::kBytes, "the partial products reuse the rings");
+    constexpr int kTokens = NT * kTok;
+    const int pitch = rows + 4;
     float* part = reinterpret_cast<float*>(smem);
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < MB; ++b)
 #pragma unroll
         for (int m = 0; m < NT; ++m)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                part[(warp * kTokens + m * kTok + 2 * t + (j & 1)) * kPitch + b * 16 + (j >> 1) * 8 + g] = acc[b][m][j];
+                if (b * 16 + (j >> 1) * 8 < rows)
+                    part[(warp * kTokens + m * kTok + 2 * t + (j & 1)) * pitch + b * 16 + (j >> 1) * 8 + g] = acc[b][m][j];
     __syncthreads();
-    const int outputs = live_tok * kStreamRows;
-    if (slices == 1) {
-        for (int o = threadIdx.x; o < outputs; o += kThreads) {
-            const int m = o / kStreamRows, col = o % kStreamRows;
-            float sum = 0.f;
+    // outputs: a warp takes tokens, its lanes rows
+    const auto cta_sum = [&](int m, int col) {
+        float sum = 0.f;
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) sum += part[(w * kTokens + m) * kPitch + col];
-            if (row0 + col < p.N) p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = sum * 256.0f;
-        }
+        for (int w = 0; w < kWarps; ++w) sum += part[(w * kTokens + m) * pitch + col];
+        return sum;
+    };
+    if (slices == 1) {
+        for (int m = warp; m < live_tok; m += kWarps)
+            for (int col = lane; col < rows_left; col += 32) p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = cta_sum(m, col) * 256.0f;
         return;
     }
-    for (int o = threadIdx.x; o < outputs; o += kThreads) {          // the CTA's sum over its warps, on top of warp 0's part
-        const int m = o / kStreamRows, col = o % kStreamRows;
-        float sum = 0.f;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) sum += part[(w * kTokens + m) * kPitch + col];
-        part[m * kPitch + col] = sum;
-    }
+    for (int m = warp; m < live_tok; m += kWarps)                    // the CTA's sum over its warps, on top of warp 0's part
+        for (int col = lane; col < rows; col += 32) part[m * pitch + col] = cta_sum(m, col);
     cluster.sync();
-    for (int o = slice * kThreads + threadIdx.x; o < outputs; o += slices * kThreads) {
-        const int m = o / kStreamRows, col = o % kStreamRows;
-        float sum = 0.f;
-        for (int r = 0; r < slices; ++r) sum += cluster.map_shared_rank(part, r)[m * kPitch + col];
-        if (row0 + col < p.N) p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = sum * 256.0f;
-    }
+    for (int m = slice * kWarps + warp; m < live_tok; m += slices * kWarps)
+        for (int col = lane; col < rows_left; col += 32) {
+            float sum = 0.f;
+            for (int r = 0; r < slices; ++r) sum += cluster.map_shared_rank(part, r)[m * pitch + col];
+            p.C[(int64_t)(m0 + m) * p.ld_c + row0 + col] = sum * 256.0f;
+        }
     cluster.sync();                            // no CTA leaves while its sums are still read
 }
 
@@ -522,25 +536,62 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 3 : 2) gemm_rows_stream_ke
 struct RowsPlan {
     bool stream;
     int nt, m_blocks, slices, steps_max;
+    int mb, rows;                    // streaming kernel: 16-row blocks a CTA has accumulators for, weight rows it covers
     double us;                       // estimated time of both launches
     int tiles() const { return nt * m_blocks; }
 };
 
 constexpr int kSmCount = 148;
 
-RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
+int stream_warp_bytes(int gs, int rows) {
+    return gs == 16 ? StreamRing<16>::warp_bytes(rows) : gs == 32 ? StreamRing<32>::warp_bytes(rows)
+         : gs == 64 ? StreamRing<64>::warp_bytes(rows) : StreamRing<128>::warp_bytes(rows);
+}
+
+// The streaming kernel's layout: weight rows per CTA and K ranges, by a time model fitted to 2700 calls with given layouts (22
+// weights of N 512 to 14336, K 512 to 14336, from HBM; 1, 16, 24 and 32 rows).  Per wave of CTAs: the start, per step of a warp
+// either the latency of its own 16-row blocks or the throughput of all blocks on the SM, the sums over the warps, and the meeting of a
+// cluster.  The layout it picks is within 1.1, 1.2, 2.4 and 4.3 % of the best on average for one to four token tiles.  (CTAs
+// of 32 rows with one and a half of them per SM by K ranges, as before: 24 rows of 6144 x 4096 18.3 us against 11.6, 16 rows of
+// 5120 x 2560 13.1 / 8.0, one row of 4096 x 4096 8.9 / 7.2.)
+RowsPlan plan_stream(int nt, int64_t N, int64_t K, int gs) {
+    struct Fit { double call, start, latency, block, rate, row, meeting, full; };
+    static constexpr Fit kFit[4] = {{0.92, 1.73, 0.36, 0.28, 0.38, 0.019, 1.63, 0.84}, {0.89, 2.26, 0.44, 0.25, 0.46, 0.019, 1.89, 0.86},
+                                    {1.48, 2.00, 0.39, 0.40, 0.50, 0.021, 2.25, 0.92}, {1.36, 2.49, 0.33, 0.50, 0.50, 0.023, 2.29, 0.93}};
+    const Fit& f = kFit[nt - 1];
+    const int steps = (int)(K / kStepK);
+    RowsPlan best{};
+    for (int s = 1; s <= kMaxSlices && (s == 1 || steps >= 8 * s); s *= 2)
+        for (int rows = 8; rows <= 112; rows += 8) {
+            const int mb = rows <= 32 ? 2 : rows <= 64 ? 4 : 7;
+            const size_t smem = (size_t)kWarps * stream_warp_bytes(gs, rows);
+            if (smem > kMaxSmem) break;
+            const int64_t sms = s <= 2 ? kSmCount : s == 4 ? 132 : 120, fit = (int64_t)(kSmSmem / (smem + kCtaSmem));
+            const int64_t per_sm = fit < stream_ctas(nt, mb) ? fit : stream_ctas(nt, mb);
+            const int64_t ctas = (N + rows - 1) / rows * s, waves = (ctas + per_sm * sms - 1) / (per_sm * sms);
+            const int64_t last = (ctas - (waves - 1) * per_sm * sms + sms - 1) / sms;
+            const int blocks = (rows + 15) / 16, n = ((steps + s - 1) / s + kWarps - 1) / kWarps;
+            auto wave = [&](double resident) {
+                const double alone = f.latency + blocks * f.block, shared = resident * blocks * f.rate;
+                return f.start + n * (alone > shared ? alone : shared) + f.row * rows + (s > 1 ? f.meeting : 0.0);
+            };
+            const double us = f.call + (double)(waves - 1) * f.full * wave((double)per_sm) + wave((double)(last < per_sm ? last : per_sm));
+            if (!best.nt || us < best.us) best = {true, nt, 1, s, (steps + s - 1) / s, mb, rows, us};
+        }
+    return best;
+}
+
+RowsPlan plan_rows(int64_t M, int64_t N, int64_t K, int gs) {
     const int64_t steps = K / kStepK;
     const int tiles = (int)((M + kTok - 1) / kTok);
     // Up to 32 tokens, or blocks of 32 tokens while all of them together are resident at once (a small layer: 6-9 us).
-    const int64_t stream_blocks = (N + kStreamRows - 1) / kStreamRows;
+    const int64_t stream_blocks = (N + 31) / 32;
     const int m_blocks32 = (tiles + 3) / 4;
-    if (tiles > 4 && stream_blocks * m_blocks32 <= 2 * kSmCount && N * K <= (1ll << 21)) return {true, 4, m_blocks32, 1, (int)steps, 9.0};
-    if (tiles <= 4) {
-        // one and a half CTAs per SM, and at least one step per warp
-        int s = 1;
-        while (s < kMaxSlices && stream_blocks * s < 3 * kSmCount / 2 && steps >= 16 * s) s *= 2;
-        return {true, tiles, 1, s, (int)((steps + s - 1) / s), 0.0};
+    if (tiles > 4 && stream_blocks * m_blocks32 <= 2 * kSmCount && N * K <= (1ll << 21)) {
+        const int rows = (N + 15) / 16 * m_blocks32 <= 2 * kSmCount ? 16 : 32;
+        return {true, 4, m_blocks32, 1, (int)steps, 2, rows, 9.0};
     }
+    if (tiles <= 4) return plan_stream(tiles, N, K, gs);
     // Time in us, fitted to 2100 calls with given layouts (39 weights of N 256 to 28672, K 512 to 16384, from HBM; 33 to 256
     // rows): 3 for the fragments and the start, then per wave of CTAs its steps' decode and MMAs, its own start and, with a
     // cluster, the meeting at the end.  Within 4 % on average for blocks of 48 and 64 rows, 9 % for 32; the layout it picks
@@ -558,7 +609,7 @@ RowsPlan plan_rows(int64_t M, int64_t N, int64_t K) {
         for (int s = 1; s <= kMaxSlices && s <= steps; ++s) {
             const int64_t ctas = row_blocks * s * m_blocks, n = (steps + s - 1) / s, sms = (nt == 4 ? kSms32 : kSms)[s - 1];
             const double us = 3.0 + (double)((ctas + sms - 1) / sms) * ((double)n * step + (s > 1 ? meeting : start));
-            if (!best.nt || us < best.us) best = {false, nt, m_blocks, s, (int)n, us};
+            if (!best.nt || us < best.us) best = {false, nt, m_blocks, s, (int)n, 0, 0, us};
         }
     }
     return best;
@@ -571,13 +622,15 @@ struct RowsKernel {
 
 template <int GS>
 RowsKernel kernel_for(const RowsPlan& pl) {
-    constexpr size_t kStream = StreamRing<GS>::kBytes;
     if (pl.stream) {
+        const size_t ring = (size_t)kWarps * StreamRing<GS>::warp_bytes(pl.rows), part = (size_t)stream_part_bytes(pl.nt, pl.rows);
+        const size_t bytes = ring > part ? ring : part;
+        auto pick = [&](auto two, auto four, auto seven) { return pl.mb <= 2 ? two : pl.mb <= 4 ? four : seven; };
         switch (pl.nt) {
-            case 1: return {gemm_rows_stream_kernel<1, GS>, kStream, 0};
-            case 2: return {gemm_rows_stream_kernel<2, GS>, kStream, 0};
-            case 3: return {gemm_rows_stream_kernel<3, GS>, kStream, 0};
-            default: return {gemm_rows_stream_kernel<4, GS>, kStream, 0};
+            case 1: return {pick(gemm_rows_stream_kernel<1, 2, GS>, gemm_rows_stream_kernel<1, 4, GS>, gemm_rows_stream_kernel<1, 7, GS>), bytes, 0};
+            case 2: return {pick(gemm_rows_stream_kernel<2, 2, GS>, gemm_rows_stream_kernel<2, 4, GS>, gemm_rows_stream_kernel<2, 7, GS>), bytes, 0};
+            case 3: return {pick(gemm_rows_stream_kernel<3, 2, GS>, gemm_rows_stream_kernel<3, 4, GS>, gemm_rows_stream_kernel<3, 7, GS>), bytes, 0};
+            default: return {pick(gemm_rows_stream_kernel<4, 2, GS>, gemm_rows_stream_kernel<4, 4, GS>, gemm_rows_stream_kernel<4, 7, GS>), bytes, 0};
         }
     }
     switch (pl.nt) {
@@ -589,10 +642,10 @@ RowsKernel kernel_for(const RowsPlan& pl) {
 
 int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cudaStream_t st) {
     const RowsKernel kernel = gs == 16 ? kernel_for<16>(pl) : gs == 32 ? kernel_for<32>(pl) : gs == 64 ? kernel_for<64>(pl) : kernel_for<128>(pl);
-    static bool configured[64][2][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
+    static bool configured[64][4][4][kMaxTiles + 1] = {};   // the opt-in to > 48 KB of shared memory: per device and kernel
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return AMX_ERR_CUDA;
-    bool& done = configured[dev][pl.stream][gs == 16 ? 0 : gs == 32 ? 1 : gs == 64 ? 2 : 3][pl.nt];
+    bool& done = configured[dev][pl.stream ? (pl.mb <= 2 ? 1 : pl.mb <= 4 ? 2 : 3) : 0][gs == 16 ? 0 : gs == 32 ? 1 : gs == 64 ? 2 : 3][pl.nt];
     if (!done) {
         if (cudaFuncSetAttribute(kernel.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess) {
             cudaGetLastError();
@@ -602,9 +655,16 @@ int launch_rows(RowsParams p, const RowsPlan& pl, int gs, bool programmatic, cud
     }
     const int held = pl.steps_max < scale_steps(gs) ? pl.steps_max : scale_steps(gs);
     p.steps_max = pl.steps_max;
-    const int cta_rows = pl.stream ? kStreamRows : kCtaRows;
+    p.rows = pl.rows;
+    const int cta_rows = pl.stream ? pl.rows : kCtaRows;
     const dim3 grid((unsigned)((p.N + cta_rows - 1) / cta_rows), (unsigned)pl.slices, (unsigned)pl.m_blocks);
-    const size_t smem = kernel.ring_bytes + (pl.stream ? 0 : (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes);
+    size_t smem = kernel.ring_bytes + (pl.stream ? 0 : (size_t)scale_bytes(held, gs) + kernel.frag_ring_bytes);
+    if (pl.stream) {
+        // Blocks crowd on the SMs that the launch before leaves first: shared memory is asked for such that an SM takes no more of
+        // them than its share.
+        const size_t share = (grid.x * grid.y * grid.z + kSmCount - 1) / kSmCount, crowded = kSmSmem / (share + 1) - kCtaSmem + 128;
+        if (share < 4 && smem < crowded) smem = crowded;
+    }
     return launch_with(dim3(1, (unsigned)pl.slices), programmatic, kernel.fn, grid, kThreads, smem, st, p);
 }
 
@@ -630,7 +690,7 @@ int launch_fragments(const uint8_t* codes, const uint8_t* scales, const uint16_t
 int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int64_t ld_x, const uint8_t* w_codes,
              const uint8_t* w_scales, int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace,
              cudaStream_t st) {
-    const RowsPlan pl = plan_rows(M, N, K);
+    const RowsPlan pl = plan_rows(M, N, K, gs);
     const bool programmatic = programmatic_launch_ok(st);      // asked once for both launches
     RowsParams p{};
     p.frag = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(workspace) + kHeaderBytes);
@@ -647,16 +707,18 @@ int run_rows(const uint8_t* a_codes, const uint8_t* a_scales, const void* x, int
 
 bool gemm_rows_supported(int64_t M, int64_t N, int64_t K, int gs) {
     return fixed_group_size(gs) && M >= 1 && M <= kRowsMaxM && N >= 1 && K >= kStepK && K % kStepK == 0 &&
-           (N + kStreamRows - 1) / kStreamRows <= 0x7FFFFFFF;
+           N <= 0x7FFFFFFFll * 8;
 }
 
 size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K) {
+    constexpr int gs = 32;                     // (the tokens' tiles do not depend on it)
     // (blocks of 32, 48 or 64 rows round M up differently: what suffices for M rows on this kernel also suffices for fewer)
-    const int64_t rows = (int64_t)plan_rows(M, N, K).tiles() * kTok, whole = M > 64 ? (M + 63) / 64 * 64 : 0;
+    const int64_t rows = (int64_t)plan_rows(M, N, K, gs).tiles() * kTok, whole = M > 64 ? (M + 63) / 64 * 64 : 0;
     return kHeaderBytes + (size_t)(rows > whole ? rows : whole) * (size_t)K * 2;
 }
 
-double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) { return plan_rows(M, N, K).us; }
+double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) {
+    constexpr int gs = 32; return plan_rows(M, N, K, gs).us; }
 
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
               int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
