@@ -3,14 +3,14 @@
 // scale decomposes into the error of elements beyond the largest representable magnitude and the rounding error
 // of all others).  An element is clamped when |x| > 6 * (the scale of its side).
 //
-// Memory-bound reduction: 2 bytes of source, half a byte of codes and the scale bytes per element are read once.
-// A thread takes 16 consecutive elements at a time (two 16-byte loads of the source, one 8-byte load of codes), the next
-// chunk's loads in flight while it works; x - xhat is exact in fp32 for the output of the casts (both have few significant
-// bits and nearby exponents).  What bounds the kernel is the arithmetic (about 20 cycles of a warp per pair of elements on
-// the FMA pipe), so it is packed: two codes are decoded by one convert and three f16 instructions (decode_math.cuh), the
-// sums are packed fp32 multiply-adds, and the clamping error needs no selection at all - with y = x clamped to the group's
-// range, x - y is the error of a clamped element and zero for every other one.  (Element by element, with the scale
-// and the clamped elements selected, it took 41 us on 4096 x 11008 instead of 22.)
+// A reduction: 2 bytes of source, half a byte of codes and the scale bytes per element are read once.  A thread takes 16
+// consecutive elements at a time (two 16-byte loads of the source, one 8-byte load of codes), two chunks ahead of the one it works
+// on; three blocks per SM have the registers for that.  What bounds the kernel is instruction issue (25 warp instructions per pair of
+// elements, 69 % of the issue slots; the bytes alone take 18 of its 27 us on 4096 x 11008), so the arithmetic is packed: two
+// codes are decoded by one convert and three f16 instructions (decode_math.cuh), the decoded f16 and the clamped bf16 values go into
+// fp32 multiply-adds as they are (converted first: 30 instructions, 30 us), the sums are packed fp32 multiply-adds, and the
+// clamping error needs no selection at all - with y = x clamped to the group's range, x - y is the error of a clamped element
+// and zero for every other one.  (Copies through a ring in shared memory: no faster, the addresses cost what the waits did.)
 // The 16 squares of a chunk are added in fp32 (relative error below 2^-20 of the chunk's sum: all terms are
 // non-negative), everything above a chunk in fp64 - fp64 arithmetic per element would bound the kernel (the
 // conversions alone cost more than the memory traffic).  The clamped count is an integer.  The summation order is fixed
@@ -27,7 +27,7 @@
 namespace amx {
 namespace {
 
-constexpr int kThreads = 256, kMaxBlocks = 2048, kGrid = 148 * 4;
+constexpr int kThreads = 256, kMaxBlocks = 2048, kBlocksPerSm = 3, kGrid = 148 * kBlocksPerSm;
 
 struct Sums {
     double x2, e2, clamp2, clamped;
@@ -81,6 +81,22 @@ __device__ __forceinline__ Sums block_sum(Sums s, double (*sh)[4]) {
     return t;
 }
 
+// x - 16 h and x - y with element H of an f16 or bf16 pair straight in an fp32 multiply-add.
+template <int H>
+__device__ __forceinline__ uint32_t minus_16_times(uint32_t pair, uint32_t x) {
+    uint32_t r;
+    if (H == 0) asm("{.reg .b16 lo, hi, m; mov.b16 m, 0xCC00; mov.b32 {lo, hi}, %1; fma.rn.f32.f16 %0, lo, m, %2;}" : "=r"(r) : "r"(pair), "r"(x));
+    else asm("{.reg .b16 lo, hi, m; mov.b16 m, 0xCC00; mov.b32 {lo, hi}, %1; fma.rn.f32.f16 %0, hi, m, %2;}" : "=r"(r) : "r"(pair), "r"(x));
+    return r;
+}
+template <int H>
+__device__ __forceinline__ uint32_t minus_bf16(uint32_t pair, uint32_t x) {
+    uint32_t r;
+    if (H == 0) asm("{.reg .b16 lo, hi, m; mov.b16 m, 0xBF80; mov.b32 {lo, hi}, %1; fma.rn.f32.bf16 %0, lo, m, %2;}" : "=r"(r) : "r"(pair), "r"(x));
+    else asm("{.reg .b16 lo, hi, m; mov.b16 m, 0xBF80; mov.b32 {lo, hi}, %1; fma.rn.f32.bf16 %0, hi, m, %2;}" : "=r"(r) : "r"(pair), "r"(x));
+    return r;
+}
+
 // The same for E5M2 scales (bytes {neg : pos}), two elements at a time.
 __device__ __forceinline__ void add16_e5m2(ThreadSums& s, const uint4 (&xw)[2], uint2 cw, uint32_t sc) {
     const uint32_t xs[8] = {xw[0].x, xw[0].y, xw[0].z, xw[0].w, xw[1].x, xw[1].y, xw[1].z, xw[1].w};
@@ -88,7 +104,6 @@ __device__ __forceinline__ void add16_e5m2(ThreadSums& s, const uint4 (&xw)[2], 
     // the largest values the two sides represent, 6 x scale: exact in bf16
     const uint32_t tp = __float_as_uint(6.0f * e5m2_to_float(sc & 0xFFu)), tn = __float_as_uint(-6.0f * e5m2_to_float((sc >> 8) & 0xFFu)),
                    top = __byte_perm(tp, tp, 0x3232), bottom = __byte_perm(tn, tn, 0x3232);
-    const uint64_t minus16 = cast::pack_f32x2(0xC1800000u, 0xC1800000u), minus1 = cast::pack_f32x2(0xBF800000u, 0xBF800000u);
     uint64_t x2 = 0, e2 = 0, c2 = 0;
     uint32_t counts = 0;
     const uint4 v[2] = {decode_f16::decode_word(cw.x, scl), decode_f16::decode_word(cw.y, scl)};
@@ -96,12 +111,11 @@ __device__ __forceinline__ void add16_e5m2(ThreadSums& s, const uint4 (&xw)[2], 
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const uint64_t x = cast::pack_f32x2(xs[i] << 16, xs[i] & 0xFFFF0000u);
-        const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&xh[i]));
-        const uint64_t e = cast::fma_f32x2(cast::pack_f32x2(__float_as_uint(h.x), __float_as_uint(h.y)), minus16, x);
+        const uint64_t e = cast::pack_f32x2(minus_16_times<0>(xh[i], xs[i] << 16), minus_16_times<1>(xh[i], xs[i] & 0xFFFF0000u));
         // clamped on the bit patterns: signed 16-bit order for the positive values (the negative ones are below), unsigned
         // order for the negative ones (larger magnitude, larger pattern; the positive ones are below)
         const uint32_t y = __vminu2(__vmins2(xs[i], top), bottom);
-        const uint64_t d = cast::fma_f32x2(cast::pack_f32x2(y << 16, y & 0xFFFF0000u), minus1, x);
+        const uint64_t d = cast::pack_f32x2(minus_bf16<0>(y, xs[i] << 16), minus_bf16<1>(y, xs[i] & 0xFFFF0000u));
         x2 = cast::fma_f32x2(x, x, x2);
         e2 = cast::fma_f32x2(e, e, e2);
         c2 = cast::fma_f32x2(d, d, c2);
@@ -119,7 +133,7 @@ __device__ __forceinline__ void add16_e5m2(ThreadSums& s, const uint4 (&xw)[2], 
 
 // CONTIG: rows without gaps, everything is indexed by the chunk number (a row holds whole groups).
 template <bool F16S, bool CONTIG>
-__global__ void __launch_bounds__(kThreads, 4) quant_error_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K,
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm) quant_error_kernel(const uint16_t* __restrict__ x, int64_t rows, int64_t K,
                                                                   int64_t ld_x, const uint8_t* __restrict__ codes,
                                                                   const uint8_t* __restrict__ scales, int gs_log2,
                                                                   double* __restrict__ partial) {
@@ -128,29 +142,40 @@ __global__ void __launch_bounds__(kThreads, 4) quant_error_kernel(const uint16_t
     const int64_t per_row = K / 16, chunks = rows * per_row, stride = (int64_t)gridDim.x * kThreads;
     int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     ThreadSums s = {0, 0, 0, 0};
-    uint4 xw[2];
-    uint2 cw;
-    uint32_t sc;
-    auto load = [&]() {
-        const uint4* xp = reinterpret_cast<const uint4*>(x) + v * 2;
-        if (!CONTIG) xp = reinterpret_cast<const uint4*>(x + (v / per_row) * ld_x) + (v % per_row) * 2;
-        xw[0] = __ldg(xp);
-        xw[1] = __ldg(xp + 1);
-        cw = __ldg(reinterpret_cast<const uint2*>(codes) + v);
-        const int64_t g = v >> (gs_log2 - 4);
-        sc = F16S ? __ldg(reinterpret_cast<const uint32_t*>(scales) + g) : __ldg(reinterpret_cast<const unsigned short*>(scales) + g);
+    struct Chunk {
+        uint4 x[2];
+        uint2 codes;
+        uint32_t sc;
     };
-    if (v < chunks) load();
-    while (v < chunks) {
-        const uint4 xc[2] = {xw[0], xw[1]};
-        const uint2 cc = cw;
-        const uint32_t scc = sc;
-        v += stride;
-        if (v < chunks) load();
+    auto load = [&](Chunk& c, int64_t u) {
+        if (u >= chunks) return;
+        const uint4* xp = reinterpret_cast<const uint4*>(x) + u * 2;
+        if (!CONTIG) xp = reinterpret_cast<const uint4*>(x + (u / per_row) * ld_x) + (u % per_row) * 2;
+        c.x[0] = __ldg(xp);
+        c.x[1] = __ldg(xp + 1);
+        c.codes = __ldg(reinterpret_cast<const uint2*>(codes) + u);
+        const int64_t g = u >> (gs_log2 - 4);
+        c.sc = F16S ? __ldg(reinterpret_cast<const uint32_t*>(scales) + g) : __ldg(reinterpret_cast<const unsigned short*>(scales) + g);
+    };
+    auto add = [&](const Chunk& c) {
         if (F16S)
-            add16(s, xc, cc, __half2float(__ushort_as_half((unsigned short)(scc & 0xFFFFu))),
-                  __half2float(__ushort_as_half((unsigned short)(scc >> 16))));
-        else add16_e5m2(s, xc, cc, scc);
+            add16(s, c.x, c.codes, __half2float(__ushort_as_half((unsigned short)(c.sc & 0xFFFFu))),
+                  __half2float(__ushort_as_half((unsigned short)(c.sc >> 16))));
+        else add16_e5m2(s, c.x, c.codes, c.sc);
+    };
+    Chunk c0, c1, c2;                                            // two chunks in flight while one is worked on
+    load(c0, v);
+    load(c1, v + stride);
+    while (v < chunks) {
+        load(c2, v + 2 * stride);
+        add(c0);
+        if ((v += stride) >= chunks) break;
+        load(c0, v + 2 * stride);
+        add(c1);
+        if ((v += stride) >= chunks) break;
+        load(c1, v + 2 * stride);
+        add(c2);
+        v += stride;
     }
     const Sums t = block_sum({s.x2, s.e2, s.clamp2, (double)s.clamped}, sh);
     if (threadIdx.x == 0) {
