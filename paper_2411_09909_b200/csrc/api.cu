@@ -678,8 +678,7 @@ extern "C" int amx_attention_gqa(const void* q, const void* k, const void* v, in
             const int64_t Lp = attn_fused_padded(L);
             const PrepOperand op[2] = {gemm_fp4_cast_operand(qh, d, hc * Lp, d, false, nullptr, w + a.qs, w + a.pq, chunk_max * Lp, L, Lp),
                                        gemm_fp4_cast_operand(kh, d, kvc * Lp, d, true, nullptr, w + a.ks, w + a.pk, chunk_max * Lp, L, Lp)};
-            rc = gemm_fp4_prepare_operands(op, 2, d, 32, st, AMX_FMT_AMXFP4, words + 1);
-            if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(vh, kvc, L, d, 128, chunk_max * 128, w + a.vs, w + a.pv, st, words + 1);
+            rc = gemm_fp4_prepare_attention(op, vh, kvc, L, d, chunk_max * 128, w + a.vs, w + a.pv, st, words + 1);
             const int kv_group = (int)(group >= chunk_max ? chunk_max : group);
             float* oh = o + (size_t)h0 * L * d;
             if (rc == AMX_OK)
@@ -785,8 +784,7 @@ extern "C" int amx_attention_map(const void* q, const void* k, const void* v, in
     if (clear_words(words, st) != AMX_OK) return AMX_ERR_CUDA;
     const PrepOperand op[2] = {gemm_fp4_cast_operand(q, d, L, d, false, nullptr, w + a.qs, w + a.pq),
                                gemm_fp4_cast_operand(k, d, L, d, true, nullptr, w + a.ks, w + a.pk)};
-    int rc = gemm_fp4_prepare_operands(op, 2, d, 32, st);
-    if (rc == AMX_OK) rc = gemm_fp4_quantize_vt_prepared(v, 1, L, d, 128, 128, w + a.vs, w + a.pv, st, nullptr);
+    const int rc = gemm_fp4_prepare_attention(op, v, 1, L, d, 128, w + a.vs, w + a.pv, st, nullptr);
     if (rc != AMX_OK) return rc;
     return attn_fused({w + a.pq, L, L, 0}, {w + a.pk, L, L, 0}, {w + a.pv, 128, 128, 0}, 1, L, d, 1.0f / sqrtf((float)d), causal,
                       false, w + a.stats, o, words, st, p_bf16, p_codes, p_scales, p_prepared);

@@ -88,10 +88,20 @@ PrepOperand gemm_fp4_split_operand(const uint8_t* codes, const uint8_t* scales, 
                                    void* prepared, int64_t layout_rows = 0);
 int gemm_fp4_prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, cudaStream_t st, int format = AMX_FMT_AMXFP4,
                               int* flushed_total = nullptr);
-int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64_t d, int64_t seg_pad, int64_t layout_rows,
-                                  uint8_t* scales, void* prepared, cudaStream_t st, int* flushed_total);
-int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int64_t seg_pad, void* pos, void* neg, uint8_t* scales,
-                         cudaStream_t st);
+// The casts of an attention call in one launch: two operands described above, and V ([kv_heads][L][d], contiguous) as V^T, 128
+// operand rows per head, laid out for layout_rows rows; its canonical scales (and no codes) are written beside.
+int gemm_fp4_prepare_attention(const PrepOperand (&qk)[2], const void* v, int64_t kv_heads, int64_t L, int64_t d, int64_t layout_rows,
+                               uint8_t* v_scales, void* v_prepared, cudaStream_t st, int* flushed_total);
+struct VtOperand {
+    const uint4* x;
+    int64_t L;
+    int d, nk64;
+    uint4 *pos, *neg;
+    uint16_t* scales;
+    uint8_t *sf_pos, *sf_neg;
+    int* row_exp;
+};
+int prepare_attention(const PrepOperand (&qk)[2], int64_t d, int nk64, const VtOperand& vt, int64_t kv_heads, cudaStream_t st, int* flushed_total);
 const int* gemm_fp4_row_words(const void* prepared, int64_t rows, int64_t K, bool is_weight);
 // Softmax of the rows of S, rounded to bf16 and cast in one launch (cols % 32 == 0); pos == nullptr: canonical
 // output only.  gemm_fp4_softmax_prepared lays the prepared operand out like gemm_fp4_quantize_prepared.

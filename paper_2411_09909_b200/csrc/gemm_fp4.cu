@@ -114,73 +114,6 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) {
 // UE4M3 scale factors (bit 23 = 0), N >> 3 at bit 17, M >> 4 at bit 24, K = 64 (bit 31 = 0).
 __host__ __device__ constexpr uint32_t instr_desc(int n) { return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24); }
 
-// ------------------------------------------------------------------------- preparation --
-// Row words and scale factors of an operand (group size 32) whose sign planes are there already, from its canonical scales:
-// V^T of an attention call, whose cast writes the planes (quantize.cu; every other operand is prepared by the kernel
-// there).  A block has kPrepRows rows; a warp per row finds the largest exponent key kmax among the row's scales (kmax - 25 is
-// the power of two by which the row's UE4M3 scales understate the true ones) and which sides occur at all; then the
-// scale factors of both planes in the layout the MMA reads: [plane][row block of 128][K/64 block][512 B], byte
-// (r%32)*16 + (r/32)*4 + (k16 % 4), one scale per 16 elements, so a group's scale is written twice.  Operand rows come in
-// segments of seg_pad rows of which the first seg_rows are in use.
-constexpr int kPrepRows = 8;
-__global__ void __launch_bounds__(256)
-scale_factors_kernel(const uint8_t* __restrict__ scales, int64_t R, int64_t K, int nk64, uint8_t* __restrict__ sf_pos,
-                     uint8_t* __restrict__ sf_neg, int* __restrict__ row_exp, int* __restrict__ flushed_total, int seg_rows, int seg_pad) {
-    begin_kernel();
-    __shared__ int kmax_s[kPrepRows];
-    const int64_t row0 = (int64_t)blockIdx.x * kPrepRows, G = K / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    auto in_use = [&](int64_t row) { return row < R && (int)(row % seg_pad) < seg_rows; };
-    for (int r = warp; r < kPrepRows; r += 8) {
-        const int64_t row = row0 + r;
-        int kmax = 0, sides = 0, flushed = 0;
-        const unsigned short* s2 = reinterpret_cast<const unsigned short*>(scales + row * G * 2);
-        if (in_use(row))
-            for (int64_t g = lane; g < G; g += 32) {
-                const uint32_t v = __ldg(s2 + g);
-                kmax = max(kmax, max(scale_key(v & 0xFF), scale_key(v >> 8)));
-                sides |= side_bits_of(v);
-            }
-        kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
-        sides = __reduce_or_sync(0xFFFFFFFFu, sides);
-        if (in_use(row))                                         // scales below the row's UE4M3 range: flushed
-            for (int64_t g = lane; g < G; g += 32) {
-                const uint32_t v = __ldg(s2 + g);
-                flushed += (int)ue4m3_flushes(v & 0xFF, kmax) + (int)ue4m3_flushes(v >> 8, kmax);
-            }
-        flushed = __reduce_add_sync(0xFFFFFFFFu, flushed);
-        if (lane == 0) {
-            kmax_s[r] = kmax;
-            if (in_use(row)) row_exp[row] = row_word(kmax, sides, flushed);
-            if (flushed && flushed_total) atomicAdd(flushed_total, flushed);
-        }
-    }
-    __syncthreads();
-    // scale factors: item = (K/64 block c, row r); consecutive threads take consecutive rows
-    const int64_t rb = row0 / 128;
-    const int r_in_blk0 = (int)(row0 % 128);
-    for (int item = threadIdx.x; item < nk64 * kPrepRows; item += 256) {
-        const int c = item / kPrepRows, r = item % kPrepRows;
-        const int64_t row = row0 + r;
-        uint32_t wp = 0, wn = 0;
-        if (in_use(row)) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {                        // the two 32-groups of this 64-element block
-                const int64_t g = (int64_t)c * 2 + h;
-                if (g < G) {
-                    const uint32_t v = __ldg(reinterpret_cast<const unsigned short*>(scales + (row * G + g) * 2));
-                    wp |= to_ue4m3(v & 0xFF, kmax_s[r]) * 0x0101u << (16 * h);
-                    wn |= to_ue4m3(v >> 8, kmax_s[r]) * 0x0101u << (16 * h);
-                }
-            }
-        }
-        const int rr = r_in_blk0 + r;                            // row inside its block of 128
-        const int64_t off = (rb * nk64 + c) * (int64_t)kSfChunk + (rr % 32) * 16 + (rr / 32) * 4;
-        *reinterpret_cast<uint32_t*>(sf_pos + off) = wp;
-        *reinterpret_cast<uint32_t*>(sf_neg + off) = wn;
-    }
-}
-
 // -------------------------------------------------------------------------------- GEMM --
 struct Params {
     const int *a_exp, *w_exp;
@@ -975,17 +908,15 @@ int gemm_fp4_prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, c
     return prepare_operands(op, n, K, gs, operand_layout(128, K, BM).nk64, st, format, flushed_total);
 }
 
-// V^T of `heads` heads [L, d], seg_pad operand rows each: cast down the rows into the planes and scales, then row words and
-// scale factors from the scales.  (The rows past d of a head, and their words, are whatever they were: not read.)
-int gemm_fp4_quantize_vt_prepared(const void* v, int64_t heads, int64_t L, int64_t d, int64_t seg_pad, int64_t layout_rows,
-                                  uint8_t* scales, void* prepared, cudaStream_t st, int* flushed_total) {
+// (The rows of V^T past d of a head, and their words, are whatever they were: not read.)
+int gemm_fp4_prepare_attention(const PrepOperand (&qk)[2], const void* v, int64_t kv_heads, int64_t L, int64_t d, int64_t layout_rows,
+                               uint8_t* v_scales, void* v_prepared, cudaStream_t st, int* flushed_total) {
     const OperandLayout o = operand_layout(layout_rows, L, BN);
-    uint8_t* base = static_cast<uint8_t*>(prepared);
-    const int rc = quantize_cols_planes(v, heads, L, d, seg_pad, base, base + o.plane, scales, st);
-    if (rc != AMX_OK) return rc;
-    return launch(scale_factors_kernel, (unsigned)(heads * seg_pad / kPrepRows), 256, 0, st, scales, heads * seg_pad, L, o.nk64,
-                  base + 2 * o.plane, base + 2 * o.plane + o.sf, reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf), flushed_total,
-                  (int)d, (int)seg_pad);
+    uint8_t* base = static_cast<uint8_t*>(v_prepared);
+    const VtOperand vt = {static_cast<const uint4*>(v), L, (int)d, o.nk64, reinterpret_cast<uint4*>(base), reinterpret_cast<uint4*>(base + o.plane),
+                          reinterpret_cast<uint16_t*>(v_scales), base + 2 * o.plane, base + 2 * o.plane + o.sf,
+                          reinterpret_cast<int*>(base + 2 * o.plane + 2 * o.sf)};
+    return prepare_attention(qk, d, operand_layout(128, d, BM).nk64, vt, kv_heads, st, flushed_total);
 }
 
 // Bytes from the first to the second sign plane of a prepared operand.

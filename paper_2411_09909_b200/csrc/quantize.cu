@@ -255,6 +255,8 @@ constexpr int kCastMaxExchangeBytes = 96 * 1024;           // above this (K > 49
 
 struct PrepParams {
     PrepOperand op[2];
+    VtOperand vt;                                          // kAttention: blocks before those of the two operands
+    unsigned vt_blocks;
     unsigned blocks0;                                      // blocks of the first operand; the others are the second's
     int G, lpr_log2, exchange, nk64, gs;
     int* flushed_total;
@@ -317,19 +319,117 @@ __device__ __forceinline__ uint32_t cast_piece_gs(const uint32_t (&w)[16], bool 
     return sc[0] | (sc[1] << 16);
 }
 
-// MODE: one cast, two casts, operands that may be canonical, or any of these with a group size other than 32.  (The plain
-// cast is kept lean - its pointers are compile-time places in constant memory: it is bound by instruction issue, and four
-// blocks have to share an SM.)
-enum PrepMode { kOneCast, kTwoCasts, kAnyKind, kAnyGroup };
+// V^T of an attention call: V cast down its keys, with everything the FP4 kernel reads, beside the casts of Q and K.  A block owns
+// eight columns of one head (eight operand rows) over all keys, so that the rows' largest scales are known inside the block and
+// the scale factors follow without another launch.  Keys come in passes of 64 groups through shared memory; a group's rows
+// are 528 bytes apart from the next group's, and lanes are eight groups x four column pairs: no bank conflicts on the way out,
+// and a column's codes leave in pieces of 128 bytes.  What bounds it is latency (one load, one cast, one exchange): as two
+// launches of its own, cast and scale factors, it cost 10 us for 8 heads x 1056 keys; here it runs beside Q and K (the call with
+// 32 query heads, causal: 62.2 -> 55.4 us; 32 heads x 8192 1872 -> 1845).
+constexpr int kVtCols = 8, kVtGroups = 64, kVtPitch = 528, kVtRows = 128, kVtKept = 256;   // kVtKept: groups whose scales stay in shared memory
+size_t vt_smem_bytes(int64_t G) { return (size_t)std::min<int64_t>(G, kVtGroups) * kVtPitch + (G <= kVtKept ? G * kVtCols * 2 : 0); }
+
+__device__ __forceinline__ void cast_vt_block(const VtOperand& o, unsigned block, uint8_t* smem, int* flushed_total) {
+    __shared__ int top_s[kVtCols][2], flushed_s[kVtCols];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t head = block / (kVtRows / kVtCols), G = o.L / 32;
+    const int c0 = (int)(block % (kVtRows / kVtCols)) * kVtCols;
+    const bool in_use = c0 < o.d;                   // head dimension 64: the other rows have zero scale factors
+    const int64_t row0 = head * kVtRows + c0;
+    const bool kept = G <= kVtKept;
+    uint16_t* sc_s = reinterpret_cast<uint16_t*>(smem + min(G, (int64_t)kVtGroups) * kVtPitch);   // [column][group]
+    if (tid < kVtCols) top_s[tid][0] = top_s[tid][1] = flushed_s[tid] = 0;
+    uint32_t top[2] = {0, 0};
+    if (in_use) {
+        const uint4* src = o.x + (head * o.L * o.d + c0) / 8;
+        const int vec = o.d / 8, cw = tid & 3, g = tid >> 2;
+        for (int64_t g0 = 0; g0 < G; g0 += kVtGroups) {
+            const int n = (int)min(G - g0, (int64_t)kVtGroups);
+            if (g0) __syncthreads();                // the pass before has been read
+            for (int i = tid; i < n * 32; i += 256) cp_async16(smem + (i >> 5) * kVtPitch + (i & 31) * 16, src + (g0 * 32 + i) * vec);
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncthreads();
+            if (g >= n) continue;
+            const uint32_t* tile = reinterpret_cast<const uint32_t*>(smem + g * kVtPitch) + cw;
+            uint32_t lo[16], hi[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint32_t a = tile[8 * i], b = tile[8 * i + 4];
+                lo[i] = __byte_perm(a, b, 0x5410);
+                hi[i] = __byte_perm(a, b, 0x7632);
+            }
+            const int64_t v = (row0 + 2 * cw) * G + g0 + g;
+            const uint32_t s0 = emit_group(lo, v, nullptr, o.scales, o.pos, o.neg), s1 = emit_group(hi, v + G, nullptr, o.scales, o.pos, o.neg);
+            if (kept) {
+                sc_s[2 * cw * G + g0 + g] = (uint16_t)s0;
+                sc_s[(2 * cw + 1) * G + g0 + g] = (uint16_t)s1;
+            }
+            top[0] = __vmaxu4(top[0], s0);
+            top[1] = __vmaxu4(top[1], s1);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int d = 4; d < 32; d <<= 1) top[j] = __vmaxu4(top[j], __shfl_xor_sync(0xFFFFFFFFu, top[j], d));
+    }
+    __syncthreads();
+    if (lane < 4)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            atomicMax(&top_s[2 * lane + j][0], (int)(top[j] & 0xFFu));
+            atomicMax(&top_s[2 * lane + j][1], (int)(top[j] >> 8));
+        }
+    __syncthreads();
+    const int r = tid & (kVtCols - 1);              // of all of this thread's items
+    const int kmax = scale_key(max(top_s[r][0], top_s[r][1]));
+    const int64_t row = row0 + r, sf_row = sf_row_offset(row, o.nk64);
+    const uint16_t* sc = kept ? sc_s + r * G : o.scales + row * G;   // (written by this block)
+    int flushed = 0;
+    for (int c = tid / kVtCols; c < o.nk64; c += 256 / kVtCols) {
+        uint32_t wp = 0, wn = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int g = 2 * c + h;
+            const uint32_t v = in_use && g < G ? sc[g] : 0u;
+            const uint32_t up = to_ue4m3(v & 0xFFu, kmax), un = to_ue4m3(v >> 8, kmax);
+            flushed += (int)((v & 0xFFu) != 0 && up == 0) + (int)((v >> 8) != 0 && un == 0);
+            wp |= up * 0x0101u << (16 * h);
+            wn |= un * 0x0101u << (16 * h);
+        }
+        const int64_t off = sf_row + (int64_t)c * kSfChunkBytes;
+        *reinterpret_cast<uint32_t*>(o.sf_pos + off) = wp;
+        *reinterpret_cast<uint32_t*>(o.sf_neg + off) = wn;
+    }
+    if (!in_use) return;                            // (nor are those rows' words read)
+#pragma unroll
+    for (int d = kVtCols; d < 32; d <<= 1) flushed += __shfl_xor_sync(0xFFFFFFFFu, flushed, d);
+    if (lane < kVtCols && flushed) atomicAdd(&flushed_s[r], flushed);
+    __syncthreads();
+    if (tid < kVtCols) {
+        o.row_exp[row] = row_word(kmax, side_bits_of((uint32_t)top_s[r][0] | ((uint32_t)top_s[r][1] << 8)), flushed_s[r]);
+        if (flushed_s[r] && flushed_total) atomicAdd(flushed_total, flushed_s[r]);
+    }
+}
+
+// MODE: one cast, two casts, operands that may be canonical, any of these with a group size other than 32, or the three casts
+// of an attention call.  (The plain cast is kept lean - its pointers are compile-time places in constant memory: it is bound by
+// instruction issue, and four blocks have to share an SM.)
+enum PrepMode { kOneCast, kTwoCasts, kAnyKind, kAnyGroup, kAttention };
 template <int FMT, int GPL, int MODE>
 __global__ void __launch_bounds__(kCastWarps * 32, 4)
 prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     begin_kernel();
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    constexpr bool SPLIT = MODE >= kAnyKind, ANY_GS = MODE == kAnyGroup;
-    const bool second = MODE != kOneCast && blockIdx.x >= p.blocks0;
+    constexpr bool SPLIT = MODE == kAnyKind || MODE == kAnyGroup, ANY_GS = MODE == kAnyGroup;
+    if (MODE == kAttention && blockIdx.x < p.vt_blocks) {
+        cast_vt_block(p.vt, blockIdx.x, smem_raw, p.flushed_total);
+        return;
+    }
+    const unsigned bid = blockIdx.x - (MODE == kAttention ? p.vt_blocks : 0u);
+    const bool second = MODE != kOneCast && bid >= p.blocks0;
     const PrepOperand& o = p.op[second];
-    const unsigned block = blockIdx.x - (second ? p.blocks0 : 0u);
+    const unsigned block = bid - (second ? p.blocks0 : 0u);
     const int G = p.G, lpr_log2 = p.lpr_log2, nk64 = p.nk64, gs = ANY_GS ? p.gs : 32;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, LPR = 1 << lpr_log2, lr = lane & (LPR - 1);
     const int RPW = 32 >> lpr_log2, sg = lane >> lpr_log2;      // rows per warp; which of them this lane works on
@@ -627,27 +727,34 @@ int launch_rows(const void* x, int64_t rows, int64_t K, int64_t ld, uint8_t* cod
 // 512 B per block of 128 rows, rows padded to padded_rows) and the row words.  format: of a cast (group size 32 unless
 // AMXFP4).  flushed_total (optional): incremented by the number of scales flushed.
 namespace {
-template <int FMT, int MODE>
-int launch_prepare(const PrepOperand* op, int n, int64_t K, int gs, int nk64, cudaStream_t st, int* flushed_total) {
-    PrepParams p{};
+// Everything but the columns of V; `blocks`: of all operands, `smem`: of a block; returns the pieces per lane.
+int fill_prepare(PrepParams& p, const PrepOperand* op, int n, int64_t K, int gs, int nk64, int* flushed_total, int64_t& blocks, int& smem) {
     p.G = (int)(K / 32);
     p.lpr_log2 = 1;
     while (p.lpr_log2 < 5 && (1 << p.lpr_log2) < p.G) ++p.lpr_log2;  // lanes per row: a power of two, 2 .. 32
-    const int gpl = (p.G + (1 << p.lpr_log2) - 1) >> p.lpr_log2;     // pieces per lane
     const int rpw = 32 >> p.lpr_log2;                                // rows per warp
-    int64_t blocks = 0;
+    blocks = 0;
     for (int i = 0; i < n; ++i) {
         p.op[i] = op[i];
         blocks += (op[i].padded_rows / 128) * (16 / rpw);            // a block has 8 * rpw rows of one 128-row block
         if (i == 0) p.blocks0 = (unsigned)blocks;
     }
-    if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
     p.nk64 = nk64;
     p.gs = gs;
     p.flushed_total = flushed_total;
     const size_t exchange_bytes = (size_t)64 * rpw * nk64;           // both planes, 4 bytes per row and 64 elements
     p.exchange = exchange_bytes <= (size_t)kCastMaxExchangeBytes;
-    const int smem = kCastRingBytes + (p.exchange ? (int)exchange_bytes : 0);
+    smem = kCastRingBytes + (p.exchange ? (int)exchange_bytes : 0);
+    return (p.G + (1 << p.lpr_log2) - 1) >> p.lpr_log2;
+}
+
+template <int FMT, int MODE>
+int launch_prepare(const PrepOperand* op, int n, int64_t K, int gs, int nk64, cudaStream_t st, int* flushed_total) {
+    PrepParams p{};
+    int64_t blocks;
+    int smem;
+    const int gpl = fill_prepare(p, op, n, K, gs, nk64, flushed_total, blocks, smem);
+    if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
     auto* kernel = gpl <= 1 ? prepare_operands_kernel<FMT, 1, MODE> : gpl <= 2 ? prepare_operands_kernel<FMT, 2, MODE>
                  : gpl <= 4 ? prepare_operands_kernel<FMT, 4, MODE> : gpl <= 8 ? prepare_operands_kernel<FMT, 8, MODE>
                  : prepare_operands_kernel<FMT, 0, MODE>;   // longer rows: the scale bytes are re-read, not kept in registers
@@ -676,6 +783,20 @@ int prepare_operands(const PrepOperand* op, int n, int64_t K, int gs, int nk64, 
                   : launch_prepare<0, kTwoCasts>(op, n, K, gs, nk64, st, flushed_total);
 }
 
+// The casts of an attention call in one launch: Q and K (head dimension 64 or 128, so one piece per lane) and V^T of `kv_heads` heads.
+int prepare_attention(const PrepOperand (&qk)[2], int64_t d, int nk64, const VtOperand& vt, int64_t kv_heads, cudaStream_t st, int* flushed_total) {
+    if (d != 64 && d != 128) return AMX_ERR_SHAPE;
+    PrepParams p{};
+    int64_t blocks;
+    int smem;
+    fill_prepare(p, qk, 2, d, 32, nk64, flushed_total, blocks, smem);
+    p.vt = vt;
+    p.vt_blocks = (unsigned)(kv_heads * (kVtRows / kVtCols));
+    blocks += p.vt_blocks;
+    if (blocks > 0x7FFFFFFF) return AMX_ERR_SHAPE;
+    return launch(prepare_operands_kernel<0, 1, kAttention>, (unsigned)blocks, kCastWarps * 32, std::max<size_t>(smem, vt_smem_bytes(vt.L / 32)), st, p);
+}
+
 // Softmax of the rows of S (fp32 [rows, ld_s], cols % 32 == 0), rounded to bf16 and cast, in one launch.  With
 // pos == nullptr only the canonical codes and scales are written.
 int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, float alpha, uint8_t* codes,
@@ -696,45 +817,6 @@ int softmax_cast_rows(const float* S, int64_t rows, int64_t cols, int64_t ld_s, 
 
 namespace {
 
-// V of an attention call (x: [batch][R keys][C] contiguous, C = 64 or 128) cast down its rows straight into the sign planes
-// of the FP4 operand V^T (seg_pad operand rows per matrix, R / 2 bytes each) and its canonical scales [row][R / 32][2]; the
-// canonical codes are the two planes or-ed together.  A block stages 128 keys x C columns in shared memory (16-byte loads,
-// one row of a key is C * 2 contiguous bytes) and a thread owns one 32-key group of two neighbouring columns: lanes are
-// four groups x eight column pairs, so that a column's 64 bytes of codes per block leave in one piece and the XOR of the
-// column word with the group keeps the shared-memory reads free of bank conflicts.  16 heads x 8192 x 128: 54 us of the
-// 64 x 64-tile cast and 11 us of preparing its codes before.
-template <int C>
-__global__ void __launch_bounds__(256)
-cast_cols_planes_kernel(const uint4* __restrict__ x, int64_t R, int64_t seg_pad, uint4* __restrict__ pos, uint4* __restrict__ neg,
-                        uint16_t* __restrict__ scales) {
-    begin_kernel();
-    constexpr int kWords = C / 2, kVec = C / 8;               // 32-bit words and 16-byte pieces per key
-    __shared__ __align__(16) uint32_t tile[128 * kWords];
-    const int64_t key0 = (int64_t)blockIdx.x * 128, batch = blockIdx.y;
-    const uint4* src = x + (batch * R + key0) * kVec;
-    const int keys = (int)min((int64_t)128, R - key0);
-    for (int i = threadIdx.x; i < keys * kVec; i += 256) {
-        const int key = i / kVec, v = i % kVec;
-        *reinterpret_cast<uint4*>(&tile[key * kWords + ((v * 4) ^ ((key >> 5) * 8))]) = __ldg(src + i);
-    }
-    __syncthreads();
-    const int g = threadIdx.x & 3;                            // the tile's 32-key group
-    if (g * 32 >= keys) return;
-    const int64_t G = R / 32;
-    for (int cw = threadIdx.x >> 2; cw < kWords; cw += 64) {  // column pair
-        uint32_t lo[16], hi[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const uint32_t a = tile[(g * 32 + 2 * i) * kWords + (cw ^ (g * 8))], b = tile[(g * 32 + 2 * i + 1) * kWords + (cw ^ (g * 8))];
-            lo[i] = __byte_perm(a, b, 0x5410);
-            hi[i] = __byte_perm(a, b, 0x7632);
-        }
-        const int64_t v = (batch * seg_pad + 2 * cw) * G + key0 / 32 + g;
-        emit_group(lo, v, nullptr, scales, pos, neg);
-        emit_group(hi, v + G, nullptr, scales, pos, neg);
-    }
-}
-
 template <int TPG>
 int launch_cols(const void* x, int64_t R, int64_t C, int64_t ld, int gs, uint8_t* codes,
                 uint8_t* scales, cudaStream_t st, int64_t batch = 1) {
@@ -745,16 +827,6 @@ int launch_cols(const void* x, int64_t R, int64_t C, int64_t ld, int gs, uint8_t
 }
 
 }  // namespace
-
-// V of `batch` heads into the planes and scales of V^T (cast_cols_planes_kernel).
-int quantize_cols_planes(const void* x, int64_t batch, int64_t R, int64_t C, int64_t seg_pad, void* pos, void* neg, uint8_t* scales,
-                         cudaStream_t st) {
-    if (batch > 65535 || (C != 64 && C != 128)) return AMX_ERR_SHAPE;
-    const dim3 grid((unsigned)((R + 127) / 128), (unsigned)batch);
-    auto* kernel = C == 128 ? cast_cols_planes_kernel<128> : cast_cols_planes_kernel<64>;
-    return launch(kernel, grid, 256, 0, st, static_cast<const uint4*>(x), R, seg_pad, static_cast<uint4*>(pos), static_cast<uint4*>(neg),
-                                 reinterpret_cast<uint16_t*>(scales));
-}
 
 // amx_quantize_t with group size 32 on `batch` matrices [R, C] stored one after another (contiguous rows); the
 // canonical outputs of their transposes follow one another too.
