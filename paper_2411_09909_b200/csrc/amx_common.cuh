@@ -115,6 +115,10 @@ __device__ __forceinline__ float e2m1_mag_to_float(uint32_t c3) {
     return (c3 & 6u) ? v : 0.5f * (float)(c3 & 1u);
 }
 
+// fp32 value of a scale byte without the format's special cases: its largest exponent field is read as one more power of two, as
+// everywhere where scales are taken apart below (casts saturate; only a NaN among the elements leaves such a byte).
+__device__ __forceinline__ float scale_value(uint32_t byte) { return __uint_as_float(byte << 21) * 5192296858534827628530496329220096.f; }   // 2^112
+
 // An E5M2 scale byte as (key << 2) | mantissa of its normalised form: key = unbiased exponent + 17 (so that
 // 2^-16 has key 1) and two mantissa bits.  Normal bytes (b >= 4) are b + 8; the subnormals 1, 2, 3 x 2^-16 are
 // 1.0 x 2^-16, 1.0 x 2^-15 and 1.5 x 2^-15: 4, 8 and 10 (read from a packed table); 0 for a zero scale.
@@ -152,15 +156,19 @@ __host__ __device__ __forceinline__ int64_t sf_row_offset(int64_t row, int nk64)
 }
 __host__ __device__ __forceinline__ int64_t sf_group_offset(int g) { return (int64_t)(g >> 1) * kSfChunkBytes + (g & 1) * 2; }
 
-// UE4M3 byte of the E5M2 byte b for a row whose largest key is kmax (0 when it does not fit): exponent field
-// key - kmax + 15 (at least 1), the two mantissa bits in bits 2..1.
-__device__ __forceinline__ uint32_t to_ue4m3(uint32_t b, int kmax) {
-    const int t = (int)scale_norm(b) + ((15 - kmax) << 2);       // (exponent field << 2) | mantissa
-    return (b != 0 && t >= 4) ? (uint32_t)t << 1 : 0u;
-}
-// Whether to_ue4m3 flushes the nonzero scale byte b: its key lies 15 or more below the row's largest.
-__device__ __forceinline__ bool ue4m3_flushes(uint32_t b, int kmax) {
-    return b != 0 && (int)scale_norm(b) + ((15 - kmax) << 2) < 4;
+// UE4M3 bytes of a pair of E5M2 scale bytes (bits 15..0 of sc; what lies above is ignored) for a row whose scales are multiplied by
+// `up` = sf_factor(the row's largest key): exponent field key - kmax + 15, the two mantissa bits in bits 2..1; zero where the
+// exponent field would be below 1.  `lost` counts, in steps of 128, the nonzero scales this flushes.  (By way of the hardware's
+// converts, both bytes at once: on integers, normal and subnormal scales apart, the preparation spent 60 instructions per group here.)
+__device__ __forceinline__ float sf_factor(int kmax) { return __uint_as_float((uint32_t)(25 - kmax + 127) << 23); }
+__device__ __forceinline__ uint32_t to_ue4m3x2(uint32_t sc, float up, uint32_t& lost) {
+    unsigned short both;
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(both) : "f"(scale_value((sc >> 8) & 0xFFu) * up), "f"(scale_value(sc & 0xFFu) * up));
+    const uint32_t t = both + 0x7878u;                          // bit 7 of a byte: it is a normal number
+    lost = __dp4a((sc + 0x7F7Fu) & ~t & 0x8080u, 0x0101u, lost);
+    uint32_t normal;                                            // selectors 8 and 9 replicate bit 7 (not with __byte_perm)
+    asm("prmt.b32 %0, %1, 0, 0x4498;" : "=r"(normal) : "r"(t));
+    return both & normal;
 }
 
 }  // namespace amx

@@ -39,15 +39,15 @@ __device__ __forceinline__ uint32_t cvt_e5m2x2(float hi, float lo) {
     return d;
 }
 
-// Reciprocal of the value of an E5M2 scale byte: the fp32 nearest to 1 / significand (significand 1, 1.25, 1.5,
-// 1.75: the byte's two low bits) times the exact power of two; 0 for a zero scale.  scale_norm() gives the
-// normalised form (exponent key << 2 | significand bits) of normal and subnormal bytes alike; the value is
-// significand x 2^(key - 17).
-__device__ __forceinline__ float inv_scale(uint32_t byte) {
-    const uint32_t n = scale_norm(byte), m = n & 3u;
-    const uint32_t r = m == 0 ? 0x3F800000u : m == 1 ? 0x3F4CCCCDu : m == 2 ? 0x3F2AAAABu : 0x3F124925u;   // 1, 0.8, 2/3, 4/7
-    return byte ? __uint_as_float(r + ((17u - (n >> 2)) << 23)) : 0.0f;
+// Reciprocal of the value of an E5M2 scale byte, rounded to nearest; 0 for a zero scale.  One Newton step
+// behind the hardware's approximation: with e = 1 - s r exact, r + r e differs from 1 / s by e^2 < 2^-40 of it before its one
+// rounding, and none of 1/1, 1/1.25, 1/1.5 and 1/1.75 lies that close to the middle between two fp32 numbers.
+__device__ __forceinline__ float inv_scale_value(float s) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
+    return s != 0.0f ? fmaf(r, fmaf(-s, r, 1.0f), r) : 0.0f;
 }
+__device__ __forceinline__ float inv_scale(uint32_t byte) { return inv_scale_value(scale_value(byte)); }
 
 // Side maxima of NW bf16x2 words as one word {nmax bits : pmax bits}.  Signed 16-bit max over the
 // raw patterns, clamped at 0, is the largest non-negative value; unsigned 16-bit max is the negative

@@ -67,8 +67,8 @@ struct PrepOperand {
     const uint4* in_codes;       // canonical operand
     const uint16_t* in_scales;
     int64_t R;                   // operand rows
-    int64_t seg_rows, seg_pad;   // seg_pad != 0: x holds segments of seg_rows rows, each padded to seg_pad operand rows with
-                                 // zero scale factors and row words
+    unsigned seg_rows, seg_blocks;   // seg_blocks != 0: x holds segments of seg_rows rows, each padded to seg_blocks blocks of 128
+                                     // operand rows with zero scale factors and row words
     uint4* codes;                // out, of a cast: canonical codes (optional) and scales
     uint16_t* scales;
     uint4 *pos, *neg;            // out: planes, scale factors, row words

@@ -890,8 +890,8 @@ PrepOperand gemm_fp4_cast_operand(const void* x, int64_t ld, int64_t rows, int64
     p.ld_vec = ld / 8;
     p.codes = reinterpret_cast<uint4*>(codes);
     p.scales = reinterpret_cast<uint16_t*>(scales);
-    p.seg_rows = seg_rows;
-    p.seg_pad = seg_pad;
+    p.seg_rows = (unsigned)seg_rows;
+    p.seg_blocks = (unsigned)(seg_pad / 128);
     if (seg_pad) p.padded_rows = (rows + 127) / 128 * 128;
     return p;
 }

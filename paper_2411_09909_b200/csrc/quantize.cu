@@ -206,22 +206,18 @@ __device__ __forceinline__ void finish_prepared_row(int64_t row, bool row_live, 
     // offset of this row's bytes inside a chunk; the chunks of one block of 128 rows are consecutive along K
     const int64_t sf_row = sf_row_offset(row, nk64);
     const int64_t v_row = row * G;
-    int flushed = 0;
+    const float factor = sf_factor(kmax);
+    uint32_t lost = 0;
     for (int g = gx; g < nk64 * 2; g += GX) {      // groups past G: padding to whole 256-element blocks
-        uint32_t up = 0, un = 0;
-        if (row_live && g < G) {
-            // a later group of a striding thread: re-read the scale bytes this thread stored before
-            const uint32_t sc = (g == gx) ? sc_first : scales[v_row + g];
-            up = to_ue4m3(sc & 0xFFu, kmax);
-            un = to_ue4m3(sc >> 8, kmax);
-            flushed += (int)((sc & 0xFFu) != 0 && up == 0) + (int)((sc >> 8) != 0 && un == 0);
-        }
+        uint32_t u = 0;
+        // a later group of a striding thread: re-read the scale bytes this thread stored before
+        if (row_live && g < G) u = to_ue4m3x2((g == gx) ? sc_first : scales[v_row + g], factor, lost);
         const int64_t off = sf_row + sf_group_offset(g);
-        *reinterpret_cast<uint16_t*>(sf_pos + off) = (uint16_t)(up | (up << 8));
-        *reinterpret_cast<uint16_t*>(sf_neg + off) = (uint16_t)(un | (un << 8));
+        *reinterpret_cast<uint16_t*>(sf_pos + off) = (uint16_t)__byte_perm(u, 0, 0x4400);
+        *reinterpret_cast<uint16_t*>(sf_neg + off) = (uint16_t)__byte_perm(u, 0, 0x4411);
     }
     if (!row_live) return;                         // uniform over the row's warps
-    flushed = __reduce_add_sync(0xFFFFFFFFu, flushed);
+    const int flushed = __reduce_add_sync(0xFFFFFFFFu, (int)(lost >> 7));
     if ((gx & 31) == 0) {
         if (flushed) atomicAdd(&slot[2], flushed);
         __threadfence_block();
@@ -258,7 +254,7 @@ struct PrepParams {
     VtOperand vt;                                          // kAttention: blocks before those of the two operands
     unsigned vt_blocks;
     unsigned blocks0;                                      // blocks of the first operand; the others are the second's
-    int G, lpr_log2, exchange, nk64, gs;
+    int G, lpr_log2, exchange, nk64, gs, gs_log2;
     int* flushed_total;
 };
 
@@ -385,23 +381,17 @@ __device__ __forceinline__ void cast_vt_block(const VtOperand& o, unsigned block
     const int kmax = scale_key(max(top_s[r][0], top_s[r][1]));
     const int64_t row = row0 + r, sf_row = sf_row_offset(row, o.nk64);
     const uint16_t* sc = kept ? sc_s + r * G : o.scales + row * G;   // (written by this block)
-    int flushed = 0;
+    const float factor = sf_factor(kmax);
+    uint32_t lost = 0;
     for (int c = tid / kVtCols; c < o.nk64; c += 256 / kVtCols) {
-        uint32_t wp = 0, wn = 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int g = 2 * c + h;
-            const uint32_t v = in_use && g < G ? sc[g] : 0u;
-            const uint32_t up = to_ue4m3(v & 0xFFu, kmax), un = to_ue4m3(v >> 8, kmax);
-            flushed += (int)((v & 0xFFu) != 0 && up == 0) + (int)((v >> 8) != 0 && un == 0);
-            wp |= up * 0x0101u << (16 * h);
-            wn |= un * 0x0101u << (16 * h);
-        }
+        const int g = 2 * c;
+        const uint32_t u = to_ue4m3x2(in_use && g < G ? sc[g] : 0u, factor, lost) | to_ue4m3x2(in_use && g + 1 < G ? sc[g + 1] : 0u, factor, lost) << 16;
         const int64_t off = sf_row + (int64_t)c * kSfChunkBytes;
-        *reinterpret_cast<uint32_t*>(o.sf_pos + off) = wp;
-        *reinterpret_cast<uint32_t*>(o.sf_neg + off) = wn;
+        *reinterpret_cast<uint32_t*>(o.sf_pos + off) = __byte_perm(u, 0, 0x2200);
+        *reinterpret_cast<uint32_t*>(o.sf_neg + off) = __byte_perm(u, 0, 0x3311);
     }
     if (!in_use) return;                            // (nor are those rows' words read)
+    int flushed = (int)(lost >> 7);
 #pragma unroll
     for (int d = kVtCols; d < 32; d <<= 1) flushed += __shfl_xor_sync(0xFFFFFFFFu, flushed, d);
     if (lane < kVtCols && flushed) atomicAdd(&flushed_s[r], flushed);
@@ -434,14 +424,18 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, LPR = 1 << lpr_log2, lr = lane & (LPR - 1);
     const int RPW = 32 >> lpr_log2, sg = lane >> lpr_log2;      // rows per warp; which of them this lane works on
     // the block's rows: 128-row block rb, sector sets k0 .. k0 + RPW - 1 (16 / RPW blocks share a 128-row block)
-    const int64_t rb = (int64_t)block >> (lpr_log2 - 1);
+    const unsigned rb = block >> (lpr_log2 - 1);
     const int k0 = ((int)block & ((16 >> (5 - lpr_log2)) - 1)) << (5 - lpr_log2);
     const int r_in = 32 * (wi >> 1) + 2 * (k0 + sg) + (wi & 1);  // row inside the 128-row block
-    const int64_t row = rb * 128 + r_in;
-    // Segments (the heads of an attention call): seg_rows source rows each, padded to seg_pad operand rows.
-    const int64_t seg = o.seg_pad ? row / o.seg_pad : 0;
-    const bool live = row < o.R && (!o.seg_pad || row - seg * o.seg_pad < o.seg_rows);
-    const int64_t src_row = o.seg_pad ? seg * o.seg_rows + (row - seg * o.seg_pad) : row;
+    const int64_t row = (int64_t)rb * 128 + r_in;
+    // Segments (the heads of an attention call): seg_rows source rows each, padded to seg_blocks blocks of 128 operand rows.
+    int64_t src_row = row;
+    bool live = row < o.R;
+    if (MODE != kOneCast && MODE != kAnyGroup && o.seg_blocks) {
+        const unsigned seg = rb / o.seg_blocks, in_seg = (rb - seg * o.seg_blocks) * 128 + r_in;
+        live = live && in_seg < o.seg_rows;
+        src_row = seg * o.seg_rows + in_seg;
+    }
     const unsigned seg_mask = LPR == 32 ? 0xFFFFFFFFu : ((1u << LPR) - 1u) << (lane & ~(LPR - 1));
     const int64_t v_row = row * G;
     // this lane's ring: kCastDepth slots of 64 bytes (one piece).  Part j of a piece sits at 16-byte position
@@ -451,8 +445,9 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     const int swz = (lane >> 1) & 3;
     const int n_own = (live && lr < G) ? ((G - lr + LPR - 1) >> lpr_log2) : 0;   // pieces this lane owns
     const int n_max = (G + LPR - 1) >> lpr_log2;      // of any lane
-    uint16_t* const row_scales = o.scales + row * ((int64_t)G * 32 / gs);        // canonical scales: written by a cast, read otherwise
-    const uint16_t* const in_scales = !SPLIT || o.x ? row_scales : o.in_scales + row * ((int64_t)G * 32 / gs);
+    const int64_t scale_row = row * (ANY_GS ? G * 32 >> p.gs_log2 : G);
+    uint16_t* const row_scales = o.scales + scale_row;                           // canonical scales: written by a cast, read otherwise
+    const uint16_t* const in_scales = !SPLIT || o.x ? row_scales : o.in_scales + scale_row;
     auto issue = [&](int i) {                        // copies of the lane's i-th piece, one commit group per call
         if (i < n_own) {
             const uint4* src = o.x + src_row * o.ld_vec + (lr + ((int64_t)i << lpr_log2)) * 4;
@@ -561,20 +556,13 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     const int64_t sf_row = sf_row_offset(row, nk64);
     // word of the exchange buffer that holds this row's bytes of chunk c: ((c * RPW + sg) * 2 + h) * 4 + q
     const int x_row = (sg * 2 + (wi & 1)) * 4 + (wi >> 1), x_plane = nk64 * RPW * 8;   // in words
-    int flushed = 0;                                // groups, not pieces, are counted
+    const float factor = sf_factor(kmax);
+    uint32_t lost = 0;
     auto put = [&](int g, uint32_t sc) {            // scale factors of piece g (zero past the row's last one)
-        uint32_t up = to_ue4m3(sc & 0xFFu, kmax), un = to_ue4m3((sc >> 8) & 0xFFu, kmax);
-        const int lost = (int)((sc & 0xFFu) != 0 && up == 0) + (int)((sc & 0xFF00u) != 0 && un == 0);
-        if (gs <= 32 || (g & ((gs >> 5) - 1)) == 0) flushed += lost;
-        if (gs == 16) {                             // the second half has its own scales
-            const uint32_t sc1 = sc >> 16, up1 = to_ue4m3(sc1 & 0xFFu, kmax), un1 = to_ue4m3(sc1 >> 8, kmax);
-            flushed += (int)((sc1 & 0xFFu) != 0 && up1 == 0) + (int)((sc1 >> 8) != 0 && un1 == 0);
-            up |= up1 << 8;
-            un |= un1 << 8;
-        } else {
-            up |= up << 8;
-            un |= un << 8;
-        }
+        const uint32_t before = lost, u0 = to_ue4m3x2(sc, factor, lost);
+        if (ANY_GS && gs > 32 && (g & ((gs >> 5) - 1))) lost = before;   // groups, not pieces, are counted
+        const uint32_t u1 = ANY_GS && gs == 16 ? to_ue4m3x2(sc >> 16, factor, lost) : u0;   // the second half has its own scales
+        const uint32_t up = __byte_perm(u0, u1, 0x0040), un = __byte_perm(u0, u1, 0x0051);
         if (p.exchange) {
             uint16_t* w16 = reinterpret_cast<uint16_t*>(xchg) + (((g >> 1) * RPW * 8 + x_row) << 1) + (g & 1);
             w16[0] = (uint16_t)up;
@@ -599,7 +587,7 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
         if (ANY_GS) __syncwarp();                   // scales of larger groups were written by neighbouring lanes
         for (int g = lr; g < g_end; g += LPR) put(g, (live && g < G) ? piece_scales(in_scales, g, gs) & keep_sc : 0u);
     }
-    flushed = __reduce_add_sync(seg_mask, flushed);
+    const int flushed = __reduce_add_sync(seg_mask, (int)(lost >> 7));
     if (lr == 0 && live) {
         o.row_exp[row] = row_word(kmax, side_bits_of(top_p | (top_n << 8)), flushed);
         if (flushed && p.flushed_total) atomicAdd(p.flushed_total, flushed);
@@ -609,12 +597,12 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     __syncthreads();
     // 16 bytes per thread: the words of rows q = 0..3 (32 rows apart) for one (plane, chunk, sector set, h);
     // two neighbouring threads (h = 0, 1) fill one sector
-    const int per_plane = nk64 * RPW * 2;
+    const int per_plane = nk64 * RPW * 2, set_log2 = 6 - lpr_log2;   // RPW * 2 = 1 << set_log2
     for (int item = threadIdx.x; item < 2 * per_plane; item += kCastWarps * 32) {
         const int plane = item >= per_plane, rest = item - plane * per_plane;
-        const int c = rest / (RPW * 2), sh = rest - c * (RPW * 2);      // sh = sector set * 2 + h
+        const int c = rest >> set_log2, sh = rest & ((1 << set_log2) - 1);   // sh = sector set * 2 + h
         const uint4 v = reinterpret_cast<const uint4*>(xchg)[item];
-        uint8_t* dst = (plane ? o.sf_neg : o.sf_pos) + (rb * nk64 + c) * (int64_t)kSfChunkBytes + (2 * k0 + sh) * 16;
+        uint8_t* dst = (plane ? o.sf_neg : o.sf_pos) + ((int64_t)rb * nk64 + c) * kSfChunkBytes + (2 * k0 + sh) * 16;
         *reinterpret_cast<uint4*>(dst) = v;
     }
 }
@@ -741,6 +729,7 @@ int fill_prepare(PrepParams& p, const PrepOperand* op, int n, int64_t K, int gs,
     }
     p.nk64 = nk64;
     p.gs = gs;
+    p.gs_log2 = gs == 16 ? 4 : gs == 32 ? 5 : gs == 64 ? 6 : 7;
     p.flushed_total = flushed_total;
     const size_t exchange_bytes = (size_t)64 * rpw * nk64;           // both planes, 4 bytes per row and 64 elements
     p.exchange = exchange_bytes <= (size_t)kCastMaxExchangeBytes;
