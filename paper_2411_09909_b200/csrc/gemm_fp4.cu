@@ -588,10 +588,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             const int64_t m = m0 + q * 32 + lane;
             const float a_fac = cur.a_fac * out_scale;
             const uint64_t a_fac2 = cast::pack_f32x2(__float_as_uint(a_fac), __float_as_uint(a_fac));
+            // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join), and has done with the
+            // tile two before, whose factors were there
+            asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
             ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
             tc_fence_after();
-            // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join)
-            asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
             // 16 columns of the tile: scaled and stored
             auto put = [&](const uint32_t (&v)[16], int col) {
                 float f[16];
@@ -632,25 +633,27 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 auto chunk_col = [&](int i) {                    // first column (inside the tile) of this warp's chunk i
                     return i < kC1 ? o1 + h * (kOvl / 2) + 16 * i : o2 + h * ((BNT - kOvl) / 2) + 16 * (i - kC1);
                 };
-                uint32_t v[2][16];
-                if (kC1 == 0) {                                  // nothing shared: the next tile may start at once
+                // (All of them before anything is scaled or stored: the tensor cores wait for this.)
+                if (kC1 == 0) released(&ctl->ovl_free);          // nothing shared: the next tile may start at once
+                uint32_t first[kC1 ? kC1 : 1][16], v[2][16];
+                if (kC1) {
+#pragma unroll
+                    for (int i = 0; i < kC1; ++i) tmem_ld16(taddr + chunk_col(i), first[i]);
+                    tmem_ld_wait();
+                    tc_fence_before();
                     released(&ctl->ovl_free);
                 }
-                tmem_ld16(taddr + chunk_col(0), v[0]);
+                tmem_ld16(taddr + chunk_col(kC1), v[0]);
 #pragma unroll
-                for (int i = 0; i < kC1 + kC2; ++i) {
-                    const int buf = i & 1;
+                for (int i = 0; i < kC1; ++i) put(first[i], chunk_col(i));
+#pragma unroll
+                for (int i = 0; i < kC2; ++i) {
                     tmem_ld_wait();
-                    if (i + 1 == kC1) {                          // the shared columns are in registers
-                        tc_fence_before();
-                        released(&ctl->ovl_free);
-                    }
-                    if (i + 1 == kC1 + kC2) {                    // so is the rest: tile t + 2 may overwrite the window
+                    if (i + 1 == kC2) {                          // the rest is in registers: tile t + 2 may overwrite the window
                         tc_fence_before();
                         released(&ctl->rest_free[odd]);
-                    }
-                    if (i + 1 < kC1 + kC2) tmem_ld16(taddr + chunk_col(i + 1), v[buf ^ 1]);   // loads while this chunk is stored
-                    put(v[buf], chunk_col(i));
+                    } else tmem_ld16(taddr + chunk_col(kC1 + i + 1), v[(i & 1) ^ 1]);   // loads while this chunk is stored
+                    put(v[i & 1], chunk_col(kC1 + i));
                 }
             }
             ++t;
