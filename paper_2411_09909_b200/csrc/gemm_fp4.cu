@@ -17,17 +17,19 @@
 // Persistent CTAs (one per SM) walk over 128 x 256 tiles of C - pairs of CTAs over 256 x 256 tiles (PAIR below) -; the tiles
 // that would leave most of a last wave idle are cut into halves or quarters of their columns.  K blocks cycle through four
 // shared-memory stages (five in a pair):
-//   warp 0   TMA producer: per stage one 3-D tile {A+, A-} and one {W+, W-} (64-byte swizzle),
-//            completion on the stage's `full` mbarrier, and the scale factors of either on `sf_full`
-//   warp 1   allocates TMEM; one lane issues the stage's MMAs (4 sign pairs x K steps of 64), then
-//            commits to the stage's `empty` mbarrier
-//   warps 2-9  (two groups of four, alternating K blocks) move each stage's scale factors, which come with its tiles, shared
-//            -> registers -> tensor memory (tcgen05.st; this keeps the copies off the in-order MMA queue) and arrive on the
-//            stage's `full` barrier; they follow only barriers and so run ahead into the next tile
-//   warps 10-17 epilogue: TMEM -> registers (double-buffered loads), power-of-two rescale, 32-byte fp32
+//   warp 0   TMA producer: per stage one 3-D tile {A+, A-} and one {W+, W-} (swizzled rows) and the scale factors of either,
+//            completion on the stage's `full` mbarrier
+//   warp 1   allocates TMEM; one lane issues, per stage, the copies of the scale factors from shared to tensor memory
+//            (tcgen05.cp, in order with the MMAs, either right before the first MMA that reads it) and the MMAs (4 sign
+//            pairs x K steps of 64), then commits to the stage's `empty` mbarrier
+//   warps 2-9 epilogue: TMEM -> registers (double-buffered loads), power-of-two rescale, 32-byte fp32
 //            stores.  While a tile's accumulator is read out the producer already prefetches the next
 //            tile's stages, and the MMA issuer starts the next tile as soon as the columns the two tiles
 //            share have been read (see "Tensor memory" below).
+// What bounds the K loop is shared memory: per K block of a pair's CTA the copies write 38 KB and the MMAs read 32 (one plane) or 64
+// (two).  Eight more warps that carried the scale factors through registers read another 24 KB (each quarter of tensor
+// memory wants a copy): MXFP4 8192 x 14336 x 4096 249 us against 233, 1000 x 11008 x 4096 93.5 against 89.2, 16384 x 10240 x 8192
+// 1897 against 1871.  (All copies of a stage ahead of its MMAs: 90.0 for the second.)
 // A preparation kernel per operand derives the planes, the UE4M3 scale-factor
 // blocks in the 128 x 4 interleaved layout the MMA reads, and the row offsets from the canonical
 // codes and scales.  Every device-side wait is bounded.
@@ -49,8 +51,8 @@ using namespace tc;
 using namespace fp4;
 
 constexpr int BM = 128, BN = 256;
-constexpr int kSfGroups = 2, kSfWarps = 4 * kSfGroups, kEpilogueWarps = 8;
-constexpr int kThreads = (2 + kSfWarps + kEpilogueWarps) * 32;
+constexpr int kEpilogueWarps = 8;
+constexpr int kThreads = (2 + kEpilogueWarps) * 32;
 constexpr int kTmemCols = 512;
 // Tensor memory.  Two fp32 accumulators of 256 columns are all 512 columns, and the block-scaled MMA reads its
 // scale factors from tensor memory too.  So consecutive tiles of a CTA alternate between two accumulator windows
@@ -84,17 +86,17 @@ struct Cfg {
     static constexpr int kSmemBytes = kStages * (kStageBytes + kSfStage) + 1024 + 2048 + 512;   // + alignment slack + Control
     // TMEM columns of one stage's scale factors: A planes (4 columns per K step), then W planes (8)
     static constexpr int kSfColsA = kPlanes * kSteps * 4, kSfCols = kSfColsA + kPlanes * kSteps * 8;
-    // the scale factors of kSfSlots K blocks are in tensor memory at a time (fewer than shared-memory stages: the
-    // scale-factor warps store block i once the MMAs of block i - kSfSlots are done, while block i - 1 is multiplied)
+    // the scale factors of kSfSlots K blocks are in tensor memory at a time, so that a block's copies do not touch what the MMAs
+    // just ahead of them read
     static constexpr int kSfSlots = kTmemSfCols / kSfCols;
-    static_assert(kSfSlots >= 2 && kSfSlots % kSfGroups == 0 && kSfSlots <= kStages, "scale-factor ring");
+    static_assert(kSfSlots >= 2 && kSfSlots <= kStages, "scale-factor ring");
     static_assert(kAccWindow + BN <= (int)kTmemSf && kTmemSf + kSfSlots * kSfCols <= kTmemCols, "tensor memory map");
     static_assert(BK == 128 || BK == 256, "rows of 64 or 128 bytes, swizzled over their length");
 };
 constexpr int kMaxStages = 5;
 
 struct __align__(16) Control {
-    uint64_t full[kMaxStages], empty[kMaxStages], sf_full[kMaxStages], accum_full;
+    uint64_t full[kMaxStages], empty[kMaxStages], accum_full;
     uint64_t ovl_free;              // the columns a finished tile shares with the next tile's accumulator have been read
     uint64_t rest_free[2];          // its other columns have been read ([i]: tiles with number % 2 == i)
     uint64_t sides_ready[2];        // the epilogue warps have written sides[i] for the CTA's tile number 2 k + i
@@ -169,7 +171,7 @@ __device__ __forceinline__ void store_row16_bf16(__nv_bfloat16* out, const float
 // wide, the stage layout keeps its size.
 // PAIR: two CTAs (a cluster) compute a tile of 256 x 256, each the accumulator of 128 of its rows and the load of its A rows and
 // of half of the W rows; their tensor cores read both halves.  The first CTA's warp 1 issues for both: all copies of a stage are
-// counted on its `full` barrier, the other CTA's scale-factor and epilogue warps arrive on its barriers too, and its commits
+// counted on its `full` barrier, the other CTA's epilogue warps arrive on its barriers too, and its commits
 // arrive on the barriers of both.
 // ONE_PLANE: the caller states that neither operand has a second sign plane (Cfg above): only the first planes and
 // their scale factors are read, one product per K step.  A tile whose row words show a second plane after all puts
@@ -247,10 +249,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
-            // producer (with the TMA byte count) + four scale-factor warps; a pair's stages are all reported to its first CTA
-            mbar_init(&ctl->full[s], 1 + 4 * (PAIR ? 2 : 1));
+            mbar_init(&ctl->full[s], 1);                         // the byte count; a pair's stages are all reported to its first CTA
             mbar_init(&ctl->empty[s], 1);
-            mbar_init(&ctl->sf_full[s], 1);
         }
         mbar_init(&ctl->accum_full, 1);
         constexpr int kReaders = kEpilogueWarps * (PAIR ? 2 : 1);      // of an accumulator (PAIR: both CTAs' halves)
@@ -337,20 +337,19 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 }
                 if (elect_one()) {
                     uint8_t *st = tiles + s * kStageBytes, *sf = sf_stages + s * C_::kSfStage;
-                    // scale factors first: they have one more step to go.  One copy per operand: {K steps, row blocks, planes}
-                    const int xs = (kb0 + kb) * (C_::kSfRun / 8);
-                    mbar_expect_tx(&ctl->sf_full[s], kPlanes * (NHALF ? 2 : 3) * C_::kSfRun);
-                    tma_load_3d(sf, &tm_sfa, xs, ysa, 0, &ctl->sf_full[s]);
-                    tma_load_3d(sf + kPlanes * C_::kSfRun, &tm_sfw, xs, ysw, 0, &ctl->sf_full[s]);
-                    const int x = (kb0 + kb) * kRowBytes;
-                    const uint32_t bytes = (a_planes == 3 ? 2 : 1) * C_::kTileA + (w_planes == 3 ? 2 : 1) * tile_w;
+                    const int x = (kb0 + kb) * kRowBytes, xs = (kb0 + kb) * (C_::kSfRun / 8);
+                    const uint32_t bytes = (a_planes == 3 ? 2 : 1) * C_::kTileA + (w_planes == 3 ? 2 : 1) * tile_w + kPlanes * (NHALF ? 2 : 3) * C_::kSfRun;
                     if (!PAIR) mbar_expect_tx(&ctl->full[s], bytes);
                     else if (rank == 0) mbar_expect_tx(&ctl->full[s], 2 * bytes);   // (the other CTA's bytes may be counted first)
                     const uint32_t full = PAIR ? cluster_addr(&ctl->full[s], 0) : 0;
-                    auto load = [&](uint8_t* dst, const CUtensorMap* map, int y, int z) {
-                        if (PAIR) tma_load_3d_pair(dst, map, x, y, z, full);
-                        else tma_load_3d(dst, map, x, y, z, &ctl->full[s]);
+                    auto load_at = [&](uint8_t* dst, const CUtensorMap* map, int x0, int y, int z) {
+                        if (PAIR) tma_load_3d_pair(dst, map, x0, y, z, full);
+                        else tma_load_3d(dst, map, x0, y, z, &ctl->full[s]);
                     };
+                    auto load = [&](uint8_t* dst, const CUtensorMap* map, int y, int z) { load_at(dst, map, x, y, z); };
+                    // the scale factors of an operand: {K steps, row blocks, planes}
+                    load_at(sf, &tm_sfa, xs, ysa, 0);
+                    load_at(sf + kPlanes * C_::kSfRun, &tm_sfw, xs, ysw, 0);
                     // one 3-D tile per operand: {row bytes, rows, both sign planes} - or the one plane that is not zero
                     if (a_planes == 3) load(st + C_::kOffAp, &tm_a, ya, 0);
                     else load(st + (a_planes == 2 ? C_::kOffAn : C_::kOffAp), &tm_a1, ya, a_planes == 2 ? 1 : 0);
@@ -369,12 +368,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         // after an abort: let the copies already in flight land before shared memory is released
         if (ctl->abort && lane == 0)
-            for (int i = max(0, it - kStages); i < it; ++i) {
-                // (PAIR: the first CTA waits for both, the other one for the first at the end of the kernel)
-                if (rank == 0)
-                    for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
-                for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->sf_full[i % kStages], (i / kStages) & 1); ++n) {}
-            }
+            // (PAIR: the first CTA waits for both, the other one for the first at the end of the kernel)
+            for (int i = max(0, it - kStages); i < it && rank == 0; ++i)
+                for (uint32_t n = 0; n < kSpinLimit && !mbar_try_wait(&ctl->full[i % kStages], (i / kStages) & 1); ++n) {}
     } else if (PAIR && warp == 1 && rank == 1) {
         // the pair's MMAs are issued by its first CTA
     } else if (warp == 1) {
@@ -383,6 +379,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         // lane issues.  All operand descriptors differ from the first stage's only in their 14-bit address
         // field (bytes >> 4); the per-plane and per-K-step offsets are compile-time constants.
         const uint64_t desc0 = kRowBytes == 128 ? smem_desc_sw128(smem_u32(tiles)) : smem_desc_sw64(smem_u32(tiles));
+        const uint64_t desc_sf0 = smem_desc_rows16(smem_u32(sf_stages));
         int it = 0, t = 0;
         bool ok = true, ready = false;                           // ready: the next K block's barrier was seen complete
         // (the planes of a tile: tile_sides above; the words of the next tile are fetched while the current one runs)
@@ -411,8 +408,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 constexpr bool ALL = decltype(all)::value, PLAIN = decltype(plain)::value;
                 for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
                     const int s = it % kStages;
-                    // tiles landed (TMA byte count) and scale factors stored (four warp arrivals); usually already
-                    // seen by the poll that was slipped between the previous block's MMAs
+                    // the stage has landed; usually already seen by the poll that was slipped between the previous block's MMAs
                     if (!ready) ok = mbar_wait(&ctl->full[s], (it / kStages) & 1, &ctl->abort, p.status);
                     if (!ok) break;
                     tc_fence_after();
@@ -422,6 +418,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     const uint32_t parity_next = ((it + 1) / kStages) & 1;
                     uint32_t seen = 0;
                     if (elect_one()) {
+                        // the stage's scale factors, 32 rows x 16 bytes to four columns
+                        const uint64_t dsf = desc_sf0 + (uint64_t)((s * C_::kSfStage) >> 4);
+                        auto copy = [&](uint32_t col, int run, int kk) {
+                            if (PAIR) tmem_cp_32x128b_warpx4_pair(col, dsf + ((run * C_::kSfRun + kk * kSfChunk) >> 4));
+                            else tmem_cp_32x128b_warpx4(col, dsf + ((run * C_::kSfRun + kk * kSfChunk) >> 4));
+                        };
+                        const uint32_t sfw = sfa + C_::kSfColsA;
+                        auto copy_a = [&](int pl, int kk) { copy(sfa + (pl * kSteps + kk) * 4, pl, kk); };
+                        auto copy_w = [&](int pl, int kk) {
+                            copy(sfw + (pl * kSteps + kk) * 8, kPlanes + pl * (NHALF ? 1 : 2), kk);
+                            if (!NHALF) copy(sfw + (pl * kSteps + kk) * 8 + 4, kPlanes + pl * 2 + 1, kk);
+                        };
                         int idx = 0;                                 // MMAs issued so far in this K block
 #pragma unroll
                         for (int pa = 0; pa < kPlanes; ++pa)
@@ -429,6 +437,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                             for (int pw = 0; pw < kPlanes; ++pw)
 #pragma unroll
                                 for (int kk = 0; kk < kSteps; ++kk) {   // 64 elements = 32 bytes along the swizzled row
+                                    if (pw == 0) copy_a(pa, kk);
+                                    if (pa == 0) copy_w(pw, kk);
                                     if (ALL || (((sides >> pa) & 1) && ((sides >> (2 + pw)) & 1))) {
                                         const uint64_t da = dstage + (((pa ? C_::kOffAn : C_::kOffAp) + kk * 32) >> 4),
                                                        dw = dstage + (!pw ? (uint32_t)C_::kOffWp >> 4 : PLAIN ? kOffWnT >> 4 : w_minus) + (kk * 32 >> 4);
@@ -459,67 +469,15 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             __syncwarp();
             ++t;
         }
-    } else if (warp < 2 + kSfWarps) {
-        // -------------------------------------------------------------- scale factors
-        // Warp w serves the 32-lane quarter w % 4 of tensor memory: every quarter has to hold a copy of the scale-factor
-        // columns.  Per K block a lane reads 16 bytes of each 512-byte chunk of the stage (the 4-byte scale words of rows
-        // lane, lane+32, lane+64, lane+96) and stores them to its quarter with tcgen05.st.  Two groups of four warps take
-        // alternate K blocks.  The chunks come to shared memory with the stage's tiles, several K blocks ahead; fetched by
-        // these warps from global memory, one block ahead each, their latency bounded products of one plane per operand
-        // (MXFP4 8192 x 14336 x 4096: 375 -> 347 us).
-        const int q = warp & 3, group = (warp - 2) >> 2;
-        int it = 0;
-        bool ok = true;
-        for (int64_t tile = worker; tile < total_items && ok; tile += workers) {
-            const int end = it + nkb_of(tile);
-            // this group's K blocks (global count it % kSfGroups == group)
-            for (int i = it + ((group - it) & (kSfGroups - 1)); i < end; i += kSfGroups) {
-                const int s = i % kStages;
-                ok = mbar_wait(&ctl->sf_full[s], (i / kStages) & 1, &ctl->abort, p.status);
-                if (!ok) break;
-                const uint8_t* sf = sf_stages + s * C_::kSfStage + lane * 16;
-                uint4 v[kPlanes * kSteps * 3];
-#pragma unroll
-                for (int pl = 0; pl < kPlanes; ++pl)
-#pragma unroll
-                    for (int kk = 0; kk < kSteps; ++kk)
-#pragma unroll
-                        for (int x = 0; x < 3; ++x)
-                            v[(pl * kSteps + kk) * 3 + x] = *reinterpret_cast<const uint4*>(sf + (x ? kPlanes + pl * (NHALF ? 1 : 2) + (NHALF ? 0 : x - 1) : pl) * C_::kSfRun + kk * kSfChunk);
-                // the slot of the scale-factor ring is free once the MMAs of K block i - kSfSlots are done (the `empty`
-                // barrier of that block's stage; it cannot complete again before this block's factors are stored)
-                if (i >= C_::kSfSlots) {
-                    const int j = i - C_::kSfSlots;
-                    ok = mbar_wait(&ctl->empty[j % kStages], (j / kStages) & 1, &ctl->abort, p.status);
-                    if (!ok) break;
-                }
-                tc_fence_after();
-                const uint32_t sfa = tmem + ((uint32_t)(q * 32) << 16) + kTmemSf + (i % C_::kSfSlots) * C_::kSfCols, sfb = sfa + C_::kSfColsA;
-#pragma unroll
-                for (int c = 0; c < kPlanes * kSteps; ++c) {
-                    tmem_st4(sfa + c * 4, v[c * 3].x, v[c * 3].y, v[c * 3].z, v[c * 3].w);
-                    tmem_st4(sfb + c * 8, v[c * 3 + 1].x, v[c * 3 + 1].y, v[c * 3 + 1].z, v[c * 3 + 1].w);
-                    tmem_st4(sfb + c * 8 + 4, v[c * 3 + 2].x, v[c * 3 + 2].y, v[c * 3 + 2].z, v[c * 3 + 2].w);
-                }
-                tmem_st_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    if (PAIR) mbar_arrive_remote(&ctl->full[s], 0);
-                    else mbar_arrive(&ctl->full[s]);
-                }
-            }
-            it = end;
-        }
     } else {
         // -------------------------------------------------------------- epilogue
         // Eight warps: quarter q = warp % 4 of the lanes (= rows), one half of the columns each.
-        const int e = warp - (2 + kSfWarps);                     // 0..7
+        const int e = warp - 2;                     // 0..7
         const int q = warp & 3;
         constexpr int kOvl = BNT > kAccWindow ? BNT - kAccWindow : 0;        // columns two consecutive tiles share
         constexpr int kC1 = kOvl / 2 / 16, kC2 = (BNT - kOvl) / 2 / 16;       // this warp's chunks of either part
         static_assert(kOvl % 32 == 0 && (BNT - kOvl) % 32 == 0, "both parts split into two halves of 16-column chunks");
-        const int tid_e = threadIdx.x - (2 + kSfWarps) * 32;
+        const int tid_e = threadIdx.x - 64;
         int t = 0;
         bool ok = true;
         static_assert(kEpilogueWarps * 32 == BN, "one column offset per epilogue thread");   // BNT <= BN
