@@ -258,6 +258,9 @@ struct PrepParams {
     int* flushed_total;
 };
 
+// The two scale bytes {neg : pos} as 16-bit halves, for packed maxima (byte-wise ones are eight instructions).
+__device__ __forceinline__ uint32_t halves(uint32_t sc) { return __byte_perm(sc, 0, 0x4140); }
+
 // Scale pairs {neg : pos} of one 32-element piece: of its first 16 elements in bits 15..0, of the others in bits 31..16
 // (equal unless the group size is 16), from a row's canonical scales.
 __device__ __forceinline__ uint32_t piece_scales(const uint16_t* __restrict__ row, int g, int gs) {
@@ -361,20 +364,20 @@ __device__ __forceinline__ void cast_vt_block(const VtOperand& o, unsigned block
                 sc_s[2 * cw * G + g0 + g] = (uint16_t)s0;
                 sc_s[(2 * cw + 1) * G + g0 + g] = (uint16_t)s1;
             }
-            top[0] = __vmaxu4(top[0], s0);
-            top[1] = __vmaxu4(top[1], s1);
+            top[0] = __vmaxu2(top[0], halves(s0));
+            top[1] = __vmaxu2(top[1], halves(s1));
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int d = 4; d < 32; d <<= 1) top[j] = __vmaxu4(top[j], __shfl_xor_sync(0xFFFFFFFFu, top[j], d));
+            for (int d = 4; d < 32; d <<= 1) top[j] = __vmaxu2(top[j], __shfl_xor_sync(0xFFFFFFFFu, top[j], d));
     }
     __syncthreads();
     if (lane < 4)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            atomicMax(&top_s[2 * lane + j][0], (int)(top[j] & 0xFFu));
-            atomicMax(&top_s[2 * lane + j][1], (int)(top[j] >> 8));
+            atomicMax(&top_s[2 * lane + j][0], (int)(top[j] & 0xFFFFu));
+            atomicMax(&top_s[2 * lane + j][1], (int)(top[j] >> 16));
         }
     __syncthreads();
     const int r = tid & (kVtCols - 1);              // of all of this thread's items
@@ -404,10 +407,12 @@ __device__ __forceinline__ void cast_vt_block(const VtOperand& o, unsigned block
 
 // MODE: one cast, two casts, operands that may be canonical, any of these with a group size other than 32, or the three casts
 // of an attention call.  (The plain cast is kept lean - its pointers are compile-time places in constant memory: it is bound by
-// instruction issue, and four blocks have to share an SM.)
+// instruction issue, and four blocks have to share an SM.  Five fit where little work per block leaves latency to hide, in the
+// attention's casts: 54.3 -> 53.4 us for 32 over 8 heads x 1056 causal; elsewhere they are no faster, and the canonical operand's
+// batch of loads spills: 1000 x 11008 x 4096 89.5 -> 94.7.)
 enum PrepMode { kOneCast, kTwoCasts, kAnyKind, kAnyGroup, kAttention };
 template <int FMT, int GPL, int MODE>
-__global__ void __launch_bounds__(kCastWarps * 32, 4)
+__global__ void __launch_bounds__(kCastWarps * 32, MODE == kAttention ? 5 : 4)
 prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     begin_kernel();
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -474,7 +479,11 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
         return sc | (sc << 16);
     };
     uint32_t sc_reg[GPL > 0 ? GPL : 1];
-    uint32_t top = 0;                               // largest scale bytes seen by this lane, {neg : pos} twice
+    uint32_t top = 0;                               // largest scale bytes seen by this lane, {neg : pos} as halves
+    auto see = [&](uint32_t sc) {
+        top = __vmaxu2(top, halves(sc));
+        if (ANY_GS && gs == 16) top = __vmaxu2(top, halves(sc >> 16));
+    };
     if (!SPLIT || o.x) {
 #pragma unroll
         for (int i = 0; i < kCastDepth - 1; ++i) issue(i);
@@ -484,13 +493,13 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
                 issue(i + kCastDepth - 1);
                 cp_async_wait<kCastDepth - 1>();
                 sc_reg[i] = cast_piece(i);
-                top = __vmaxu4(top, sc_reg[i]);     // byte-wise maximum
+                see(sc_reg[i]);
             }
         } else {
             for (int i = 0; i < n_max; ++i) {
                 issue(i + kCastDepth - 1);
                 cp_async_wait<kCastDepth - 1>();
-                top = __vmaxu4(top, cast_piece(i));
+                see(cast_piece(i));
             }
         }
         cp_async_wait<0>();
@@ -510,21 +519,21 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
 #pragma unroll
             for (int i = 0; i < GPL; ++i) {
                 sc_reg[i] = i < n_own ? piece_scales(in_scales, lr + (i << lpr_log2), gs) : 0u;
-                top = __vmaxu4(top, sc_reg[i]);
-                differ |= (sc_reg[i] ^ (sc_reg[i] >> 8)) & 0x00FF00FFu;
+                see(sc_reg[i]);
+                differ |= sc_reg[i] ^ __byte_perm(sc_reg[i], 0, 0x2301);
             }
         } else {
             for (int i = 0; i < n_own; ++i) {
                 const uint32_t sc = piece_scales(in_scales, lr + (i << lpr_log2), gs);
-                top = __vmaxu4(top, sc);
-                differ |= (sc ^ (sc >> 8)) & 0x00FF00FFu;
+                see(sc);
+                differ |= sc ^ __byte_perm(sc, 0, 0x2301);
             }
         }
         // A row whose two scales agree in every group (a symmetric format) needs no split: sum over both signs of
         // code x scale_side = code x scale.  Its signed codes go to the positive plane as they are.
         const bool unsplit = __reduce_or_sync(seg_mask, differ) == 0;
         const uint32_t keep_sc = unsplit ? 0x00FF00FFu : 0xFFFFFFFFu, keep = unsplit ? 0u : 0xFFFFFFFFu;
-        top &= keep_sc;
+        if (unsplit) top &= 0xFFFFu;
         if (GPL > 0) {
 #pragma unroll
             for (int i = 0; i < GPL; ++i) sc_reg[i] &= keep_sc;
@@ -550,8 +559,7 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
         if (GPL == 0) sc_reg[0] = keep_sc;          // for the second sweep
     }
     // The key of an E5M2 byte grows with the byte (scales carry no sign bit): the largest byte has the largest key.
-    top = __vmaxu4(top, top >> 16);
-    const uint32_t top_p = __reduce_max_sync(seg_mask, top & 0xFFu), top_n = __reduce_max_sync(seg_mask, (top >> 8) & 0xFFu);
+    const uint32_t top_p = __reduce_max_sync(seg_mask, top & 0xFFFFu), top_n = __reduce_max_sync(seg_mask, top >> 16);
     const int kmax = scale_key(max(top_p, top_n));
     const int64_t sf_row = sf_row_offset(row, nk64);
     // word of the exchange buffer that holds this row's bytes of chunk c: ((c * RPW + sg) * 2 + h) * 4 + q
