@@ -54,3 +54,21 @@ def test_prepared_form_of_every_scale(rows, K):
     whole = ~np.any((s > 0) & (exp.max(1, keepdims=True) - exp >= 15), 1)
     err = np.linalg.norm(got - ref, axis=1)[whole] / np.linalg.norm(ref, axis=1)[whole]
     assert np.all(err <= 1e-5)                                       # up to 1280 fp32 additions: at random signs some 36 x 2^-23
+
+
+@pytest.mark.parametrize("gs", [16, 32])
+def test_error_of_every_scale(gs):
+    """Group by group, so that no large scale hides a small one: decoded values down to the smallest subnormals of the format the
+    kernel multiplies in, elements off their codes, clamped ones wherever the scale was rounded down."""
+    for factor in (1.06, 1.11):
+        bits = inputs.f32_to_bf16_bits((factor * groups()).astype(np.float32))
+        codes, scales = oracle.quantize(bits, gs)
+        clamped = 0
+        for i in range(len(bits)):
+            one = [np.ascontiguousarray(t[i:i + 1]) for t in (bits, codes, scales)]
+            dev = torch.from_numpy(one[0].view(np.int16)).cuda().view(torch.bfloat16)
+            got = amx.quant_error(dev, torch.from_numpy(one[1]).cuda(), torch.from_numpy(one[2]).cuda(), gs).cpu().numpy()
+            ref = oracle.quant_error(*one, gs)
+            assert got[3] == ref[3] and np.allclose(got[:3], ref[:3], rtol=2.0 ** -20, atol=0), (i, got, ref)
+            clamped += ref[3]
+        assert clamped > 0 and 0 < ref[1] < ref[0]
