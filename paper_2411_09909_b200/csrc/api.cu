@@ -18,8 +18,9 @@ bool gemm_shape_ok(int64_t M, int64_t N, int64_t K, int gs) {
 constexpr uint32_t kKernelMask = AMX_GEMM_SIMT | AMX_GEMM_TC | AMX_GEMM_FP4 | AMX_GEMM_ROWS;
 
 // Time of the FP4 route under AUTO for 65 to 256 rows, us: preparation of the whole weight, one or two waves of tiles, the result,
-// and the gated exact kernel behind it, whose reduction (groups of 32, K from 1024, less than a wave of tiles) is a launch of
-// M N / 256 blocks even when it has nothing to do.  Fitted to 320 calls of 31 weights, within 20 % from 2^21 weight elements on.
+// and the gated exact kernel behind it, whose reduction (groups of 32, K from 1024, less than a wave of tiles) was a launch of
+// M N / 256 blocks even when it had nothing to do.  Fitted to 320 calls of 31 weights, within 20 % from 2^21 weight elements on,
+// before that launch became one wave and the FP4 kernel faster (12288 x 4096 at 128 rows 45 -> 40 us, 4096 x 4096 at 256 43 -> 32).
 // Taken at M = 128: with the streaming kernel's time growing with the rows, the choice then changes once as rows are added.
 double fp4_route_us(int64_t N, int64_t K, int gs) {
     const double mn = 128.0 * (double)N;
