@@ -695,10 +695,11 @@ int launch_fp4(const uint8_t* pa, const uint8_t* pw, const OperandLayout& oa, co
         return AMX_ERR_CUDA;
     if (PAIR) p.band = (p.band + 1) / 2;
     const unsigned grid = (unsigned)workers * kCtas;
-    // Chained up to 4.4e11 issued products (about 170 us).  Cast and product of 2048 x 12288 x 4096: ordinary 173 us, chained 153 to
-    // 161; 4096 x 11008 x 4096 265 / 274.  One plane, 8192 x 6144 x 4096: 136 / 132, 8192 x 14336 x 4096 269 / 267.
+    // Chained up to 8e11 issued products, 5.5e11 of one plane (260 and 200 us with the cast).  Cast and product, ordinary / chained:
+    // 4096 x 11008 x 4096 265.5 / 258.5, MXFP4 8192 x 14336 x 4096 200.3 / 197.1, 9000 x 4096 x 14336 263.6 / 259; from there on no
+    // difference beyond the runs' own (MXFP4 12000 x 12288 x 4096 316 / 319, 16384 x 14336 x 4096 416 / 415).
     const double products = (double)p.M * (double)p.N * (double)p.K * (ONE_PLANE ? 1.0 : 4.0);
-    return launch_clusters(kCtas, products <= 4.4e11, gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w,
+    return launch_clusters(kCtas, products <= (ONE_PLANE ? 5.5e11 : 8e11), gemm_fp4_kernel<BK_, SLICED, NHALF, ONE_PLANE, PAIR>, grid, kThreads, C_::kSmemBytes, st, tm_a, tm_w,
                            tm_a1, tm_w1, tm_wt, tm_wt1, tm_sfa, tm_sfw, p);
 }
 
