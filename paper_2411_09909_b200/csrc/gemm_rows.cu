@@ -49,6 +49,7 @@
 #include "cp_async.cuh"
 #include "decode_math.cuh"
 #include "gemm.cuh"
+#include "scale_words.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -149,9 +150,9 @@ struct Ring {
     static constexpr int kPart = NT * kTok * kPartPitch * 4;
     static_assert(kPart <= kBytes, "the partial-product tile reuses the rings");
 };
-// Scales of one weight row over `n` steps: 4-byte words copied (groups of 128: two bytes per step, copied as the aligned
-// words around them), and the pitch of the rows in shared memory - twice an odd number of words, so that the words of
-// eight rows that a warp reads together lie in different banks (groups of 16: four words per step, four times an odd number).
+// Scales of one weight row over `n` steps: the most 4-byte words copied (groups of 128: two bytes per step, copied as the aligned
+// words around them, scale_words.cuh), and the pitch of the rows in shared memory - twice an odd number of words, so that the words
+// of eight rows that a warp reads together lie in different banks (groups of 16: four words per step, four times an odd number).
 __host__ __device__ constexpr int scale_words(int n, int gs) { return gs == 128 ? n / 2 + 1 : n * (64 / gs); }
 __host__ __device__ constexpr int scale_pitch(int n, int gs) {
     return gs == 16 ? (n | 1) * 4 : gs == 32 ? (n | 1) * 2 : gs == 64 ? (n | 1) : (n / 2 + 1) | 1;
@@ -206,9 +207,12 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
             const int r_in = i / words, w = i - r_in * words;
             int64_t r = row0 + r_in;
             r = r < p.N ? r : p.N - 1;
-            const uint8_t* src = p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2;
-            if (GS == 128) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
-            cp_async4(scale_s + r_in * pitch + w, src + w * 4);
+            if (GS == 128) {
+                const int64_t pair = r * steps + s_begin + first, word = (pair >> 1) + w;
+                if (w < pair_words(pair, n)) cp_async4(scale_s + r_in * pitch + w, p.w_scales + word * 4, pair_word_bytes(word, p.N * steps));
+            } else {
+                cp_async4(scale_s + r_in * pitch + w, p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2 + w * 4);
+            }
         }
     };
     auto issue_frags = [&](int i) {            // the four warps of a step parity share the copies
@@ -414,12 +418,15 @@ __global__ void __launch_bounds__(kThreads, stream_ctas(NT, MB)) gemm_rows_strea
             return;
         }
         // words past the warp's last step may lie past the end of the tensor
-        const int words = min(R::kWords, GS == 128 ? (min(n - first, kScaleSlotSteps)) / 2 + 1 : (n - first) * (64 / GS));
+        const int held = min(n - first, kScaleSlotSteps);
         for (int item = lane; item < rows_left * R::kWords; item += 32) {
             const int r = item / R::kWords, w = item - r * R::kWords;
-            const uint8_t* src = src0 + r * scale_pitch;
-            if (GS == 128) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(src) & ~uintptr_t(3));
-            if (w < words) cp_async4(dst + R::at(r, w), src + w * 4);
+            if (GS == 128) {
+                const int64_t pair = (row0 + r) * steps + s_begin + first, word = (pair >> 1) + w;
+                if (w < pair_words(pair, held)) cp_async4(dst + R::at(r, w), p.w_scales + word * 4, pair_word_bytes(word, p.N * steps));
+            } else if (w < held * (64 / GS)) {
+                cp_async4(dst + R::at(r, w), src0 + r * scale_pitch + w * 4);
+            }
         }
     };
     issue(0);
