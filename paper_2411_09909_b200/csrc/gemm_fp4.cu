@@ -534,7 +534,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         int64_t tile = worker;
         TileConsts nxt = load_consts(tile);
         publish(nxt, tile, 0);
-        while (tile < total_items && ok) {
+        // (After a timeout the loop runs out without work: one warp may have seen the barrier complete where another saw the abort flag,
+        // and every tile's named barrier wants all eight.)
+        while (tile < total_items) {
             const TileConsts cur = nxt;
             const int64_t tile_after = tile + workers;
             nxt = load_consts(tile_after);                       // in flight while this tile is worked on
@@ -549,7 +551,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join), and has done with the
             // tile two before, whose factors were there
             asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
-            ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
+            if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status)) != 0;
             tc_fence_after();
             // 16 columns of the tile: scaled and stored
             auto put = [&](const uint32_t (&v)[16], int col) {
