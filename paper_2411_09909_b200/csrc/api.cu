@@ -17,16 +17,24 @@ bool gemm_shape_ok(int64_t M, int64_t N, int64_t K, int gs) {
 
 constexpr uint32_t kKernelMask = AMX_GEMM_SIMT | AMX_GEMM_TC | AMX_GEMM_FP4 | AMX_GEMM_ROWS;
 
-// Time of the FP4 route under AUTO for 65 to 256 rows, us: preparation of the whole weight, one or two waves of tiles, the result,
-// and the gated exact kernel behind it, whose reduction (groups of 32, K from 1024, less than a wave of tiles) was a launch of
-// M N / 256 blocks even when it had nothing to do.  Fitted to 320 calls of 31 weights, within 20 % from 2^21 weight elements on,
-// before that launch became one wave and the FP4 kernel faster (12288 x 4096 at 128 rows 45 -> 40 us, 4096 x 4096 at 256 43 -> 32).
-// Taken at M = 128: with the streaming kernel's time growing with the rows, the choice then changes once as rows are added.
-double fp4_route_us(int64_t N, int64_t K, int gs) {
-    const double mn = 128.0 * (double)N;
-    const bool second_wave = (N + 255) / 256 > 148;
-    return 12.5 + 5.6e-3 * (double)K + 3.2e-7 * (double)N * (double)K + 1.4e-6 * mn + (second_wave ? 4.7 : 0.0) +
-           (gs == 32 && K >= 1024 && !second_wave ? 2.7e-6 * mn : 0.0);
+// Time of the FP4 route under AUTO for 65 to 256 rows, us: the launches (cast, preparation, product, gated exact kernel), the K loop of
+// the tiles' waves - a last wave of few tiles in parts, which take 0.68 and 0.79 of a whole tile's time -, preparation and reading of
+// the weight, dearer where its planes no longer fit the L2, and the result.  Whole blocks of 128 rows.  Fitted to 204 calls of
+// 34 weights (N 512 to 28672, K 512 to 28672, from HBM), rms error 5 %.
+double fp4_route_us(int64_t M, int64_t N, int64_t K) {
+    const int64_t m_blocks = (M + 127) / 128, tiles = m_blocks * ((N + 255) / 256), last = tiles % 148;
+    const double waves = (double)(tiles / 148) + (last == 0 ? 0.0 : last * 4 <= 148 ? 0.68 : last * 2 <= 148 ? 0.79 : 1.0);
+    const double nk = (double)N * (double)K;
+    return 9.8 + 0.66 * (double)((K + 127) / 128) * waves + 2.5e-7 * (nk + (nk > 1e8 ? nk - 1e8 : 0.0)) + 0.9e-6 * 128.0 * (double)m_blocks * (double)N;
+}
+
+// Whether the streaming kernel is the faster one between 65 and 256 rows.  Its time grows with the rows, that of the FP4 route only
+// from 128 to 129: taking the answer for 128 rows along, the choice changes at most once as rows are added.  (Groups of 16: an
+// eighth more decoding.)
+bool rows_pay(int64_t M, int64_t N, int64_t K, int gs) {
+    const double more = gs == 16 ? 1.12 : 1.0;
+    return more * gemm_rows_estimated_us(M, N, K) <= fp4_route_us(M, N, K) &&
+           (M <= 128 || more * gemm_rows_estimated_us(128, N, K) <= fp4_route_us(128, N, K));
 }
 
 // The kernel to run (one AMX_GEMM_* bit), or 0 when the flags cannot be honoured for this shape.
@@ -47,14 +55,15 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // FP4 kernel would have to prepare the whole weight for them; the bf16-decode kernel slices K over CTAs.
     // At most 64 token rows: the weight-streaming kernel reads the canonical weight once.  Up to 256 rows, in blocks of 64
     // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route
-    // (fp4_route_us).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 23 / 41 and at 256 36 / 43, 12288 x 4096 at
-    // 96 rows 52 / 51 and at 128 58 / 54, 4096 x 11008 at 192 rows 72 / 86, 28672 x 4096 at 72 rows 106 / 82, 14336 x 512 at
-    // 128 rows 17 / 20 and at 200 28 / 20.
+    // (rows_pay).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 24 / 29, at 160 31 / 30 and at 256 36 / 30, 12288 x 4096
+    // at 72 rows 52 / 39 and at 128 59 / 40, 8192 x 4096 at 96 rows 31 / 33 and at 128 36 / 33, 4096 x 11008 at 128 rows 50 / 62 and at
+    // 160 73 / 63, 14336 x 512 at 96 rows 14.5 / 14.6 and at 192 22 / 19.  Over the fit's calls and 243 of other weights and rows the choice
+    // costs 0.1 % on average, 7 and 9 % at most.
     // A narrow weight (below 512 rows and 2^23 elements) stays on the FP4 route from 2^28 multiply-adds on, slower as it is
-    // (256 x 8192 at 128 rows: 14 / 70): callers read the count of flushed scales that this route leaves in the workspace.
+    // (256 x 8192 at 128 rows: 12 / 43): callers read the count of flushed scales that this route leaves in the workspace.
     const double mnk = (double)M * (double)N * (double)K;
     const bool narrow = N < 512 && N * K < (1ll << 23) && mnk >= 268435456.0;
-    if (rows && K >= 512 && (M <= 64 || (!narrow && gemm_rows_estimated_us(M, N, K) <= fp4_route_us(N, K, gs)))) return AMX_GEMM_ROWS;
+    if (rows && K >= 512 && (M <= 64 || (!narrow && rows_pay(M, N, K, gs)))) return AMX_GEMM_ROWS;
     const int64_t tiles = ((M + 127) / 128) * ((N + 255) / 256);
     if (tc && M <= 64 && tiles < 148 && K >= 1024) return AMX_GEMM_TC;      // K not a multiple of 128
     // (any fixed group size: the preparation turns the scales into the MMA's one per 16 elements)

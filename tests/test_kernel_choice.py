@@ -5,14 +5,17 @@ import pytest
 from paper_2411_09909_b200 import amx
 
 MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
-    (72, 28672, 4096, 105.9, 81.8), (128, 28672, 4096, 129.0, 90.2), (256, 28672, 4096, 223.6, 97.4),
-    (128, 12288, 4096, 58.0, 54.3), (256, 12288, 4096, 98.2, 63.5), (256, 6144, 4096, 57.6, 46.0), (160, 8192, 4096, 59.1, 48.2),
-    (72, 6144, 4096, 26.2, 40.0), (128, 8192, 4096, 35.8, 47.7), (192, 6144, 4096, 36.1, 45.3), (256, 4096, 4096, 36.2, 43.4),
-    (128, 4096, 4096, 23.5, 41.4), (128, 4096, 11008, 50.0, 85.1), (72, 4096, 14336, 62.2, 103.2), (128, 4096, 14336, 62.3, 107.8),
-    (256, 1024, 4096, 15.4, 38.0), (256, 2048, 2048, 15.6, 27.9), (192, 256, 4096, 11.0, 40.7), (72, 12288, 640, 11.9, 21.3),
-    (256, 12288, 640, 27.8, 22.8), (200, 14336, 512, 28.2, 20.0), (128, 8192, 640, 10.7, 20.6), (256, 28672, 1024, 78.2, 42.0),
-    (96, 5120, 2560, 18.5, 31.1), (256, 4096, 512, 9.9, 17.5),
-    (128, 1024, 1024, 6.3, 22.7)]
+    (72, 28672, 4096, 106.0, 70.3), (128, 28672, 4096, 129.2, 72.1), (256, 28672, 4096, 224.3, 88.2),
+    (128, 12288, 4096, 58.1, 41.3), (256, 12288, 4096, 98.7, 49.1), (256, 6144, 4096, 57.7, 32.9),
+    (160, 8192, 4096, 56.9, 35.8), (72, 6144, 4096, 27.2, 29.3), (128, 8192, 4096, 36.2, 33.0), (192, 6144, 4096, 36.3, 32.7),
+    (256, 4096, 4096, 36.3, 29.8), (128, 4096, 4096, 23.7, 29.1), (128, 4096, 11008, 50.2, 62.9),
+    (72, 4096, 14336, 52.3, 79.3), (128, 4096, 14336, 62.8, 81.1), (256, 1024, 4096, 15.1, 26.9),
+    (256, 2048, 2048, 16.0, 19.0), (192, 256, 4096, 8.5, 28.6), (72, 12288, 640, 11.6, 16.1), (256, 12288, 640, 27.9, 20.5),
+    (200, 14336, 512, 23.5, 18.4), (128, 8192, 640, 10.8, 14.2), (256, 28672, 1024, 78.6, 37.7), (96, 5120, 2560, 18.7, 22.8),
+    (256, 4096, 512, 9.7, 14.0), (128, 1024, 1024, 7.6, 16.4), (96, 12288, 4096, 52.1, 40.1), (80, 14336, 4096, 56.4, 43.1),
+    (160, 4096, 11008, 72.8, 63.4), (144, 5120, 2560, 21.1, 25.6),
+    (192, 16384, 2048, 57.0, 35.4), (128, 16384, 2048, 39.3, 29.8), (72, 18944, 3584, 52.3, 45.8),
+    (144, 9216, 3072, 46.8, 31.1), (256, 2304, 9216, 44.2, 50.3)]
 
 
 @pytest.mark.parametrize("M,N,K,rows_us,fp4_us", MEASURED)
