@@ -749,18 +749,22 @@ int gemm_fp4_slices(int64_t M, int64_t N, int64_t K) {
     if (s > 8) s = 8;
     return s < 2 ? 1 : s;
 }
-// K ranges or parts of tiles (launch_fp4) for a call of so few tiles, by estimates in us: a K block of a whole tile, a half or a
-// quarter takes 0.57, 0.45 or 0.39; ranges pay for the launch that adds them and for writing and reading the partial products.
-// Two planes, ranges / parts measured: 96 x 4096 x 14336 22.9 / 47.9, 250 x 4096 x 14336 35 / 48, 368 x 4096 x 11008 37 / 42,
-// 500 x 4096 x 11008 46 / 42, 368 x 4096 x 4096 26 / 19, 96 x 2560 x 2560 15 / 12.  One plane (a K block 0.16 to 0.13): parts
-// always, 500 x 4096 x 4096 26 / 9.7, 96 x 4096 x 14336 18.7 / 18.5.
+// K ranges or parts of tiles (launch_fp4) for a call of so few tiles, by estimates in us: the launches and a K block of a range's
+// tile, the partial products written and read, against the launches and a K block of a half or a quarter.  Fitted to 222 products
+// of M 64 to 500, N 512 to 14336, K 2048 to 28672.  Ranges / parts of two planes: 128 x 4096 x 14336 30 / 52, 256 x 4096 x 14336 40 / 52,
+// 500 x 4096 x 11008 54 / 46, 256 x 4096 x 4096 27 / 19; of one: 128 x 512 x 14336 17 / 22, 128 x 1024 x 28672 23 / 44,
+// 128 x 8192 x 28672 53 / 47, 500 x 4096 x 4096 34 / 13.  (Tiles of 128 columns have no parts and take a quarter's time; both
+// planes' figures, which a product of one plane is 3 to 20 % below.)  The choice costs 0.2 % on average.
 namespace {
-bool slices_pay(int64_t M, int64_t N, int64_t K, int slices, int sms, bool one_plane) {
-    if (slices < 2 || one_plane) return false;
-    const double blocks = (double)((K + 127) / 128);
-    static constexpr double kBlock[3] = {0.57, 0.45, 0.39};
-    const double parts = blocks * kBlock[parts_log2(((N + BN - 1) / BN) * ((M + BM - 1) / BM), sms)];
-    return blocks / slices * kBlock[0] + 4.0 + 0.6e-6 * 4.0 * slices * (double)M * (double)N < parts;
+bool slices_pay(int64_t M, int64_t N, int64_t K, int slices, int sms, bool one_plane, bool half) {
+    if (slices < 2) return false;
+    struct Fit { double ranges, block, parts, of_half, of_quarter; };
+    static constexpr Fit kFit[2] = {{8.0, 0.73, 5.4, 0.50, 0.41}, {8.4, 0.48, 5.2, 0.224, 0.166}};
+    const Fit& f = kFit[one_plane && !half];
+    const int64_t blocks = (K + 127) / 128;
+    const bool quarters = half || parts_log2(((N + BN - 1) / BN) * ((M + BM - 1) / BM), sms) == 2;
+    return f.ranges + f.block * (double)((blocks + slices - 1) / slices) + 3.0e-6 * slices * (double)M * (double)N <
+           f.parts + (quarters ? f.of_quarter : f.of_half) * (double)blocks;
 }
 }  // namespace
 size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K) {
@@ -792,7 +796,7 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
     const int slices = gemm_fp4_slices(M, N, K);
     // at most 128 columns: tiles of 128 x 128, so that no half of a W tile is padding
     const bool half = N <= BN / 2 && !getenv("AMX_FP4_NO_HALF_TILE");
-    if (!gate && !scale_a && !out_bf16 && slices_pay(M, N, K, slices, sm_count(dev), one_plane && !half) &&
+    if (!gate && !scale_a && !out_bf16 && slices_pay(M, N, K, slices, sm_count(dev), one_plane, half) &&
         workspace_bytes >= gemm_fp4_prepared_workspace_bytes(M, N, K)) {
         float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
         p.C = part;

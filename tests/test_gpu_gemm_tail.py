@@ -40,3 +40,25 @@ def test_parts_of_tiles(M, N, fmt, out):
     got = amx.gemm_prepared(a, b, M, N, K, out=wide[:, :N], sym=fmt != amx.FMT_AMXFP4, out_dtype=out)
     assert torch.all(wide[:, N:] == -3.0)
     assert float((got.double() - ref).norm() / ref.norm()) <= (2.0 ** -12 if out is torch.float32 else 2.0 ** -8)
+
+
+@pytest.mark.parametrize("M,N,K,ranges", [(128, 512, 14336, True), (100, 1000, 28672, True), (64, 300, 8192, True), (300, 520, 11008, True),
+                                          (128, 8192, 14336, False), (500, 4096, 4096, False), (128, 512, 4096, False)])
+def test_ranges_of_one_plane(M, N, K, ranges):
+    """Products promised to be of one plane: long and narrow ones are cut into K ranges on the general kernel, where the promise changes
+    nothing; the others, and all of them without scratch for ranges, check it."""
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    x = (torch.randn(M, K, device="cuda", generator=g) + 0.3).to(torch.bfloat16)
+    w = (0.02 * torch.randn(N, K, device="cuda", generator=g)).to(torch.bfloat16)
+    for fmt in (amx.FMT_MXFP4, amx.FMT_AMXFP4):
+        ac, as_, a = amx.quantize_prepared(x, False, fmt=fmt)
+        wc, ws, b = amx.quantize_prepared(w, True, fmt=fmt)
+        ref = amx.dequantize(ac, as_, 32, torch.float32).double() @ amx.dequantize(wc, ws, 32, torch.float32).double().T
+        for nbytes in (amx.lib().amx_gemm_prepared_workspace_bytes(M, N, K, 32), 256):
+            work = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+            got = amx.gemm_prepared(a, b, M, N, K, workspace=work, sym=True)
+            if fmt == amx.FMT_MXFP4 or (ranges and nbytes > 256):
+                assert amx.gemm_status(work) == 0
+                assert float((got.double() - ref).norm() / ref.norm()) <= 2.0 ** -12
+            else:
+                assert amx.gemm_status(work) == -5
