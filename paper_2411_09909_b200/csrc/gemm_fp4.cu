@@ -551,7 +551,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join), and has done with the
             // tile two before, whose factors were there
             asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
-            if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status)) != 0;
+            if (ok) ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
             tc_fence_after();
             // 16 columns of the tile: scaled and stored
             auto put = [&](const uint32_t (&v)[16], int col) {
