@@ -86,8 +86,13 @@ struct Cfg {
     static constexpr int kSmemBytes = kStages * (kStageBytes + kSfStage) + 1024 + 2048 + 512;   // + alignment slack + Control
     // TMEM columns of one stage's scale factors: A planes (4 columns per K step), then W planes (8)
     static constexpr int kSfColsA = kPlanes * kSteps * 4, kSfCols = kSfColsA + kPlanes * kSteps * 8;
-    // the scale factors of kSfSlots K blocks are in tensor memory at a time, so that a block's copies do not touch what the MMAs
-    // just ahead of them read
+    // The scale factors of kSfSlots K blocks are in tensor memory at a time, so that a block's copies do not touch what the MMAs
+    // just ahead of them read.  They do overwrite what the MMAs of block b - kSfSlots read, with no barrier between: that a
+    // tcgen05.cp does not overtake the tcgen05.mma issued before it by the same thread is an ASSUMPTION.  PTX names the order of
+    // a copy and a later MMA only; the other one is taken from the hardware, which works both off in the order of issue (CUTLASS's
+    // block-scaled main loop relies on it as well: one place for the factors of all K blocks).  A wait for those MMAs costs products
+    // of one plane 2 to 8 % (1000 x 11008 x 4096 26.0 -> 26.6 us, 500 x 4096 x 4096 12.7 -> 13.6), with three slots and the poll
+    // moved between the MMAs still 3 % (8192 x 14336 x 4096 209 -> 215).
     static constexpr int kSfSlots = kTmemSfCols / kSfCols;
     static_assert(kSfSlots >= 2 && kSfSlots <= kStages, "scale-factor ring");
     static_assert(kAccWindow + BN <= (int)kTmemSf && kTmemSf + kSfSlots * kSfCols <= kTmemCols, "tensor memory map");
