@@ -75,8 +75,8 @@ int launch_with(dim3 cluster, bool programmatic, void (*kernel)(P...), dim3 grid
 
 // chained = false: an ordinary launch.  For long kernels with one block per SM: started while their predecessor leaves, the
 // blocks land on the SMs in another order (operands shared by neighbouring tiles cross the two halves of the L2 more often).
-// That costs the longest of them 2-5 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
-// measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 250 and at 100 us.
+// That costs the longest of them up to 1 %; a call whose long kernel takes 40 us is 3-4 % faster chained.  Where the line lies was
+// measured for each of the two kernels (gemm_fp4.cu, attention_fp4.cu): at 260 us (200 of one plane) and at 350 us.
 template <typename... P, typename... A>
 int launch_clusters(dim3 cluster, bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     return launch_with(cluster, chained && programmatic_launch_ok(st), kernel, grid, block, smem, st, static_cast<A&&>(args)...);

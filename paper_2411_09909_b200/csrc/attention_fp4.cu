@@ -758,11 +758,11 @@ int launch_pass(const Maps& maps, const Params& p, int dev, int sms,
         configured[dev] = true;
     }
     const int items = p.heads * p.m_tiles;
-    // Chained up to about 100 us in the map pass.  32 heads of 128, the whole call: 1536 keys 128.7 us ordinary, 128.0 chained, 2048
-    // 194.6 / 195.9, 3072 369 / 380, causal 1024 76.3 / 72.9, 2560 186.7 / 186.8, 3072 237 / 241; of 64: 2048 206.8 / 205.4, 2560
-    // 297 / 300.
+    // Chained up to about 350 us.  The whole call, ordinary / chained: 32 heads of 128, 1536 keys 120.0 / 116.5 us, 2048 185.3 / 180.2,
+    // 2560 262 / 260, 3072 353.7 / 354.4, 6144 1127 / 1132, causal 2048 130 / 125, 3072 225.6 / 221.7, 4096 351.5 / 346.2; of 64: 2560
+    // 271.7 / 269.6, 4096 562.8 / 560.3.
     const double work = (double)p.heads * (double)p.L * (double)p.L * HD / (MASK == kMaskCausal ? 2.0 : 1.0);
-    return launch_chained(work <= 1.1e10, attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS),
+    return launch_chained(work <= 3.6e10, attention_fp4_kernel<PASS, MASK, HD>, (unsigned)(items < sms ? items : sms), threads(PASS),
                           Smem<PASS>::kBytes, st, maps.q, maps.k, maps.v, maps.sfq, maps.sfk, maps.sfv, p);
 }
 
