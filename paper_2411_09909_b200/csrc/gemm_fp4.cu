@@ -484,7 +484,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         static_assert(kOvl % 32 == 0 && (BNT - kOvl) % 32 == 0, "both parts split into two halves of 16-column chunks");
         const int tid_e = threadIdx.x - 64;
         int t = 0;
-        bool ok = true;
         static_assert(kEpilogueWarps * 32 == BN, "one column offset per epilogue thread");   // BNT <= BN
         // The per-tile constants (this thread's column offset and row offset) are fetched one tile ahead, so that
         // their latency is off the path between two tiles.
@@ -539,8 +538,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         int64_t tile = worker;
         TileConsts nxt = load_consts(tile);
         publish(nxt, tile, 0);
-        // (After a timeout the loop runs out without work: one warp may have seen the barrier complete where another saw the abort flag,
-        // and every tile's named barrier wants all eight.)
         while (tile < total_items) {
             const TileConsts cur = nxt;
             const int64_t tile_after = tile + workers;
@@ -556,7 +553,14 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             // every epilogue warp has written its part of w_fac (named barrier: the other roles do not join), and has done with the
             // tile two before, whose factors were there
             asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
-            if (ok) ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
+            const bool ok = mbar_wait(&ctl->accum_full, t & 1, &ctl->abort, p.status);
+            // After a timeout one warp may see the barrier complete where another saw the abort flag, and every tile's named barrier
+            // wants all eight.  (Here, out of the way: with the outcome carried through the loop 1000 x 11008 x 4096 took 1.8 us longer.)
+            if (__builtin_expect(!ok, 0)) {
+#pragma unroll 1
+                for (tile = tile_after; tile < total_items; tile += workers) asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");
+                break;
+            }
             tc_fence_after();
             // 16 columns of the tile: scaled and stored
             auto put = [&](const uint32_t (&v)[16], int col) {
@@ -578,7 +582,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             const int h = e >> 2, odd = t & 1;
             const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(odd ? kAccWindow : 0);
             const int part = part_log2(tile);
-            if (ok && part) {                                    // the CTA's last item: no accumulator follows
+            if (part) {                                    // the CTA's last item: no accumulator follows
                 const int cols = (BNT / 2) >> part, col0 = part_col(tile);   // of this warp: half h of the item's
                 uint32_t v[2][16];
                 tmem_ld16(taddr + h * cols, v[0]);
@@ -590,7 +594,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                     if (i + 32 < cols) tmem_ld16(taddr + h * cols + i + 32, v[0]);
                     put(v[1], col0 + h * cols + i + 16);
                 }
-            } else if (ok) {
+            } else {
                 // The tile's window starts at column 0 (even t) or kAccWindow (odd t).  The kOvl columns it shares with
                 // the next tile's window - its last ones when even, its first ones when odd - are read first; this warp
                 // takes its half h of both parts, kC1 + kC2 chunks of 16 columns.
