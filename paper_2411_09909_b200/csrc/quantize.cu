@@ -436,7 +436,7 @@ prepare_operands_kernel(const __grid_constant__ PrepParams p) {
     // Segments (the heads of an attention call): seg_rows source rows each, padded to seg_blocks blocks of 128 operand rows.
     int64_t src_row = row;
     bool live = row < o.R;
-    if (MODE != kOneCast && MODE != kAnyGroup && o.seg_blocks) {
+    if (MODE == kAttention && o.seg_blocks) {
         const unsigned seg = rb / o.seg_blocks, in_seg = (rb - seg * o.seg_blocks) * 128 + r_in;
         live = live && in_seg < o.seg_rows;
         src_row = seg * o.seg_rows + in_seg;
