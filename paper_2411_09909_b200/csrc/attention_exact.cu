@@ -19,7 +19,7 @@
 namespace amx {
 namespace {
 
-constexpr int kRows = 16, kThreads = 256, kKeys = 64;
+constexpr int kRows = 16, kThreads = 256, kKeys = 64, kSmCount = 148;
 
 __device__ __forceinline__ float code_value(uint32_t c, float sp, float sn) {
     const float mag = e2m1_mag_to_float(c & 7u);
@@ -129,8 +129,8 @@ int attn_exact(const ExactOperand& q, const ExactOperand& k, const ExactOperand&
         configured[dev] = true;
     }
     const int64_t items = (L + kRows - 1) / kRows * heads, resident = std::min<int64_t>(4, (int64_t)(228 * 1024 / (smem_bytes(L, d) + 1024)));
-    return launch(attention_exact_kernel, (unsigned)std::min(items, resident * 148), kThreads, smem_bytes(L, d), st, q, k, vt, L, attn_fused_padded(L), (int)d, kv_group, alpha, causal, O,
-                                                                     run_if_nonzero, heads);
+    return launch(attention_exact_kernel, (unsigned)std::min(items, resident * kSmCount), kThreads, smem_bytes(L, d), st, q, k, vt, L,
+                  attn_fused_padded(L), (int)d, kv_group, alpha, causal, O, run_if_nonzero, heads);
 }
 
 }  // namespace amx

@@ -128,7 +128,7 @@ struct Params {
     int64_t a_row0, w_row0;      // first rows of this product's operands inside the (stacked) prepared operands
 
     float* C;
-    int nk64, vec_store;
+    int vec_store;
     int out_bf16;                // C holds bf16 (each fp32 result rounded to nearest even) instead of fp32
     int band;                    // tile order: row blocks of A per band, see blk_m / blk_n
     int whole, split_log2;       // tail: work items below `whole` are tiles, the others 1 / 2^split_log2 of a tile's columns
@@ -733,7 +733,6 @@ int fill_params(const Fp4Operand& a, const Fp4Operand& w, int64_t M, int64_t N, 
     p.w_exp = reinterpret_cast<const int*>(pw + 2 * ow.plane + 2 * ow.sf) + w.row0;
     p.M = M; p.N = N; p.K = K; p.ld_c = ld_c; p.C = C;
     p.a_row0 = a.row0; p.w_row0 = w.row0;
-    p.nk64 = oa.nk64;
     p.vec_store = C && aligned(C, 32) && ld_c % 8 == 0;     // 32-byte stores in the epilogue
     p.status = status;
     {

@@ -739,8 +739,7 @@ size_t gemm_rows_workspace_bytes(int64_t M, int64_t N, int64_t K) {
     return kHeaderBytes + (size_t)(rows > whole ? rows : whole) * (size_t)K * 2;
 }
 
-double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) {
-    constexpr int gs = 32; return plan_rows(M, N, K, gs).us; }
+double gemm_rows_estimated_us(int64_t M, int64_t N, int64_t K) { return plan_rows(M, N, K, 32).us; }
 
 int gemm_rows(const uint8_t* a_codes, const uint8_t* a_scales, const uint8_t* w_codes, const uint8_t* w_scales,
               int64_t M, int64_t N, int64_t K, int gs, float* C, int64_t ld_c, void* workspace, cudaStream_t st) {
