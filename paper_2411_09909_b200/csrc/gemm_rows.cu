@@ -31,11 +31,11 @@
 //
 // What bounds it (times inside a chain of calls, weights from HBM).  One row of 12288 x 4096, 12.8 us: 1.9 from the end of the call
 // before to the first block (the fragments kernel and a launch), 2.4 to the first step's data, 5 for the steps - decode at 6
-// cycles of a warp per pair, six warps to a scheduler - 0.5 for the sums.  From two token tiles on mma.sync: an m16n8k16 takes a
-// scheduler about 16 cycles, for 24 rows 12 per pair of the 13 that a pair takes (14336 x 4096: 20.5 us).  Fragments are
-// re-read by every CTA, which is why few CTAs of many rows are better from 17 tokens on.  (Decoded to shared memory for
-// tcgen05.mma instead, whatever the number of tokens: 23 us - the way from the decoding warps through the MMA and back takes a
-// microsecond, and four steps of 32 KB are all that fits.)
+// cycles of a warp per pair, six warps to a scheduler - 0.5 for the sums; the other 3 lie between these points and have not
+// been traced.  From two token tiles on mma.sync: an m16n8k16 takes a scheduler about 16 cycles, for 24 rows 12 per pair of the 13
+// that a pair takes (14336 x 4096: 20.5 us).  Fragments are re-read by every CTA, which is why few CTAs of many rows are better
+// from 17 tokens on.  (Decoded to shared memory for tcgen05.mma instead, whatever the number of tokens: 23 us - the way from the
+// decoding warps through the MMA and back takes a microsecond, and four steps of 32 KB are all that fits.)
 //
 // The token rows are cast (or decoded) once by a small kernel into the fragment order.  (Cast inside the main kernel by
 // every CTA, one launch less, measured the same for one row and slower for more.)
@@ -418,14 +418,19 @@ __global__ void __launch_bounds__(kThreads, stream_ctas(NT, MB)) gemm_rows_strea
             return;
         }
         // words past the warp's last step may lie past the end of the tensor
-        const int held = min(n - first, kScaleSlotSteps);
-        for (int item = lane; item < rows_left * R::kWords; item += 32) {
-            const int r = item / R::kWords, w = item - r * R::kWords;
-            if (GS == 128) {
+        if constexpr (GS == 128) {
+            const int held = min(n - first, kScaleSlotSteps);
+            for (int item = lane; item < rows_left * R::kWords; item += 32) {
+                const int r = item / R::kWords, w = item - r * R::kWords;
                 const int64_t pair = (row0 + r) * steps + s_begin + first, word = (pair >> 1) + w;
                 if (w < pair_words(pair, held)) cp_async4(dst + R::at(r, w), p.w_scales + word * 4, pair_word_bytes(word, p.N * steps));
-            } else if (w < held * (64 / GS)) {
-                cp_async4(dst + R::at(r, w), src0 + r * scale_pitch + w * 4);
+            }
+        } else {
+            const int words = min(R::kWords, (n - first) * (64 / GS));
+            for (int item = lane; item < rows_left * R::kWords; item += 32) {
+                const int r = item / R::kWords, w = item - r * R::kWords;
+                const uint8_t* src = src0 + r * scale_pitch;
+                if (w < words) cp_async4(dst + R::at(r, w), src + w * 4);
             }
         }
     };
@@ -752,3 +757,16 @@ int gemm_rows_cast(const void* x, int64_t ld_x, const uint8_t* w_codes, const ui
 }
 
 }  // namespace amx
+
+// For tests: the layout a call on these kernels takes - {streaming kernel, token tiles of a block, blocks of tokens, weight rows of a
+// CTA, K ranges} -, so that they can say which they cover.
+extern "C" int amx_diag_rows_layout(int64_t M, int64_t N, int64_t K, int gs, int* layout) {
+    if (!amx::gemm_rows_supported(M, N, K, gs) || !layout) return AMX_ERR_SHAPE;
+    const amx::RowsPlan pl = amx::plan_rows(M, N, K, gs);
+    layout[0] = pl.stream;
+    layout[1] = pl.nt;
+    layout[2] = pl.m_blocks;
+    layout[3] = pl.stream ? pl.rows : amx::kCtaRows;
+    layout[4] = pl.slices;
+    return AMX_OK;
+}

@@ -12,7 +12,10 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 14331, 1024), (8, 4096, 2048), (1, 520, 4096), (16, 9597, 1152), (16, 5120, 640), (24, 14336, 512), (24, 11003, 1024),
           (24, 6144, 1024), (20, 1500, 4096), (32, 14330, 640), (32, 12281, 512), (32, 2500, 2304), (12, 700, 3072), (31, 1024, 8192),
-          (128, 1024, 1024), (200, 800, 512)]
+          (128, 1024, 1024), (200, 800, 512),
+          # K ranges, and rows of a CTA in between
+          (15, 65, 8192), (15, 1063, 5248), (8, 121, 8320), (10, 2647, 11776), (24, 1217, 7424), (12, 568, 8192), (13, 1327, 7296),
+          (13, 5993, 512), (31, 4755, 7424), (17, 1061, 14720), (18, 13039, 512), (24, 15413, 512)]
 
 
 @pytest.mark.parametrize("gs", [16, 32, 64, 128])

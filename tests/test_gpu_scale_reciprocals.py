@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 TIES = np.array([0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.0, 6.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 5.5, 0.0])
 
 
-def groups(nan=False):
+def groups():
     """One group of 32 per pair of scale bytes: multiples of the positive one, negative multiples of the other."""
     b = np.arange(1, 0x7C, dtype=np.uint16)
     s = (b << 8).view(np.float16).astype(np.float64)
@@ -25,13 +25,41 @@ def groups(nan=False):
 
 @pytest.mark.parametrize("gs", [16, 32, 64, 128])
 def test_codes_and_scales_of_every_scale(gs):
-    x = groups()
-    x = x.reshape(-1, 32)[: len(x) // 4 * 4].reshape(-1, 128)        # rows of 128: groups of every size hold midpoints
+    x = np.tile(groups(), (1, max(1, gs // 32)))                     # every scale is some group's largest, whatever the size
     bits = inputs.f32_to_bf16_bits(x)
     dev = torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
     codes, scales = amx.quantize(dev, gs)
     rc, rs = oracle.quantize(bits, gs)
     assert np.array_equal(codes.cpu().numpy(), rc) and np.array_equal(scales.cpu().numpy(), rs)
+
+
+@pytest.mark.parametrize("gs", [16, 32, 64, 128])
+def test_nan_among_the_elements(gs):
+    """Outside the format, but always the same: the NaN's side gets the scale byte 0x7F, read as 1.75 x 2^16, under which its other
+    elements here are zero; a NaN of either sign gets code 7.  The other side and the other groups do not notice."""
+    K = 256
+    bits = inputs.f32_to_bf16_bits(np.random.default_rng(gs).standard_normal((4, K)).astype(np.float32))
+    nans = [(0, 5, 0x7FC0), (1, 70, 0xFFC0), (2, 130, 0x7FFF), (2, 131, 0xFF81), (3, 255, 0x7F81)]
+    clean = bits.copy()
+    for r, k, b in nans:
+        bits[r, k], clean[r, k] = b, 0
+    codes, scales = oracle.quantize(clean, gs)
+    nib = np.stack([codes & 15, codes >> 4], -1).reshape(4, K)
+    scales = scales.reshape(4, K // gs, 2).copy()
+    for r, k, b in nans:
+        side, group = b >> 15, slice(k // gs * gs, (k // gs + 1) * gs)
+        scales[r, k // gs, side] = 0x7F
+        of_side = (clean[r, group] >> 15) == side
+        nib[r, group][of_side] = side << 3
+    for r, k, b in nans:
+        nib[r, k] = 7
+    want = (nib[:, 0::2] | (nib[:, 1::2] << 4)).astype(np.uint8)
+    dev = torch.from_numpy(bits.view(np.int16)).cuda().view(torch.bfloat16)
+    got = [amx.quantize(dev, gs)] + ([amx.quantize_prepared(dev, False)[:2]] if gs == 32 else [])
+    for c, s in got:
+        c, s = c.cpu().numpy(), s.cpu().numpy().reshape(4, K // gs, 2)
+        assert np.array_equal(s, scales)
+        assert np.array_equal(c.reshape(want.shape), want)
 
 
 @pytest.mark.parametrize("rows,K", [(123, 32), (30, 128), (3, 1280)])

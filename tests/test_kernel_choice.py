@@ -1,6 +1,10 @@
 """What AMX_GEMM_AUTO picks between 65 and 256 rows, where both the weight-streaming kernel and the FP4 kernel take the call:
-the one that measured faster, at shapes where the two differ by more than a twentieth (us, weights from HBM, one call)."""
+the one that measured faster, at shapes where the two differ by more than a twentieth (us, weights from HBM, one call).  And that the
+shapes at which the streaming kernel is tested take the layouts they are there for."""
+import ctypes
+
 import pytest
+import test_gpu_gemm_rows_layouts
 
 from paper_2411_09909_b200 import amx
 
@@ -45,3 +49,20 @@ def test_the_choice_changes_once_as_rows_are_added(N, K, gs):
     assert kernels == sorted(kernels, reverse=True)                     # GEMM_ROWS (0x100), then GEMM_FP4 (0x40)
     need = [L.amx_quant_gemm_workspace_bytes(M + 1, N, K, gs, 0) for M, k in enumerate(kernels) if k == amx.GEMM_ROWS]
     assert need == sorted(need)
+
+
+@pytest.mark.parametrize("gs", [16, 32, 64, 128])
+def test_the_tested_shapes_cover_the_layouts(gs):
+    diag = amx.lib().amx_diag_rows_layout
+    diag.argtypes = [ctypes.c_int64] * 3 + [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    taken = set()
+    for M, N, K in test_gpu_gemm_rows_layouts.SHAPES:
+        layout = (ctypes.c_int * 5)()
+        assert diag(M, N, K, gs, layout) == 0 and layout[0] == 1
+        taken.add(tuple(layout[1:]))
+    tiles, blocks, rows, ranges = (set(v) for v in zip(*taken))
+    assert tiles == {1, 2, 3, 4} and {1, 4, 7} <= blocks
+    assert rows >= {8, 16, 24, 32, 40, 48, 72, 80} | (set() if gs == 16 else {56, 88, 96, 104, 112})   # (groups of 16: less room)
+    assert ranges == {1, 2, 4, 8}
+    assert {(r, s) for _, _, r, s in taken} >= {(8, 1), (8, 4), (8, 8), (16, 1), (16, 2), (16, 4), (16, 8), (40, 1), (40, 2), (40, 4), (40, 8),
+                                               (48, 1), (48, 4), (72, 1), (72, 2), (72, 8)}
