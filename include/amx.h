@@ -219,8 +219,9 @@ int amx_gemm_prepared(const void* a_prepared, const void* w_prepared, int64_t M,
                       void* stream);
 /* amx_gemm_prepared for two operands that the caller knows to be single planes: each prepared in a symmetric
  * format (AMX_FMT_SYM_FP8 or AMX_FMT_MXFP4 through amx_quantize_prepared_fmt; any canonical operand whose two
- * scales agree in every group through amx_prepare), or with all its values non-negative.  Same arguments and result.  With one product per K step the tensor cores wait for the operand loads, so this form
- * keeps twice as many K blocks in flight, in the shared memory the second planes would have taken.  The promise
+ * scales agree in every group through amx_prepare), or with all its values non-negative.  Same arguments and result.
+ * With one product per K step the tensor cores wait for the operand loads, so this form has K blocks of twice the
+ * length, in the shared memory the second planes would have taken.  The promise
  * is checked on the device, per output tile, against the operands' row words: if a tile has a second plane,
  * amx_gemm_status(workspace) returns AMX_ERR_FLAGS and C is not the product (the kernel still runs to its end
  * and touches nothing outside C).  Products narrower than 129 columns, or cut into K ranges, run the general

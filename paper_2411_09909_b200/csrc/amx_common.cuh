@@ -20,14 +20,16 @@ inline int launch_status() { return cudaGetLastError() == cudaSuccess ? AMX_OK :
 
 // ---- launches ---------------------------------------------------------------------------------
 // Kernels of this library are chained by programmatic dependent launch: a kernel lets its successor onto the SMs as soon
-// as all of its own blocks run (grid_launch_dependents), and waits for its predecessors to complete before it touches
-// memory (grid_dependency_wait; it returns at once when the launch carried no such dependency).  The order of the stream
+// as all of its own blocks run (grid_launch_dependents; the FP4 GEMM and the fused attention, whose blocks fill an SM, as their last
+// act), and waits for its predecessors to complete before it touches memory (grid_dependency_wait; it returns at once when the launch
+// carried no such dependency).  What needs no memory comes before the wait in those two: barriers, tensor memory.  The few-row kernels
+// copy weights before it: the fragments kernel ahead of them lets them start only after its own wait.  The order of the stream
 // is kept, the launch latency and the gap between two kernels are not: chains of ordinary launches cost about 2 us per
 // kernel boundary.  A stream that is being captured gets ordinary launches (replayed from a graph the chains of short
 // kernels were slower with these edges).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// First statement of a kernel.  (Every kernel waits before anything else, so "my predecessor has completed" implies the
+// First statement of the other kernels.  (Every kernel waits before it ends, so "my predecessor has completed" implies the
 // same of everything before it.)
 __device__ __forceinline__ void begin_kernel() {
     grid_launch_dependents();
