@@ -19,13 +19,17 @@ constexpr uint32_t kKernelMask = AMX_GEMM_SIMT | AMX_GEMM_TC | AMX_GEMM_FP4 | AM
 
 // Time of the FP4 route under AUTO for 65 to 256 rows, us: the launches (cast, preparation, product, gated exact kernel), the K loop of
 // the tiles' waves - a last wave of few tiles in parts, which take 0.68 and 0.79 of a whole tile's time -, preparation and reading of
-// the weight, dearer where its planes no longer fit the L2, and the result.  Whole blocks of 128 rows.  Fitted to 204 calls of
-// 34 weights (N 512 to 28672, K 512 to 28672, from HBM), rms error 5 %.
+// the weight, dearer where its planes no longer fit the L2 and for rows of 4096 to 8192 elements (eight pieces of a row per lane of the
+// preparation: 68 x 11472 x 4224 49, 72 x 12288 x 4096 39), and the result, whose rows are stored number by number where they are no
+// multiple of 32 bytes (256 x 4327 x 2304 27.6, 192 x 4781 x 2688 37.5).  Whole blocks of 128 rows.  Fitted to 204 calls of
+// 34 weights (N 512 to 28672, K 512 to 28672, from HBM), rms error 5 %, and for ragged N and the other group sizes to 278 more.
 double fp4_route_us(int64_t M, int64_t N, int64_t K) {
     const int64_t m_blocks = (M + 127) / 128, tiles = m_blocks * ((N + 255) / 256), last = tiles % 148;
     const double waves = (double)(tiles / 148) + (last == 0 ? 0.0 : last * 4 <= 148 ? 0.68 : last * 2 <= 148 ? 0.79 : 1.0);
     const double nk = (double)N * (double)K;
-    return 9.8 + 0.66 * (double)((K + 127) / 128) * waves + 2.5e-7 * (nk + (nk > 1e8 ? nk - 1e8 : 0.0)) + 0.9e-6 * 128.0 * (double)m_blocks * (double)N;
+    const double mn = 128.0 * (double)m_blocks * (double)N, ragged = N % 8 ? 1.3 + 4.8e-6 * mn : 0.0;
+    const double weight = (K > 4096 && K <= 8192 ? 3.5e-7 : 2.5e-7) * nk + (nk > 1e8 ? 2.5e-7 * (nk - 1e8) : 0.0);
+    return 9.8 + 0.66 * (double)((K + 127) / 128) * waves + weight + 0.9e-6 * mn + ragged;
 }
 
 // Whether the streaming kernel is the faster one between 65 and 256 rows.  Its time grows with the rows, that of the FP4 route only
@@ -57,8 +61,8 @@ uint32_t pick_kernel(int64_t M, int64_t N, int64_t K, int gs, uint32_t flags) {
     // rows that each decode the weight again, it runs where its estimated time is below that of the FP4 route
     // (rows_pay).  Streaming kernel / FP4 route, us: 4096 x 4096 at 128 rows 24 / 29, at 160 31 / 30 and at 256 36 / 30, 12288 x 4096
     // at 72 rows 52 / 39 and at 128 59 / 40, 8192 x 4096 at 96 rows 31 / 33 and at 128 36 / 33, 4096 x 11008 at 128 rows 50 / 62 and at
-    // 160 73 / 63, 14336 x 512 at 96 rows 14.5 / 14.6 and at 192 22 / 19.  Over the fit's calls and 243 of other weights and rows the choice
-    // costs 0.1 % on average, 7 and 9 % at most.
+    // 160 73 / 63, 14336 x 512 at 96 rows 14.5 / 14.6 and at 192 22 / 19.  Over 257 calls outside the fit, a third
+    // of ragged N, all group sizes, bf16 weights among them, the choice costs 0.5 % on average, 31 % at most.
     // A narrow weight (below 512 rows and 2^23 elements) stays on the FP4 route from 2^28 multiply-adds on, slower as it is
     // (256 x 8192 at 128 rows: 12 / 43): callers read the count of flushed scales that this route leaves in the workspace.
     const double mnk = (double)M * (double)N * (double)K;

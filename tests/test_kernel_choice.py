@@ -21,6 +21,20 @@ MEASURED = [  # M, N, K, streaming kernel (its best layout), FP4 route
     (192, 16384, 2048, 57.0, 35.4), (128, 16384, 2048, 39.3, 29.8), (72, 18944, 3584, 52.3, 45.8),
     (144, 9216, 3072, 46.8, 31.1), (256, 2304, 9216, 44.2, 50.3)]
 
+# Ragged N, rows of the weight of 4096 to 8192 elements, and other group sizes: M, N, K, group size, streaming kernel, FP4 route
+MEASURED_OTHERS = [
+    (197, 2645, 4864, 16, 33.5, 46.5), (192, 4781, 2688, 16, 28.2, 37.5), (96, 7424, 4864, 16, 39.2, 43.1), (225, 7279, 768, 64, 17.5, 24.9),
+    (256, 4327, 2304, 32, 23.3, 27.6), (74, 13017, 1280, 64, 22.4, 27.7), (192, 8287, 1664, 32, 28.7, 32.1), (189, 12907, 896, 32, 28.4, 39.6),
+    (128, 27658, 768, 64, 30.5, 48.7), (104, 4081, 3840, 32, 22.7, 30.6), (192, 20844, 1920, 32, 71.8, 62.3), (132, 13625, 4352, 32, 87.6, 73.4),
+    (239, 14618, 3456, 32, 97.9, 66.1), (192, 8799, 3584, 32, 51.2, 43.8), (192, 8254, 7040, 64, 90.1, 72.1), (192, 11776, 3840, 128, 61.9, 44.9),
+    (148, 8786, 6016, 16, 92.2, 66.8), (175, 9112, 1152, 128, 22.7, 18.9)]
+
+
+@pytest.mark.parametrize("M,N,K,gs,rows_us,fp4_us", MEASURED_OTHERS)
+def test_auto_takes_the_faster_kernel_ragged_or_other_groups(M, N, K, gs, rows_us, fp4_us):
+    want = amx.GEMM_ROWS if rows_us < fp4_us else amx.GEMM_FP4
+    assert amx.lib().amx_gemm_kernel_for(M, N, K, gs, amx.GEMM_AUTO) == want
+
 
 @pytest.mark.parametrize("M,N,K,rows_us,fp4_us", MEASURED)
 def test_auto_takes_the_faster_kernel(M, N, K, rows_us, fp4_us):
@@ -40,7 +54,7 @@ def test_up_to_64_rows_stream_the_weight(M):
 
 
 @pytest.mark.parametrize("gs", [16, 32, 128])
-@pytest.mark.parametrize("N,K", [(512, 512), (1024, 4096), (4096, 4096), (12288, 4096), (28672, 1024), (28672, 512), (4096, 14336), (768, 8192),
+@pytest.mark.parametrize("N,K", [(512, 512), (1024, 4096), (4096, 4096), (12288, 4096), (28672, 1024), (28672, 512), (4096, 14336), (768, 8192), (4781, 2688), (11472, 4224),
                                  (16384, 2048), (5120, 2560)])
 def test_the_choice_changes_once_as_rows_are_added(N, K, gs):
     """And within the streaming kernel's range no call needs more scratch than one of more rows."""
