@@ -762,17 +762,21 @@ int gemm_fp4_slices(int64_t M, int64_t N, int64_t K) {
 // of M 64 to 500, N 512 to 14336, K 2048 to 28672.  Ranges / parts of two planes: 128 x 4096 x 14336 30 / 52, 256 x 4096 x 14336 40 / 52,
 // 500 x 4096 x 11008 54 / 46, 256 x 4096 x 4096 27 / 19; of one: 128 x 512 x 14336 17 / 22, 128 x 1024 x 28672 23 / 44,
 // 128 x 8192 x 28672 53 / 47, 500 x 4096 x 4096 34 / 13.  (Tiles of 128 columns have no parts and take a quarter's time; both
-// planes' figures, which a product of one plane is 3 to 20 % below.)  The choice costs 0.2 % on average.
+// planes' figures, which a product of one plane is 3 to 20 % below.)  Rows of results that are no multiple of 32 bytes are stored one
+// by one, which a range's whole tile takes 0.11 us a row for, a half 0.07, a quarter 0.025: 92 x 412 x 8192 of one plane 23 / 16,
+// 121 x 315 x 2304 of two 26 / 15.  The choice costs 0.2 % on average over these and 420 others, M from 8, N from 64, a third of them ragged.
 namespace {
-bool slices_pay(int64_t M, int64_t N, int64_t K, int slices, int sms, bool one_plane, bool half) {
+bool slices_pay(int64_t M, int64_t N, int64_t K, int slices, int sms, bool one_plane, bool half, bool vec_store) {
     if (slices < 2) return false;
     struct Fit { double ranges, block, parts, of_half, of_quarter; };
     static constexpr Fit kFit[2] = {{8.0, 0.73, 5.4, 0.50, 0.41}, {8.4, 0.48, 5.2, 0.224, 0.166}};
     const Fit& f = kFit[one_plane && !half];
     const int64_t blocks = (K + 127) / 128;
     const bool quarters = half || parts_log2(((N + BN - 1) / BN) * ((M + BM - 1) / BM), sms) == 2;
-    return f.ranges + f.block * (double)((blocks + slices - 1) / slices) + 3.0e-6 * slices * (double)M * (double)N <
-           f.parts + (quarters ? f.of_quarter : f.of_half) * (double)blocks;
+    const double rows = half ? 0.0 : (double)std::min<int64_t>(M, BM);
+    const double ranges = f.ranges + f.block * (double)((blocks + slices - 1) / slices) + 3.0e-6 * slices * (double)M * (double)N;
+    const double parts = f.parts + (quarters ? f.of_quarter : f.of_half) * (double)blocks;
+    return ranges + (N % 8 ? 0.11 * rows : 0.0) < parts + (vec_store ? 0.0 : (quarters ? 0.025 : 0.07) * rows);
 }
 }  // namespace
 size_t gemm_fp4_prepared_workspace_bytes(int64_t M, int64_t N, int64_t K) {
@@ -804,7 +808,7 @@ int gemm_fp4_prepared_at(const Fp4Operand& a, const Fp4Operand& w, int64_t M, in
     const int slices = gemm_fp4_slices(M, N, K);
     // at most 128 columns: tiles of 128 x 128, so that no half of a W tile is padding
     const bool half = N <= BN / 2 && !getenv("AMX_FP4_NO_HALF_TILE");
-    if (!gate && !scale_a && !out_bf16 && slices_pay(M, N, K, slices, sm_count(dev), one_plane, half) &&
+    if (!gate && !scale_a && !out_bf16 && slices_pay(M, N, K, slices, sm_count(dev), one_plane, half, p.vec_store != 0) &&
         workspace_bytes >= gemm_fp4_prepared_workspace_bytes(M, N, K)) {
         float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + 256);
         p.C = part;
