@@ -150,6 +150,14 @@ struct Ring {
     static constexpr int kPart = NT * kTok * kPartPitch * 4;
     static_assert(kPart <= kBytes, "the partial-product tile reuses the rings");
 };
+// Groups of 128, an odd number of scale pairs in the tensor: its last half word, which the copies of words leave out, for a run of n steps
+// that ends with the weight's last row.  row: where that row's words lie.  (Copies of a variable number of bytes instead cost calls with
+// such groups 3 to 5 %: 73 x 4096 x 8576 33.9 us, so 32.5.)
+__device__ __forceinline__ void load_last_pair(uint32_t* row, const uint8_t* scales, int64_t pairs, int n) {
+    const int64_t word = pairs >> 1;
+    row[word - ((pairs - n) >> 1)] = __ldg(reinterpret_cast<const uint16_t*>(scales + word * 4));
+}
+
 // Scales of one weight row over `n` steps: the most 4-byte words copied (groups of 128: two bytes per step, copied as the aligned
 // words around them, scale_words.cuh), and the pitch of the rows in shared memory - twice an odd number of words, so that the words
 // of eight rows that a warp reads together lie in different banks (groups of 16: four words per step, four times an odd number).
@@ -203,17 +211,20 @@ __global__ void __launch_bounds__(kThreads, NT <= 4 ? 2 : 1) gemm_rows_kernel(co
     // scales of steps [first, first + n) of the range, all 128 rows: consecutive threads copy consecutive words of a row
     auto issue_scales = [&](int first, int n) {
         const int words = scale_words(n, GS);
+        const int64_t pairs = p.N * steps;
         for (int i = threadIdx.x; i < kCtaRows * words; i += kThreads) {
             const int r_in = i / words, w = i - r_in * words;
             int64_t r = row0 + r_in;
             r = r < p.N ? r : p.N - 1;
             if (GS == 128) {
                 const int64_t pair = r * steps + s_begin + first, word = (pair >> 1) + w;
-                if (w < pair_words(pair, n)) cp_async4(scale_s + r_in * pitch + w, p.w_scales + word * 4, pair_word_bytes(word, p.N * steps));
+                if (w < pair_words(pair, n) && pair_word_whole(word, pairs)) cp_async4(scale_s + r_in * pitch + w, p.w_scales + word * 4);
             } else {
                 cp_async4(scale_s + r_in * pitch + w, p.w_scales + (r * (p.K / GS) + (s_begin + first) * (kStepK / GS)) * 2 + w * 4);
             }
         }
+        if (GS == 128 && threadIdx.x == 0 && (pairs & 1) && row0 + kCtaRows >= p.N && s_begin + first + n == steps)
+            load_last_pair(scale_s + (p.N - 1 - row0) * pitch, p.w_scales, pairs, n);
     };
     auto issue_frags = [&](int i) {            // the four warps of a step parity share the copies
         if (i < n_mine) {
@@ -420,11 +431,14 @@ __global__ void __launch_bounds__(kThreads, stream_ctas(NT, MB)) gemm_rows_strea
         // words past the warp's last step may lie past the end of the tensor
         if constexpr (GS == 128) {
             const int held = min(n - first, kScaleSlotSteps);
+            const int64_t pairs = p.N * steps;
             for (int item = lane; item < rows_left * R::kWords; item += 32) {
                 const int r = item / R::kWords, w = item - r * R::kWords;
                 const int64_t pair = (row0 + r) * steps + s_begin + first, word = (pair >> 1) + w;
-                if (w < pair_words(pair, held)) cp_async4(dst + R::at(r, w), p.w_scales + word * 4, pair_word_bytes(word, p.N * steps));
+                if (w < pair_words(pair, held) && pair_word_whole(word, pairs)) cp_async4(dst + R::at(r, w), p.w_scales + word * 4);
             }
+            if (lane == 0 && (pairs & 1) && row0 + rows_left == p.N && s_begin + first + held == steps)
+                load_last_pair(dst + R::at(rows_left - 1, 0), p.w_scales, pairs, held);
         } else {
             const int words = min(R::kWords, (n - first) * (64 / GS));
             for (int item = lane; item < rows_left * R::kWords; item += 32) {

@@ -8,7 +8,7 @@ namespace amx {
 
 // Words around the pairs first .. first + n - 1, counted from the tensor's (4-byte aligned) start: from word first / 2 on.
 __host__ __device__ constexpr int pair_words(int64_t first, int n) { return ((int)(first & 1) + n + 1) >> 1; }
-// Bytes of word `word` inside a tensor of `pairs` pairs: an odd number ends in the middle of a word.
-__host__ __device__ constexpr int pair_word_bytes(int64_t word, int64_t pairs) { return 2 * word + 2 <= pairs ? 4 : 2; }
+// Whether all of word `word` belongs to a tensor of `pairs` pairs: an odd number ends in the middle of a word.
+__host__ __device__ constexpr bool pair_word_whole(int64_t word, int64_t pairs) { return 2 * word + 2 <= pairs; }
 
 }  // namespace amx
